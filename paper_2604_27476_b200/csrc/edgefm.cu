@@ -15,13 +15,7 @@
 #include "megakernel_types.cuh"
 #include "step_plan.h"
 #include "prefill.h"
-// the persistent kernel is built twice: 11 consumer warps per CTA (short contexts, here) and 7 (long contexts,
-// in the megakernel_long_*.cu translation units), plus the warp that prefetches into L2
-#define MK_NS mk_short
-#define MK_NW_VALUE MK_NW_SHORT
-#include "megakernel.cuh"
-#undef MK_NS
-#undef MK_NW_VALUE
+#include "step_types.h"
 
 namespace edgefm {
 
@@ -118,25 +112,10 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint16_t *src, c
     }
 }
 
-// long_ctx = false: the variant without the grouped (one CTA per GQA group) attention code, for contexts that
-// never need it.
 MegaKernel mega_kernel_block2(int head_dim);   // megakernel_block2.cu
 MegaKernel mega_kernel_block4(int head_dim);   // megakernel_block4.cu
 
-template <int D>
-MegaKernel mega_kernel_g(int G, bool long_ctx, bool kv8 = false, int block_tokens = 1) {
-    if (block_tokens == 2) return mega_kernel_block2(D);
-    if (block_tokens == 4) return mega_kernel_block4(D);
-    if (kv8) {
-        if (D == 64) return G <= 4 ? mega_kernel_q8_d64_lo(G) : mega_kernel_q8_d64_hi(G);
-        return G <= 4 ? mega_kernel_q8_d128_lo(G) : mega_kernel_q8_d128_hi(G);
-    }
-    if (!long_ctx) return mk_short::decode_megakernel<D, 1, false>;   // G is only used by the grouped attention
-    if (D == 64) return G <= 4 ? mega_kernel_long_d64_lo(G) : mega_kernel_long_d64_hi(G);
-    return G <= 4 ? mega_kernel_long_d128_lo(G) : mega_kernel_long_d128_hi(G);
-}
-
-// ---- launch plan of the persistent step kernel (shared by edgefm_create and edgefm_decode_step_static) ----------------
+// ---- launch plan of the kernel for blocks of several tokens -----------------------------------------------------------
 struct StepPlan {
     MegaKernel kernel = nullptr;
     bool long_ctx = false;
@@ -153,14 +132,13 @@ struct StepPlan {
 // Kernel variant and shared-memory split for a model shape.  Returns null, or why the shape does not fit.
 // sched_reserve: bytes to set aside for the CTA's tile lists.
 inline const char *plan_step(const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, size_t sched_reserve, StepPlan *pl, cudaError_t *cuda_err,
-                             bool kv8 = false, int block_tokens = 1) {
+                             int block_tokens) {
     const int H = sh.hidden, d = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, G = nq / nkv;
     *cuda_err = cudaSuccess;
-    // (the compressed cache is attended by the grouped attention of the long-context build only)
-    pl->long_ctx = kv8 || max_context > 8192 || static_cast<long long>(nq) * MK_ATT_SPLIT_MAXC * 2 > MK_PARTIAL_FLOATS;
+    pl->long_ctx = max_context > 8192 || static_cast<long long>(nq) * MK_ATT_SPLIT_MAXC * 2 > MK_PARTIAL_FLOATS;
     if (block_tokens > 1 && pl->long_ctx) return "blocks of several tokens need the plain cache and max_context <= 8192";
     pl->block_tokens = block_tokens;
-    pl->kernel = d == 64 ? mega_kernel_g<64>(G, pl->long_ctx, kv8, block_tokens) : mega_kernel_g<128>(G, pl->long_ctx, kv8, block_tokens);
+    pl->kernel = block_tokens == 2 ? mega_kernel_block2(d) : mega_kernel_block4(d);
     pl->nw = pl->long_ctx ? MK_NW_LONG : MK_NW_SHORT;
     pl->grid = num_sms;
     pl->max_chunks = pl->grid / nkv > 0 ? pl->grid / nkv : 1;
@@ -205,7 +183,8 @@ inline const char *plan_step(const edgefm_shape &sh, int max_context, int num_sm
 
 // Raise the kernel's dynamic shared-memory limit to the most any plan can ask for (a function attribute, not an
 // allocation).  Always the same value, so contexts and static calls of different shapes never lower it for one another.
-inline cudaError_t allow_max_dynamic_smem(MegaKernel kern, int smem_optin) {
+template <typename Kernel>
+inline cudaError_t allow_max_dynamic_smem(Kernel kern, int smem_optin) {
     cudaFuncAttributes fa{};
     cudaError_t e = cudaFuncGetAttributes(&fa, kern);
     if (e != cudaSuccess) return e;
@@ -263,10 +242,10 @@ inline const char *plan_schedule(const StepPlan &pl, const edgefm_shape &sh, int
 // Shared-memory plan and tile schedule together: the tile lists live in shared memory, so their size (known only once
 // the schedule exists) takes room from the rings, whose slot size shapes the schedule.  A few rounds settle it.
 inline const char *plan_step_and_schedule(const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, StepPlan *pl, StepSchedule *ss,
-                                          cudaError_t *cuda_err, bool kv8 = false, int block_tokens = 1) {
+                                          cudaError_t *cuda_err, int block_tokens) {
     size_t reserve = 0;
     for (int attempt = 0; attempt < 6; ++attempt) {
-        if (const char *why = plan_step(sh, max_context, num_sms, smem_optin, reserve, pl, cuda_err, kv8, block_tokens)) return why;
+        if (const char *why = plan_step(sh, max_context, num_sms, smem_optin, reserve, pl, cuda_err, block_tokens)) return why;
         if (const char *why = plan_schedule(*pl, sh, sh.vocab, ss)) return why;
         const size_t need = ss->smem_bytes();
         if (need <= pl->sched_bytes) return nullptr;
@@ -335,7 +314,6 @@ struct edgefm_ctx {
     int kv_format = EDGEFM_KV_BF16;
     int block_tokens = 1;        // tokens a call may carry (edgefm_verify_block)
     float *k_scale = nullptr, *v_scale = nullptr;     // compressed cache: [L][nkv][max_context]
-    float *kv_stage = nullptr;                        // compressed cache: fp32 k, v rows of the step's token [2][nkv][d]
     float *x = nullptr;          // residual stream [H]
     float *q = nullptr;          // rotated queries [nq*d]
     float *attn = nullptr;       // attention output [nq*d]
@@ -358,7 +336,11 @@ struct edgefm_ctx {
     unsigned long long *prof = nullptr;
     int prof_stride = 0;
 
-    // the persistent step kernel
+    // the persistent step kernel: one token per call (step) ...
+    StepLaunch step;
+    StepLayer *d_layers = nullptr;        // [n_layers + 1]
+    unsigned long long *ll = nullptr;     // exchange buffers
+    // ... or, on a context for blocks of several tokens, the tile kernel (plan, mk)
     StepPlan plan;
     MkParams mk{};
     // vocabulary pruning: the full-vocabulary schedule and maps to return to, the gathered rows of the current subset
@@ -429,7 +411,7 @@ void free_all(edgefm_ctx *c) {
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
     void *bufs[] = {c->k_cache, c->v_cache, c->x, c->q, c->attn, c->act, c->inv_freq, c->part_m, c->part_l,
                     c->part_o, c->lm_part_val, c->lm_part_idx, c->tickets, c->state, c->req, c->d_ops, c->d_op_w, c->d_maps, c->d_tiles,
-                    c->d_cta_tab, c->d_combines, c->grid_bar, c->prof, c->vocab_ids, c->sub_lm, c->k_scale, c->v_scale, c->kv_stage};
+                    c->d_cta_tab, c->d_combines, c->grid_bar, c->prof, c->vocab_ids, c->sub_lm, c->k_scale, c->v_scale, c->d_layers, c->ll};
     for (void *b : bufs) if (b) cudaFree(b);
     if (c->pf.chunk) prefill_free(&c->pf);
 }
@@ -440,18 +422,19 @@ PrefillModel prefill_model(edgefm_ctx *ctx);
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // One cooperative launch of the step kernel: all CTAs are co-resident, which the grid barriers rely on.
-cudaError_t launch_step(MegaKernel kern, const StepPlan &pl, const MkParams &mk, cudaStream_t s) {
+template <typename Kernel, typename Params>
+cudaError_t launch_step(Kernel kern, int grid, int threads, size_t dyn_smem, const Params &params, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pl.grid);
-    cfg.blockDim = dim3((pl.nw + 1) * 32);
-    cfg.dynamicSmemBytes = pl.dyn_smem;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = dyn_smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, mk);
+    return cudaLaunchKernelEx(&cfg, kern, params);
 }
 
 // Record the step once; every decode step replays this graph (one kernel node).
@@ -460,7 +443,8 @@ cudaError_t record_graph(edgefm_ctx *c) {
     if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
     cudaError_t e = cudaStreamBeginCapture(c->build_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    const cudaError_t le = launch_step(c->plan.kernel, c->plan, c->mk, c->build_stream);
+    const cudaError_t le = c->block_tokens == 1 ? launch_step(c->step.kernel, c->step.grid, ST_THREADS, c->step.dyn_smem, c->step.p, c->build_stream)
+                                                : launch_step(c->plan.kernel, c->plan.grid, (c->plan.nw + 1) * 32, c->plan.dyn_smem, c->mk, c->build_stream);
     e = cudaStreamEndCapture(c->build_stream, &c->graph);
     if (le != cudaSuccess) return le;
     if (e != cudaSuccess) return e;
@@ -558,17 +542,17 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
 
     const int H = sh.hidden, d = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, F = sh.ffn;
 
-    StepPlan &pl = c->plan;
     int smem_optin = 0, coop = 0;
     CREATE_TRY(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     CREATE_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     if (!coop) return bail(EDGEFM_ERR_CUDA, "device lacks cooperative launch", cudaErrorNotSupported);
-    {
+    if (M == 1) {
+        if (const char *why = step_plan(sh, max_context, c->num_sms, smem_optin, kv8, &c->step)) return bail(EDGEFM_ERR_BAD_SHAPE, why, cudaErrorInvalidValue);
+    } else {
         cudaError_t ce = cudaSuccess;
-        if (const char *why = plan_step_and_schedule(sh, max_context, c->num_sms, smem_optin, &pl, &c->sched_full, &ce, kv8, M))
+        if (const char *why = plan_step_and_schedule(sh, max_context, c->num_sms, smem_optin, &c->plan, &c->sched_full, &ce, M))
             return bail(ce != cudaSuccess ? EDGEFM_ERR_CUDA : EDGEFM_ERR_BAD_SHAPE, why, ce != cudaSuccess ? ce : cudaErrorInvalidValue);
     }
-    const StepSchedule &ss = c->sched_full;
 
     const size_t kv_elems = static_cast<size_t>(sh.n_layers) * nkv * max_context * d;
     const size_t kv_bytes = kv8 ? kv_elems : kv_elems * 2;
@@ -578,30 +562,17 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
         const size_t kv_rows = static_cast<size_t>(sh.n_layers) * nkv * max_context;
         CREATE_TRY(dev_alloc(&c->k_scale, kv_rows));
         CREATE_TRY(dev_alloc(&c->v_scale, kv_rows));
-        CREATE_TRY(dev_alloc(&c->kv_stage, static_cast<size_t>(2) * nkv * d));
         CREATE_TRY(cudaMemset(c->k_scale, 0, kv_rows * sizeof(float)));
         CREATE_TRY(cudaMemset(c->v_scale, 0, kv_rows * sizeof(float)));
-        CREATE_TRY(cudaMemset(c->kv_stage, 0, static_cast<size_t>(2) * nkv * d * sizeof(float)));
     }
-    // (work buffers hold one vector per token of a block)
-    CREATE_TRY(dev_alloc(&c->x, static_cast<size_t>(M) * H));
-    CREATE_TRY(dev_alloc(&c->q, static_cast<size_t>(M) * nq * d));
-    CREATE_TRY(dev_alloc(&c->attn, static_cast<size_t>(M) * nq * d));
-    CREATE_TRY(dev_alloc(&c->act, static_cast<size_t>(M) * mk_splits(M) * ((F + MK_TILE_COLS - 1) / MK_TILE_COLS * MK_TILE_COLS) / 2));   // three bf16 arrays of F rounded
-                                                                                         // up to whole column pieces (the pieces of every value)
     CREATE_TRY(dev_alloc(&c->inv_freq, d / 2));
-    CREATE_TRY(dev_alloc(&c->part_m, static_cast<size_t>(M) * nq * pl.max_chunks));
-    CREATE_TRY(dev_alloc(&c->part_l, static_cast<size_t>(M) * nq * pl.max_chunks));
-    CREATE_TRY(dev_alloc(&c->part_o, static_cast<size_t>(M) * nq * pl.max_chunks * d));
-    CREATE_TRY(dev_alloc(&c->lm_part_val, static_cast<size_t>(M) * pl.grid));
-    CREATE_TRY(dev_alloc(&c->lm_part_idx, static_cast<size_t>(M) * pl.grid));
-    CREATE_TRY(dev_alloc(&c->tickets, nq + nkv + 2 + nq + 2 * nkv));   // tickets, then the per-head counters of the QKV projection
     CREATE_TRY(dev_alloc(&c->state, 1));
     CREATE_TRY(dev_alloc(&c->req, 1));
     CREATE_TRY(cudaMemset(c->k_cache, 0, kv_bytes));
     CREATE_TRY(cudaMemset(c->v_cache, 0, kv_bytes));
-    CREATE_TRY(cudaMemset(c->tickets, 0, (nq + nkv + 2 + nq + 2 * nkv) * sizeof(unsigned)));
     CREATE_TRY(cudaMemset(c->state, 0, sizeof(StepState)));
+    CREATE_TRY(dev_alloc(&c->vocab_ids, static_cast<size_t>(sh.vocab)));
+    CREATE_TRY(cudaMemset(c->vocab_ids, 0, static_cast<size_t>(sh.vocab) * sizeof(int)));
     {
         StepRequest r{-1, -1, nullptr, nullptr};
         CREATE_TRY(cudaMemcpy(c->req, &r, sizeof r, cudaMemcpyHostToDevice));
@@ -609,7 +580,46 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
         for (int i = 0; i < d / 2; ++i) inv[i] = std::pow(static_cast<double>(sh.rope_theta), -2.0 * i / d);
         CREATE_TRY(cudaMemcpy(c->inv_freq, inv.data(), inv.size() * sizeof(double), cudaMemcpyHostToDevice));
     }
-
+    const char *pe_ = getenv("EDGEFM_PROFILE");
+    if (pe_ && pe_[0] == '1') {
+        c->prof_stride = 3 + 14 * sh.n_layers;
+        const size_t n_prof = static_cast<size_t>(c->num_sms) * c->prof_stride + MK_NW_MAX * 16 * 4 + 8;   // + the optional per-warp trace
+        CREATE_TRY(dev_alloc(&c->prof, n_prof));
+        CREATE_TRY(cudaMemset(c->prof, 0, n_prof * 8));
+    }
+    if (M == 1) {
+        StepLaunch &sl = c->step;
+        CREATE_TRY(dev_alloc(&c->ll, sl.ll_bytes / 8));
+        CREATE_TRY(cudaMemset(c->ll, 0, sl.ll_bytes));
+        step_wire(&sl, c->ll);
+        std::vector<StepLayer> layers(static_cast<size_t>(sh.n_layers) + 1);
+        step_layers(sh, c->layers.data(), c->final_norm, c->lm_head, layers.data());
+        CREATE_TRY(dev_alloc(&c->d_layers, layers.size()));
+        CREATE_TRY(cudaMemcpy(c->d_layers, layers.data(), layers.size() * sizeof(StepLayer), cudaMemcpyHostToDevice));
+        StepParams &p = sl.p;
+        p.k_cache = c->k_cache; p.v_cache = c->v_cache; p.k_scale = c->k_scale; p.v_scale = c->v_scale;
+        p.embed = static_cast<const uint16_t *>(c->embed); p.inv_freq = c->inv_freq; p.layers = c->d_layers; p.vocab_ids = c->vocab_ids;
+        p.state = c->state; p.req = c->req; p.prof = c->prof; p.prof_stride = c->prof_stride;
+        CREATE_TRY(allow_max_dynamic_smem(sl.kernel, smem_optin));
+        int per_sm = 0;
+        CREATE_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sl.kernel, ST_THREADS, sl.dyn_smem));
+        if (per_sm < 1) return bail(EDGEFM_ERR_CUDA, "persistent kernel does not fit one CTA per SM", cudaErrorInvalidValue);
+    } else {
+    StepPlan &pl = c->plan;
+    const StepSchedule &ss = c->sched_full;
+    // (work buffers hold one vector per token of a block)
+    CREATE_TRY(dev_alloc(&c->x, static_cast<size_t>(M) * H));
+    CREATE_TRY(dev_alloc(&c->q, static_cast<size_t>(M) * nq * d));
+    CREATE_TRY(dev_alloc(&c->attn, static_cast<size_t>(M) * nq * d));
+    CREATE_TRY(dev_alloc(&c->act, static_cast<size_t>(M) * mk_splits(M) * ((F + MK_TILE_COLS - 1) / MK_TILE_COLS * MK_TILE_COLS) / 2));   // three bf16 arrays of F rounded
+                                                                                         // up to whole column pieces (the pieces of every value)
+    CREATE_TRY(dev_alloc(&c->part_m, static_cast<size_t>(M) * nq * pl.max_chunks));
+    CREATE_TRY(dev_alloc(&c->part_l, static_cast<size_t>(M) * nq * pl.max_chunks));
+    CREATE_TRY(dev_alloc(&c->part_o, static_cast<size_t>(M) * nq * pl.max_chunks * d));
+    CREATE_TRY(dev_alloc(&c->lm_part_val, static_cast<size_t>(M) * pl.grid));
+    CREATE_TRY(dev_alloc(&c->lm_part_idx, static_cast<size_t>(M) * pl.grid));
+    CREATE_TRY(dev_alloc(&c->tickets, nq + nkv + 2 + nq + 2 * nkv));   // tickets, then the per-head counters of the QKV projection
+    CREATE_TRY(cudaMemset(c->tickets, 0, (nq + nkv + 2 + nq + 2 * nkv) * sizeof(unsigned)));
     // the operators of the step wired to the work buffers, the tile schedule and the tensor maps of the weights
     {
         std::vector<MkOp> ops(static_cast<size_t>(pl.n_ops));
@@ -643,25 +653,16 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
     if (per_sm < 1) return bail(EDGEFM_ERR_CUDA, "persistent kernel does not fit one CTA per SM", cudaErrorInvalidValue);
     CREATE_TRY(dev_alloc(&c->grid_bar, 1));
     CREATE_TRY(cudaMemset(c->grid_bar, 0, sizeof(unsigned)));
-    CREATE_TRY(dev_alloc(&c->vocab_ids, static_cast<size_t>(sh.vocab)));
-    CREATE_TRY(cudaMemset(c->vocab_ids, 0, static_cast<size_t>(sh.vocab) * sizeof(int)));
     MkParams &m = c->mk;
     fill_shape_params(&m, sh, max_context, pl, ss);
     m.ops = c->d_ops; m.op_weights = c->d_op_w; m.maps = c->d_maps; m.tiles = c->d_tiles; m.cta_tab = c->d_cta_tab; m.combines = c->d_combines;
     m.vocab_ids = c->vocab_ids;
     m.k_cache = c->k_cache; m.v_cache = c->v_cache; m.embed = (const uint16_t *)c->embed;
-    m.kv8 = kv8 ? 1 : 0; m.k_scale = c->k_scale; m.v_scale = c->v_scale; m.kv_stage = c->kv_stage;
     m.inv_freq = c->inv_freq; m.x = c->x; m.q = c->q; m.attn = c->attn; m.part_m = c->part_m; m.part_l = c->part_l;
     m.part_o = c->part_o; m.tickets = c->tickets; m.barrier = c->grid_bar;
     m.head_ready = c->tickets + nq + nkv + 2; m.head_flags = pl.long_ctx ? 0 : MK_HEAD_FLAGS;
     m.lm_part_val = c->lm_part_val; m.lm_part_idx = c->lm_part_idx; m.state = c->state; m.req = c->req;
-    const char *pe_ = getenv("EDGEFM_PROFILE");
-    if (pe_ && pe_[0] == '1') {
-        c->prof_stride = 3 + 14 * sh.n_layers;
-        const size_t n_prof = static_cast<size_t>(pl.grid) * c->prof_stride + MK_NW_MAX * 16 * 4 + 8;   // + the optional per-warp trace
-        CREATE_TRY(dev_alloc(&c->prof, n_prof));
-        CREATE_TRY(cudaMemset(c->prof, 0, n_prof * 8));
-        m.prof = c->prof; m.prof_stride = c->prof_stride;
+    m.prof = c->prof; m.prof_stride = c->prof_stride;
     }
 
     CREATE_TRY(cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking));
@@ -963,15 +964,16 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
     DeviceGuard guard(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int H = ctx->shape.hidden;
-    const StepPlan &pl = ctx->plan;
-    // the schedule of the step with the output layer cut down to n rows (the other operators keep their lists), its
-    // tensor maps over the gathered rows, and the operator descriptor
+    uint16_t *fresh = nullptr;
     StepSchedule sub;
     const StepSchedule *ss = &ctx->sched_full;
     std::vector<CUtensorMap> lm_maps = ctx->maps_full_lm;
     MkOp op = ctx->lm_op_full;
-    uint16_t *fresh = nullptr;
-    if (n > 0) {
+    if (n > 0 && ctx->block_tokens == 1) CUDA_TRY(ctx, cudaMalloc(&fresh, static_cast<size_t>(n) * H * sizeof(uint16_t)));
+    const StepPlan &pl = ctx->plan;
+    // tile kernel: the schedule of the step with the output layer cut down to n rows (the other operators keep their lists), its
+    // tensor maps over the gathered rows, and the operator descriptor
+    if (n > 0 && ctx->block_tokens > 1) {
         for (int o = 0; o < 4; ++o) sub.ops[o] = ctx->sched_full.ops[o];
         OpShape os[5];
         op_shapes(ctx->shape, n, os);
@@ -1004,8 +1006,12 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
             e = cudaGetLastError();
         }
     }
-    const size_t lm_index = static_cast<size_t>(ctx->mk.nph - 1);
     const uint16_t *lm_w = n > 0 ? fresh : static_cast<const uint16_t *>(ctx->lm_head);
+    const StepHead head{lm_w, static_cast<const uint16_t *>(ctx->final_norm), n > 0 ? n : ctx->shape.vocab, n > 0 ? 1 : 0, {}};
+    if (ctx->block_tokens == 1) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_layers + ctx->shape.n_layers, &head, sizeof head, cudaMemcpyHostToDevice, s);
+    } else {
+    const size_t lm_index = static_cast<size_t>(ctx->mk.nph - 1);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_ops + lm_index, &op, sizeof op, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_op_w + lm_index, &lm_w, sizeof lm_w, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
@@ -1015,6 +1021,7 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_cta_tab, ss->cta_tab.data(), ss->cta_tab.size() * sizeof(int), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && !ss->combines.empty())
         e = cudaMemcpyAsync(ctx->d_combines, ss->combines.data(), ss->combines.size() * sizeof(MkCombine), cudaMemcpyHostToDevice, s);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host buffers are read before the call returns
     if (e != cudaSuccess) {
         if (fresh) cudaFree(fresh);
@@ -1035,10 +1042,11 @@ edgefm_status edgefm_get_launches_per_step(const edgefm_ctx *ctx, int32_t *n) {
 
 edgefm_status edgefm_debug_profile(edgefm_ctx *ctx, uint64_t *out_host, int64_t capacity, int32_t *n_ctas, int32_t *stride) {
     if (!ctx || !n_ctas || !stride) return EDGEFM_ERR_INVALID_ARG;
-    *n_ctas = ctx->prof ? ctx->plan.grid : 0;
+    const int grid = ctx->block_tokens == 1 ? ctx->step.grid : ctx->plan.grid;
+    *n_ctas = ctx->prof ? grid : 0;
     *stride = ctx->prof_stride;
     if (!ctx->prof || !out_host) return EDGEFM_OK;
-    int64_t n = static_cast<int64_t>(ctx->plan.grid) * ctx->prof_stride;
+    int64_t n = static_cast<int64_t>(grid) * ctx->prof_stride;
     if (capacity < n) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "profile buffer too small");
     if (capacity >= n + MK_NW_MAX * 16 * 4 + 8) n += MK_NW_MAX * 16 * 4 + 8;   // optional per-warp trace behind the table
     DeviceGuard guard(ctx->device);
@@ -1049,6 +1057,12 @@ edgefm_status edgefm_debug_profile(edgefm_ctx *ctx, uint64_t *out_host, int64_t 
 
 edgefm_status edgefm_debug_plan(const edgefm_ctx *ctx, int32_t *out8) {
     if (!ctx || !out8) return EDGEFM_ERR_INVALID_ARG;
+    if (ctx->block_tokens == 1) {
+        const StepLaunch &sl = ctx->step;
+        const int32_t v[8] = {sl.grid, ST_NW, ST_BARS, sl.max_chunk_bytes, static_cast<int32_t>(sl.dyn_smem), sl.p.ring_bytes, sl.p.table_bytes, 0};
+        std::copy(v, v + 8, out8);
+        return EDGEFM_OK;
+    }
     const StepPlan &pl = ctx->plan;
     out8[0] = pl.grid; out8[1] = pl.nw; out8[2] = pl.slots; out8[3] = pl.slot_bytes; out8[4] = static_cast<int32_t>(pl.dyn_smem);
     out8[5] = ctx->sched_full.max_cta_tiles; out8[6] = static_cast<int32_t>(pl.sched_bytes); out8[7] = pl.long_ctx ? 1 : 0;
@@ -1063,6 +1077,8 @@ edgefm_status edgefm_debug_set_wait_limit(edgefm_ctx *ctx, uint32_t limit_ns, in
     CUDA_TRY(ctx, cudaDeviceSynchronize());
     ctx->mk.spin_limit = limit_ns;
     ctx->mk.barrier_extra = extra_barrier_arrivals;
+    ctx->step.p.spin_limit = limit_ns;
+    ctx->step.p.barrier_extra = extra_barrier_arrivals;
     CUDA_TRY(ctx, record_graph(ctx));
     ctx->err.clear();
     return EDGEFM_OK;
@@ -1198,7 +1214,7 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
         if (cap != cudaStreamCaptureStatusNone)
             return fail(nullptr, EDGEFM_ERR_INVALID_ARG, "edgefm_decode_step_static must not be called on a stream that is being captured");
     }
-    const int H = sh.hidden, d = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, F = sh.ffn;
+    const int d = sh.head_dim;
     int num_sms = 0, smem_optin = 0, coop = 0;
     CUDA_TRY(nullptr, cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
     CUDA_TRY(nullptr, cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -1213,60 +1229,27 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
         g_scratch_dev_ptr[dev] = ptr;
     }
     // ---- the same plan edgefm_create makes, in host memory -------------------------------------------------
-    StepPlan pl;
-    StepSchedule ss;
-    {
-        cudaError_t ce = cudaSuccess;
-        if (const char *why = plan_step_and_schedule(sh, max_context, num_sms, smem_optin, &pl, &ss, &ce))
-            return fail(nullptr, ce != cudaSuccess ? EDGEFM_ERR_CUDA : EDGEFM_ERR_BAD_SHAPE, "%s", why);
-    }
-    const int grid = pl.grid, max_chunks = pl.max_chunks, n_ops = pl.n_ops;
+    StepLaunch sl;
+    if (const char *why = step_plan(sh, max_context, num_sms, smem_optin, false, &sl)) return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "%s", why);
 
     // carve the scratch array; reject shapes that need more than it holds
     ScratchCarver sc{g_scratch_dev_ptr[dev]};
-    unsigned char *d_maps = sc.take<unsigned char>(static_cast<size_t>(n_ops) * MK_MAX_VARIANTS * sizeof(CUtensorMap));
-    MkOp *d_ops = sc.take<MkOp>(n_ops);
-    const uint16_t **d_op_w = sc.take<const uint16_t *>(n_ops);
-    uint2 *d_tiles = sc.take<uint2>(ss.tiles.size());
-    int *d_cta_tab = sc.take<int>(ss.cta_tab.size());
-    MkCombine *d_combines = sc.take<MkCombine>(ss.combines.size() + 1);
-    float *x = sc.take<float>(H);
-    float *q = sc.take<float>(static_cast<size_t>(nq) * d);
-    float *attn = sc.take<float>(static_cast<size_t>(nq) * d);
-    float *act = sc.take<float>(static_cast<size_t>(MK_X_SPLITS) * ((F + MK_TILE_COLS - 1) / MK_TILE_COLS * MK_TILE_COLS) / 2);
+    StepLayer *d_layers = sc.take<StepLayer>(static_cast<size_t>(sh.n_layers) + 1);
     double *inv_freq = sc.take<double>(d / 2);
-    float *part_m = sc.take<float>(static_cast<size_t>(nq) * max_chunks);
-    float *part_l = sc.take<float>(static_cast<size_t>(nq) * max_chunks);
-    float *part_o = sc.take<float>(static_cast<size_t>(nq) * max_chunks * d);
-    float *lm_val = sc.take<float>(grid);
-    int *lm_idx = sc.take<int>(grid);
-    unsigned *counters = sc.take<unsigned>(static_cast<size_t>(nq) + nkv + 2 + 64 + nq + 2 * nkv);   // tickets, the grid barrier counter, the per-head counters
     StepState *state = sc.take<StepState>(1);
     StepRequest *req = sc.take<StepRequest>(1);
+    unsigned long long *ll = sc.take<unsigned long long>(sl.ll_bytes / 8);
     if (sc.off > EDGEFM_STATIC_SCRATCH_BYTES)
         return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "this shape needs %zu bytes of work buffers; the static scratch holds %zu", sc.off,
                     EDGEFM_STATIC_SCRATCH_BYTES);
-    unsigned *tickets = counters;
-    unsigned *grid_bar = counters + nq + nkv + 2 + 32;
-
-    std::vector<MkOp> ops(static_cast<size_t>(n_ops));
-    std::vector<const uint16_t *> op_w(static_cast<size_t>(n_ops));
-    fill_ops(sh, weights->layers, weights->final_norm, weights->lm_head, x, attn, q, act, ops.data(), op_w.data());
-    std::vector<CUtensorMap> maps(static_cast<size_t>(n_ops) * MK_MAX_VARIANTS);
-    if (const char *why = encode_maps(ss, sh, weights->layers, weights->lm_head, sh.vocab, maps.data()))
-        return fail(nullptr, EDGEFM_ERR_CUDA, "%s", why);
-    CUDA_TRY(nullptr, allow_max_dynamic_smem(pl.kernel, smem_optin));
-
-    MkParams m{};
-    fill_shape_params(&m, sh, max_context, pl, ss);
-    m.ops = d_ops; m.op_weights = d_op_w; m.maps = d_maps; m.tiles = d_tiles; m.cta_tab = d_cta_tab; m.combines = d_combines;
-    m.k_cache = static_cast<uint16_t *>(k_cache); m.v_cache = static_cast<uint16_t *>(v_cache);
-    m.embed = (const uint16_t *)weights->embed; m.inv_freq = inv_freq; m.x = x; m.q = q; m.attn = attn;
-    m.part_m = part_m; m.part_l = part_l; m.part_o = part_o;
-    m.head_ready = counters + nq + nkv + 2 + 64; m.head_flags = pl.long_ctx ? 0 : MK_HEAD_FLAGS;
-    m.tickets = tickets; m.barrier = grid_bar; m.lm_part_val = lm_val; m.lm_part_idx = lm_idx; m.state = state; m.req = req;
-    m.prof = nullptr; m.prof_stride = 0;
-    m.map_fence = 2;   // every call rewrites all tensor maps in the shared scratch
+    std::vector<StepLayer> layers(static_cast<size_t>(sh.n_layers) + 1);
+    step_layers(sh, weights->layers, weights->final_norm, weights->lm_head, layers.data());
+    CUDA_TRY(nullptr, allow_max_dynamic_smem(sl.kernel, smem_optin));
+    step_wire(&sl, ll);
+    StepParams &p = sl.p;
+    p.k_cache = static_cast<uint16_t *>(k_cache); p.v_cache = static_cast<uint16_t *>(v_cache);
+    p.embed = static_cast<const uint16_t *>(weights->embed); p.inv_freq = inv_freq; p.layers = d_layers;
+    p.state = state; p.req = req;
 
     // ---- stream-ordered set-up of the shared scratch: it still holds the previous call's contents ----------
     double inv[64];
@@ -1274,20 +1257,14 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     StepState st{};
     st.cur_len = cur_len; st.next_position = position;
     StepRequest rq{token_id, position, logits_out, next_token_out};
-    // counters (attention tickets, lm_head ticket, grid barrier) must start at zero
-    CUDA_TRY(nullptr, cudaMemsetAsync(counters, 0, (static_cast<size_t>(nq) + nkv + 2 + 64 + nq + 2 * nkv) * sizeof(unsigned), s));
+    // no packet of an earlier call (of any shape) may carry a tag of this one
+    CUDA_TRY(nullptr, cudaMemsetAsync(ll, 0, sl.ll_bytes, s));
     // pageable copies: the runtime stages the bytes before returning, so the sources may be freed after the call
-    CUDA_TRY(nullptr, cudaMemcpyAsync(d_ops, ops.data(), ops.size() * sizeof(MkOp), cudaMemcpyHostToDevice, s));
-    CUDA_TRY(nullptr, cudaMemcpyAsync(d_op_w, op_w.data(), op_w.size() * sizeof(op_w[0]), cudaMemcpyHostToDevice, s));
-    CUDA_TRY(nullptr, cudaMemcpyAsync(d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, s));
-    CUDA_TRY(nullptr, cudaMemcpyAsync(d_tiles, ss.tiles.data(), ss.tiles.size() * sizeof(uint2), cudaMemcpyHostToDevice, s));
-    CUDA_TRY(nullptr, cudaMemcpyAsync(d_cta_tab, ss.cta_tab.data(), ss.cta_tab.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-    if (!ss.combines.empty())
-        CUDA_TRY(nullptr, cudaMemcpyAsync(d_combines, ss.combines.data(), ss.combines.size() * sizeof(MkCombine), cudaMemcpyHostToDevice, s));
+    CUDA_TRY(nullptr, cudaMemcpyAsync(d_layers, layers.data(), layers.size() * sizeof(StepLayer), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(inv_freq, inv, static_cast<size_t>(d / 2) * sizeof(double), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(state, &st, sizeof st, cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(req, &rq, sizeof rq, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(nullptr, launch_step(pl.kernel, pl, m, s));
+    CUDA_TRY(nullptr, launch_step(sl.kernel, sl.grid, ST_THREADS, sl.dyn_smem, p, s));
     g_static_state[dev] = state;
     g_create_error.clear();
     return EDGEFM_OK;

@@ -1,0 +1,242 @@
+// Primitives of the decode-step kernel: barriers, bounded waits, packets, packed fp32 arithmetic.
+#pragma once
+#include "step_types.h"
+
+namespace edgefm {
+namespace step {
+
+__device__ __forceinline__ unsigned smem_u32(const void *p) { return static_cast<unsigned>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void mbar_init(unsigned long long *b, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(unsigned long long *b, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long *b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait(unsigned long long *b, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(b)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ unsigned long long global_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+// Bookkeeping of a bounded wait: called after every unsuccessful poll, false = give up.
+struct Spin {
+    unsigned it = 0;
+    unsigned long long t0 = 0;
+    __device__ __forceinline__ bool again(volatile int *abort_flag, unsigned limit_ns) {
+        if ((++it & 127u) == 0u) {
+            if (*abort_flag) return false;
+            const unsigned long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > limit_ns) { *abort_flag = 1; return false; }
+        }
+        return true;
+    }
+};
+__device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned parity, volatile int *abort_flag, unsigned limit_ns) {
+    if (mbar_try_wait(b, parity)) return true;
+    Spin sp;
+    while (sp.again(abort_flag, limit_ns))
+        if (mbar_try_wait(b, parity)) return true;
+    return false;
+}
+// All consumer threads meet; true = every one of them came with ok (the decision is the same for all, so that nobody is left
+// waiting at the next one).
+__device__ __forceinline__ bool cta_vote(bool ok) {
+    unsigned bad;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.eq.u32 q, %1, 0;\n\t"
+        "barrier.cta.red.or.pred p, 1, %2, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(bad)
+        : "r"(ok ? 1u : 0u), "n"(ST_NT)
+        : "memory");
+    return bad == 0;
+}
+
+// Packets.  Each 8-byte element of a vector access is written and read as a whole.
+__device__ __forceinline__ unsigned long long packet(float v, unsigned tag) {
+    return static_cast<unsigned long long>(tag) << 32 | __float_as_uint(v);
+}
+__device__ __forceinline__ float packet_value(unsigned long long p) { return __uint_as_float(static_cast<unsigned>(p)); }
+__device__ __forceinline__ unsigned packet_tag(unsigned long long p) { return static_cast<unsigned>(p >> 32); }
+__device__ __forceinline__ void put1(unsigned long long *at, float v, unsigned tag) {
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(at), "l"(packet(v, tag)) : "memory");
+}
+__device__ __forceinline__ void put2(unsigned long long *at, float a, float b, unsigned tag) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(at), "l"(packet(a, tag)), "l"(packet(b, tag)) : "memory");
+}
+// (Initialised where it is declared: a register that is only written under a predicate counts as live before it, in a persistent
+// loop everywhere, and the kernel then spills around everything else.)
+struct Two { unsigned long long a = 0ull, b = 0ull; };
+__device__ __forceinline__ Two get2(const unsigned long long *at) {
+    Two t;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(t.a), "=l"(t.b) : "l"(at) : "memory");
+    return t;
+}
+__device__ __forceinline__ bool both(const Two &t, unsigned tag) { return packet_tag(t.a) == tag && packet_tag(t.b) == tag; }
+
+// Two fp32 values in one 64-bit register pair.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 pack2(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 bf16x2_f2(uint32_t w) { return pack2(bf16lo(w), bf16hi(w)); }
+__device__ __forceinline__ float exp2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// sum over the lanes of a row (lpr of them) of N values at once: halves the values while it folds, then sums what is left
+template <int N>
+__device__ __forceinline__ float fold(float (&v)[N], int sub, int lpr) {
+    int mask = lpr >> 1;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n >>= 1) {
+        const bool up = (sub & mask) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+        }
+        mask >>= 1;
+    }
+#pragma unroll 1
+    for (; mask; mask >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
+    return v[0];
+}
+// which of the N values fold() left in a lane
+template <int N>
+__device__ __forceinline__ int folded(int sub, int lpr) {
+    int idx = 0, mask = lpr >> 1;
+#pragma unroll
+    for (int n = N; n > 1; n >>= 1) { idx = idx * 2 + ((sub & mask) ? 1 : 0); mask >>= 1; }
+    return idx;
+}
+
+// ---- shared memory ---------------------------------------------------------------------------------------------------
+// Dynamic: Shared | ring | layer table, unit tables, residual rows | staged vector, attention scratch (the MLP activations take the
+// place of both: their first packet is awaited after the vote behind the gate/up products, the last readers of the vector).
+extern __shared__ __align__(128) unsigned char st_smem[];
+// The cached positions a CTA attends to.
+struct KvShare { int g, chunk, n_chunks, t0, t1, tail, any; };
+struct Shared {
+    unsigned long long full[ST_BARS], empty[ST_BARS];
+    unsigned chunk_at[ST_BARS];                            // ring offset of the chunk behind every barrier
+    float rope[128];                                       // cos | sin of the step's position
+    float ss[ST_NW];                                       // partial sums of squares (RMSNorm)
+    float part[2][2 * ST_BATCH * ST_NW];                   // partial row sums [row][warp], two batches
+    float merged[2 * ST_NT];                               // attention outputs this CTA owns
+    float best_v[ST_NW];
+    int best_i[ST_NW];
+    int u0[5], u1[5];                                      // this CTA's units of every operator
+    KvShare share;
+    unsigned tag0, odd;                                    // tag of layer 0; test hook: a bit no tag has
+    int token, pos, n_old, total_x, total_a;               // the step's token, position, cache length; sizes of the unit tables
+    unsigned sent;                                         // 16-byte units the feeding thread has asked for
+    int abort;
+};
+constexpr int ST_SHARED_BYTES = (static_cast<int>(sizeof(Shared)) + 127) / 128 * 128;
+
+// What the device functions share: the parameter block (constant bank), the thread's place and the ring position; everything else
+// stands in shared memory, so that little is carried in registers from one operator to the next.
+struct Ctx {
+    const StepParams &par;
+    int tid, warp, lane, cta, ncta;
+    unsigned chunk;          // next ring chunk to consume
+    __device__ __forceinline__ explicit Ctx(const StepParams &p_)
+        : par(p_), tid(static_cast<int>(threadIdx.x)), warp(tid >> 5), lane(tid & 31), cta(static_cast<int>(blockIdx.x)), ncta(static_cast<int>(gridDim.x)), chunk(0u) {}
+    __device__ __forceinline__ Shared &sh() const { return *reinterpret_cast<Shared *>(st_smem); }
+    __device__ __forceinline__ const StepParams &p() const { return par; }
+    __device__ __forceinline__ volatile int *abort() const { return &sh().abort; }
+    __device__ __forceinline__ unsigned char *ring() const { return st_smem + ST_SHARED_BYTES; }
+    __device__ __forceinline__ unsigned char *tables() const { return ring() + p().ring_bytes; }
+    __device__ __forceinline__ const StepLayer *layer(int l) const { return reinterpret_cast<const StepLayer *>(tables()) + l; }
+    __device__ __forceinline__ const StepHead &head() const { return *reinterpret_cast<const StepHead *>(layer(p().n_layers)); }
+    __device__ __forceinline__ unsigned *unit_table() const { return reinterpret_cast<unsigned *>(tables() + (p().n_layers + 1) * 64); }
+    __device__ __forceinline__ float *resid() const { return reinterpret_cast<float *>(tables() + p().resid_at); }   // this CTA's rows of the residual stream
+    __device__ __forceinline__ float *xs() const { return reinterpret_cast<float *>(tables() + p().table_bytes); }
+    __device__ __forceinline__ float *scratch() const { return xs() + p().xs_floats; }     // attention
+};
+
+__device__ __forceinline__ void stamp(const Ctx &c, int &idx) {
+    const StepParams &p = c.p();
+    if (p.prof && c.tid == 0) {
+        if (idx < p.prof_stride) p.prof[static_cast<size_t>(c.cta) * p.prof_stride + idx] = global_ns();
+        ++idx;
+    }
+}
+
+// ---- ring: consumer side -----------------------------------------------------------------------------------------------
+__device__ __forceinline__ bool chunk_wait(Ctx &c, const unsigned char *&at) {
+    Shared &sh = c.sh();
+    const unsigned b = c.chunk & (ST_BARS - 1), parity = (c.chunk / ST_BARS) & 1u;
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[b], parity, c.abort(), c.p().spin_limit));
+    at = c.ring() + *reinterpret_cast<volatile unsigned *>(&sh.chunk_at[b]);
+    return ok;
+}
+__device__ __forceinline__ void chunk_release(Ctx &c) {
+    __syncwarp();
+    if (c.lane == 0) mbar_arrive(&c.sh().empty[c.chunk & (ST_BARS - 1)]);
+    ++c.chunk;
+}
+
+// ---- the order of the stream (the same arithmetic on the feeding and on the consuming side) --------------------------------
+__device__ __forceinline__ int op_units(const StepParams &p, int op, int lm_rows) {
+    switch (op) {
+        case ST_QKV: return (p.nq + 2 * p.nkv) << p.half_shift;
+        case ST_GU: return p.F;
+        case ST_LM: return lm_rows;
+        default: return p.H;
+    }
+}
+__device__ __forceinline__ bool op_paired(int op) { return op == ST_QKV || op == ST_GU; }
+__device__ __forceinline__ int units_per_batch(int op) { return op_paired(op) ? ST_BATCH : 2 * ST_BATCH; }
+// Units of the chunk that starts at unit u of [.., u1).
+__device__ __forceinline__ int chunk_units(const StepParams &p, int op, int u, int u1) {
+    const int rows = p.cols[op].rows_per_chunk;
+    int n = min(op_paired(op) ? rows >> 1 : rows, u1 - u);
+    if (op == ST_QKV) n = min(n, (1 << p.half_shift) - (u & ((1 << p.half_shift) - 1)));   // rows of one head are contiguous, heads are not
+    return n;
+}
+// The cached positions CTA `cta` attends to: a chunk of the `n` old positions.
+__device__ __forceinline__ KvShare kv_share(const StepParams &p, int n, int cta, int ncta) {
+    KvShare s;
+    s.n_chunks = max(1, min(max(1, ncta / p.nkv), (n + ST_MIN_CHUNK - 1) / ST_MIN_CHUNK));
+    s.g = cta / s.n_chunks;
+    s.chunk = cta - s.g * s.n_chunks;
+    s.t0 = st_first(n, s.chunk, s.n_chunks);
+    s.t1 = st_first(n, s.chunk + 1, s.n_chunks);
+    s.tail = s.chunk == s.n_chunks - 1;
+    s.any = s.g < p.nkv;
+    return s;
+}
+
+}  // namespace step
+}  // namespace edgefm

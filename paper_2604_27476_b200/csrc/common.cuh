@@ -17,7 +17,8 @@ struct StepState {
     int status;         // 0 = ok (reserved for bounded-wait failures)
     int pad[2];
     int n_accepted;     // tokens of the last block the cache was advanced by (1 for a plain step)
-    int reserved[3];
+    int epoch[2];       // finished calls of the step kernel (of each of a context's two builds): what its packets are tagged with
+    int reserved;
 };
 
 // What the host asks of the next step; uploaded only when it differs from the previous request.
@@ -27,7 +28,7 @@ struct StepRequest {
     float *logits_out;  // device fp32[V] (a block of m tokens: [m][V]) or null
     int *next_token_out;  // device int32[1] or null
     int m;              // tokens in this call: 1 = a plain decode step; > 1 = a block to verify (Sec. 3.11): `token` followed by
-    int draft[3];       // ... the proposed continuation draft[0 .. m-2]
+    int draft[7];       // ... the proposed continuation draft[0 .. m-2]
     int flags;          // bit 0: the tokens are given, not proposed (prompt tokens): all m enter the cache
     int pad_;
     int *n_accepted_out;  // device int32[1] or null: how many of the m tokens entered the cache (1 + accepted proposals)

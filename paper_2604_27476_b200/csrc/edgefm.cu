@@ -12,7 +12,6 @@
 #include <vector>
 
 #include "common.cuh"
-#include "megakernel_types.cuh"
 #include "step_plan.h"
 #include "prefill.h"
 #include "step_types.h"
@@ -112,187 +111,13 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint16_t *src, c
     }
 }
 
-MegaKernel mega_kernel_block2(int head_dim);   // megakernel_block2.cu
-MegaKernel mega_kernel_block4(int head_dim);   // megakernel_block4.cu
-
-// ---- launch plan of the kernel for blocks of several tokens -----------------------------------------------------------
-struct StepPlan {
-    MegaKernel kernel = nullptr;
-    bool long_ctx = false;
-    int nw = 0;            // consumer warps per CTA of the chosen kernel build
-    int grid = 0;          // CTAs (one per SM)
-    int max_chunks = 0;    // row stride of the attention partial buffers
-    int n_ops = 0;         // 4 per layer + lm_head
-    size_t xbuf = 0, ops_bytes = 0, tab_bytes = 0, sched_bytes = 0;   // shared memory: activation / attention scratch, operators, schedule table, tile lists
-    int slots = 0, slot_bytes = 0, slot_rows = 0;   // ring of one consumer warp
-    size_t dyn_smem = 0;
-    int block_tokens = 1;  // tokens a call may carry (the M of the chosen kernel build)
-};
-
-// Kernel variant and shared-memory split for a model shape.  Returns null, or why the shape does not fit.
-// sched_reserve: bytes to set aside for the CTA's tile lists.
-inline const char *plan_step(const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, size_t sched_reserve, StepPlan *pl, cudaError_t *cuda_err,
-                             int block_tokens) {
-    const int H = sh.hidden, d = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, G = nq / nkv;
-    *cuda_err = cudaSuccess;
-    pl->long_ctx = max_context > 8192 || static_cast<long long>(nq) * MK_ATT_SPLIT_MAXC * 2 > MK_PARTIAL_FLOATS;
-    if (block_tokens > 1 && pl->long_ctx) return "blocks of several tokens need the plain cache and max_context <= 8192";
-    pl->block_tokens = block_tokens;
-    pl->kernel = block_tokens == 2 ? mega_kernel_block2(d) : mega_kernel_block4(d);
-    pl->nw = pl->long_ctx ? MK_NW_LONG : MK_NW_SHORT;
-    pl->grid = num_sms;
-    pl->max_chunks = pl->grid / nkv > 0 ? pl->grid / nkv : 1;
-    pl->n_ops = 4 * sh.n_layers + 1;
-    const int NW = pl->nw, ATT_MW = NW;   // every warp has an entry in the attention merge area
-    int max_k = H;                       // vectors staged in shared memory: the residual stream and the attention output
-    if (nq * d > max_k) max_k = nq * d;   // (the down projection reads the MLP activations from global memory)
-    max_k = (max_k + MK_TILE_COLS - 1) / MK_TILE_COLS * MK_TILE_COLS;   // whole 256-column pieces (zero-padded)
-    // attention scratch: queries, probabilities, warp merge area, chunk statistics
-    // (the short-context build always runs attention with one query head per CTA)
-    const int AG = pl->long_ctx ? G : 1;
-    const size_t att_bytes = (static_cast<size_t>(AG) * d + NW * (AG * MK_ATT_TILE > 32 / MK_ATT_LPP_SPLIT ? AG * MK_ATT_TILE : 32 / MK_ATT_LPP_SPLIT) +
-                              2 * ATT_MW * AG + static_cast<size_t>(ATT_MW) * AG * d + 2 * static_cast<size_t>(AG) * pl->max_chunks) * 4;
-    size_t xbuf = block_tokens * mk_splits(block_tokens) * (static_cast<size_t>(max_k) * 2 + MK_XS_PAD);   // the staged activations: three bf16 arrays per token
-    if (att_bytes > xbuf) xbuf = att_bytes;
-    pl->xbuf = (xbuf + 1023) / 1024 * 1024;
-    cudaFuncAttributes fa{};
-    *cuda_err = cudaFuncGetAttributes(&fa, pl->kernel);
-    if (*cuda_err != cudaSuccess) return "cudaFuncGetAttributes";
-    const size_t static_smem = fa.sharedSizeBytes + (1024 - fa.sharedSizeBytes % 1024) % 1024;   // the kernel's static shared memory (mbarriers, tables, scratch) + the padding in
-                                                            // front of the 1 KB-aligned dynamic part
-    pl->ops_bytes = static_cast<size_t>(pl->n_ops) * sizeof(MkOp);
-    const size_t tab = static_cast<size_t>(cta_tab_ints_for(NW)) * sizeof(int);
-    pl->tab_bytes = (tab + 15) / 16 * 16;
-    const size_t head = (pl->ops_bytes + pl->tab_bytes + sched_reserve + 1023) / 1024 * 1024;   // the rings start on a 1 KB boundary
-    pl->sched_bytes = head - pl->ops_bytes - pl->tab_bytes;
-    const size_t tail = pl->xbuf + static_cast<size_t>(NW) * mk_wbuf_bytes(block_tokens);   // behind the rings: the activation vector and the warps' small buffers
-    if (head + tail + static_smem + static_cast<size_t>(NW) * 2 * 2048 > static_cast<size_t>(smem_optin))
-        return "model shape does not fit the shared-memory plan";
-    const size_t per_warp = (smem_optin - static_smem - head - tail) / NW;
-    // two slots per warp at least; a slot holds up to 16 rows x 256 columns (8 KB) and is a whole number of KB (an even number of rows)
-    size_t slot = per_warp / 2 / 1024 * 1024;
-    if (slot > static_cast<size_t>(MK_TILE_ROWS) * MK_TILE_COLS * 2) slot = static_cast<size_t>(MK_TILE_ROWS) * MK_TILE_COLS * 2;
-    if (slot < 2048) return "model shape does not fit the shared-memory plan";
-    pl->slot_bytes = static_cast<int>(slot);
-    pl->slot_rows = pl->slot_bytes / (MK_TILE_COLS * 2);
-    pl->slots = static_cast<int>(per_warp / slot);
-    if (pl->slots > MK_MAX_SLOTS) pl->slots = MK_MAX_SLOTS;
-    pl->dyn_smem = head + static_cast<size_t>(NW) * pl->slots * slot + tail;
-    return nullptr;
-}
-
 // Raise the kernel's dynamic shared-memory limit to the most any plan can ask for (a function attribute, not an
 // allocation).  Always the same value, so contexts and static calls of different shapes never lower it for one another.
-template <typename Kernel>
-inline cudaError_t allow_max_dynamic_smem(Kernel kern, int smem_optin) {
+inline cudaError_t allow_max_dynamic_smem(StepKernel kern, int smem_optin) {
     cudaFuncAttributes fa{};
     cudaError_t e = cudaFuncGetAttributes(&fa, kern);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - static_cast<int>(fa.sharedSizeBytes));
-}
-
-// Shapes of the five streaming operators (0..3 of a layer, 4 = output layer over `lm_rows` rows).
-inline void op_shapes(const edgefm_shape &sh, int lm_rows, OpShape os[5]) {
-    const int H = sh.hidden, d = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, F = sh.ffn;
-    const int R = (nq + 2 * nkv) * d;
-    os[0] = {PH_QKV, R / 2, H, R, d / 2};
-    os[1] = {PH_RESID, H, nq * d, H, 0};
-    os[2] = {PH_SWIGLU, F, H, 2 * F, 0};
-    os[3] = {PH_RESID, H, F, H, 0};
-    os[4] = {PH_LMHEAD, lm_rows, H, lm_rows, 0};
-}
-
-// The operators of the step in execution order, wired to the work buffers.
-inline void fill_ops(const edgefm_shape &sh, const edgefm_layer_weights *layers, const void *final_norm, const void *lm_head, float *x, float *attn, float *q,
-                     float *act, MkOp *out, const uint16_t **weights_out, int block_tokens = 1) {
-    // distance between the vectors of consecutive tokens of a block (see MkParams::block_tokens)
-    const int sx = sh.hidden, sq = sh.n_q_heads * sh.head_dim, sa = mk_splits(block_tokens) * ((sh.ffn + MK_TILE_COLS - 1) / MK_TILE_COLS * MK_TILE_COLS);
-    OpShape os[5];
-    op_shapes(sh, sh.vocab, os);
-    int n = 0;
-    auto mk = [&](const OpShape &o, const void *W, const void *bias, const void *norm, const float *x_src, float *dst, int layer, int flags, int xs_ = 0,
-                  int os_ = 0) {
-        MkOp op{};
-        op.x_tok_stride = xs_; op.out_tok_stride = os_;
-        weights_out[n] = static_cast<const uint16_t *>(W);
-        op.bias = static_cast<const uint16_t *>(bias); op.norm_w = static_cast<const uint16_t *>(norm); op.x_src = x_src; op.out = dst;
-        op.K = o.K; op.kind = o.kind; op.units_total = o.units; op.layer_flags = layer << 8 | flags | (o.K % 64 ? PHF_RAGGED : 0);
-        out[n++] = op;
-    };
-    for (int l = 0; l < sh.n_layers; ++l) {
-        const edgefm_layer_weights &w = layers[l];
-        mk(os[0], w.wqkv, sh.qkv_bias ? w.bqkv : nullptr, w.input_norm, l == 0 ? nullptr : x, q, l, 0, sx, sq);
-        mk(os[1], w.wo, nullptr, nullptr, attn, x, l, 0, sq, sx);
-        mk(os[2], w.w_gate_up, nullptr, w.post_norm, x, act, l, PHF_OUT_SPLIT, sx, sa);  // the MLP activations go to memory in the form the down projection multiplies
-        mk(os[3], w.w_down, nullptr, nullptr, act, x, l, PHF_X_GLOBAL, sa, sx);
-    }
-    mk(os[4], lm_head, nullptr, final_norm, x, nullptr, sh.n_layers, 0, sx, 0);
-}
-
-// Tile schedule of the step for the plan's geometry.  Returns null, or why the shape does not fit.
-inline const char *plan_schedule(const StepPlan &pl, const edgefm_shape &sh, int lm_rows, StepSchedule *ss) {
-    OpShape os[5];
-    op_shapes(sh, lm_rows, os);
-    for (int o = 0; o < 5; ++o)
-        if (const char *why = plan_op(os[o], o, pl.grid, pl.nw, pl.slot_rows, &ss->ops[o])) return why;
-    assemble_schedule(ss, pl.grid, pl.nw);
-    return nullptr;
-}
-
-// Shared-memory plan and tile schedule together: the tile lists live in shared memory, so their size (known only once
-// the schedule exists) takes room from the rings, whose slot size shapes the schedule.  A few rounds settle it.
-inline const char *plan_step_and_schedule(const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, StepPlan *pl, StepSchedule *ss,
-                                          cudaError_t *cuda_err, int block_tokens) {
-    size_t reserve = 0;
-    for (int attempt = 0; attempt < 6; ++attempt) {
-        if (const char *why = plan_step(sh, max_context, num_sms, smem_optin, reserve, pl, cuda_err, block_tokens)) return why;
-        if (const char *why = plan_schedule(*pl, sh, sh.vocab, ss)) return why;
-        const size_t need = ss->smem_bytes();
-        if (need <= pl->sched_bytes) return nullptr;
-        reserve = need + (attempt > 0 ? need / 8 : 0);
-    }
-    return "model shape does not fit the shared-memory plan";
-}
-
-// Tensor maps of all weight matrices: [(4 l + op) * MK_MAX_VARIANTS + variant]; the output layer's come last.
-inline const char *encode_maps(const StepSchedule &ss, const edgefm_shape &sh, const edgefm_layer_weights *layers, const void *lm_head, int lm_rows,
-                               CUtensorMap *maps) {
-    OpShape os[5];
-    op_shapes(sh, lm_rows, os);
-    auto enc = [&](int opi, int o, const void *W) {
-        for (int v = 0; v < MK_MAX_VARIANTS; ++v) {
-            CUtensorMap *m = &maps[static_cast<size_t>(opi) * MK_MAX_VARIANTS + v];
-            if (v >= ss.ops[o].n_variants) { std::memset(m, 0, sizeof *m); continue; }
-            const int pair_rows = os[o].kind == PH_QKV ? os[o].head_half : (os[o].kind == PH_SWIGLU ? os[o].units : 0);
-            if (!encode_weight_map(m, W, os[o].rows, os[o].K, ss.ops[o].variant_rows[v], pair_rows, os[o].kind == PH_QKV)) return false;
-        }
-        return true;
-    };
-    for (int l = 0; l < sh.n_layers; ++l) {
-        const edgefm_layer_weights &w = layers[l];
-        if (!enc(4 * l + 0, 0, w.wqkv) || !enc(4 * l + 1, 1, w.wo) || !enc(4 * l + 2, 2, w.w_gate_up) || !enc(4 * l + 3, 3, w.w_down))
-            return "cuTensorMapEncodeTiled failed";
-    }
-    if (!enc(4 * sh.n_layers, 4, lm_head)) return "cuTensorMapEncodeTiled failed";
-    return nullptr;
-}
-
-// Shape-derived kernel parameters common to both entry points (buffers, cache and schedule pointers are the caller's).
-inline void fill_shape_params(MkParams *m, const edgefm_shape &sh, int max_context, const StepPlan &pl, const StepSchedule &ss) {
-    m->nph = pl.n_ops; m->n_layers = sh.n_layers; m->H = sh.hidden; m->nq = sh.n_q_heads; m->nkv = sh.n_kv_heads;
-    m->d = sh.head_dim; m->F = sh.ffn; m->V = sh.vocab;
-    m->half_shift = sh.head_dim == 64 ? 5 : 6;
-    m->eps = sh.rms_eps; m->scale = static_cast<float>(1.0 / std::sqrt(static_cast<double>(sh.head_dim)));
-    m->max_context = max_context; m->max_chunks = pl.max_chunks; m->block_tokens = pl.block_tokens;
-    m->att_chunk_shared = 256; m->att_chunk_split = 64; m->att_split_max_n = 8192;
-    m->slots = pl.slots; m->slot_bytes = pl.slot_bytes;
-    m->xbuf_bytes = static_cast<int>(pl.xbuf); m->ops_bytes = static_cast<int>(pl.ops_bytes); m->tab_bytes = static_cast<int>(pl.tab_bytes);
-    m->sched_bytes = static_cast<int>(pl.sched_bytes);
-    m->cta_tab_ints = ss.cta_tab_ints;
-    m->barrier_extra = 0;
-    m->pf_tiles = MK_PF_TILES;   // measured: 3 .. 8 equal, 16 thrashes L2 (1.5B shape)
-    m->map_fence = 1;   // edgefm_set_vocab_subset rewrites the output layer's maps between steps
-    m->spin_limit = 1000000000u;   // 1 s
 }
 
 }  // namespace edgefm
@@ -314,51 +139,34 @@ struct edgefm_ctx {
     int kv_format = EDGEFM_KV_BF16;
     int block_tokens = 1;        // tokens a call may carry (edgefm_verify_block)
     float *k_scale = nullptr, *v_scale = nullptr;     // compressed cache: [L][nkv][max_context]
-    float *x = nullptr;          // residual stream [H]
-    float *q = nullptr;          // rotated queries [nq*d]
-    float *attn = nullptr;       // attention output [nq*d]
-    float *act = nullptr;        // SwiGLU output [F]
     double *inv_freq = nullptr;  // [d/2]
-    float *part_m = nullptr, *part_l = nullptr, *part_o = nullptr;
-    float *lm_part_val = nullptr;
-    int *lm_part_idx = nullptr;
-    unsigned *tickets = nullptr;  // [nq] attention + [1] lm_head
     StepState *state = nullptr;
     StepRequest *req = nullptr;
-    MkOp *d_ops = nullptr;
-    const uint16_t **d_op_w = nullptr;   // base of every operator's weight matrix
-    unsigned char *d_maps = nullptr;   // CUtensorMap [(4 L + 1) * MK_MAX_VARIANTS]
-    uint2 *d_tiles = nullptr;
-    int *d_cta_tab = nullptr;
-    MkCombine *d_combines = nullptr;
-    size_t tiles_cap = 0, combines_cap = 0;
-    unsigned *grid_bar = nullptr;
     unsigned long long *prof = nullptr;
     int prof_stride = 0;
 
-    // the persistent step kernel: one token per call (step) ...
-    StepLaunch step;
+    // the persistent step kernel: the build for block_tokens tokens per call, and, from the first longer block on, the one for eight
+    struct Build {
+        StepLaunch launch;
+        unsigned long long *ll = nullptr;     // exchange buffers
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+    } step, wide;
+    bool wide_refused = false;
     StepLayer *d_layers = nullptr;        // [n_layers + 1]
-    unsigned long long *ll = nullptr;     // exchange buffers
-    // ... or, on a context for blocks of several tokens, the tile kernel (plan, mk)
-    StepPlan plan;
-    MkParams mk{};
-    // vocabulary pruning: the full-vocabulary schedule and maps to return to, the gathered rows of the current subset
-    // and their token ids
-    StepSchedule sched_full;
-    std::vector<CUtensorMap> maps_full_lm;   // MK_MAX_VARIANTS maps of the full output layer
-    MkOp lm_op_full{};
+    // vocabulary pruning: the gathered rows of the current subset and their token ids
     int *vocab_ids = nullptr;       // [vocab]
     uint16_t *sub_lm = nullptr;     // [vocab_subset][hidden] or null
     int vocab_subset = 0;           // 0 = full vocabulary
 
     cudaStream_t build_stream = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
     int launches_per_step = 0;
     PrefillBuffers pf;           // work buffers of edgefm_prefill, allocated at its first call
     int prefill_launches = 0;    // kernels the last edgefm_prefill enqueued
     uint32_t pf_wait_limit = 1u << 24, pf_extra_arrivals = 0;   // edgefm_debug_set_prefill_wait
+
+    uint32_t spin_limit = 1000000000u;   // edgefm_debug_set_wait_limit: 1 s
+    int barrier_extra = 0;
 
     // host mirrors
     int cur_len = 0;
@@ -406,12 +214,13 @@ cudaError_t dev_alloc(T **p, size_t count) {
 }
 
 void free_all(edgefm_ctx *c) {
-    if (c->exec) cudaGraphExecDestroy(c->exec);
-    if (c->graph) cudaGraphDestroy(c->graph);
+    for (edgefm_ctx::Build *b : {&c->step, &c->wide}) {
+        if (b->exec) cudaGraphExecDestroy(b->exec);
+        if (b->graph) cudaGraphDestroy(b->graph);
+        if (b->ll) cudaFree(b->ll);
+    }
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
-    void *bufs[] = {c->k_cache, c->v_cache, c->x, c->q, c->attn, c->act, c->inv_freq, c->part_m, c->part_l,
-                    c->part_o, c->lm_part_val, c->lm_part_idx, c->tickets, c->state, c->req, c->d_ops, c->d_op_w, c->d_maps, c->d_tiles,
-                    c->d_cta_tab, c->d_combines, c->grid_bar, c->prof, c->vocab_ids, c->sub_lm, c->k_scale, c->v_scale, c->d_layers, c->ll};
+    void *bufs[] = {c->k_cache, c->v_cache, c->inv_freq, c->state, c->req, c->prof, c->vocab_ids, c->sub_lm, c->k_scale, c->v_scale, c->d_layers};
     for (void *b : bufs) if (b) cudaFree(b);
     if (c->pf.chunk) prefill_free(&c->pf);
 }
@@ -422,34 +231,56 @@ PrefillModel prefill_model(edgefm_ctx *ctx);
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // One cooperative launch of the step kernel: all CTAs are co-resident, which the grid barriers rely on.
-template <typename Kernel, typename Params>
-cudaError_t launch_step(Kernel kern, int grid, int threads, size_t dyn_smem, const Params &params, cudaStream_t s) {
+cudaError_t launch_step(const StepLaunch &sl, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = dyn_smem;
+    cfg.gridDim = dim3(sl.grid);
+    cfg.blockDim = dim3(ST_THREADS);
+    cfg.dynamicSmemBytes = sl.dyn_smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, params);
+    return cudaLaunchKernelEx(&cfg, sl.kernel, sl.p);
 }
 
 // Record the step once; every decode step replays this graph (one kernel node).
-cudaError_t record_graph(edgefm_ctx *c) {
-    if (c->exec) { cudaGraphExecDestroy(c->exec); c->exec = nullptr; }
-    if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
+cudaError_t record_graph(edgefm_ctx *c, edgefm_ctx::Build *b) {
+    if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
+    if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
     cudaError_t e = cudaStreamBeginCapture(c->build_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    const cudaError_t le = c->block_tokens == 1 ? launch_step(c->step.kernel, c->step.grid, ST_THREADS, c->step.dyn_smem, c->step.p, c->build_stream)
-                                                : launch_step(c->plan.kernel, c->plan.grid, (c->plan.nw + 1) * 32, c->plan.dyn_smem, c->mk, c->build_stream);
-    e = cudaStreamEndCapture(c->build_stream, &c->graph);
+    const cudaError_t le = launch_step(b->launch, c->build_stream);
+    e = cudaStreamEndCapture(c->build_stream, &b->graph);
     if (le != cudaSuccess) return le;
     if (e != cudaSuccess) return e;
     c->launches_per_step = 1;
-    return cudaGraphInstantiate(&c->exec, c->graph, 0);
+    return cudaGraphInstantiate(&b->exec, b->graph, 0);
+}
+
+// Plan, buffers and graph of the build for `mt` tokens per call.  *why: the shape does not fit.
+cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char **why) {
+    int smem_optin = 0, per_sm = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    if (e != cudaSuccess) return e;
+    StepLaunch &sl = b->launch;
+    if ((*why = step_plan(c->shape, c->max_context, c->num_sms, smem_optin, c->kv_format == EDGEFM_KV_INT8, mt, &sl))) return cudaSuccess;
+    if (!b->ll) {
+        if ((e = dev_alloc(&b->ll, sl.ll_bytes / 8)) != cudaSuccess) return e;
+        if ((e = cudaMemset(b->ll, 0, sl.ll_bytes)) != cudaSuccess) return e;
+    }
+    step_wire(&sl, mt, b->ll);
+    StepParams &p = sl.p;
+    p.k_cache = c->k_cache; p.v_cache = c->v_cache; p.k_scale = c->k_scale; p.v_scale = c->v_scale;
+    p.embed = static_cast<const uint16_t *>(c->embed); p.inv_freq = c->inv_freq; p.layers = c->d_layers; p.vocab_ids = c->vocab_ids;
+    p.state = c->state; p.req = c->req; p.prof = c->prof; p.prof_stride = c->prof_stride;
+    p.epoch_slot = b == &c->wide ? 1 : 0;
+    p.spin_limit = c->spin_limit; p.barrier_extra = c->barrier_extra;
+    if ((e = allow_max_dynamic_smem(sl.kernel, smem_optin)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sl.kernel, ST_THREADS, sl.dyn_smem)) != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidValue;
+    return record_graph(c, b);
 }
 
 }  // namespace
@@ -540,19 +371,12 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
         if (e_ != cudaSuccess) return bail(e_ == cudaErrorMemoryAllocation ? EDGEFM_ERR_OUT_OF_MEMORY : EDGEFM_ERR_CUDA, #call, e_); \
     } while (0)
 
-    const int H = sh.hidden, d = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, F = sh.ffn;
+    const int d = sh.head_dim, nkv = sh.n_kv_heads;
 
-    int smem_optin = 0, coop = 0;
-    CREATE_TRY(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    int coop = 0;
     CREATE_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     if (!coop) return bail(EDGEFM_ERR_CUDA, "device lacks cooperative launch", cudaErrorNotSupported);
-    if (M == 1) {
-        if (const char *why = step_plan(sh, max_context, c->num_sms, smem_optin, kv8, &c->step)) return bail(EDGEFM_ERR_BAD_SHAPE, why, cudaErrorInvalidValue);
-    } else {
-        cudaError_t ce = cudaSuccess;
-        if (const char *why = plan_step_and_schedule(sh, max_context, c->num_sms, smem_optin, &c->plan, &c->sched_full, &ce, M))
-            return bail(ce != cudaSuccess ? EDGEFM_ERR_CUDA : EDGEFM_ERR_BAD_SHAPE, why, ce != cudaSuccess ? ce : cudaErrorInvalidValue);
-    }
+    if (M > 1 && max_context > 8192) return bail(EDGEFM_ERR_BAD_SHAPE, "blocks of several tokens need max_context <= 8192", cudaErrorInvalidValue);
 
     const size_t kv_elems = static_cast<size_t>(sh.n_layers) * nkv * max_context * d;
     const size_t kv_bytes = kv8 ? kv_elems : kv_elems * 2;
@@ -583,90 +407,22 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
     const char *pe_ = getenv("EDGEFM_PROFILE");
     if (pe_ && pe_[0] == '1') {
         c->prof_stride = 3 + 14 * sh.n_layers;
-        const size_t n_prof = static_cast<size_t>(c->num_sms) * c->prof_stride + MK_NW_MAX * 16 * 4 + 8;   // + the optional per-warp trace
+        const size_t n_prof = static_cast<size_t>(c->num_sms) * c->prof_stride;
         CREATE_TRY(dev_alloc(&c->prof, n_prof));
         CREATE_TRY(cudaMemset(c->prof, 0, n_prof * 8));
     }
-    if (M == 1) {
-        StepLaunch &sl = c->step;
-        CREATE_TRY(dev_alloc(&c->ll, sl.ll_bytes / 8));
-        CREATE_TRY(cudaMemset(c->ll, 0, sl.ll_bytes));
-        step_wire(&sl, c->ll);
+    {
         std::vector<StepLayer> layers(static_cast<size_t>(sh.n_layers) + 1);
         step_layers(sh, c->layers.data(), c->final_norm, c->lm_head, layers.data());
         CREATE_TRY(dev_alloc(&c->d_layers, layers.size()));
         CREATE_TRY(cudaMemcpy(c->d_layers, layers.data(), layers.size() * sizeof(StepLayer), cudaMemcpyHostToDevice));
-        StepParams &p = sl.p;
-        p.k_cache = c->k_cache; p.v_cache = c->v_cache; p.k_scale = c->k_scale; p.v_scale = c->v_scale;
-        p.embed = static_cast<const uint16_t *>(c->embed); p.inv_freq = c->inv_freq; p.layers = c->d_layers; p.vocab_ids = c->vocab_ids;
-        p.state = c->state; p.req = c->req; p.prof = c->prof; p.prof_stride = c->prof_stride;
-        CREATE_TRY(allow_max_dynamic_smem(sl.kernel, smem_optin));
-        int per_sm = 0;
-        CREATE_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sl.kernel, ST_THREADS, sl.dyn_smem));
-        if (per_sm < 1) return bail(EDGEFM_ERR_CUDA, "persistent kernel does not fit one CTA per SM", cudaErrorInvalidValue);
-    } else {
-    StepPlan &pl = c->plan;
-    const StepSchedule &ss = c->sched_full;
-    // (work buffers hold one vector per token of a block)
-    CREATE_TRY(dev_alloc(&c->x, static_cast<size_t>(M) * H));
-    CREATE_TRY(dev_alloc(&c->q, static_cast<size_t>(M) * nq * d));
-    CREATE_TRY(dev_alloc(&c->attn, static_cast<size_t>(M) * nq * d));
-    CREATE_TRY(dev_alloc(&c->act, static_cast<size_t>(M) * mk_splits(M) * ((F + MK_TILE_COLS - 1) / MK_TILE_COLS * MK_TILE_COLS) / 2));   // three bf16 arrays of F rounded
-                                                                                         // up to whole column pieces (the pieces of every value)
-    CREATE_TRY(dev_alloc(&c->part_m, static_cast<size_t>(M) * nq * pl.max_chunks));
-    CREATE_TRY(dev_alloc(&c->part_l, static_cast<size_t>(M) * nq * pl.max_chunks));
-    CREATE_TRY(dev_alloc(&c->part_o, static_cast<size_t>(M) * nq * pl.max_chunks * d));
-    CREATE_TRY(dev_alloc(&c->lm_part_val, static_cast<size_t>(M) * pl.grid));
-    CREATE_TRY(dev_alloc(&c->lm_part_idx, static_cast<size_t>(M) * pl.grid));
-    CREATE_TRY(dev_alloc(&c->tickets, nq + nkv + 2 + nq + 2 * nkv));   // tickets, then the per-head counters of the QKV projection
-    CREATE_TRY(cudaMemset(c->tickets, 0, (nq + nkv + 2 + nq + 2 * nkv) * sizeof(unsigned)));
-    // the operators of the step wired to the work buffers, the tile schedule and the tensor maps of the weights
-    {
-        std::vector<MkOp> ops(static_cast<size_t>(pl.n_ops));
-        std::vector<const uint16_t *> op_w(static_cast<size_t>(pl.n_ops));
-        fill_ops(sh, c->layers.data(), c->final_norm, c->lm_head, c->x, c->attn, c->q, c->act, ops.data(), op_w.data(), M);
-        c->lm_op_full = ops.back();
-        std::vector<CUtensorMap> maps(static_cast<size_t>(pl.n_ops) * MK_MAX_VARIANTS);
-        if (const char *why = encode_maps(ss, sh, c->layers.data(), c->lm_head, sh.vocab, maps.data()))
-            return bail(EDGEFM_ERR_CUDA, why, cudaErrorUnknown);
-        c->maps_full_lm.assign(maps.end() - MK_MAX_VARIANTS, maps.end());
-        c->tiles_cap = ss.tiles.size();
-        c->combines_cap = static_cast<size_t>(pl.grid) * 5 * (2 * pl.nw + 4);
-        if (ss.combines.size() > c->combines_cap) c->combines_cap = ss.combines.size();
-        CREATE_TRY(dev_alloc(&c->d_ops, ops.size()));
-        CREATE_TRY(dev_alloc(&c->d_op_w, op_w.size()));
-        CREATE_TRY(cudaMemcpy(c->d_op_w, op_w.data(), op_w.size() * sizeof(op_w[0]), cudaMemcpyHostToDevice));
-        CREATE_TRY(cudaMalloc(reinterpret_cast<void **>(&c->d_maps), maps.size() * sizeof(CUtensorMap)));
-        CREATE_TRY(dev_alloc(&c->d_tiles, c->tiles_cap));
-        CREATE_TRY(dev_alloc(&c->d_cta_tab, ss.cta_tab.size()));
-        CREATE_TRY(dev_alloc(&c->d_combines, c->combines_cap));
-        CREATE_TRY(cudaMemcpy(c->d_ops, ops.data(), ops.size() * sizeof(MkOp), cudaMemcpyHostToDevice));
-        CREATE_TRY(cudaMemcpy(c->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
-        CREATE_TRY(cudaMemcpy(c->d_tiles, ss.tiles.data(), ss.tiles.size() * sizeof(uint2), cudaMemcpyHostToDevice));
-        CREATE_TRY(cudaMemcpy(c->d_cta_tab, ss.cta_tab.data(), ss.cta_tab.size() * sizeof(int), cudaMemcpyHostToDevice));
-        if (!ss.combines.empty())
-            CREATE_TRY(cudaMemcpy(c->d_combines, ss.combines.data(), ss.combines.size() * sizeof(MkCombine), cudaMemcpyHostToDevice));
     }
-    CREATE_TRY(allow_max_dynamic_smem(pl.kernel, smem_optin));
-    int per_sm = 0;
-    CREATE_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pl.kernel, (pl.nw + 1) * 32, pl.dyn_smem));
-    if (per_sm < 1) return bail(EDGEFM_ERR_CUDA, "persistent kernel does not fit one CTA per SM", cudaErrorInvalidValue);
-    CREATE_TRY(dev_alloc(&c->grid_bar, 1));
-    CREATE_TRY(cudaMemset(c->grid_bar, 0, sizeof(unsigned)));
-    MkParams &m = c->mk;
-    fill_shape_params(&m, sh, max_context, pl, ss);
-    m.ops = c->d_ops; m.op_weights = c->d_op_w; m.maps = c->d_maps; m.tiles = c->d_tiles; m.cta_tab = c->d_cta_tab; m.combines = c->d_combines;
-    m.vocab_ids = c->vocab_ids;
-    m.k_cache = c->k_cache; m.v_cache = c->v_cache; m.embed = (const uint16_t *)c->embed;
-    m.inv_freq = c->inv_freq; m.x = c->x; m.q = c->q; m.attn = c->attn; m.part_m = c->part_m; m.part_l = c->part_l;
-    m.part_o = c->part_o; m.tickets = c->tickets; m.barrier = c->grid_bar;
-    m.head_ready = c->tickets + nq + nkv + 2; m.head_flags = pl.long_ctx ? 0 : MK_HEAD_FLAGS;
-    m.lm_part_val = c->lm_part_val; m.lm_part_idx = c->lm_part_idx; m.state = c->state; m.req = c->req;
-    m.prof = c->prof; m.prof_stride = c->prof_stride;
-    }
-
     CREATE_TRY(cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking));
-    CREATE_TRY(record_graph(c));
+    {
+        const char *why = nullptr;
+        CREATE_TRY(make_build(c, M, &c->step, &why));
+        if (why) return bail(EDGEFM_ERR_BAD_SHAPE, why, cudaErrorInvalidValue);
+    }
     CREATE_TRY(cudaDeviceSynchronize());
 #undef CREATE_TRY
     g_create_error.clear();
@@ -749,7 +505,7 @@ edgefm_status edgefm_decode_step(edgefm_ctx *ctx, int32_t token_id, int32_t posi
         ctx->last_req = r;
         ctx->req_valid = true;
     }
-    CUDA_TRY(ctx, cudaGraphLaunch(ctx->exec, s));
+    CUDA_TRY(ctx, cudaGraphLaunch(ctx->step.exec, s));
     ctx->cur_len += 1;
     ctx->have_token = true;
     ctx->err.clear();
@@ -760,13 +516,13 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
                                   int32_t *n_accepted_out, int32_t *next_token_out) {
     if (!ctx) return EDGEFM_ERR_INVALID_ARG;
     if (!tokens) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "null tokens");
-    const bool dense = m > ctx->block_tokens;   // longer blocks go through the dense path (the prefill kernels)
+    const bool longer = m > ctx->block_tokens;   // than the context's build carries: the build for eight tokens, or the dense path
     if (m < 1 || m > std::max(ctx->block_tokens, PF_VERIFY_MAX))
         return fail(ctx, EDGEFM_ERR_INVALID_ARG, "m = %d: blocks of 1 .. %d tokens", m, std::max(ctx->block_tokens, PF_VERIFY_MAX));
-    if (dense && (tokens[0] < 0 || position < 0))
-        return fail(ctx, EDGEFM_ERR_INVALID_ARG, "a block of %d tokens on this context (block_tokens = %d) takes the dense path, which needs tokens[0] and position given", m, ctx->block_tokens);
-    if (dense && !ctx->len_exact)
-        return fail(ctx, EDGEFM_ERR_INVALID_ARG, "the dense path places the block behind the host's cache length: call edgefm_sync_length after the previous block first");
+    if (longer && (tokens[0] < 0 || position < 0))
+        return fail(ctx, EDGEFM_ERR_INVALID_ARG, "a block of %d tokens on this context (block_tokens = %d) needs tokens[0] and position given", m, ctx->block_tokens);
+    if (longer && !ctx->len_exact)
+        return fail(ctx, EDGEFM_ERR_INVALID_ARG, "the block is placed behind the host's cache length: call edgefm_sync_length after the previous block first");
     if (tokens[0] < -1 || tokens[0] >= ctx->shape.vocab) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "tokens[0] = %d out of range", tokens[0]);
     for (int t = 1; t < m; ++t)
         if (tokens[t] < 0 || tokens[t] >= ctx->shape.vocab) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "tokens[%d] = %d out of range", t, tokens[t]);
@@ -776,7 +532,16 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
         return fail(ctx, EDGEFM_ERR_CONTEXT_FULL, "%d tokens do not fit behind %d of %d cache slots", m, ctx->cur_len, ctx->max_context);
     DeviceGuard guard(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (dense) {
+    edgefm_ctx::Build *build = &ctx->step;
+    if (longer) {
+        if (!ctx->wide.exec && !ctx->wide_refused) {   // made at the first longer block, kept
+            const char *why = nullptr;
+            CUDA_TRY(ctx, make_build(ctx, PF_VERIFY_MAX, &ctx->wide, &why));
+            ctx->wide_refused = why != nullptr;
+        }
+        build = &ctx->wide;
+    }
+    if (longer && ctx->wide_refused) {   // a shape whose vectors for eight tokens do not fit the shared memory: the prompt kernels
         if (const edgefm_status st = ensure_prefill_buffers(ctx)) return st;
         PrefillModel pm = prefill_model(ctx);
         int launches = 0;
@@ -801,14 +566,14 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
     }
     StepRequest r{tokens[0], position, logits_out, next_token_out};
     r.m = m;
-    for (int t = 1; t < m && t <= 3; ++t) r.draft[t - 1] = tokens[t];
+    for (int t = 1; t < m; ++t) r.draft[t - 1] = tokens[t];
     r.n_accepted_out = n_accepted_out;
     if (!ctx->req_valid || std::memcmp(&r, &ctx->last_req, sizeof r) != 0) {
         CUDA_TRY(ctx, cudaMemcpyAsync(ctx->req, &r, sizeof r, cudaMemcpyHostToDevice, s));
         ctx->last_req = r;
         ctx->req_valid = true;
     }
-    CUDA_TRY(ctx, cudaGraphLaunch(ctx->exec, s));
+    CUDA_TRY(ctx, cudaGraphLaunch(build->exec, s));
     ctx->cur_len += m;     // an upper bound until edgefm_sync_length: the device decides how many tokens are accepted
     if (m > 1) ctx->len_exact = false;
     ctx->have_token = true;
@@ -836,7 +601,7 @@ edgefm_status edgefm_prefill_tokens(edgefm_ctx *ctx, const int32_t *tokens, int3
         CUDA_TRY(ctx, cudaMemcpyAsync(ctx->req, &r, sizeof r, cudaMemcpyHostToDevice, s));
         ctx->last_req = r;
         ctx->req_valid = true;
-        CUDA_TRY(ctx, cudaGraphLaunch(ctx->exec, s));
+        CUDA_TRY(ctx, cudaGraphLaunch(ctx->step.exec, s));
         ctx->cur_len += m;
         ctx->have_token = true;
     }
@@ -965,36 +730,7 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int H = ctx->shape.hidden;
     uint16_t *fresh = nullptr;
-    StepSchedule sub;
-    const StepSchedule *ss = &ctx->sched_full;
-    std::vector<CUtensorMap> lm_maps = ctx->maps_full_lm;
-    MkOp op = ctx->lm_op_full;
-    if (n > 0 && ctx->block_tokens == 1) CUDA_TRY(ctx, cudaMalloc(&fresh, static_cast<size_t>(n) * H * sizeof(uint16_t)));
-    const StepPlan &pl = ctx->plan;
-    // tile kernel: the schedule of the step with the output layer cut down to n rows (the other operators keep their lists), its
-    // tensor maps over the gathered rows, and the operator descriptor
-    if (n > 0 && ctx->block_tokens > 1) {
-        for (int o = 0; o < 4; ++o) sub.ops[o] = ctx->sched_full.ops[o];
-        OpShape os[5];
-        op_shapes(ctx->shape, n, os);
-        if (const char *why = plan_op(os[4], 4, pl.grid, pl.nw, pl.slot_rows, &sub.ops[4]))
-            return fail(ctx, EDGEFM_ERR_BAD_SHAPE, "a subset of %d rows does not fit the tile plan of this context: %s", n, why);
-        assemble_schedule(&sub, pl.grid, pl.nw);
-        if (sub.tiles.size() > ctx->tiles_cap || sub.combines.size() > ctx->combines_cap ||
-            sub.smem_bytes() > static_cast<size_t>(ctx->mk.sched_bytes))
-            return fail(ctx, EDGEFM_ERR_BAD_SHAPE, "a subset of %d rows does not fit the tile plan of this context", n);
-        ss = &sub;
-        CUDA_TRY(ctx, cudaMalloc(&fresh, static_cast<size_t>(n) * H * sizeof(uint16_t)));
-        for (int v = 0; v < MK_MAX_VARIANTS; ++v) {
-            std::memset(&lm_maps[v], 0, sizeof(CUtensorMap));
-            if (v < sub.ops[4].n_variants && !encode_weight_map(&lm_maps[v], fresh, n, H, sub.ops[4].variant_rows[v])) {
-                cudaFree(fresh);
-                return fail(ctx, EDGEFM_ERR_CUDA, "cuTensorMapEncodeTiled failed");
-            }
-        }
-        op.units_total = n;
-        op.layer_flags = (op.layer_flags & ~0xff) | PHF_REMAP;
-    }
+    if (n > 0) CUDA_TRY(ctx, cudaMalloc(&fresh, static_cast<size_t>(n) * H * sizeof(uint16_t)));
     // steps already enqueued on the stream still read the previous subset
     cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess && n > 0) {
@@ -1008,20 +744,7 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
     }
     const uint16_t *lm_w = n > 0 ? fresh : static_cast<const uint16_t *>(ctx->lm_head);
     const StepHead head{lm_w, static_cast<const uint16_t *>(ctx->final_norm), n > 0 ? n : ctx->shape.vocab, n > 0 ? 1 : 0, {}};
-    if (ctx->block_tokens == 1) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_layers + ctx->shape.n_layers, &head, sizeof head, cudaMemcpyHostToDevice, s);
-    } else {
-    const size_t lm_index = static_cast<size_t>(ctx->mk.nph - 1);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_ops + lm_index, &op, sizeof op, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_op_w + lm_index, &lm_w, sizeof lm_w, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->d_maps + lm_index * MK_MAX_VARIANTS * sizeof(CUtensorMap), lm_maps.data(), MK_MAX_VARIANTS * sizeof(CUtensorMap),
-                            cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_tiles, ss->tiles.data(), ss->tiles.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_cta_tab, ss->cta_tab.data(), ss->cta_tab.size() * sizeof(int), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && !ss->combines.empty())
-        e = cudaMemcpyAsync(ctx->d_combines, ss->combines.data(), ss->combines.size() * sizeof(MkCombine), cudaMemcpyHostToDevice, s);
-    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_layers + ctx->shape.n_layers, &head, sizeof head, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host buffers are read before the call returns
     if (e != cudaSuccess) {
         if (fresh) cudaFree(fresh);
@@ -1042,13 +765,12 @@ edgefm_status edgefm_get_launches_per_step(const edgefm_ctx *ctx, int32_t *n) {
 
 edgefm_status edgefm_debug_profile(edgefm_ctx *ctx, uint64_t *out_host, int64_t capacity, int32_t *n_ctas, int32_t *stride) {
     if (!ctx || !n_ctas || !stride) return EDGEFM_ERR_INVALID_ARG;
-    const int grid = ctx->block_tokens == 1 ? ctx->step.grid : ctx->plan.grid;
+    const int grid = ctx->step.launch.grid;
     *n_ctas = ctx->prof ? grid : 0;
     *stride = ctx->prof_stride;
     if (!ctx->prof || !out_host) return EDGEFM_OK;
-    int64_t n = static_cast<int64_t>(grid) * ctx->prof_stride;
+    const int64_t n = static_cast<int64_t>(grid) * ctx->prof_stride;
     if (capacity < n) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "profile buffer too small");
-    if (capacity >= n + MK_NW_MAX * 16 * 4 + 8) n += MK_NW_MAX * 16 * 4 + 8;   // optional per-warp trace behind the table
     DeviceGuard guard(ctx->device);
     CUDA_TRY(ctx, cudaDeviceSynchronize());
     CUDA_TRY(ctx, cudaMemcpy(out_host, ctx->prof, static_cast<size_t>(n) * 8, cudaMemcpyDeviceToHost));
@@ -1057,15 +779,9 @@ edgefm_status edgefm_debug_profile(edgefm_ctx *ctx, uint64_t *out_host, int64_t 
 
 edgefm_status edgefm_debug_plan(const edgefm_ctx *ctx, int32_t *out8) {
     if (!ctx || !out8) return EDGEFM_ERR_INVALID_ARG;
-    if (ctx->block_tokens == 1) {
-        const StepLaunch &sl = ctx->step;
-        const int32_t v[8] = {sl.grid, ST_NW, ST_BARS, sl.max_chunk_bytes, static_cast<int32_t>(sl.dyn_smem), sl.p.ring_bytes, sl.p.table_bytes, 0};
-        std::copy(v, v + 8, out8);
-        return EDGEFM_OK;
-    }
-    const StepPlan &pl = ctx->plan;
-    out8[0] = pl.grid; out8[1] = pl.nw; out8[2] = pl.slots; out8[3] = pl.slot_bytes; out8[4] = static_cast<int32_t>(pl.dyn_smem);
-    out8[5] = ctx->sched_full.max_cta_tiles; out8[6] = static_cast<int32_t>(pl.sched_bytes); out8[7] = pl.long_ctx ? 1 : 0;
+    const StepLaunch &sl = ctx->step.launch;
+    const int32_t v[8] = {sl.grid, ST_NW, ST_BARS, sl.max_chunk_bytes, static_cast<int32_t>(sl.dyn_smem), sl.p.ring_bytes, sl.p.table_bytes, 0};
+    std::copy(v, v + 8, out8);
     return EDGEFM_OK;
 }
 
@@ -1075,11 +791,14 @@ edgefm_status edgefm_debug_set_wait_limit(edgefm_ctx *ctx, uint32_t limit_ns, in
         return fail(ctx, EDGEFM_ERR_INVALID_ARG, "limit_ns must be >= 1000 and extra_barrier_arrivals 0 or 1");
     DeviceGuard guard(ctx->device);
     CUDA_TRY(ctx, cudaDeviceSynchronize());
-    ctx->mk.spin_limit = limit_ns;
-    ctx->mk.barrier_extra = extra_barrier_arrivals;
-    ctx->step.p.spin_limit = limit_ns;
-    ctx->step.p.barrier_extra = extra_barrier_arrivals;
-    CUDA_TRY(ctx, record_graph(ctx));
+    ctx->spin_limit = limit_ns;
+    ctx->barrier_extra = extra_barrier_arrivals;
+    for (edgefm_ctx::Build *b : {&ctx->step, &ctx->wide}) {
+        if (!b->exec) continue;
+        b->launch.p.spin_limit = limit_ns;
+        b->launch.p.barrier_extra = extra_barrier_arrivals;
+        CUDA_TRY(ctx, record_graph(ctx, b));
+    }
     ctx->err.clear();
     return EDGEFM_OK;
 }
@@ -1230,7 +949,7 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     }
     // ---- the same plan edgefm_create makes, in host memory -------------------------------------------------
     StepLaunch sl;
-    if (const char *why = step_plan(sh, max_context, num_sms, smem_optin, false, &sl)) return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "%s", why);
+    if (const char *why = step_plan(sh, max_context, num_sms, smem_optin, false, 1, &sl)) return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "%s", why);
 
     // carve the scratch array; reject shapes that need more than it holds
     ScratchCarver sc{g_scratch_dev_ptr[dev]};
@@ -1245,7 +964,7 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     std::vector<StepLayer> layers(static_cast<size_t>(sh.n_layers) + 1);
     step_layers(sh, weights->layers, weights->final_norm, weights->lm_head, layers.data());
     CUDA_TRY(nullptr, allow_max_dynamic_smem(sl.kernel, smem_optin));
-    step_wire(&sl, ll);
+    step_wire(&sl, 1, ll);
     StepParams &p = sl.p;
     p.k_cache = static_cast<uint16_t *>(k_cache); p.v_cache = static_cast<uint16_t *>(v_cache);
     p.embed = static_cast<const uint16_t *>(weights->embed); p.inv_freq = inv_freq; p.layers = d_layers;
@@ -1264,7 +983,7 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     CUDA_TRY(nullptr, cudaMemcpyAsync(inv_freq, inv, static_cast<size_t>(d / 2) * sizeof(double), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(state, &st, sizeof st, cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(req, &rq, sizeof rq, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(nullptr, launch_step(sl.kernel, sl.grid, ST_THREADS, sl.dyn_smem, p, s));
+    CUDA_TRY(nullptr, launch_step(sl, s));
     g_static_state[dev] = state;
     g_create_error.clear();
     return EDGEFM_OK;

@@ -145,38 +145,41 @@ struct WarpAttention {
     }
 };
 
-// Shared-memory scratch of the attention, in floats from Ctx::scratch(): queries | new k, v row (as cached) and its scales |
-// probabilities | warp maxima, denominators, outputs | scales of the warps' rows (compressed cache).
-template <int D, int G> struct AttScratch {
-    static constexpr int QS = 0, NEW = QS + G * D, NSC = NEW + D, PW = NSC + 8, MM = PW + ST_NW * 64, ML = MM + ST_NW * 8, MO = ML + ST_NW * 8,
-                         SC = MO + ST_NW * G * D, FLOATS = SC + 2 * ST_KV_BLOCK;
+// Shared-memory scratch of the attention, in floats: queries | new k rows, new v rows (as cached), their scales | probabilities | warp
+// maxima, denominators, outputs | scales of the warps' rows (compressed cache).  The fp32 new rows share the place of the warp outputs.
+template <int D, int G, int MT> struct AttScratch {
+    static constexpr int QS = 0, NEW = QS + G * D, NSC = NEW + MT * D, PW = NSC + 16, MM = PW + ST_NW * 64, ML = MM + ST_NW * 8, MO = ML + ST_NW * 8,
+                         RAW = 2 * MT * D, SC = MO + (ST_NW * G * D > RAW ? ST_NW * G * D : RAW), FLOATS = SC + 2 * ST_KV_BLOCK;
 };
 
-template <int D, int G, bool Q8>
-__device__ __forceinline__ bool attend(Ctx &c, int layer, unsigned tag) {
-    using A = AttScratch<D, G>;
+// Token share.tok, kv head share.g, the chunk [t0, t1) of the old positions; the last chunk also attends to the rows of the call's tokens
+// 0 .. tok, which travel as packets.
+template <int D, int G, bool Q8, int MT>
+__device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &share, unsigned tag) {
+    using A = AttScratch<D, G, MT>;
     using W = WarpAttention<D, G, Q8>;
     const StepParams &p = c.p();
-    const KvShare &share = c.sh().share;
-    float *base = c.scratch();
+    float *base = reinterpret_cast<float *>(c.area());
     constexpr int half = D / 2;
-    const int n_units = (p.nq + 2 * p.nkv) * half;
+    const int n_units = (p.nq + 2 * p.nkv) * half, n_new = share.tail ? share.tok + 1 : 0;
     bool ok = true;
-    // queries of the group (and, in the CTA that ends with the new position, the new k and v rows): one row pair per packet pair
-    const int q_units = G * half, mine = q_units + (share.tail ? 2 * half : 0);
-    constexpr int U = ((G + 2) * half + ST_NT - 1) / ST_NT;   // in flight per thread
-    {
+    // queries of the group, then the new k and v rows: one row pair per packet pair
+    constexpr int q_units = G * half, U = 3;                  // in flight per thread
+    const int mine = q_units + n_new * 2 * half;
+#pragma unroll 1
+    for (int j0 = c.tid; j0 < mine; j0 += U * ST_NT) {
         Two t[U];
         const unsigned long long *at[U];
         unsigned todo = 0;
 #pragma unroll
         for (int i = 0; i < U; ++i) {
-            const int j = c.tid + i * ST_NT, kv = j - q_units;
+            const int j = j0 + i * ST_NT, kv = j - q_units;
             at[i] = p.q_ll;
             if (j < mine) {
-                const int unit = kv < 0 ? share.g * G * half + j : (kv < half ? (p.nq + share.g) * half + kv : (p.nq + p.nkv + share.g) * half + kv - half);
-                const int w = ((unit + 1) * c.ncta - 1) / n_units;      // its writer: the CTA c with first(c) <= unit < first(c + 1)
-                at[i] = p.q_ll + static_cast<size_t>(w) * p.q_line + 2 * (unit - st_first(n_units, w, c.ncta));
+                const int row = kv < 0 ? share.g * G * half + j : (kv & half) ? (p.nq + p.nkv + share.g) * half + (kv & (half - 1)) : (p.nq + share.g) * half + (kv & (half - 1));
+                const int tok = kv < 0 ? share.tok : kv / (2 * half);
+                const int w = ((row + 1) * c.ncta - 1) / n_units;      // its writer: the CTA c with first(c) <= row < first(c + 1)
+                at[i] = p.q_ll + (static_cast<size_t>(tok) * c.ncta + w) * p.q_line + 2 * (row - st_first(n_units, w, c.ncta));
                 todo |= 1u << i;
             }
         }
@@ -191,32 +194,37 @@ __device__ __forceinline__ bool attend(Ctx &c, int layer, unsigned tag) {
                 if ((todo >> i & 1u) && both(t[i], tag)) todo &= ~(1u << i);
             if (todo && !sp.again(c.abort(), p.spin_limit)) { ok = false; break; }
         }
+        if (!ok) break;
 #pragma unroll
         for (int i = 0; i < U; ++i)
             if (all >> i & 1u) {
-                const int j = c.tid + i * ST_NT, kv = j - q_units;
+                const int j = j0 + i * ST_NT, kv = j - q_units;
                 const float lo = packet_value(t[i].a), hi = packet_value(t[i].b);
                 if (kv < 0) {
                     float *d = base + A::QS + (j / half) * D + (j & (half - 1));
                     d[0] = lo * p.q_scale;
                     d[half] = hi * p.q_scale;
-                } else if constexpr (Q8) {      // fp32 for the compression below (the two rows share the place of the probabilities)
-                    float *d = base + A::PW + (kv < half ? 0 : D) + (kv & (half - 1));
-                    d[0] = lo;
-                    d[half] = hi;
                 } else {
-                    uint16_t *d = reinterpret_cast<uint16_t *>(base + A::NEW) + (kv < half ? 0 : D) + (kv & (half - 1));
-                    d[0] = f32_to_bf16_bits(lo);
-                    d[half] = f32_to_bf16_bits(hi);
+                    const int at_row = ((kv & half) ? n_new : 0) + kv / (2 * half);       // k rows, then v rows
+                    if constexpr (Q8) {          // fp32 for the compression below
+                        float *d = base + A::MO + at_row * D + (kv & (half - 1));
+                        d[0] = lo;
+                        d[half] = hi;
+                    } else {
+                        uint16_t *d = reinterpret_cast<uint16_t *>(base + A::NEW) + at_row * D + (kv & (half - 1));
+                        d[0] = f32_to_bf16_bits(lo);
+                        d[half] = f32_to_bf16_bits(hi);
+                    }
                 }
             }
     }
     if (!cta_vote(ok)) return false;
     if constexpr (Q8) {
-        if (share.tail) {               // compress the new row: warp 0 k, warp 1 v; into the cache and into shared memory
-            if (c.warp < 2) {
+        if (n_new > 0) {                // compress the new rows, a warp per row; the last one (this token's own) also goes to the cache
+#pragma unroll 1
+            for (int r = c.warp; r < 2 * n_new; r += ST_NW) {
                 constexpr int DV = D / 32;
-                const float *src = base + A::PW + c.warp * D + c.lane * DV;
+                const float *src = base + A::MO + r * D + c.lane * DV;
                 float xv[DV], amax = 0.f;
 #pragma unroll
                 for (int e = 0; e < DV; ++e) { xv[e] = src[e]; amax = fmaxf(amax, fabsf(xv[e])); }
@@ -228,13 +236,15 @@ __device__ __forceinline__ bool attend(Ctx &c, int layer, unsigned tag) {
                     const float q = fminf(fmaxf(rintf(__fmul_rn(xv[e], inv)), -127.f), 127.f);
                     packed |= (static_cast<uint32_t>(static_cast<int>(q)) & 0xffu) << (8 * e);
                 }
-                const size_t row = (static_cast<size_t>(layer) * p.nkv + share.g) * p.max_context + c.sh().n_old;
-                unsigned char *dst = reinterpret_cast<unsigned char *>(c.warp == 0 ? p.k_cache : p.v_cache) + row * D + c.lane * DV;
-                unsigned char *own = reinterpret_cast<unsigned char *>(base + A::NEW) + c.warp * D + c.lane * DV;
-                if constexpr (DV == 4) { *reinterpret_cast<uint32_t *>(dst) = packed; *reinterpret_cast<uint32_t *>(own) = packed; }
-                else { *reinterpret_cast<uint16_t *>(dst) = static_cast<uint16_t>(packed); *reinterpret_cast<uint16_t *>(own) = static_cast<uint16_t>(packed); }
                 const float sc = amax > 0.f ? __fdiv_rn(amax, 127.0f) : 0.f;
-                if (c.lane == 0) { (c.warp == 0 ? p.k_scale : p.v_scale)[row] = sc; base[A::NSC + c.warp] = sc; }
+                const bool is_v = r >= n_new;
+                const int k = is_v ? r - n_new : r;
+                unsigned char *own = reinterpret_cast<unsigned char *>(base + A::NEW) + r * D + c.lane * DV;
+                const size_t row = (static_cast<size_t>(layer) * p.nkv + share.g) * p.max_context + c.sh().n_old + k;
+                unsigned char *dst = reinterpret_cast<unsigned char *>(is_v ? p.v_cache : p.k_cache) + row * D + c.lane * DV;
+                if constexpr (DV == 4) { *reinterpret_cast<uint32_t *>(own) = packed; if (k == share.tok) *reinterpret_cast<uint32_t *>(dst) = packed; }
+                else { *reinterpret_cast<uint16_t *>(own) = static_cast<uint16_t>(packed); if (k == share.tok) *reinterpret_cast<uint16_t *>(dst) = static_cast<uint16_t>(packed); }
+                if (c.lane == 0) { base[A::NSC + (is_v ? 8 : 0) + k] = sc; if (k == share.tok) (is_v ? p.v_scale : p.k_scale)[row] = sc; }
             }
             if (!cta_vote(true)) return false;
         }
@@ -242,19 +252,19 @@ __device__ __forceinline__ bool attend(Ctx &c, int layer, unsigned tag) {
     W att;
     att.start(base + A::QS, c.lane);
     float *pw = base + A::PW + c.warp * 64;
-    // (the new row comes last, alone, by the last warp of the CTA that ends with it)
+    // (the new rows come last, by the last warp of the CTA that ends with them)
 #pragma unroll 1
     for (int t = share.t0;; t += ST_KV_BLOCK) {
         const bool fresh = t >= share.t1;
-        if (fresh && !share.tail) break;
-        const int n = fresh ? 1 : min(ST_KV_BLOCK, share.t1 - t);
+        if (fresh && n_new == 0) break;
+        const int n = fresh ? n_new : min(ST_KV_BLOCK, share.t1 - t);
         const int steps = (n + W::SP - 1) / W::SP, per_warp = (steps + ST_NW - 1) / ST_NW * W::SP;   // positions of a warp, whole steps
         int first = c.warp * per_warp, cnt = min(per_warp, n - first);
-        const float *ksc = base + A::NSC, *vsc = ksc + 1;
+        const float *ksc = base + A::NSC, *vsc = ksc + 8;
         const unsigned char *at = reinterpret_cast<const unsigned char *>(base + A::NEW);
         if (fresh) {
             first = 0;
-            cnt = c.warp == ST_NW - 1 ? 1 : 0;
+            cnt = c.warp == ST_NW - 1 ? n : 0;
         } else {
             if constexpr (Q8) {         // every warp fetches the scales of its own positions
                 float *own = base + A::SC + c.warp * 16;
@@ -273,6 +283,7 @@ __device__ __forceinline__ bool attend(Ctx &c, int layer, unsigned tag) {
     att.leave(base + A::MM, base + A::ML, base + A::MO, c.warp, c.lane);
     if (!cta_vote(ok)) return false;
     // merge the warps and publish: one pair of dims per thread
+    const size_t slot = static_cast<size_t>(share.tok) * c.sh().n_chunks + share.chunk;
 #pragma unroll 1
     for (int j = c.tid; j < G * half; j += ST_NT) {
         const int h = j / half, d2 = j - h * half;
@@ -287,8 +298,7 @@ __device__ __forceinline__ bool attend(Ctx &c, int layer, unsigned tag) {
             a = fmaf(v.x, e, a);
             b = fmaf(v.y, e, b);
         }
-        const size_t at = static_cast<size_t>(share.chunk) * p.nq + share.g * G + h;
-        put2(p.part_ll + at * D + 2 * d2, a, b, tag);
+        put2(p.part_ll + slot * p.qd + (share.g * G + h) * D + 2 * d2, a, b, tag);
     }
     if (c.tid < G) {                    // maximum and denominator of every head, one store
         float mm = -INFINITY, ll = 0.f;
@@ -296,36 +306,39 @@ __device__ __forceinline__ bool attend(Ctx &c, int layer, unsigned tag) {
         for (int w = 0; w < ST_NW; ++w) mm = fmaxf(mm, base[A::MM + w * 8 + c.tid]);
 #pragma unroll
         for (int w = 0; w < ST_NW; ++w) ll = fmaf(base[A::ML + w * 8 + c.tid], exp2_approx(base[A::MM + w * 8 + c.tid] - mm), ll);
-        put2(p.stat_ll + (static_cast<size_t>(share.chunk) * p.nq + share.g * G + c.tid) * 2, mm, ll, tag);
+        put2(p.stat_ll + (slot * p.nq + share.g * G + c.tid) * 2, mm, ll, tag);
     }
     return true;
 }
-// The owner of an output pair merges its chunks: one warp per pair, lanes over chunks, in a fixed order.
-__device__ __forceinline__ bool merge_chunks(Ctx &c, unsigned tag) {
+// The owner of an output pair merges its chunks, in a fixed order: LP lanes per (token, pair), lanes over chunks.
+template <int MT>
+__device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag, unsigned real_tag) {
     constexpr int NJ = 3;                // chunks per lane in flight
     const StepParams &p = c.p();
-    const int n_chunks = c.sh().share.n_chunks;
-    const int pairs = p.qd / 2, a0 = st_first(pairs, c.cta, c.ncta), a1 = st_first(pairs, c.cta + 1, c.ncta);
-    float *const out = c.sh().merged;
+    const int n_chunks = c.sh().n_chunks, m = c.sh().m;
+    const int pairs = p.qd / 2, a0 = st_first(pairs, c.cta, c.ncta), n_pairs = st_first(pairs, c.cta + 1, c.ncta) - a0;
+    const int lp = MT == 1 || n_chunks > 16 ? 32 : n_chunks > 8 ? 16 : 8, sub = c.lane & (lp - 1), per_warp = 32 / lp;
     bool ok = true;
 #pragma unroll 1
-    for (int pr = a0 + c.warp; pr < a1; pr += ST_NW) {
-        const int h = 2 * pr / p.D;
-        float m = -INFINITY, l = 0.f, a = 0.f, b = 0.f;      // of this lane's chunks
+    for (int it = c.warp * per_warp; it < n_pairs * m && ok; it += ST_NW * per_warp) {
+        const int item = it + c.lane / lp;
+        const bool on = item < n_pairs * m;
+        const int tok = on ? item / n_pairs : 0, k_pair = on ? item - tok * n_pairs : 0, pr = a0 + k_pair, h = 2 * pr / p.D;
+        float mx = -INFINITY, l = 0.f, a = 0.f, b = 0.f;      // of this lane's chunks
 #pragma unroll 1
-        for (int k0 = c.lane; k0 < n_chunks; k0 += 32 * NJ) {
+        for (int k0 = sub; k0 < n_chunks && on; k0 += lp * NJ) {
             Two st[NJ], ov[NJ];
             unsigned todo = 0;
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
-                if (k0 + 32 * j < n_chunks) todo |= 1u << j;
+                if (k0 + lp * j < n_chunks) todo |= 1u << j;
             const unsigned mine = todo;
             Spin sp;
             while (todo) {
 #pragma unroll
                 for (int j = 0; j < NJ; ++j)
                     if (todo >> j & 1u) {
-                        const size_t k = static_cast<size_t>(k0 + 32 * j);
+                        const size_t k = static_cast<size_t>(tok) * n_chunks + k0 + lp * j;
                         st[j] = get2(p.stat_ll + (k * p.nq + h) * 2);
                         ov[j] = get2(p.part_ll + k * p.qd + 2 * pr);
                     }
@@ -335,13 +348,13 @@ __device__ __forceinline__ bool merge_chunks(Ctx &c, unsigned tag) {
                 if (todo && !sp.again(c.abort(), p.spin_limit)) break;
             }
             if (todo) { ok = false; break; }
-            float mn = m;
+            float mn = mx;
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
                 if (mine >> j & 1u) mn = fmaxf(mn, packet_value(st[j].a));
-            const float f = m == -INFINITY ? 0.f : exp2_approx(m - mn);
+            const float f = mx == -INFINITY ? 0.f : exp2_approx(mx - mn);
             l *= f; a *= f; b *= f;
-            m = mn;
+            mx = mn;
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
                 if (mine >> j & 1u) {
@@ -351,19 +364,25 @@ __device__ __forceinline__ bool merge_chunks(Ctx &c, unsigned tag) {
                     b = fmaf(packet_value(ov[j].b), e, b);
                 }
         }
-        const float mm = warp_max(m), f = m == -INFINITY ? 0.f : exp2_approx(m - mm);
-        l = warp_sum(l * f);
-        a = warp_sum(a * f);
-        b = warp_sum(b * f);
         ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        if (c.lane == 0) *reinterpret_cast<float2 *>(out + 2 * (pr - a0)) = make_float2(a / l, b / l);
+        float mm = mx;
+        for (int k = lp >> 1; k; k >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, k));
+        const float f = mx == -INFINITY ? 0.f : exp2_approx(mx - mm);
+        l *= f; a *= f; b *= f;
+        for (int k = lp >> 1; k; k >>= 1) {
+            l += __shfl_xor_sync(0xffffffffu, l, k);
+            a += __shfl_xor_sync(0xffffffffu, a, k);
+            b += __shfl_xor_sync(0xffffffffu, b, k);
+        }
+        if (on && sub == 0) *reinterpret_cast<float2 *>(&c.sh().merged[tok][2 * k_pair]) = make_float2(a / l, b / l);
     }
     // a line is written by one instruction: every further write invalidates the pollers' copies of it (+ 1.5 us)
     if (!cta_vote(ok)) return false;
-    if (c.tid < a1 - a0) {
-        const float2 v = *reinterpret_cast<const float2 *>(out + 2 * c.tid);
-        put2(p.ao_ll + static_cast<size_t>(c.cta) * p.ao_line + 2 * c.tid, v.x, v.y, tag);
+#pragma unroll 1
+    for (int i = c.tid; i < n_pairs * MT; i += ST_NT) {        // (unused tokens too: their slots keep up with the tags)
+        const int tok = i / n_pairs, k = i - tok * n_pairs;
+        const float2 v = tok < m ? *reinterpret_cast<const float2 *>(&c.sh().merged[tok][2 * k]) : make_float2(0.f, 0.f);
+        put_raw2(p.ao_ll + (static_cast<size_t>(tok) * c.ncta + c.cta) * p.ao_line + 2 * k, pieces_packet(v.x, real_tag), pieces_packet(v.y, real_tag));
     }
     return true;
 }

@@ -1,0 +1,4 @@
+#include "step_kernel.cuh"
+namespace edgefm {
+StepKernel step_d64_m1(int G) { return step::kernel_for<64, false, 1>(G); }
+}  // namespace edgefm

@@ -9,22 +9,26 @@
 //     QKV rows, this CTA's K/V cache rows, O rows, gate/up rows, down rows, next layer, ..., output layer -- independent of the
 //     computation; another asks L2 for what comes after the ring.  (A bulk copy costs its issuer the same few hundred cycles
 //     whatever its size: measured from L2, 6 / 24 / 48 KB copies from one such loop reached 2.2 / 9 / 18 TB/s over the chip.)
-//   * Products (step_products.cuh).  All 8 consumer warps work on every row; warp w multiplies columns [K w / 8, K (w + 1) / 8) with
-//     its slice of the input vector, fp32.  bf16 weights become fp32 by a shift or a mask, products and sums are packed fp32
-//     FMAs.  Row sums: shuffles over the lanes of a row (several rows folded at once), then the 8 partial sums of a row meet in
-//     shared memory and one thread per output unit runs the fused epilogue (bias + RoPE + cache row, residual add, SwiGLU,
-//     logits + argmax).
-//   * Exchanges.  A value travels as an 8-byte packet {fp32 value, tag}; the tag names step and layer, so a reader polls the data
-//     itself: one trip to L2 instead of store, fence, counter, poll, load.  Every CTA writes its values into a 128-byte line of
-//     its own (packets of several writers in one line cost 0.3 - 1 us: the pollers' copies of the line are invalidated by every
+//   * Products (step_products.cuh).  All 8 consumer warps work on every tile of 16 rows (or 8 row pairs); warp w multiplies its share of
+//     the columns on the tensor cores, mma.m16n8k16 as a dot-product unit: the activations enter as bf16 pieces (three for one or
+//     two tokens, two for more), one B column per piece and token, so that a block of tokens costs the weights' traffic and the
+//     instructions of one.  The 8 partial sums of a row meet in shared memory and one thread per output unit and token runs the
+//     fused epilogue (bias + RoPE + cache row, residual add, SwiGLU, logits + argmax).
+//   * Exchanges.  A value travels as an 8-byte packet with a tag that names step and layer, so a reader polls the data itself: one
+//     trip to L2 instead of store, fence, counter, poll, load.  Vectors that are multiplied next travel as their bf16 pieces, split
+//     (and weighted for the norm) once by the owner instead of by every reader.  Every CTA writes its values into a 128-byte line
+//     of its own (packets of several writers in one line cost 0.3 - 1 us: the pollers' copies of the line are invalidated by every
 //     write).  Measured, 148 CTAs, 1536 values everywhere: 1.3 us per round, against 1.7 us for a counter barrier and a read
 //     (which leaves out the staging of the vector).  A buffer is rewritten one layer later; a CTA that writes it then has
 //     read, in between, an exchange to which every CTA contributes only after reading the old contents.
-//   * Attention (step_attention.cuh).  CTA (kv head, chunk) holds the chunk's K/V rows in its ring before the queries exist, serves
-//     the whole GQA group from one read, and publishes unnormalised partial results; the owner of an output pair merges them
-//     (one warp per pair, lanes over chunks) and publishes the finished vector.  The row this step appends travels as packets too.
+//   * Attention (step_attention.cuh).  CTA (token, kv head, chunk) holds the chunk's K/V rows in its ring before the queries exist,
+//     serves the whole GQA group from one read, and publishes unnormalised partial results; the owner of an output pair merges
+//     them (lanes over chunks) and publishes the finished vector.  The rows this call appends travel as packets too.
+//   * Several tokens (Sec. 3.11 of the paper: the base model verifies a proposed block): tokens[0] and the proposed continuation pass
+//     through the step together, at consecutive positions and cache slots; CTA 0 accepts the longest prefix that greedy decoding
+//     would have produced.
 //
-// Every wait is bounded: on expiry the CTA records status 6, all its warps leave at the next CTA-wide vote, the feeding thread
+// Every wait is bounded: on expiry the CTA records status 6, all its warps leave at the next CTA-wide vote, the feeding warp
 // waits (bounded) for its copies in flight.
 #include "step_attention.cuh"
 #include "step_feed.cuh"
@@ -33,50 +37,43 @@
 namespace edgefm {
 namespace step {
 
-// The epilogue of output unit j (its row sum, or the sums of its two rows) of an operator.
-template <int D, bool Q8>
-__device__ __forceinline__ void finish_unit(const Ctx &c, int op, int layer, int j, int u0, float lo, float hi, float add_lo, float add_hi, float &best_v,
+// The epilogue of output unit j of token `tok` (its row sum, or the sums of its two rows) of the QKV, gate/up and output layer operators.
+template <int D, bool Q8, int MT>
+__device__ __forceinline__ void finish_unit(const Ctx<MT> &c, int op, int layer, int tok, int j, int u0, float lo, float hi, float add_lo, float add_hi, float &best_v,
                                             int &best_i) {
-    const Shared &sh = c.sh();
+    const Shared<MT> &sh = c.sh();
     const StepParams &p = c.p();
     constexpr int half = D / 2;
     const unsigned tag = sh.tag0 + static_cast<unsigned>(layer);
-    if (op != ST_O && op != ST_DN) {       // the deferred RMSNorm factor
-        float tot = 0.f;
-#pragma unroll
-        for (int w = 0; w < ST_NW; ++w) tot += sh.ss[w];
-        const float r = rsqrtf(tot / static_cast<float>(p.H) + p.eps);
-        lo *= r;
-        hi *= r;
-    }
     if (op == ST_QKV) {
         const int head = j >> p.half_shift, i = j & (half - 1);
         lo += add_lo;
         hi += add_hi;
         if (head < p.nq + p.nkv) {
-            const float cs = sh.rope[i], sn = sh.rope[half + i];
+            const float cs = sh.rope[tok][i], sn = sh.rope[tok][half + i];
             const float a = lo * cs - hi * sn, b = hi * cs + lo * sn;
             lo = a;
             hi = b;
         }
-        put2(p.q_ll + static_cast<size_t>(c.cta) * p.q_line + 2 * (j - u0), lo, hi, tag);
-        if (!Q8 && head >= p.nq) {
+        put2(p.q_ll + (static_cast<size_t>(tok) * c.ncta + c.cta) * p.q_line + 2 * (j - u0), lo, hi, tag);
+        if (!Q8 && head >= p.nq && tok < sh.m) {
             const bool is_v = head >= p.nq + p.nkv;
             const int g = head - p.nq - (is_v ? p.nkv : 0);
-            uint16_t *d = (is_v ? p.v_cache : p.k_cache) + ((static_cast<size_t>(layer) * p.nkv + g) * p.max_context + sh.n_old) * D + i;
+            uint16_t *d = (is_v ? p.v_cache : p.k_cache) + ((static_cast<size_t>(layer) * p.nkv + g) * p.max_context + sh.n_old + tok) * D + i;
             d[0] = f32_to_bf16_bits(lo);
             d[half] = f32_to_bf16_bits(hi);
         }
     } else if (op == ST_GU) {
-        put1(p.act_ll + j, lo / (1.f + expf(-lo)) * hi, tag);
-    } else if (op == ST_LM) {
+        put_raw(p.act_ll + static_cast<size_t>(tok) * p.act_len + j, pieces_packet(lo / (1.f + expf(-lo)) * hi, tag));
+    } else if (tok < sh.m) {
         float *logits = p.req->logits_out;
-        if (logits) logits[j] = lo;
+        if (logits) logits[static_cast<size_t>(tok) * c.head().rows + j] = lo;
         if (arg_better(lo, j, best_v, best_i)) { best_v = lo; best_i = j; }
-    } else {
-        const float resid = c.resid()[j - u0] += lo;
-        put1((op == ST_O ? p.xo_ll : p.x_ll) + static_cast<size_t>(c.cta) * p.x_line + (j - u0), resid, tag);
     }
+}
+__device__ __forceinline__ float sum8(const float *at) {
+    const float4 a = *reinterpret_cast<const float4 *>(at), b = *reinterpret_cast<const float4 *>(at + 4);
+    return ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
 }
 
 __device__ __forceinline__ void arg_fold(float &v, int &i) {
@@ -88,13 +85,13 @@ __device__ __forceinline__ void arg_fold(float &v, int &i) {
     }
 }
 
-template <int D, int G, bool Q8>
+template <int D, int G, bool Q8, int MT>
 __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_constant__ StepParams p) {
-    Ctx c(p);
+    Ctx<MT> c(p);
     {
-        Shared &sh = c.sh();
+        Shared<MT> &sh = c.sh();
         const uint4 *src = reinterpret_cast<const uint4 *>(p.layers);
-        uint4 *dst = reinterpret_cast<uint4 *>(st_smem + ST_SHARED_BYTES + p.ring_bytes);
+        uint4 *dst = reinterpret_cast<uint4 *>(st_smem + st_shared_bytes<MT>() + p.ring_bytes);
         for (int i = c.tid; i < (p.n_layers + 1) * 4; i += ST_THREADS) dst[i] = src[i];
         if (c.tid == 0) {
             for (int i = 0; i < ST_BARS; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], ST_NW); }
@@ -102,19 +99,24 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.sent = 0u;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             const int rt = p.req->token, rp = p.req->position;
-            sh.token = rt >= 0 ? rt : p.state->next_token;
+            sh.m = MT > 1 ? min(max(p.req->m, 1), MT) : 1;
+            sh.tokens[0] = rt >= 0 ? rt : p.state->next_token;
+            for (int t = 1; t < MT; ++t) sh.tokens[t] = t < sh.m ? p.req->draft[t - 1] : 0;
             sh.pos = rp >= 0 ? rp : p.state->next_position;
             sh.n_old = p.state->cur_len;
-            sh.tag0 = static_cast<unsigned>(p.state->reserved[0]) * static_cast<unsigned>(p.n_layers + 2) + 1u;
-            sh.odd = static_cast<unsigned>(p.barrier_extra) << 31;
+            sh.n_chunks = kv_chunks(p, sh.n_old, sh.m, c.ncta);
+            sh.tag0 = static_cast<unsigned>(p.state->epoch[p.epoch_slot]) * static_cast<unsigned>(p.n_layers + 2) + 1u;
+            sh.odd = static_cast<unsigned>(p.barrier_extra) << 31 | static_cast<unsigned>(p.barrier_extra) << 15;
             sh.total_x = c.ncta * line_units(p.H, c.ncta, 1);
             sh.total_a = c.ncta * line_units(p.qd, c.ncta, 2);
         }
         __syncthreads();
         const int lm_rows = c.head().rows;
+        bool sane = true;
+        for (int t = 0; t < MT; ++t) sane = sane && sh.tokens[t] >= 0 && sh.tokens[t] < p.V;
         // a corrupt request or state: compute nothing
-        if (sh.token < 0 || sh.token >= p.V || sh.n_old < 0 || sh.n_old >= p.max_context || sh.pos < 0 || lm_rows < 1 || lm_rows > p.V) {
-            if (c.tid == 0 && atomicCAS(&p.state->status, 0, 103) == 0) { p.state->pad[0] = sh.token; p.state->pad[1] = sh.n_old; }
+        if (!sane || sh.n_old < 0 || sh.n_old + sh.m > p.max_context || sh.pos < 0 || lm_rows < 1 || lm_rows > p.V) {
+            if (c.tid == 0 && atomicCAS(&p.state->status, 0, 103) == 0) { p.state->pad[0] = sh.tokens[0]; p.state->pad[1] = sh.n_old; }
             return;
         }
         if (c.tid < 5) {
@@ -122,17 +124,16 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.u0[c.tid] = st_first(n, c.cta, c.ncta);
             sh.u1[c.tid] = st_first(n, c.cta + 1, c.ncta);
         }
-        if (c.tid == 32) sh.share = kv_share(p, sh.n_old, c.cta, c.ncta);
         __syncthreads();                 // the last sync of all threads
     }
     if (c.warp >= ST_NW) {               // the feeding warpgroup: gives its registers to the others
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ST_REGS_FEED));
-        if (c.warp == ST_NW && c.lane == 0) feed_ring<Q8>(c);
-        if (c.warp == ST_NW + 1 && c.lane == 0) feed_l2<Q8>(c);
+        if (c.warp == ST_NW) feed_ring<Q8, MT>(c);
+        if (c.warp == ST_NW + 1) feed_l2<Q8, MT>(c);
         return;
     }
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ST_REGS));
-    constexpr int half = D / 2;
+    constexpr int half = D / 2, RB = Ctx<MT>::RB, RB_LOG2 = RB == 128 ? 7 : RB == 64 ? 6 : 5;
     int prof_idx = 0;
     stamp(c, prof_idx);
     // The small per-layer vectors are read on the critical path right behind an exchange: ask L2 for all of them now (they stay, the
@@ -149,20 +150,23 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             if (v) asm volatile("prefetch.global.L2 [%0];" ::"l"(v));
         }
     }
+    const int x0 = c.sh().u0[ST_DN], my_rows = c.sh().u1[ST_DN] - x0;      // rows of the residual stream this CTA owns
     {
-        Shared &sh = c.sh();
-        for (int i = c.tid; i < half; i += ST_NT) {        // rotary table of the step's position; fp64 angle, rounded once
+        Shared<MT> &sh = c.sh();
+        for (int i = c.tid; i < sh.m * half; i += ST_NT) {        // rotary tables of the tokens' positions; fp64 angle, rounded once
+            const int t = i / half, f = i - t * half;
             double sn, cs;
-            sincos(static_cast<double>(sh.pos) * p.inv_freq[i], &sn, &cs);
-            sh.rope[i] = static_cast<float>(cs);
-            sh.rope[half + i] = static_cast<float>(sn);
+            sincos(static_cast<double>(sh.pos + t) * p.inv_freq[f], &sn, &cs);
+            sh.rope[t][f] = static_cast<float>(cs);
+            sh.rope[t][half + f] = static_cast<float>(sn);
         }
-        if (c.cta == 0 && c.tid == 0) { p.state->token = sh.token; p.state->position = sh.pos; }
+        if (c.cta == 0 && c.tid == 0) { p.state->token = sh.tokens[0]; p.state->position = sh.pos; }
         make_table(c, c.unit_table(), p.H, 1, p.x_line);
         make_table(c, c.unit_table() + sh.total_x, p.qd, 2, p.ao_line);
-        const uint16_t *erow = p.embed + static_cast<size_t>(sh.token) * p.H;
-        const int x0 = sh.u0[ST_DN], x1 = sh.u1[ST_DN];
-        for (int i = c.tid; i < x1 - x0; i += ST_NT) c.resid()[i] = bf16_bits_to_f32(erow[x0 + i]);
+        for (int i = c.tid; i < MT * my_rows; i += ST_NT) {
+            const int t = i / my_rows;
+            c.resid()[i] = bf16_bits_to_f32(p.embed[static_cast<size_t>(sh.tokens[t]) * p.H + x0 + i - t * my_rows]);
+        }
     }
     float best_v = -INFINITY;
     int best_i = 0x7fffffff;
@@ -177,16 +181,20 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         asm volatile("" : "+r"(op), "+r"(c.tid), "+r"(c.cta), "+r"(c.ncta));
         c.warp = c.tid >> 5;
         c.lane = c.tid & 31;
-        Shared &sh = c.sh();
-        const unsigned tag = (sh.tag0 + static_cast<unsigned>(layer)) ^ sh.odd;      // what this layer's packets are expected to carry
+        Shared<MT> &sh = c.sh();
+        const unsigned real_tag = sh.tag0 + static_cast<unsigned>(layer), tag = real_tag ^ sh.odd;      // what this layer's packets carry / are expected to carry
         const StepLayer *L = c.layer(layer);
         // -- the input vector --
         if (op == ST_O) {
             stamp(c, prof_idx);
-            if (sh.share.any) ok = attend<D, G, Q8>(c, layer, tag);
+#pragma unroll 1
+            for (int idx = c.cta; idx < sh.m * p.nkv * sh.n_chunks && ok; idx += c.ncta) {
+                ok = attend<D, G, Q8, MT>(c, layer, kv_share(p, sh.n_old, sh.n_chunks, idx), tag);
+                if (ok && idx + c.ncta < sh.m * p.nkv * sh.n_chunks) ok = cta_vote(true);
+            }
             if (!ok) break;
             stamp(c, prof_idx);                       // chunk done
-            ok = merge_chunks(c, tag);
+            ok = merge_chunks(c, tag, real_tag);
             if (!ok) break;
             stamp(c, prof_idx);                       // partial results merged
         }
@@ -194,103 +202,141 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             ok = stage_embedding(c, L->input_norm);
         } else if (op != ST_DN) {                     // (one call for the three exchanges: the loop's code has to stay small)
             const bool ao = op == ST_O, gu = op == ST_GU;
-            ok = stage_lines(c, c.unit_table() + (ao ? sh.total_x : 0), ao ? sh.total_a : sh.total_x, (ao ? p.qd : p.H) / 8, ao ? p.ao_ll : gu ? p.xo_ll : p.x_ll,
-                             ao ? nullptr : gu ? L->post_norm : op == ST_QKV ? L->input_norm : c.head().final_norm,
-                             ao || gu ? tag : (sh.tag0 + static_cast<unsigned>(layer) - 1u) ^ sh.odd);
+            ok = stage_lines(c, c.unit_table() + (ao ? sh.total_x : 0), ao ? sh.total_a : sh.total_x, ao ? p.qd : p.H, ao ? p.ao_ll : gu ? p.xo_ll : p.x_ll,
+                             ao ? p.ao_line : p.x_line, !ao, ao || gu ? tag : (real_tag - 1u) ^ sh.odd);
         }
         if (!ok) break;
-        if (op == ST_DN) ok = stage_slice(c, p.act_ll, tag);       // (of this warp; the vote follows the products)
         stamp(c, prof_idx);
         // -- products, batch by batch, and their epilogues --
-        const int u0 = sh.u0[op], u1 = sh.u1[op], per_batch = units_per_batch(op);
+        const int u0 = sh.u0[op], u1 = sh.u1[op];
+        const bool paired = op_paired(op), resid = op == ST_O || op == ST_DN;
+        const int batch_log2 = paired ? RB_LOG2 - 1 : RB_LOG2, per_batch = 1 << batch_log2;
+        float sq = 0.f;                               // residual operators: this lane's share of the next norm's sum of squares
 #pragma unroll 1
         for (int ub = u0; ub == u0 || ub < u1; ub += per_batch) {
-            const int ue = min(u1, ub + per_batch), j = ub + c.tid;
-            float add_lo = 0.f, add_hi = 0.f;          // biases, fetched ahead
-            if (op == ST_QKV && L->bqkv && j < ue) {
-                const int row = (j >> p.half_shift) * D + (j & (half - 1));
-                add_lo = bf16_bits_to_f32(__ldg(L->bqkv + row));
-                add_hi = bf16_bits_to_f32(__ldg(L->bqkv + row + half));
+            const int ue = min(u1, ub + per_batch);
+            // thread -> (token, unit): residual operators take a warp per token, lanes over rows
+            const int tok = resid ? c.warp : c.tid >> batch_log2, j = ub + (resid ? c.lane : c.tid & (per_batch - 1));
+            const bool mine = tok < MT && j < ue;
+            float add_lo = 0.f, add_hi = 0.f;          // biases / the next norm's weight, fetched ahead
+            if (mine) {
+                if (op == ST_QKV && L->bqkv) {
+                    const int row = (j >> p.half_shift) * D + (j & (half - 1));
+                    add_lo = bf16_bits_to_f32(__ldg(L->bqkv + row));
+                    add_hi = bf16_bits_to_f32(__ldg(L->bqkv + row + half));
+                }
             }
-            ok = ok && multiply_any(c, Slice{ub, ue, op, static_cast<int>(batch & 1u)});
+            const uint16_t *next_norm = op == ST_O ? L->post_norm : layer + 1 == p.n_layers ? c.head().final_norm : c.layer(min(layer + 1, p.n_layers - 1))->input_norm;
+            if (resid && mine) add_lo = bf16_bits_to_f32(__ldg(next_norm + j));
+            ok = ok && multiply_any<MT>(c, Slice{ub, ue, op, static_cast<int>(batch & 1u)}, tag);
             ok = cta_vote(ok);
             if (!ok) break;
-            const float *a = sh.part[batch & 1u] + c.tid * ST_NW, *b = a + ST_BATCH * ST_NW;
+            const float *part = sh.part[batch & 1u];
             ++batch;
-            if (j < ue) {
-                float lo = 0.f, hi = 0.f;
-#pragma unroll
-                for (int w = 0; w < ST_NW; ++w) lo += a[w];
-                if (op_paired(op)) {
-#pragma unroll
-                    for (int w = 0; w < ST_NW; ++w) hi += b[w];
+            if (resid) {
+                if (tok < MT) {
+                    unsigned long long *line = (op == ST_O ? p.xo_ll : p.x_ll) + (static_cast<size_t>(tok) * c.ncta + c.cta) * p.x_line;
+#pragma unroll 1
+                    for (int r = j; r < ue; r += 32) {
+                        if (r != j) add_lo = bf16_bits_to_f32(__ldg(next_norm + r));
+                        float &x = c.resid()[tok * my_rows + r - u0];
+                        x += sum8(part + (tok * RB + r - ub) * ST_NW);
+                        sq = fmaf(x, x, sq);
+                        put_raw(line + r - u0, pieces_packet(x * add_lo, real_tag));
+                    }
+                    if (ue == u1) {
+                        const float all = warp_sum(sq);
+                        if (c.lane == 0) put1(line + p.x_line - 1, all, real_tag);
+                    }
                 }
-                finish_unit<D, Q8>(c, op, layer, j, u0, lo, hi, add_lo, add_hi, best_v, best_i);
+            } else if (mine) {
+                const float tot = sum8(sh.ss[tok]), r = rsqrtf(tot / static_cast<float>(p.H) + p.eps);       // the deferred RMSNorm factor
+                const float *a = part + (tok * RB + j - ub) * ST_NW;
+                const float lo = sum8(a) * r, hi = paired ? sum8(a + RB / 2 * ST_NW) * r : 0.f;
+                finish_unit<D, Q8, MT>(c, op, layer, tok, j, u0, lo, hi, add_lo, add_hi, best_v, best_i);
             }
         }
         stamp(c, prof_idx);
         if (op != ST_QKV && op != ST_LM) stamp(c, prof_idx);
     }
-    Shared &sh = c.sh();
+    Shared<MT> &sh = c.sh();
     if (!ok) {
         *c.abort() = 1;
         if (c.tid == 0) atomicCAS(&p.state->status, 0, 6);
         return;
     }
-    // ---- greedy token: thread -> CTA -> CTA 0 -> state --------------------------------------------------------------------
+    // ---- greedy tokens: thread -> warp -> CTA -> CTA 0 -> state ------------------------------------------------------------
+    // (threads tok * RB .. tok * RB + RB - 1 hold candidates of token tok: whole warps)
     arg_fold(best_v, best_i);
     if (c.lane == 0) { sh.best_v[c.warp] = best_v; sh.best_i[c.warp] = best_i; }
     cta_vote(true);
     const unsigned tag = sh.tag0 + static_cast<unsigned>(p.n_layers);
-    if (c.tid == 0) {
-        for (int w = 1; w < ST_NW; ++w)
-            if (arg_better(sh.best_v[w], sh.best_i[w], best_v, best_i)) { best_v = sh.best_v[w]; best_i = sh.best_i[w]; }
-        put2(p.lm_ll + static_cast<size_t>(c.cta) * 16, best_v, __int_as_float(best_i), tag);
+    constexpr int WT = RB / 32;          // warps per token
+    if (c.tid < sh.m) {
+        best_v = sh.best_v[c.tid * WT];
+        best_i = sh.best_i[c.tid * WT];
+        for (int w = 1; w < WT; ++w)
+            if (arg_better(sh.best_v[c.tid * WT + w], sh.best_i[c.tid * WT + w], best_v, best_i)) { best_v = sh.best_v[c.tid * WT + w]; best_i = sh.best_i[c.tid * WT + w]; }
+        put2(p.lm_ll + static_cast<size_t>(c.cta) * 16 + 2 * c.tid, best_v, __int_as_float(best_i), tag);
     }
-    if (c.cta != 0 || c.warp != 0) return;
+    if (c.cta != 0) return;
+    cta_vote(true);                      // (best_v / best_i have been read)
     best_v = -INFINITY;
     best_i = 0x7fffffff;
-    for (int i = c.lane; i < c.ncta && ok; i += 32) {
-        Two t = get2(p.lm_ll + static_cast<size_t>(i) * 16);
-        Spin sp;
-        while (ok && !both(t, tag)) {
-            ok = sp.again(c.abort(), p.spin_limit);
-            t = get2(p.lm_ll + static_cast<size_t>(i) * 16);
+    if (c.warp < sh.m) {                 // warp t: token t
+        for (int i = c.lane; i < c.ncta && ok; i += 32) {
+            const unsigned long long *at = p.lm_ll + static_cast<size_t>(i) * 16 + 2 * c.warp;
+            Two t = get2(at);
+            Spin sp;
+            while (ok && !both(t, tag)) {
+                ok = sp.again(c.abort(), p.spin_limit);
+                t = get2(at);
+            }
+            const float v = packet_value(t.a);
+            const int ix = __float_as_int(packet_value(t.b));
+            if (arg_better(v, ix, best_v, best_i)) { best_v = v; best_i = ix; }
         }
-        const float v = packet_value(t.a);
-        const int ix = __float_as_int(packet_value(t.b));
-        if (arg_better(v, ix, best_v, best_i)) { best_v = v; best_i = ix; }
+        arg_fold(best_v, best_i);
+        if (c.lane == 0) {
+            if (best_i < 0 || best_i >= c.head().rows) best_i = 0;       // (no logit compared as larger than -inf)
+            if (c.head().remap) best_i = p.vocab_ids[best_i];
+            sh.best_i[c.warp] = best_i;
+        }
     }
-    if (!__all_sync(0xffffffffu, ok)) {
-        if (c.lane == 0) atomicCAS(&p.state->status, 0, 6);
+    if (!cta_vote(ok)) {
+        if (c.tid == 0) atomicCAS(&p.state->status, 0, 6);
         return;
     }
-    arg_fold(best_v, best_i);
-    if (c.lane == 0) {
-        if (best_i < 0 || best_i >= c.head().rows) best_i = 0;       // (no logit compared as larger than -inf)
-        if (c.head().remap) best_i = p.vocab_ids[best_i];
-        if (p.req->next_token_out) *p.req->next_token_out = best_i;
-        if (p.req->n_accepted_out) *p.req->n_accepted_out = 1;
+    if (c.tid == 0) {
+        // Verification (Sec. 3.11): proposal t is accepted if it is the greedy choice after token t - 1; it stops at the first
+        // rejection.  The cache advances by the accepted tokens; the rows of the rejected ones stay behind the cache length and are
+        // overwritten by the next call.
+        int n_acc = 1;
+        const bool given = MT > 1 && (p.req->flags & 1);   // prompt tokens: nothing to verify
+        while (n_acc < sh.m && (given || sh.tokens[n_acc] == sh.best_i[n_acc - 1])) ++n_acc;
+        const int next = sh.best_i[n_acc - 1];
+        if (p.req->next_token_out) *p.req->next_token_out = next;
+        if (p.req->n_accepted_out) *p.req->n_accepted_out = n_acc;
         StepState *st = p.state;
-        st->next_token = best_i;
-        st->next_position = sh.pos + 1;
-        st->cur_len = sh.n_old + 1;
-        st->n_accepted = 1;
-        st->reserved[0] += 1;
+        st->next_token = next;
+        st->next_position = sh.pos + n_acc;
+        st->cur_len = sh.n_old + n_acc;
+        st->n_accepted = n_acc;
+        st->epoch[p.epoch_slot] += 1;
     }
 }
 
-template <int D, bool Q8>
+template <int D, bool Q8, int MT>
 StepKernel kernel_for(int G) {
     switch (G) {
-        case 1: return step_kernel<D, 1, Q8>;
-        case 2: return step_kernel<D, 2, Q8>;
-        case 3: return step_kernel<D, 3, Q8>;
-        case 4: return step_kernel<D, 4, Q8>;
-        case 5: return step_kernel<D, 5, Q8>;
-        case 6: return step_kernel<D, 6, Q8>;
-        case 7: return step_kernel<D, 7, Q8>;
-        default: return step_kernel<D, 8, Q8>;
+        case 1: return step_kernel<D, 1, Q8, MT>;
+        case 2: return step_kernel<D, 2, Q8, MT>;
+        case 3: return step_kernel<D, 3, Q8, MT>;
+        case 4: return step_kernel<D, 4, Q8, MT>;
+        case 5: return step_kernel<D, 5, Q8, MT>;
+        case 6: return step_kernel<D, 6, Q8, MT>;
+        case 7: return step_kernel<D, 7, Q8, MT>;
+        default: return step_kernel<D, 8, Q8, MT>;
     }
 }
 

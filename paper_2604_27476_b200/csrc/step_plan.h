@@ -1,21 +1,42 @@
-// Host side of the persistent step kernel: the static tile schedule of the weight stream and its tensor maps.
+// Host-side tile schedules (edgefm_debug_plan_operator) and the tensor-map encoder of the prompt path.
 //
+// A schedule deals the rows of a matrix-vector operator out to CTAs and consumer warps as tiles of up to 16 rows x 256 columns.
 // Every weight matrix is row-major bf16 [rows][K].  A CTA owns a contiguous range of the "units" of every operator (a
 // unit is an output row; for the QKV and gate/up operators a pair of rows whose sums meet in one epilogue: the rotate-half
 // RoPE partners i, i + d/2 of a head, or gate row i and up row F + i).  The range is cut into blocks of up to 16 rows (8
 // pairs), every block into tiles of 256 columns, and the tiles, in (block, column) order, into one contiguous run per
-// consumer warp.  A warp therefore sees consecutive column pieces of the same rows: it keeps their 16 sums in
-// registers and reduces them once per run; runs that cover all columns of a block finish the rows in the warp, the
-// others leave partial sums in shared-memory slots that are added in slot order after the operator (deterministic).
+// consumer warp.  Runs that cover all columns of a block finish the rows in the warp, the others leave partial sums in slots that
+// are added in slot order (deterministic).
 #pragma once
 #include <cuda.h>   // CUtensorMap and its enums only: the encoder is looked up at run time, nothing links against the driver library
+#include <cuda_runtime.h>
+#include <stdint.h>
 #include <algorithm>
-#include <cstring>
 #include <vector>
 
-#include "megakernel_types.cuh"
-
 namespace edgefm {
+
+constexpr int MK_PARTIAL_SLOTS = 48;   // partial sums a CTA has room for
+constexpr int MK_TILE_COLS = 256, MK_TILE_ROWS = 16;
+constexpr int MK_MAX_VARIANTS = 4;     // tile heights per matrix
+enum { PH_QKV = 0, PH_RESID = 1, PH_SWIGLU = 2, PH_LMHEAD = 3 };
+
+// 8 bytes per tile:
+//   x: unit_base [0,20) | column piece [20,28) | height variant [28,30) | FIRST 30 | FLUSH 31
+//   y: m [0,5) | first valid unit v0 [5,9) | DIRECT 9 | partial slot [10,20) | operator in layer (4 = output layer) [20,23) |
+//      RAGGED 23 (K is not a multiple of 64)
+// FIRST: a run of tiles starts.  FLUSH: it ends; DIRECT: the warp has seen all columns of these rows, otherwise the sums go to
+// partial slot `slot`.
+constexpr uint32_t MKT_FIRST = 1u << 30, MKT_FLUSH = 1u << 31, MKT_DIRECT = 1u << 9, MKT_RAGGED = 1u << 23;
+inline uint2 mk_tile_desc(uint32_t unit_base, uint32_t kcol, uint32_t variant, bool first, bool flush, uint32_t m, uint32_t v0, bool direct,
+                          uint32_t slot, uint32_t op, bool ragged) {
+    uint2 d;
+    d.x = (unit_base & 0xfffffu) | (kcol & 0xffu) << 20 | (variant & 3u) << 28 | (first ? MKT_FIRST : 0u) | (flush ? MKT_FLUSH : 0u);
+    d.y = (m & 31u) | (v0 & 15u) << 5 | (direct ? MKT_DIRECT : 0u) | (slot & 1023u) << 10 | (op & 7u) << 20 | (ragged ? MKT_RAGGED : 0u);
+    return d;
+}
+// Units whose row sums were left in partial slots: unit_base, m | v0 << 8, first slot, number of slots.
+using MkCombine = uint4;
 
 struct OpShape {
     int kind = 0;        // PH_*
@@ -123,65 +144,6 @@ inline const char *plan_op(const OpShape &os, int op_index, int ncta, int nw, in
     return nullptr;
 }
 
-// The step's schedule in the form the kernel reads.
-struct StepSchedule {
-    OpSchedule ops[5];
-    std::vector<uint2> tiles;        // per CTA one block: the warps' layer lists (operators 0..3), then their output-layer lists
-    std::vector<int> cta_tab;        // [ncta][cta_tab_ints]
-    std::vector<MkCombine> combines;
-    int cta_tab_ints = 0;
-    int max_cta_tiles = 0;           // largest block (sizes the shared-memory copy)
-    int max_cta_combines = 0;
-    // bytes of shared memory the largest CTA block needs: tiles (8 bytes each, padded to 16), then combine entries (16 bytes each)
-    size_t smem_bytes() const { return (static_cast<size_t>(max_cta_tiles) * 8 + 15) / 16 * 16 + static_cast<size_t>(max_cta_combines) * 16; }
-};
-
-inline int cta_tab_ints_for(int nw) { return (nw * MK_WARP_TAB + 14 + 3) / 4 * 4; }
-
-inline void assemble_schedule(StepSchedule *ss, int ncta, int nw) {
-    ss->cta_tab_ints = cta_tab_ints_for(nw);
-    ss->cta_tab.assign(static_cast<size_t>(ncta) * ss->cta_tab_ints, 0);
-    ss->tiles.clear();
-    ss->combines.clear();
-    ss->max_cta_tiles = 0;
-    ss->max_cta_combines = 0;
-    for (int c = 0; c < ncta; ++c) {
-        int *ctab = &ss->cta_tab[static_cast<size_t>(c) * ss->cta_tab_ints];
-        const size_t base = ss->tiles.size();
-        for (int w = 0; w < nw; ++w) {
-            int *tab = ctab + w * MK_WARP_TAB;
-            tab[0] = static_cast<int>(ss->tiles.size() - base);
-            for (int o = 0; o < 4; ++o) {
-                const auto &l = ss->ops[o].tiles[c][w];
-                tab[1 + o] = static_cast<int>(l.size());
-                tab[7] += static_cast<int>(l.size());          // tiles per layer
-                ss->tiles.insert(ss->tiles.end(), l.begin(), l.end());
-            }
-        }
-        for (int w = 0; w < nw; ++w) {
-            int *tab = ctab + w * MK_WARP_TAB;
-            const auto &l = ss->ops[4].tiles[c][w];
-            tab[5] = static_cast<int>(ss->tiles.size() - base);
-            tab[6] = static_cast<int>(l.size());
-            ss->tiles.insert(ss->tiles.end(), l.begin(), l.end());
-        }
-        const size_t cbase = ss->combines.size();
-        for (int o = 0; o < 5; ++o) {
-            int *ct = ctab + nw * MK_WARP_TAB + 2 * o;
-            const auto &l = ss->ops[o].combines[c];
-            ct[0] = static_cast<int>(ss->combines.size() - cbase);     // inside the CTA's block
-            ct[1] = static_cast<int>(l.size());
-            ss->combines.insert(ss->combines.end(), l.begin(), l.end());
-        }
-        ctab[nw * MK_WARP_TAB + 10] = static_cast<int>(base);
-        ctab[nw * MK_WARP_TAB + 11] = static_cast<int>(ss->tiles.size() - base);
-        ctab[nw * MK_WARP_TAB + 12] = static_cast<int>(cbase);
-        ctab[nw * MK_WARP_TAB + 13] = static_cast<int>(ss->combines.size() - cbase);
-        ss->max_cta_combines = std::max(ss->max_cta_combines, static_cast<int>(ss->combines.size() - cbase));
-        ss->max_cta_tiles = std::max(ss->max_cta_tiles, static_cast<int>(ss->tiles.size() - base));
-    }
-}
-
 // ---- tensor maps ---------------------------------------------------------------------------------------------------
 using TensorMapEncodeFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                        const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -198,50 +160,6 @@ inline TensorMapEncodeFn tensor_map_encoder() {
         return reinterpret_cast<TensorMapEncodeFn>(p);
     }();
     return fn;
-}
-
-// Tensor map of a row-major bf16 [rows][K] matrix on THIS GPU.  A box is box_rows rows x 256 columns, delivered to shared
-// memory as four blocks of 64 columns ([block][rows][128 bytes], 128-byte swizzle); columns and rows outside the matrix read as
-// zero.  The 64-column blocks of a row are the LAST dimension of the map (stride 128 bytes), so the column coordinate is
-// always 0 and the block coordinate is 4 * (column piece).  (No multicast is ever used with these maps.)
-//   pair_rows == 0                : (0, row, block);
-//   pair_rows  > 0, !grouped      : view [2][pair_rows][K] (gate rows, up rows): (0, row, 0, block), a box = box_rows low rows
-//                                   and their partners;
-//   pair_rows  > 0, grouped       : view [rows / (2 pair_rows)][2][pair_rows][K] (heads of the QKV matrix, rotate-half partners):
-//                                   (0, row in half, 0, head, block).
-// K not a multiple of 64: the block dimension is left out (its last block would reach into the next row); the map's first
-// dimension is then the K columns, a box is ONE 64-column block, and the caller copies the four blocks of a tile one by one.
-inline bool encode_weight_map(CUtensorMap *m, const void *base, int rows, int K, int box_rows, int pair_rows = 0, bool grouped = false) {
-    TensorMapEncodeFn enc = tensor_map_encoder();
-    if (!enc) return false;
-    const cuuint64_t row_bytes = static_cast<cuuint64_t>(K) * 2;
-    const bool ragged = K % 64 != 0;
-    // dimensions, innermost first: 64 columns (or all K columns when K has a ragged last block), rows [, partner, head],
-    // and last the 64-column blocks of a row (128 bytes apart), so that a box lands block by block
-    cuuint64_t dims[5] = {static_cast<cuuint64_t>(ragged ? K : 64), static_cast<cuuint64_t>(rows), 1, 1, 1};
-    cuuint64_t strides[4] = {row_bytes, 0, 0, 0};
-    cuuint32_t box[5] = {64, static_cast<cuuint32_t>(box_rows), 1, 1, 1};
-    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
-    cuuint32_t rank = 2;
-    if (pair_rows > 0) {
-        dims[1] = static_cast<cuuint64_t>(pair_rows); dims[2] = 2;
-        strides[1] = row_bytes * pair_rows;
-        box[2] = 2;
-        rank = 3;
-        if (grouped) {
-            dims[3] = static_cast<cuuint64_t>(rows / (2 * pair_rows));
-            strides[2] = row_bytes * pair_rows * 2;
-            rank = 4;
-        }
-    }
-    if (!ragged) {
-        dims[rank] = static_cast<cuuint64_t>(K / 64);
-        strides[rank - 1] = 128;
-        box[rank] = MK_TILE_COLS / 64;
-        ++rank;
-    }
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void *>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace edgefm

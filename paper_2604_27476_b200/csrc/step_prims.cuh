@@ -89,6 +89,29 @@ __device__ __forceinline__ Two get2(const unsigned long long *at) {
 }
 __device__ __forceinline__ bool both(const Two &t, unsigned tag) { return packet_tag(t.a) == tag && packet_tag(t.b) == tag; }
 
+// Packets of pieces: three bf16 (value = their sum) and the low 16 bits of the tag.  A slot is rewritten with the next tag every layer
+// (every token's, used or not), so 16 bits tell the contents apart.
+__device__ __forceinline__ unsigned long long pieces_packet(float v, unsigned tag) {
+    const uint16_t hi = f32_to_bf16_bits(v);
+    v -= bf16_bits_to_f32(hi);           // exact: the remainder is what the next piece holds
+    const uint16_t mid = f32_to_bf16_bits(v);
+    const uint16_t lo = f32_to_bf16_bits(v - bf16_bits_to_f32(mid));
+    return static_cast<unsigned long long>(hi | static_cast<unsigned>(mid) << 16) | static_cast<unsigned long long>(lo | tag << 16) << 32;
+}
+__device__ __forceinline__ bool pieces_tag(unsigned long long p, unsigned tag) { return static_cast<unsigned>(p >> 48) == (tag & 0xffffu); }
+__device__ __forceinline__ uint16_t piece(unsigned long long p, int i) { return static_cast<uint16_t>(p >> (16 * i)); }
+__device__ __forceinline__ void put_raw(unsigned long long *at, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(at), "l"(v) : "memory");
+}
+__device__ __forceinline__ void put_raw2(unsigned long long *at, unsigned long long a, unsigned long long b) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(at), "l"(a), "l"(b) : "memory");
+}
+__device__ __forceinline__ unsigned long long get1(const unsigned long long *at) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(at) : "memory");
+    return v;
+}
+
 // Two fp32 values in one 64-bit register pair.
 using f2 = unsigned long long;
 __device__ __forceinline__ f2 pack2(float a, float b) {
@@ -141,51 +164,52 @@ __device__ __forceinline__ int folded(int sub, int lpr) {
 }
 
 // ---- shared memory ---------------------------------------------------------------------------------------------------
-// Dynamic: Shared | ring | layer table, unit tables, residual rows | staged vector, attention scratch (the MLP activations take the
-// place of both: their first packet is awaited after the vote behind the gate/up products, the last readers of the vector).
+// Dynamic: Shared | ring | layer table, unit tables, residual rows | one area for the staged vector, the attention's scratch and the
+// segments of the MLP activations (they follow one another; between the last reader of one and the first writer of the next
+// lies a CTA-wide vote).
 extern __shared__ __align__(128) unsigned char st_smem[];
-// The cached positions a CTA attends to.
-struct KvShare { int g, chunk, n_chunks, t0, t1, tail, any; };
-struct Shared {
+template <int MT> struct Shared {
     unsigned long long full[ST_BARS], empty[ST_BARS];
     unsigned chunk_at[ST_BARS];                            // ring offset of the chunk behind every barrier
-    float rope[128];                                       // cos | sin of the step's position
-    float ss[ST_NW];                                       // partial sums of squares (RMSNorm)
-    float part[2][2 * ST_BATCH * ST_NW];                   // partial row sums [row][warp], two batches
-    float merged[2 * ST_NT];                               // attention outputs this CTA owns
+    float rope[MT][128];                                   // per token: cos | sin of its position
+    alignas(16) float ss[MT][ST_NW];                       // partial sums of squares (RMSNorm)
+    alignas(16) float part[2][MT * st_batch(MT) * ST_NW];  // partial row sums [token][row][warp], two batches
+    alignas(16) float merged[MT][128];                     // attention outputs this CTA owns
     float best_v[ST_NW];
     int best_i[ST_NW];
     int u0[5], u1[5];                                      // this CTA's units of every operator
-    KvShare share;
     unsigned tag0, odd;                                    // tag of layer 0; test hook: a bit no tag has
-    int token, pos, n_old, total_x, total_a;               // the step's token, position, cache length; sizes of the unit tables
-    unsigned sent;                                         // 16-byte units the feeding thread has asked for
+    int tokens[MT];
+    int m, pos, n_old, n_chunks, total_x, total_a;         // the call's tokens, first position, cache length; attention chunks per kv head and token; sizes of the unit tables
+    unsigned sent;                                         // 16-byte units the feeding warp has asked for
     int abort;
 };
-constexpr int ST_SHARED_BYTES = (static_cast<int>(sizeof(Shared)) + 127) / 128 * 128;
+template <int MT> __host__ __device__ constexpr int st_shared_bytes() { return (static_cast<int>(sizeof(Shared<MT>)) + 127) / 128 * 128; }
 
 // What the device functions share: the parameter block (constant bank), the thread's place and the ring position; everything else
 // stands in shared memory, so that little is carried in registers from one operator to the next.
-struct Ctx {
+template <int MT> struct Ctx {
+    static constexpr int S = st_pieces(MT), NA = st_arrays(MT), RB = st_batch(MT);
     const StepParams &par;
     int tid, warp, lane, cta, ncta;
     unsigned chunk;          // next ring chunk to consume
     __device__ __forceinline__ explicit Ctx(const StepParams &p_)
         : par(p_), tid(static_cast<int>(threadIdx.x)), warp(tid >> 5), lane(tid & 31), cta(static_cast<int>(blockIdx.x)), ncta(static_cast<int>(gridDim.x)), chunk(0u) {}
-    __device__ __forceinline__ Shared &sh() const { return *reinterpret_cast<Shared *>(st_smem); }
+    __device__ __forceinline__ Shared<MT> &sh() const { return *reinterpret_cast<Shared<MT> *>(st_smem); }
     __device__ __forceinline__ const StepParams &p() const { return par; }
     __device__ __forceinline__ volatile int *abort() const { return &sh().abort; }
-    __device__ __forceinline__ unsigned char *ring() const { return st_smem + ST_SHARED_BYTES; }
+    __device__ __forceinline__ unsigned char *ring() const { return st_smem + st_shared_bytes<MT>(); }
     __device__ __forceinline__ unsigned char *tables() const { return ring() + p().ring_bytes; }
     __device__ __forceinline__ const StepLayer *layer(int l) const { return reinterpret_cast<const StepLayer *>(tables()) + l; }
     __device__ __forceinline__ const StepHead &head() const { return *reinterpret_cast<const StepHead *>(layer(p().n_layers)); }
     __device__ __forceinline__ unsigned *unit_table() const { return reinterpret_cast<unsigned *>(tables() + (p().n_layers + 1) * 64); }
-    __device__ __forceinline__ float *resid() const { return reinterpret_cast<float *>(tables() + p().resid_at); }   // this CTA's rows of the residual stream
-    __device__ __forceinline__ float *xs() const { return reinterpret_cast<float *>(tables() + p().table_bytes); }
-    __device__ __forceinline__ float *scratch() const { return xs() + p().xs_floats; }     // attention
+    __device__ __forceinline__ float *resid() const { return reinterpret_cast<float *>(tables() + p().resid_at); }   // [token][this CTA's rows of the residual stream]
+    __device__ __forceinline__ unsigned char *area() const { return tables() + p().table_bytes; }
+    // Column `col` of array `a` of a staged vector of K columns: array = token * S + piece, bf16, in natural order.
+    __device__ __forceinline__ uint16_t *xs(int a, int col, int K) const { return reinterpret_cast<uint16_t *>(area() + a * st_array_bytes(K)) + col; }
 };
 
-__device__ __forceinline__ void stamp(const Ctx &c, int &idx) {
+template <int MT> __device__ __forceinline__ void stamp(const Ctx<MT> &c, int &idx) {
     const StepParams &p = c.p();
     if (p.prof && c.tid == 0) {
         if (idx < p.prof_stride) p.prof[static_cast<size_t>(c.cta) * p.prof_stride + idx] = global_ns();
@@ -194,14 +218,14 @@ __device__ __forceinline__ void stamp(const Ctx &c, int &idx) {
 }
 
 // ---- ring: consumer side -----------------------------------------------------------------------------------------------
-__device__ __forceinline__ bool chunk_wait(Ctx &c, const unsigned char *&at) {
-    Shared &sh = c.sh();
+template <int MT> __device__ __forceinline__ bool chunk_wait(Ctx<MT> &c, const unsigned char *&at) {
+    Shared<MT> &sh = c.sh();
     const unsigned b = c.chunk & (ST_BARS - 1), parity = (c.chunk / ST_BARS) & 1u;
     const bool ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[b], parity, c.abort(), c.p().spin_limit));
     at = c.ring() + *reinterpret_cast<volatile unsigned *>(&sh.chunk_at[b]);
     return ok;
 }
-__device__ __forceinline__ void chunk_release(Ctx &c) {
+template <int MT> __device__ __forceinline__ void chunk_release(Ctx<MT> &c) {
     __syncwarp();
     if (c.lane == 0) mbar_arrive(&c.sh().empty[c.chunk & (ST_BARS - 1)]);
     ++c.chunk;
@@ -217,24 +241,24 @@ __device__ __forceinline__ int op_units(const StepParams &p, int op, int lm_rows
     }
 }
 __device__ __forceinline__ bool op_paired(int op) { return op == ST_QKV || op == ST_GU; }
-__device__ __forceinline__ int units_per_batch(int op) { return op_paired(op) ? ST_BATCH : 2 * ST_BATCH; }
-// Units of the chunk that starts at unit u of [.., u1).
-__device__ __forceinline__ int chunk_units(const StepParams &p, int op, int u, int u1) {
-    const int rows = p.cols[op].rows_per_chunk;
-    int n = min(op_paired(op) ? rows >> 1 : rows, u1 - u);
+// Units of the tile that starts at unit u of [.., u1).
+__device__ __forceinline__ int tile_units(const StepParams &p, int op, int u, int u1) {
+    int n = min(op_paired(op) ? ST_TILE / 2 : ST_TILE, u1 - u);
     if (op == ST_QKV) n = min(n, (1 << p.half_shift) - (u & ((1 << p.half_shift) - 1)));   // rows of one head are contiguous, heads are not
     return n;
 }
-// The cached positions CTA `cta` attends to: a chunk of the `n` old positions.
-__device__ __forceinline__ KvShare kv_share(const StepParams &p, int n, int cta, int ncta) {
+// Attention is dealt out by (token, kv head, chunk of the n_old cached positions); a CTA serves the shares cta, cta + ncta, ...
+struct KvShare { int tok, g, chunk, t0, t1, tail; };
+__device__ __forceinline__ int kv_chunks(const StepParams &p, int n, int m, int ncta) { return max(1, min(ncta / (p.nkv * m), (n + ST_MIN_CHUNK - 1) / ST_MIN_CHUNK)); }
+__device__ __forceinline__ KvShare kv_share(const StepParams &p, int n, int n_chunks, int idx) {
     KvShare s;
-    s.n_chunks = max(1, min(max(1, ncta / p.nkv), (n + ST_MIN_CHUNK - 1) / ST_MIN_CHUNK));
-    s.g = cta / s.n_chunks;
-    s.chunk = cta - s.g * s.n_chunks;
-    s.t0 = st_first(n, s.chunk, s.n_chunks);
-    s.t1 = st_first(n, s.chunk + 1, s.n_chunks);
-    s.tail = s.chunk == s.n_chunks - 1;
-    s.any = s.g < p.nkv;
+    const int tg = idx / n_chunks;
+    s.chunk = idx - tg * n_chunks;
+    s.tok = tg / p.nkv;
+    s.g = tg - s.tok * p.nkv;
+    s.t0 = st_first(n, s.chunk, n_chunks);
+    s.t1 = st_first(n, s.chunk + 1, n_chunks);
+    s.tail = s.chunk == n_chunks - 1;
     return s;
 }
 

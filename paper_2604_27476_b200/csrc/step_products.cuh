@@ -5,15 +5,11 @@
 namespace edgefm {
 namespace step {
 
-// Place of value j of a staged vector of 8 * k8 values: two planes of 16-byte halves of its pieces, so that neighbouring lanes read
-// neighbouring 16 bytes.
-__device__ __forceinline__ int xs_at(int j, int k8) { return ((j & 4) ? k8 * 4 : 0) + (j >> 3) * 4 + (j & 3); }
-
 // ---- exchanges: everybody reads a vector that lies in lines ---------------------------------------------------------------
 // Table of the 16-byte units of such a vector: row | values << 16 | unit << 18 (unit = index of the packet pair).
 // The tables of the residual stream and of the attention output stand in shared memory, made once per launch.
 __device__ __forceinline__ int line_units(int n, int ncta, int grain) { return ((n / grain + ncta - 1) / ncta * grain + 1) / 2; }
-__device__ __forceinline__ void make_table(const Ctx &c, unsigned *tab, int n, int grain, int line) {
+template <int MT> __device__ __forceinline__ void make_table(const Ctx<MT> &c, unsigned *tab, int n, int grain, int line) {
     const int upl = line_units(n, c.ncta, grain), total = c.ncta * upl;
 #pragma unroll 1
     for (int i = c.tid; i < total; i += ST_NT) {
@@ -22,206 +18,375 @@ __device__ __forceinline__ void make_table(const Ctx &c, unsigned *tab, int n, i
         tab[i] = static_cast<unsigned>(row & 0xffff) | static_cast<unsigned>(max(0, min(2, r1 - row))) << 16 | static_cast<unsigned>(w * (line >> 1) + e) << 18;
     }
 }
-__device__ __forceinline__ bool staged(Ctx &c, bool ok, float ss) {      // publish the sums of squares, meet
-    ss = warp_sum(ss);
-    if (c.lane == 0) c.sh().ss[c.warp] = ss;
-    return cta_vote(ok);
+template <int MT> __device__ __forceinline__ void store_pieces(const Ctx<MT> &c, int tok, int col, int K, unsigned long long v) {
+    constexpr int S = Ctx<MT>::S;
+#pragma unroll
+    for (int i = 0; i < S; ++i) *c.xs(tok * S + i, col, K) = piece(v, i);
 }
-// First operator of the step: the embedding row is the residual stream.
-__device__ __forceinline__ bool stage_embedding(Ctx &c, const uint16_t *norm_w) {
+// Columns past K of the last 64-column block are multiplied by zero.
+template <int MT> __device__ __forceinline__ void zero_tail(const Ctx<MT> &c, int K) {
+    const int pad = (64 - (K & 63)) & 63;
+    for (int i = c.tid; i < pad * Ctx<MT>::NA; i += ST_NT) *c.xs(i / pad, K + i % pad, K) = 0;
+}
+// First operator of the step: the embedding rows are the residual streams.
+template <int MT> __device__ __forceinline__ bool stage_embedding(Ctx<MT> &c, const uint16_t *norm_w) {
     const StepParams &p = c.p();
-    const uint16_t *erow = p.embed + static_cast<size_t>(c.sh().token) * p.H;
-    float ss = 0.f;
 #pragma unroll 1
-    for (int i = c.tid; i < p.H; i += ST_NT) {
-        const float v = bf16_bits_to_f32(erow[i]);
-        ss = fmaf(v, v, ss);
-        c.xs()[xs_at(i, p.H / 8)] = v * bf16_bits_to_f32(norm_w[i]);
-    }
-    return staged(c, true, ss);
-}
-// Wait for all values of the vector, times norm_w (RMSNorm weight, or null), into xs, and meet.
-__device__ __forceinline__ bool stage_lines(Ctx &c, const unsigned *tab, int total, int k8, const unsigned long long *ll, const uint16_t *norm_w,
-                                            unsigned tag) {
-    constexpr int U = 4;     // units in flight per thread
-    float *xs = c.xs();
-    float ss = 0.f;
-    bool ok = true;
+    for (int t = 0; t < c.sh().m; ++t) {
+        const uint16_t *erow = p.embed + static_cast<size_t>(c.sh().tokens[t]) * p.H;
+        float ss = 0.f;
 #pragma unroll 1
-    for (int base = c.tid; base < total; base += U * ST_NT) {
-        unsigned e[U];
-        float w0[U], w1[U];
-        Two t[U];
-        unsigned todo = 0;
-#pragma unroll
-        for (int i = 0; i < U; ++i) {
-            const int u = base + i * ST_NT;
-            e[i] = u < total ? tab[u] : 0u;
-            const int cnt = (e[i] >> 16) & 3u;
-            w0[i] = w1[i] = 1.f;
-            if (cnt) {
-                todo |= 1u << i;
-                if (norm_w) {
-                    w0[i] = bf16_bits_to_f32(__ldg(norm_w + (e[i] & 0xffffu)));
-                    if (cnt > 1) w1[i] = bf16_bits_to_f32(__ldg(norm_w + (e[i] & 0xffffu) + 1));
-                }
-            }
+        for (int i = c.tid; i < p.H; i += ST_NT) {
+            const float v = bf16_bits_to_f32(erow[i]);
+            ss = fmaf(v, v, ss);
+            store_pieces(c, t, i, p.H, pieces_packet(v * bf16_bits_to_f32(norm_w[i]), 0u));
         }
-        Spin sp;
-        for (;;) {
+        ss = warp_sum(ss);
+        if (c.lane == 0) c.sh().ss[t][c.warp] = ss;
+    }
+    zero_tail(c, p.H);
+    return cta_vote(true);
+}
+// Wait for all values of the vectors of all tokens (K columns, lines of `line` packets) and leave their pieces in shared memory, and meet.
+// sums: the last packet of every line is a partial sum of squares.
+template <int MT>
+__device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int total, int K, const unsigned long long *ll, int line, bool sums, unsigned tag) {
+    constexpr int U = 4;     // units in flight per thread
+    const int m = c.sh().m;
+    bool ok = true;
+    zero_tail(c, K);
+#pragma unroll 1
+    for (int tok = 0; tok < m && ok; ++tok) {
+        const unsigned long long *lt = ll + static_cast<size_t>(tok) * c.ncta * line;
+#pragma unroll 1
+        for (int base = c.tid; base < total; base += U * ST_NT) {
+            unsigned e[U];
+            Two t[U];
+            unsigned todo = 0;
 #pragma unroll
-            for (int i = 0; i < U; ++i)
-                if (todo >> i & 1u) t[i] = get2(ll + static_cast<size_t>(e[i] >> 18) * 2);
+            for (int i = 0; i < U; ++i) {
+                const int u = base + i * ST_NT;
+                e[i] = u < total ? tab[u] : 0u;
+                if ((e[i] >> 16) & 3u) todo |= 1u << i;
+            }
+            Spin sp;
+            for (;;) {
 #pragma unroll
-            for (int i = 0; i < U; ++i)
-                if (todo >> i & 1u) {
-                    const bool two = (e[i] >> 16 & 3u) > 1;
-                    if (packet_tag(t[i].a) == tag && (!two || packet_tag(t[i].b) == tag)) {
-                        todo &= ~(1u << i);
-                        const int row = e[i] & 0xffffu;
-                        const float a = packet_value(t[i].a);
-                        ss = fmaf(a, a, ss);
-                        xs[xs_at(row, k8)] = a * w0[i];
-                        if (two) {
-                            const float b = packet_value(t[i].b);
-                            ss = fmaf(b, b, ss);
-                            xs[xs_at(row + 1, k8)] = b * w1[i];
+                for (int i = 0; i < U; ++i)
+                    if (todo >> i & 1u) t[i] = get2(lt + static_cast<size_t>(e[i] >> 18) * 2);
+#pragma unroll
+                for (int i = 0; i < U; ++i)
+                    if (todo >> i & 1u) {
+                        const bool two = (e[i] >> 16 & 3u) > 1;
+                        if (pieces_tag(t[i].a, tag) && (!two || pieces_tag(t[i].b, tag))) {
+                            todo &= ~(1u << i);
+                            const int row = e[i] & 0xffffu;
+                            store_pieces(c, tok, row, K, t[i].a);
+                            if (two) store_pieces(c, tok, row + 1, K, t[i].b);
                         }
                     }
-                }
-            if (!todo) break;
-            if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+                if (!todo) break;
+                if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+            }
+            if (!ok) break;
         }
-        if (!ok) break;
-    }
-    return staged(c, ok, ss);
-}
-// The MLP activations: every warp waits for its own slice (as the products deal out the columns) and leaves it in xs.
-__device__ __forceinline__ bool stage_slice(Ctx &c, const unsigned long long *ll, unsigned tag) {
-    constexpr int U = 6;     // packet pairs in flight per lane
-    const int k8 = c.p().cols[ST_DN].K8;
-    const int v0 = (k8 * c.warp / ST_NW) * 4, v1 = (k8 * (c.warp + 1) / ST_NW) * 4;      // pairs of values
-    bool ok = true;
+        if (sums) {
+            float ss = 0.f;
 #pragma unroll 1
-    for (int base = v0 + c.lane; base < v1; base += U * 32) {
-        Two t[U];
-        unsigned todo = 0;
-#pragma unroll
-        for (int i = 0; i < U; ++i)
-            if (base + i * 32 < v1) todo |= 1u << i;
-        Spin sp;
-        for (;;) {
-#pragma unroll
-            for (int i = 0; i < U; ++i)
-                if (todo >> i & 1u) t[i] = get2(ll + static_cast<size_t>(base + i * 32) * 2);
-#pragma unroll
-            for (int i = 0; i < U; ++i)
-                if ((todo >> i & 1u) && both(t[i], tag)) {
-                    todo &= ~(1u << i);
-                    *reinterpret_cast<float2 *>(c.xs() + xs_at((base + i * 32) * 2, k8)) = make_float2(packet_value(t[i].a), packet_value(t[i].b));
+            for (int w = c.tid; w < c.ncta && ok; w += ST_NT) {
+                const unsigned long long *at = lt + static_cast<size_t>(w) * line + line - 1;
+                unsigned long long v = get1(at);
+                Spin sp;
+                while (packet_tag(v) != tag) {
+                    if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+                    v = get1(at);
                 }
-            if (!todo) break;
-            if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+                ss += packet_value(v);
+            }
+            ss = warp_sum(ss);
+            if (c.lane == 0) c.sh().ss[tok][c.warp] = ss;
         }
-        if (!ok) break;
     }
-    return __all_sync(0xffffffffu, ok);
+    return cta_vote(ok);
 }
 
 // ---- products ------------------------------------------------------------------------------------------------------------
-// Rows [u, u1) (units) of operator `op`: this warp's column slice of every row, its sums to part[row][warp]; the input vector
-// stands in xs.  PG pieces per lane are multiplied at once with ST row groups; up to PG pieces stay in registers for the whole
-// operator, more are re-read for every group of rows.
-struct Slice { int u, u1, op, batch; };
-
-template <int PG, int ST>
-__device__ __forceinline__ bool multiply(Ctx &c, const Slice &sl) {
-    const StepParams &p = c.p();
-    const StepCols &cols = p.cols[sl.op];
-    float *const part = c.sh().part[sl.batch & 1];
-    const int lpr_log2 = cols.lpr_log2, lpr = 1 << lpr_log2, rp = 32 >> lpr_log2;   // lanes of a row, rows at a time
-    const int sub = c.lane & (lpr - 1), grp = c.lane >> lpr_log2;
-    const int c0 = cols.K8 * c.warp / ST_NW + sub, c1 = cols.K8 * (c.warp + 1) / ST_NW, pieces = cols.pieces, k8 = cols.K8;
-    const bool paired = op_paired(sl.op);
-    const int row_bytes = cols.K * 2;
-    const bool kept = pieces <= PG;
-    const float *const xs = c.xs();
-    f2 x[PG][4];
+// One mma.m16n8k16 multiplies a 16-row x 16-column block of bf16 weights (A) by B = [16 x 8], whose columns are the pieces of the
+// tokens' activations (token * S + piece); products of two bf16 values are exact in fp32, accumulation is fp32.  The instruction
+// serves as a dot-product unit: 16 bytes of weights cost 8 conversions and 4 packed FMAs otherwise (measured from L2 over the
+// chip, 48 KB chunks: 13 TB/s; this form 16 TB/s; the copies alone 19 TB/s; HBM 7 TB/s).
+//   A lane reads 16 bytes (8 columns) of rows g = lane / 4 and g + 8 at piece t = lane % 4 of a 32-column half of a 64-column block:
+// the four words are the A registers of two instructions (which columns a "k" stands for does not matter as long as B agrees:
+// its lane (n = g, t) reads the same 16 bytes of array n).  All rows start on the same banks, so odd rows read the block's second
+// half first and swap afterwards.
+__device__ __forceinline__ void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint4 pick(bool second, const uint4 &a, const uint4 &b) {
+    return make_uint4(second ? b.x : a.x, second ? b.y : a.y, second ? b.z : a.z, second ? b.w : a.w);
+}
+template <int SETS> struct Acc {       // row sums of a tile: two independent chains per 8 B columns
+    float d[SETS][2][4];
+    __device__ __forceinline__ void clear() {
 #pragma unroll
-    for (int i = 0; i < PG; ++i) x[i][0] = x[i][1] = x[i][2] = x[i][3] = 0ull;      // (see Two)
-    auto load_x = [&](int i0) {
+        for (int s = 0; s < SETS; ++s)
 #pragma unroll
-        for (int i = 0; i < PG; ++i) {
-            const int pc = c0 + ((i0 + i) << lpr_log2);
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-            if (pc < c1) {
-                a = *reinterpret_cast<const float4 *>(xs + pc * 4);
-                b = *reinterpret_cast<const float4 *>(xs + (k8 + pc) * 4);
+            for (int q = 0; q < 2; ++q) d[s][q][0] = d[s][q][1] = d[s][q][2] = d[s][q][3] = 0.f;
+    }
+};
+// Block j (64 columns) of a chunk: rows ra / rb (this lane's), `last` = offset of the last 16 bytes of a row; bv: B registers.
+template <int SETS>
+__device__ __forceinline__ void block_mma(Acc<SETS> &acc, const unsigned char *ra, const unsigned char *rb, int off, bool odd, int last, const uint4 (&b0)[SETS], const uint4 (&b1)[SETS]) {
+    const int o0 = min(off + (odd ? 64 : 0), last), o1 = min(off + (odd ? 0 : 64), last);    // (past the row: the vector is zero there)
+    const uint4 p0 = *reinterpret_cast<const uint4 *>(ra + o0), q0 = *reinterpret_cast<const uint4 *>(rb + o0);
+    const uint4 p1 = *reinterpret_cast<const uint4 *>(ra + o1), q1 = *reinterpret_cast<const uint4 *>(rb + o1);
+    const uint4 a = pick(odd, p0, p1), b = pick(odd, q0, q1), e = pick(odd, p1, p0), f = pick(odd, q1, q0);
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+        mma(acc.d[s][0], a.x, b.x, a.y, b.y, b0[s].x, b0[s].y);
+        mma(acc.d[s][1], a.z, b.z, a.w, b.w, b0[s].z, b0[s].w);
+        mma(acc.d[s][0], e.x, f.x, e.y, f.y, b1[s].x, b1[s].y);
+        mma(acc.d[s][1], e.z, f.z, e.w, f.w, b1[s].z, b1[s].w);
+    }
+}
+// The row sums of a finished tile to part[token][row][warp]; row r of the tile (MMA rows 0..7) is row `first` + r of the batch, MMA rows
+// 8..15 are `second` + 0..7.
+template <int MT, int SETS>
+__device__ __forceinline__ void flush(const Ctx<MT> &c, Acc<SETS> &acc, float *part, int first, int n_first, int second, int n_second) {
+    const int g = c.lane >> 2, t = c.lane & 3;
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+        float d[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) d[e] = acc.d[s][0][e] + acc.d[s][1][e];
+        if constexpr (Ctx<MT>::S == 2) {                  // columns 2 t, 2 t + 1 are the pieces of token 4 s + t
+            float *at = part + (4 * s + t) * Ctx<MT>::RB * ST_NW + c.warp;
+            if (4 * s + t < MT) {
+                if (g < n_first) at[(first + g) * ST_NW] = d[0] + d[1];
+                if (g < n_second) at[(second + g) * ST_NW] = d[2] + d[3];
             }
-            x[i][0] = pack2(a.x, a.y); x[i][1] = pack2(a.z, a.w); x[i][2] = pack2(b.x, b.y); x[i][3] = pack2(b.z, b.w);
+        } else {                                          // token 0: columns 0, 1, 2; token 1: columns 3, 4, 5
+            const float n0 = __shfl_down_sync(0xffffffffu, d[0], 1), n2 = __shfl_down_sync(0xffffffffu, d[2], 1);
+            float *at = part + c.warp;
+            if (t == 0) {
+                if (g < n_first) at[(first + g) * ST_NW] = d[0] + d[1] + n0;
+                if (g < n_second) at[(second + g) * ST_NW] = d[2] + d[3] + n2;
+            }
+            if constexpr (MT == 2) {
+                const float m0 = __shfl_down_sync(0xffffffffu, d[1], 1), m2 = __shfl_down_sync(0xffffffffu, d[3], 1);
+                const float k0 = __shfl_down_sync(0xffffffffu, d[0] + d[1], 2), k2 = __shfl_down_sync(0xffffffffu, d[2] + d[3], 2);
+                at += Ctx<MT>::RB * ST_NW;
+                if (t == 0) {
+                    if (g < n_first) at[(first + g) * ST_NW] = m0 + k0;
+                    if (g < n_second) at[(second + g) * ST_NW] = m2 + k2;
+                }
+            }
         }
-    };
-    bool loaded = false;
-    int done = 0;                              // units of this call finished
+    }
+}
+
+struct Slice { int u, u1, op, batch; };      // units [u, u1) of an operator; the batch of partial sums they go to
+
+// KEEP > 0: rows are whole in a chunk and a warp's blocks of the vector (at most KEEP) stay in registers for all tiles.
+// KEEP == 0: tiles cut by columns, the vector is read again for every tile.
+template <int KEEP, int MT>
+__device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
+    constexpr int SETS = (Ctx<MT>::NA + 7) / 8;
+    const StepParams &p = c.p();
+    const int K = p.cols[sl.op].K, seg = p.cols[sl.op].seg;
+    float *const part = c.sh().part[sl.batch & 1];
+    const int g = c.lane >> 2, t16 = (c.lane & 3) * 16;
+    const bool odd = (g & 1) != 0, paired = op_paired(sl.op);
+    const unsigned char *xb[SETS];           // this lane's array of the staged vector (columns of B past the last array: any)
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) xb[s] = reinterpret_cast<const unsigned char *>(c.xs(min(8 * s + g, Ctx<MT>::NA - 1), 0, K)) + t16;
+    constexpr int NK = KEEP > 0 ? KEEP : 1;
+    uint4 k0[NK][SETS], k1[NK][SETS];
+    const int nb_all = (K + 63) / 64, first_all = nb_all * c.warp / ST_NW, mine_all = nb_all * (c.warp + 1) / ST_NW - first_all;
+    if constexpr (KEEP > 0) {
+#pragma unroll
+        for (int i = 0; i < NK; ++i)
+#pragma unroll
+            for (int s = 0; s < SETS; ++s) {
+                const bool on = i < mine_all;
+                const unsigned char *at = xb[s] + (first_all + (on ? i : 0)) * 128;
+                k0[i][s] = on ? *reinterpret_cast<const uint4 *>(at) : make_uint4(0u, 0u, 0u, 0u);
+                k1[i][s] = on ? *reinterpret_cast<const uint4 *>(at + 64) : make_uint4(0u, 0u, 0u, 0u);
+            }
+    }
+    Acc<SETS> acc;
+    acc.clear();
 #pragma unroll 1
     for (int u = sl.u; u < sl.u1;) {
-        const int n = chunk_units(p, sl.op, u, sl.u1), rows = paired ? 2 * n : n;
-        const unsigned char *at;
-        if (!chunk_wait(c, at)) return false;
+        const int n = tile_units(p, sl.op, u, sl.u1);
+        const int na = paired ? n : min(n, 8), nb = paired ? n : n - na;                       // rows in the upper and lower half of the MMA
+        if constexpr (KEEP > 0) {
+            const unsigned char *at;
+            if (!chunk_wait(c, at)) return false;
+            const int rb = K * 2;
+            const unsigned char *ra = at + min(g, na - 1) * rb + t16 + first_all * 128, *rc = at + min(na + g, na + nb - 1) * rb + t16 + first_all * 128;
+            const int last = rb - 16 - t16 - first_all * 128;
+#pragma unroll
+            for (int i = 0; i < NK; ++i) block_mma<SETS>(acc, ra, rc, i * 128, odd, last, k0[i], k1[i]);
+            chunk_release(c);
+        } else {
 #pragma unroll 1
-        for (int s0 = 0; s0 < rows; s0 += rp * ST) {
-            f2 acc[ST][2];
-            const unsigned char *row[ST];
+            for (int col = 0; col < K; col += seg) {
+                const unsigned char *at;
+                if (!chunk_wait(c, at)) return false;
+                const int cols = min(seg, K - col), rb = cols * 2, nblk = (cols + 63) / 64;
+                const int j0 = nblk * c.warp / ST_NW, j1 = nblk * (c.warp + 1) / ST_NW;
+                const unsigned char *ra = at + min(g, na - 1) * rb + t16, *rc = at + min(na + g, na + nb - 1) * rb + t16;
+#pragma unroll 2
+                for (int j = j0; j < j1; ++j) {
+                    uint4 b0[SETS], b1[SETS];
 #pragma unroll
-            for (int s = 0; s < ST; ++s) {
-                row[s] = at + min(s0 + s * rp + grp, rows - 1) * row_bytes;
-                acc[s][0] = acc[s][1] = 0ull;
-            }
-#pragma unroll 1
-            for (int i0 = 0; i0 < pieces; i0 += PG) {
-                if (!(kept && loaded)) load_x(i0);
-                loaded = true;
-                uint4 w[PG][ST];
-#pragma unroll
-                for (int i = 0; i < PG; ++i) {
-                    const int off = min(c0 + ((i0 + i) << lpr_log2), k8 - 1) * 16;     // (past the slice: the vector is zero there)
-#pragma unroll
-                    for (int s = 0; s < ST; ++s) w[i][s] = *reinterpret_cast<const uint4 *>(row[s] + off);
-                }
-#pragma unroll
-                for (int i = 0; i < PG; ++i)
-#pragma unroll
-                    for (int s = 0; s < ST; ++s) {
-                        acc[s][0] = fma2(bf16x2_f2(w[i][s].x), x[i][0], acc[s][0]);
-                        acc[s][1] = fma2(bf16x2_f2(w[i][s].y), x[i][1], acc[s][1]);
-                        acc[s][0] = fma2(bf16x2_f2(w[i][s].z), x[i][2], acc[s][0]);
-                        acc[s][1] = fma2(bf16x2_f2(w[i][s].w), x[i][3], acc[s][1]);
+                    for (int s = 0; s < SETS; ++s) {
+                        const unsigned char *x = xb[s] + (col + j * 64) * 2;
+                        b0[s] = *reinterpret_cast<const uint4 *>(x);
+                        b1[s] = *reinterpret_cast<const uint4 *>(x + 64);
                     }
+                    block_mma<SETS>(acc, ra, rc, j * 128, odd, rb - 16 - t16, b0, b1);
+                }
+                chunk_release(c);
             }
-            float sum[ST];
-#pragma unroll
-            for (int s = 0; s < ST; ++s) {
-                const float2 a = unpack2(acc[s][0]), b = unpack2(acc[s][1]);
-                sum[s] = (a.x + a.y) + (b.x + b.y);
-            }
-            const float v = fold<ST>(sum, sub, lpr);
-            const int r = s0 + folded<ST>(sub, lpr) * rp + grp;
-            if ((sub & (lpr / ST - 1)) == 0 && r < rows) part[(done + (r < n ? r : r - n + ST_BATCH)) * ST_NW + c.warp] = v;
         }
-        chunk_release(c);
+        const int done = u - sl.u;
+        flush<MT, SETS>(c, acc, part, done, na, paired ? Ctx<MT>::RB / 2 + done : done + 8, nb);
+        acc.clear();
         u += n;
-        done += n;
     }
     return true;
 }
-__device__ __forceinline__ bool multiply_any(Ctx &c, const Slice &sl) {
-    switch (c.p().cols[sl.op].variant) {
-        case ST_V14: return multiply<1, 4>(c, sl);
-        case ST_V24: return multiply<2, 4>(c, sl);
-        case ST_V34: return multiply<3, 4>(c, sl);
-        case ST_V62: return multiply<6, 2>(c, sl);
-        case ST_V101: return multiply<10, 1>(c, sl);
-        default: return multiply<5, 2>(c, sl);
+
+// Down projection: its input, the MLP activations, is too long to be staged whole.  Every warp needs only its own blocks of a segment; it
+// polls them a segment ahead (the loads are on their way while it multiplies) into one of two small buffers of its own.
+template <int MT>
+__device__ __forceinline__ bool multiply_down(Ctx<MT> &c, const Slice &sl, unsigned tag) {
+    constexpr int NA = Ctx<MT>::NA, S = Ctx<MT>::S, SETS = (NA + 7) / 8, U = MT <= 2 ? 4 : 2;      // packet pairs in flight per lane and token
+    const StepParams &p = c.p();
+    const int K = p.cols[ST_DN].K, seg = p.cols[ST_DN].seg, stride = st_array_bytes(p.dn_cols);
+    float *const part = c.sh().part[sl.batch & 1];
+    const int g = c.lane >> 2, t16 = (c.lane & 3) * 16, m = c.sh().m;
+    const bool odd = (g & 1) != 0;
+    unsigned char *const own = c.area() + c.warp * (2 * NA * stride);
+    // the columns [a0, a1) of segment `col` are this warp's
+    auto range = [&](int col, int &a0, int &a1) {
+        const int cols = min(seg, K - col), nblk = (cols + 63) / 64;
+        a0 = nblk * c.warp / ST_NW * 64;
+        a1 = min(nblk * (c.warp + 1) / ST_NW * 64, cols);
+    };
+    Two v[MT][U];
+    auto ask = [&](int col, int from) {
+        int a0, a1;
+        range(col, a0, a1);
+#pragma unroll
+        for (int t = 0; t < MT; ++t)
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int k = a0 + from + (i * 32 + c.lane) * 2;
+                if (t < m && k < a1) v[t][i] = get2(p.act_ll + static_cast<size_t>(t) * p.act_len + col + k);
+            }
+    };
+    auto take = [&](int col, int from, unsigned char *buf) {
+        int a0, a1;
+        range(col, a0, a1);
+        Spin sp;
+        for (;;) {
+            bool here = true;
+#pragma unroll
+            for (int t = 0; t < MT; ++t)
+#pragma unroll
+                for (int i = 0; i < U; ++i)
+                    if (t < m && a0 + from + (i * 32 + c.lane) * 2 < a1) here = here && pieces_tag(v[t][i].a, tag) && pieces_tag(v[t][i].b, tag);
+            if (__all_sync(0xffffffffu, here)) break;
+            if (!__all_sync(0xffffffffu, sp.again(c.abort(), p.spin_limit))) return false;
+            ask(col, from);
+        }
+        const int padded = (a1 + 63) / 64 * 64;
+#pragma unroll
+        for (int t = 0; t < MT; ++t)
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int k = a0 + from + (i * 32 + c.lane) * 2;
+                const bool on = t < m && k < a1;               // (K is a multiple of 8: pairs are whole; columns past K are zero)
+                if (k < padded)
+#pragma unroll
+                    for (int q = 0; q < S; ++q)
+                        *reinterpret_cast<uint32_t *>(buf + (t * S + q) * stride + (k - a0) * 2) =
+                            on ? static_cast<uint32_t>(piece(v[t][i].a, q)) | static_cast<uint32_t>(piece(v[t][i].b, q)) << 16 : 0u;
+            }
+        return true;
+    };
+    // (a segment of a warp's columns is taken in rounds of 64 U columns; all but the last one wait here)
+    auto stage = [&](int col, unsigned char *buf, bool asked) {
+        int a0, a1;
+        range(col, a0, a1);
+#pragma unroll 1
+        for (int from = 0; from == 0 || a0 + from < a1; from += 64 * U) {
+            if (!(asked && from == 0)) ask(col, from);
+            if (!take(col, from, buf)) return false;
+        }
+        __syncwarp();
+        return true;
+    };
+    int which = 0;
+    bool staged = false;
+    Acc<SETS> acc;
+    acc.clear();
+#pragma unroll 1
+    for (int u = sl.u; u < sl.u1;) {
+        const int n = tile_units(p, ST_DN, u, sl.u1), na = min(n, 8), nb = n - na;
+#pragma unroll 1
+        for (int col = 0; col < K; col += seg) {
+            unsigned char *buf = own + which * NA * stride;
+            if (!staged && !stage(col, buf, false)) return false;
+            const int next = col + seg < K ? col + seg : 0;                    // (0: the next tile starts over)
+            const bool more = next > 0 || u + n < sl.u1;
+            if (more) ask(next, 0);
+            const unsigned char *at;
+            if (!chunk_wait(c, at)) return false;
+            const int cols = min(seg, K - col), rb = cols * 2, nblk = (cols + 63) / 64;
+            const int j0 = nblk * c.warp / ST_NW, j1 = nblk * (c.warp + 1) / ST_NW;
+            const unsigned char *ra = at + min(g, na - 1) * rb + t16, *rc = at + min(na + g, na + nb - 1) * rb + t16;
+            const unsigned char *xb[SETS];
+#pragma unroll
+            for (int s = 0; s < SETS; ++s) xb[s] = buf + min(8 * s + g, NA - 1) * stride + t16;
+#pragma unroll 2
+            for (int j = j0; j < j1; ++j) {
+                uint4 b0[SETS], b1[SETS];
+#pragma unroll
+                for (int s = 0; s < SETS; ++s) {
+                    b0[s] = *reinterpret_cast<const uint4 *>(xb[s] + (j - j0) * 128);
+                    b1[s] = *reinterpret_cast<const uint4 *>(xb[s] + (j - j0) * 128 + 64);
+                }
+                block_mma<SETS>(acc, ra, rc, j * 128, odd, rb - 16 - t16, b0, b1);
+            }
+            chunk_release(c);
+            which ^= 1;
+            staged = more;
+            if (more && !stage(next, own + which * NA * stride, true)) return false;
+        }
+        const int done = u - sl.u;
+        flush<MT, SETS>(c, acc, part, done, na, done + 8, nb);
+        acc.clear();
+        u += n;
+    }
+    return true;
+}
+
+template <int MT> __device__ __forceinline__ bool multiply_any(Ctx<MT> &c, const Slice &sl, unsigned tag) {
+    if (sl.op == ST_DN) return multiply_down<MT>(c, sl, tag);
+    const StepCols &cols = c.p().cols[sl.op];
+    if (cols.segs > 1) return multiply<0, MT>(c, sl);
+    switch (((cols.K + 63) / 64 + ST_NW - 1) / ST_NW) {
+        case 1: return multiply<1, MT>(c, sl);
+        case 2: return multiply<2, MT>(c, sl);
+        case 3: return multiply<3, MT>(c, sl);
+        case 4: return multiply<4, MT>(c, sl);
+        default: return multiply<0, MT>(c, sl);
     }
 }
 

@@ -1,0 +1,4 @@
+#include "step_kernel.cuh"
+namespace edgefm {
+StepKernel step_q8_d128_m1(int G) { return step::kernel_for<128, true, 1>(G); }
+}  // namespace edgefm

@@ -1,0 +1,4 @@
+#include "step_kernel.cuh"
+namespace edgefm {
+StepKernel step_q8_d64_m8(int G) { return step::kernel_for<64, true, 8>(G); }
+}  // namespace edgefm

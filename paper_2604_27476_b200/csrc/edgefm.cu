@@ -149,6 +149,7 @@ struct edgefm_ctx {
     struct Build {
         StepLaunch launch;
         unsigned long long *ll = nullptr;     // exchange buffers
+        unsigned char *maps = nullptr;        // tensor maps of the operators cut into boxes
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
     } step, wide;
@@ -218,6 +219,7 @@ void free_all(edgefm_ctx *c) {
         if (b->exec) cudaGraphExecDestroy(b->exec);
         if (b->graph) cudaGraphDestroy(b->graph);
         if (b->ll) cudaFree(b->ll);
+        if (b->maps) cudaFree(b->maps);
     }
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
     void *bufs[] = {c->k_cache, c->v_cache, c->inv_freq, c->state, c->req, c->prof, c->vocab_ids, c->sub_lm, c->k_scale, c->v_scale, c->d_layers};
@@ -272,6 +274,15 @@ cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char *
     }
     step_wire(&sl, mt, b->ll);
     StepParams &p = sl.p;
+    {
+        std::vector<CUtensorMap> maps(static_cast<size_t>(4 * c->shape.n_layers) + 1);
+        const bool sub = c->vocab_subset > 0;
+        if (!step_maps(p, c->layers.data(), sub ? static_cast<const void *>(c->sub_lm) : c->lm_head, sub ? c->vocab_subset : c->shape.vocab, maps.data())) return cudaErrorUnknown;
+        if (!b->maps && (e = cudaMalloc(reinterpret_cast<void **>(&b->maps), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
+        if ((e = cudaMemcpy(b->maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+        p.maps = b->maps;
+        p.map_fence = 1;   // edgefm_set_vocab_subset rewrites the output layer's map
+    }
     p.k_cache = c->k_cache; p.v_cache = c->v_cache; p.k_scale = c->k_scale; p.v_scale = c->v_scale;
     p.embed = static_cast<const uint16_t *>(c->embed); p.inv_freq = c->inv_freq; p.layers = c->d_layers; p.vocab_ids = c->vocab_ids;
     p.state = c->state; p.req = c->req; p.prof = c->prof; p.prof_stride = c->prof_stride;
@@ -745,6 +756,14 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
     const uint16_t *lm_w = n > 0 ? fresh : static_cast<const uint16_t *>(ctx->lm_head);
     const StepHead head{lm_w, static_cast<const uint16_t *>(ctx->final_norm), n > 0 ? n : ctx->shape.vocab, n > 0 ? 1 : 0, {}};
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_layers + ctx->shape.n_layers, &head, sizeof head, cudaMemcpyHostToDevice, s);
+    CUtensorMap map[2];
+    int k = 0;
+    for (edgefm_ctx::Build *b : {&ctx->step, &ctx->wide}) {
+        if (!b->exec) continue;
+        if (!step_map(&map[k], b->launch.p.cols[ST_LM], lm_w, head.rows)) e = cudaErrorUnknown;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(b->maps + static_cast<size_t>(4 * ctx->shape.n_layers) * sizeof(CUtensorMap), &map[k], sizeof(CUtensorMap), cudaMemcpyHostToDevice, s);
+        ++k;
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host buffers are read before the call returns
     if (e != cudaSuccess) {
         if (fresh) cudaFree(fresh);
@@ -957,6 +976,7 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     double *inv_freq = sc.take<double>(d / 2);
     StepState *state = sc.take<StepState>(1);
     StepRequest *req = sc.take<StepRequest>(1);
+    CUtensorMap *d_maps = sc.take<CUtensorMap>(static_cast<size_t>(4 * sh.n_layers) + 1);
     unsigned long long *ll = sc.take<unsigned long long>(sl.ll_bytes / 8);
     if (sc.off > EDGEFM_STATIC_SCRATCH_BYTES)
         return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "this shape needs %zu bytes of work buffers; the static scratch holds %zu", sc.off,
@@ -969,6 +989,10 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     p.k_cache = static_cast<uint16_t *>(k_cache); p.v_cache = static_cast<uint16_t *>(v_cache);
     p.embed = static_cast<const uint16_t *>(weights->embed); p.inv_freq = inv_freq; p.layers = d_layers;
     p.state = state; p.req = req;
+    p.maps = reinterpret_cast<const unsigned char *>(d_maps);
+    p.map_fence = 2;   // every call rewrites all tensor maps in the shared scratch
+    std::vector<CUtensorMap> maps(static_cast<size_t>(4 * sh.n_layers) + 1);
+    if (!step_maps(p, weights->layers, weights->lm_head, sh.vocab, maps.data())) return fail(nullptr, EDGEFM_ERR_CUDA, "cuTensorMapEncodeTiled failed");
 
     // ---- stream-ordered set-up of the shared scratch: it still holds the previous call's contents ----------
     double inv[64];
@@ -980,6 +1004,7 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     CUDA_TRY(nullptr, cudaMemsetAsync(ll, 0, sl.ll_bytes, s));
     // pageable copies: the runtime stages the bytes before returning, so the sources may be freed after the call
     CUDA_TRY(nullptr, cudaMemcpyAsync(d_layers, layers.data(), layers.size() * sizeof(StepLayer), cudaMemcpyHostToDevice, s));
+    CUDA_TRY(nullptr, cudaMemcpyAsync(d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(inv_freq, inv, static_cast<size_t>(d / 2) * sizeof(double), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(state, &st, sizeof st, cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(req, &rq, sizeof rq, cudaMemcpyHostToDevice, s));

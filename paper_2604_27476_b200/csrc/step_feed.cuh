@@ -8,7 +8,8 @@ namespace step {
 // Calls f(part) for every chunk of the whole step in order, until f returns false.  A chunk is one or two parts of `rows` segments of
 // `seg` bytes, `stride` bytes apart in memory and packed in the ring (p1 null: one part).  Run by whole warps: the lanes share out the
 // copies.
-struct Part { const unsigned char *p0, *p1; int rows; unsigned seg, stride; bool kv; };
+// With a tensor map: boxes at (0, row, block) and, for pairs, (0, row1, block) of `seg` bytes each.
+struct Part { const unsigned char *p0, *p1; int rows; unsigned seg, stride; bool kv; const unsigned char *map; int row, row1, block; };
 template <bool Q8, int MT, typename F>
 __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f) {
     const Shared<MT> &sh = c.sh();
@@ -24,7 +25,7 @@ __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f) {
                 for (int idx = c.cta; idx < sh.m * p.nkv * sh.n_chunks; idx += c.ncta) {
                     const KvShare share = kv_share(p, sh.n_old, sh.n_chunks, idx);
                     const size_t at = ((static_cast<size_t>(layer) * p.nkv + share.g) * p.max_context + share.t0) * (p.D * E);
-                    Part t{reinterpret_cast<const unsigned char *>(p.k_cache) + at, reinterpret_cast<const unsigned char *>(p.v_cache) + at, 1, 0u, 0u, true};
+                    Part t{reinterpret_cast<const unsigned char *>(p.k_cache) + at, reinterpret_cast<const unsigned char *>(p.v_cache) + at, 1, 0u, 0u, true, nullptr, 0, 0, 0};
 #pragma unroll 1
                     for (int pos = share.t0; pos < share.t1; pos += ST_KV_BLOCK) {
                         t.seg = static_cast<unsigned>(min(ST_KV_BLOCK, share.t1 - pos) * p.D * E);
@@ -45,9 +46,20 @@ __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f) {
 #pragma unroll 1
             for (int u = u0; u < u1;) {
                 const int n = tile_units(p, op, u, u1);
-                Part t{w, paired ? w + partner : nullptr, whole ? 1 : n, whole ? static_cast<unsigned>(n) * row_bytes : seg, row_bytes, false};
+                Part t{w, paired ? w + partner : nullptr, whole ? 1 : n, whole ? static_cast<unsigned>(n) * row_bytes : seg, row_bytes, false, nullptr, 0, 0, 0};
                 if (whole) {
                     if (!f(t)) return;
+                } else if (p.cols[op].box_rows) {
+                    t.map = p.maps + static_cast<size_t>(4 * layer + (op == ST_LM ? 0 : op)) * 128;
+                    t.rows = 1;
+                    t.seg = seg * static_cast<unsigned>(p.cols[op].box_rows);
+                    t.row = op == ST_QKV ? (u >> p.half_shift) * p.D + (u & (half - 1)) : u;
+                    t.row1 = t.row + (op == ST_QKV ? half : p.F);
+#pragma unroll 1
+                    for (int k = p.cols[op].segs; k > 0; --k) {
+                        if (!f(t)) return;
+                        t.block += p.cols[op].seg >> 6;
+                    }
                 } else {
 #pragma unroll 1
                     for (unsigned at = 0; at < row_bytes; at += seg) {
@@ -77,6 +89,7 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
     unsigned issued = 0, freed = 0;              // chunks copied / released so far
     unsigned at = 0, tail = 0;                   // next offset; start of the oldest chunk still in use
     unsigned sent = 0;                           // 16-byte units copied so far
+    const unsigned char *fenced = nullptr;
     bool ok = true;
     for_each_chunk<Q8>(c, [&](const Part &t) {
         const unsigned part = static_cast<unsigned>(t.rows) * t.seg, bytes = t.p1 ? 2 * part : part, need = (bytes + 127u) & ~127u;
@@ -100,7 +113,21 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
         }
         __syncwarp();
         const int r = c.lane & 15;
-        if (r < t.rows && (c.lane < 16 || t.p1)) {
+        if (t.map) {
+            if (c.lane == 0 && (p.map_fence == 2 || (p.map_fence == 1 && t.map == p.maps + static_cast<size_t>(4 * p.n_layers) * 128)) && t.map != fenced) {
+                // order the copy engine's view of a map the host may have rewritten behind what is in memory now
+                fenced = t.map;
+                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(t.map) : "memory");
+            }
+            if (c.lane == 0)
+                asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(ring_at + at),
+                             "l"(t.map), "r"(0), "r"(t.row), "r"(t.block), "r"(bar), "l"(once)
+                             : "memory");
+            if (c.lane == 0 && t.p1)
+                asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(ring_at + at + part),
+                             "l"(t.map), "r"(0), "r"(t.row1), "r"(t.block), "r"(bar), "l"(once)
+                             : "memory");
+        } else if (r < t.rows && (c.lane < 16 || t.p1)) {
             const unsigned char *src = (c.lane < 16 ? t.p0 : t.p1) + static_cast<size_t>(r) * t.stride;
             const unsigned dst = ring_at + at + (c.lane < 16 ? 0u : part) + static_cast<unsigned>(r) * t.seg;
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(dst), "l"(src), "r"(t.seg),
@@ -137,7 +164,12 @@ __device__ __forceinline__ void feed_l2(Ctx<MT> &c) {
         }
         if (lead <= 0) return true;              // the ring has it already
         const int r = c.lane & 15;
-        if (r < t.rows && (c.lane < 16 || t.p1))
+        if (t.map) {
+            if (c.lane == 0 && c.p().map_fence != 2 && t.map != c.p().maps + static_cast<size_t>(4 * c.p().n_layers) * 128) {   // (only through maps that are never rewritten)
+                asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(t.map), "r"(0), "r"(t.row), "r"(t.block) : "memory");
+                if (t.p1) asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(t.map), "r"(0), "r"(t.row1), "r"(t.block) : "memory");
+            }
+        } else if (r < t.rows && (c.lane < 16 || t.p1))
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((c.lane < 16 ? t.p0 : t.p1) + static_cast<size_t>(r) * t.stride), "r"(t.seg) : "memory");
         return true;
     });

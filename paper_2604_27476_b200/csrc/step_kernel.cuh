@@ -71,11 +71,6 @@ __device__ __forceinline__ void finish_unit(const Ctx<MT> &c, int op, int layer,
         if (arg_better(lo, j, best_v, best_i)) { best_v = lo; best_i = j; }
     }
 }
-__device__ __forceinline__ float sum8(const float *at) {
-    const float4 a = *reinterpret_cast<const float4 *>(at), b = *reinterpret_cast<const float4 *>(at + 4);
-    return ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
-}
-
 __device__ __forceinline__ void arg_fold(float &v, int &i) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -250,7 +245,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
                     }
                 }
             } else if (mine) {
-                const float tot = sum8(sh.ss[tok]), r = rsqrtf(tot / static_cast<float>(p.H) + p.eps);       // the deferred RMSNorm factor
+                const float r = rsqrtf(sh.ss[tok] / static_cast<float>(p.H) + p.eps);       // the deferred RMSNorm factor
                 const float *a = part + (tok * RB + j - ub) * ST_NW;
                 const float lo = sum8(a) * r, hi = paired ? sum8(a + RB / 2 * ST_NW) * r : 0.f;
                 finish_unit<D, Q8, MT>(c, op, layer, tok, j, u0, lo, hi, add_lo, add_hi, best_v, best_i);

@@ -163,6 +163,11 @@ __device__ __forceinline__ int folded(int sub, int lpr) {
     return idx;
 }
 
+__device__ __forceinline__ float sum8(const float *at) {
+    const float4 a = *reinterpret_cast<const float4 *>(at), b = *reinterpret_cast<const float4 *>(at + 4);
+    return ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
+}
+
 // ---- shared memory ---------------------------------------------------------------------------------------------------
 // Dynamic: Shared | ring | layer table, unit tables, residual rows | one area for the staged vector, the attention's scratch and the
 // segments of the MLP activations (they follow one another; between the last reader of one and the first writer of the next
@@ -172,7 +177,7 @@ template <int MT> struct Shared {
     unsigned long long full[ST_BARS], empty[ST_BARS];
     unsigned chunk_at[ST_BARS];                            // ring offset of the chunk behind every barrier
     float rope[MT][128];                                   // per token: cos | sin of its position
-    alignas(16) float ss[MT][ST_NW];                       // partial sums of squares (RMSNorm)
+    float ss[MT];                                          // sums of squares (RMSNorm)
     alignas(16) float part[2][MT * st_batch(MT) * ST_NW];  // partial row sums [token][row][warp], two batches
     alignas(16) float merged[MT][128];                     // attention outputs this CTA owns
     float best_v[ST_NW];

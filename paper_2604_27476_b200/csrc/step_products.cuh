@@ -42,70 +42,88 @@ template <int MT> __device__ __forceinline__ bool stage_embedding(Ctx<MT> &c, co
             store_pieces(c, t, i, p.H, pieces_packet(v * bf16_bits_to_f32(norm_w[i]), 0u));
         }
         ss = warp_sum(ss);
-        if (c.lane == 0) c.sh().ss[t][c.warp] = ss;
+        if (c.lane == 0) c.sh().merged[0][t * ST_NW + c.warp] = ss;      // (not in use yet)
     }
     zero_tail(c, p.H);
+    if (!cta_vote(true)) return false;
+    if (c.tid < c.sh().m) c.sh().ss[c.tid] = sum8(&c.sh().merged[0][c.tid * ST_NW]);
     return cta_vote(true);
 }
 // Wait for all values of the vectors of all tokens (K columns, lines of `line` packets) and leave their pieces in shared memory, and meet.
 // sums: the last packet of every line is a partial sum of squares.
 template <int MT>
 __device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int total, int K, const unsigned long long *ll, int line, bool sums, unsigned tag) {
-    constexpr int U = 4;     // units in flight per thread
-    const int m = c.sh().m;
+    constexpr int U = MT == 1 ? 4 : 7, W = 5;     // units in flight per thread; lines whose sums a lane reads together
+    const int m = c.sh().m, all = m * total;
     bool ok = true;
+    // the sums of squares of token w are added by warp w; asked for first, awaited last
+    const unsigned long long *const sums_at = ll + static_cast<size_t>(c.warp) * c.ncta * line + line - 1;
+    const bool adds = sums && c.warp < m;
+    unsigned long long s[W] = {0ull, 0ull, 0ull, 0ull, 0ull};
+    auto ask = [&](int base) {
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (base + 32 * i < c.ncta) s[i] = get1(sums_at + static_cast<size_t>(base + 32 * i) * line);
+    };
+    if (adds) ask(c.lane);
     zero_tail(c, K);
 #pragma unroll 1
-    for (int tok = 0; tok < m && ok; ++tok) {
-        const unsigned long long *lt = ll + static_cast<size_t>(tok) * c.ncta * line;
-#pragma unroll 1
-        for (int base = c.tid; base < total; base += U * ST_NT) {
-            unsigned e[U];
-            Two t[U];
-            unsigned todo = 0;
+    for (int base = c.tid; base < all; base += U * ST_NT) {
+        unsigned e[U], at[U];
+        Two t[U];
+        unsigned todo = 0;
 #pragma unroll
-            for (int i = 0; i < U; ++i) {
-                const int u = base + i * ST_NT;
-                e[i] = u < total ? tab[u] : 0u;
-                if ((e[i] >> 16) & 3u) todo |= 1u << i;
-            }
+        for (int i = 0; i < U; ++i) {
+            const int u = base + i * ST_NT;
+            int tok = 0;
+            if constexpr (MT > 1) tok = u / total;
+            e[i] = u < all ? tab[u - tok * total] : 0u;
+            at[i] = (e[i] >> 18) * 2 + static_cast<unsigned>(tok * c.ncta * line);
+            e[i] = (e[i] & 0x3ffffu) | static_cast<unsigned>(tok) << 18;
+            if ((e[i] >> 16) & 3u) todo |= 1u << i;
+        }
+        Spin sp;
+        for (;;) {
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                if (todo >> i & 1u) t[i] = get2(ll + at[i]);
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                if (todo >> i & 1u) {
+                    const bool two = (e[i] >> 16 & 3u) > 1;
+                    if (pieces_tag(t[i].a, tag) && (!two || pieces_tag(t[i].b, tag))) {
+                        todo &= ~(1u << i);
+                        const int row = e[i] & 0xffffu, tok = static_cast<int>(e[i] >> 18);
+                        store_pieces(c, tok, row, K, t[i].a);
+                        if (two) store_pieces(c, tok, row + 1, K, t[i].b);
+                    }
+                }
+            if (!todo) break;
+            if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+        }
+        if (!ok) break;
+    }
+    if (adds) {
+        float ss = 0.f;
+#pragma unroll 1
+        for (int base = c.lane; base < c.ncta && ok; base += 32 * W) {
+            if (base != c.lane) ask(base);
             Spin sp;
             for (;;) {
+                bool here = true;
 #pragma unroll
-                for (int i = 0; i < U; ++i)
-                    if (todo >> i & 1u) t[i] = get2(lt + static_cast<size_t>(e[i] >> 18) * 2);
-#pragma unroll
-                for (int i = 0; i < U; ++i)
-                    if (todo >> i & 1u) {
-                        const bool two = (e[i] >> 16 & 3u) > 1;
-                        if (pieces_tag(t[i].a, tag) && (!two || pieces_tag(t[i].b, tag))) {
-                            todo &= ~(1u << i);
-                            const int row = e[i] & 0xffffu;
-                            store_pieces(c, tok, row, K, t[i].a);
-                            if (two) store_pieces(c, tok, row + 1, K, t[i].b);
-                        }
-                    }
-                if (!todo) break;
+                for (int i = 0; i < W; ++i)
+                    if (base + 32 * i < c.ncta) here = here && packet_tag(s[i]) == tag;
+                if (here) break;
                 if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+                ask(base);
             }
-            if (!ok) break;
+#pragma unroll
+            for (int i = 0; i < W; ++i)
+                if (base + 32 * i < c.ncta) ss += packet_value(s[i]);
         }
-        if (sums) {
-            float ss = 0.f;
-#pragma unroll 1
-            for (int w = c.tid; w < c.ncta && ok; w += ST_NT) {
-                const unsigned long long *at = lt + static_cast<size_t>(w) * line + line - 1;
-                unsigned long long v = get1(at);
-                Spin sp;
-                while (packet_tag(v) != tag) {
-                    if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
-                    v = get1(at);
-                }
-                ss += packet_value(v);
-            }
-            ss = warp_sum(ss);
-            if (c.lane == 0) c.sh().ss[tok][c.warp] = ss;
-        }
+        ss = warp_sum(ss);
+        if (c.lane == 0) c.sh().ss[c.warp] = ss;
     }
     return cta_vote(ok);
 }
@@ -136,7 +154,7 @@ template <int SETS> struct Acc {       // row sums of a tile: two independent ch
             for (int q = 0; q < 2; ++q) d[s][q][0] = d[s][q][1] = d[s][q][2] = d[s][q][3] = 0.f;
     }
 };
-// Block j (64 columns) of a chunk: rows ra / rb (this lane's), `last` = offset of the last 16 bytes of a row; bv: B registers.
+// A block (64 columns) of a chunk at offset `off`: rows ra / rb (this lane's), `last` = offset of the last 16 bytes of a row.
 template <int SETS>
 __device__ __forceinline__ void block_mma(Acc<SETS> &acc, const unsigned char *ra, const unsigned char *rb, int off, bool odd, int last, const uint4 (&b0)[SETS], const uint4 (&b1)[SETS]) {
     const int o0 = min(off + (odd ? 64 : 0), last), o1 = min(off + (odd ? 0 : 64), last);    // (past the row: the vector is zero there)
@@ -185,6 +203,17 @@ __device__ __forceinline__ void flush(const Ctx<MT> &c, Acc<SETS> &acc, float *p
             }
         }
     }
+}
+
+// This lane's two rows of a chunk cut by columns: their first bytes, the distance of the 64-column blocks, the last readable offset.
+struct Rows { const unsigned char *a, *b; int block, last; };
+__device__ __forceinline__ Rows rows_of(const unsigned char *at, int g, int na, int nb, int row_bytes, bool paired, const StepCols &cols, int t16) {
+    const int r0 = min(g, na - 1);
+    if (cols.box_rows == 0) return Rows{at + r0 * row_bytes + t16, at + min(na + g, na + nb - 1) * row_bytes + t16, 128, row_bytes - 16 - t16};
+    // boxes: [block][row][128 bytes]; the partners of a pair are a box of their own
+    const int r1 = paired ? r0 : min(na + g, na + nb - 1);
+    const unsigned char *second = paired ? at + cols.box_rows * cols.seg * 2 : at;
+    return Rows{at + r0 * 128 + t16, second + r1 * 128 + t16, cols.box_rows * 128, 1 << 30};
 }
 
 struct Slice { int u, u1, op, batch; };      // units [u, u1) of an operator; the batch of partial sums they go to
@@ -236,9 +265,9 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
             for (int col = 0; col < K; col += seg) {
                 const unsigned char *at;
                 if (!chunk_wait(c, at)) return false;
-                const int cols = min(seg, K - col), rb = cols * 2, nblk = (cols + 63) / 64;
+                const int cols = min(seg, K - col), nblk = (cols + 63) / 64;
                 const int j0 = nblk * c.warp / ST_NW, j1 = nblk * (c.warp + 1) / ST_NW;
-                const unsigned char *ra = at + min(g, na - 1) * rb + t16, *rc = at + min(na + g, na + nb - 1) * rb + t16;
+                const Rows r = rows_of(at, g, na, nb, cols * 2, paired, p.cols[sl.op], t16);
 #pragma unroll 2
                 for (int j = j0; j < j1; ++j) {
                     uint4 b0[SETS], b1[SETS];
@@ -248,7 +277,7 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
                         b0[s] = *reinterpret_cast<const uint4 *>(x);
                         b1[s] = *reinterpret_cast<const uint4 *>(x + 64);
                     }
-                    block_mma<SETS>(acc, ra, rc, j * 128, odd, rb - 16 - t16, b0, b1);
+                    block_mma<SETS>(acc, r.a, r.b, j * r.block, odd, r.last, b0, b1);
                 }
                 chunk_release(c);
             }
@@ -348,9 +377,9 @@ __device__ __forceinline__ bool multiply_down(Ctx<MT> &c, const Slice &sl, unsig
             if (more) ask(next, 0);
             const unsigned char *at;
             if (!chunk_wait(c, at)) return false;
-            const int cols = min(seg, K - col), rb = cols * 2, nblk = (cols + 63) / 64;
+            const int cols = min(seg, K - col), nblk = (cols + 63) / 64;
             const int j0 = nblk * c.warp / ST_NW, j1 = nblk * (c.warp + 1) / ST_NW;
-            const unsigned char *ra = at + min(g, na - 1) * rb + t16, *rc = at + min(na + g, na + nb - 1) * rb + t16;
+            const Rows r = rows_of(at, g, na, nb, cols * 2, false, p.cols[ST_DN], t16);
             const unsigned char *xb[SETS];
 #pragma unroll
             for (int s = 0; s < SETS; ++s) xb[s] = buf + min(8 * s + g, NA - 1) * stride + t16;
@@ -362,7 +391,7 @@ __device__ __forceinline__ bool multiply_down(Ctx<MT> &c, const Slice &sl, unsig
                     b0[s] = *reinterpret_cast<const uint4 *>(xb[s] + (j - j0) * 128);
                     b1[s] = *reinterpret_cast<const uint4 *>(xb[s] + (j - j0) * 128 + 64);
                 }
-                block_mma<SETS>(acc, ra, rc, j * 128, odd, rb - 16 - t16, b0, b1);
+                block_mma<SETS>(acc, r.a, r.b, j * r.block, odd, r.last, b0, b1);
             }
             chunk_release(c);
             which ^= 1;

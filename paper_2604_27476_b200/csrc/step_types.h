@@ -6,6 +6,7 @@
 
 #include "../../include/edgefm.h"
 #include "common.cuh"
+#include "step_plan.h"
 
 namespace edgefm {
 
@@ -37,8 +38,12 @@ enum { ST_QKV = 0, ST_O = 1, ST_GU = 2, ST_DN = 3, ST_LM = 4 };
 // How an operator with rows of K values is cut: tiles of 16 rows (8 pairs); a tile whose rows are too long for a ring chunk is cut into
 // `segs` segments of `seg` columns.  All warps work on every chunk: warp w multiplies the 64-column blocks [nb w / 8, nb (w + 1) / 8) of
 // the nb blocks of the chunk, and so needs only that part of the input vector.
+// A segment comes as one box (two for pairs) of a tensor map: box_rows rows (8 or 16, or the most a CTA owns; what lies past the tile
+// is not used) x seg columns, delivered as [64-column block][row][128 bytes].  (One bulk copy per row segment costs the copy unit about
+// 150 cycles whatever its size: 11 rows of 4 KB took 2.6 TB/s, as a box they come at the rate of whole rows.)  box_rows 0: K is not a
+// multiple of 64, one copy per row segment.
 struct StepCols {
-    int K, seg, segs;
+    int K, seg, segs, box_rows;
 };
 
 // Pointers of a layer; entry [n_layers] describes the output layer.
@@ -65,6 +70,8 @@ struct StepParams {
     const uint16_t *embed;
     const double *inv_freq;        // [D / 2]
     const StepLayer *layers;       // [n_layers + 1]
+    const unsigned char *maps;     // CUtensorMap [4 n_layers + 1] of the operators that are cut into boxes (128 bytes each)
+    int map_fence;                 // maps the host may have rewritten since the last launch: 1 the output layer's, 2 all
     const int *vocab_ids;
     StepState *state;
     const StepRequest *req;
@@ -98,13 +105,14 @@ __host__ __device__ inline int st_first(int n, int c, int ncta) { return static_
 __host__ __device__ inline int st_line(int most) { return (most + 15) / 16 * 16; }   // packets of a line: whole 128 bytes
 
 // How an operator with rows of K values and at most `rows` of them in a tile is cut.
-inline StepCols step_cols(int K, int rows, int max_seg = 1 << 30) {
-    StepCols c{K, K, 1};
+inline StepCols step_cols(int K, int rows, bool paired, int max_seg = 1 << 30) {
+    StepCols c{K, K, 1, 0};
     if (rows * K * 2 <= ST_CHUNK_WHOLE && K <= max_seg) return c;
     const int most = std::min(max_seg, std::max(512, ST_CHUNK_BYTES / (2 * rows) / 512 * 512));
     const int n = (K + most - 1) / most;
     c.seg = std::min(most, ((K + n - 1) / n + 511) / 512 * 512);      // a whole number of blocks for every warp
     c.segs = (K + c.seg - 1) / c.seg;
+    if (K % 64 == 0) c.box_rows = paired ? rows / 2 : rows;
     return c;
 }
 // Bytes between the arrays of a staged vector of n columns: whole 64-column blocks, + 64 so that neighbouring arrays use other banks.
@@ -139,10 +147,10 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.max_context = max_context;
     auto most = [&](int n) { return (n + grid - 1) / grid; };
     const int h_rows = std::min(ST_TILE, most(H));
-    p.cols[ST_QKV] = p.cols[ST_GU] = step_cols(H, ST_TILE);
-    p.cols[ST_LM] = step_cols(H, ST_TILE);
-    p.cols[ST_O] = step_cols(qd, h_rows);
-    p.cols[ST_DN] = step_cols(F, h_rows, mt <= 2 ? 2048 : 1024);      // (two segments of activations are in shared memory, as pieces)
+    p.cols[ST_QKV] = p.cols[ST_GU] = step_cols(H, ST_TILE, true);
+    p.cols[ST_LM] = step_cols(H, ST_TILE, false);
+    p.cols[ST_O] = step_cols(qd, h_rows, false);
+    p.cols[ST_DN] = step_cols(F, h_rows, false, mt <= 2 ? 2048 : 1024);      // (two segments of activations are in shared memory, as pieces)
     p.x_line = st_line(most(H) + 1);
     p.q_line = st_line(2 * most((nq + 2 * nkv) * D / 2));
     p.ao_line = st_line(2 * most(qd / 2));
@@ -180,6 +188,27 @@ inline void step_wire(StepLaunch *sl, int mt, unsigned long long *base) {
     p.act_ll = base; base += m * p.act_len;
     p.part_ll = base; base += chunks * p.qd;
     p.stat_ll = base;
+}
+// Tensor map of a row-major bf16 [rows][K] matrix for the boxes of an operator: the 64-column blocks of a row are the last dimension.
+inline bool step_map(CUtensorMap *m, const StepCols &c, const void *base, int rows) {
+    std::memset(m, 0, sizeof *m);
+    if (c.box_rows == 0) return true;
+    TensorMapEncodeFn enc = tensor_map_encoder();
+    if (!enc) return false;
+    const cuuint64_t dims[3] = {64, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(c.K / 64)}, strides[2] = {static_cast<cuuint64_t>(c.K) * 2, 128};
+    const cuuint32_t box[3] = {64, static_cast<cuuint32_t>(c.box_rows), static_cast<cuuint32_t>(c.seg / 64)}, es[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// All of them: [4 layer + operator], the output layer last.
+inline bool step_maps(const StepParams &p, const edgefm_layer_weights *layers, const void *lm_head, int lm_rows, CUtensorMap *maps) {
+    for (int l = 0; l < p.n_layers; ++l) {
+        const edgefm_layer_weights &w = layers[l];
+        if (!step_map(maps + 4 * l + ST_QKV, p.cols[ST_QKV], w.wqkv, (p.nq + 2 * p.nkv) * p.D) || !step_map(maps + 4 * l + ST_O, p.cols[ST_O], w.wo, p.H) ||
+            !step_map(maps + 4 * l + ST_GU, p.cols[ST_GU], w.w_gate_up, 2 * p.F) || !step_map(maps + 4 * l + ST_DN, p.cols[ST_DN], w.w_down, p.H))
+            return false;
+    }
+    return step_map(maps + 4 * p.n_layers, p.cols[ST_LM], lm_head, lm_rows);
 }
 // One entry per layer, then the output layer.
 inline void step_layers(const edgefm_shape &sh, const edgefm_layer_weights *layers, const void *final_norm, const void *lm_head, StepLayer *out) {

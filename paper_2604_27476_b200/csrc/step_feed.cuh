@@ -175,5 +175,66 @@ __device__ __forceinline__ void feed_l2(Ctx<MT> &c) {
     });
 }
 
+// A third warp brings the vectors: when all CTAs have arrived, one bulk copy (they lie in memory as they are wanted in shared memory).
+// MLP activations come segment by segment, a few ahead of the products.  That a copy may overwrite the area follows from this CTA's
+// own arrival: it comes after the last read of what was there.
+template <int MT>
+__device__ __forceinline__ void feed_vectors(Ctx<MT> &c) {
+    Shared<MT> &sh = c.sh();
+    const StepParams &p = c.p();
+    constexpr int NA = Ctx<MT>::NA;
+    unsigned k = 0, target = static_cast<unsigned>(p.state->epoch[p.epoch_slot]) * static_cast<unsigned>(4 * p.n_layers * c.ncta) + static_cast<unsigned>(p.barrier_extra);
+    bool ok = true;
+    auto everybody = [&]() {                     // wait for the next exchange's arrivals
+        target += static_cast<unsigned>(c.ncta);
+        Spin sp;
+        for (;;) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.arrivals) : "memory");
+            if (static_cast<int>(v - target) >= 0) break;
+            if (!sp.again(c.abort(), p.spin_limit)) return false;
+        }
+        asm volatile("fence.proxy.async;" ::: "memory");
+        return true;
+    };
+    auto copy = [&](const unsigned char *from, unsigned to, int bytes) {
+        unsigned long long *bar = &sh.x_full[k & 3u];
+        mbar_expect_tx(bar, static_cast<unsigned>(bytes));
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(c.area()) + to), "l"(from), "r"(bytes),
+                     "r"(smem_u32(bar))
+                     : "memory");
+        ++k;
+    };
+    const int vec = NA * st_array_bytes(p.H) + 4 * MT * p.ss_stride, slot = NA * st_array_bytes(p.cols[ST_DN].seg), segs = p.cols[ST_DN].segs;
+    const int tiles = (sh.u1[ST_DN] - sh.u0[ST_DN] + ST_TILE - 1) / ST_TILE;
+#pragma unroll 1
+    for (int layer = 0; layer <= p.n_layers && ok; ++layer) {
+        if (layer > 0) {
+            ok = everybody();
+            if (ok) copy(p.x_vec, 0u, vec);
+        }
+        if (!ok || layer == p.n_layers) break;
+        ok = everybody();
+        if (!ok) break;
+        copy(p.ao_vec, 0u, NA * st_array_bytes(p.qd));
+        ok = everybody();
+        if (!ok) break;
+        copy(p.xo_vec, 0u, vec);
+        ok = everybody();
+        if (!ok) break;
+        const unsigned first = k;
+#pragma unroll 1
+        for (int i = 0; i < tiles * segs && ok; ++i) {
+            const unsigned back = k - static_cast<unsigned>(p.act_slots);
+            if (k - first >= static_cast<unsigned>(p.act_slots)) ok = mbar_wait(&sh.x_empty[back & 3u], (back >> 2) & 1u, c.abort(), p.spin_limit);
+            if (ok) copy(p.act_vec + static_cast<size_t>(i % segs) * slot, static_cast<unsigned>(i % p.act_slots) * slot, slot);
+        }
+    }
+    if (!ok) {               // giving up: the copies in flight must land before the CTA's shared memory is released
+        int dummy = 0;
+        for (unsigned j = k > 4 ? k - 4 : 0; j < k; ++j) mbar_wait(&sh.x_full[j & 3u], (j >> 2) & 1u, &dummy, p.spin_limit);
+    }
+}
+
 }  // namespace step
 }  // namespace edgefm

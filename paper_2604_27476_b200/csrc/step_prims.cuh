@@ -89,29 +89,6 @@ __device__ __forceinline__ Two get2(const unsigned long long *at) {
 }
 __device__ __forceinline__ bool both(const Two &t, unsigned tag) { return packet_tag(t.a) == tag && packet_tag(t.b) == tag; }
 
-// Packets of pieces: three bf16 (value = their sum) and the low 16 bits of the tag.  A slot is rewritten with the next tag every layer
-// (every token's, used or not), so 16 bits tell the contents apart.
-__device__ __forceinline__ unsigned long long pieces_packet(float v, unsigned tag) {
-    const uint16_t hi = f32_to_bf16_bits(v);
-    v -= bf16_bits_to_f32(hi);           // exact: the remainder is what the next piece holds
-    const uint16_t mid = f32_to_bf16_bits(v);
-    const uint16_t lo = f32_to_bf16_bits(v - bf16_bits_to_f32(mid));
-    return static_cast<unsigned long long>(hi | static_cast<unsigned>(mid) << 16) | static_cast<unsigned long long>(lo | tag << 16) << 32;
-}
-__device__ __forceinline__ bool pieces_tag(unsigned long long p, unsigned tag) { return static_cast<unsigned>(p >> 48) == (tag & 0xffffu); }
-__device__ __forceinline__ uint16_t piece(unsigned long long p, int i) { return static_cast<uint16_t>(p >> (16 * i)); }
-__device__ __forceinline__ void put_raw(unsigned long long *at, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(at), "l"(v) : "memory");
-}
-__device__ __forceinline__ void put_raw2(unsigned long long *at, unsigned long long a, unsigned long long b) {
-    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(at), "l"(a), "l"(b) : "memory");
-}
-__device__ __forceinline__ unsigned long long get1(const unsigned long long *at) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(at) : "memory");
-    return v;
-}
-
 // Two fp32 values in one 64-bit register pair.
 using f2 = unsigned long long;
 __device__ __forceinline__ f2 pack2(float a, float b) {
@@ -169,12 +146,13 @@ __device__ __forceinline__ float sum8(const float *at) {
 }
 
 // ---- shared memory ---------------------------------------------------------------------------------------------------
-// Dynamic: Shared | ring | layer table, unit tables, residual rows | one area for the staged vector, the attention's scratch and the
+// Dynamic: Shared | ring | layer table, residual rows | one area for the staged vector, the attention's scratch and the
 // segments of the MLP activations (they follow one another; between the last reader of one and the first writer of the next
 // lies a CTA-wide vote).
 extern __shared__ __align__(128) unsigned char st_smem[];
 template <int MT> struct Shared {
     unsigned long long full[ST_BARS], empty[ST_BARS];
+    unsigned long long x_full[4], x_empty[4];              // staged vectors / segments of the MLP activations
     unsigned chunk_at[ST_BARS];                            // ring offset of the chunk behind every barrier
     float rope[MT][128];                                   // per token: cos | sin of its position
     float ss[MT];                                          // sums of squares (RMSNorm)
@@ -183,9 +161,9 @@ template <int MT> struct Shared {
     float best_v[ST_NW];
     int best_i[ST_NW];
     int u0[5], u1[5];                                      // this CTA's units of every operator
-    unsigned tag0, odd;                                    // tag of layer 0; test hook: a bit no tag has
+    unsigned tag0;                                         // tag of layer 0
     int tokens[MT];
-    int m, pos, n_old, n_chunks, total_x, total_a;         // the call's tokens, first position, cache length; attention chunks per kv head and token; sizes of the unit tables
+    int m, pos, n_old, n_chunks;                           // the call's tokens, first position, cache length; attention chunks per kv head and token
     unsigned sent;                                         // 16-byte units the feeding warp has asked for
     int abort;
 };
@@ -197,9 +175,10 @@ template <int MT> struct Ctx {
     static constexpr int S = st_pieces(MT), NA = st_arrays(MT), RB = st_batch(MT);
     const StepParams &par;
     int tid, warp, lane, cta, ncta;
-    unsigned chunk;          // next ring chunk to consume
+    unsigned chunk, xchunk;  // next ring chunk / staged vector to consume
+    int act_slot;            // MLP activations: which of the segments in shared memory is next
     __device__ __forceinline__ explicit Ctx(const StepParams &p_)
-        : par(p_), tid(static_cast<int>(threadIdx.x)), warp(tid >> 5), lane(tid & 31), cta(static_cast<int>(blockIdx.x)), ncta(static_cast<int>(gridDim.x)), chunk(0u) {}
+        : par(p_), tid(static_cast<int>(threadIdx.x)), warp(tid >> 5), lane(tid & 31), cta(static_cast<int>(blockIdx.x)), ncta(static_cast<int>(gridDim.x)), chunk(0u), xchunk(0u), act_slot(0) {}
     __device__ __forceinline__ Shared<MT> &sh() const { return *reinterpret_cast<Shared<MT> *>(st_smem); }
     __device__ __forceinline__ const StepParams &p() const { return par; }
     __device__ __forceinline__ volatile int *abort() const { return &sh().abort; }
@@ -207,11 +186,8 @@ template <int MT> struct Ctx {
     __device__ __forceinline__ unsigned char *tables() const { return ring() + p().ring_bytes; }
     __device__ __forceinline__ const StepLayer *layer(int l) const { return reinterpret_cast<const StepLayer *>(tables()) + l; }
     __device__ __forceinline__ const StepHead &head() const { return *reinterpret_cast<const StepHead *>(layer(p().n_layers)); }
-    __device__ __forceinline__ unsigned *unit_table() const { return reinterpret_cast<unsigned *>(tables() + (p().n_layers + 1) * 64); }
     __device__ __forceinline__ float *resid() const { return reinterpret_cast<float *>(tables() + p().resid_at); }   // [token][this CTA's rows of the residual stream]
     __device__ __forceinline__ unsigned char *area() const { return tables() + p().table_bytes; }
-    // Column `col` of array `a` of a staged vector of K columns: array = token * S + piece, bf16, in natural order.
-    __device__ __forceinline__ uint16_t *xs(int a, int col, int K) const { return reinterpret_cast<uint16_t *>(area() + a * st_array_bytes(K)) + col; }
 };
 
 template <int MT> __device__ __forceinline__ void stamp(const Ctx<MT> &c, int &idx) {
@@ -234,6 +210,38 @@ template <int MT> __device__ __forceinline__ void chunk_release(Ctx<MT> &c) {
     __syncwarp();
     if (c.lane == 0) mbar_arrive(&c.sh().empty[c.chunk & (ST_BARS - 1)]);
     ++c.chunk;
+}
+
+__device__ __forceinline__ void store_u16(unsigned char *at, uint16_t v) { *reinterpret_cast<uint16_t *>(at) = v; }
+// The pieces of value v to column `col` of token tok's arrays (`stride` bytes apart) at `base`.
+template <int MT> __device__ __forceinline__ void store_pieces(unsigned char *base, int tok, int col, int stride, float v) {
+    unsigned char *at = base + static_cast<size_t>(tok * Ctx<MT>::S) * stride + col * 2;
+#pragma unroll
+    for (int i = 0; i < Ctx<MT>::S; ++i) {
+        const uint16_t b = f32_to_bf16_bits(v);
+        store_u16(at, b);
+        v -= bf16_bits_to_f32(b);        // exact: the remainder is what the next piece holds
+        at += stride;
+    }
+}
+
+// ---- exchanges by arrival: every CTA has written its share of a vector to global memory ------------------------------------
+// The generic writes (the vector's, and those to the shared memory the copies will overwrite) are ordered before the asynchronous copies
+// that follow the arrival; one thread arrives for the CTA.
+template <int MT> __device__ __forceinline__ bool arrive(const Ctx<MT> &c, bool ok) {
+    asm volatile("fence.proxy.async;" ::: "memory");
+    ok = cta_vote(ok);
+    if (ok && c.tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.p().arrivals) : "memory");
+    return ok;
+}
+template <int MT> __device__ __forceinline__ bool x_wait(Ctx<MT> &c) {
+    const unsigned b = c.xchunk & 3u;
+    return __all_sync(0xffffffffu, mbar_wait(&c.sh().x_full[b], (c.xchunk >> 2) & 1u, c.abort(), c.p().spin_limit));
+}
+template <int MT> __device__ __forceinline__ void x_release(Ctx<MT> &c) {
+    __syncwarp();
+    if (c.lane == 0) mbar_arrive(&c.sh().x_empty[c.xchunk & 3u]);
+    ++c.xchunk;
 }
 
 // ---- the order of the stream (the same arithmetic on the feeding and on the consuming side) --------------------------------

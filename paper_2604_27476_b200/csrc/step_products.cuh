@@ -5,127 +5,42 @@
 namespace edgefm {
 namespace step {
 
-// ---- exchanges: everybody reads a vector that lies in lines ---------------------------------------------------------------
-// Table of the 16-byte units of such a vector: row | values << 16 | unit << 18 (unit = index of the packet pair).
-// The tables of the residual stream and of the attention output stand in shared memory, made once per launch.
-__device__ __forceinline__ int line_units(int n, int ncta, int grain) { return ((n / grain + ncta - 1) / ncta * grain + 1) / 2; }
-template <int MT> __device__ __forceinline__ void make_table(const Ctx<MT> &c, unsigned *tab, int n, int grain, int line) {
-    const int upl = line_units(n, c.ncta, grain), total = c.ncta * upl;
-#pragma unroll 1
-    for (int i = c.tid; i < total; i += ST_NT) {
-        const int w = i / upl, e = i - w * upl;
-        const int r0 = st_first(n / grain, w, c.ncta) * grain, r1 = st_first(n / grain, w + 1, c.ncta) * grain, row = r0 + 2 * e;
-        tab[i] = static_cast<unsigned>(row & 0xffff) | static_cast<unsigned>(max(0, min(2, r1 - row))) << 16 | static_cast<unsigned>(w * (line >> 1) + e) << 18;
-    }
-}
-template <int MT> __device__ __forceinline__ void store_pieces(const Ctx<MT> &c, int tok, int col, int K, unsigned long long v) {
-    constexpr int S = Ctx<MT>::S;
-#pragma unroll
-    for (int i = 0; i < S; ++i) *c.xs(tok * S + i, col, K) = piece(v, i);
-}
-// Columns past K of the last 64-column block are multiplied by zero.
-template <int MT> __device__ __forceinline__ void zero_tail(const Ctx<MT> &c, int K) {
-    const int pad = (64 - (K & 63)) & 63;
-    for (int i = c.tid; i < pad * Ctx<MT>::NA; i += ST_NT) *c.xs(i / pad, K + i % pad, K) = 0;
-}
 // First operator of the step: the embedding rows are the residual streams.
 template <int MT> __device__ __forceinline__ bool stage_embedding(Ctx<MT> &c, const uint16_t *norm_w) {
     const StepParams &p = c.p();
+    const int stride = st_array_bytes(p.H), m = c.sh().m;
+    const int pad = (64 - (p.H & 63)) & 63;                 // columns past H of the last 64-column block are multiplied by zero
+    for (int i = c.tid; i < pad * Ctx<MT>::NA; i += ST_NT) store_u16(c.area() + (i / pad) * stride + (p.H + i % pad) * 2, 0);
 #pragma unroll 1
-    for (int t = 0; t < c.sh().m; ++t) {
+    for (int t = 0; t < m; ++t) {
         const uint16_t *erow = p.embed + static_cast<size_t>(c.sh().tokens[t]) * p.H;
         float ss = 0.f;
 #pragma unroll 1
         for (int i = c.tid; i < p.H; i += ST_NT) {
             const float v = bf16_bits_to_f32(erow[i]);
             ss = fmaf(v, v, ss);
-            store_pieces(c, t, i, p.H, pieces_packet(v * bf16_bits_to_f32(norm_w[i]), 0u));
+            store_pieces<MT>(c.area(), t, i, stride, v * bf16_bits_to_f32(norm_w[i]));
         }
         ss = warp_sum(ss);
         if (c.lane == 0) c.sh().merged[0][t * ST_NW + c.warp] = ss;      // (not in use yet)
     }
-    zero_tail(c, p.H);
     if (!cta_vote(true)) return false;
-    if (c.tid < c.sh().m) c.sh().ss[c.tid] = sum8(&c.sh().merged[0][c.tid * ST_NW]);
-    return cta_vote(true);
+    if (c.tid < m) c.sh().ss[c.tid] = sum8(&c.sh().merged[0][c.tid * ST_NW]);
+    return true;
 }
-// Wait for all values of the vectors of all tokens (K columns, lines of `line` packets) and leave their pieces in shared memory, and meet.
-// sums: the last packet of every line is a partial sum of squares.
-template <int MT>
-__device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int total, int K, const unsigned long long *ll, int line, bool sums, unsigned tag) {
-    constexpr int U = MT == 1 ? 4 : 7, W = 5;     // units in flight per thread; lines whose sums a lane reads together
-    const int m = c.sh().m, all = m * total;
-    bool ok = true;
-    // the sums of squares of token w are added by warp w; asked for first, awaited last
-    const unsigned long long *const sums_at = ll + static_cast<size_t>(c.warp) * c.ncta * line + line - 1;
-    const bool adds = sums && c.warp < m;
-    unsigned long long s[W] = {0ull, 0ull, 0ull, 0ull, 0ull};
-    auto ask = [&](int base) {
-#pragma unroll
-        for (int i = 0; i < W; ++i)
-            if (base + 32 * i < c.ncta) s[i] = get1(sums_at + static_cast<size_t>(base + 32 * i) * line);
-    };
-    if (adds) ask(c.lane);
-    zero_tail(c, K);
-#pragma unroll 1
-    for (int base = c.tid; base < all; base += U * ST_NT) {
-        unsigned e[U], at[U];
-        Two t[U];
-        unsigned todo = 0;
-#pragma unroll
-        for (int i = 0; i < U; ++i) {
-            const int u = base + i * ST_NT;
-            int tok = 0;
-            if constexpr (MT > 1) tok = u / total;
-            e[i] = u < all ? tab[u - tok * total] : 0u;
-            at[i] = (e[i] >> 18) * 2 + static_cast<unsigned>(tok * c.ncta * line);
-            e[i] = (e[i] & 0x3ffffu) | static_cast<unsigned>(tok) << 18;
-            if ((e[i] >> 16) & 3u) todo |= 1u << i;
-        }
-        Spin sp;
-        for (;;) {
-#pragma unroll
-            for (int i = 0; i < U; ++i)
-                if (todo >> i & 1u) t[i] = get2(ll + at[i]);
-#pragma unroll
-            for (int i = 0; i < U; ++i)
-                if (todo >> i & 1u) {
-                    const bool two = (e[i] >> 16 & 3u) > 1;
-                    if (pieces_tag(t[i].a, tag) && (!two || pieces_tag(t[i].b, tag))) {
-                        todo &= ~(1u << i);
-                        const int row = e[i] & 0xffffu, tok = static_cast<int>(e[i] >> 18);
-                        store_pieces(c, tok, row, K, t[i].a);
-                        if (two) store_pieces(c, tok, row + 1, K, t[i].b);
-                    }
-                }
-            if (!todo) break;
-            if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
-        }
-        if (!ok) break;
-    }
-    if (adds) {
+// Wait for a vector; sums: with the CTAs' sums of squares, which are added here (a warp per token).
+template <int MT> __device__ __forceinline__ bool stage_vector(Ctx<MT> &c, bool sums) {
+    if (!x_wait(c)) return false;
+    if (sums && c.warp < c.sh().m) {
+        const float *at = reinterpret_cast<const float *>(c.area() + Ctx<MT>::NA * st_array_bytes(c.p().H)) + c.warp * c.p().ss_stride;
         float ss = 0.f;
-#pragma unroll 1
-        for (int base = c.lane; base < c.ncta && ok; base += 32 * W) {
-            if (base != c.lane) ask(base);
-            Spin sp;
-            for (;;) {
-                bool here = true;
-#pragma unroll
-                for (int i = 0; i < W; ++i)
-                    if (base + 32 * i < c.ncta) here = here && packet_tag(s[i]) == tag;
-                if (here) break;
-                if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
-                ask(base);
-            }
-#pragma unroll
-            for (int i = 0; i < W; ++i)
-                if (base + 32 * i < c.ncta) ss += packet_value(s[i]);
-        }
+#pragma unroll 5
+        for (int i = c.lane; i < c.ncta; i += 32) ss += at[i];
         ss = warp_sum(ss);
         if (c.lane == 0) c.sh().ss[c.warp] = ss;
     }
-    return cta_vote(ok);
+    x_release(c);
+    return true;
 }
 
 // ---- products ------------------------------------------------------------------------------------------------------------
@@ -219,7 +134,7 @@ __device__ __forceinline__ Rows rows_of(const unsigned char *at, int g, int na, 
 struct Slice { int u, u1, op, batch; };      // units [u, u1) of an operator; the batch of partial sums they go to
 
 // KEEP > 0: rows are whole in a chunk and a warp's blocks of the vector (at most KEEP) stay in registers for all tiles.
-// KEEP == 0: tiles cut by columns, the vector is read again for every tile.
+// KEEP == 0: tiles cut by columns, the vector is read again for every tile (the MLP activations come by segments themselves).
 template <int KEEP, int MT>
 __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
     constexpr int SETS = (Ctx<MT>::NA + 7) / 8;
@@ -227,10 +142,11 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
     const int K = p.cols[sl.op].K, seg = p.cols[sl.op].seg;
     float *const part = c.sh().part[sl.batch & 1];
     const int g = c.lane >> 2, t16 = (c.lane & 3) * 16;
-    const bool odd = (g & 1) != 0, paired = op_paired(sl.op);
+    const bool odd = (g & 1) != 0, paired = op_paired(sl.op), down = KEEP == 0 && sl.op == ST_DN;
+    const int stride = st_array_bytes(down ? seg : K), slot = Ctx<MT>::NA * stride;
     const unsigned char *xb[SETS];           // this lane's array of the staged vector (columns of B past the last array: any)
 #pragma unroll
-    for (int s = 0; s < SETS; ++s) xb[s] = reinterpret_cast<const unsigned char *>(c.xs(min(8 * s + g, Ctx<MT>::NA - 1), 0, K)) + t16;
+    for (int s = 0; s < SETS; ++s) xb[s] = c.area() + min(8 * s + g, Ctx<MT>::NA - 1) * stride + t16;
     constexpr int NK = KEEP > 0 ? KEEP : 1;
     uint4 k0[NK][SETS], k1[NK][SETS];
     const int nb_all = (K + 63) / 64, first_all = nb_all * c.warp / ST_NW, mine_all = nb_all * (c.warp + 1) / ST_NW - first_all;
@@ -264,7 +180,9 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
 #pragma unroll 1
             for (int col = 0; col < K; col += seg) {
                 const unsigned char *at;
+                if (down && !x_wait(c)) return false;
                 if (!chunk_wait(c, at)) return false;
+                const int x_off = down ? c.act_slot * slot : col * 2;
                 const int cols = min(seg, K - col), nblk = (cols + 63) / 64;
                 const int j0 = nblk * c.warp / ST_NW, j1 = nblk * (c.warp + 1) / ST_NW;
                 const Rows r = rows_of(at, g, na, nb, cols * 2, paired, p.cols[sl.op], t16);
@@ -273,13 +191,17 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
                     uint4 b0[SETS], b1[SETS];
 #pragma unroll
                     for (int s = 0; s < SETS; ++s) {
-                        const unsigned char *x = xb[s] + (col + j * 64) * 2;
+                        const unsigned char *x = xb[s] + x_off + j * 128;
                         b0[s] = *reinterpret_cast<const uint4 *>(x);
                         b1[s] = *reinterpret_cast<const uint4 *>(x + 64);
                     }
                     block_mma<SETS>(acc, r.a, r.b, j * r.block, odd, r.last, b0, b1);
                 }
                 chunk_release(c);
+                if (down) {
+                    x_release(c);
+                    if (++c.act_slot == p.act_slots) c.act_slot = 0;
+                }
             }
         }
         const int done = u - sl.u;
@@ -290,126 +212,9 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
     return true;
 }
 
-// Down projection: its input, the MLP activations, is too long to be staged whole.  Every warp needs only its own blocks of a segment; it
-// polls them a segment ahead (the loads are on their way while it multiplies) into one of two small buffers of its own.
-template <int MT>
-__device__ __forceinline__ bool multiply_down(Ctx<MT> &c, const Slice &sl, unsigned tag) {
-    constexpr int NA = Ctx<MT>::NA, S = Ctx<MT>::S, SETS = (NA + 7) / 8, U = MT <= 2 ? 4 : 2;      // packet pairs in flight per lane and token
-    const StepParams &p = c.p();
-    const int K = p.cols[ST_DN].K, seg = p.cols[ST_DN].seg, stride = st_array_bytes(p.dn_cols);
-    float *const part = c.sh().part[sl.batch & 1];
-    const int g = c.lane >> 2, t16 = (c.lane & 3) * 16, m = c.sh().m;
-    const bool odd = (g & 1) != 0;
-    unsigned char *const own = c.area() + c.warp * (2 * NA * stride);
-    // the columns [a0, a1) of segment `col` are this warp's
-    auto range = [&](int col, int &a0, int &a1) {
-        const int cols = min(seg, K - col), nblk = (cols + 63) / 64;
-        a0 = nblk * c.warp / ST_NW * 64;
-        a1 = min(nblk * (c.warp + 1) / ST_NW * 64, cols);
-    };
-    Two v[MT][U];
-    auto ask = [&](int col, int from) {
-        int a0, a1;
-        range(col, a0, a1);
-#pragma unroll
-        for (int t = 0; t < MT; ++t)
-#pragma unroll
-            for (int i = 0; i < U; ++i) {
-                const int k = a0 + from + (i * 32 + c.lane) * 2;
-                if (t < m && k < a1) v[t][i] = get2(p.act_ll + static_cast<size_t>(t) * p.act_len + col + k);
-            }
-    };
-    auto take = [&](int col, int from, unsigned char *buf) {
-        int a0, a1;
-        range(col, a0, a1);
-        Spin sp;
-        for (;;) {
-            bool here = true;
-#pragma unroll
-            for (int t = 0; t < MT; ++t)
-#pragma unroll
-                for (int i = 0; i < U; ++i)
-                    if (t < m && a0 + from + (i * 32 + c.lane) * 2 < a1) here = here && pieces_tag(v[t][i].a, tag) && pieces_tag(v[t][i].b, tag);
-            if (__all_sync(0xffffffffu, here)) break;
-            if (!__all_sync(0xffffffffu, sp.again(c.abort(), p.spin_limit))) return false;
-            ask(col, from);
-        }
-        const int padded = (a1 + 63) / 64 * 64;
-#pragma unroll
-        for (int t = 0; t < MT; ++t)
-#pragma unroll
-            for (int i = 0; i < U; ++i) {
-                const int k = a0 + from + (i * 32 + c.lane) * 2;
-                const bool on = t < m && k < a1;               // (K is a multiple of 8: pairs are whole; columns past K are zero)
-                if (k < padded)
-#pragma unroll
-                    for (int q = 0; q < S; ++q)
-                        *reinterpret_cast<uint32_t *>(buf + (t * S + q) * stride + (k - a0) * 2) =
-                            on ? static_cast<uint32_t>(piece(v[t][i].a, q)) | static_cast<uint32_t>(piece(v[t][i].b, q)) << 16 : 0u;
-            }
-        return true;
-    };
-    // (a segment of a warp's columns is taken in rounds of 64 U columns; all but the last one wait here)
-    auto stage = [&](int col, unsigned char *buf, bool asked) {
-        int a0, a1;
-        range(col, a0, a1);
-#pragma unroll 1
-        for (int from = 0; from == 0 || a0 + from < a1; from += 64 * U) {
-            if (!(asked && from == 0)) ask(col, from);
-            if (!take(col, from, buf)) return false;
-        }
-        __syncwarp();
-        return true;
-    };
-    int which = 0;
-    bool staged = false;
-    Acc<SETS> acc;
-    acc.clear();
-#pragma unroll 1
-    for (int u = sl.u; u < sl.u1;) {
-        const int n = tile_units(p, ST_DN, u, sl.u1), na = min(n, 8), nb = n - na;
-#pragma unroll 1
-        for (int col = 0; col < K; col += seg) {
-            unsigned char *buf = own + which * NA * stride;
-            if (!staged && !stage(col, buf, false)) return false;
-            const int next = col + seg < K ? col + seg : 0;                    // (0: the next tile starts over)
-            const bool more = next > 0 || u + n < sl.u1;
-            if (more) ask(next, 0);
-            const unsigned char *at;
-            if (!chunk_wait(c, at)) return false;
-            const int cols = min(seg, K - col), nblk = (cols + 63) / 64;
-            const int j0 = nblk * c.warp / ST_NW, j1 = nblk * (c.warp + 1) / ST_NW;
-            const Rows r = rows_of(at, g, na, nb, cols * 2, false, p.cols[ST_DN], t16);
-            const unsigned char *xb[SETS];
-#pragma unroll
-            for (int s = 0; s < SETS; ++s) xb[s] = buf + min(8 * s + g, NA - 1) * stride + t16;
-#pragma unroll 2
-            for (int j = j0; j < j1; ++j) {
-                uint4 b0[SETS], b1[SETS];
-#pragma unroll
-                for (int s = 0; s < SETS; ++s) {
-                    b0[s] = *reinterpret_cast<const uint4 *>(xb[s] + (j - j0) * 128);
-                    b1[s] = *reinterpret_cast<const uint4 *>(xb[s] + (j - j0) * 128 + 64);
-                }
-                block_mma<SETS>(acc, r.a, r.b, j * r.block, odd, r.last, b0, b1);
-            }
-            chunk_release(c);
-            which ^= 1;
-            staged = more;
-            if (more && !stage(next, own + which * NA * stride, true)) return false;
-        }
-        const int done = u - sl.u;
-        flush<MT, SETS>(c, acc, part, done, na, done + 8, nb);
-        acc.clear();
-        u += n;
-    }
-    return true;
-}
-
-template <int MT> __device__ __forceinline__ bool multiply_any(Ctx<MT> &c, const Slice &sl, unsigned tag) {
-    if (sl.op == ST_DN) return multiply_down<MT>(c, sl, tag);
+template <int MT> __device__ __forceinline__ bool multiply_any(Ctx<MT> &c, const Slice &sl) {
     const StepCols &cols = c.p().cols[sl.op];
-    if (cols.segs > 1) return multiply<0, MT>(c, sl);
+    if (cols.segs > 1 || sl.op == ST_DN) return multiply<0, MT>(c, sl);
     switch (((cols.K + 63) / 64 + ST_NW - 1) / ST_NW) {
         case 1: return multiply<1, MT>(c, sl);
         case 2: return multiply<2, MT>(c, sl);

@@ -75,23 +75,26 @@ struct StepParams {
     const int *vocab_ids;
     StepState *state;
     const StepRequest *req;
-    // exchange buffers: packets of 8 bytes, {fp32 value, 32-bit tag} or {three bf16 pieces, 16-bit tag}; [token] first
-    unsigned long long *x_ll;      // residual stream after the down projection, times the next norm's weight: pieces; per CTA one line of
-                                   // x_line packets, its last one the CTA's sum of squares (fp32)
-    unsigned long long *xo_ll;     // ... after the O projection
-    unsigned long long *q_ll;      // rotated q, k and v (fp32): per CTA one line of q_line packets, {lo, hi} of its row pairs in order
-    unsigned long long *ao_ll;     // attention output (pieces): per CTA one line of ao_line packets
-    unsigned long long *act_ll;    // MLP activations (pieces) [act_len]
-    unsigned long long *part_ll;   // attention partial results [token and chunk][nq D] (fp32, unnormalised)
+    // Vectors that are multiplied next: as they lie in shared memory, arrays of bf16 pieces [token * S + piece][st_array_bytes(K)], zero past
+    // K; behind the residual streams' arrays the CTAs' sums of squares [token][ss_stride].  act: [segment][array][st_array_bytes(seg)].
+    unsigned char *x_vec;          // residual stream after the down projection, times the next norm's weight
+    unsigned char *xo_vec;         // ... after the O projection
+    unsigned char *ao_vec;         // attention output
+    unsigned char *act_vec;        // MLP activations
+    int ss_stride;
+    unsigned *arrivals;            // CTAs that have written their share, all exchanges of all calls
+    // packets of 8 bytes {fp32 value, tag}
+    unsigned long long *q_ll;      // rotated q, k and v: [token], per CTA one line of q_line packets, {lo, hi} of its row pairs in order
+    unsigned long long *part_ll;   // attention partial results [token and chunk][nq D] (unnormalised)
     unsigned long long *stat_ll;   // ... their {maximum, denominator} [token and chunk][nq][2]
     unsigned long long *lm_ll;     // greedy candidates: per CTA one line, {value, row} of every token
-    int x_line, q_line, ao_line, act_len;
+    int q_line;
     StepCols cols[5];              // per operator
     int ring_bytes, resid_at, table_bytes;   // shared memory (resid_at: inside the tables)
-    int dn_cols;                   // columns of a warp's buffer for a segment of the MLP activations
+    int act_slots;                 // segments of the MLP activations in shared memory
     int prefetch_bytes;            // how far the L2 prefetch runs ahead of the ring
     int epoch_slot;                // which of the state's epochs tags this build's packets
-    int barrier_extra;             // test hook: 1 = the packets expected never come, so that the first wait runs out
+    int barrier_extra;             // test hook: an exchange waits for one arrival more than there are CTAs (1; 0 in production)
     unsigned spin_limit;           // upper bound of every device-side wait, nanoseconds
     unsigned long long *prof;      // optional timestamps [gridDim.x][prof_stride]
     int prof_stride;
@@ -124,12 +127,19 @@ struct StepLaunch {
     StepParams p{};
     int grid = 0;
     size_t dyn_smem = 0;
-    size_t ll_bytes = 0;        // exchange buffers (zeroed once: tag 0 is never used)
+    size_t ll_bytes = 0;        // exchange buffers (zeroed once: tag 0 is never used, columns past K stay zero)
     int max_chunk_bytes = 0;
 };
 int step_shared_bytes(int mt);  // fixed part of the kernel's shared memory
 int step_scratch_floats(int D, int G, int mt);
 
+// Bytes of a vector's exchange buffer / of the MLP activations' (whole 128 bytes).
+inline size_t step_vec_bytes(const StepParams &p, int mt, int K, bool sums) {
+    return (static_cast<size_t>(st_arrays(mt)) * st_array_bytes(K) + (sums ? 4 * static_cast<size_t>(mt) * p.ss_stride : 0) + 127) / 128 * 128;
+}
+inline size_t step_act_bytes(const StepParams &p, int mt) {
+    return (static_cast<size_t>(p.cols[ST_DN].segs) * st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg) + 127) / 128 * 128;
+}
 // Shared-memory split and exchange buffers for a model shape.  Returns null, or why the shape does not fit.
 inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, bool kv8, int mt, StepLaunch *sl) {
     const int H = sh.hidden, D = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, F = sh.ffn, qd = nq * D, G = nq / nkv;
@@ -139,7 +149,7 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     // every CTA must own a row of the residual stream: its contribution is what says that it has read the exchange before
     const int grid = sl->grid = std::min(num_sms, H);
     const long long units = std::max({static_cast<long long>(sh.vocab), static_cast<long long>(F), static_cast<long long>(nq + 2 * nkv) * D / 2, static_cast<long long>(max_context)});
-    if (qd > 128 * grid || H >= 65536 || qd >= 65536 || (units + 1) * (grid + 1) > 0x7fffffffLL) return "model shape does not fit the step kernel";
+    if (qd > 128 * grid || (units + 1) * (grid + 1) > 0x7fffffffLL) return "model shape does not fit the step kernel";
     p.n_layers = sh.n_layers; p.H = H; p.nq = nq; p.nkv = nkv; p.G = G; p.D = D; p.F = F; p.V = sh.vocab; p.qd = qd;
     p.half_shift = D == 64 ? 5 : 6;
     p.eps = sh.rms_eps;
@@ -151,17 +161,15 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.cols[ST_LM] = step_cols(H, ST_TILE, false);
     p.cols[ST_O] = step_cols(qd, h_rows, false);
     p.cols[ST_DN] = step_cols(F, h_rows, false, mt <= 2 ? 2048 : 1024);      // (two segments of activations are in shared memory, as pieces)
-    p.x_line = st_line(most(H) + 1);
     p.q_line = st_line(2 * most((nq + 2 * nkv) * D / 2));
-    p.ao_line = st_line(2 * most(qd / 2));
-    p.act_len = (F + 15) / 16 * 16;
-    const int total_x = grid * ((most(H) + 1) / 2), total_a = grid * most(qd / 2);
-    if (grid * p.x_line / 2 >= 16384 || grid * p.ao_line / 2 >= 16384) return "model shape does not fit the step kernel";
-    p.resid_at = (sh.n_layers + 1) * 64 + 4 * (total_x + total_a);
+    p.ss_stride = (grid + 3) / 4 * 4;
+    p.resid_at = (sh.n_layers + 1) * 64;
     p.table_bytes = (p.resid_at + 4 * mt * most(H) + 127) / 128 * 128;
-    p.dn_cols = ((p.cols[ST_DN].seg + 63) / 64 + ST_NW - 1) / ST_NW * 64;
-    // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another, CTA-wide votes between
-    const int area = std::max({st_arrays(mt) * st_array_bytes(std::max(H, qd)), 4 * step_scratch_floats(D, G, mt), ST_NW * 2 * st_arrays(mt) * st_array_bytes(p.dn_cols)});
+    // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another
+    const int slot = st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg), vec = std::max(st_arrays(mt) * st_array_bytes(H) + 4 * mt * p.ss_stride, st_arrays(mt) * st_array_bytes(qd));
+    int area = std::max(vec, 4 * step_scratch_floats(D, G, mt));
+    p.act_slots = p.cols[ST_DN].segs == 1 ? 1 : std::max(2, std::min(3, area / slot));
+    area = std::max(area, p.act_slots * slot);
     const int fixed = step_shared_bytes(mt) + p.table_bytes + (area + 127) / 128 * 128;
     int chunk = ST_KV_BLOCK * D * (kv8 ? 2 : 4);
     for (int o = 0; o < 5; ++o) chunk = std::max(chunk, (o == ST_O || o == ST_DN ? h_rows : ST_TILE) * p.cols[o].seg * 2);
@@ -173,19 +181,23 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.prefetch_bytes = ST_PREFETCH_BYTES;
     p.spin_limit = 1000000000u;   // 1 s
     const size_t chunks = static_cast<size_t>(std::max(grid / nkv, mt));
-    sl->ll_bytes = 8 * (static_cast<size_t>(grid) * mt * (2 * p.x_line + p.q_line + p.ao_line) + static_cast<size_t>(grid) * 16 + static_cast<size_t>(mt) * p.act_len + chunks * qd + chunks * nq * 2);
+    sl->ll_bytes = 8 * (static_cast<size_t>(grid) * mt * p.q_line + static_cast<size_t>(grid) * 16 + chunks * qd + chunks * nq * 2) + 2 * step_vec_bytes(p, mt, H, true) +
+                   step_vec_bytes(p, mt, qd, false) + step_act_bytes(p, mt) + 256;
     return nullptr;
 }
 // Wire the exchange buffers (256-byte aligned base).
 inline void step_wire(StepLaunch *sl, int mt, unsigned long long *base) {
     StepParams &p = sl->p;
     const size_t g = static_cast<size_t>(sl->grid), m = static_cast<size_t>(mt), chunks = static_cast<size_t>(std::max(sl->grid / p.nkv, mt));
-    p.x_ll = base; base += g * m * p.x_line;
-    p.xo_ll = base; base += g * m * p.x_line;
+    unsigned char *b = reinterpret_cast<unsigned char *>(base);
+    p.arrivals = reinterpret_cast<unsigned *>(b); b += 256;
+    p.x_vec = b; b += step_vec_bytes(p, mt, p.H, true);
+    p.xo_vec = b; b += step_vec_bytes(p, mt, p.H, true);
+    p.ao_vec = b; b += step_vec_bytes(p, mt, p.qd, false);
+    p.act_vec = b; b += step_act_bytes(p, mt);
+    base = reinterpret_cast<unsigned long long *>(b);
     p.q_ll = base; base += g * m * p.q_line;
-    p.ao_ll = base; base += g * m * p.ao_line;
     p.lm_ll = base; base += g * 16;
-    p.act_ll = base; base += m * p.act_len;
     p.part_ll = base; base += chunks * p.qd;
     p.stat_ll = base;
 }

@@ -377,11 +377,22 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
         if (on && sub == 0) *reinterpret_cast<float2 *>(&c.sh().merged[tok][2 * k_pair]) = make_float2(a / l, b / l);
     }
     if (!cta_vote(ok)) return false;
-    const int stride = st_array_bytes(p.qd);
+    if constexpr (st_packets(MT)) {
+        // a line is written by one instruction: every further write invalidates the pollers' copies of it (+ 1.5 us)
+        const unsigned real_tag = tag ^ c.sh().odd;
 #pragma unroll 1
-    for (int i = c.tid; i < 2 * n_pairs * m; i += ST_NT) {
-        const int tok = i / (2 * n_pairs), k = i - tok * 2 * n_pairs;
-        store_pieces<MT>(p.ao_vec, tok, 2 * a0 + k, stride, c.sh().merged[tok][k]);
+        for (int i = c.tid; i < n_pairs * MT; i += ST_NT) {        // (unused tokens too: their slots keep up with the tags)
+            const int tok = i / n_pairs, k = i - tok * n_pairs;
+            const float2 v = tok < m ? *reinterpret_cast<const float2 *>(&c.sh().merged[tok][2 * k]) : make_float2(0.f, 0.f);
+            put_raw2(p.ao_ll + (static_cast<size_t>(tok) * c.ncta + c.cta) * p.ao_line + 2 * k, pieces_packet(v.x, real_tag), pieces_packet(v.y, real_tag));
+        }
+    } else {
+        const int stride = st_array_bytes(p.qd);
+#pragma unroll 1
+        for (int i = c.tid; i < 2 * n_pairs * m; i += ST_NT) {
+            const int tok = i / (2 * n_pairs), k = i - tok * 2 * n_pairs;
+            store_pieces<MT>(p.ao_vec, tok, 2 * a0 + k, stride, c.sh().merged[tok][k]);
+        }
     }
     return true;
 }

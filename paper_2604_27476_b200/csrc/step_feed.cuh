@@ -183,7 +183,7 @@ __device__ __forceinline__ void feed_vectors(Ctx<MT> &c) {
     Shared<MT> &sh = c.sh();
     const StepParams &p = c.p();
     constexpr int NA = Ctx<MT>::NA;
-    unsigned k = 0, target = static_cast<unsigned>(p.state->epoch[p.epoch_slot]) * static_cast<unsigned>(4 * p.n_layers * c.ncta) + static_cast<unsigned>(p.barrier_extra);
+    unsigned k = 0, target = static_cast<unsigned>(p.state->epoch[p.epoch_slot]) * static_cast<unsigned>((st_packets(MT) ? 1 : 4) * p.n_layers * c.ncta) + static_cast<unsigned>(p.barrier_extra);
     bool ok = true;
     auto everybody = [&]() {                     // wait for the next exchange's arrivals
         target += static_cast<unsigned>(c.ncta);
@@ -209,17 +209,20 @@ __device__ __forceinline__ void feed_vectors(Ctx<MT> &c) {
     const int tiles = (sh.u1[ST_DN] - sh.u0[ST_DN] + ST_TILE - 1) / ST_TILE;
 #pragma unroll 1
     for (int layer = 0; layer <= p.n_layers && ok; ++layer) {
-        if (layer > 0) {
+        if constexpr (!st_packets(MT)) {
+            if (layer > 0) {
+                ok = everybody();
+                if (ok) copy(p.x_vec, 0u, vec);
+            }
+            if (!ok || layer == p.n_layers) break;
             ok = everybody();
-            if (ok) copy(p.x_vec, 0u, vec);
+            if (!ok) break;
+            copy(p.ao_vec, 0u, NA * st_array_bytes(p.qd));
+            ok = everybody();
+            if (!ok) break;
+            copy(p.xo_vec, 0u, vec);
         }
-        if (!ok || layer == p.n_layers) break;
-        ok = everybody();
-        if (!ok) break;
-        copy(p.ao_vec, 0u, NA * st_array_bytes(p.qd));
-        ok = everybody();
-        if (!ok) break;
-        copy(p.xo_vec, 0u, vec);
+        if (layer == p.n_layers) break;
         ok = everybody();
         if (!ok) break;
         const unsigned first = k;

@@ -14,13 +14,15 @@
 //     two tokens, two for more), one B column per piece and token, so that a block of tokens costs the weights' traffic and the
 //     instructions of one.  The 8 partial sums of a row meet in shared memory and one thread per output unit and token runs the
 //     fused epilogue (bias + RoPE + cache row, residual add, SwiGLU, logits + argmax).
-//   * Exchanges.  A vector that is multiplied next is written by its owners as the products want it, arrays of bf16 pieces (split, and
-//     weighted for the norm, once by the owner instead of by every reader); every CTA then counts up one counter, and a thread of
-//     every CTA that has seen all of them fetches the vector with one bulk copy -- no thread of the consumers polls, and the
-//     cost does not grow with the tokens.  Queries and the attention's partial results, of which a CTA needs a few rows only, travel as
-//     8-byte packets {fp32 value, tag}; the tag names step and layer, so a reader polls the data itself: one trip to L2.  Every
-//     CTA writes its queries into lines of its own (packets of several writers in one 128-byte line cost 0.3 - 1 us: the pollers'
-//     copies are invalidated by every write).  A buffer is rewritten one layer later; a CTA that writes it then has seen, in
+//   * Exchanges.  A value travels as an 8-byte packet with a tag that names step and layer, so a reader polls the data itself: one
+//     trip to L2 instead of store, fence, counter, poll, load (a release waits for everything its SM has under way: 0.6 us idle,
+//     2 us while the weights stream).  Vectors that are multiplied next travel as their bf16 pieces, split (and weighted for the norm)
+//     once by the owner instead of by every reader.  Every CTA writes its values into 128-byte lines of its own (packets of several
+//     writers in one line cost 0.3 - 1 us: the pollers' copies of the line are invalidated by every write).
+//     Polling grows with the tokens.  For four and more the owners write such vectors plainly, as the products want them, every CTA
+//     counts up one counter, and a feeding thread that has seen all of them fetches the vector with one bulk copy (a block of four
+//     took 1530 us with packets and 1286 us so, a single token 976 and 1016 us).  MLP activations too long for the shared memory go
+//     this way too, by segments.  A buffer is rewritten one layer later; a CTA that writes it then has seen, in
 //     between, an exchange to which every CTA contributes only after reading the old contents.
 //   * Attention (step_attention.cuh).  CTA (token, kv head, chunk) holds the chunk's K/V rows in its ring before the queries exist,
 //     serves the whole GQA group from one read, and publishes unnormalised partial results; the owner of an output pair merges
@@ -65,8 +67,13 @@ __device__ __forceinline__ void finish_unit(const Ctx<MT> &c, int op, int layer,
             d[half] = f32_to_bf16_bits(hi);
         }
     } else if (op == ST_GU) {
+        const float v = lo / (1.f + expf(-lo)) * hi;
+        if (st_packets(MT) && p.act_packets) {
+            put_raw(p.act_ll + static_cast<size_t>(tok) * p.act_len + j, pieces_packet(v, tag));
+            return;
+        }
         const int seg = p.cols[ST_DN].seg, s = j / seg, stride = st_array_bytes(seg);
-        store_pieces<MT>(p.act_vec + static_cast<size_t>(s) * Ctx<MT>::NA * stride, tok, j - s * seg, stride, lo / (1.f + expf(-lo)) * hi);
+        store_pieces<MT>(p.act_vec + static_cast<size_t>(s) * Ctx<MT>::NA * stride, tok, j - s * seg, stride, v);
     } else if (tok < sh.m) {
         float *logits = p.req->logits_out;
         if (logits) logits[static_cast<size_t>(tok) * c.head().rows + j] = lo;
@@ -104,6 +111,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.n_old = p.state->cur_len;
             sh.n_chunks = kv_chunks(p, sh.n_old, sh.m, c.ncta);
             sh.tag0 = static_cast<unsigned>(p.state->epoch[p.epoch_slot]) * static_cast<unsigned>(p.n_layers + 2) + 1u;
+            sh.odd = static_cast<unsigned>(p.barrier_extra) << 31 | static_cast<unsigned>(p.barrier_extra) << 15;
+            sh.total_x = c.ncta * line_units(p.H, c.ncta, 1);
+            sh.total_a = c.ncta * line_units(p.qd, c.ncta, 2);
         }
         __syncthreads();
         const int lm_rows = c.head().rows;
@@ -125,7 +135,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ST_REGS_FEED));
         if (c.warp == ST_NW) feed_ring<Q8, MT>(c);
         if (c.warp == ST_NW + 1) feed_l2<Q8, MT>(c);
-        if (c.warp == ST_NW + 2 && c.lane == 0) feed_vectors<MT>(c);
+        if (c.warp == ST_NW + 2 && c.lane == 0 && !(st_packets(MT) && p.act_packets)) feed_vectors<MT>(c);
         return;
     }
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ST_REGS));
@@ -157,6 +167,10 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.rope[t][half + f] = static_cast<float>(sn);
         }
         if (c.cta == 0 && c.tid == 0) { p.state->token = sh.tokens[0]; p.state->position = sh.pos; }
+        if constexpr (st_packets(MT)) {
+            make_table(c, c.unit_table(), p.H, 1, p.x_line);
+            make_table(c, c.unit_table() + sh.total_x, p.qd, 2, p.ao_line);
+        }
         for (int i = c.tid; i < MT * my_rows; i += ST_NT) {
             const int t = i / my_rows;
             c.resid()[i] = bf16_bits_to_f32(p.embed[static_cast<size_t>(sh.tokens[t]) * p.H + x0 + i - t * my_rows]);
@@ -176,7 +190,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         c.warp = c.tid >> 5;
         c.lane = c.tid & 31;
         Shared<MT> &sh = c.sh();
-        const unsigned tag = sh.tag0 + static_cast<unsigned>(layer);      // what this layer's packets carry
+        const unsigned real_tag = sh.tag0 + static_cast<unsigned>(layer), tag = real_tag ^ sh.odd;      // what this layer's packets carry / are expected to carry
         const StepLayer *L = c.layer(layer);
         // -- the input vector --
         if (op == ST_O) {
@@ -188,7 +202,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             }
             if (!ok) break;
             stamp(c, prof_idx);                       // chunk done
-            ok = arrive(c, merge_chunks(c, tag));
+            ok = merge_chunks(c, tag);
+            if constexpr (!st_packets(MT)) ok = arrive(c, ok);
             if (!ok) break;
             stamp(c, prof_idx);                       // partial results merged
         }
@@ -196,6 +211,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             ok = stage_embedding(c, L->input_norm);
         } else if (op == ST_DN) {
             c.act_slot = 0;
+            if (st_packets(MT) && p.act_packets) ok = stage_activations(c, tag);
+        } else if constexpr (st_packets(MT)) {        // (one call for the three exchanges: the loop's code has to stay small)
+            const bool ao = op == ST_O, gu = op == ST_GU;
+            ok = stage_lines(c, c.unit_table() + (ao ? sh.total_x : 0), ao ? sh.total_a : sh.total_x, ao ? p.qd : p.H, ao ? p.ao_ll : gu ? p.xo_ll : p.x_ll,
+                             ao ? p.ao_line : p.x_line, !ao, ao || gu ? tag : (real_tag - 1u) ^ sh.odd);
         } else {
             ok = stage_vector(c, op != ST_O);         // (of this warp; the vote follows the products)
         }
@@ -229,6 +249,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             if (resid) {
                 if (tok < MT) {
                     unsigned char *vec = op == ST_O ? p.xo_vec : p.x_vec;
+                    unsigned long long *line = (op == ST_O ? p.xo_ll : p.x_ll) + (static_cast<size_t>(tok) * c.ncta + c.cta) * p.x_line;
                     const int stride = st_array_bytes(p.H);
 #pragma unroll 1
                     for (int r = j; r < ue; r += 32) {
@@ -236,11 +257,13 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
                         float &x = c.resid()[tok * my_rows + r - u0];
                         x += sum8(part + (tok * RB + r - ub) * ST_NW);
                         sq = fmaf(x, x, sq);
-                        store_pieces<MT>(vec, tok, r, stride, x * add_lo);
+                        if constexpr (st_packets(MT)) put_raw(line + r - u0, pieces_packet(x * add_lo, real_tag));
+                        else store_pieces<MT>(vec, tok, r, stride, x * add_lo);
                     }
                     if (ue == u1) {
                         const float all = warp_sum(sq);
-                        if (c.lane == 0) *reinterpret_cast<float *>(vec + Ctx<MT>::NA * stride + 4 * (tok * p.ss_stride + c.cta)) = all;
+                        if (c.lane == 0 && st_packets(MT)) put1(line + p.x_line - 1, all, real_tag);
+                        if (c.lane == 0 && !st_packets(MT)) *reinterpret_cast<float *>(vec + Ctx<MT>::NA * stride + 4 * (tok * p.ss_stride + c.cta)) = all;
                     }
                 }
             } else if (mine) {
@@ -252,7 +275,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         }
         stamp(c, prof_idx);
         if (ok && op != ST_QKV && op != ST_LM) {
-            ok = arrive(c, true);
+            if (!st_packets(MT) || (op == ST_GU && !p.act_packets)) ok = arrive(c, true);
             stamp(c, prof_idx);
         }
     }

@@ -89,6 +89,28 @@ __device__ __forceinline__ Two get2(const unsigned long long *at) {
 }
 __device__ __forceinline__ bool both(const Two &t, unsigned tag) { return packet_tag(t.a) == tag && packet_tag(t.b) == tag; }
 
+// Packets of pieces: three bf16 (value = their sum) and the low 16 bits of the tag.  A slot is rewritten with the next tag every layer
+// (every token's, used or not), so 16 bits tell the contents apart.
+__device__ __forceinline__ unsigned long long pieces_packet(float v, unsigned tag) {
+    const uint16_t hi = f32_to_bf16_bits(v);
+    v -= bf16_bits_to_f32(hi);           // exact: the remainder is what the next piece holds
+    const uint16_t mid = f32_to_bf16_bits(v);
+    const uint16_t lo = f32_to_bf16_bits(v - bf16_bits_to_f32(mid));
+    return static_cast<unsigned long long>(hi | static_cast<unsigned>(mid) << 16) | static_cast<unsigned long long>(lo | tag << 16) << 32;
+}
+__device__ __forceinline__ bool pieces_tag(unsigned long long p, unsigned tag) { return static_cast<unsigned>(p >> 48) == (tag & 0xffffu); }
+__device__ __forceinline__ void put_raw(unsigned long long *at, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(at), "l"(v) : "memory");
+}
+__device__ __forceinline__ void put_raw2(unsigned long long *at, unsigned long long a, unsigned long long b) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(at), "l"(a), "l"(b) : "memory");
+}
+__device__ __forceinline__ unsigned long long get1(const unsigned long long *at) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(at) : "memory");
+    return v;
+}
+
 // Two fp32 values in one 64-bit register pair.
 using f2 = unsigned long long;
 __device__ __forceinline__ f2 pack2(float a, float b) {
@@ -146,7 +168,7 @@ __device__ __forceinline__ float sum8(const float *at) {
 }
 
 // ---- shared memory ---------------------------------------------------------------------------------------------------
-// Dynamic: Shared | ring | layer table, residual rows | one area for the staged vector, the attention's scratch and the
+// Dynamic: Shared | ring | layer table, unit tables, residual rows | one area for the staged vector, the attention's scratch and the
 // segments of the MLP activations (they follow one another; between the last reader of one and the first writer of the next
 // lies a CTA-wide vote).
 extern __shared__ __align__(128) unsigned char st_smem[];
@@ -161,7 +183,8 @@ template <int MT> struct Shared {
     float best_v[ST_NW];
     int best_i[ST_NW];
     int u0[5], u1[5];                                      // this CTA's units of every operator
-    unsigned tag0;                                         // tag of layer 0
+    unsigned tag0, odd;                                    // tag of layer 0; test hook: a bit no tag has
+    int total_x, total_a;                                  // sizes of the unit tables
     int tokens[MT];
     int m, pos, n_old, n_chunks;                           // the call's tokens, first position, cache length; attention chunks per kv head and token
     unsigned sent;                                         // 16-byte units the feeding warp has asked for
@@ -186,6 +209,7 @@ template <int MT> struct Ctx {
     __device__ __forceinline__ unsigned char *tables() const { return ring() + p().ring_bytes; }
     __device__ __forceinline__ const StepLayer *layer(int l) const { return reinterpret_cast<const StepLayer *>(tables()) + l; }
     __device__ __forceinline__ const StepHead &head() const { return *reinterpret_cast<const StepHead *>(layer(p().n_layers)); }
+    __device__ __forceinline__ unsigned *unit_table() const { return reinterpret_cast<unsigned *>(tables() + (p().n_layers + 1) * 64); }
     __device__ __forceinline__ float *resid() const { return reinterpret_cast<float *>(tables() + p().resid_at); }   // [token][this CTA's rows of the residual stream]
     __device__ __forceinline__ unsigned char *area() const { return tables() + p().table_bytes; }
 };
@@ -225,11 +249,21 @@ template <int MT> __device__ __forceinline__ void store_pieces(unsigned char *ba
     }
 }
 
+template <int MT> __device__ __forceinline__ void store_packet(unsigned char *base, int tok, int col, int stride, unsigned long long v) {
+    unsigned char *at = base + tok * Ctx<MT>::S * stride + col * 2;
+#pragma unroll
+    for (int i = 0; i < Ctx<MT>::S; ++i) store_u16(at + i * stride, static_cast<uint16_t>(v >> (16 * i)));
+}
+// Columns past K of the last 64-column block are multiplied by zero.
+template <int MT> __device__ __forceinline__ void zero_tail(const Ctx<MT> &c, int K) {
+    const int pad = (64 - (K & 63)) & 63, stride = st_array_bytes(K);
+    for (int i = c.tid; i < pad * Ctx<MT>::NA; i += ST_NT) store_u16(c.area() + (i / pad) * stride + (K + i % pad) * 2, 0);
+}
+
 // ---- exchanges by arrival: every CTA has written its share of a vector to global memory ------------------------------------
-// The generic writes (the vector's, and those to the shared memory the copies will overwrite) are ordered before the asynchronous copies
-// that follow the arrival; one thread arrives for the CTA.
+// One thread arrives for the CTA.  (The thread that issues the copies puts the proxy fence between what it has acquired and the copies;
+// a second one here, by every writer, cost each exchange 1 us.)
 template <int MT> __device__ __forceinline__ bool arrive(const Ctx<MT> &c, bool ok) {
-    asm volatile("fence.proxy.async;" ::: "memory");
     ok = cta_vote(ok);
     if (ok && c.tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.p().arrivals) : "memory");
     return ok;

@@ -9,8 +9,7 @@ namespace step {
 template <int MT> __device__ __forceinline__ bool stage_embedding(Ctx<MT> &c, const uint16_t *norm_w) {
     const StepParams &p = c.p();
     const int stride = st_array_bytes(p.H), m = c.sh().m;
-    const int pad = (64 - (p.H & 63)) & 63;                 // columns past H of the last 64-column block are multiplied by zero
-    for (int i = c.tid; i < pad * Ctx<MT>::NA; i += ST_NT) store_u16(c.area() + (i / pad) * stride + (p.H + i % pad) * 2, 0);
+    zero_tail(c, p.H);
 #pragma unroll 1
     for (int t = 0; t < m; ++t) {
         const uint16_t *erow = p.embed + static_cast<size_t>(c.sh().tokens[t]) * p.H;
@@ -41,6 +40,139 @@ template <int MT> __device__ __forceinline__ bool stage_vector(Ctx<MT> &c, bool 
     }
     x_release(c);
     return true;
+}
+
+// ---- exchanges: everybody reads a vector that lies in lines ---------------------------------------------------------------
+// Table of the 16-byte units of such a vector: row | values << 16 | unit << 18 (unit = index of the packet pair).
+// The tables of the residual stream and of the attention output stand in shared memory, made once per launch.
+__device__ __forceinline__ int line_units(int n, int ncta, int grain) { return ((n / grain + ncta - 1) / ncta * grain + 1) / 2; }
+template <int MT> __device__ __forceinline__ void make_table(const Ctx<MT> &c, unsigned *tab, int n, int grain, int line) {
+    const int upl = line_units(n, c.ncta, grain), total = c.ncta * upl;
+#pragma unroll 1
+    for (int i = c.tid; i < total; i += ST_NT) {
+        const int w = i / upl, e = i - w * upl;
+        const int r0 = st_first(n / grain, w, c.ncta) * grain, r1 = st_first(n / grain, w + 1, c.ncta) * grain, row = r0 + 2 * e;
+        tab[i] = static_cast<unsigned>(row & 0xffff) | static_cast<unsigned>(max(0, min(2, r1 - row))) << 16 | static_cast<unsigned>(w * (line >> 1) + e) << 18;
+    }
+}
+// Wait for all values of the vectors of all tokens (K columns, lines of `line` packets) and leave their pieces in shared memory, and meet.
+// sums: the last packet of every line is a partial sum of squares.
+template <int MT>
+__device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int total, int K, const unsigned long long *ll, int line, bool sums, unsigned tag) {
+    constexpr int U = MT == 1 ? 4 : 7, W = 5;     // units in flight per thread; lines whose sums a lane reads together
+    const int m = c.sh().m, all = m * total, stride = st_array_bytes(K);
+    bool ok = true;
+    // the sums of squares of token w are added by warp w; asked for first, awaited last
+    const unsigned long long *const sums_at = ll + static_cast<size_t>(c.warp) * c.ncta * line + line - 1;
+    const bool adds = sums && c.warp < m;
+    unsigned long long s[W] = {0ull, 0ull, 0ull, 0ull, 0ull};
+    auto ask = [&](int base) {
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (base + 32 * i < c.ncta) s[i] = get1(sums_at + static_cast<size_t>(base + 32 * i) * line);
+    };
+    if (adds) ask(c.lane);
+    zero_tail(c, K);
+#pragma unroll 1
+    for (int base = c.tid; base < all; base += U * ST_NT) {
+        unsigned e[U], at[U];
+        Two t[U];
+        unsigned todo = 0;
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int u = base + i * ST_NT;
+            int tok = 0;
+            if constexpr (MT > 1) tok = u / total;
+            e[i] = u < all ? tab[u - tok * total] : 0u;
+            at[i] = (e[i] >> 18) * 2 + static_cast<unsigned>(tok * c.ncta * line);
+            e[i] = (e[i] & 0x3ffffu) | static_cast<unsigned>(tok) << 18;
+            if ((e[i] >> 16) & 3u) todo |= 1u << i;
+        }
+        Spin sp;
+        for (;;) {
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                if (todo >> i & 1u) t[i] = get2(ll + at[i]);
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                if (todo >> i & 1u) {
+                    const bool two = (e[i] >> 16 & 3u) > 1;
+                    if (pieces_tag(t[i].a, tag) && (!two || pieces_tag(t[i].b, tag))) {
+                        todo &= ~(1u << i);
+                        const int row = e[i] & 0xffffu, tok = static_cast<int>(e[i] >> 18);
+                        store_packet<MT>(c.area(), tok, row, stride, t[i].a);
+                        if (two) store_packet<MT>(c.area(), tok, row + 1, stride, t[i].b);
+                    }
+                }
+            if (!todo) break;
+            if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+        }
+        if (!ok) break;
+    }
+    if (adds) {
+        float ss = 0.f;
+#pragma unroll 1
+        for (int base = c.lane; base < c.ncta && ok; base += 32 * W) {
+            if (base != c.lane) ask(base);
+            Spin sp;
+            for (;;) {
+                bool here = true;
+#pragma unroll
+                for (int i = 0; i < W; ++i)
+                    if (base + 32 * i < c.ncta) here = here && packet_tag(s[i]) == tag;
+                if (here) break;
+                if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+                ask(base);
+            }
+#pragma unroll
+            for (int i = 0; i < W; ++i)
+                if (base + 32 * i < c.ncta) ss += packet_value(s[i]);
+        }
+        ss = warp_sum(ss);
+        if (c.lane == 0) c.sh().ss[c.warp] = ss;
+    }
+    return cta_vote(ok);
+}
+
+// The MLP activations whole (K columns), from packets in natural order.
+template <int MT> __device__ __forceinline__ bool stage_activations(Ctx<MT> &c, unsigned tag) {
+    constexpr int U = 9;     // packet pairs in flight per thread
+    const StepParams &p = c.p();
+    const int K = p.F, pairs = K / 2, all = c.sh().m * pairs, stride = st_array_bytes(K);
+    bool ok = true;
+    zero_tail(c, K);
+#pragma unroll 1
+    for (int base = c.tid; base < all; base += U * ST_NT) {
+        Two t[U];
+        unsigned todo = 0;
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+            if (base + i * ST_NT < all) todo |= 1u << i;
+        auto at = [&](int i) {
+            const int u = base + i * ST_NT, tok = MT > 1 && u >= pairs ? 1 : 0;
+            return p.act_ll + static_cast<size_t>(tok) * p.act_len + 2 * (u - tok * pairs);
+        };
+        Spin sp;
+        for (;;) {
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                if (todo >> i & 1u) t[i] = get2(at(i));
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                if ((todo >> i & 1u) && pieces_tag(t[i].a, tag) && pieces_tag(t[i].b, tag)) {
+                    todo &= ~(1u << i);
+                    const int u = base + i * ST_NT, tok = MT > 1 && u >= pairs ? 1 : 0;
+                    unsigned char *to = c.area() + tok * Ctx<MT>::S * stride + (u - tok * pairs) * 4;
+#pragma unroll
+                    for (int q = 0; q < Ctx<MT>::S; ++q)
+                        *reinterpret_cast<uint32_t *>(to + q * stride) = (static_cast<uint32_t>(t[i].a >> (16 * q)) & 0xffffu) | static_cast<uint32_t>(t[i].b >> (16 * q)) << 16;
+                }
+            if (!todo) break;
+            if (!sp.again(c.abort(), p.spin_limit)) { ok = false; break; }
+        }
+        if (!ok) break;
+    }
+    return cta_vote(ok);
 }
 
 // ---- products ------------------------------------------------------------------------------------------------------------
@@ -142,7 +274,7 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
     const int K = p.cols[sl.op].K, seg = p.cols[sl.op].seg;
     float *const part = c.sh().part[sl.batch & 1];
     const int g = c.lane >> 2, t16 = (c.lane & 3) * 16;
-    const bool odd = (g & 1) != 0, paired = op_paired(sl.op), down = KEEP == 0 && sl.op == ST_DN;
+    const bool odd = (g & 1) != 0, paired = op_paired(sl.op), down = KEEP == 0 && sl.op == ST_DN && !p.act_packets;
     const int stride = st_array_bytes(down ? seg : K), slot = Ctx<MT>::NA * stride;
     const unsigned char *xb[SETS];           // this lane's array of the staged vector (columns of B past the last array: any)
 #pragma unroll

@@ -30,6 +30,8 @@ constexpr int ST_KEEP = 4;                   // 64-column blocks of the input ve
 // of the tensor-core instruction's B operand, 8 per instruction.
 __host__ __device__ constexpr int st_pieces(int mt) { return mt <= 2 ? 3 : 2; }
 __host__ __device__ constexpr int st_arrays(int mt) { return mt * st_pieces(mt); }
+// How vectors are exchanged (step_kernel.cuh): polled packets, or written plainly and fetched after an arrival.
+__host__ __device__ constexpr bool st_packets(int mt) { return mt <= 2; }
 // rows whose partial sums meet in shared memory at a time
 __host__ __device__ constexpr int st_batch(int mt) { return mt <= 2 ? 128 : mt == 4 ? 64 : 32; }
 
@@ -83,6 +85,12 @@ struct StepParams {
     unsigned char *act_vec;        // MLP activations
     int ss_stride;
     unsigned *arrivals;            // CTAs that have written their share, all exchanges of all calls
+    // One or two tokens: the same vectors as packets of 8 bytes, {three bf16 pieces, 16-bit tag}, [token] first
+    unsigned long long *x_ll, *xo_ll;   // per CTA one line of x_line packets, its last one the CTA's sum of squares {fp32, 32-bit tag}
+    unsigned long long *ao_ll;     // per CTA one line of ao_line packets
+    unsigned long long *act_ll;    // [act_len]
+    int x_line, ao_line, act_len;
+    int act_packets;               // 1: the MLP activations are staged whole, from packets; 0: they come by segments
     // packets of 8 bytes {fp32 value, tag}
     unsigned long long *q_ll;      // rotated q, k and v: [token], per CTA one line of q_line packets, {lo, hi} of its row pairs in order
     unsigned long long *part_ll;   // attention partial results [token and chunk][nq D] (unnormalised)
@@ -163,13 +171,20 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.cols[ST_DN] = step_cols(F, h_rows, false, mt <= 2 ? 2048 : 1024);      // (two segments of activations are in shared memory, as pieces)
     p.q_line = st_line(2 * most((nq + 2 * nkv) * D / 2));
     p.ss_stride = (grid + 3) / 4 * 4;
-    p.resid_at = (sh.n_layers + 1) * 64;
+    p.x_line = st_line(most(H) + 1);
+    p.ao_line = st_line(2 * most(qd / 2));
+    p.act_len = (F + 15) / 16 * 16;
+    const int total_x = grid * ((most(H) + 1) / 2), total_a = grid * most(qd / 2);
+    if (st_packets(mt) && (H >= 65536 || qd >= 65536 || grid * p.x_line / 2 >= 16384 || grid * p.ao_line / 2 >= 16384)) return "model shape does not fit the step kernel";
+    p.resid_at = (sh.n_layers + 1) * 64 + (st_packets(mt) ? 4 * (total_x + total_a) : 0);
     p.table_bytes = (p.resid_at + 4 * mt * most(H) + 127) / 128 * 128;
     // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another
     const int slot = st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg), vec = std::max(st_arrays(mt) * st_array_bytes(H) + 4 * mt * p.ss_stride, st_arrays(mt) * st_array_bytes(qd));
     int area = std::max(vec, 4 * step_scratch_floats(D, G, mt));
+    // the activations whole, if that leaves the ring half of the shared memory
+    p.act_packets = st_packets(mt) && st_arrays(mt) * st_array_bytes(F) <= smem_optin / 2;
     p.act_slots = p.cols[ST_DN].segs == 1 ? 1 : std::max(2, std::min(3, area / slot));
-    area = std::max(area, p.act_slots * slot);
+    area = std::max(area, p.act_packets ? st_arrays(mt) * st_array_bytes(F) : p.act_slots * slot);
     const int fixed = step_shared_bytes(mt) + p.table_bytes + (area + 127) / 128 * 128;
     int chunk = ST_KV_BLOCK * D * (kv8 ? 2 : 4);
     for (int o = 0; o < 5; ++o) chunk = std::max(chunk, (o == ST_O || o == ST_DN ? h_rows : ST_TILE) * p.cols[o].seg * 2);
@@ -182,7 +197,8 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.spin_limit = 1000000000u;   // 1 s
     const size_t chunks = static_cast<size_t>(std::max(grid / nkv, mt));
     sl->ll_bytes = 8 * (static_cast<size_t>(grid) * mt * p.q_line + static_cast<size_t>(grid) * 16 + chunks * qd + chunks * nq * 2) + 2 * step_vec_bytes(p, mt, H, true) +
-                   step_vec_bytes(p, mt, qd, false) + step_act_bytes(p, mt) + 256;
+                   step_vec_bytes(p, mt, qd, false) + step_act_bytes(p, mt) + 256 +
+                   (st_packets(mt) ? 8 * (static_cast<size_t>(grid) * mt * (2 * p.x_line + p.ao_line) + static_cast<size_t>(mt) * p.act_len) : 0);
     return nullptr;
 }
 // Wire the exchange buffers (256-byte aligned base).
@@ -199,7 +215,12 @@ inline void step_wire(StepLaunch *sl, int mt, unsigned long long *base) {
     p.q_ll = base; base += g * m * p.q_line;
     p.lm_ll = base; base += g * 16;
     p.part_ll = base; base += chunks * p.qd;
-    p.stat_ll = base;
+    p.stat_ll = base; base += chunks * p.nq * 2;
+    if (!st_packets(mt)) return;
+    p.x_ll = base; base += g * m * p.x_line;
+    p.xo_ll = base; base += g * m * p.x_line;
+    p.ao_ll = base; base += g * m * p.ao_line;
+    p.act_ll = base;
 }
 // Tensor map of a row-major bf16 [rows][K] matrix for the boxes of an operator: the 64-column blocks of a row are the last dimension.
 inline bool step_map(CUtensorMap *m, const StepCols &c, const void *base, int rows) {

@@ -181,8 +181,8 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another
     const int slot = st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg), vec = std::max(st_arrays(mt) * st_array_bytes(H) + 4 * mt * p.ss_stride, st_arrays(mt) * st_array_bytes(qd));
     int area = std::max(vec, 4 * step_scratch_floats(D, G, mt));
-    // the activations whole, if that leaves the ring half of the shared memory
-    p.act_packets = st_packets(mt) && st_arrays(mt) * st_array_bytes(F) <= smem_optin / 2;
+    // the activations whole if they leave the ring room to cover the latency of HBM (7B: 113 KB for them, and the stream fell to 3.9 TB/s)
+    p.act_packets = st_packets(mt) && st_arrays(mt) * st_array_bytes(F) <= 64 * 1024;
     p.act_slots = p.cols[ST_DN].segs == 1 ? 1 : std::max(2, std::min(3, area / slot));
     area = std::max(area, p.act_packets ? st_arrays(mt) * st_array_bytes(F) : p.act_slots * slot);
     const int fixed = step_shared_bytes(mt) + p.table_bytes + (area + 127) / 128 * 128;

@@ -1,83 +1,94 @@
-// The weight stream of the decode-step kernel: the order of its chunks, the ring, the L2 look-ahead.
+// The weight stream of the decode-step kernel: the list of its chunks, the ring, the L2 look-ahead, the vectors.
 #pragma once
 #include "step_prims.cuh"
 
 namespace edgefm {
 namespace step {
 
-// Calls f(part) for every chunk of the whole step in order, until f returns false.  A chunk is one or two parts of `rows` segments of
-// `seg` bytes, `stride` bytes apart in memory and packed in the ring (p1 null: one part).  Run by whole warps: the lanes share out the
-// copies.
-// With a tensor map: boxes at (0, row, block) and, for pairs, (0, row1, block) of `seg` bytes each.
-struct Part { const unsigned char *p0, *p1; int rows; unsigned seg, stride; bool kv; const unsigned char *map; int row, row1, block; };
-template <bool Q8, int MT, typename F>
-__device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f) {
+// The order of the chunks is the same in every layer, so every CTA lists them once per launch (the feeding thread's time per chunk
+// bounds the stream: with the addresses derived chunk by chunk it took about 1000 cycles from a freed slot to the next copy, and
+// a ring of three 48 KB chunks delivered 9 instead of 17 TB/s from L2).  An entry:
+//   x, y: first and second part, offset from the operator's matrix / 16 bytes (boxes: their first rows); y = ~0: one part
+//   z: bytes of a part
+//   w: 64-column block of a box | rows << 16, the row segments copied one by one (0: one copy; boxes: ST_BOX)
+constexpr unsigned ST_BOX = 255u;
+template <int MT> __device__ __forceinline__ uint4 chunk_entry(const Ctx<MT> &c, int op, int u, int n, int seg_i) {
+    const StepParams &p = c.p();
+    const StepCols &cols = p.cols[op];
+    const int half = 1 << p.half_shift;
+    const unsigned row = static_cast<unsigned>(op == ST_QKV ? (u >> p.half_shift) * p.D + (u & (half - 1)) : u), partner = row + static_cast<unsigned>(op == ST_QKV ? half : p.F);
+    const bool paired = op_paired(op);
+    const unsigned row16 = static_cast<unsigned>(cols.K) >> 3, at16 = static_cast<unsigned>(seg_i * cols.seg) >> 3;     // 16-byte units
+    if (cols.segs == 1) return make_uint4(row * row16, paired ? partner * row16 : ~0u, static_cast<unsigned>(n) * row16 * 16u, 0u);
+    if (cols.box_rows) return make_uint4(row, paired ? partner : ~0u, static_cast<unsigned>(cols.box_rows * cols.seg) * 2u, at16 >> 3 | ST_BOX << 16);
+    return make_uint4(row * row16 + at16, paired ? partner * row16 + at16 : ~0u, min(static_cast<unsigned>(cols.seg) >> 3, row16 - at16) * 16u, static_cast<unsigned>(n) << 16);
+}
+// By all threads; published by the caller's sync.
+template <int MT> __device__ __forceinline__ void make_list(const Ctx<MT> &c) {
+    Shared<MT> &sh = c.sh();
+    const StepParams &p = c.p();
+    // QKV tiles are cut at the ends of head halves, the others are regular
+    int at = 0;
+    for (int u = sh.u0[ST_QKV]; u < sh.u1[ST_QKV];) {
+        const int n = tile_units(p, ST_QKV, u, sh.u1[ST_QKV]);
+        for (int s = 0; s < p.cols[ST_QKV].segs; ++s, ++at)
+            if (c.tid == at % ST_THREADS) c.list()[at] = chunk_entry(c, ST_QKV, u, n, s);
+        u += n;
+    }
+    for (int op = ST_O; op <= ST_LM; ++op) {
+        const int tile = op_paired(op) ? ST_TILE / 2 : ST_TILE, segs = p.cols[op].segs, u0 = sh.u0[op], u1 = sh.u1[op], count = (u1 - u0 + tile - 1) / tile * segs;
+        if (c.tid == 0) sh.list[op] = at;
+        for (int i = c.tid; i < count; i += ST_THREADS) {
+            const int k = i / segs, u = u0 + k * tile;
+            c.list()[at + i] = chunk_entry(c, op, u, min(tile, u1 - u), i - k * segs);
+        }
+        at += count;
+    }
+    if (c.tid == 0) { sh.list[ST_QKV] = 0; sh.list[5] = at; }
+}
+// Calls f(base, entry, map) for the weights and f_kv(k, v, bytes) for the cache rows of the whole step in order, until one returns false.
+template <bool Q8, int MT, typename F, typename FKV>
+__device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f, FKV f_kv) {
     const Shared<MT> &sh = c.sh();
     const StepParams &p = c.p();
-    const int half = 1 << p.half_shift;
+    const uint4 *const list = c.list();
+    constexpr int E = Q8 ? 1 : 2;
+    const int shares = sh.m * p.nkv * sh.n_chunks;
+    const unsigned char *map = p.maps;
 #pragma unroll 1
     for (int layer = 0; layer <= p.n_layers; ++layer) {
+        const bool lm = layer == p.n_layers;
+        const StepLayer *L = c.layer(layer);
 #pragma unroll 1
-        for (int op = layer == p.n_layers ? ST_LM : ST_QKV; op <= (layer == p.n_layers ? ST_LM : ST_DN); ++op) {
+        for (int op = lm ? ST_LM : ST_QKV; op <= (lm ? ST_LM : ST_DN); ++op) {
             if (op == ST_O) {                                   // the cache rows come between the QKV and the O rows
-                constexpr int E = Q8 ? 1 : 2;
 #pragma unroll 1
-                for (int idx = c.cta; idx < sh.m * p.nkv * sh.n_chunks; idx += c.ncta) {
+                for (int idx = c.cta; idx < shares; idx += c.ncta) {
                     const KvShare share = kv_share(p, sh.n_old, sh.n_chunks, idx);
                     const size_t at = ((static_cast<size_t>(layer) * p.nkv + share.g) * p.max_context + share.t0) * (p.D * E);
-                    Part t{reinterpret_cast<const unsigned char *>(p.k_cache) + at, reinterpret_cast<const unsigned char *>(p.v_cache) + at, 1, 0u, 0u, true, nullptr, 0, 0, 0};
+                    const unsigned char *k = reinterpret_cast<const unsigned char *>(p.k_cache) + at, *v = reinterpret_cast<const unsigned char *>(p.v_cache) + at;
 #pragma unroll 1
                     for (int pos = share.t0; pos < share.t1; pos += ST_KV_BLOCK) {
-                        t.seg = static_cast<unsigned>(min(ST_KV_BLOCK, share.t1 - pos) * p.D * E);
-                        if (!f(t)) return;
-                        t.p0 += t.seg;
-                        t.p1 += t.seg;
+                        const unsigned bytes = static_cast<unsigned>(min(ST_KV_BLOCK, share.t1 - pos) * p.D * E);
+                        if (!f_kv(k, v, bytes)) return;
+                        k += bytes;
+                        v += bytes;
                     }
                 }
             }
-            const StepLayer *L = c.layer(layer);
-            const unsigned char *w = reinterpret_cast<const unsigned char *>(op == ST_QKV ? L->wqkv : op == ST_O ? L->wo : op == ST_GU ? L->w_gate_up
-                                                                             : op == ST_DN ? L->w_down : c.head().lm_head);
-            const unsigned row_bytes = static_cast<unsigned>(p.cols[op].K) * 2u, seg = static_cast<unsigned>(p.cols[op].seg) * 2u;
-            const int u0 = sh.u0[op], u1 = sh.u1[op];
-            const bool paired = op_paired(op), whole = seg == row_bytes;
-            const size_t partner = static_cast<size_t>(op == ST_QKV ? half : p.F) * row_bytes;
-            w += static_cast<size_t>(op == ST_QKV ? (u0 >> p.half_shift) * p.D + (u0 & (half - 1)) : u0) * row_bytes;
+            // (the first four pointers of a layer are its matrices in this order; the output layer's entry begins with its matrix)
+            const unsigned char *base = lm ? reinterpret_cast<const unsigned char *>(c.head().lm_head)
+                                           : reinterpret_cast<const unsigned char *>(reinterpret_cast<const uint16_t *const *>(L)[op]);
+            const int end = sh.list[op + 1];
 #pragma unroll 1
-            for (int u = u0; u < u1;) {
-                const int n = tile_units(p, op, u, u1);
-                Part t{w, paired ? w + partner : nullptr, whole ? 1 : n, whole ? static_cast<unsigned>(n) * row_bytes : seg, row_bytes, false, nullptr, 0, 0, 0};
-                if (whole) {
-                    if (!f(t)) return;
-                } else if (p.cols[op].box_rows) {
-                    t.map = p.maps + static_cast<size_t>(4 * layer + (op == ST_LM ? 0 : op)) * 128;
-                    t.rows = 1;
-                    t.seg = seg * static_cast<unsigned>(p.cols[op].box_rows);
-                    t.row = op == ST_QKV ? (u >> p.half_shift) * p.D + (u & (half - 1)) : u;
-                    t.row1 = t.row + (op == ST_QKV ? half : p.F);
-#pragma unroll 1
-                    for (int k = p.cols[op].segs; k > 0; --k) {
-                        if (!f(t)) return;
-                        t.block += p.cols[op].seg >> 6;
-                    }
-                } else {
-#pragma unroll 1
-                    for (unsigned at = 0; at < row_bytes; at += seg) {
-                        t.seg = min(seg, row_bytes - at);
-                        if (!f(t)) return;
-                        t.p0 += seg;
-                        if (paired) t.p1 += seg;
-                    }
-                }
-                w += static_cast<size_t>(n) * row_bytes;
-                u += n;
-                if (op == ST_QKV && (u & (half - 1)) == 0) w += partner;                    // past the partner rows of the head just finished
-            }
+            for (int i = sh.list[op]; i < end; ++i)
+                if (!f(base, list[i], map)) return;
+            map += 128;
         }
     }
 }
 
-// One warp fills the ring ...
+// One thread fills the ring ...
 template <bool Q8, int MT>
 __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
     Shared<MT> &sh = c.sh();
@@ -89,11 +100,12 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
     unsigned issued = 0, freed = 0;              // chunks copied / released so far
     unsigned at = 0, tail = 0;                   // next offset; start of the oldest chunk still in use
     unsigned sent = 0;                           // 16-byte units copied so far
-    const unsigned char *fenced = nullptr;
+    const unsigned char *fenced = nullptr, *const lm_map = p.maps + static_cast<size_t>(4 * p.n_layers) * 128;
     bool ok = true;
-    for_each_chunk<Q8>(c, [&](const Part &t) {
-        const unsigned part = static_cast<unsigned>(t.rows) * t.seg, bytes = t.p1 ? 2 * part : part, need = (bytes + 127u) & ~127u;
-        // room: chunks lie one behind the other and are never cut; the oldest are waited for until this one fits
+    // room for a chunk: chunks lie one behind the other and are never cut; the oldest are waited for until this one fits.  Returns the
+    // shared-memory address, and the barrier to complete on; 0: gave up.
+    auto room = [&](unsigned bytes, unsigned &bar) {
+        const unsigned need = (bytes + 127u) & ~127u;
         for (;;) {
             if (issued == freed) { at = 0; tail = 0; break; }
             if (issued - freed < ST_BARS) {
@@ -102,44 +114,66 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
                     if (tail > need) { at = 0; break; }
                 } else if (tail - at > need) break;
             }
-            if (!__all_sync(0xffffffffu, mbar_wait(&sh.empty[freed & (ST_BARS - 1)], (freed / ST_BARS) & 1u, c.abort(), limit))) { ok = false; return false; }
+            if (!mbar_wait(&sh.empty[freed & (ST_BARS - 1)], (freed / ST_BARS) & 1u, c.abort(), limit)) { ok = false; return 0u; }
             ++freed;
             tail = freed == issued ? at : *reinterpret_cast<volatile unsigned *>(&sh.chunk_at[freed & (ST_BARS - 1)]);
         }
-        const unsigned b = issued & (ST_BARS - 1), bar = smem_u32(&sh.full[b]);
-        if (c.lane == 0) {
-            *reinterpret_cast<volatile unsigned *>(&sh.chunk_at[b]) = at;
-            mbar_expect_tx(&sh.full[b], bytes);
-        }
-        __syncwarp();
-        const int r = c.lane & 15;
-        if (t.map) {
-            if (c.lane == 0 && (p.map_fence == 2 || (p.map_fence == 1 && t.map == p.maps + static_cast<size_t>(4 * p.n_layers) * 128)) && t.map != fenced) {
-                // order the copy engine's view of a map the host may have rewritten behind what is in memory now
-                fenced = t.map;
-                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(t.map) : "memory");
-            }
-            if (c.lane == 0)
-                asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(ring_at + at),
-                             "l"(t.map), "r"(0), "r"(t.row), "r"(t.block), "r"(bar), "l"(once)
-                             : "memory");
-            if (c.lane == 0 && t.p1)
-                asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(ring_at + at + part),
-                             "l"(t.map), "r"(0), "r"(t.row1), "r"(t.block), "r"(bar), "l"(once)
-                             : "memory");
-        } else if (r < t.rows && (c.lane < 16 || t.p1)) {
-            const unsigned char *src = (c.lane < 16 ? t.p0 : t.p1) + static_cast<size_t>(r) * t.stride;
-            const unsigned dst = ring_at + at + (c.lane < 16 ? 0u : part) + static_cast<unsigned>(r) * t.seg;
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(dst), "l"(src), "r"(t.seg),
-                         "r"(bar), "l"(t.kv ? keep : once)
-                         : "memory");
-        }
+        const unsigned b = issued & (ST_BARS - 1), to = ring_at + at;
+        bar = smem_u32(&sh.full[b]);
+        *reinterpret_cast<volatile unsigned *>(&sh.chunk_at[b]) = at;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
         at += need;
         ++issued;
         sent += bytes >> 4;
-        if (c.lane == 0) *reinterpret_cast<volatile unsigned *>(&sh.sent) = sent;
-        return true;
-    });
+        *reinterpret_cast<volatile unsigned *>(&sh.sent) = sent;
+        return to;
+    };
+    auto bulk = [&](unsigned to, const unsigned char *from, unsigned bytes, unsigned bar, unsigned long long policy) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(to), "l"(from), "r"(bytes), "r"(bar), "l"(policy)
+                     : "memory");
+    };
+    for_each_chunk<Q8>(
+        c,
+        [&](const unsigned char *base, const uint4 &e, const unsigned char *map) {
+            const bool two = e.y != ~0u;
+            const unsigned rows = e.w >> 16, part = e.z * (rows == 0u || rows == ST_BOX ? 1u : rows);
+            unsigned bar;
+            const unsigned to = room(two ? 2u * part : part, bar);
+            if (!ok) return false;
+            if (rows == 0u) {
+                bulk(to, base + static_cast<size_t>(e.x) * 16u, part, bar, once);
+                if (two) bulk(to + part, base + static_cast<size_t>(e.y) * 16u, part, bar, once);
+            } else if (rows == ST_BOX) {
+                if (map != fenced && (p.map_fence == 2 || (p.map_fence == 1 && map == lm_map))) {
+                    // order the copy engine's view of a map the host may have rewritten behind what is in memory now
+                    fenced = map;
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
+                }
+                asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(to), "l"(map),
+                             "r"(0), "r"(e.x), "r"(e.w & 0xffffu), "r"(bar), "l"(once)
+                             : "memory");
+                if (two)
+                    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(to + part),
+                                 "l"(map), "r"(0), "r"(e.y), "r"(e.w & 0xffffu), "r"(bar), "l"(once)
+                                 : "memory");
+            } else {
+                const size_t stride = static_cast<size_t>(p.cols[map == lm_map ? ST_LM : ((map - p.maps) >> 7) & 3].K) * 2;
+#pragma unroll 1
+                for (unsigned r = 0; r < rows; ++r) {
+                    bulk(to + r * e.z, base + static_cast<size_t>(e.x) * 16u + r * stride, e.z, bar, once);
+                    if (two) bulk(to + part + r * e.z, base + static_cast<size_t>(e.y) * 16u + r * stride, e.z, bar, once);
+                }
+            }
+            return true;
+        },
+        [&](const unsigned char *k, const unsigned char *v, unsigned bytes) {
+            unsigned bar;
+            const unsigned to = room(2u * bytes, bar);
+            if (!ok) return false;
+            bulk(to, k, bytes, bar, keep);
+            bulk(to + bytes, v, bytes, bar, keep);
+            return true;
+        });
     if (!ok) {               // giving up: the copies in flight must land before the CTA's shared memory is released
         int dummy = 0;
         for (unsigned k = issued > ST_BARS ? issued - ST_BARS : 0; k < issued; ++k)
@@ -151,30 +185,45 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
 template <bool Q8, int MT>
 __device__ __forceinline__ void feed_l2(Ctx<MT> &c) {
     Shared<MT> &sh = c.sh();
-    const unsigned ahead = static_cast<unsigned>(c.p().prefetch_bytes) >> 4;
+    const StepParams &p = c.p();
+    const unsigned ahead = static_cast<unsigned>(p.prefetch_bytes) >> 4;
     if (ahead == 0) return;
+    const unsigned char *const lm_map = p.maps + static_cast<size_t>(4 * p.n_layers) * 128;
     unsigned pos = 0;
-    for_each_chunk<Q8>(c, [&](const Part &t) {
-        pos += (static_cast<unsigned>(t.rows) * t.seg * (t.p1 ? 2 : 1)) >> 4;
+    bool ok = true;
+    auto due = [&](unsigned bytes) {             // waits until the chunk is near enough; false: the ring has it already (or gave up)
+        pos += bytes >> 4;
         unsigned spins = 0;
         int lead;                                // (differences: the counters may wrap)
-        while ((lead = static_cast<int>(pos - __shfl_sync(0xffffffffu, *reinterpret_cast<volatile unsigned *>(&sh.sent), 0))) > static_cast<int>(ahead)) {
-            if (__any_sync(0xffffffffu, *c.abort()) || ++spins > (1u << 22)) return false;      // bounded; a hint not given costs only time
+        while ((lead = static_cast<int>(pos - *reinterpret_cast<volatile unsigned *>(&sh.sent))) > static_cast<int>(ahead)) {
+            if (*c.abort() || ++spins > (1u << 22)) { ok = false; return false; }      // bounded; a hint not given costs only time
             __nanosleep(64);
         }
-        if (lead <= 0) return true;              // the ring has it already
-        const int r = c.lane & 15;
-        if (t.map) {
-            if (c.lane == 0 && c.p().map_fence != 2 && t.map != c.p().maps + static_cast<size_t>(4 * c.p().n_layers) * 128) {   // (only through maps that are never rewritten)
-                asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(t.map), "r"(0), "r"(t.row), "r"(t.block) : "memory");
-                if (t.p1) asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(t.map), "r"(0), "r"(t.row1), "r"(t.block) : "memory");
+        return lead > 0;
+    };
+    auto ask = [&](const unsigned char *from, unsigned bytes) { asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(from), "r"(bytes) : "memory"); };
+    for_each_chunk<Q8>(
+        c,
+        [&](const unsigned char *base, const uint4 &e, const unsigned char *map) {
+            const bool two = e.y != ~0u;
+            const unsigned rows = e.w >> 16, part = e.z * (rows == 0u || rows == ST_BOX ? 1u : rows);
+            if (!due(two ? 2u * part : part)) return ok;
+            if (rows == 0u) {
+                ask(base + static_cast<size_t>(e.x) * 16u, part);
+                if (two) ask(base + static_cast<size_t>(e.y) * 16u, part);
+            } else if (rows == ST_BOX && p.map_fence != 2 && map != lm_map) {          // (only through maps that are never rewritten)
+                asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(0), "r"(e.x), "r"(e.w & 0xffffu) : "memory");
+                if (two) asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(0), "r"(e.y), "r"(e.w & 0xffffu) : "memory");
             }
-        } else if (r < t.rows && (c.lane < 16 || t.p1))
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((c.lane < 16 ? t.p0 : t.p1) + static_cast<size_t>(r) * t.stride), "r"(t.seg) : "memory");
-        return true;
-    });
+            return true;
+        },
+        [&](const unsigned char *k, const unsigned char *v, unsigned bytes) {
+            if (!due(2u * bytes)) return ok;
+            ask(k, bytes);
+            ask(v, bytes);
+            return true;
+        });
 }
-
 // A third warp brings the vectors: when all CTAs have arrived, one bulk copy (they lie in memory as they are wanted in shared memory).
 // MLP activations come segment by segment, a few ahead of the products.  That a copy may overwrite the area follows from this CTA's
 // own arrival: it comes after the last read of what was there.

@@ -129,12 +129,14 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.u0[c.tid] = st_first(n, c.cta, c.ncta);
             sh.u1[c.tid] = st_first(n, c.cta + 1, c.ncta);
         }
+        __syncthreads();
+        make_list(c);
         __syncthreads();                 // the last sync of all threads
     }
     if (c.warp >= ST_NW) {               // the feeding warpgroup: gives its registers to the others
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ST_REGS_FEED));
-        if (c.warp == ST_NW) feed_ring<Q8, MT>(c);
-        if (c.warp == ST_NW + 1) feed_l2<Q8, MT>(c);
+        if (c.warp == ST_NW && c.lane == 0) feed_ring<Q8, MT>(c);
+        if (c.warp == ST_NW + 1 && c.lane == 0) feed_l2<Q8, MT>(c);
         if (c.warp == ST_NW + 2 && c.lane == 0 && !(st_packets(MT) && p.act_packets)) feed_vectors<MT>(c);
         return;
     }

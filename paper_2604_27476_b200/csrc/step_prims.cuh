@@ -183,6 +183,7 @@ template <int MT> struct Shared {
     float best_v[ST_NW];
     int best_i[ST_NW];
     int u0[5], u1[5];                                      // this CTA's units of every operator
+    int list[6];                                           // first entry of every operator in the chunk list
     unsigned tag0, odd;                                    // tag of layer 0; test hook: a bit no tag has
     int total_x, total_a;                                  // sizes of the unit tables
     int tokens[MT];
@@ -210,6 +211,7 @@ template <int MT> struct Ctx {
     __device__ __forceinline__ const StepLayer *layer(int l) const { return reinterpret_cast<const StepLayer *>(tables()) + l; }
     __device__ __forceinline__ const StepHead &head() const { return *reinterpret_cast<const StepHead *>(layer(p().n_layers)); }
     __device__ __forceinline__ unsigned *unit_table() const { return reinterpret_cast<unsigned *>(tables() + (p().n_layers + 1) * 64); }
+    __device__ __forceinline__ uint4 *list() const { return reinterpret_cast<uint4 *>(tables() + p().list_at); }           // chunk list
     __device__ __forceinline__ float *resid() const { return reinterpret_cast<float *>(tables() + p().resid_at); }   // [token][this CTA's rows of the residual stream]
     __device__ __forceinline__ unsigned char *area() const { return tables() + p().table_bytes; }
 };

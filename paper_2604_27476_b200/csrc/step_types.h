@@ -98,7 +98,7 @@ struct StepParams {
     unsigned long long *lm_ll;     // greedy candidates: per CTA one line, {value, row} of every token
     int q_line;
     StepCols cols[5];              // per operator
-    int ring_bytes, resid_at, table_bytes;   // shared memory (resid_at: inside the tables)
+    int ring_bytes, list_at, resid_at, table_bytes;   // shared memory (list_at, resid_at: inside the tables)
     int act_slots;                 // segments of the MLP activations in shared memory
     int prefetch_bytes;            // how far the L2 prefetch runs ahead of the ring
     int epoch_slot;                // which of the state's epochs tags this build's packets
@@ -176,7 +176,13 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.act_len = (F + 15) / 16 * 16;
     const int total_x = grid * ((most(H) + 1) / 2), total_a = grid * most(qd / 2);
     if (st_packets(mt) && (H >= 65536 || qd >= 65536 || grid * p.x_line / 2 >= 16384 || grid * p.ao_line / 2 >= 16384)) return "model shape does not fit the step kernel";
-    p.resid_at = (sh.n_layers + 1) * 64 + (st_packets(mt) ? 4 * (total_x + total_a) : 0);
+    p.list_at = ((sh.n_layers + 1) * 64 + (st_packets(mt) ? 4 * (total_x + total_a) : 0) + 15) / 16 * 16;
+    // the chunk list: tiles of the busiest CTA (QKV tiles are also cut at the ends of head halves) x segments
+    auto tiles = [&](int n, int per) { return (most(n) + per - 1) / per; };
+    const int q_most = most((nq + 2 * nkv) * D / 2);
+    const int chunks_listed = (q_most / 8 + 2 * (q_most / (D / 2) + 2)) * p.cols[ST_QKV].segs + tiles(H, ST_TILE) * (p.cols[ST_O].segs + p.cols[ST_DN].segs) +
+                              tiles(F, ST_TILE / 2) * p.cols[ST_GU].segs + tiles(sh.vocab, ST_TILE) * p.cols[ST_LM].segs;
+    p.resid_at = p.list_at + 16 * chunks_listed;
     p.table_bytes = (p.resid_at + 4 * mt * most(H) + 127) / 128 * 128;
     // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another
     const int slot = st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg), vec = std::max(st_arrays(mt) * st_array_bytes(H) + 4 * mt * p.ss_stride, st_arrays(mt) * st_array_bytes(qd));

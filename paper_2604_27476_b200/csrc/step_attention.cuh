@@ -1,155 +1,181 @@
 // Attention of the decode-step kernel: this CTA's chunk of the cached positions, the merge of the chunks.
 #pragma once
-#include "step_prims.cuh"
+#include "step_products.cuh"
 
 namespace edgefm {
 namespace step {
 
-// Queries of the group in registers (8 dims of every head per lane), K and V rows from the ring; every warp keeps a running
-// reference maximum, denominator and output of its own positions.  A score is the dot product over the D / 8 lanes of a
-// position, all heads folded at once, so that a lane ends up with the score of one (position, head).
-__device__ __forceinline__ float code_f32(uint32_t u, unsigned sel) {     // byte + 128 in the mantissa of 2^23: a signed code, exactly
-    return __uint_as_float(__byte_perm(u, 0x4B000000u, sel)) - 8388736.f;
+// The group's heads are the rows of tensor-core products: scores[head][position] = Q K^T takes the 8 heads' first two bf16 pieces as rows
+// 0-7 and 8-15 of one m16n8k16 and the third as the rows of another (24 bits of the query, as the fp32 query it was), and
+// out[head][dim] = P V the same of the probabilities; K and V enter as they are cached (signed bytes are exact in bf16).  The scores'
+// registers are P's operand as they stand.  (With packed FMAs the phase took 30 us per layer for 32768 positions of 4 x 7 heads of
+// 128, 2.3 TB/s of K and V.)
+//   A tile is 16 positions.  Which positions is free as long as K's rows, V's rows and P agree: a block of n positions falls into four
+// quarters of R rows, and tile i takes rows 4 i .. 4 i + 3 of every quarter, so that the four lanes of a V operand read from four
+// quarters; those lie 32 bytes further apart than their rows fill, and the reads are free of bank conflicts.
+__device__ __forceinline__ uint32_t codes_bf16(uint32_t w, unsigned sel) {     // two signed bytes: (128 + low 7 bits) - (128 or 256)
+    const uint32_t x = __byte_perm(w, 0x43434343u, sel), lo = x & 0xff7fff7fu, sign = x & 0xff80ff80u;
+    uint32_t r;
+    asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(lo), "r"(sign));
+    return r;
 }
-__device__ __forceinline__ void codes8_to_f2(uint2 w, f2 (&f)[4]) {
-    const uint32_t a = w.x ^ 0x80808080u, b = w.y ^ 0x80808080u;
-    f[0] = pack2(code_f32(a, 0x7440), code_f32(a, 0x7441)); f[1] = pack2(code_f32(a, 0x7442), code_f32(a, 0x7443));
-    f[2] = pack2(code_f32(b, 0x7440), code_f32(b, 0x7441)); f[3] = pack2(code_f32(b, 0x7442), code_f32(b, 0x7443));
+__device__ __forceinline__ uint32_t two_bf16(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
 }
+// The split of a block of n cached positions (kv_block) in shared memory: K rows one behind the other, then the quarters of V.
+struct KvBlock {
+    int n, R, v_at, v_stride;
+    __device__ __forceinline__ KvBlock(int n_, int row_bytes) : n(n_), R((n_ + 15) / 16 * 4), v_at((n_ * row_bytes + 127) / 128 * 128), v_stride(R * row_bytes + 32) {}
+    __device__ __forceinline__ int bytes() const { return v_at + 4 * v_stride; }
+};
 
 template <int D, int G, bool Q8>
 struct WarpAttention {
-    static constexpr int LPR = D / 8, SP = 32 / LPR, DV = D / 32;   // eight positions per warp and block, SP at a time
-    static constexpr int ROW = Q8 ? D : 2 * D;
-    f2 q[G][4];
-    f2 o[G][DV / 2];
-    float m, l;                       // of this lane's head
-    __device__ __forceinline__ void start(const float *qs, int lane) {
-        const int sub = lane & (LPR - 1);
+    static constexpr int KS = D / 16, ROW = Q8 ? D : 2 * D, WD = D / 64;    // a warp multiplies P by 64 dims of V: WD warps per tile
+    uint32_t q[KS][3][2];             // pieces of the query of head lane / 4
+    float o[8][4];                    // dims 16 (lane % 4) + 8 e + i of this lane's head: o[i][e] + o[i][e + 2]
+    float m, l;                       // of this lane's head; l: of this lane's positions
+    static __device__ __forceinline__ int dim_of(int k, int t) { return Q8 ? 64 * (k >> 2) + 16 * t + 4 * (k & 3) : 32 * (k >> 1) + 8 * t + 4 * (k & 1); }
+    __device__ __forceinline__ void start(const unsigned char *qs, int lane) {
+        const int g = lane >> 2, t = lane & 3;
 #pragma unroll
-        for (int h = 0; h < G; ++h) {
-            const float4 a = *reinterpret_cast<const float4 *>(qs + h * D + sub * 8), b = *reinterpret_cast<const float4 *>(qs + h * D + sub * 8 + 4);
-            q[h][0] = pack2(a.x, a.y); q[h][1] = pack2(a.z, a.w); q[h][2] = pack2(b.x, b.y); q[h][3] = pack2(b.z, b.w);
+        for (int k = 0; k < KS; ++k)
 #pragma unroll
-            for (int e = 0; e < DV / 2; ++e) o[h][e] = 0ull;
-        }
+            for (int i = 0; i < 3; ++i) {
+                const uint2 w = g < G ? *reinterpret_cast<const uint2 *>(qs + ((i * G + g) * D + dim_of(k, t)) * 2) : make_uint2(0u, 0u);
+                q[k][i][0] = w.x;
+                q[k][i][1] = w.y;
+            }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
         m = -INFINITY;
         l = 0.f;
     }
-    static __device__ __forceinline__ int head_of(int lane) { return folded<8>(lane & (LPR - 1), LPR); }
-    // Positions [first, first + cnt) (cnt <= 8) of the block at kb / vb; ks / vs: scales of these rows (compressed cache);
-    // pw: this warp's 8 x 8 probabilities.
-    __device__ __forceinline__ void block(const unsigned char *kb, const unsigned char *vb, const float *ks, const float *vs, int first, int cnt, float *pw, int lane) {
-        const int sub = lane & (LPR - 1), grp = lane / LPR, h_mine = head_of(lane);
-        // (a loop, the scores parked in shared memory by the lane that needs them again: unrolled, the code of a layer outgrows the
-        // instruction cache and every phase starts with misses)
-        float mx = -INFINITY;
-#pragma unroll 1
-        for (int st = 0; st * SP < cnt; ++st) {
-            const int pos = first + min(st * SP + grp, cnt - 1);
-            f2 kf[4];
-            if constexpr (Q8) {
-                codes8_to_f2(*reinterpret_cast<const uint2 *>(kb + pos * ROW + sub * 8), kf);
-            } else {
-                const uint4 w = *reinterpret_cast<const uint4 *>(kb + pos * ROW + sub * 16);
-                kf[0] = bf16x2_f2(w.x); kf[1] = bf16x2_f2(w.y); kf[2] = bf16x2_f2(w.z); kf[3] = bf16x2_f2(w.w);
-            }
-            float v[8];
+    // Tile i of a block; ks / vs: scales of this lane's four positions (compressed cache); dg: which 64 dims of V.
+    __device__ __forceinline__ void tile(const unsigned char *kb, const unsigned char *vb, const KvBlock &b, int i, const float (&ks)[4], const float (&vs)[4], int dg, int lane) {
+        const int g = lane >> 2, t = lane & 3, own = t * b.R + 4 * i;       // this lane's positions: own .. own + 3
+        const bool odd = (g & 1) != 0;
+        // V first: its loads fly while the scores are made
+        uint32_t v[4][Q8 ? 2 : 4];
+        const int last = b.n - 1, lq = (last >= b.R) + (last >= 2 * b.R) + (last >= 3 * b.R);
 #pragma unroll
-            for (int h = 0; h < 8; ++h) {
-                v[h] = 0.f;
-                if (h < G) {
-                    f2 a = fma2(kf[0], q[h < G ? h : 0][0], 0ull);
-                    a = fma2(kf[1], q[h < G ? h : 0][1], a);
-                    a = fma2(kf[2], q[h < G ? h : 0][2], a);
-                    a = fma2(kf[3], q[h < G ? h : 0][3], a);
-                    const float2 t = unpack2(a);
-                    v[h] = t.x + t.y;
+        for (int k = 0; k < 4; ++k) {
+            const bool in = own + k < b.n;                                  // (past the end: any row, its probability is zero)
+            const unsigned char *row = vb + (in ? t : lq) * b.v_stride + (in ? 4 * i + k : last - lq * b.R) * ROW;
+            if constexpr (Q8) {
+                const uint2 w = *reinterpret_cast<const uint2 *>(row + dg * 64 + g * 8);
+                v[k][0] = w.x; v[k][1] = w.y;
+            } else {
+                const uint4 w = *reinterpret_cast<const uint4 *>(row + dg * 128 + g * 16);
+                v[k][0] = w.x; v[k][1] = w.y; v[k][Q8 ? 0 : 2] = w.z; v[k][Q8 ? 1 : 3] = w.w;
+            }
+        }
+        float s[4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const unsigned char *row = kb + min((g >> 1) * b.R + 4 * i + (g & 1) + 2 * j, last) * ROW + t * 16;
+            float a[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
+            auto step = [&](int k, uint32_t b0, uint32_t b1) {
+                mma(a, q[k][0][0], q[k][1][0], q[k][0][1], q[k][1][1], b0, b1);
+                mma(e, q[k][2][0], 0u, q[k][2][1], 0u, b0, b1);
+            };
+            auto codes = [&](int k, uint32_t w) { step(k, codes_bf16(w, 0x4140), codes_bf16(w, 0x4342)); };
+            // rows 128 bytes (or a multiple) apart start on the same bank: odd ones read the second 64 bytes first
+            if constexpr (Q8 && D == 64) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(row);
+                codes(0, w.x); codes(1, w.y); codes(2, w.z); codes(3, w.w);
+            } else {
+#pragma unroll
+                for (int k = 0; k < ROW / 128; ++k) {
+                    const uint4 x = *reinterpret_cast<const uint4 *>(row + k * 128 + (odd ? 64 : 0)), y = *reinterpret_cast<const uint4 *>(row + k * 128 + (odd ? 0 : 64));
+                    const uint4 w = pick(odd, x, y), z = pick(odd, y, x);
+                    if constexpr (Q8) {
+                        codes(0, w.x); codes(1, w.y); codes(2, w.z); codes(3, w.w);
+                        codes(KS - 4, z.x); codes(KS - 3, z.y); codes(KS - 2, z.z); codes(KS - 1, z.w);
+                    } else {
+                        step(4 * k, w.x, w.y); step(4 * k + 1, w.z, w.w);
+                        step(4 * k + 2, z.x, z.y); step(4 * k + 3, z.z, z.w);
+                    }
                 }
             }
-            float r = fold<8>(v, sub, LPR);
-            if (Q8 && st * SP + grp < cnt) r *= ks[st * SP + grp];
-            if (st * SP + grp >= cnt) r = -INFINITY;
-            mx = fmaxf(mx, r);
-            pw[(st * SP + grp) * 8 + h_mine] = r;
+            s[2 * j] = a[0] + a[2] + e[0];
+            s[2 * j + 1] = a[1] + a[3] + e[1];
         }
+        float mx = -INFINITY;
 #pragma unroll
-        for (int k = LPR; k < 32; k <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, k));
+        for (int k = 0; k < 4; ++k) {
+            if constexpr (Q8) s[k] *= ks[k];
+            if (own + k >= b.n) s[k] = -INFINITY;
+            mx = fmaxf(mx, s[k]);
+        }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         // the reference maximum moves only when it has grown by more than 2^8 (the probabilities may then reach 2^8)
         if (__any_sync(0xffffffffu, mx > m + 8.f)) {
             const float mn = fmaxf(m, mx), f = m == -INFINITY ? 0.f : exp2_approx(m - mn);
             l *= f;
             m = mn;
 #pragma unroll
-            for (int h = 0; h < G; ++h) {
-                // a lane that holds head h: the bits of folded() from the top
-                constexpr int S1 = LPR >> 1, S2 = LPR >> 2, S3 = LPR >> 3;
-                const float fh = __shfl_sync(0xffffffffu, f, ((h & 4) ? S1 : 0) | ((h & 2) ? S2 : 0) | ((h & 1) ? S3 : 0));
-                const f2 fh2 = pack2(fh, fh);
+            for (int k = 0; k < 8; ++k) { o[k][0] *= f; o[k][1] *= f; o[k][2] *= f; o[k][3] *= f; }
+        }
+        uint32_t p[3][2];
 #pragma unroll
-                for (int e = 0; e < DV / 2; ++e) o[h][e] = fma2(o[h][e], fh2, 0ull);
+        for (int j = 0; j < 2; ++j) {
+            float x = exp2_approx(s[2 * j] - m), y = exp2_approx(s[2 * j + 1] - m);
+            l += x + y;
+            if constexpr (Q8) { x *= vs[2 * j]; y *= vs[2 * j + 1]; }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                p[k][j] = two_bf16(x, y);
+                x -= bf16lo(p[k][j]);
+                y -= bf16hi(p[k][j]);
             }
         }
-#pragma unroll 1
-        for (int i = grp; i < cnt; i += SP) {
-            const float pr = exp2_approx(pw[i * 8 + h_mine] - m);
-            l += pr;
-            pw[i * 8 + h_mine] = Q8 ? pr * vs[i] : pr;
-        }
-        __syncwarp();
-#pragma unroll 2
-        for (int i = 0; i < cnt; ++i) {
-            f2 v[DV / 2];
-            const unsigned char *row = vb + (first + i) * ROW;
-            if constexpr (Q8) {
-                uint32_t w;
-                if constexpr (DV == 4) w = *reinterpret_cast<const uint32_t *>(row + lane * 4);
-                else w = *reinterpret_cast<const uint16_t *>(row + lane * 2);
-                const uint32_t u = w ^ 0x80808080u;
+        auto out = [&](int k, uint32_t b0, uint32_t b1) {
+            mma(o[k], p[0][0], p[1][0], p[0][1], p[1][1], b0, b1);
+            mma(o[k], p[2][0], 0u, p[2][1], 0u, b0, b1);
+        };
+        if constexpr (Q8) {
 #pragma unroll
-                for (int e = 0; e < DV / 2; ++e) v[e] = pack2(code_f32(u, 0x7440 + 2 * e), code_f32(u, 0x7441 + 2 * e));
-            } else if constexpr (DV == 4) {
-                const uint2 w = *reinterpret_cast<const uint2 *>(row + lane * 8);
-                v[0] = bf16x2_f2(w.x);
-                v[DV / 2 - 1] = bf16x2_f2(w.y);
-            } else {
-                v[0] = bf16x2_f2(*reinterpret_cast<const uint32_t *>(row + lane * 4));
-            }
-            const float4 pa = *reinterpret_cast<const float4 *>(pw + i * 8), pb = *reinterpret_cast<const float4 *>(pw + i * 8 + 4);
-            const float pr[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+            for (int w = 0; w < 2; ++w)
 #pragma unroll
-            for (int h = 0; h < G; ++h) {
-                const f2 pp = pack2(pr[h], pr[h]);
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t x = __byte_perm(v[0][w], v[1][w], h ? 0x7362 : 0x5140), y = __byte_perm(v[2][w], v[3][w], h ? 0x7362 : 0x5140);
+                    out(4 * w + 2 * h, codes_bf16(x, 0x4140), codes_bf16(y, 0x4140));
+                    out(4 * w + 2 * h + 1, codes_bf16(x, 0x4342), codes_bf16(y, 0x4342));
+                }
+        } else {
 #pragma unroll
-                for (int e = 0; e < DV / 2; ++e) o[h][e] = fma2(pp, v[e], o[h][e]);
+            for (int w = 0; w < 4; ++w) {
+                constexpr int Z = Q8 ? 1 : 3;
+                out(2 * w, __byte_perm(v[0][w & Z], v[1][w & Z], 0x5410), __byte_perm(v[2][w & Z], v[3][w & Z], 0x5410));
+                out(2 * w + 1, __byte_perm(v[0][w & Z], v[1][w & Z], 0x7632), __byte_perm(v[2][w & Z], v[3][w & Z], 0x7632));
             }
         }
-        __syncwarp();
     }
-    // (m, l, o) to shared memory: mm, ml [NW][8], mo [NW][G][D]
+    // (m, l, o) to shared memory: mm, ml [NW][8], mo [NW][G][64]
     __device__ __forceinline__ void leave(float *mm, float *ml, float *mo, int warp, int lane) {
-        float lt = l;
+        const int g = lane >> 2, t = lane & 3;
+        l += __shfl_xor_sync(0xffffffffu, l, 1);
+        l += __shfl_xor_sync(0xffffffffu, l, 2);
+        if (g >= G) return;
+        if (t == 0) { mm[warp * 8 + g] = m; ml[warp * 8 + g] = l; }
+        float *d = mo + (warp * G + g) * 64 + 16 * t;
 #pragma unroll
-        for (int k = LPR; k < 32; k <<= 1) lt += __shfl_xor_sync(0xffffffffu, lt, k);
-        if (lane < LPR) { mm[warp * 8 + head_of(lane)] = m; ml[warp * 8 + head_of(lane)] = lt; }
+        for (int e = 0; e < 2; ++e)
 #pragma unroll
-        for (int h = 0; h < G; ++h) {
-            float *d = mo + (warp * G + h) * D + lane * DV;
-            if constexpr (DV == 4) {
-                const float2 a = unpack2(o[h][0]), b = unpack2(o[h][DV / 2 - 1]);
-                *reinterpret_cast<float4 *>(d) = make_float4(a.x, a.y, b.x, b.y);
-            } else {
-                *reinterpret_cast<float2 *>(d) = unpack2(o[h][0]);
-            }
-        }
+            for (int i = 0; i < 8; i += 4)
+                *reinterpret_cast<float4 *>(d + 8 * e + i) = make_float4(o[i][e] + o[i][e + 2], o[i + 1][e] + o[i + 1][e + 2], o[i + 2][e] + o[i + 2][e + 2], o[i + 3][e] + o[i + 3][e + 2]);
     }
 };
 
-// Shared-memory scratch of the attention, in floats: queries | new k rows, new v rows (as cached), their scales | probabilities | warp
-// maxima, denominators, outputs | scales of the warps' rows (compressed cache).  The fp32 new rows share the place of the warp outputs.
+// Shared-memory scratch of the attention, in floats: the queries' pieces | new k rows, new v rows (as cached), their scales | warp maxima,
+// denominators, outputs.  The fp32 new rows share the place of the warp outputs.
 template <int D, int G, int MT> struct AttScratch {
-    static constexpr int QS = 0, NEW = QS + G * D, NSC = NEW + MT * D, PW = NSC + 16, MM = PW + ST_NW * 64, ML = MM + ST_NW * 8, MO = ML + ST_NW * 8,
-                         RAW = 2 * MT * D, SC = MO + (ST_NW * G * D > RAW ? ST_NW * G * D : RAW), FLOATS = SC + 2 * ST_KV_BLOCK;
+    static constexpr int QS = 0, NEW = QS + (3 * G * D / 2 + 3) / 4 * 4, NSC = NEW + MT * D, MM = NSC + 16, ML = MM + ST_NW * 8, MO = ML + ST_NW * 8,
+                         RAW = 2 * MT * D, FLOATS = MO + (ST_NW * G * 64 > RAW ? ST_NW * G * 64 : RAW);
 };
 
 // Token share.tok, kv head share.g, the chunk [t0, t1) of the old positions; the last chunk also attends to the rows of the call's tokens
@@ -201,9 +227,16 @@ __device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &sha
                 const int j = j0 + i * ST_NT, kv = j - q_units;
                 const float lo = packet_value(t[i].a), hi = packet_value(t[i].b);
                 if (kv < 0) {
-                    float *d = base + A::QS + (j / half) * D + (j & (half - 1));
-                    d[0] = lo * p.q_scale;
-                    d[half] = hi * p.q_scale;
+                    unsigned char *d = reinterpret_cast<unsigned char *>(base + A::QS) + ((j / half) * D + (j & (half - 1))) * 2;
+                    float x = lo * p.q_scale, y = hi * p.q_scale;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const uint32_t w = two_bf16(x, y);
+                        store_u16(d + k * G * D * 2, static_cast<uint16_t>(w));
+                        store_u16(d + k * G * D * 2 + half * 2, static_cast<uint16_t>(w >> 16));
+                        x -= bf16lo(w);
+                        y -= bf16hi(w);
+                    }
                 } else {
                     const int at_row = ((kv & half) ? n_new : 0) + kv / (2 * half);       // k rows, then v rows
                     if constexpr (Q8) {          // fp32 for the compression below
@@ -250,33 +283,35 @@ __device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &sha
         }
     }
     W att;
-    att.start(base + A::QS, c.lane);
-    float *pw = base + A::PW + c.warp * 64;
-    // (the new rows come last, by the last warp of the CTA that ends with them)
+    att.start(reinterpret_cast<const unsigned char *>(base + A::QS), c.lane);
+    const int my_tile = c.warp / W::WD, dg = c.warp & (W::WD - 1), quad = c.lane & 3;
+    // (the new rows come last, by the last warps of the CTA that ends with them)
 #pragma unroll 1
-    for (int t = share.t0;; t += ST_KV_BLOCK) {
+    for (int t = share.t0;; t += kv_block(D)) {
         const bool fresh = t >= share.t1;
         if (fresh && n_new == 0) break;
-        const int n = fresh ? n_new : min(ST_KV_BLOCK, share.t1 - t);
-        const int steps = (n + W::SP - 1) / W::SP, per_warp = (steps + ST_NW - 1) / ST_NW * W::SP;   // positions of a warp, whole steps
-        int first = c.warp * per_warp, cnt = min(per_warp, n - first);
-        const float *ksc = base + A::NSC, *vsc = ksc + 8;
+        KvBlock b(fresh ? n_new : min(kv_block(D), share.t1 - t), W::ROW);
+        const int i = fresh ? ST_NW / W::WD - 1 - my_tile : my_tile, own = quad * b.R + 4 * i;
+        const bool on = 4 * i < b.R;
+        float ks[4] = {0.f, 0.f, 0.f, 0.f}, vs[4] = {0.f, 0.f, 0.f, 0.f};
         const unsigned char *at = reinterpret_cast<const unsigned char *>(base + A::NEW);
-        if (fresh) {
-            first = 0;
-            cnt = c.warp == ST_NW - 1 ? n : 0;
-        } else {
-            if constexpr (Q8) {         // every warp fetches the scales of its own positions
-                float *own = base + A::SC + c.warp * 16;
-                const size_t row = (static_cast<size_t>(layer) * p.nkv + share.g) * p.max_context + t + first;
-                if (c.lane < cnt) { own[c.lane] = __ldcg(p.k_scale + row + c.lane); own[8 + c.lane] = __ldcg(p.v_scale + row + c.lane); }
-                __syncwarp();
-                ksc = own;
-                vsc = own + 8;
-            }
-            if (!chunk_wait(c, at)) { ok = false; break; }
+        if constexpr (Q8) {             // the scales of this lane's positions, asked for before the rows are awaited
+            const size_t row = (static_cast<size_t>(layer) * p.nkv + share.g) * p.max_context + t + own;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (on && own + k < b.n) {
+                    ks[k] = fresh ? base[A::NSC + own + k] : __ldcg(p.k_scale + row + k);
+                    vs[k] = fresh ? base[A::NSC + 8 + own + k] : __ldcg(p.v_scale + row + k);
+                }
         }
-        if (cnt > 0) att.block(at, at + n * W::ROW, ksc, vsc, first, cnt, pw, c.lane);
+        if (fresh) {
+            b.v_at = n_new * W::ROW;
+            b.v_stride = b.R * W::ROW;
+        } else if (!chunk_wait(c, at)) {
+            ok = false;
+            break;
+        }
+        if (on) att.tile(at, at + b.v_at, b, i, ks, vs, dg, c.lane);
         if (fresh) break;
         chunk_release(c);
     }
@@ -286,15 +321,15 @@ __device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &sha
     const size_t slot = static_cast<size_t>(share.tok) * c.sh().n_chunks + share.chunk;
 #pragma unroll 1
     for (int j = c.tid; j < G * half; j += ST_NT) {
-        const int h = j / half, d2 = j - h * half;
-        float mw[ST_NW], mm = -INFINITY;
+        const int h = j / half, d2 = j - h * half, dg = D == 64 ? 0 : d2 >> 5;      // (dims of group dg: every WD-th warp)
+        float mw[ST_NW / W::WD], mm = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < ST_NW; ++w) { mw[w] = base[A::MM + w * 8 + h]; mm = fmaxf(mm, mw[w]); }
+        for (int w = 0; w < ST_NW / W::WD; ++w) { mw[w] = base[A::MM + w * W::WD * 8 + h]; mm = fmaxf(mm, mw[w]); }
         float a = 0.f, b = 0.f;
 #pragma unroll
-        for (int w = 0; w < ST_NW; ++w) {
+        for (int w = 0; w < ST_NW / W::WD; ++w) {
             const float e = exp2_approx(mw[w] - mm);
-            const float2 v = *reinterpret_cast<const float2 *>(base + A::MO + (w * G + h) * D + 2 * d2);
+            const float2 v = *reinterpret_cast<const float2 *>(base + A::MO + ((w * W::WD + dg) * G + h) * 64 + 2 * (d2 & 31));
             a = fmaf(v.x, e, a);
             b = fmaf(v.y, e, b);
         }
@@ -303,9 +338,9 @@ __device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &sha
     if (c.tid < G) {                    // maximum and denominator of every head, one store
         float mm = -INFINITY, ll = 0.f;
 #pragma unroll
-        for (int w = 0; w < ST_NW; ++w) mm = fmaxf(mm, base[A::MM + w * 8 + c.tid]);
+        for (int w = 0; w < ST_NW; w += W::WD) mm = fmaxf(mm, base[A::MM + w * 8 + c.tid]);
 #pragma unroll
-        for (int w = 0; w < ST_NW; ++w) ll = fmaf(base[A::ML + w * 8 + c.tid], exp2_approx(base[A::MM + w * 8 + c.tid] - mm), ll);
+        for (int w = 0; w < ST_NW; w += W::WD) ll = fmaf(base[A::ML + w * 8 + c.tid], exp2_approx(base[A::MM + w * 8 + c.tid] - mm), ll);
         put2(p.stat_ll + (slot * p.nq + share.g * G + c.tid) * 2, mm, ll, tag);
     }
     return true;

@@ -1,6 +1,6 @@
 // The weight stream of the decode-step kernel: the list of its chunks, the ring, the L2 look-ahead, the vectors.
 #pragma once
-#include "step_prims.cuh"
+#include "step_attention.cuh"
 
 namespace edgefm {
 namespace step {
@@ -46,13 +46,14 @@ template <int MT> __device__ __forceinline__ void make_list(const Ctx<MT> &c) {
     }
     if (c.tid == 0) { sh.list[ST_QKV] = 0; sh.list[5] = at; }
 }
-// Calls f(base, entry, map) for the weights and f_kv(k, v, bytes) for the cache rows of the whole step in order, until one returns false.
+// Calls f(base, entry, map) for the weights and f_kv(k, v, rows, bytes of each) for the cache rows of the whole step in order, until one returns false.
 template <bool Q8, int MT, typename F, typename FKV>
 __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f, FKV f_kv) {
     const Shared<MT> &sh = c.sh();
     const StepParams &p = c.p();
     const uint4 *const list = c.list();
     constexpr int E = Q8 ? 1 : 2;
+    const int block = kv_block(p.D), row_bytes = p.D * E;
     const int shares = sh.m * p.nkv * sh.n_chunks;
     const unsigned char *map = p.maps;
 #pragma unroll 1
@@ -68,9 +69,10 @@ __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f, FKV f_kv) 
                     const size_t at = ((static_cast<size_t>(layer) * p.nkv + share.g) * p.max_context + share.t0) * (p.D * E);
                     const unsigned char *k = reinterpret_cast<const unsigned char *>(p.k_cache) + at, *v = reinterpret_cast<const unsigned char *>(p.v_cache) + at;
 #pragma unroll 1
-                    for (int pos = share.t0; pos < share.t1; pos += ST_KV_BLOCK) {
-                        const unsigned bytes = static_cast<unsigned>(min(ST_KV_BLOCK, share.t1 - pos) * p.D * E);
-                        if (!f_kv(k, v, bytes)) return;
+                    for (int pos = share.t0; pos < share.t1; pos += block) {
+                        const int n = min(block, share.t1 - pos);
+                        const unsigned bytes = static_cast<unsigned>(n * row_bytes);
+                        if (!f_kv(k, v, n, bytes)) return;
                         k += bytes;
                         v += bytes;
                     }
@@ -104,8 +106,8 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
     bool ok = true;
     // room for a chunk: chunks lie one behind the other and are never cut; the oldest are waited for until this one fits.  Returns the
     // shared-memory address, and the barrier to complete on; 0: gave up.
-    auto room = [&](unsigned bytes, unsigned &bar) {
-        const unsigned need = (bytes + 127u) & ~127u;
+    auto room = [&](unsigned bytes, unsigned space, unsigned &bar) {
+        const unsigned need = (space + 127u) & ~127u;
         for (;;) {
             if (issued == freed) { at = 0; tail = 0; break; }
             if (issued - freed < ST_BARS) {
@@ -138,7 +140,7 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
             const bool two = e.y != ~0u;
             const unsigned rows = e.w >> 16, part = e.z * (rows == 0u || rows == ST_BOX ? 1u : rows);
             unsigned bar;
-            const unsigned to = room(two ? 2u * part : part, bar);
+            const unsigned all = two ? 2u * part : part, to = room(all, all, bar);
             if (!ok) return false;
             if (rows == 0u) {
                 bulk(to, base + static_cast<size_t>(e.x) * 16u, part, bar, once);
@@ -166,12 +168,16 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
             }
             return true;
         },
-        [&](const unsigned char *k, const unsigned char *v, unsigned bytes) {
+        [&](const unsigned char *k, const unsigned char *v, int n, unsigned bytes) {
+            const int row_bytes = p.D * (Q8 ? 1 : 2);
+            const KvBlock b(n, row_bytes);
             unsigned bar;
-            const unsigned to = room(2u * bytes, bar);
+            const unsigned to = room(2u * bytes, static_cast<unsigned>(b.bytes()), bar);
             if (!ok) return false;
             bulk(to, k, bytes, bar, keep);
-            bulk(to + bytes, v, bytes, bar, keep);
+#pragma unroll 1
+            for (int i = 0; i * b.R < n; ++i)
+                bulk(to + b.v_at + i * b.v_stride, v + static_cast<size_t>(i * b.R) * row_bytes, static_cast<unsigned>(min(b.R, n - i * b.R) * row_bytes), bar, keep);
             return true;
         });
     if (!ok) {               // giving up: the copies in flight must land before the CTA's shared memory is released
@@ -217,7 +223,7 @@ __device__ __forceinline__ void feed_l2(Ctx<MT> &c) {
             }
             return true;
         },
-        [&](const unsigned char *k, const unsigned char *v, unsigned bytes) {
+        [&](const unsigned char *k, const unsigned char *v, int, unsigned bytes) {
             if (!due(2u * bytes)) return ok;
             ask(k, bytes);
             ask(v, bytes);

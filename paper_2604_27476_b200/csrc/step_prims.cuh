@@ -1,4 +1,4 @@
-// Primitives of the decode-step kernel: barriers, bounded waits, packets, packed fp32 arithmetic.
+// Primitives of the decode-step kernel: barriers, bounded waits, packets.
 #pragma once
 #include "step_types.h"
 
@@ -111,55 +111,10 @@ __device__ __forceinline__ unsigned long long get1(const unsigned long long *at)
     return v;
 }
 
-// Two fp32 values in one 64-bit register pair.
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 pack2(float a, float b) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f2 bf16x2_f2(uint32_t w) { return pack2(bf16lo(w), bf16hi(w)); }
 __device__ __forceinline__ float exp2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-// sum over the lanes of a row (lpr of them) of N values at once: halves the values while it folds, then sums what is left
-template <int N>
-__device__ __forceinline__ float fold(float (&v)[N], int sub, int lpr) {
-    int mask = lpr >> 1;
-#pragma unroll
-    for (int n = N / 2; n >= 1; n >>= 1) {
-        const bool up = (sub & mask) != 0;
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-            const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
-        }
-        mask >>= 1;
-    }
-#pragma unroll 1
-    for (; mask; mask >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
-    return v[0];
-}
-// which of the N values fold() left in a lane
-template <int N>
-__device__ __forceinline__ int folded(int sub, int lpr) {
-    int idx = 0, mask = lpr >> 1;
-#pragma unroll
-    for (int n = N; n > 1; n >>= 1) { idx = idx * 2 + ((sub & mask) ? 1 : 0); mask >>= 1; }
-    return idx;
 }
 
 __device__ __forceinline__ float sum8(const float *at) {

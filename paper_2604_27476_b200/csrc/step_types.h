@@ -20,7 +20,8 @@ constexpr int ST_BARS = 16;                  // chunks the ring can hold at once
 constexpr int ST_CHUNK_BYTES = 52 * 1024;    // aimed at for a ring chunk cut by columns
 constexpr int ST_CHUNK_WHOLE = 68 * 1024;    // a tile of whole rows may be this large
 constexpr int ST_TILE = 16;                  // rows of a tile: the M of one m16n8k16 tensor-core instruction (pairs: 8 and their partners)
-constexpr int ST_KV_BLOCK = 8 * ST_NW;       // cached positions per ring chunk: eight per warp
+// cached positions per ring chunk: a warp multiplies 16 of them by 64 dims
+__host__ __device__ constexpr int kv_block(int D) { return 16 * ST_NW / (D / 64); }
 constexpr int ST_MIN_CHUNK = 16;             // fewest cached positions a CTA attends to (shorter contexts occupy fewer CTAs)
 constexpr int ST_PREFETCH_BYTES = 352 * 1024;   // L2 look-ahead per CTA beyond the ring
 constexpr int ST_KEEP = 4;                   // 64-column blocks of the input vector a warp can keep in registers
@@ -192,7 +193,7 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.act_slots = p.cols[ST_DN].segs == 1 ? 1 : std::max(2, std::min(3, area / slot));
     area = std::max(area, p.act_packets ? st_arrays(mt) * st_array_bytes(F) : p.act_slots * slot);
     const int fixed = step_shared_bytes(mt) + p.table_bytes + (area + 127) / 128 * 128;
-    int chunk = ST_KV_BLOCK * D * (kv8 ? 2 : 4);
+    int chunk = kv_block(D) * D * (kv8 ? 2 : 4) + 4 * 32;      // (K rows, then V in four quarters 32 bytes apart)
     for (int o = 0; o < 5; ++o) chunk = std::max(chunk, (o == ST_O || o == ST_DN ? h_rows : ST_TILE) * p.cols[o].seg * 2);
     sl->max_chunk_bytes = (chunk + 127) / 128 * 128;
     const int ring = (smem_optin - fixed) / 128 * 128;

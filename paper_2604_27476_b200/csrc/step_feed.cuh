@@ -36,7 +36,7 @@ template <int MT> __device__ __forceinline__ void make_list(const Ctx<MT> &c) {
         u += n;
     }
     for (int op = ST_O; op <= ST_LM; ++op) {
-        const int tile = op_paired(op) ? ST_TILE / 2 : ST_TILE, segs = p.cols[op].segs, u0 = sh.u0[op], u1 = sh.u1[op], count = (u1 - u0 + tile - 1) / tile * segs;
+        const int tile = p.cols[op].tile, segs = p.cols[op].segs, u0 = sh.u0[op], u1 = sh.u1[op], count = (u1 - u0 + tile - 1) / tile * segs;
         if (c.tid == 0) sh.list[op] = at;
         for (int i = c.tid; i < count; i += ST_THREADS) {
             const int k = i / segs, u = u0 + k * tile;

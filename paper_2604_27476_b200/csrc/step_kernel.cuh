@@ -228,8 +228,13 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         const int batch_log2 = paired ? RB_LOG2 - 1 : RB_LOG2, per_batch = 1 << batch_log2;
         float sq = 0.f;                               // residual operators: this lane's share of the next norm's sum of squares
 #pragma unroll 1
-        for (int ub = u0; ub == u0 || ub < u1; ub += per_batch) {
-            const int ue = min(u1, ub + per_batch);
+        for (int ub = u0, ue = u0, more = 1; more; ub = ue, more = ub < u1) {       // (once if the CTA owns nothing)
+            ue = u1;                                   // a batch is whole tiles
+            if (u1 - ub > per_batch) {
+                ue = ub;
+#pragma unroll 1
+                for (int n; (n = tile_units(p, op, ue, u1)) <= per_batch - (ue - ub) && ue < u1;) ue += n;
+            }
             // thread -> (token, unit): residual operators take a warp per token, lanes over rows
             const int tok = resid ? c.warp : c.tid >> batch_log2, j = ub + (resid ? c.lane : c.tid & (per_batch - 1));
             const bool mine = tok < MT && j < ue;

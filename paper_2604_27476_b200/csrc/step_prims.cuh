@@ -247,7 +247,7 @@ __device__ __forceinline__ int op_units(const StepParams &p, int op, int lm_rows
 __device__ __forceinline__ bool op_paired(int op) { return op == ST_QKV || op == ST_GU; }
 // Units of the tile that starts at unit u of [.., u1).
 __device__ __forceinline__ int tile_units(const StepParams &p, int op, int u, int u1) {
-    int n = min(op_paired(op) ? ST_TILE / 2 : ST_TILE, u1 - u);
+    int n = min(p.cols[op].tile, u1 - u);
     if (op == ST_QKV) n = min(n, (1 << p.half_shift) - (u & ((1 << p.half_shift) - 1)));   // rows of one head are contiguous, heads are not
     return n;
 }

@@ -202,11 +202,13 @@ template <int SETS> struct Acc {       // row sums of a tile: two independent ch
     }
 };
 // A block (64 columns) of a chunk at offset `off`: rows ra / rb (this lane's), `last` = offset of the last 16 bytes of a row.
-template <int SETS>
+// HALF: there is no row rb (the lower half of the MMA is zero).
+template <int SETS, bool HALF = false>
 __device__ __forceinline__ void block_mma(Acc<SETS> &acc, const unsigned char *ra, const unsigned char *rb, int off, bool odd, int last, const uint4 (&b0)[SETS], const uint4 (&b1)[SETS]) {
     const int o0 = min(off + (odd ? 64 : 0), last), o1 = min(off + (odd ? 0 : 64), last);    // (past the row: the vector is zero there)
-    const uint4 p0 = *reinterpret_cast<const uint4 *>(ra + o0), q0 = *reinterpret_cast<const uint4 *>(rb + o0);
-    const uint4 p1 = *reinterpret_cast<const uint4 *>(ra + o1), q1 = *reinterpret_cast<const uint4 *>(rb + o1);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const uint4 p0 = *reinterpret_cast<const uint4 *>(ra + o0), q0 = HALF ? zero : *reinterpret_cast<const uint4 *>(rb + o0);
+    const uint4 p1 = *reinterpret_cast<const uint4 *>(ra + o1), q1 = HALF ? zero : *reinterpret_cast<const uint4 *>(rb + o1);
     const uint4 a = pick(odd, p0, p1), b = pick(odd, q0, q1), e = pick(odd, p1, p0), f = pick(odd, q1, q0);
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
@@ -216,11 +218,10 @@ __device__ __forceinline__ void block_mma(Acc<SETS> &acc, const unsigned char *r
         mma(acc.d[s][1], e.z, f.z, e.w, f.w, b1[s].z, b1[s].w);
     }
 }
-// The row sums of a finished tile to part[token][row][warp]; row r of the tile (MMA rows 0..7) is row `first` + r of the batch, MMA rows
-// 8..15 are `second` + 0..7.
+// The row sums of a finished tile to part[token][row][warp]; this lane's two MMA rows are rows ra and rb of the batch (-1: none).
 template <int MT, int SETS>
-__device__ __forceinline__ void flush(const Ctx<MT> &c, Acc<SETS> &acc, float *part, int first, int n_first, int second, int n_second) {
-    const int g = c.lane >> 2, t = c.lane & 3;
+__device__ __forceinline__ void flush(const Ctx<MT> &c, Acc<SETS> &acc, float *part, int ra, int rb) {
+    const int t = c.lane & 3;
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
         float d[4];
@@ -229,23 +230,23 @@ __device__ __forceinline__ void flush(const Ctx<MT> &c, Acc<SETS> &acc, float *p
         if constexpr (Ctx<MT>::S == 2) {                  // columns 2 t, 2 t + 1 are the pieces of token 4 s + t
             float *at = part + (4 * s + t) * Ctx<MT>::RB * ST_NW + c.warp;
             if (4 * s + t < MT) {
-                if (g < n_first) at[(first + g) * ST_NW] = d[0] + d[1];
-                if (g < n_second) at[(second + g) * ST_NW] = d[2] + d[3];
+                if (ra >= 0) at[ra * ST_NW] = d[0] + d[1];
+                if (rb >= 0) at[rb * ST_NW] = d[2] + d[3];
             }
         } else {                                          // token 0: columns 0, 1, 2; token 1: columns 3, 4, 5
             const float n0 = __shfl_down_sync(0xffffffffu, d[0], 1), n2 = __shfl_down_sync(0xffffffffu, d[2], 1);
             float *at = part + c.warp;
             if (t == 0) {
-                if (g < n_first) at[(first + g) * ST_NW] = d[0] + d[1] + n0;
-                if (g < n_second) at[(second + g) * ST_NW] = d[2] + d[3] + n2;
+                if (ra >= 0) at[ra * ST_NW] = d[0] + d[1] + n0;
+                if (rb >= 0) at[rb * ST_NW] = d[2] + d[3] + n2;
             }
             if constexpr (MT == 2) {
                 const float m0 = __shfl_down_sync(0xffffffffu, d[1], 1), m2 = __shfl_down_sync(0xffffffffu, d[3], 1);
                 const float k0 = __shfl_down_sync(0xffffffffu, d[0] + d[1], 2), k2 = __shfl_down_sync(0xffffffffu, d[2] + d[3], 2);
                 at += Ctx<MT>::RB * ST_NW;
                 if (t == 0) {
-                    if (g < n_first) at[(first + g) * ST_NW] = m0 + k0;
-                    if (g < n_second) at[(second + g) * ST_NW] = m2 + k2;
+                    if (ra >= 0) at[ra * ST_NW] = m0 + k0;
+                    if (rb >= 0) at[rb * ST_NW] = m2 + k2;
                 }
             }
         }
@@ -265,11 +266,13 @@ __device__ __forceinline__ Rows rows_of(const unsigned char *at, int g, int na, 
 
 struct Slice { int u, u1, op, batch; };      // units [u, u1) of an operator; the batch of partial sums they go to
 
-// KEEP > 0: rows are whole in a chunk and a warp's blocks of the vector (at most KEEP) stay in registers for all tiles.
+// KEEP > 0: rows are whole in a chunk and a warp's blocks of the vector (at most KEEP) stay in registers for all tiles; more than
+// ST_KEEP: tiles of 8 rows in all, the upper half of the MMA.
 // KEEP == 0: tiles cut by columns, the vector is read again for every tile (the MLP activations come by segments themselves).
 template <int KEEP, int MT>
 __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
     constexpr int SETS = (Ctx<MT>::NA + 7) / 8;
+    constexpr bool HALF = KEEP > ST_KEEP;
     const StepParams &p = c.p();
     const int K = p.cols[sl.op].K, seg = p.cols[sl.op].seg;
     float *const part = c.sh().part[sl.batch & 1];
@@ -303,10 +306,11 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
             const unsigned char *at;
             if (!chunk_wait(c, at)) return false;
             const int rb = K * 2;
-            const unsigned char *ra = at + min(g, na - 1) * rb + t16 + first_all * 128, *rc = at + min(na + g, na + nb - 1) * rb + t16 + first_all * 128;
+            const unsigned char *ra = at + min(g, (HALF ? na + nb : na) - 1) * rb + t16 + first_all * 128, *rc = at + min(na + g, na + nb - 1) * rb + t16 + first_all * 128;
             const int last = rb - 16 - t16 - first_all * 128;
 #pragma unroll
-            for (int i = 0; i < NK; ++i) block_mma<SETS>(acc, ra, rc, i * 128, odd, last, k0[i], k1[i]);
+            for (int i = 0; i < NK; ++i)
+                if (!HALF || i < mine_all) block_mma<SETS, HALF>(acc, ra, rc, i * 128, odd, last, k0[i], k1[i]);
             chunk_release(c);
         } else {
 #pragma unroll 1
@@ -336,8 +340,9 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
                 }
             }
         }
-        const int done = u - sl.u;
-        flush<MT, SETS>(c, acc, part, done, na, paired ? Ctx<MT>::RB / 2 + done : done + 8, nb);
+        const int done = u - sl.u, second = paired ? Ctx<MT>::RB / 2 + done : done + 8;
+        if constexpr (HALF) flush<MT, SETS>(c, acc, part, g < na ? done + g : g < na + nb ? second + g - na : -1, -1);
+        else flush<MT, SETS>(c, acc, part, g < na ? done + g : -1, g < nb ? second + g : -1);
         acc.clear();
         u += n;
     }
@@ -347,7 +352,10 @@ __device__ __forceinline__ bool multiply(Ctx<MT> &c, const Slice &sl) {
 template <int MT> __device__ __forceinline__ bool multiply_any(Ctx<MT> &c, const Slice &sl) {
     const StepCols &cols = c.p().cols[sl.op];
     if (cols.segs > 1 || sl.op == ST_DN) return multiply<0, MT>(c, sl);
-    switch (((cols.K + 63) / 64 + ST_NW - 1) / ST_NW) {
+    const int most = ((cols.K + 63) / 64 + ST_NW - 1) / ST_NW;
+    if constexpr (Ctx<MT>::NA <= 8)          // (with two sets of B columns the vector does not fit the registers)
+        if (most > ST_KEEP && most <= ST_KEEP_HALF && cols.tile == (op_paired(sl.op) ? ST_TILE / 4 : ST_TILE / 2)) return multiply<ST_KEEP_HALF, MT>(c, sl);
+    switch (most) {
         case 1: return multiply<1, MT>(c, sl);
         case 2: return multiply<2, MT>(c, sl);
         case 3: return multiply<3, MT>(c, sl);

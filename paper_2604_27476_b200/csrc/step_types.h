@@ -24,7 +24,8 @@ constexpr int ST_TILE = 16;                  // rows of a tile: the M of one m16
 __host__ __device__ constexpr int kv_block(int D) { return 16 * ST_NW / (D / 64); }
 constexpr int ST_MIN_CHUNK = 16;             // fewest cached positions a CTA attends to (shorter contexts occupy fewer CTAs)
 constexpr int ST_PREFETCH_BYTES = 352 * 1024;   // L2 look-ahead per CTA beyond the ring
-constexpr int ST_KEEP = 4;                   // 64-column blocks of the input vector a warp can keep in registers
+constexpr int ST_KEEP = 4;                   // 64-column blocks of the input vector a warp can keep in registers with tiles of 16 rows ...
+constexpr int ST_KEEP_HALF = 8;              // ... and of 8
 
 // Tokens a call may carry (a build of the kernel each): 1, 2, 4 or 8.  bf16 pieces an activation value is multiplied as: three (24 mantissa
 // bits) for one or two tokens, two (16 bits, twice the precision of the weights) for more; the pieces of all tokens are columns
@@ -38,15 +39,17 @@ __host__ __device__ constexpr int st_batch(int mt) { return mt <= 2 ? 128 : mt =
 
 enum { ST_QKV = 0, ST_O = 1, ST_GU = 2, ST_DN = 3, ST_LM = 4 };
 
-// How an operator with rows of K values is cut: tiles of 16 rows (8 pairs); a tile whose rows are too long for a ring chunk is cut into
-// `segs` segments of `seg` columns.  All warps work on every chunk: warp w multiplies the 64-column blocks [nb w / 8, nb (w + 1) / 8) of
+// How an operator with rows of K values is cut: tiles of 16 rows (8 pairs), or of 8 rows (4 pairs) where 16 whole ones are too long for a
+// ring chunk (half of the MMA idles, but chunks stay contiguous and the input vector in registers: K = 3584, gate/up 5.9 TB/s by
+// segments and 6.6 so); a tile whose rows are longer still is cut into `segs` segments of `seg` columns.  All warps work on every chunk: warp w multiplies the 64-column blocks [nb w / 8, nb (w + 1) / 8) of
 // the nb blocks of the chunk, and so needs only that part of the input vector.
-// A segment comes as one box (two for pairs) of a tensor map: box_rows rows (8 or 16, or the most a CTA owns; what lies past the tile
-// is not used) x seg columns, delivered as [64-column block][row][128 bytes].  (One bulk copy per row segment costs the copy unit about
+// A segment comes as one box (two for pairs) of a tensor map: box_rows rows (what lies past the tile is fetched and not used, so a
+// CTA's rows are dealt out evenly to its tiles: 25 rows as 13 + 12, not 16 + 9) x seg columns, delivered as [64-column block][row][128 bytes].  (One bulk copy per row segment costs the copy unit about
 // 150 cycles whatever its size: 11 rows of 4 KB took 2.6 TB/s, as a box they come at the rate of whole rows.)  box_rows 0: K is not a
 // multiple of 64, one copy per row segment.
 struct StepCols {
     int K, seg, segs, box_rows;
+    int tile;            // units (rows or pairs) of a tile
 };
 
 // Pointers of a layer; entry [n_layers] describes the output layer.
@@ -116,15 +119,21 @@ StepKernel step_kernel_for(int D, int G, bool kv8, int mt);
 __host__ __device__ inline int st_first(int n, int c, int ncta) { return static_cast<int>(static_cast<unsigned>(n) * static_cast<unsigned>(c) / static_cast<unsigned>(ncta)); }
 __host__ __device__ inline int st_line(int most) { return (most + 15) / 16 * 16; }   // packets of a line: whole 128 bytes
 
-// How an operator with rows of K values and at most `rows` of them in a tile is cut.
-inline StepCols step_cols(int K, int rows, bool paired, int max_seg = 1 << 30) {
-    StepCols c{K, K, 1, 0};
-    if (rows * K * 2 <= ST_CHUNK_WHOLE && K <= max_seg) return c;
-    const int most = std::min(max_seg, std::max(512, ST_CHUNK_BYTES / (2 * rows) / 512 * 512));
-    const int n = (K + most - 1) / most;
-    c.seg = std::min(most, ((K + n - 1) / n + 511) / 512 * 512);      // a whole number of blocks for every warp
+// How an operator with rows of K values is cut of which a CTA owns at most `most` units (rows, or pairs).
+inline StepCols step_cols(int K, int most, bool paired, int max_seg = 1 << 30) {
+    const int full = paired ? ST_TILE / 2 : ST_TILE, per_unit = paired ? 4 * K : 2 * K;     // bytes
+    StepCols c{K, K, 1, 0, full};
+    if (K <= max_seg && std::min(most, full) * per_unit <= ST_CHUNK_WHOLE) return c;
+    c.tile = full / 2;
+    if (K <= max_seg && c.tile * per_unit <= ST_CHUNK_WHOLE && K <= ST_KEEP_HALF * ST_NW * 64) return c;
+    const int tiles = (most + full - 1) / full;
+    c.tile = (most + tiles - 1) / tiles;
+    const int rows = paired ? 2 * c.tile : c.tile;
+    const int cols = std::min(max_seg, std::max(512, ST_CHUNK_BYTES / (2 * rows) / 512 * 512));
+    const int n = (K + cols - 1) / cols;
+    c.seg = std::min(cols, ((K + n - 1) / n + 511) / 512 * 512);      // a whole number of blocks for every warp
     c.segs = (K + c.seg - 1) / c.seg;
-    if (K % 64 == 0) c.box_rows = paired ? rows / 2 : rows;
+    if (K % 64 == 0) c.box_rows = c.tile;
     return c;
 }
 // Bytes between the arrays of a staged vector of n columns: whole 64-column blocks, + 64 so that neighbouring arrays use other banks.
@@ -165,11 +174,12 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.q_scale = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(D)));
     p.max_context = max_context;
     auto most = [&](int n) { return (n + grid - 1) / grid; };
-    const int h_rows = std::min(ST_TILE, most(H));
-    p.cols[ST_QKV] = p.cols[ST_GU] = step_cols(H, ST_TILE, true);
-    p.cols[ST_LM] = step_cols(H, ST_TILE, false);
-    p.cols[ST_O] = step_cols(qd, h_rows, false);
-    p.cols[ST_DN] = step_cols(F, h_rows, false, mt <= 2 ? 2048 : 1024);      // (two segments of activations are in shared memory, as pieces)
+    const int q_most = most((nq + 2 * nkv) * D / 2);
+    p.cols[ST_QKV] = step_cols(H, q_most, true);
+    p.cols[ST_GU] = step_cols(H, most(F), true);
+    p.cols[ST_LM] = step_cols(H, most(sh.vocab), false);
+    p.cols[ST_O] = step_cols(qd, most(H), false);
+    p.cols[ST_DN] = step_cols(F, most(H), false, mt <= 2 ? 2048 : 1024);      // (two segments of activations are in shared memory, as pieces)
     p.q_line = st_line(2 * most((nq + 2 * nkv) * D / 2));
     p.ss_stride = (grid + 3) / 4 * 4;
     p.x_line = st_line(most(H) + 1);
@@ -179,10 +189,8 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     if (st_packets(mt) && (H >= 65536 || qd >= 65536 || grid * p.x_line / 2 >= 16384 || grid * p.ao_line / 2 >= 16384)) return "model shape does not fit the step kernel";
     p.list_at = ((sh.n_layers + 1) * 64 + (st_packets(mt) ? 4 * (total_x + total_a) : 0) + 15) / 16 * 16;
     // the chunk list: tiles of the busiest CTA (QKV tiles are also cut at the ends of head halves) x segments
-    auto tiles = [&](int n, int per) { return (most(n) + per - 1) / per; };
-    const int q_most = most((nq + 2 * nkv) * D / 2);
-    const int chunks_listed = (q_most / 8 + 2 * (q_most / (D / 2) + 2)) * p.cols[ST_QKV].segs + tiles(H, ST_TILE) * (p.cols[ST_O].segs + p.cols[ST_DN].segs) +
-                              tiles(F, ST_TILE / 2) * p.cols[ST_GU].segs + tiles(sh.vocab, ST_TILE) * p.cols[ST_LM].segs;
+    auto listed = [&](int op, int n) { return (most(n) + p.cols[op].tile - 1) / p.cols[op].tile * p.cols[op].segs; };
+    const int chunks_listed = (q_most / p.cols[ST_QKV].tile + 2 * (q_most / (D / 2) + 2)) * p.cols[ST_QKV].segs + listed(ST_O, H) + listed(ST_DN, H) + listed(ST_GU, F) + listed(ST_LM, sh.vocab);
     p.resid_at = p.list_at + 16 * chunks_listed;
     p.table_bytes = (p.resid_at + 4 * mt * most(H) + 127) / 128 * 128;
     // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another
@@ -194,7 +202,8 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     area = std::max(area, p.act_packets ? st_arrays(mt) * st_array_bytes(F) : p.act_slots * slot);
     const int fixed = step_shared_bytes(mt) + p.table_bytes + (area + 127) / 128 * 128;
     int chunk = kv_block(D) * D * (kv8 ? 2 : 4) + 4 * 32;      // (K rows, then V in four quarters 32 bytes apart)
-    for (int o = 0; o < 5; ++o) chunk = std::max(chunk, (o == ST_O || o == ST_DN ? h_rows : ST_TILE) * p.cols[o].seg * 2);
+    const int owned[5] = {q_most, most(H), most(F), most(H), most(sh.vocab)};
+    for (int o = 0; o < 5; ++o) chunk = std::max(chunk, std::min(owned[o], p.cols[o].tile) * (o == ST_QKV || o == ST_GU ? 4 : 2) * p.cols[o].seg);
     sl->max_chunk_bytes = (chunk + 127) / 128 * 128;
     const int ring = (smem_optin - fixed) / 128 * 128;
     if (ring < sl->max_chunk_bytes) return "model shape does not fit the shared memory";

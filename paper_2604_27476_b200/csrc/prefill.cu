@@ -336,22 +336,34 @@ __global__ void __launch_bounds__(256) prefill_head_kernel(const float *x, const
     float bv = -INFINITY;
     int bi = 0x7fffffff;
     const int stride = gridDim.x * 8;
-    for (int row = blockIdx.x * 8 + warp; row < rows; row += 2 * stride) {   // two rows per round: more loads in flight
-        const int row2 = row + stride;
-        const uint16_t *w0 = lm + static_cast<size_t>(row) * H, *w1 = lm + static_cast<size_t>(row2 < rows ? row2 : row) * H;
-        float a0 = 0.f, a1 = 0.f;
-        for (int j = lane * 8; j < H; j += 256) {
-            const uint4 u0 = *reinterpret_cast<const uint4 *>(w0 + j), u1 = *reinterpret_cast<const uint4 *>(w1 + j);
-            const float4 x0 = *reinterpret_cast<const float4 *>(pf_xs + j), x1 = *reinterpret_cast<const float4 *>(pf_xs + j + 4);
-            a0 = dot8(u0, x0, x1, a0);
-            a1 = dot8(u1, x0, x1, a1);
+    // four rows per round, two rounds of columns unrolled: 64 KB of loads in flight per SM (two rows, 16 KB: 2.6 TB/s)
+    constexpr int R = 4;
+    for (int row = blockIdx.x * 8 + warp; row < rows; row += R * stride) {
+        const uint16_t *w[R];
+        float a[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const int r = row + i * stride;
+            w[i] = lm + static_cast<size_t>(r < rows ? r : row) * H;
+            a[i] = 0.f;
         }
-        a0 = warp_sum(a0);
-        a1 = warp_sum(a1);
-        if (lane == 0) {
-            if (logits_out) { logits_out[row] = a0; if (row2 < rows) logits_out[row2] = a1; }
-            if (arg_better(a0, row, bv, bi)) { bv = a0; bi = row; }
-            if (row2 < rows && arg_better(a1, row2, bv, bi)) { bv = a1; bi = row2; }
+#pragma unroll 2
+        for (int j = lane * 8; j < H; j += 256) {
+            uint4 u[R];
+#pragma unroll
+            for (int i = 0; i < R; ++i) u[i] = __ldcs(reinterpret_cast<const uint4 *>(w[i] + j));
+            const float4 x0 = *reinterpret_cast<const float4 *>(pf_xs + j), x1 = *reinterpret_cast<const float4 *>(pf_xs + j + 4);
+#pragma unroll
+            for (int i = 0; i < R; ++i) a[i] = dot8(u[i], x0, x1, a[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const int r = row + i * stride;
+            a[i] = warp_sum(a[i]);
+            if (lane == 0 && r < rows) {
+                if (logits_out) logits_out[r] = a[i];
+                if (arg_better(a[i], r, bv, bi)) { bv = a[i]; bi = r; }
+            }
         }
     }
     if (lane == 0) { bvs[warp] = bv; bis[warp] = bi; }
@@ -500,13 +512,16 @@ constexpr int PF_SPLIT_MAX = 8;               // K splits of a contraction that 
 
 // Tile shapes.  PF_NARROW: 128 output columns, 4 stages of 48 KB.  PF_WIDE: 256 output columns, 3 stages of 64 KB: per k-block
 // 64 KB of operands feed twice the multiplies of a narrow tile's 48 KB, which matters because operand delivery from L2, not
-// the tensor pipe, bounds the narrow tiles.  Gate/up always runs wide: 128 gate columns and their 128 up partners.
+// the tensor pipe, bounds the narrow tiles.  Gate/up runs wide: 128 gate columns and their 128 up partners.
+// Few tokens leave most SMs idle with these tiles, and the pass is a chain of latencies: every CTA pulls its whole K through one SM
+// (77 tokens, 0.5B shape: QKV on 9 CTAs 17 us, O on 7 CTAs 22 us, gate/up on 38 CTAs 23 us).  Where tiles of half the columns still
+// fit the SMs in one round they are taken: PF_SLIM, 64 columns, or PF_NARROW for gate/up, 64 + 64 (use_slim).
 // The kernel is persistent (one CTA per SM, tiles dealt round-robin, neighbours sharing a weight tile) with TWO accumulators
 // in tensor memory, so that the epilogue of a tile runs under the main loop of the next.
-enum { PF_NARROW = 0, PF_WIDE = 2 };
+enum { PF_NARROW = 0, PF_SLIM = 1, PF_WIDE = 2 };
 template <int SHAPE> struct GemmCfg {
-    static constexpr int BN = SHAPE == PF_WIDE ? 256 : 128;
-    static constexpr int STAGES = SHAPE == PF_WIDE ? 3 : 4;
+    static constexpr int BN = SHAPE == PF_WIDE ? 256 : SHAPE == PF_SLIM ? 64 : 128;
+    static constexpr int STAGES = SHAPE == PF_WIDE ? 3 : SHAPE == PF_SLIM ? 5 : 4;
     static constexpr int A_BYTES = PF_BM * PF_BK * 2, B_BYTES = BN * PF_BK * 2;
     static constexpr int STAGE_BYTES = 2 * A_BYTES + B_BYTES;          // A hi, A lo, B
     static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;   // + room to align the first stage to 1024 bytes
@@ -518,8 +533,8 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
                                                            const __grid_constant__ CUtensorMap map_b, const GemmArgs g) {
     pdl_trigger();
     using C = GemmCfg<SHAPE>;
-    static_assert(EPI != EPI_SWIGLU || SHAPE == PF_WIDE, "gate and up share one accumulator");
-    constexpr int N_STEP = EPI == EPI_SWIGLU ? 128 : C::BN;   // output columns (of g.N) a CTA covers
+    static_assert(EPI != EPI_SWIGLU || SHAPE != PF_SLIM, "gate and up share one accumulator");
+    constexpr int N_STEP = EPI == EPI_SWIGLU ? C::BN / 2 : C::BN;   // output columns (of g.N) a CTA covers
     extern __shared__ uint8_t pf_dyn[];
     __shared__ uint64_t full_bar[C::STAGES], empty_bar[C::STAGES], acc_full[2], acc_empty[2], drain_bar;
     __shared__ uint32_t tmem_slot;
@@ -572,7 +587,8 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
             tma_load_2d(a, &map_a_hi, kb * PF_BK, m0, &full_bar[s]);
             tma_load_2d(a + C::A_BYTES, &map_a_lo, kb * PF_BK, m0, &full_bar[s]);
             tma_load_2d(b, &map_b, kb * PF_BK, n0, &full_bar[s]);
-            if (C::BN == 256) tma_load_2d(b + 128 * PF_BK * 2, &map_b, kb * PF_BK, (EPI == EPI_SWIGLU ? g.N : 128) + n0, &full_bar[s]);
+            if (EPI == EPI_SWIGLU) tma_load_2d(b + N_STEP * PF_BK * 2, &map_b, kb * PF_BK, g.N + n0, &full_bar[s]);
+            else if (C::BN == 256) tma_load_2d(b + 128 * PF_BK * 2, &map_b, kb * PF_BK, 128 + n0, &full_bar[s]);
             issued = it + 1;
           }
         }
@@ -662,12 +678,12 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
                     }
                 }
             } else if (EPI == EPI_SWIGLU) {
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < N_STEP / 32; ++c) {
                     const int n = n0 + c * 32;
                     if (n >= g.N) break;
                     float gt[32], up[32];
                     tmem_ld32(trow + c * 32, gt);
-                    tmem_ld32(trow + 128 + c * 32, up);
+                    tmem_ld32(trow + N_STEP + c * 32, up);
                     tmem_ld_wait();
                     if (live) {
                         uint4 *p = reinterpret_cast<uint4 *>(g.act + static_cast<size_t>(row) * g.N + n);
@@ -1305,7 +1321,7 @@ const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const 
     using C = GemmCfg<SHAPE>;
     if (cudaFuncSetAttribute(prefill_gemm_kernel<EPI, SHAPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
         return "cudaFuncSetAttribute failed";
-    const int n_step = EPI == EPI_SWIGLU ? 128 : C::BN;
+    const int n_step = EPI == EPI_SWIGLU ? C::BN / 2 : C::BN;
     const int units = ((g.N + n_step - 1) / n_step) * ((g.M + PF_BM - 1) / PF_BM) * (EPI == EPI_RESID ? g.splits : 1);
     launch_pdl(prefill_gemm_kernel<EPI, SHAPE>, dim3(units < num_sms ? units : num_sms), dim3(192), C::SMEM, s, ma, ml, mb, g);
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill GEMM launch failed";
@@ -1317,16 +1333,24 @@ const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const 
 // norm kernel that follows, in a fixed order); a split keeps at least 12 k-blocks per unit and is considered only when the
 // unsplit tiles do not fill the SMs once (with more tiles the partial-sum traffic costs more than the better balance gains:
 // 7B shape, 2048 tokens, 48.0 -> 50.7 ms).
+// Half as many columns per tile where the tiles (and their K splits) still fit the SMs in one round; a QKV tile is whole heads.
+bool use_slim(int epilogue, int M, int N, int d, int splits, int num_sms) {
+    if (epilogue == EPI_LOGITS || (epilogue == EPI_QKV && d != 64)) return false;
+    return ((N + 63) / 64) * ((M + PF_BM - 1) / PF_BM) * splits <= num_sms;
+}
 template <int EPI>
 const char *launch_gemm(const uint16_t *a, size_t a_plane, const void *w, long long w_rows, GemmArgs &g, int num_sms, cudaStream_t s) {
     CUtensorMap ma, ml, mb;
-    if (!encode_operand_map(&ma, a, g.M, g.K) || !encode_operand_map(&ml, a + a_plane, g.M, g.K) || !encode_operand_map(&mb, w, w_rows, g.K))
-        return "cuTensorMapEncodeTiled failed";
     int wide = 1;
     prefill_plan_contraction(EPI, g.M, g.N, g.K, num_sms, &wide, &g.splits);
+    const bool slim = use_slim(EPI, g.M, g.N, g.d, g.splits, num_sms);
+    if (!encode_operand_map(&ma, a, g.M, g.K) || !encode_operand_map(&ml, a + a_plane, g.M, g.K) || !encode_operand_map(&mb, w, w_rows, g.K, slim ? 64 : 128))
+        return "cuTensorMapEncodeTiled failed";
     if constexpr (EPI == EPI_SWIGLU) {
-        return launch_gemm_cfg<EPI, PF_WIDE>(ma, ml, mb, g, num_sms, s);
+        return slim ? launch_gemm_cfg<EPI, PF_NARROW>(ma, ml, mb, g, num_sms, s) : launch_gemm_cfg<EPI, PF_WIDE>(ma, ml, mb, g, num_sms, s);
     } else {
+        if constexpr (EPI != EPI_LOGITS)
+            if (slim) return launch_gemm_cfg<EPI, PF_SLIM>(ma, ml, mb, g, num_sms, s);
         return wide ? launch_gemm_cfg<EPI, PF_WIDE>(ma, ml, mb, g, num_sms, s) : launch_gemm_cfg<EPI, PF_NARROW>(ma, ml, mb, g, num_sms, s);
     }
 }

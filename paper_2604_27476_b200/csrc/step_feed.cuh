@@ -261,7 +261,7 @@ __device__ __forceinline__ void feed_vectors(Ctx<MT> &c) {
         ++k;
     };
     const int vec = NA * st_array_bytes(p.H) + 4 * MT * p.ss_stride, slot = NA * st_array_bytes(p.cols[ST_DN].seg), segs = p.cols[ST_DN].segs;
-    const int tiles = (sh.u1[ST_DN] - sh.u0[ST_DN] + ST_TILE - 1) / ST_TILE;
+    const int tiles = (sh.u1[ST_DN] - sh.u0[ST_DN] + p.cols[ST_DN].tile - 1) / p.cols[ST_DN].tile;
 #pragma unroll 1
     for (int layer = 0; layer <= p.n_layers && ok; ++layer) {
         if constexpr (!st_packets(MT)) {

@@ -79,6 +79,8 @@ def test_cuts_match_the_oracle(name):
             if m > 1:
                 assert int(pair.ctx.n_accepted.item()) == acc
             assert int(pair.ctx.next_token.item()) == nxt
+            if m > 1:
+                assert pair.ctx.sync_length() == pair.oracle.cur_len
             tok, pos = nxt, pos + acc
     finally:
         pair.close()

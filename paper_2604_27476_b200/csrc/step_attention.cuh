@@ -352,7 +352,8 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
     const StepParams &p = c.p();
     const int n_chunks = c.sh().n_chunks, m = c.sh().m;
     const int pairs = p.qd / 2, a0 = st_first(pairs, c.cta, c.ncta), n_pairs = st_first(pairs, c.cta + 1, c.ncta) - a0;
-    const int lp = MT == 1 || n_chunks > 16 ? 32 : n_chunks > 8 ? 16 : 8, sub = c.lane & (lp - 1), per_warp = 32 / lp;
+    // (several tokens: as few lanes as hold the chunks, so that all outputs are merged in one round)
+    const int lp = MT == 1 || n_chunks > 16 * NJ ? 32 : n_chunks > 8 * NJ ? 16 : 8, sub = c.lane & (lp - 1), per_warp = 32 / lp;
     bool ok = true;
 #pragma unroll 1
     for (int it = c.warp * per_warp; it < n_pairs * m && ok; it += ST_NW * per_warp) {

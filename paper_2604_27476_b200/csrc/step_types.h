@@ -18,12 +18,14 @@ constexpr int ST_REGS_LAUNCH = 168, ST_REGS = 208, ST_REGS_FEED = 88;
 static_assert(ST_NT * ST_REGS + 128 * ST_REGS_FEED <= ST_THREADS * ST_REGS_LAUNCH, "setmaxnreg only redistributes the launch's registers");
 constexpr int ST_BARS = 16;                  // chunks the ring can hold at once (a power of two)
 constexpr int ST_CHUNK_BYTES = 52 * 1024;    // aimed at for a ring chunk cut by columns
+constexpr int ST_CHUNK_SMALL = 28 * 1024;    // ... where a segment needs no exchange of its own: the ring refills in finer steps (1.5B shape, 8960 columns: 6.0 -> 5.5 us)
+constexpr int ST_ACT_WHOLE = 72 * 1024;      // MLP activations up to this size are staged whole
 constexpr int ST_CHUNK_WHOLE = 68 * 1024;    // a tile of whole rows may be this large
 constexpr int ST_TILE = 16;                  // rows of a tile: the M of one m16n8k16 tensor-core instruction (pairs: 8 and their partners)
 // cached positions per ring chunk: a warp multiplies 16 of them by 64 dims
 __host__ __device__ constexpr int kv_block(int D) { return 16 * ST_NW / (D / 64); }
 constexpr int ST_MIN_CHUNK = 16;             // fewest cached positions a CTA attends to (shorter contexts occupy fewer CTAs)
-constexpr int ST_PREFETCH_BYTES = 352 * 1024;   // L2 look-ahead per CTA beyond the ring
+constexpr int ST_PREFETCH_BYTES = 256 * 1024;   // L2 look-ahead per CTA beyond the ring (160 KB: 1.5B shape + 1 %; 352 KB: 7B shape + 1 %)
 constexpr int ST_KEEP = 4;                   // 64-column blocks of the input vector a warp can keep in registers with tiles of 16 rows ...
 constexpr int ST_KEEP_HALF = 8;              // ... and of 8
 
@@ -120,7 +122,7 @@ __host__ __device__ inline int st_first(int n, int c, int ncta) { return static_
 __host__ __device__ inline int st_line(int most) { return (most + 15) / 16 * 16; }   // packets of a line: whole 128 bytes
 
 // How an operator with rows of K values is cut of which a CTA owns at most `most` units (rows, or pairs).
-inline StepCols step_cols(int K, int most, bool paired, int max_seg = 1 << 30) {
+inline StepCols step_cols(int K, int most, bool paired, int max_seg = 1 << 30, int chunk_bytes = ST_CHUNK_BYTES) {
     const int full = paired ? ST_TILE / 2 : ST_TILE, per_unit = paired ? 4 * K : 2 * K;     // bytes
     StepCols c{K, K, 1, 0, full};
     if (K <= max_seg && std::min(most, full) * per_unit <= ST_CHUNK_WHOLE) return c;
@@ -129,7 +131,7 @@ inline StepCols step_cols(int K, int most, bool paired, int max_seg = 1 << 30) {
     const int tiles = (most + full - 1) / full;
     c.tile = (most + tiles - 1) / tiles;
     const int rows = paired ? 2 * c.tile : c.tile;
-    const int cols = std::min(max_seg, std::max(512, ST_CHUNK_BYTES / (2 * rows) / 512 * 512));
+    const int cols = std::min(max_seg, std::max(512, chunk_bytes / (2 * rows) / 512 * 512));
     const int n = (K + cols - 1) / cols;
     c.seg = std::min(cols, ((K + n - 1) / n + 511) / 512 * 512);      // a whole number of blocks for every warp
     c.segs = (K + c.seg - 1) / c.seg;
@@ -179,7 +181,10 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.cols[ST_GU] = step_cols(H, most(F), true);
     p.cols[ST_LM] = step_cols(H, most(sh.vocab), false);
     p.cols[ST_O] = step_cols(qd, most(H), false);
-    p.cols[ST_DN] = step_cols(F, most(H), false, mt <= 2 ? 2048 : 1024);      // (two segments of activations are in shared memory, as pieces)
+    // the activations whole if they leave the ring room to cover the latency of HBM (7B: 113 KB for them, and the stream fell to 3.9 TB/s)
+    p.act_packets = st_packets(mt) && st_arrays(mt) * st_array_bytes(F) <= ST_ACT_WHOLE;
+    p.cols[ST_DN] = step_cols(F, most(H), false, mt <= 2 ? 2048 : 1024,       // (two segments of activations are in shared memory, as pieces)
+                              p.act_packets ? ST_CHUNK_SMALL : ST_CHUNK_BYTES);
     p.q_line = st_line(2 * most((nq + 2 * nkv) * D / 2));
     p.ss_stride = (grid + 3) / 4 * 4;
     p.x_line = st_line(most(H) + 1);
@@ -196,9 +201,7 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another
     const int slot = st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg), vec = std::max(st_arrays(mt) * st_array_bytes(H) + 4 * mt * p.ss_stride, st_arrays(mt) * st_array_bytes(qd));
     int area = std::max(vec, 4 * step_scratch_floats(D, G, mt));
-    // the activations whole if they leave the ring room to cover the latency of HBM (7B: 113 KB for them, and the stream fell to 3.9 TB/s)
-    p.act_packets = st_packets(mt) && st_arrays(mt) * st_array_bytes(F) <= 64 * 1024;
-    p.act_slots = p.cols[ST_DN].segs == 1 ? 1 : std::max(2, std::min(3, area / slot));
+    p.act_slots = p.cols[ST_DN].segs == 1 ? 1 : std::max(mt == 4 ? 3 : 2, std::min(3, area / slot));     // (every slot is taken from the ring)
     area = std::max(area, p.act_packets ? st_arrays(mt) * st_array_bytes(F) : p.act_slots * slot);
     const int fixed = step_shared_bytes(mt) + p.table_bytes + (area + 127) / 128 * 128;
     int chunk = kv_block(D) * D * (kv8 ? 2 : 4) + 4 * 32;      // (K rows, then V in four quarters 32 bytes apart)

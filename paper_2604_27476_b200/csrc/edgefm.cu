@@ -1,4 +1,4 @@
-// C ABI of the batch-1 decode step (see include/edgefm.h) and the assembly of the step as a CUDA graph.
+// C ABI of the batch-1 decode step (see include/edgefm.h) and the launches of the step kernel.
 #include "../../include/edgefm.h"
 
 #include <algorithm>
@@ -141,7 +141,6 @@ struct edgefm_ctx {
     float *k_scale = nullptr, *v_scale = nullptr;     // compressed cache: [L][nkv][max_context]
     double *inv_freq = nullptr;  // [d/2]
     StepState *state = nullptr;
-    StepRequest *req = nullptr;
     unsigned long long *prof = nullptr;
     int prof_stride = 0;
 
@@ -150,8 +149,7 @@ struct edgefm_ctx {
         StepLaunch launch;
         unsigned long long *ll = nullptr;     // exchange buffers
         unsigned char *maps = nullptr;        // tensor maps of the operators cut into boxes
-        cudaGraph_t graph = nullptr;
-        cudaGraphExec_t exec = nullptr;
+        bool made = false;
     } step, wide;
     bool wide_refused = false;
     StepLayer *d_layers = nullptr;        // [n_layers + 1]
@@ -160,7 +158,7 @@ struct edgefm_ctx {
     uint16_t *sub_lm = nullptr;     // [vocab_subset][hidden] or null
     int vocab_subset = 0;           // 0 = full vocabulary
 
-    cudaStream_t build_stream = nullptr;
+    StepState *host_state = nullptr;      // pinned: edgefm_sync_length reads the device's state with one wait
     int launches_per_step = 0;
     PrefillBuffers pf;           // work buffers of edgefm_prefill, allocated at its first call
     int prefill_launches = 0;    // kernels the last edgefm_prefill enqueued
@@ -173,8 +171,6 @@ struct edgefm_ctx {
     int cur_len = 0;
     bool have_token = false;
     bool len_exact = true;       // false between a verified block (the device decides how far the cache grows) and edgefm_sync_length
-    bool req_valid = false;
-    StepRequest last_req{};
     std::string err;
 };
 
@@ -216,13 +212,11 @@ cudaError_t dev_alloc(T **p, size_t count) {
 
 void free_all(edgefm_ctx *c) {
     for (edgefm_ctx::Build *b : {&c->step, &c->wide}) {
-        if (b->exec) cudaGraphExecDestroy(b->exec);
-        if (b->graph) cudaGraphDestroy(b->graph);
         if (b->ll) cudaFree(b->ll);
         if (b->maps) cudaFree(b->maps);
     }
-    if (c->build_stream) cudaStreamDestroy(c->build_stream);
-    void *bufs[] = {c->k_cache, c->v_cache, c->inv_freq, c->state, c->req, c->prof, c->vocab_ids, c->sub_lm, c->k_scale, c->v_scale, c->d_layers};
+    if (c->host_state) cudaFreeHost(c->host_state);
+    void *bufs[] = {c->k_cache, c->v_cache, c->inv_freq, c->state, c->prof, c->vocab_ids, c->sub_lm, c->k_scale, c->v_scale, c->d_layers};
     for (void *b : bufs) if (b) cudaFree(b);
     if (c->pf.chunk) prefill_free(&c->pf);
 }
@@ -232,7 +226,7 @@ PrefillModel prefill_model(edgefm_ctx *ctx);
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// One cooperative launch of the step kernel: all CTAs are co-resident, which the grid barriers rely on.
+// One cooperative launch of the step kernel: all CTAs are co-resident, which the exchanges rely on.
 cudaError_t launch_step(const StepLaunch &sl, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(sl.grid);
@@ -247,21 +241,13 @@ cudaError_t launch_step(const StepLaunch &sl, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, sl.kernel, sl.p);
 }
 
-// Record the step once; every decode step replays this graph (one kernel node).
-cudaError_t record_graph(edgefm_ctx *c, edgefm_ctx::Build *b) {
-    if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
-    if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
-    cudaError_t e = cudaStreamBeginCapture(c->build_stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return e;
-    const cudaError_t le = launch_step(b->launch, c->build_stream);
-    e = cudaStreamEndCapture(c->build_stream, &b->graph);
-    if (le != cudaSuccess) return le;
-    if (e != cudaSuccess) return e;
-    c->launches_per_step = 1;
-    return cudaGraphInstantiate(&b->exec, b->graph, 0);
+// A step of a build: the request travels with the launch.
+cudaError_t run_step(edgefm_ctx::Build *b, const StepRequest &r, cudaStream_t s) {
+    b->launch.p.req = r;
+    return launch_step(b->launch, s);
 }
 
-// Plan, buffers and graph of the build for `mt` tokens per call.  *why: the shape does not fit.
+// Plan and buffers of the build for `mt` tokens per call.  *why: the shape does not fit.
 cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char **why) {
     int smem_optin = 0, per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
@@ -285,13 +271,15 @@ cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char *
     }
     p.k_cache = c->k_cache; p.v_cache = c->v_cache; p.k_scale = c->k_scale; p.v_scale = c->v_scale;
     p.embed = static_cast<const uint16_t *>(c->embed); p.inv_freq = c->inv_freq; p.layers = c->d_layers; p.vocab_ids = c->vocab_ids;
-    p.state = c->state; p.req = c->req; p.prof = c->prof; p.prof_stride = c->prof_stride;
+    p.state = c->state; p.prof = c->prof; p.prof_stride = c->prof_stride;
     p.epoch_slot = b == &c->wide ? 1 : 0;
     p.spin_limit = c->spin_limit; p.barrier_extra = c->barrier_extra;
     if ((e = allow_max_dynamic_smem(sl.kernel, smem_optin)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sl.kernel, ST_THREADS, sl.dyn_smem)) != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidValue;
-    return record_graph(c, b);
+    c->launches_per_step = 1;
+    b->made = true;
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -402,15 +390,13 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
     }
     CREATE_TRY(dev_alloc(&c->inv_freq, d / 2));
     CREATE_TRY(dev_alloc(&c->state, 1));
-    CREATE_TRY(dev_alloc(&c->req, 1));
+    CREATE_TRY(cudaHostAlloc(reinterpret_cast<void **>(&c->host_state), sizeof(StepState), cudaHostAllocDefault));
     CREATE_TRY(cudaMemset(c->k_cache, 0, kv_bytes));
     CREATE_TRY(cudaMemset(c->v_cache, 0, kv_bytes));
     CREATE_TRY(cudaMemset(c->state, 0, sizeof(StepState)));
     CREATE_TRY(dev_alloc(&c->vocab_ids, static_cast<size_t>(sh.vocab)));
     CREATE_TRY(cudaMemset(c->vocab_ids, 0, static_cast<size_t>(sh.vocab) * sizeof(int)));
     {
-        StepRequest r{-1, -1, nullptr, nullptr};
-        CREATE_TRY(cudaMemcpy(c->req, &r, sizeof r, cudaMemcpyHostToDevice));
         std::vector<double> inv(d / 2);
         for (int i = 0; i < d / 2; ++i) inv[i] = std::pow(static_cast<double>(sh.rope_theta), -2.0 * i / d);
         CREATE_TRY(cudaMemcpy(c->inv_freq, inv.data(), inv.size() * sizeof(double), cudaMemcpyHostToDevice));
@@ -428,7 +414,6 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
         CREATE_TRY(dev_alloc(&c->d_layers, layers.size()));
         CREATE_TRY(cudaMemcpy(c->d_layers, layers.data(), layers.size() * sizeof(StepLayer), cudaMemcpyHostToDevice));
     }
-    CREATE_TRY(cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking));
     {
         const char *why = nullptr;
         CREATE_TRY(make_build(c, M, &c->step, &why));
@@ -510,13 +495,7 @@ edgefm_status edgefm_decode_step(edgefm_ctx *ctx, int32_t token_id, int32_t posi
     DeviceGuard guard(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     StepRequest r{token_id, position, logits_out, next_token_out};
-    if (!ctx->req_valid || std::memcmp(&r, &ctx->last_req, sizeof r) != 0) {
-        // small pageable copy: the runtime stages the bytes before returning, so `r` may live on the stack
-        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->req, &r, sizeof r, cudaMemcpyHostToDevice, s));
-        ctx->last_req = r;
-        ctx->req_valid = true;
-    }
-    CUDA_TRY(ctx, cudaGraphLaunch(ctx->step.exec, s));
+    CUDA_TRY(ctx, run_step(&ctx->step, r, s));
     ctx->cur_len += 1;
     ctx->have_token = true;
     ctx->err.clear();
@@ -545,7 +524,7 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     edgefm_ctx::Build *build = &ctx->step;
     if (longer) {
-        if (!ctx->wide.exec && !ctx->wide_refused) {   // made at the first longer block, kept
+        if (!ctx->wide.made && !ctx->wide_refused) {   // made at the first longer block, kept
             const char *why = nullptr;
             CUDA_TRY(ctx, make_build(ctx, PF_VERIFY_MAX, &ctx->wide, &why));
             ctx->wide_refused = why != nullptr;
@@ -579,12 +558,7 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
     r.m = m;
     for (int t = 1; t < m; ++t) r.draft[t - 1] = tokens[t];
     r.n_accepted_out = n_accepted_out;
-    if (!ctx->req_valid || std::memcmp(&r, &ctx->last_req, sizeof r) != 0) {
-        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->req, &r, sizeof r, cudaMemcpyHostToDevice, s));
-        ctx->last_req = r;
-        ctx->req_valid = true;
-    }
-    CUDA_TRY(ctx, cudaGraphLaunch(build->exec, s));
+    CUDA_TRY(ctx, run_step(build, r, s));
     ctx->cur_len += m;     // an upper bound until edgefm_sync_length: the device decides how many tokens are accepted
     if (m > 1) ctx->len_exact = false;
     ctx->have_token = true;
@@ -609,10 +583,7 @@ edgefm_status edgefm_prefill_tokens(edgefm_ctx *ctx, const int32_t *tokens, int3
         r.m = m;
         for (int t = 1; t < m; ++t) r.draft[t - 1] = tokens[i + t];
         r.flags = 1;
-        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->req, &r, sizeof r, cudaMemcpyHostToDevice, s));
-        ctx->last_req = r;
-        ctx->req_valid = true;
-        CUDA_TRY(ctx, cudaGraphLaunch(ctx->step.exec, s));
+        CUDA_TRY(ctx, run_step(&ctx->step, r, s));
         ctx->cur_len += m;
         ctx->have_token = true;
     }
@@ -703,12 +674,12 @@ edgefm_status edgefm_prefill(edgefm_ctx *ctx, const int32_t *tokens, int32_t n, 
 edgefm_status edgefm_sync_length(edgefm_ctx *ctx, void *stream, int32_t *cur_len_host) {
     if (!ctx || !cur_len_host) return EDGEFM_ERR_INVALID_ARG;
     DeviceGuard guard(ctx->device);
-    CUDA_TRY(ctx, cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
-    StepState st{};
-    CUDA_TRY(ctx, cudaMemcpy(&st, ctx->state, sizeof st, cudaMemcpyDeviceToHost));
-    ctx->cur_len = st.cur_len;
+    const cudaStream_t s = static_cast<cudaStream_t>(stream);
+    CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_state, ctx->state, sizeof(StepState), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    ctx->cur_len = ctx->host_state->cur_len;
     ctx->len_exact = true;
-    *cur_len_host = st.cur_len;
+    *cur_len_host = ctx->cur_len;
     return EDGEFM_OK;
 }
 
@@ -759,7 +730,7 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
     CUtensorMap map[2];
     int k = 0;
     for (edgefm_ctx::Build *b : {&ctx->step, &ctx->wide}) {
-        if (!b->exec) continue;
+        if (!b->made) continue;
         if (!step_map(&map[k], b->launch.p.cols[ST_LM], lm_w, head.rows)) e = cudaErrorUnknown;
         if (e == cudaSuccess) e = cudaMemcpyAsync(b->maps + static_cast<size_t>(4 * ctx->shape.n_layers) * sizeof(CUtensorMap), &map[k], sizeof(CUtensorMap), cudaMemcpyHostToDevice, s);
         ++k;
@@ -813,10 +784,9 @@ edgefm_status edgefm_debug_set_wait_limit(edgefm_ctx *ctx, uint32_t limit_ns, in
     ctx->spin_limit = limit_ns;
     ctx->barrier_extra = extra_barrier_arrivals;
     for (edgefm_ctx::Build *b : {&ctx->step, &ctx->wide}) {
-        if (!b->exec) continue;
+        if (!b->made) continue;
         b->launch.p.spin_limit = limit_ns;
         b->launch.p.barrier_extra = extra_barrier_arrivals;
-        CUDA_TRY(ctx, record_graph(ctx, b));
     }
     ctx->err.clear();
     return EDGEFM_OK;
@@ -975,7 +945,6 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     StepLayer *d_layers = sc.take<StepLayer>(static_cast<size_t>(sh.n_layers) + 1);
     double *inv_freq = sc.take<double>(d / 2);
     StepState *state = sc.take<StepState>(1);
-    StepRequest *req = sc.take<StepRequest>(1);
     CUtensorMap *d_maps = sc.take<CUtensorMap>(static_cast<size_t>(4 * sh.n_layers) + 1);
     unsigned long long *ll = sc.take<unsigned long long>(sl.ll_bytes / 8);
     if (sc.off > EDGEFM_STATIC_SCRATCH_BYTES)
@@ -988,7 +957,8 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     StepParams &p = sl.p;
     p.k_cache = static_cast<uint16_t *>(k_cache); p.v_cache = static_cast<uint16_t *>(v_cache);
     p.embed = static_cast<const uint16_t *>(weights->embed); p.inv_freq = inv_freq; p.layers = d_layers;
-    p.state = state; p.req = req;
+    p.state = state;
+    p.req = StepRequest{token_id, position, logits_out, next_token_out};
     p.maps = reinterpret_cast<const unsigned char *>(d_maps);
     p.map_fence = 2;   // every call rewrites all tensor maps in the shared scratch
     std::vector<CUtensorMap> maps(static_cast<size_t>(4 * sh.n_layers) + 1);
@@ -999,7 +969,6 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     for (int i = 0; i < d / 2; ++i) inv[i] = std::pow(static_cast<double>(sh.rope_theta), -2.0 * i / d);
     StepState st{};
     st.cur_len = cur_len; st.next_position = position;
-    StepRequest rq{token_id, position, logits_out, next_token_out};
     // no packet of an earlier call (of any shape) may carry a tag of this one
     CUDA_TRY(nullptr, cudaMemsetAsync(ll, 0, sl.ll_bytes, s));
     // pageable copies: the runtime stages the bytes before returning, so the sources may be freed after the call
@@ -1007,7 +976,6 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     CUDA_TRY(nullptr, cudaMemcpyAsync(d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(inv_freq, inv, static_cast<size_t>(d / 2) * sizeof(double), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(state, &st, sizeof st, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(nullptr, cudaMemcpyAsync(req, &rq, sizeof rq, cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, launch_step(sl, s));
     g_static_state[dev] = state;
     g_create_error.clear();

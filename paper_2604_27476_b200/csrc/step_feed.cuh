@@ -23,8 +23,10 @@ template <int MT> __device__ __forceinline__ uint4 chunk_entry(const Ctx<MT> &c,
     if (cols.box_rows) return make_uint4(row, paired ? partner : ~0u, static_cast<unsigned>(cols.box_rows * cols.seg) * 2u, at16 >> 3 | ST_BOX << 16);
     return make_uint4(row * row16 + at16, paired ? partner * row16 + at16 : ~0u, min(static_cast<unsigned>(cols.seg) >> 3, row16 - at16) * 16u, static_cast<unsigned>(n) << 16);
 }
-// By all threads; published by the caller's sync.
+// By the feeding warpgroup, for itself.
 template <int MT> __device__ __forceinline__ void make_list(const Ctx<MT> &c) {
+    constexpr int THREADS = ST_THREADS - ST_NT;
+    const int tid = c.tid - ST_NT;
     Shared<MT> &sh = c.sh();
     const StepParams &p = c.p();
     // QKV tiles are cut at the ends of head halves, the others are regular
@@ -32,19 +34,20 @@ template <int MT> __device__ __forceinline__ void make_list(const Ctx<MT> &c) {
     for (int u = sh.u0[ST_QKV]; u < sh.u1[ST_QKV];) {
         const int n = tile_units(p, ST_QKV, u, sh.u1[ST_QKV]);
         for (int s = 0; s < p.cols[ST_QKV].segs; ++s, ++at)
-            if (c.tid == at % ST_THREADS) c.list()[at] = chunk_entry(c, ST_QKV, u, n, s);
+            if (tid == at % THREADS) c.list()[at] = chunk_entry(c, ST_QKV, u, n, s);
         u += n;
     }
     for (int op = ST_O; op <= ST_LM; ++op) {
         const int tile = p.cols[op].tile, segs = p.cols[op].segs, u0 = sh.u0[op], u1 = sh.u1[op], count = (u1 - u0 + tile - 1) / tile * segs;
-        if (c.tid == 0) sh.list[op] = at;
-        for (int i = c.tid; i < count; i += ST_THREADS) {
+        if (tid == 0) sh.list[op] = at;
+        for (int i = tid; i < count; i += THREADS) {
             const int k = i / segs, u = u0 + k * tile;
             c.list()[at + i] = chunk_entry(c, op, u, min(tile, u1 - u), i - k * segs);
         }
         at += count;
     }
-    if (c.tid == 0) { sh.list[ST_QKV] = 0; sh.list[5] = at; }
+    if (tid == 0) { sh.list[ST_QKV] = 0; sh.list[5] = at; }
+    asm volatile("barrier.cta.sync 2, %0;" ::"n"(THREADS) : "memory");
 }
 // Calls f(base, entry, map) for the weights and f_kv(k, v, rows, bytes of each) for the cache rows of the whole step in order, until one returns false.
 template <bool Q8, int MT, typename F, typename FKV>

@@ -75,7 +75,7 @@ __device__ __forceinline__ void finish_unit(const Ctx<MT> &c, int op, int layer,
         const int seg = p.cols[ST_DN].seg, s = j / seg, stride = st_array_bytes(seg);
         store_pieces<MT>(p.act_vec + static_cast<size_t>(s) * Ctx<MT>::NA * stride, tok, j - s * seg, stride, v);
     } else if (tok < sh.m) {
-        float *logits = p.req->logits_out;
+        float *logits = p.req.logits_out;
         if (logits) logits[static_cast<size_t>(tok) * c.head().rows + j] = lo;
         if (arg_better(lo, j, best_v, best_i)) { best_v = lo; best_i = j; }
     }
@@ -103,14 +103,15 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.abort = 0;
             sh.sent = 0u;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            const int rt = p.req->token, rp = p.req->position;
-            sh.m = MT > 1 ? min(max(p.req->m, 1), MT) : 1;
-            sh.tokens[0] = rt >= 0 ? rt : p.state->next_token;
-            for (int t = 1; t < MT; ++t) sh.tokens[t] = t < sh.m ? p.req->draft[t - 1] : 0;
-            sh.pos = rp >= 0 ? rp : p.state->next_position;
-            sh.n_old = p.state->cur_len;
+            const int rt = p.req.token, rp = p.req.position, st_token = p.state->next_token, st_pos = p.state->next_position, st_len = p.state->cur_len;
+            const unsigned epoch = static_cast<unsigned>(p.state->epoch[p.epoch_slot]);
+            sh.m = MT > 1 ? min(max(p.req.m, 1), MT) : 1;
+            sh.tokens[0] = rt >= 0 ? rt : st_token;
+            for (int t = 1; t < MT; ++t) sh.tokens[t] = t < sh.m ? p.req.draft[t - 1] : 0;
+            sh.pos = rp >= 0 ? rp : st_pos;
+            sh.n_old = st_len;
             sh.n_chunks = kv_chunks(p, sh.n_old, sh.m, c.ncta);
-            sh.tag0 = static_cast<unsigned>(p.state->epoch[p.epoch_slot]) * static_cast<unsigned>(p.n_layers + 2) + 1u;
+            sh.tag0 = epoch * static_cast<unsigned>(p.n_layers + 2) + 1u;
             sh.odd = static_cast<unsigned>(p.barrier_extra) << 31 | static_cast<unsigned>(p.barrier_extra) << 15;
             sh.total_x = c.ncta * line_units(p.H, c.ncta, 1);
             sh.total_a = c.ncta * line_units(p.qd, c.ncta, 2);
@@ -129,12 +130,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.u0[c.tid] = st_first(n, c.cta, c.ncta);
             sh.u1[c.tid] = st_first(n, c.cta + 1, c.ncta);
         }
-        __syncthreads();
-        make_list(c);
         __syncthreads();                 // the last sync of all threads
     }
     if (c.warp >= ST_NW) {               // the feeding warpgroup: gives its registers to the others
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ST_REGS_FEED));
+        make_list(c);
         if (c.warp == ST_NW && c.lane == 0) feed_ring<Q8, MT>(c);
         if (c.warp == ST_NW + 1 && c.lane == 0) feed_l2<Q8, MT>(c);
         if (c.warp == ST_NW + 2 && c.lane == 0 && !(st_packets(MT) && p.act_packets)) feed_vectors<MT>(c);
@@ -161,7 +161,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
     const int x0 = c.sh().u0[ST_DN], my_rows = c.sh().u1[ST_DN] - x0;      // rows of the residual stream this CTA owns
     {
         Shared<MT> &sh = c.sh();
-        for (int i = c.tid; i < sh.m * half; i += ST_NT) {        // rotary tables of the tokens' positions; fp64 angle, rounded once
+        // warps 0 .. rw - 1 make the rotary tables of the tokens' positions (fp64 angle, rounded once), the others the unit tables
+        const int rw = st_packets(MT) ? MT * half / 32 : ST_NW;
+        for (int i = c.tid; i < sh.m * half && c.warp < rw; i += rw * 32) {
             const int t = i / half, f = i - t * half;
             double sn, cs;
             sincos(static_cast<double>(sh.pos + t) * p.inv_freq[f], &sn, &cs);
@@ -170,18 +172,17 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         }
         if (c.cta == 0 && c.tid == 0) { p.state->token = sh.tokens[0]; p.state->position = sh.pos; }
         if constexpr (st_packets(MT)) {
-            make_table(c, c.unit_table(), p.H, 1, p.x_line);
-            make_table(c, c.unit_table() + sh.total_x, p.qd, 2, p.ao_line);
-        }
-        for (int i = c.tid; i < MT * my_rows; i += ST_NT) {
-            const int t = i / my_rows;
-            c.resid()[i] = bf16_bits_to_f32(p.embed[static_cast<size_t>(sh.tokens[t]) * p.H + x0 + i - t * my_rows]);
+            const int threads = (ST_NW - rw) * 32, first = c.tid - rw * 32;
+            if (first >= 0) {
+                make_table(c, c.unit_table(), p.H, 1, p.x_line, first, threads);
+                make_table(c, c.unit_table() + sh.total_x, p.qd, 2, p.ao_line, first, threads);
+            }
         }
     }
     float best_v = -INFINITY;
     int best_i = 0x7fffffff;
     unsigned batch = 0;
-    bool ok = cta_vote(true);            // tables
+    bool ok = true;
 
 #pragma unroll 1
     for (int ph = 0; ph <= 4 * p.n_layers && ok; ++ph) {
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             stamp(c, prof_idx);                       // partial results merged
         }
         if (op == ST_QKV && layer == 0) {
-            ok = stage_embedding(c, L->input_norm);
+            ok = stage_embedding(c, L->input_norm, x0, my_rows);     // (its vote also publishes the tables)
         } else if (op == ST_DN) {
             c.act_slot = 0;
             if (st_packets(MT) && p.act_packets) ok = stage_activations(c, tag);
@@ -339,11 +340,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         // rejection.  The cache advances by the accepted tokens; the rows of the rejected ones stay behind the cache length and are
         // overwritten by the next call.
         int n_acc = 1;
-        const bool given = MT > 1 && (p.req->flags & 1);   // prompt tokens: nothing to verify
+        const bool given = MT > 1 && (p.req.flags & 1);   // prompt tokens: nothing to verify
         while (n_acc < sh.m && (given || sh.tokens[n_acc] == sh.best_i[n_acc - 1])) ++n_acc;
         const int next = sh.best_i[n_acc - 1];
-        if (p.req->next_token_out) *p.req->next_token_out = next;
-        if (p.req->n_accepted_out) *p.req->n_accepted_out = n_acc;
+        if (p.req.next_token_out) *p.req.next_token_out = next;
+        if (p.req.n_accepted_out) *p.req.n_accepted_out = n_acc;
         StepState *st = p.state;
         st->next_token = next;
         st->next_position = sh.pos + n_acc;

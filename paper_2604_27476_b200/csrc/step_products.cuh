@@ -5,8 +5,10 @@
 namespace edgefm {
 namespace step {
 
-// First operator of the step: the embedding rows are the residual streams.
-template <int MT> __device__ __forceinline__ bool stage_embedding(Ctx<MT> &c, const uint16_t *norm_w) {
+// First operator of the step: the embedding rows are the residual streams; this CTA keeps its rows [x0, x0 + my_rows) of them.
+// (The loads of U columns are under way together: one by one they took a trip to HBM each, 4 us for 1536 columns.)
+template <int MT> __device__ __forceinline__ bool stage_embedding(Ctx<MT> &c, const uint16_t *norm_w, int x0, int my_rows) {
+    constexpr int U = 8;
     const StepParams &p = c.p();
     const int stride = st_array_bytes(p.H), m = c.sh().m;
     zero_tail(c, p.H);
@@ -15,14 +17,29 @@ template <int MT> __device__ __forceinline__ bool stage_embedding(Ctx<MT> &c, co
         const uint16_t *erow = p.embed + static_cast<size_t>(c.sh().tokens[t]) * p.H;
         float ss = 0.f;
 #pragma unroll 1
-        for (int i = c.tid; i < p.H; i += ST_NT) {
-            const float v = bf16_bits_to_f32(erow[i]);
-            ss = fmaf(v, v, ss);
-            store_pieces<MT>(c.area(), t, i, stride, v * bf16_bits_to_f32(norm_w[i]));
+        for (int base = c.tid; base < p.H; base += U * ST_NT) {
+            uint16_t e[U], w[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int j = min(base + i * ST_NT, p.H - 1);
+                e[i] = __ldg(erow + j);
+                w[i] = __ldg(norm_w + j);
+            }
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int j = base + i * ST_NT;
+                if (j >= p.H) break;
+                const float v = bf16_bits_to_f32(e[i]);
+                ss = fmaf(v, v, ss);
+                store_pieces<MT>(c.area(), t, j, stride, v * bf16_bits_to_f32(w[i]));
+                if (j >= x0 && j < x0 + my_rows) c.resid()[t * my_rows + j - x0] = v;
+            }
         }
         ss = warp_sum(ss);
         if (c.lane == 0) c.sh().merged[0][t * ST_NW + c.warp] = ss;      // (not in use yet)
     }
+#pragma unroll 1
+    for (int i = m * my_rows + c.tid; i < MT * my_rows; i += ST_NT) c.resid()[i] = 0.f;      // unused tokens
     if (!cta_vote(true)) return false;
     if (c.tid < m) c.sh().ss[c.tid] = sum8(&c.sh().merged[0][c.tid * ST_NW]);
     return true;
@@ -46,13 +63,16 @@ template <int MT> __device__ __forceinline__ bool stage_vector(Ctx<MT> &c, bool 
 // Table of the 16-byte units of such a vector: row | values << 16 | unit << 18 (unit = index of the packet pair).
 // The tables of the residual stream and of the attention output stand in shared memory, made once per launch.
 __device__ __forceinline__ int line_units(int n, int ncta, int grain) { return ((n / grain + ncta - 1) / ncta * grain + 1) / 2; }
-template <int MT> __device__ __forceinline__ void make_table(const Ctx<MT> &c, unsigned *tab, int n, int grain, int line) {
-    const int upl = line_units(n, c.ncta, grain), total = c.ncta * upl;
+// By `threads` threads, this one the `first`: a line each.
+template <int MT> __device__ __forceinline__ void make_table(const Ctx<MT> &c, unsigned *tab, int n, int grain, int line, int first, int threads) {
+    const int upl = line_units(n, c.ncta, grain);
 #pragma unroll 1
-    for (int i = c.tid; i < total; i += ST_NT) {
-        const int w = i / upl, e = i - w * upl;
-        const int r0 = st_first(n / grain, w, c.ncta) * grain, r1 = st_first(n / grain, w + 1, c.ncta) * grain, row = r0 + 2 * e;
-        tab[i] = static_cast<unsigned>(row & 0xffff) | static_cast<unsigned>(max(0, min(2, r1 - row))) << 16 | static_cast<unsigned>(w * (line >> 1) + e) << 18;
+    for (int w = first; w < c.ncta; w += threads) {
+        int row = st_first(n / grain, w, c.ncta) * grain;
+        const int r1 = st_first(n / grain, w + 1, c.ncta) * grain;
+#pragma unroll 1
+        for (int e = 0; e < upl; ++e, row += 2)
+            tab[w * upl + e] = static_cast<unsigned>(row & 0xffff) | static_cast<unsigned>(max(0, min(2, r1 - row))) << 16 | static_cast<unsigned>(w * (line >> 1) + e) << 18;
     }
 }
 // Wait for all values of the vectors of all tokens (K columns, lines of `line` packets) and leave their pieces in shared memory, and meet.

@@ -82,7 +82,7 @@ struct StepParams {
     int map_fence;                 // maps the host may have rewritten since the last launch: 1 the output layer's, 2 all
     const int *vocab_ids;
     StepState *state;
-    const StepRequest *req;
+    StepRequest req;
     // Vectors that are multiplied next: as they lie in shared memory, arrays of bf16 pieces [token * S + piece][st_array_bytes(K)], zero past
     // K; behind the residual streams' arrays the CTAs' sums of squares [token][ss_stride].  act: [segment][array][st_array_bytes(seg)].
     unsigned char *x_vec;          // residual stream after the down projection, times the next norm's weight

@@ -193,7 +193,8 @@ __device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &sha
     constexpr int q_units = G * half, U = 3;                  // in flight per thread
     const int mine = q_units + n_new * 2 * half;
 #pragma unroll 1
-    for (int j0 = c.tid; j0 < mine; j0 += U * ST_NT) {
+    for (int jb = 0; jb < mine; jb += U * ST_NT) {
+        const int j0 = jb + c.tid;
         Two t[U];
         const unsigned long long *at[U];
         unsigned todo = 0;
@@ -211,16 +212,17 @@ __device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &sha
         }
         const unsigned all = todo;
         Spin sp;
-        while (todo) {
+        int more;
+        do {
 #pragma unroll
             for (int i = 0; i < U; ++i)
                 if (todo >> i & 1u) t[i] = get2(at[i]);
 #pragma unroll
             for (int i = 0; i < U; ++i)
                 if ((todo >> i & 1u) && both(t[i], tag)) todo &= ~(1u << i);
-            if (todo && !sp.again(c.abort(), p.spin_limit)) { ok = false; break; }
-        }
-        if (!ok) break;
+            more = warp_again(sp, todo != 0u, c.abort(), p.spin_limit);
+        } while (more > 0);
+        if (more == 0) { ok = false; break; }
 #pragma unroll
         for (int i = 0; i < U; ++i)
             if (all >> i & 1u) {
@@ -362,15 +364,17 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
         const int tok = on ? item / n_pairs : 0, k_pair = on ? item - tok * n_pairs : 0, pr = a0 + k_pair, h = 2 * pr / p.D;
         float mx = -INFINITY, l = 0.f, a = 0.f, b = 0.f;      // of this lane's chunks
 #pragma unroll 1
-        for (int k0 = sub; k0 < n_chunks && on; k0 += lp * NJ) {
+        for (int kb = 0; kb < n_chunks; kb += lp * NJ) {
+            const int k0 = kb + sub;
             Two st[NJ], ov[NJ];
             unsigned todo = 0;
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
-                if (k0 + lp * j < n_chunks) todo |= 1u << j;
+                if (on && k0 + lp * j < n_chunks) todo |= 1u << j;
             const unsigned mine = todo;
             Spin sp;
-            while (todo) {
+            int more;
+            do {
 #pragma unroll
                 for (int j = 0; j < NJ; ++j)
                     if (todo >> j & 1u) {
@@ -381,14 +385,14 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
 #pragma unroll
                 for (int j = 0; j < NJ; ++j)
                     if ((todo >> j & 1u) && both(st[j], tag) && both(ov[j], tag)) todo &= ~(1u << j);
-                if (todo && !sp.again(c.abort(), p.spin_limit)) break;
-            }
-            if (todo) { ok = false; break; }
+                more = warp_again(sp, todo != 0u, c.abort(), p.spin_limit);
+            } while (more > 0);
+            if (more == 0) { ok = false; break; }
             float mn = mx;
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
                 if (mine >> j & 1u) mn = fmaxf(mn, packet_value(st[j].a));
-            const float f = mx == -INFINITY ? 0.f : exp2_approx(mx - mn);
+            const float f = mx == -INFINITY ? 0.f : exp2_approx(mx - mn);      // (a lane without chunks keeps -inf)
             l *= f; a *= f; b *= f;
             mx = mn;
 #pragma unroll
@@ -400,7 +404,6 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
                     b = fmaf(packet_value(ov[j].b), e, b);
                 }
         }
-        ok = __all_sync(0xffffffffu, ok);
         float mm = mx;
         for (int k = lp >> 1; k; k >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, k));
         const float f = mx == -INFINITY ? 0.f : exp2_approx(mx - mm);

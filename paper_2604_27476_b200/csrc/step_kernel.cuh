@@ -312,14 +312,17 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
     best_v = -INFINITY;
     best_i = 0x7fffffff;
     if (c.warp < sh.m) {                 // warp t: token t
-        for (int i = c.lane; i < c.ncta && ok; i += 32) {
+        for (int base = 0; base < c.ncta && ok; base += 32) {
+            const int i = min(base + c.lane, c.ncta - 1);
             const unsigned long long *at = p.lm_ll + static_cast<size_t>(i) * 16 + 2 * c.warp;
-            Two t = get2(at);
+            Two t;
             Spin sp;
-            while (ok && !both(t, tag)) {
-                ok = sp.again(c.abort(), p.spin_limit);
+            int more;
+            do {
                 t = get2(at);
-            }
+                more = warp_again(sp, !both(t, tag), c.abort(), p.spin_limit);
+            } while (more > 0);
+            if (more == 0) { ok = false; break; }
             const float v = packet_value(t.a);
             const int ix = __float_as_int(packet_value(t.b));
             if (arg_better(v, ix, best_v, best_i)) { best_v = v; best_i = ix; }

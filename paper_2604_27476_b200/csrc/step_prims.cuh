@@ -45,6 +45,13 @@ struct Spin {
         return true;
     }
 };
+// The same for a warp whose lanes poll together: they leave together, too.  (Lanes that leave one by one stay apart for a while, and the
+// shuffles behind the loop then cost microseconds: CTAs that had waited long were 3 - 4 us late at the next exchange.)
+// -1: everything is there, 0: gave up, 1: poll again.
+__device__ __forceinline__ int warp_again(Spin &sp, bool waiting, volatile int *abort_flag, unsigned limit_ns) {
+    if (!__any_sync(0xffffffffu, waiting)) return -1;
+    return __any_sync(0xffffffffu, !sp.again(abort_flag, limit_ns)) ? 0 : 1;
+}
 __device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned parity, volatile int *abort_flag, unsigned limit_ns) {
     if (mbar_try_wait(b, parity)) return true;
     Spin sp;

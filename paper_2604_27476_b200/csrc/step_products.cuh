@@ -94,7 +94,8 @@ __device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int
     if (adds) ask(c.lane);
     zero_tail(c, K);
 #pragma unroll 1
-    for (int base = c.tid; base < all; base += U * ST_NT) {
+    for (int base0 = 0; base0 < all; base0 += U * ST_NT) {
+        const int base = base0 + c.tid;
         unsigned e[U], at[U];
         Two t[U];
         unsigned todo = 0;
@@ -124,24 +125,27 @@ __device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int
                         if (two) store_packet<MT>(c.area(), tok, row + 1, stride, t[i].b);
                     }
                 }
-            if (!todo) break;
-            if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+            const int more = warp_again(sp, todo != 0u, c.abort(), c.p().spin_limit);
+            if (more == 0) ok = false;
+            if (more <= 0) break;
         }
         if (!ok) break;
     }
     if (adds) {
         float ss = 0.f;
 #pragma unroll 1
-        for (int base = c.lane; base < c.ncta && ok; base += 32 * W) {
-            if (base != c.lane) ask(base);
+        for (int base0 = 0; base0 < c.ncta && ok; base0 += 32 * W) {
+            const int base = base0 + c.lane;
+            if (base0 != 0) ask(base);
             Spin sp;
             for (;;) {
                 bool here = true;
 #pragma unroll
                 for (int i = 0; i < W; ++i)
                     if (base + 32 * i < c.ncta) here = here && packet_tag(s[i]) == tag;
-                if (here) break;
-                if (!sp.again(c.abort(), c.p().spin_limit)) { ok = false; break; }
+                const int more = warp_again(sp, !here, c.abort(), c.p().spin_limit);
+                if (more == 0) ok = false;
+                if (more <= 0) break;
                 ask(base);
             }
 #pragma unroll
@@ -162,7 +166,8 @@ template <int MT> __device__ __forceinline__ bool stage_activations(Ctx<MT> &c, 
     bool ok = true;
     zero_tail(c, K);
 #pragma unroll 1
-    for (int base = c.tid; base < all; base += U * ST_NT) {
+    for (int base0 = 0; base0 < all; base0 += U * ST_NT) {
+        const int base = base0 + c.tid;
         Two t[U];
         unsigned todo = 0;
 #pragma unroll
@@ -187,8 +192,9 @@ template <int MT> __device__ __forceinline__ bool stage_activations(Ctx<MT> &c, 
                     for (int q = 0; q < Ctx<MT>::S; ++q)
                         *reinterpret_cast<uint32_t *>(to + q * stride) = (static_cast<uint32_t>(t[i].a >> (16 * q)) & 0xffffu) | static_cast<uint32_t>(t[i].b >> (16 * q)) << 16;
                 }
-            if (!todo) break;
-            if (!sp.again(c.abort(), p.spin_limit)) { ok = false; break; }
+            const int more = warp_again(sp, todo != 0u, c.abort(), p.spin_limit);
+            if (more == 0) ok = false;
+            if (more <= 0) break;
         }
         if (!ok) break;
     }

@@ -94,6 +94,12 @@ __device__ __forceinline__ Two get2(const unsigned long long *at) {
     asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(t.a), "=l"(t.b) : "l"(at) : "memory");
     return t;
 }
+struct Four { unsigned long long a = 0ull, b = 0ull, c = 0ull, d = 0ull; };
+__device__ __forceinline__ Four get4(const unsigned long long *at) {
+    Four t;
+    asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(t.a), "=l"(t.b), "=l"(t.c), "=l"(t.d) : "l"(at) : "memory");
+    return t;
+}
 __device__ __forceinline__ bool both(const Two &t, unsigned tag) { return packet_tag(t.a) == tag && packet_tag(t.b) == tag; }
 
 // Packets of pieces: three bf16 (value = their sum) and the low 16 bits of the tag.  A slot is rewritten with the next tag every layer

@@ -158,39 +158,42 @@ __device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int
     return cta_vote(ok);
 }
 
-// The MLP activations whole (K columns), from packets in natural order.
+// The MLP activations whole (K columns), from packets in natural order, four at a time (32-byte loads; K is a multiple of 8).  All of a
+// round's loads are under way together: with pairs, 8960 columns took two rounds of polls.
 template <int MT> __device__ __forceinline__ bool stage_activations(Ctx<MT> &c, unsigned tag) {
-    constexpr int U = 9;     // packet pairs in flight per thread
+    constexpr int U = 9;     // quads in flight per thread
     const StepParams &p = c.p();
-    const int K = p.F, pairs = K / 2, all = c.sh().m * pairs, stride = st_array_bytes(K);
+    const int K = p.F, quads = K / 4, all = c.sh().m * quads, stride = st_array_bytes(K);
     bool ok = true;
     zero_tail(c, K);
 #pragma unroll 1
     for (int base0 = 0; base0 < all; base0 += U * ST_NT) {
         const int base = base0 + c.tid;
-        Two t[U];
+        Four t[U];
         unsigned todo = 0;
 #pragma unroll
         for (int i = 0; i < U; ++i)
             if (base + i * ST_NT < all) todo |= 1u << i;
         auto at = [&](int i) {
-            const int u = base + i * ST_NT, tok = MT > 1 && u >= pairs ? 1 : 0;
-            return p.act_ll + static_cast<size_t>(tok) * p.act_len + 2 * (u - tok * pairs);
+            const int u = base + i * ST_NT, tok = MT > 1 && u >= quads ? 1 : 0;
+            return p.act_ll + static_cast<size_t>(tok) * p.act_len + 4 * (u - tok * quads);
         };
         Spin sp;
         for (;;) {
 #pragma unroll
             for (int i = 0; i < U; ++i)
-                if (todo >> i & 1u) t[i] = get2(at(i));
+                if (todo >> i & 1u) t[i] = get4(at(i));
 #pragma unroll
             for (int i = 0; i < U; ++i)
-                if ((todo >> i & 1u) && pieces_tag(t[i].a, tag) && pieces_tag(t[i].b, tag)) {
+                if ((todo >> i & 1u) && pieces_tag(t[i].a, tag) && pieces_tag(t[i].b, tag) && pieces_tag(t[i].c, tag) && pieces_tag(t[i].d, tag)) {
                     todo &= ~(1u << i);
-                    const int u = base + i * ST_NT, tok = MT > 1 && u >= pairs ? 1 : 0;
-                    unsigned char *to = c.area() + tok * Ctx<MT>::S * stride + (u - tok * pairs) * 4;
-#pragma unroll
-                    for (int q = 0; q < Ctx<MT>::S; ++q)
-                        *reinterpret_cast<uint32_t *>(to + q * stride) = (static_cast<uint32_t>(t[i].a >> (16 * q)) & 0xffffu) | static_cast<uint32_t>(t[i].b >> (16 * q)) << 16;
+                    const int u = base + i * ST_NT, tok = MT > 1 && u >= quads ? 1 : 0;
+                    unsigned char *to = c.area() + tok * Ctx<MT>::S * stride + (u - tok * quads) * 8;
+                    const uint32_t a0 = static_cast<uint32_t>(t[i].a), b0 = static_cast<uint32_t>(t[i].b), c0 = static_cast<uint32_t>(t[i].c), d0 = static_cast<uint32_t>(t[i].d);
+                    const uint32_t a1 = static_cast<uint32_t>(t[i].a >> 32), b1 = static_cast<uint32_t>(t[i].b >> 32), c1 = static_cast<uint32_t>(t[i].c >> 32), d1 = static_cast<uint32_t>(t[i].d >> 32);
+                    *reinterpret_cast<uint2 *>(to) = make_uint2(__byte_perm(a0, b0, 0x5410), __byte_perm(c0, d0, 0x5410));
+                    *reinterpret_cast<uint2 *>(to + stride) = make_uint2(__byte_perm(a0, b0, 0x7632), __byte_perm(c0, d0, 0x7632));
+                    *reinterpret_cast<uint2 *>(to + 2 * stride) = make_uint2(__byte_perm(a1, b1, 0x5410), __byte_perm(c1, d1, 0x5410));
                 }
             const int more = warp_again(sp, todo != 0u, c.abort(), p.spin_limit);
             if (more == 0) ok = false;

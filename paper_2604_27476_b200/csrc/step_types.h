@@ -153,6 +153,8 @@ struct StepLaunch {
 int step_shared_bytes(int mt);  // fixed part of the kernel's shared memory
 int step_scratch_floats(int D, int G, int mt);
 
+// Packets of the attention's maxima and denominators; whole lines (what follows is lines with one writer each: 64 bytes off, two share one).
+inline size_t step_stat_len(size_t chunks, int nq) { return (chunks * nq * 2 + 15) / 16 * 16; }
 // Bytes of a vector's exchange buffer / of the MLP activations' (whole 128 bytes).
 inline size_t step_vec_bytes(const StepParams &p, int mt, int K, bool sums) {
     return (static_cast<size_t>(st_arrays(mt)) * st_array_bytes(K) + (sums ? 4 * static_cast<size_t>(mt) * p.ss_stride : 0) + 127) / 128 * 128;
@@ -215,7 +217,7 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.prefetch_bytes = ST_PREFETCH_BYTES;
     p.spin_limit = 1000000000u;   // 1 s
     const size_t chunks = static_cast<size_t>(std::max(grid / nkv, mt));
-    sl->ll_bytes = 8 * (static_cast<size_t>(grid) * mt * p.q_line + static_cast<size_t>(grid) * 16 + chunks * qd + chunks * nq * 2) + 2 * step_vec_bytes(p, mt, H, true) +
+    sl->ll_bytes = 8 * (static_cast<size_t>(grid) * mt * p.q_line + static_cast<size_t>(grid) * 16 + chunks * qd + step_stat_len(chunks, nq)) + 2 * step_vec_bytes(p, mt, H, true) +
                    step_vec_bytes(p, mt, qd, false) + step_act_bytes(p, mt) + 256 +
                    (st_packets(mt) ? 8 * (static_cast<size_t>(grid) * mt * (2 * p.x_line + p.ao_line) + static_cast<size_t>(mt) * p.act_len) : 0);
     return nullptr;
@@ -234,7 +236,7 @@ inline void step_wire(StepLaunch *sl, int mt, unsigned long long *base) {
     p.q_ll = base; base += g * m * p.q_line;
     p.lm_ll = base; base += g * 16;
     p.part_ll = base; base += chunks * p.qd;
-    p.stat_ll = base; base += chunks * p.nq * 2;
+    p.stat_ll = base; base += step_stat_len(chunks, p.nq);
     if (!st_packets(mt)) return;
     p.x_ll = base; base += g * m * p.x_line;
     p.xo_ll = base; base += g * m * p.x_line;

@@ -4,7 +4,7 @@
   python bench.py [--gpus N] [--steps K] [--warmup W] [--config NAME] [--impl ours|reference]
 
 One "step" is one decode step (one token) of the named decoder shape over its pre-filled KV cache,
-i.e. one replay of the step graph.  The default workload is the Qwen2.5-1.5B-shaped decoder with a
+i.e. one launch of the step kernel.  The default workload is the Qwen2.5-1.5B-shaped decoder with a
 2048-position cache.  With N > 1 (torchrun) every rank runs an independent replica of the same
 request (the step does not shard; there is no collective on the data path).
 """
@@ -30,7 +30,7 @@ from edgefm_synth import CONFIGS, GLOBAL_SEED, first_token, make_kv, make_weight
 # DRAM traffic of one launch of the step kernel: dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of
 # that kernel, per configuration, with the profile summary (and the source revision it names) the figure comes from.
 # Only captured configurations have a value; a figure is only as current as its summary says.
-NCU_TRAFFIC = {"qwen2.5-1.5b": {"bytes": None, "source": "profiles/decode_megakernel_qwen2.5-1.5b_ctx2048.md"}}
+NCU_TRAFFIC = {"qwen2.5-1.5b": {"bytes": None, "source": "profiles/step_kernel_qwen2.5-1.5b_ctx2048.md"}}
 
 
 def ncu_traffic(name):
@@ -410,7 +410,7 @@ def main():
     workload = workload_name(cfg, args.kv_format) + (f", output layer pruned to {n_sub} of {cfg.vocab} token ids" if n_sub else "")
 
     def free_run(n):
-        """n chained greedy steps, token and position carried on the device (one graph launch per token)."""
+        """n chained greedy steps, token and position carried on the device (one launch per token)."""
         ctx.prefill_kv(kd, vd)
         edgefm_decode_step(handle, tok0, pos0, stream, None, None)
         for _ in range(n - 1):
@@ -489,7 +489,7 @@ def main():
             "config": config_block(cfg, workload, world, pruned_bytes),
             "timed_sequences": n_seq, "ms_per_token_min": ms_per_token_min,
             "tokens_per_s": tokens / (dev_ms * 1e-3),
-            "roofline": {"bound": "hbm", "kernel": f"decode_megakernel: the whole decode step ({launches} kernel launch per token, one CUDA graph node)",
+            "roofline": {"bound": "hbm", "kernel": f"step_kernel: the whole decode step ({launches} kernel launch per token)",
                          "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "peak_source": peak_src,
                          "bytes_per_launch": bytes_per_step, "frac_of_nominal_8TBs": gbs / NOMINAL_HBM_GBS, "traffic": traffic, "traffic_source": traffic_src},
             "e2e": {"value": e2e_ms / tokens, "unit": UNIT, "h2d_bytes_per_step": 48, "d2h_bytes_per_step": 4},

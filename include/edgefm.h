@@ -4,14 +4,14 @@
  * The library implements the decode phase of Eq. 4 of the paper,
  *     y_t <- DecodeStep(y_{t-1}, KV; theta_d),   KV <- UpdateKV(KV, y_t),
  * for one request slot (Sec. 3.7, 3.9: a slot owns a pre-allocated KV cache) with greedy sampling
- * (Sec. 4.2: temperature 0, top_k = 1), replayed as one fixed CUDA graph per token whose dynamic
- * parameters (token, position, cache length) live in device memory (Sec. 3.10).
+ * (Sec. 4.2: temperature 0, top_k = 1): one launch of one persistent kernel per token, whose dynamic
+ * state (token, position, cache length) lives in device memory (Sec. 3.10).
  *
  * Conventions
  *   - "device" pointers are CUDA device pointers on the device that was current at edgefm_create;
  *     "host" pointers are ordinary host memory.  All bf16 data is raw 16-bit patterns.
  *   - Weights are BORROWED: the caller allocates them, keeps them alive and unmodified until
- *     edgefm_destroy.  The context OWNS its KV cache, work buffers, device state and CUDA graph.
+ *     edgefm_destroy.  The context OWNS its KV cache, work buffers and device state.
  *   - edgefm_prefill_kv and edgefm_decode_step only enqueue work on `stream` (a cudaStream_t passed
  *     as void*; NULL = the legacy default stream) and return without synchronising.  All calls on
  *     one context must be issued on one stream or be externally ordered; a context is not
@@ -79,7 +79,7 @@ typedef struct {
 /*
  * edgefm_create -- build a context for one request slot (Sec. 3.7 step 1, Sec. 3.9 pre-allocation).
  * Allocates the KV cache K,V : bf16 [n_layers][n_kv_heads][max_context][head_dim] (cache length 0),
- * the work buffers and the device state, and records the step as a CUDA graph.
+ * the work buffers and the device state.
  * All matrix base pointers must be 16-byte aligned.  `shape` and `weights` (and the `layers` array)
  * are read during the call only; the device buffers they point to are borrowed until destroy.
  * Errors: INVALID_ARG (null pointers, max_context < 1), BAD_SHAPE, OUT_OF_MEMORY, CUDA.
@@ -101,8 +101,7 @@ edgefm_status edgefm_create(const edgefm_shape *shape, const edgefm_weights *wei
  *     edgefm_export_kv is refused on such a context (use edgefm_export_kv_int8), and so is edgefm_decode_step_static.
  *   options->block_tokens = 0 or 1 : plain decode steps only;
  *                           2 or 4 : the context can also verify a block of up to that many tokens per call
- *     (edgefm_verify_block).  It then runs a build of the step kernel that carries the tokens side by side (work buffers
- *     per token, somewhat smaller weight tiles); edgefm_decode_step works as before on such a context.  The 2-token
+ *     (edgefm_verify_block).  It then runs a build of the step kernel that carries the tokens side by side; edgefm_decode_step works as before on such a context.  The 2-token
  *     build multiplies with the same 24-bit activations as the plain step; the 4-token build stages every activation as
  *     two bf16 pieces (16 mantissa bits) so that four tokens fit one tensor-core operand.  Needs the plain bf16 cache and
  *     max_context <= 8192.
@@ -161,10 +160,10 @@ edgefm_status edgefm_decode_step(edgefm_ctx *ctx, int32_t token_id, int32_t posi
  * grows by n_accepted (the rows of rejected tokens stay behind it and are overwritten later); the next token is
  * g_{n_accepted - 1}.  The result is what n_accepted plain decode steps would have produced.
  *   tokens          : HOST int32 [m], read during the call.  m = 1 .. block_tokens of the context (m = 1 is a decode step)
- *                     through the step kernel.  Longer blocks, up to 8 tokens (on any context, also block_tokens = 0), take the
- *                     DENSE path: the prefill kernels of edgefm_prefill for the m tokens, one pass over the output matrix for
- *                     all m rows, the same acceptance rule on the device.  That path needs tokens[0] and position given (no
- *                     -1) and an exact host-side cache length: after a verified block, edgefm_sync_length comes first.
+ *                     through the step kernel.  Longer blocks, up to 8 tokens (on any context, also block_tokens = 0), take a build
+ *                     of the kernel for 8 tokens, made at the first such call and kept, or, where a shape does not fit it, the
+ *                     kernels of edgefm_prefill.  They need tokens[0] and position given (no -1) and an exact host-side
+ *                     cache length: after a verified block, edgefm_sync_length comes first.
  *   logits_out      : DEVICE fp32 [m][vocab] (row t: the logits after token t; rows >= n_accepted belong to rejected
  *                     tokens) or NULL.  With a vocabulary subset of n ids (edgefm_set_vocab_subset) the rows are n long,
  *                     [m][n], and the greedy tokens -- hence the acceptance -- are taken over the subset.
@@ -237,7 +236,7 @@ edgefm_status edgefm_export_kv(edgefm_ctx *ctx, void *k_out, void *v_out, void *
 edgefm_status edgefm_export_kv_int8(edgefm_ctx *ctx, void *k_codes_out, void *v_codes_out, float *k_scales_out,
                                     float *v_scales_out, void *stream);
 
-/* Number of kernel launches one decode step performs (nodes of the step graph). */
+/* Number of kernel launches one decode step performs (always 1). */
 edgefm_status edgefm_get_launches_per_step(const edgefm_ctx *ctx, int32_t *n_launches_host);
 
 /* Synchronise `stream`, then report whether a bounded device-side wait of the persistent step kernel
@@ -285,16 +284,15 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
  * out_host (capacity in elements).  n_ctas = 0 when profiling is off; out_host may be NULL to query the sizes. */
 edgefm_status edgefm_debug_profile(edgefm_ctx *ctx, uint64_t *out_host, int64_t capacity, int32_t *n_ctas, int32_t *stride);
 
-/* Launch geometry of the context's step kernel: out8 = {CTAs, consumer warps per CTA, ring slots per warp, bytes per slot,
- * dynamic shared memory, tiles of the busiest CTA, shared-memory bytes reserved for the tile lists, 1 = long-context
- * build of the kernel}.  Host only. */
+/* Launch geometry of the context's step kernel: out8 = {CTAs, consumer warps per CTA, chunks the weight ring can hold at once, bytes of the
+ * largest chunk, dynamic shared memory, bytes of the ring, shared-memory bytes of the tables, 0}.  Host only. */
 edgefm_status edgefm_debug_plan(const edgefm_ctx *ctx, int32_t *out8);
 
-/* Every device-side wait of the step kernel (tile arrival, grid barrier) gives up after a bound (1 s by default), records
+/* Every device-side wait of the step kernel (chunk arrival, exchange) gives up after a bound (1 s by default), records
  * EDGEFM_ERR_TIMEOUT in the device state and lets the kernel return; edgefm_sync_status reports it.  This call changes
  * the bound (limit_ns >= 1000) of the steps enqueued afterwards and, for testing that path without any fault, can make the
- * grid barrier expect one arrival more than there are CTAs (extra_barrier_arrivals = 1; 0 in production), so that the
- * first barrier of the next step runs into the bound.  Synchronises the device and re-records the step graph. */
+ * exchanges expect what no CTA sends (extra_barrier_arrivals = 1; 0 in production), so that the first exchange of the
+ * next step runs into the bound.  Synchronises the device. */
 edgefm_status edgefm_debug_set_wait_limit(edgefm_ctx *ctx, uint32_t limit_ns, int32_t extra_barrier_arrivals);
 
 /* The same for the contractions of edgefm_prefill: every wait on a shared-memory barrier gives up after `polls` polls

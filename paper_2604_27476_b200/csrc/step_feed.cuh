@@ -93,6 +93,14 @@ __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f, FKV f_kv) 
     }
 }
 
+// The last of a feeding thread's `issued` copies (`n` barriers, a power of two, used in turn) must land before the CTA's shared memory is
+// released.  The products wait for them anyway, unless one has given up: then they may still be on their way when all other
+// threads have left, whether the feeding thread had more to copy or not.  The bound is its own: the waits' may be shorter than a copy.
+__device__ __forceinline__ void drain(unsigned long long *bars, unsigned n, unsigned issued) {
+    int never = 0;
+    for (unsigned k = issued > n ? issued - n : 0u; k < issued; ++k) mbar_wait(&bars[k & (n - 1u)], (k / n) & 1u, &never, ST_DRAIN_NS);
+}
+
 // One thread fills the ring ...
 template <bool Q8, int MT>
 __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
@@ -183,11 +191,7 @@ __device__ __forceinline__ void feed_ring(Ctx<MT> &c) {
                 bulk(to + b.v_at + i * b.v_stride, v + static_cast<size_t>(i * b.R) * row_bytes, static_cast<unsigned>(min(b.R, n - i * b.R) * row_bytes), bar, keep);
             return true;
         });
-    if (!ok) {               // giving up: the copies in flight must land before the CTA's shared memory is released
-        int dummy = 0;
-        for (unsigned k = issued > ST_BARS ? issued - ST_BARS : 0; k < issued; ++k)
-            mbar_wait(&sh.full[k & (ST_BARS - 1)], (k / ST_BARS) & 1u, &dummy, limit);
-    }
+    drain(sh.full, ST_BARS, issued);
 }
 // ... another asks L2 for what comes after it, at most prefetch_bytes ahead: the ring alone holds too little to keep HBM busy
 // through the exchanges, and a refill from L2 comes at more than twice the rate of HBM.
@@ -291,10 +295,7 @@ __device__ __forceinline__ void feed_vectors(Ctx<MT> &c) {
             if (ok) copy(p.act_vec + static_cast<size_t>(i % segs) * slot, static_cast<unsigned>(i % p.act_slots) * slot, slot);
         }
     }
-    if (!ok) {               // giving up: the copies in flight must land before the CTA's shared memory is released
-        int dummy = 0;
-        for (unsigned j = k > 4 ? k - 4 : 0; j < k; ++j) mbar_wait(&sh.x_full[j & 3u], (j >> 2) & 1u, &dummy, p.spin_limit);
-    }
+    drain(sh.x_full, 4u, k);
 }
 
 }  // namespace step

@@ -31,8 +31,8 @@
 //     through the step together, at consecutive positions and cache slots; CTA 0 accepts the longest prefix that greedy decoding
 //     would have produced.
 //
-// Every wait is bounded: on expiry the CTA records status 6, all its warps leave at the next CTA-wide vote, the feeding warp
-// waits (bounded) for its copies in flight.
+// Every wait is bounded: on expiry the CTA records status 6 and all its warps leave at the next CTA-wide vote; the feeding threads
+// leave when their copies have landed (bounded, too).
 #include "step_attention.cuh"
 #include "step_feed.cuh"
 #include "step_products.cuh"

@@ -16,6 +16,7 @@ constexpr int ST_THREADS = ST_NT + 128;      // + the feeding warpgroup (two of 
 // Registers: 384 threads are launched with 168 each; 256 x 208 + 128 x 88 is what they were launched with.
 constexpr int ST_REGS_LAUNCH = 168, ST_REGS = 208, ST_REGS_FEED = 88;
 static_assert(ST_NT * ST_REGS + 128 * ST_REGS_FEED <= ST_THREADS * ST_REGS_LAUNCH, "setmaxnreg only redistributes the launch's registers");
+constexpr unsigned ST_DRAIN_NS = 2000000000u;   // how long a CTA that leaves waits for its copies in flight
 constexpr int ST_BARS = 16;                  // chunks the ring can hold at once (a power of two)
 constexpr int ST_CHUNK_BYTES = 52 * 1024;    // aimed at for a ring chunk cut by columns
 constexpr int ST_CHUNK_SMALL = 28 * 1024;    // ... where a segment needs no exchange of its own: the ring refills in finer steps (1.5B shape, 8960 columns: 6.0 -> 5.5 us)

@@ -45,6 +45,42 @@ def test_grid_barrier_wait_expires_and_is_reported():
         pair.close()                                               # destroying the timed-out context succeeds
 
 
+@pytest.mark.parametrize("m,block_tokens", [(1, 0), (4, 4), (8, 0)], ids=["step", "block4", "block8"])
+@pytest.mark.parametrize("limit_ns", [1000, 200_000])
+def test_a_cta_that_gives_up_waits_for_its_copies(m, block_tokens, limit_ns):
+    """Waits so short that every CTA gives up with its copies under way (1 us: before the first chunk is there; 200 us: the whole of this
+    small step has been asked for and the feeding threads are done).  The copies must land before the CTA's shared memory is
+    someone else's: other contexts, whose kernels follow at once on the same stream, compute what they always do."""
+    import torch
+    from paper_2604_27476_b200 import DecodeContext, EdgefmError, Status, edgefm_debug_set_wait_limit
+    cfg = CONFIGS["tiny"]
+    pair = Pair(cfg, max_context=cfg.cache_len + 8, block_tokens=block_tokens)
+    others = [DecodeContext(cfg, pair.ptrs, cfg.cache_len + 8, block_tokens=block_tokens) for _ in range(3)]
+    try:
+        tok, pos = first_token(cfg), cfg.first_position
+        ref, _ = pair.oracle.step(tok, pos)
+        block = [tok] + [5] * (m - 1)
+        run = lambda ctx: ctx.step(tok, pos) if m == 1 else ctx.verify_block(block, pos)
+        for o in others:
+            o.prefill_kv(pair.kd, pair.vd)
+        torch.cuda.synchronize()
+        edgefm_debug_set_wait_limit(pair.ctx.handle, limit_ns, 1)
+        run(pair.ctx)
+        for o in others:
+            run(o)
+        torch.cuda.synchronize()
+        with pytest.raises(EdgefmError) as ei:
+            pair.ctx.sync_status()
+        assert ei.value.status == Status.ERR_TIMEOUT
+        for o in others:
+            o.sync_status()
+            assert_logits_close(o.logits.cpu().numpy(), ref, "a context behind the one that gave up")
+    finally:
+        for o in others:
+            o.close()
+        pair.close()
+
+
 def test_prefill_contraction_wait_expires_and_is_reported():
     """The same for the contractions of edgefm_prefill: their stage barriers are told to expect an arrival nobody makes and
     the bound is shortened to 2^16 polls; every contraction gives up at its first wait, drains and returns."""

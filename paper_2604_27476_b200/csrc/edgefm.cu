@@ -247,6 +247,19 @@ cudaError_t run_step(edgefm_ctx::Build *b, const StepRequest &r, cudaStream_t s)
     return launch_step(b->launch, s);
 }
 
+// Zeroed exchange buffers and tensor maps of a build, complete when the call returns: the first launch may go to any stream, and work on the
+// legacy stream is ordered against neither a non-blocking one nor the return of a pageable copy.
+cudaError_t init_build(void *ll, size_t ll_bytes, void *maps, const void *host_maps, size_t map_bytes) {
+    cudaStream_t own = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(ll, 0, ll_bytes, own);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(maps, host_maps, map_bytes, cudaMemcpyHostToDevice, own);
+    const cudaError_t done = cudaStreamSynchronize(own);
+    cudaStreamDestroy(own);
+    return e != cudaSuccess ? e : done;
+}
+
 // Plan and buffers of the build for `mt` tokens per call.  *why: the shape does not fit.
 cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char **why) {
     int smem_optin = 0, per_sm = 0;
@@ -254,10 +267,7 @@ cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char *
     if (e != cudaSuccess) return e;
     StepLaunch &sl = b->launch;
     if ((*why = step_plan(c->shape, c->max_context, c->num_sms, smem_optin, c->kv_format == EDGEFM_KV_INT8, mt, &sl))) return cudaSuccess;
-    if (!b->ll) {
-        if ((e = dev_alloc(&b->ll, sl.ll_bytes / 8)) != cudaSuccess) return e;
-        if ((e = cudaMemset(b->ll, 0, sl.ll_bytes)) != cudaSuccess) return e;
-    }
+    if (!b->ll && (e = dev_alloc(&b->ll, sl.ll_bytes / 8)) != cudaSuccess) return e;
     step_wire(&sl, mt, b->ll);
     StepParams &p = sl.p;
     {
@@ -265,7 +275,7 @@ cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char *
         const bool sub = c->vocab_subset > 0;
         if (!step_maps(p, c->layers.data(), sub ? static_cast<const void *>(c->sub_lm) : c->lm_head, sub ? c->vocab_subset : c->shape.vocab, maps.data())) return cudaErrorUnknown;
         if (!b->maps && (e = cudaMalloc(reinterpret_cast<void **>(&b->maps), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
-        if ((e = cudaMemcpy(b->maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+        if ((e = init_build(b->ll, sl.ll_bytes, b->maps, maps.data(), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
         p.maps = b->maps;
         p.map_fence = 1;   // edgefm_set_vocab_subset rewrites the output layer's map
     }

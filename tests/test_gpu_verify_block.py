@@ -296,3 +296,30 @@ def test_dense_block_with_a_pruned_output_layer():
             assert pair.ctx.sync_length() == start + ref_acc
     finally:
         pair.close()
+
+
+def test_first_long_block_on_a_side_stream():
+    """The build for eight tokens is made at the first block that needs it.  It is ready for any stream when it is launched: here the
+    first block goes to a non-blocking stream while the legacy stream is busy, and does not wait for that either."""
+    import torch
+    cfg = CONFIGS["tiny"]
+    pair = Pair(cfg, cache_len=40, max_context=64)
+    try:
+        tok, pos = first_token(cfg), 40
+        block = [tok] + _peek_chain(pair, tok, pos, 5)
+        ref_rows, ref_acc, _ = pair.oracle.verify_block(block, pos)
+        side, busy = torch.cuda.Stream(), torch.cuda.Event()
+        torch.cuda._sleep(1_000_000_000)                     # about half a second of the legacy stream
+        busy.record()
+        with torch.cuda.stream(side):
+            pair.ctx.verify_block(block, pos)
+            assert not busy.query()
+            assert pair.ctx.sync_length() == pair.oracle.cur_len
+            pair.ctx.sync_status()
+        got = pair.ctx.block_logits.cpu().numpy()
+        for i in range(ref_acc):
+            assert_logits_close(got[i], ref_rows[i], f"row {i}")
+        assert int(pair.ctx.n_accepted.item()) == ref_acc
+    finally:
+        torch.cuda.synchronize()
+        pair.close()

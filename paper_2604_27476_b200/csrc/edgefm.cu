@@ -533,15 +533,21 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
     DeviceGuard guard(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     edgefm_ctx::Build *build = &ctx->step;
-    if (longer) {
-        if (!ctx->wide.made && !ctx->wide_refused) {   // made at the first longer block, kept
+    bool prompt_kernels = longer && ctx->wide_refused;
+    if (longer && !ctx->wide.made && !prompt_kernels) {
+        // The build for eight tokens is made at the first longer block and kept, but not while a stream is being captured (it allocates)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CUDA_TRY(ctx, cudaStreamIsCapturing(s, &cap));
+        if (cap != cudaStreamCaptureStatusNone) {
+            prompt_kernels = true;
+        } else {
             const char *why = nullptr;
             CUDA_TRY(ctx, make_build(ctx, PF_VERIFY_MAX, &ctx->wide, &why));
-            ctx->wide_refused = why != nullptr;
+            prompt_kernels = ctx->wide_refused = why != nullptr;
         }
-        build = &ctx->wide;
     }
-    if (longer && ctx->wide_refused) {   // a shape whose vectors for eight tokens do not fit the shared memory: the prompt kernels
+    if (longer) build = &ctx->wide;
+    if (prompt_kernels) {   // also for a shape whose vectors for eight tokens do not fit the shared memory
         if (const edgefm_status st = ensure_prefill_buffers(ctx)) return st;
         PrefillModel pm = prefill_model(ctx);
         int launches = 0;

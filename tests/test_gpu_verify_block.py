@@ -323,3 +323,44 @@ def test_first_long_block_on_a_side_stream():
     finally:
         torch.cuda.synchronize()
         pair.close()
+
+
+def test_first_long_block_in_a_capture():
+    """A captured first long block cannot make the build for eight tokens (that allocates): it is recorded with the prompt kernels, whose
+    buffers an earlier prompt made; behind the capture the build is made as usual."""
+    import ctypes
+
+    import torch
+    from paper_2604_27476_b200 import binding as B
+    cfg = CONFIGS["tiny"]
+    T0 = 40
+    pair = Pair(cfg, cache_len=T0, max_context=80)
+    try:
+        pair.ctx.prefill(list(range(1, 20)), T0)
+        pair.ctx.append_kv(T0)
+        block = [first_token(cfg)] + _peek_chain(pair, first_token(cfg), T0, 5)
+        ref_rows, ref_acc, ref_next = pair.oracle.verify_block(block, T0)
+        tokens = (ctypes.c_int32 * len(block))(*block)       # a replay copies the tokens from here
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            status = B.load_library().edgefm_verify_block(pair.ctx.handle, tokens, len(block), T0, torch.cuda.current_stream().cuda_stream,
+                                                          pair.ctx.block_logits.data_ptr(), pair.ctx.n_accepted.data_ptr(), pair.ctx.next_token.data_ptr())
+        assert status == 0, B.edgefm_last_error(pair.ctx.handle)
+        for again in range(2):                               # the recorded block, then an ordinary one
+            pair.ctx.block_logits.zero_()
+            if again == 0:
+                graph.replay()
+            else:
+                pair.ctx.append_kv(T0)
+                pair.ctx.verify_block(block, T0)
+            assert pair.ctx.sync_length() == pair.oracle.cur_len
+            pair.ctx.sync_status()
+            got = pair.ctx.block_logits.cpu().numpy()
+            for i in range(ref_acc):
+                assert_logits_close(got[i], ref_rows[i], f"row {i}")
+            assert int(pair.ctx.n_accepted.item()) == ref_acc
+            if top2_margin(ref_rows[ref_acc - 1]) > TOKEN_MARGIN:
+                assert int(pair.ctx.next_token.item()) == ref_next
+    finally:
+        pair.close()

@@ -191,9 +191,11 @@ edgefm_status fail(edgefm_ctx *ctx, edgefm_status st, const char *fmt, ...) {
 #define CUDA_TRY(ctx, call)                                                                                   \
     do {                                                                                                      \
         cudaError_t e_ = (call);                                                                              \
-        if (e_ != cudaSuccess)                                                                                \
+        if (e_ != cudaSuccess) {                                                                              \
+            cudaGetLastError();   /* reported here: the check behind a later launch must not find it again */ \
             return fail(ctx, e_ == cudaErrorMemoryAllocation ? EDGEFM_ERR_OUT_OF_MEMORY : EDGEFM_ERR_CUDA,    \
                         "%s failed: %s", #call, cudaGetErrorString(e_));                                      \
+        }                                                                                                     \
     } while (0)
 
 struct DeviceGuard {

@@ -99,3 +99,30 @@ def test_unaligned_strided_prefill_takes_the_scalar_path():
         assert torch.equal(kc[:, :, :9], k) and torch.equal(vc[:, :, :9], k) and pair.ctx.cur_len == 9
     finally:
         pair.close()
+
+
+def test_a_failed_call_leaves_no_error_behind():
+    """A CUDA error is reported by the call it belongs to (here: waiting for a stream under capture) and not again by the next one."""
+    import torch
+    from paper_2604_27476_b200 import EdgefmError, Status
+    pair = Pair(TINY, cache_len=2, max_context=4)
+    try:
+        other = torch.cuda.Stream()
+        failed, behind = None, None
+        with pytest.raises(RuntimeError):                                      # the capture itself is lost
+            with torch.cuda.graph(torch.cuda.CUDAGraph()):
+                try:
+                    pair.ctx.sync_length()
+                except EdgefmError as e:
+                    failed = e
+                with torch.cuda.stream(other):
+                    try:
+                        pair.ctx.append_kv(1)
+                    except EdgefmError as e:
+                        behind = e
+        assert failed is not None and failed.status == Status.ERR_CUDA
+        assert behind is None, behind
+        torch.cuda.synchronize()
+        assert pair.ctx.sync_length() == 1
+    finally:
+        pair.close()

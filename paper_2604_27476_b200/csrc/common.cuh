@@ -6,6 +6,10 @@
 
 namespace edgefm {
 
+// A bounded wait of the step kernel ran out.  Its exchange buffers then hold packets and arrivals of a step that was never finished, which
+// the next one would take for its own: the status stays, whatever happens to the cache, and later steps do nothing.
+constexpr int STATUS_TIMEOUT = 6;
+
 // Device-resident dynamic parameters of the step (Sec. 3.10 of the paper: dynamic parameters live in GPU buffers, so that one fixed
 // launch serves every decode iteration).
 struct StepState {
@@ -14,7 +18,7 @@ struct StepState {
     int cur_len;        // filled cache slots before the step == slot the step writes
     int next_token;     // greedy result of the last finished step
     int next_position;  // position the next step uses when the caller passes -1
-    int status;         // 0 = ok (reserved for bounded-wait failures)
+    int status;         // 0 = ok, STATUS_TIMEOUT, or the code of a self-check (100 and up)
     int pad[2];
     int n_accepted;     // tokens of the last block the cache was advanced by (1 for a plain step)
     int epoch[2];       // finished calls of the step kernel (of each of a context's two builds): what its packets are tagged with

@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(256) prefill_copy_kernel(const uint16_t *k, co
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->cur_len = slot0 + n;
         st->next_position = slot0 + n;
-        st->status = 0;
+        if (st->status != STATUS_TIMEOUT) st->status = 0;
     }
     const long long total = static_cast<long long>(L) * nkv * n * d;
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(256) prefill_quantize_kernel(const uint16_t *k
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->cur_len = slot0 + n;
         st->next_position = slot0 + n;
-        st->status = 0;
+        if (st->status != STATUS_TIMEOUT) st->status = 0;
     }
     const int warps = (gridDim.x * blockDim.x) >> 5, lane = threadIdx.x & 31;
     const long long rows = static_cast<long long>(L) * nkv * n * 2;          // K rows, then V rows

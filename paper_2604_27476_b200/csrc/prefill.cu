@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(128) prefill_norm_kernel(float *resid, uint16_
     if (st && blockIdx.x == 0 && threadIdx.x == 0) {
         st->cur_len = new_len;
         st->next_position = new_pos;
-        st->status = 0;
+        if (st->status != STATUS_TIMEOUT) st->status = 0;
     }
     __shared__ float red[4];
     const int row = blockIdx.x, tid = threadIdx.x;

@@ -31,7 +31,7 @@
 //     through the step together, at consecutive positions and cache slots; CTA 0 accepts the longest prefix that greedy decoding
 //     would have produced.
 //
-// Every wait is bounded: on expiry the CTA records status 6 and all its warps leave at the next CTA-wide vote; the feeding threads
+// Every wait is bounded: on expiry the CTA records STATUS_TIMEOUT and all its warps leave at the next CTA-wide vote; the feeding threads
 // leave when their copies have landed (bounded, too).
 #include "step_attention.cuh"
 #include "step_feed.cuh"
@@ -103,13 +103,13 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.abort = 0;
             sh.sent = 0u;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            const int rt = p.req.token, rp = p.req.position, st_token = p.state->next_token, st_pos = p.state->next_position, st_len = p.state->cur_len;
+            const int rt = p.req.token, rp = p.req.position, st_token = p.state->next_token, st_pos = p.state->next_position, st_len = p.state->cur_len, st_status = p.state->status;
             const unsigned epoch = static_cast<unsigned>(p.state->epoch[p.epoch_slot]);
             sh.m = MT > 1 ? min(max(p.req.m, 1), MT) : 1;
             sh.tokens[0] = rt >= 0 ? rt : st_token;
             for (int t = 1; t < MT; ++t) sh.tokens[t] = t < sh.m ? p.req.draft[t - 1] : 0;
             sh.pos = rp >= 0 ? rp : st_pos;
-            sh.n_old = st_len;
+            sh.n_old = st_status == STATUS_TIMEOUT ? -1 : st_len;
             sh.n_chunks = kv_chunks(p, sh.n_old, sh.m, c.ncta);
             sh.tag0 = epoch * static_cast<unsigned>(p.n_layers + 2) + 1u;
             sh.odd = static_cast<unsigned>(p.barrier_extra) << 31 | static_cast<unsigned>(p.barrier_extra) << 15;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         const int lm_rows = c.head().rows;
         bool sane = true;
         for (int t = 0; t < MT; ++t) sane = sane && sh.tokens[t] >= 0 && sh.tokens[t] < p.V;
-        // a corrupt request or state: compute nothing
+        // a corrupt request or state, or an earlier step that ran into the bound of a wait: compute nothing
         if (!sane || sh.n_old < 0 || sh.n_old + sh.m > p.max_context || sh.pos < 0 || lm_rows < 1 || lm_rows > p.V) {
             if (c.tid == 0 && atomicCAS(&p.state->status, 0, 103) == 0) { p.state->pad[0] = sh.tokens[0]; p.state->pad[1] = sh.n_old; }
             return;
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
     Shared<MT> &sh = c.sh();
     if (!ok) {
         *c.abort() = 1;
-        if (c.tid == 0) atomicCAS(&p.state->status, 0, 6);
+        if (c.tid == 0) atomicExch(&p.state->status, STATUS_TIMEOUT);
         return;
     }
     // ---- greedy tokens: thread -> warp -> CTA -> CTA 0 -> state ------------------------------------------------------------
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
         }
     }
     if (!cta_vote(ok)) {
-        if (c.tid == 0) atomicCAS(&p.state->status, 0, 6);
+        if (c.tid == 0) atomicExch(&p.state->status, STATUS_TIMEOUT);
         return;
     }
     if (c.tid == 0) {

@@ -81,6 +81,46 @@ def test_a_cta_that_gives_up_waits_for_its_copies(m, block_tokens, limit_ns):
         pair.close()
 
 
+@pytest.mark.parametrize("m,block_tokens,kv_format", [(1, 0, None), (4, 4, None), (8, 0, None), (1, 0, "int8"), (8, 0, "int8")],
+                         ids=["step", "block4", "block8", "step_int8", "block8_int8"])
+def test_a_timeout_is_not_forgotten(m, block_tokens, kv_format):
+    """Behind an expired wait the exchange buffers hold what a step left that was never finished.  Neither new cache rows nor a prompt nor
+    further steps, with the bound restored, may make the context look sound again: the status stays until it is destroyed."""
+    import torch
+    from paper_2604_27476_b200 import EdgefmError, Status, edgefm_debug_set_wait_limit
+    cfg = CONFIGS["tiny"]
+    pair = Pair(cfg, cache_len=32, max_context=128, block_tokens=block_tokens, kv_format=kv_format)
+    try:
+        tok, pos = first_token(cfg), 32
+        run = lambda: pair.ctx.step(tok, pos) if m == 1 else pair.ctx.verify_block([tok] + [5] * (m - 1), pos)
+
+        def expired():
+            with pytest.raises(EdgefmError) as ei:
+                pair.ctx.sync_status()
+            return ei.value.status == Status.ERR_TIMEOUT
+
+        run()
+        pair.ctx.sync_status()
+        pair.ctx.append_kv(32)
+        edgefm_debug_set_wait_limit(pair.ctx.handle, 2_000_000, 1)
+        run()
+        assert expired()
+        edgefm_debug_set_wait_limit(pair.ctx.handle, 1_000_000_000, 0)
+        pair.ctx.prefill_kv(pair.kd, pair.vd)
+        assert expired()
+        pair.ctx.append_kv(32)
+        pair.ctx.next_token.fill_(-7)
+        run()
+        assert expired()
+        assert int(pair.ctx.next_token.item()) == -7              # the step did nothing
+        pair.ctx.append_kv(30)
+        pair.ctx.prefill(list(range(1, 12)), 30)
+        assert expired()
+    finally:
+        torch.cuda.synchronize()
+        pair.close()
+
+
 def test_prefill_contraction_wait_expires_and_is_reported():
     """The same for the contractions of edgefm_prefill: their stage barriers are told to expect an arrival nobody makes and
     the bound is shortened to 2^16 polls; every contraction gives up at its first wait, drains and returns."""

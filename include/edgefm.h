@@ -307,6 +307,19 @@ edgefm_status edgefm_debug_set_prefill_wait(edgefm_ctx *ctx, uint32_t polls, int
  * these split K), 2 = gate/up (always wide, never split).  Host only: for checking the planner without a GPU. */
 edgefm_status edgefm_debug_prefill_plan(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t *out2);
 
+/* Host-only check of the planner: how the step kernel for `tokens` tokens per call (1, 2, 4 or 8) is laid out for a shape on n_sms SMs with
+ * smem_bytes of shared memory per CTA.  out40 = {CTAs, dynamic shared memory, bytes of the ring, bytes of its largest chunk, bytes of the
+ * tables, chunks the list has room for, 1 = a tight build (no list, unit tables in global memory), bytes of these tables, cached
+ * positions per chunk, segments of MLP activations in shared memory, 1 = activations travel as packets, attention outputs per CTA at
+ * most, packets of the activations, packets of a line of the residual stream, of the attention output, then for each operator (QKV, O,
+ * gate/up, down, output layer) its columns, columns of a segment, segments, rows of a box (0: no boxes), units of a tile}.
+ * chunks_out: the chunks CTA `cta` streams of operator `op`, six words each {first part, second part or ~0 (16-byte units from the matrix;
+ * boxes: rows), bytes of a part, 64-column block | rows copied one by one << 16 (255: a box), first unit, units}; NULL to count them
+ * in *n_chunks.  Needs no GPU.  BAD_SHAPE when the shape does not fit. */
+edgefm_status edgefm_debug_step_plan(const edgefm_shape *shape, int32_t max_context, int32_t kv_format, int32_t tokens, int32_t n_sms,
+                                     int32_t smem_bytes, int32_t *out40, int32_t op, int32_t cta, uint32_t *chunks_out, int32_t capacity,
+                                     int32_t *n_chunks);
+
 /* Host-only check of the planner: the tile schedule of one weight-streaming operator (kind: 0 QKV pairs, 1 residual rows,
  * 2 gate/up pairs, 3 output-layer rows; units rows or pairs; K columns; head_half = head_dim / 2 for kind 0) for n_ctas CTAs
  * of n_warps consumer warps whose ring slots hold slot_rows rows.  tiles_out receives one 64-bit descriptor per tile, CTA by

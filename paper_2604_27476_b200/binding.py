@@ -51,7 +51,7 @@ class _Weights(ctypes.Structure):
 
 EXPORTS = ("edgefm_create", "edgefm_prefill_kv", "edgefm_decode_step", "edgefm_destroy", "edgefm_get_length",
            "edgefm_export_kv", "edgefm_get_launches_per_step", "edgefm_last_error", "edgefm_version",
-           "edgefm_sync_status", "edgefm_debug_profile", "edgefm_debug_set_wait_limit", "edgefm_debug_set_prefill_wait", "edgefm_debug_prefill_plan", "edgefm_debug_plan", "edgefm_debug_plan_operator", "edgefm_decode_step_static", "edgefm_set_vocab_subset",
+           "edgefm_sync_status", "edgefm_debug_profile", "edgefm_debug_set_wait_limit", "edgefm_debug_set_prefill_wait", "edgefm_debug_prefill_plan", "edgefm_debug_plan", "edgefm_debug_step_plan", "edgefm_debug_plan_operator", "edgefm_decode_step_static", "edgefm_set_vocab_subset",
            "edgefm_append_kv", "edgefm_create_with_options", "edgefm_export_kv_int8", "edgefm_verify_block", "edgefm_sync_length", "edgefm_prefill_tokens", "edgefm_prefill")
 
 
@@ -105,6 +105,8 @@ def load_library():
     L.edgefm_debug_set_prefill_wait.argtypes = [vp, ctypes.c_uint32, i32]
     L.edgefm_debug_plan.restype = ctypes.c_int
     L.edgefm_debug_plan.argtypes = [vp, ctypes.POINTER(i32)]
+    L.edgefm_debug_step_plan.restype = ctypes.c_int
+    L.edgefm_debug_step_plan.argtypes = [ctypes.POINTER(_Shape)] + [i32] * 5 + [ctypes.POINTER(i32), i32, i32, vp, i32, ctypes.POINTER(i32)]
     L.edgefm_debug_plan_operator.restype = ctypes.c_int
     L.edgefm_debug_plan_operator.argtypes = [i32] * 8 + [vp, i64, vp, vp, i64, vp, vp, ctypes.POINTER(i64), ctypes.POINTER(i64)]
     L.edgefm_decode_step_static.restype = ctypes.c_int
@@ -244,6 +246,30 @@ def edgefm_debug_plan(ctx) -> dict:
     keys = ("ctas", "consumer_warps", "ring_slots_per_warp", "slot_bytes", "dynamic_smem_bytes", "max_tiles_per_cta", "schedule_smem_bytes",
             "long_context_build")
     return dict(zip(keys, list(out)))
+
+
+STEP_PLAN = ("ctas", "dynamic_smem_bytes", "ring_bytes", "max_chunk_bytes", "table_bytes", "list_len", "tight", "unit_table_bytes", "kv_block", "act_slots",
+             "act_packets", "merged_len", "act_len", "x_line", "ao_line")
+
+
+def edgefm_debug_step_plan(shape: dict, max_context, kv_format="bf16", tokens=1, n_sms=148, smem_bytes=232448, op=None, cta=0):
+    """Host only: the step kernel's plan for a shape as a dict (`cols`: per operator its columns, segment, segments, box rows, tile units); with
+    `op`, also the chunks that CTA `cta` streams of that operator, a uint32 array [n][6]."""
+    import numpy as np
+    out, n, sh = (ctypes.c_int32 * 40)(), ctypes.c_int32(), _Shape(**shape)
+
+    def call(at, capacity):
+        _check(load_library().edgefm_debug_step_plan(ctypes.byref(sh), max_context, KV_FORMATS[kv_format], tokens, n_sms, smem_bytes, out, op or 0, cta, at,
+                                                     capacity, ctypes.byref(n)))
+
+    call(None, 0)
+    plan = dict(zip(STEP_PLAN, out[:15]))
+    plan["cols"] = [dict(zip(("K", "seg", "segs", "box_rows", "tile"), out[15 + 5 * o: 20 + 5 * o])) for o in range(5)]
+    if op is None:
+        return plan
+    chunks = np.zeros((n.value, 6), np.uint32)
+    call(chunks.ctypes.data, n.value)
+    return plan, chunks
 
 
 def edgefm_debug_plan_operator(kind, units, K, head_half, op_index, n_ctas, n_warps, slot_rows):

@@ -249,14 +249,19 @@ cudaError_t run_step(edgefm_ctx::Build *b, const StepRequest &r, cudaStream_t s)
     return launch_step(b->launch, s);
 }
 
-// Zeroed exchange buffers and tensor maps of a build, complete when the call returns: the first launch may go to any stream, and work on the
-// legacy stream is ordered against neither a non-blocking one nor the return of a pageable copy.
-cudaError_t init_build(void *ll, size_t ll_bytes, void *maps, const void *host_maps, size_t map_bytes) {
+// Zeroed exchange buffers (with unit tables) and tensor maps of a build, complete when the call returns: the first launch may go to any stream,
+// and work on the legacy stream is ordered against neither a non-blocking one nor the return of a pageable copy.
+cudaError_t init_build(const StepLaunch &sl, void *ll, void *maps, const void *host_maps, size_t map_bytes) {
     cudaStream_t own = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(ll, 0, ll_bytes, own);
+    std::vector<unsigned> units(sl.unit_tab_bytes / 4);
+    e = cudaMemsetAsync(ll, 0, sl.ll_bytes, own);
     if (e == cudaSuccess) e = cudaMemcpyAsync(maps, host_maps, map_bytes, cudaMemcpyHostToDevice, own);
+    if (e == cudaSuccess && !units.empty()) {
+        step_unit_table(sl, units.data());
+        e = cudaMemcpyAsync(const_cast<unsigned *>(sl.p.unit_tab), units.data(), sl.unit_tab_bytes, cudaMemcpyHostToDevice, own);
+    }
     const cudaError_t done = cudaStreamSynchronize(own);
     cudaStreamDestroy(own);
     return e != cudaSuccess ? e : done;
@@ -277,7 +282,7 @@ cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char *
         const bool sub = c->vocab_subset > 0;
         if (!step_maps(p, c->layers.data(), sub ? static_cast<const void *>(c->sub_lm) : c->lm_head, sub ? c->vocab_subset : c->shape.vocab, maps.data())) return cudaErrorUnknown;
         if (!b->maps && (e = cudaMalloc(reinterpret_cast<void **>(&b->maps), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
-        if ((e = init_build(b->ll, sl.ll_bytes, b->maps, maps.data(), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
+        if ((e = init_build(sl, b->ll, b->maps, maps.data(), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
         p.maps = b->maps;
         p.map_fence = 1;   // edgefm_set_vocab_subset rewrites the output layer's map
     }
@@ -989,7 +994,10 @@ extern "C" edgefm_status edgefm_decode_step_static(const edgefm_shape *shape, co
     st.cur_len = cur_len; st.next_position = position;
     // no packet of an earlier call (of any shape) may carry a tag of this one
     CUDA_TRY(nullptr, cudaMemsetAsync(ll, 0, sl.ll_bytes, s));
+    std::vector<unsigned> units(sl.unit_tab_bytes / 4);
+    if (!units.empty()) step_unit_table(sl, units.data());
     // pageable copies: the runtime stages the bytes before returning, so the sources may be freed after the call
+    if (!units.empty()) CUDA_TRY(nullptr, cudaMemcpyAsync(const_cast<unsigned *>(p.unit_tab), units.data(), sl.unit_tab_bytes, cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(d_layers, layers.data(), layers.size() * sizeof(StepLayer), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, s));
     CUDA_TRY(nullptr, cudaMemcpyAsync(inv_freq, inv, static_cast<size_t>(d / 2) * sizeof(double), cudaMemcpyHostToDevice, s));
@@ -1025,6 +1033,29 @@ extern "C" edgefm_status edgefm_sync_status(edgefm_ctx *ctx, void *stream) {
     if (st.status != 0)
         return fail(ctx, EDGEFM_ERR_TIMEOUT, "device status %d (6 = a bounded wait expired, 100+ = self-check code) operands %d %d; "
                     "the context must be destroyed", st.status, st.pad[0], st.pad[1]);
+    return EDGEFM_OK;
+}
+
+// Host-only diagnostics: the plan of the step kernel for a shape, and the chunks one CTA streams of one operator, with the kernel's own arithmetic.
+extern "C" edgefm_status edgefm_debug_step_plan(const edgefm_shape *shape, int32_t max_context, int32_t kv_format, int32_t tokens, int32_t n_sms, int32_t smem_bytes,
+                                                int32_t *out40, int32_t op, int32_t cta, uint32_t *chunks_out, int32_t capacity, int32_t *n_chunks) {
+    if (!shape || !out40 || !n_chunks || max_context < 1 || n_sms < 1 || op < 0 || op > ST_LM || cta < 0) return fail(nullptr, EDGEFM_ERR_INVALID_ARG, "bad argument");
+    const edgefm_shape &sh = *shape;
+    if (sh.n_layers < 1 || sh.hidden < 8 || sh.hidden % 8 || sh.ffn < 8 || sh.ffn % 8 || (sh.head_dim != 64 && sh.head_dim != 128) || sh.n_q_heads < 1 || sh.n_kv_heads < 1 ||
+        sh.n_q_heads % sh.n_kv_heads || sh.n_q_heads / sh.n_kv_heads > 8 || sh.vocab < 1)
+        return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "unsupported model shape");
+    StepLaunch sl;
+    if (const char *why = step_plan(sh, max_context, n_sms, smem_bytes, kv_format == EDGEFM_KV_INT8, tokens, &sl)) return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "%s", why);
+    const StepParams &p = sl.p;
+    const int32_t head[15] = {sl.grid, static_cast<int32_t>(sl.dyn_smem), p.ring_bytes, sl.max_chunk_bytes, p.table_bytes, sl.list_len, sl.list_len == 0, static_cast<int32_t>(sl.unit_tab_bytes),
+                              p.kv_block, p.act_slots, p.act_packets, p.merged_len, p.act_len, p.x_line, p.ao_line};
+    std::copy(head, head + 15, out40);
+    for (int o = 0; o < 5; ++o) {
+        const StepCols &c = p.cols[o];
+        const int32_t v[5] = {c.K, c.seg, c.segs, c.box_rows, c.tile};
+        std::copy(v, v + 5, out40 + 15 + 5 * o);
+    }
+    *n_chunks = cta < sl.grid ? step_chunks(sl, op, cta, chunks_out, chunks_out ? capacity : 0) : 0;
     return EDGEFM_OK;
 }
 

@@ -3,7 +3,7 @@
 #include "step_products.cuh"
 
 namespace edgefm {
-namespace step {
+namespace ST_NS {
 
 // The group's heads are the rows of tensor-core products: scores[head][position] = Q K^T takes the 8 heads' first two bf16 pieces as rows
 // 0-7 and 8-15 of one m16n8k16 and the third as the rows of another (24 bits of the query, as the fp32 query it was), and
@@ -289,10 +289,10 @@ __device__ __forceinline__ bool attend(Ctx<MT> &c, int layer, const KvShare &sha
     const int my_tile = c.warp / W::WD, dg = c.warp & (W::WD - 1), quad = c.lane & 3;
     // (the new rows come last, by the last warps of the CTA that ends with them)
 #pragma unroll 1
-    for (int t = share.t0;; t += kv_block(D)) {
+    for (int t = share.t0;; t += kv_positions(p, D)) {
         const bool fresh = t >= share.t1;
         if (fresh && n_new == 0) break;
-        KvBlock b(fresh ? n_new : min(kv_block(D), share.t1 - t), W::ROW);
+        KvBlock b(fresh ? n_new : min(kv_positions(p, D), share.t1 - t), W::ROW);
         const int i = fresh ? ST_NW / W::WD - 1 - my_tile : my_tile, own = quad * b.R + 4 * i;
         const bool on = 4 * i < b.R;
         float ks[4] = {0.f, 0.f, 0.f, 0.f}, vs[4] = {0.f, 0.f, 0.f, 0.f};
@@ -413,7 +413,7 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
             a += __shfl_xor_sync(0xffffffffu, a, k);
             b += __shfl_xor_sync(0xffffffffu, b, k);
         }
-        if (on && sub == 0) *reinterpret_cast<float2 *>(&c.sh().merged[tok][2 * k_pair]) = make_float2(a / l, b / l);
+        if (on && sub == 0) *reinterpret_cast<float2 *>(c.merged(tok) + 2 * k_pair) = make_float2(a / l, b / l);
     }
     if (!cta_vote(ok)) return false;
     if constexpr (st_packets(MT)) {
@@ -422,7 +422,7 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
 #pragma unroll 1
         for (int i = c.tid; i < n_pairs * MT; i += ST_NT) {        // (unused tokens too: their slots keep up with the tags)
             const int tok = i / n_pairs, k = i - tok * n_pairs;
-            const float2 v = tok < m ? *reinterpret_cast<const float2 *>(&c.sh().merged[tok][2 * k]) : make_float2(0.f, 0.f);
+            const float2 v = tok < m ? *reinterpret_cast<const float2 *>(c.merged(tok) + 2 * k) : make_float2(0.f, 0.f);
             put_raw2(p.ao_ll + (static_cast<size_t>(tok) * c.ncta + c.cta) * p.ao_line + 2 * k, pieces_packet(v.x, real_tag), pieces_packet(v.y, real_tag));
         }
     } else {
@@ -430,11 +430,11 @@ __device__ __forceinline__ bool merge_chunks(Ctx<MT> &c, unsigned tag) {
 #pragma unroll 1
         for (int i = c.tid; i < 2 * n_pairs * m; i += ST_NT) {
             const int tok = i / (2 * n_pairs), k = i - tok * 2 * n_pairs;
-            store_pieces<MT>(p.ao_vec, tok, 2 * a0 + k, stride, c.sh().merged[tok][k]);
+            store_pieces<MT>(p.ao_vec, tok, 2 * a0 + k, stride, c.merged(tok)[k]);
         }
     }
     return true;
 }
 
-}  // namespace step
+}  // namespace ST_NS
 }  // namespace edgefm

@@ -3,7 +3,7 @@
 #include "step_attention.cuh"
 
 namespace edgefm {
-namespace step {
+namespace ST_NS {
 
 // The order of the chunks is the same in every layer, so every CTA lists them once per launch (the feeding thread's time per chunk
 // bounds the stream: with the addresses derived chunk by chunk it took about 1000 cycles from a freed slot to the next copy, and
@@ -12,8 +12,7 @@ namespace step {
 //   z: bytes of a part
 //   w: 64-column block of a box | rows << 16, the row segments copied one by one (0: one copy; boxes: ST_BOX)
 constexpr unsigned ST_BOX = 255u;
-template <int MT> __device__ __forceinline__ uint4 chunk_entry(const Ctx<MT> &c, int op, int u, int n, int seg_i) {
-    const StepParams &p = c.p();
+__host__ __device__ __forceinline__ uint4 chunk_entry(const StepParams &p, int op, int u, int n, int seg_i) {
     const StepCols &cols = p.cols[op];
     const int half = 1 << p.half_shift;
     const unsigned row = static_cast<unsigned>(op == ST_QKV ? (u >> p.half_shift) * p.D + (u & (half - 1)) : u), partner = row + static_cast<unsigned>(op == ST_QKV ? half : p.F);
@@ -34,7 +33,7 @@ template <int MT> __device__ __forceinline__ void make_list(const Ctx<MT> &c) {
     for (int u = sh.u0[ST_QKV]; u < sh.u1[ST_QKV];) {
         const int n = tile_units(p, ST_QKV, u, sh.u1[ST_QKV]);
         for (int s = 0; s < p.cols[ST_QKV].segs; ++s, ++at)
-            if (tid == at % THREADS) c.list()[at] = chunk_entry(c, ST_QKV, u, n, s);
+            if (tid == at % THREADS) c.list()[at] = chunk_entry(p, ST_QKV, u, n, s);
         u += n;
     }
     for (int op = ST_O; op <= ST_LM; ++op) {
@@ -42,7 +41,7 @@ template <int MT> __device__ __forceinline__ void make_list(const Ctx<MT> &c) {
         if (tid == 0) sh.list[op] = at;
         for (int i = tid; i < count; i += THREADS) {
             const int k = i / segs, u = u0 + k * tile;
-            c.list()[at + i] = chunk_entry(c, op, u, min(tile, u1 - u), i - k * segs);
+            c.list()[at + i] = chunk_entry(p, op, u, min(tile, u1 - u), i - k * segs);
         }
         at += count;
     }
@@ -56,7 +55,7 @@ __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f, FKV f_kv) 
     const StepParams &p = c.p();
     const uint4 *const list = c.list();
     constexpr int E = Q8 ? 1 : 2;
-    const int block = kv_block(p.D), row_bytes = p.D * E;
+    const int block = kv_positions(p, p.D), row_bytes = p.D * E;
     const int shares = sh.m * p.nkv * sh.n_chunks;
     const unsigned char *map = p.maps;
 #pragma unroll 1
@@ -84,10 +83,21 @@ __device__ __forceinline__ void for_each_chunk(const Ctx<MT> &c, F f, FKV f_kv) 
             // (the first four pointers of a layer are its matrices in this order; the output layer's entry begins with its matrix)
             const unsigned char *base = lm ? reinterpret_cast<const unsigned char *>(c.head().lm_head)
                                            : reinterpret_cast<const unsigned char *>(reinterpret_cast<const uint16_t *const *>(L)[op]);
-            const int end = sh.list[op + 1];
+            if constexpr (TIGHT) {                              // (no list)
+                int n;
 #pragma unroll 1
-            for (int i = sh.list[op]; i < end; ++i)
-                if (!f(base, list[i], map)) return;
+                for (int u = sh.u0[op]; u < sh.u1[op]; u += n) {
+                    n = tile_units(p, op, u, sh.u1[op]);
+#pragma unroll 1
+                    for (int seg = 0; seg < p.cols[op].segs; ++seg)
+                        if (!f(base, chunk_entry(p, op, u, n, seg), map)) return;
+                }
+            } else {
+                const int end = sh.list[op + 1];
+#pragma unroll 1
+                for (int i = sh.list[op]; i < end; ++i)
+                    if (!f(base, list[i], map)) return;
+            }
             map += 128;
         }
     }
@@ -298,5 +308,5 @@ __device__ __forceinline__ void feed_vectors(Ctx<MT> &c) {
     drain(sh.x_full, 4u, k);
 }
 
-}  // namespace step
+}  // namespace ST_NS
 }  // namespace edgefm

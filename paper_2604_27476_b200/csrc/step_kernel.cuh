@@ -38,7 +38,7 @@
 #include "step_products.cuh"
 
 namespace edgefm {
-namespace step {
+namespace ST_NS {
 
 // The epilogue of output unit j of token `tok` (its row sum, or the sums of its two rows) of the QKV, gate/up and output layer operators.
 template <int D, bool Q8, int MT>
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
     }
     if (c.warp >= ST_NW) {               // the feeding warpgroup: gives its registers to the others
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ST_REGS_FEED));
-        make_list(c);
+        if constexpr (!TIGHT) make_list(c);
         if (c.warp == ST_NW && c.lane == 0) feed_ring<Q8, MT>(c);
         if (c.warp == ST_NW + 1 && c.lane == 0) feed_l2<Q8, MT>(c);
         if (c.warp == ST_NW + 2 && c.lane == 0 && !(st_packets(MT) && p.act_packets)) feed_vectors<MT>(c);
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             sh.rope[t][half + f] = static_cast<float>(sn);
         }
         if (c.cta == 0 && c.tid == 0) { p.state->token = sh.tokens[0]; p.state->position = sh.pos; }
-        if constexpr (st_packets(MT)) {
+        if constexpr (st_packets(MT) && !TIGHT) {
             const int threads = (ST_NW - rw) * 32, first = c.tid - rw * 32;
             if (first >= 0) {
                 make_table(c, c.unit_table(), p.H, 1, p.x_line, first, threads);
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) step_kernel(const __grid_consta
             if (st_packets(MT) && p.act_packets) ok = stage_activations(c, tag);
         } else if constexpr (st_packets(MT)) {        // (one call for the three exchanges: the loop's code has to stay small)
             const bool ao = op == ST_O, gu = op == ST_GU;
-            ok = stage_lines(c, c.unit_table() + (ao ? sh.total_x : 0), ao ? sh.total_a : sh.total_x, ao ? p.qd : p.H, ao ? p.ao_ll : gu ? p.xo_ll : p.x_ll,
+            ok = stage_lines(c, (TIGHT ? p.unit_tab : c.unit_table()) + (ao ? sh.total_x : 0), ao ? sh.total_a : sh.total_x, ao ? p.qd : p.H, ao ? p.ao_ll : gu ? p.xo_ll : p.x_ll,
                              ao ? p.ao_line : p.x_line, !ao, ao || gu ? tag : (real_tag - 1u) ^ sh.odd);
         } else {
             ok = stage_vector(c, op != ST_O);         // (of this warp; the vote follows the products)
@@ -371,5 +371,5 @@ StepKernel kernel_for(int G) {
     }
 }
 
-}  // namespace step
+}  // namespace ST_NS
 }  // namespace edgefm

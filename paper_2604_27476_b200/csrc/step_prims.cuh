@@ -2,8 +2,23 @@
 #pragma once
 #include "step_types.h"
 
+// These headers are built twice.  ST_TIGHT: for shapes that leave the shared memory no room for the tables and the chunk list, or for chunks of
+// the usual size.  (As run-time choices in the one kernel they cost every shape 1 - 4 %.)
+#ifndef ST_TIGHT
+#define ST_TIGHT 0
+#endif
+#if ST_TIGHT
+#define ST_NS step_tight
+#else
+#define ST_NS step
+#endif
+
 namespace edgefm {
-namespace step {
+namespace ST_NS {
+
+constexpr bool TIGHT = ST_TIGHT != 0;
+constexpr int ROW_BITS = TIGHT ? ST_TIGHT_ROW_BITS : 16;     // of a unit table's entry: row | values << ROW_BITS | unit << (ROW_BITS + 2)
+__device__ __forceinline__ int kv_positions(const StepParams &p, int D) { return TIGHT ? p.kv_block : kv_block(D); }   // cached positions per ring chunk
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return static_cast<unsigned>(__cvta_generic_to_shared(p)); }
 __device__ __forceinline__ void mbar_init(unsigned long long *b, unsigned count) {
@@ -147,7 +162,7 @@ template <int MT> struct Shared {
     float rope[MT][128];                                   // per token: cos | sin of its position
     float ss[MT];                                          // sums of squares (RMSNorm)
     alignas(16) float part[2][MT * st_batch(MT) * ST_NW];  // partial row sums [token][row][warp], two batches
-    alignas(16) float merged[MT][128];                     // attention outputs this CTA owns
+    alignas(16) float merged[MT][128];                     // attention outputs this CTA owns (Ctx::merged)
     float best_v[ST_NW];
     int best_i[ST_NW];
     int u0[5], u1[5];                                      // this CTA's units of every operator
@@ -181,6 +196,9 @@ template <int MT> struct Ctx {
     __device__ __forceinline__ unsigned *unit_table() const { return reinterpret_cast<unsigned *>(tables() + (p().n_layers + 1) * 64); }
     __device__ __forceinline__ uint4 *list() const { return reinterpret_cast<uint4 *>(tables() + p().list_at); }           // chunk list
     __device__ __forceinline__ float *resid() const { return reinterpret_cast<float *>(tables() + p().resid_at); }   // [token][this CTA's rows of the residual stream]
+    __device__ __forceinline__ float *merged(int tok) const {      // attention outputs this CTA owns
+        return TIGHT ? reinterpret_cast<float *>(tables() + p().merged_at) + tok * p().merged_len : sh().merged[tok];
+    }
     __device__ __forceinline__ unsigned char *area() const { return tables() + p().table_bytes; }
 };
 
@@ -249,7 +267,7 @@ template <int MT> __device__ __forceinline__ void x_release(Ctx<MT> &c) {
 }
 
 // ---- the order of the stream (the same arithmetic on the feeding and on the consuming side) --------------------------------
-__device__ __forceinline__ int op_units(const StepParams &p, int op, int lm_rows) {
+__host__ __device__ __forceinline__ int op_units(const StepParams &p, int op, int lm_rows) {
     switch (op) {
         case ST_QKV: return (p.nq + 2 * p.nkv) << p.half_shift;
         case ST_GU: return p.F;
@@ -257,9 +275,9 @@ __device__ __forceinline__ int op_units(const StepParams &p, int op, int lm_rows
         default: return p.H;
     }
 }
-__device__ __forceinline__ bool op_paired(int op) { return op == ST_QKV || op == ST_GU; }
+__host__ __device__ __forceinline__ bool op_paired(int op) { return op == ST_QKV || op == ST_GU; }
 // Units of the tile that starts at unit u of [.., u1).
-__device__ __forceinline__ int tile_units(const StepParams &p, int op, int u, int u1) {
+__host__ __device__ __forceinline__ int tile_units(const StepParams &p, int op, int u, int u1) {
     int n = min(p.cols[op].tile, u1 - u);
     if (op == ST_QKV) n = min(n, (1 << p.half_shift) - (u & ((1 << p.half_shift) - 1)));   // rows of one head are contiguous, heads are not
     return n;
@@ -279,5 +297,5 @@ __device__ __forceinline__ KvShare kv_share(const StepParams &p, int n, int n_ch
     return s;
 }
 
-}  // namespace step
+}  // namespace ST_NS
 }  // namespace edgefm

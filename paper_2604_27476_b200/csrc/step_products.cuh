@@ -3,7 +3,7 @@
 #include "step_prims.cuh"
 
 namespace edgefm {
-namespace step {
+namespace ST_NS {
 
 // First operator of the step: the embedding rows are the residual streams; this CTA keeps its rows [x0, x0 + my_rows) of them.
 // (The loads of U columns are under way together: one by one they took a trip to HBM each, 4 us for 1536 columns.)
@@ -60,8 +60,8 @@ template <int MT> __device__ __forceinline__ bool stage_vector(Ctx<MT> &c, bool 
 }
 
 // ---- exchanges: everybody reads a vector that lies in lines ---------------------------------------------------------------
-// Table of the 16-byte units of such a vector: row | values << 16 | unit << 18 (unit = index of the packet pair).
-// The tables of the residual stream and of the attention output stand in shared memory, made once per launch.
+// Table of the 16-byte units of such a vector: row | values | unit (unit = index of the packet pair).  The tables of the residual stream and of
+// the attention output stand in shared memory, made once per launch (tight builds: in global memory, made by the host).
 __device__ __forceinline__ int line_units(int n, int ncta, int grain) { return ((n / grain + ncta - 1) / ncta * grain + 1) / 2; }
 // By `threads` threads, this one the `first`: a line each.
 template <int MT> __device__ __forceinline__ void make_table(const Ctx<MT> &c, unsigned *tab, int n, int grain, int line, int first, int threads) {
@@ -72,7 +72,7 @@ template <int MT> __device__ __forceinline__ void make_table(const Ctx<MT> &c, u
         const int r1 = st_first(n / grain, w + 1, c.ncta) * grain;
 #pragma unroll 1
         for (int e = 0; e < upl; ++e, row += 2)
-            tab[w * upl + e] = static_cast<unsigned>(row & 0xffff) | static_cast<unsigned>(max(0, min(2, r1 - row))) << 16 | static_cast<unsigned>(w * (line >> 1) + e) << 18;
+            tab[w * upl + e] = static_cast<unsigned>(row & ((1 << ROW_BITS) - 1)) | static_cast<unsigned>(max(0, min(2, r1 - row))) << ROW_BITS | static_cast<unsigned>(w * (line >> 1) + e) << (ROW_BITS + 2);
     }
 }
 // Wait for all values of the vectors of all tokens (K columns, lines of `line` packets) and leave their pieces in shared memory, and meet.
@@ -105,9 +105,9 @@ __device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int
             int tok = 0;
             if constexpr (MT > 1) tok = u / total;
             e[i] = u < all ? tab[u - tok * total] : 0u;
-            at[i] = (e[i] >> 18) * 2 + static_cast<unsigned>(tok * c.ncta * line);
-            e[i] = (e[i] & 0x3ffffu) | static_cast<unsigned>(tok) << 18;
-            if ((e[i] >> 16) & 3u) todo |= 1u << i;
+            at[i] = (e[i] >> (ROW_BITS + 2)) * 2 + static_cast<unsigned>(tok * c.ncta * line);
+            e[i] = (e[i] & ((4u << ROW_BITS) - 1u)) | static_cast<unsigned>(tok) << (ROW_BITS + 2);
+            if ((e[i] >> ROW_BITS) & 3u) todo |= 1u << i;
         }
         Spin sp;
         for (;;) {
@@ -117,10 +117,10 @@ __device__ __forceinline__ bool stage_lines(Ctx<MT> &c, const unsigned *tab, int
 #pragma unroll
             for (int i = 0; i < U; ++i)
                 if (todo >> i & 1u) {
-                    const bool two = (e[i] >> 16 & 3u) > 1;
+                    const bool two = (e[i] >> ROW_BITS & 3u) > 1;
                     if (pieces_tag(t[i].a, tag) && (!two || pieces_tag(t[i].b, tag))) {
                         todo &= ~(1u << i);
-                        const int row = e[i] & 0xffffu, tok = static_cast<int>(e[i] >> 18);
+                        const int row = e[i] & ((1u << ROW_BITS) - 1u), tok = static_cast<int>(e[i] >> (ROW_BITS + 2));
                         store_packet<MT>(c.area(), tok, row, stride, t[i].a);
                         if (two) store_packet<MT>(c.area(), tok, row + 1, stride, t[i].b);
                     }
@@ -393,5 +393,5 @@ template <int MT> __device__ __forceinline__ bool multiply_any(Ctx<MT> &c, const
     }
 }
 
-}  // namespace step
+}  // namespace ST_NS
 }  // namespace edgefm

@@ -1,5 +1,6 @@
 // The builds of the decode-step kernel and what the host has to know about them.
 #include "step_attention.cuh"
+#include "step_feed.cuh"
 
 namespace edgefm {
 StepKernel step_d64_m1(int G);
@@ -14,8 +15,25 @@ StepKernel step_d128_m4(int G);
 StepKernel step_d128_m8(int G);
 StepKernel step_q8_d128_m1(int G);
 StepKernel step_q8_d128_m8(int G);
+StepKernel step_tight_d64_m1(int G);
+StepKernel step_tight_d64_m2(int G);
+StepKernel step_tight_d64_m4(int G);
+StepKernel step_tight_q8_d64_m1(int G);
+StepKernel step_tight_d128_m1(int G);
+StepKernel step_tight_d128_m2(int G);
+StepKernel step_tight_d128_m4(int G);
+StepKernel step_tight_q8_d128_m1(int G);
 
-StepKernel step_kernel_for(int D, int G, bool kv8, int mt) {
+StepKernel step_kernel_for(int D, int G, bool kv8, int mt, bool tight) {
+    if (tight) {
+        if (kv8) return mt != 1 ? nullptr : D == 64 ? step_tight_q8_d64_m1(G) : step_tight_q8_d128_m1(G);
+        switch (mt) {
+            case 1: return D == 64 ? step_tight_d64_m1(G) : step_tight_d128_m1(G);
+            case 2: return D == 64 ? step_tight_d64_m2(G) : step_tight_d128_m2(G);
+            case 4: return D == 64 ? step_tight_d64_m4(G) : step_tight_d128_m4(G);
+            default: return nullptr;
+        }
+    }
     if (kv8) {
         if (mt == 1) return D == 64 ? step_q8_d64_m1(G) : step_q8_d128_m1(G);
         if (mt == 8) return D == 64 ? step_q8_d64_m8(G) : step_q8_d128_m8(G);
@@ -48,4 +66,19 @@ template <int D, int MT> static int scratch(int G) {
 }
 template <int D> static int scratch_of(int G, int mt) { return mt == 1 ? scratch<D, 1>(G) : mt == 2 ? scratch<D, 2>(G) : mt == 4 ? scratch<D, 4>(G) : scratch<D, 8>(G); }
 int step_scratch_floats(int D, int G, int mt) { return D == 64 ? scratch_of<64>(G, mt) : scratch_of<128>(G, mt); }
+int step_chunks(const StepLaunch &sl, int op, int cta, unsigned *out, int capacity) {
+    const StepParams &p = sl.p;
+    const int units = step::op_units(p, op, p.V);
+    int at = 0;
+    for (int u = st_first(units, cta, sl.grid), u1 = st_first(units, cta + 1, sl.grid), n; u < u1; u += n) {
+        n = step::tile_units(p, op, u, u1);
+        for (int s = 0; s < p.cols[op].segs; ++s, ++at) {
+            if (at >= capacity) continue;
+            const uint4 e = step::chunk_entry(p, op, u, n, s);
+            const unsigned v[6] = {e.x, e.y, e.z, e.w, static_cast<unsigned>(u), static_cast<unsigned>(n)};
+            std::copy(v, v + 6, out + 6 * static_cast<size_t>(at));
+        }
+    }
+    return at;
+}
 }  // namespace edgefm

@@ -113,22 +113,26 @@ struct StepParams {
     unsigned spin_limit;           // upper bound of every device-side wait, nanoseconds
     unsigned long long *prof;      // optional timestamps [gridDim.x][prof_stride]
     int prof_stride;
+    // tight builds only
+    int kv_block;                  // cached positions per ring chunk
+    const unsigned *unit_tab;      // unit tables of the lines (residual stream, attention output)
+    int merged_at, merged_len;     // attention outputs of this CTA: inside the tables; at most per token
 };
 
 using StepKernel = void (*)(const StepParams);
-// one kernel per head size, query heads per kv head, cache format and tokens per call (null: not built)
-StepKernel step_kernel_for(int D, int G, bool kv8, int mt);
+// one kernel per head size, query heads per kv head, cache format, tokens per call and room in shared memory (null: not built)
+StepKernel step_kernel_for(int D, int G, bool kv8, int mt, bool tight);
 // First unit (of n) of CTA c (n * ncta below 2^32: checked by step_plan; a 64-bit division would cost the feeding thread more than a copy).
 __host__ __device__ inline int st_first(int n, int c, int ncta) { return static_cast<int>(static_cast<unsigned>(n) * static_cast<unsigned>(c) / static_cast<unsigned>(ncta)); }
 __host__ __device__ inline int st_line(int most) { return (most + 15) / 16 * 16; }   // packets of a line: whole 128 bytes
 
 // How an operator with rows of K values is cut of which a CTA owns at most `most` units (rows, or pairs).
-inline StepCols step_cols(int K, int most, bool paired, int max_seg = 1 << 30, int chunk_bytes = ST_CHUNK_BYTES) {
+inline StepCols step_cols(int K, int most, bool paired, int max_seg, int chunk_bytes, int chunk_whole) {
     const int full = paired ? ST_TILE / 2 : ST_TILE, per_unit = paired ? 4 * K : 2 * K;     // bytes
     StepCols c{K, K, 1, 0, full};
-    if (K <= max_seg && std::min(most, full) * per_unit <= ST_CHUNK_WHOLE) return c;
+    if (K <= max_seg && std::min(most, full) * per_unit <= chunk_whole) return c;
     c.tile = full / 2;
-    if (K <= max_seg && c.tile * per_unit <= ST_CHUNK_WHOLE && K <= ST_KEEP_HALF * ST_NW * 64) return c;
+    if (K <= max_seg && c.tile * per_unit <= chunk_whole && K <= ST_KEEP_HALF * ST_NW * 64) return c;
     const int tiles = (most + full - 1) / full;
     c.tile = (most + tiles - 1) / tiles;
     const int rows = paired ? 2 * c.tile : c.tile;
@@ -148,11 +152,15 @@ struct StepLaunch {
     StepParams p{};
     int grid = 0;
     size_t dyn_smem = 0;
-    size_t ll_bytes = 0;        // exchange buffers (zeroed once: tag 0 is never used, columns past K stay zero)
+    size_t ll_bytes = 0;        // exchange buffers (zeroed once: tag 0 is never used, columns past K stay zero), then the unit tables of a tight build
+    size_t unit_tab_bytes = 0;  // unit tables in global memory (0: in shared memory)
     int max_chunk_bytes = 0;
+    int list_len = 0;           // chunks the list in shared memory has room for
 };
 int step_shared_bytes(int mt);  // fixed part of the kernel's shared memory
 int step_scratch_floats(int D, int G, int mt);
+// The chunks CTA `cta` streams of an operator, six words each: the entry (chunk_entry), first unit, units.  Returns how many there are.
+int step_chunks(const StepLaunch &sl, int op, int cta, unsigned *out, int capacity);
 
 // Packets of the attention's maxima and denominators; whole lines (what follows is lines with one writer each: 64 bytes off, two share one).
 inline size_t step_stat_len(size_t chunks, int nq) { return (chunks * nq * 2 + 15) / 16 * 16; }
@@ -163,16 +171,24 @@ inline size_t step_vec_bytes(const StepParams &p, int mt, int K, bool sums) {
 inline size_t step_act_bytes(const StepParams &p, int mt) {
     return (static_cast<size_t>(p.cols[ST_DN].segs) * st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg) + 127) / 128 * 128;
 }
+// What a plan asks of the shared memory.  The first form suits every shape in use.  The tight ones give up speed for room where a CTA owns more than
+// 128 attention outputs, or vectors, rows or the vocabulary are so long that it does not fit: tables and chunk list out of shared
+// memory, then smaller chunks, then fewer cached positions per chunk.
+struct StepRoom { bool tight; int chunk_bytes, chunk_small, chunk_whole, kv_share; };
+constexpr StepRoom ST_ROOM[] = {{false, ST_CHUNK_BYTES, ST_CHUNK_SMALL, ST_CHUNK_WHOLE, 1}, {true, ST_CHUNK_BYTES, ST_CHUNK_SMALL, ST_CHUNK_WHOLE, 1},
+                                {true, 32 * 1024, ST_CHUNK_SMALL, 32 * 1024, 1}, {true, 16 * 1024, 16 * 1024, 16 * 1024, 2}};
+constexpr int ST_TIGHT_ROW_BITS = 15;     // row of an entry of the tight builds' unit tables
+
 // Shared-memory split and exchange buffers for a model shape.  Returns null, or why the shape does not fit.
-inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, bool kv8, int mt, StepLaunch *sl) {
+inline const char *step_plan_in(const StepRoom &room, const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, bool kv8, int mt, StepLaunch *sl) {
     const int H = sh.hidden, D = sh.head_dim, nq = sh.n_q_heads, nkv = sh.n_kv_heads, F = sh.ffn, qd = nq * D, G = nq / nkv;
     StepParams &p = sl->p;
-    sl->kernel = step_kernel_for(D, G, kv8, mt);
+    sl->kernel = step_kernel_for(D, G, kv8, mt, room.tight);
     if (!sl->kernel) return "no step kernel for this combination of options";
     // every CTA must own a row of the residual stream: its contribution is what says that it has read the exchange before
     const int grid = sl->grid = std::min(num_sms, H);
     const long long units = std::max({static_cast<long long>(sh.vocab), static_cast<long long>(F), static_cast<long long>(nq + 2 * nkv) * D / 2, static_cast<long long>(max_context)});
-    if (qd > 128 * grid || (units + 1) * (grid + 1) > 0x7fffffffLL) return "model shape does not fit the step kernel";
+    if ((!room.tight && qd > 128 * grid) || (units + 1) * (grid + 1) > 0x7fffffffLL) return "model shape does not fit the step kernel";
     p.n_layers = sh.n_layers; p.H = H; p.nq = nq; p.nkv = nkv; p.G = G; p.D = D; p.F = F; p.V = sh.vocab; p.qd = qd;
     p.half_shift = D == 64 ? 5 : 6;
     p.eps = sh.rms_eps;
@@ -180,26 +196,31 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.max_context = max_context;
     auto most = [&](int n) { return (n + grid - 1) / grid; };
     const int q_most = most((nq + 2 * nkv) * D / 2);
-    p.cols[ST_QKV] = step_cols(H, q_most, true);
-    p.cols[ST_GU] = step_cols(H, most(F), true);
-    p.cols[ST_LM] = step_cols(H, most(sh.vocab), false);
-    p.cols[ST_O] = step_cols(qd, most(H), false);
+    p.cols[ST_QKV] = step_cols(H, q_most, true, 1 << 30, room.chunk_bytes, room.chunk_whole);
+    p.cols[ST_GU] = step_cols(H, most(F), true, 1 << 30, room.chunk_bytes, room.chunk_whole);
+    p.cols[ST_LM] = step_cols(H, most(sh.vocab), false, 1 << 30, room.chunk_bytes, room.chunk_whole);
+    p.cols[ST_O] = step_cols(qd, most(H), false, 1 << 30, room.chunk_bytes, room.chunk_whole);
     // the activations whole if they leave the ring room to cover the latency of HBM (7B: 113 KB for them, and the stream fell to 3.9 TB/s)
     p.act_packets = st_packets(mt) && st_arrays(mt) * st_array_bytes(F) <= ST_ACT_WHOLE;
     p.cols[ST_DN] = step_cols(F, most(H), false, mt <= 2 ? 2048 : 1024,       // (two segments of activations are in shared memory, as pieces)
-                              p.act_packets ? ST_CHUNK_SMALL : ST_CHUNK_BYTES);
+                              p.act_packets ? room.chunk_small : room.chunk_bytes, room.chunk_whole);
     p.q_line = st_line(2 * most((nq + 2 * nkv) * D / 2));
     p.ss_stride = (grid + 3) / 4 * 4;
     p.x_line = st_line(most(H) + 1);
     p.ao_line = st_line(2 * most(qd / 2));
     p.act_len = (F + 15) / 16 * 16;
-    const int total_x = grid * ((most(H) + 1) / 2), total_a = grid * most(qd / 2);
-    if (st_packets(mt) && (H >= 65536 || qd >= 65536 || grid * p.x_line / 2 >= 16384 || grid * p.ao_line / 2 >= 16384)) return "model shape does not fit the step kernel";
-    p.list_at = ((sh.n_layers + 1) * 64 + (st_packets(mt) ? 4 * (total_x + total_a) : 0) + 15) / 16 * 16;
+    const int total_x = grid * ((most(H) + 1) / 2), total_a = grid * most(qd / 2), row_bits = room.tight ? ST_TIGHT_ROW_BITS : 16, rows = 1 << row_bits, lines = 1 << (30 - row_bits);
+    if (st_packets(mt) && (H >= rows || qd >= rows || grid * p.x_line / 2 >= lines || grid * p.ao_line / 2 >= lines)) return "model shape does not fit the step kernel";
+    const int unit_bytes = st_packets(mt) ? 4 * (total_x + total_a) : 0;
+    sl->unit_tab_bytes = room.tight ? unit_bytes : 0;
+    p.list_at = ((sh.n_layers + 1) * 64 + (room.tight ? 0 : unit_bytes) + 15) / 16 * 16;
     // the chunk list: tiles of the busiest CTA (QKV tiles are also cut at the ends of head halves) x segments
     auto listed = [&](int op, int n) { return (most(n) + p.cols[op].tile - 1) / p.cols[op].tile * p.cols[op].segs; };
     const int chunks_listed = (q_most / p.cols[ST_QKV].tile + 2 * (q_most / (D / 2) + 2)) * p.cols[ST_QKV].segs + listed(ST_O, H) + listed(ST_DN, H) + listed(ST_GU, F) + listed(ST_LM, sh.vocab);
-    p.resid_at = p.list_at + 16 * chunks_listed;
+    sl->list_len = room.tight ? 0 : chunks_listed;
+    p.merged_at = p.list_at + 16 * sl->list_len;
+    p.merged_len = 2 * most(qd / 2);
+    p.resid_at = p.merged_at + (room.tight ? 4 * mt * p.merged_len : 0);
     p.table_bytes = (p.resid_at + 4 * mt * most(H) + 127) / 128 * 128;
     // one area for the staged vector, the attention's scratch and the segments of the MLP activations: they follow one another
     const int slot = st_arrays(mt) * st_array_bytes(p.cols[ST_DN].seg), vec = std::max(st_arrays(mt) * st_array_bytes(H) + 4 * mt * p.ss_stride, st_arrays(mt) * st_array_bytes(qd));
@@ -207,7 +228,8 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     p.act_slots = p.cols[ST_DN].segs == 1 ? 1 : std::max(mt == 4 ? 3 : 2, std::min(3, area / slot));     // (every slot is taken from the ring)
     area = std::max(area, p.act_packets ? st_arrays(mt) * st_array_bytes(F) : p.act_slots * slot);
     const int fixed = step_shared_bytes(mt) + p.table_bytes + (area + 127) / 128 * 128;
-    int chunk = kv_block(D) * D * (kv8 ? 2 : 4) + 4 * 32;      // (K rows, then V in four quarters 32 bytes apart)
+    p.kv_block = kv_block(D) / room.kv_share;
+    int chunk = p.kv_block * D * (kv8 ? 2 : 4) + 4 * 32;      // (K rows, then V in four quarters 32 bytes apart)
     const int owned[5] = {q_most, most(H), most(F), most(H), most(sh.vocab)};
     for (int o = 0; o < 5; ++o) chunk = std::max(chunk, std::min(owned[o], p.cols[o].tile) * (o == ST_QKV || o == ST_GU ? 4 : 2) * p.cols[o].seg);
     sl->max_chunk_bytes = (chunk + 127) / 128 * 128;
@@ -220,8 +242,30 @@ inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sm
     const size_t chunks = static_cast<size_t>(std::max(grid / nkv, mt));
     sl->ll_bytes = 8 * (static_cast<size_t>(grid) * mt * p.q_line + static_cast<size_t>(grid) * 16 + chunks * qd + step_stat_len(chunks, nq)) + 2 * step_vec_bytes(p, mt, H, true) +
                    step_vec_bytes(p, mt, qd, false) + step_act_bytes(p, mt) + 256 +
-                   (st_packets(mt) ? 8 * (static_cast<size_t>(grid) * mt * (2 * p.x_line + p.ao_line) + static_cast<size_t>(mt) * p.act_len) : 0);
+                   (st_packets(mt) ? 8 * (static_cast<size_t>(grid) * mt * (2 * p.x_line + p.ao_line) + static_cast<size_t>(mt) * p.act_len) : 0) + (sl->unit_tab_bytes + 255) / 256 * 256;
     return nullptr;
+}
+inline const char *step_plan(const edgefm_shape &sh, int max_context, int num_sms, int smem_optin, bool kv8, int mt, StepLaunch *sl) {
+    const char *why = nullptr;
+    for (const StepRoom &room : ST_ROOM) {
+        if (!(why = step_plan_in(room, sh, max_context, num_sms, smem_optin, kv8, mt, sl))) return nullptr;
+        if (mt == 8) break;      // (the prompt kernels verify such a block)
+    }
+    return why;
+}
+// The unit tables of a tight build, as the others make them in shared memory (make_table).
+inline void step_unit_table(const StepLaunch &sl, unsigned *tab) {
+    const StepParams &p = sl.p;
+    for (int v = 0; v < 2; ++v) {
+        const int n = v ? p.qd : p.H, grain = v ? 2 : 1, line = v ? p.ao_line : p.x_line, upl = ((n / grain + sl.grid - 1) / sl.grid * grain + 1) / 2;
+        for (int w = 0; w < sl.grid; ++w) {
+            int row = st_first(n / grain, w, sl.grid) * grain;
+            const int r1 = st_first(n / grain, w + 1, sl.grid) * grain;
+            for (int e = 0; e < upl; ++e, row += 2)
+                *tab++ = static_cast<unsigned>(row & ((1 << ST_TIGHT_ROW_BITS) - 1)) | static_cast<unsigned>(std::max(0, std::min(2, r1 - row))) << ST_TIGHT_ROW_BITS |
+                         static_cast<unsigned>(w * (line >> 1) + e) << (ST_TIGHT_ROW_BITS + 2);
+        }
+    }
 }
 // Wire the exchange buffers (256-byte aligned base).
 inline void step_wire(StepLaunch *sl, int mt, unsigned long long *base) {
@@ -242,7 +286,8 @@ inline void step_wire(StepLaunch *sl, int mt, unsigned long long *base) {
     p.x_ll = base; base += g * m * p.x_line;
     p.xo_ll = base; base += g * m * p.x_line;
     p.ao_ll = base; base += g * m * p.ao_line;
-    p.act_ll = base;
+    p.act_ll = base; base += m * p.act_len;
+    p.unit_tab = sl->unit_tab_bytes ? reinterpret_cast<const unsigned *>(base) : nullptr;
 }
 // Tensor map of a row-major bf16 [rows][K] matrix for the boxes of an operator: the 64-column blocks of a row are the last dimension.
 inline bool step_map(CUtensorMap *m, const StepCols &c, const void *base, int rows) {

@@ -34,6 +34,20 @@ CASES = {
     # fewer rows than CTAs
     "narrow": (dict(hidden=72, ffn=40, n_q_heads=1, n_kv_heads=1), 3, 1, None),
     "narrow_8": (dict(hidden=72, ffn=40, n_q_heads=1, n_kv_heads=1), 3, 8, None),
+    # more attention outputs than 128 per CTA: few rows (and so few CTAs) with many heads; 24576 on all CTAs (tables out of shared memory)
+    "few_rows_many_heads": (dict(hidden=8, n_q_heads=44, n_kv_heads=22, head_dim=128, ffn=40), 20, 1, None),
+    "few_rows_many_heads_int8": (dict(hidden=8, n_q_heads=44, n_kv_heads=22, head_dim=128, ffn=40), 20, 1, "int8"),
+    "few_rows_many_heads_2": (dict(hidden=8, n_q_heads=15, n_kv_heads=3, head_dim=128, ffn=64), 20, 2, None),
+    "few_rows_many_heads_4": (dict(hidden=8, n_q_heads=12, n_kv_heads=3, head_dim=128, ffn=256), 20, 4, None),
+    "few_rows_many_heads_8": (dict(hidden=8, n_q_heads=12, n_kv_heads=3, head_dim=128, ffn=256), 20, 8, None),
+    "outputs_24576": (dict(hidden=152, n_q_heads=192, n_kv_heads=24, head_dim=128, n_layers=1), 20, 1, None),
+    # vectors that leave no room for tables and chunk lists, then for smaller chunks only, then for half blocks of cached positions, too
+    "far_tables": (dict(hidden=24056, n_kv_heads=4, ffn=160, n_layers=1), 300, 1, None),
+    "small_chunks_boxes": (dict(hidden=28800, n_kv_heads=4, ffn=64, n_layers=1), 300, 1, None),
+    "small_chunks_rows": (dict(hidden=30600, n_kv_heads=4, ffn=64, n_layers=1), 300, 1, "int8"),
+    "half_blocks_rows_2": (dict(hidden=15600, n_q_heads=8, n_kv_heads=4, ffn=64, n_layers=1), 148 * 8 + 21, 2, None),
+    "half_blocks_boxes_2": (dict(hidden=15616, n_q_heads=8, n_kv_heads=4, head_dim=128, ffn=64, n_layers=1), 148 * 8 + 21, 2, None),
+    "small_chunks_4": (dict(hidden=11000, n_q_heads=8, n_kv_heads=4, ffn=64, n_layers=1), 40, 4, None),
     # attention: tiles of 16 positions in quarters, blocks of 64 (heads of 128) or 128; one position, one more than a tile, than a block
     **{f"attention_{d}_{n}_{m}{q or ''}": (dict(head_dim=d, n_q_heads=g, n_kv_heads=1), n, m, q)
        for d, g in ((64, 3), (128, 8)) for n, m, q in ((1, 1, None), (17, 2, None), (148 * 16 + 1, 1, None), (148 * 64 + 5, 1, None), (148 * 128 + 9, 8, None),

@@ -14,7 +14,7 @@ from helpers import LOGIT_MAX_ABS, LOGIT_REL_L2, Pair, compare_logits
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("variant", ["tiny", "bias_long_rows", "long_context_build"])
+@pytest.mark.parametrize("variant", ["tiny", "bias_long_rows", "long_context_build", "far_tables"])
 def test_static_scratch_step_matches_context_step_twice(variant):
     import torch
     from paper_2604_27476_b200 import edgefm_decode_step_static, edgefm_sync_status
@@ -22,6 +22,8 @@ def test_static_scratch_step_matches_context_step_twice(variant):
     cfg = CONFIGS["tiny"]
     if variant == "bias_long_rows":   # K slices, several tiles per warp, biases, many attention chunks
         cfg = cfg.with_(hidden=512, ffn=6144, vocab=20000, n_layers=3, qkv_bias=True, cache_len=700)
+    if variant == "far_tables":       # the unit tables lie in the scratch array, too
+        cfg = cfg.with_(hidden=24056, ffn=160, vocab=300, n_layers=1)
     T0, Tmax = cfg.cache_len, cfg.cache_len + 4
     if variant == "long_context_build":   # max_context > 8192 selects the other build of the kernel
         T0, Tmax = 300, 8300

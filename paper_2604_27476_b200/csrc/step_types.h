@@ -204,6 +204,10 @@ inline const char *step_plan_in(const StepRoom &room, const edgefm_shape &sh, in
     p.act_packets = st_packets(mt) && st_arrays(mt) * st_array_bytes(F) <= ST_ACT_WHOLE;
     p.cols[ST_DN] = step_cols(F, most(H), false, mt <= 2 ? 2048 : 1024,       // (two segments of activations are in shared memory, as pieces)
                               p.act_packets ? room.chunk_small : room.chunk_bytes, room.chunk_whole);
+    // (a chunk's place is counted in 16-byte units of its matrix, 32 bits of them; boxes are placed by rows)
+    const long long rows_of[5] = {static_cast<long long>(nq + 2 * nkv) * D, H, 2LL * F, H, sh.vocab};
+    for (int o = 0; o < 5; ++o)
+        if (p.cols[o].box_rows == 0 && rows_of[o] * (p.cols[o].K / 8) > 0xffffffffLL) return "a weight matrix is larger than 64 GiB";
     p.q_line = st_line(2 * most((nq + 2 * nkv) * D / 2));
     p.ss_stride = (grid + 3) / 4 * 4;
     p.x_line = st_line(most(H) + 1);

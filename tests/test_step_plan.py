@@ -109,6 +109,20 @@ def test_shapes_that_leave_little_room(name):
     assert check_plan(sh, max_context, kv_format, tokens, ctas=(0, 1, 63))["tight"]
 
 
+def test_matrices_past_the_offsets_of_a_chunk_are_refused():
+    """Offsets are 32 bits of 16-byte units: the last row of a 64 GiB matrix is in reach, one of a larger matrix would be taken from its start."""
+    from paper_2604_27476_b200 import EdgefmError, Status
+    last = 2 ** 32 // 300                                         # rows of 2400 columns
+    _, chunks = edgefm_debug_step_plan(shape_of(H=2400, V=last), 64, op=LM, cta=147)
+    x, _, z, _, u, n = chunks[-1].astype(np.int64)
+    assert u + n == last and x == u * 300 and z == n * 4800
+    with pytest.raises(EdgefmError) as ei:
+        edgefm_debug_step_plan(shape_of(H=2400, V=last + 1), 64)
+    assert ei.value.status == Status.ERR_BAD_SHAPE and "64 GiB" in str(ei.value)
+    with pytest.raises(EdgefmError):
+        edgefm_debug_step_plan(shape_of(H=2400, F=last // 2 // 8 * 8 + 8), 64)      # gate and up rows are one matrix
+
+
 def test_what_gives_way():
     """In order: tables and lists, chunk sizes, the cached positions of a chunk."""
     far = edgefm_debug_step_plan(shape_of(H=24056, nq=4, nkv=4, F=160, V=300), 4096)

@@ -302,9 +302,10 @@ edgefm_status edgefm_debug_set_wait_limit(edgefm_ctx *ctx, uint32_t limit_ns, in
  * into the bound without any fault.  Host only. */
 edgefm_status edgefm_debug_set_prefill_wait(edgefm_ctx *ctx, uint32_t polls, int32_t extra_arrivals);
 
-/* How edgefm_prefill tiles a contraction of [M tokens x K] x [K x N] on num_sms SMs: out2 = {1 = 256-column output tiles
- * (0 = 128), K units per output tile}.  epilogue: 0 = QKV, 1 = added to the residual stream (O and down projection; only
- * these split K), 2 = gate/up (always wide, never split).  Host only: for checking the planner without a GPU. */
+/* How edgefm_prefill tiles a contraction of [M tokens x K] x [K x N] on num_sms SMs: out2 = {output tile: 0 = 128 columns, 1 = 256,
+ * 2 = 64, K units per output tile}.  epilogue: 0 = QKV with heads of 128, 3 = with heads of 64, 1 = added to the residual stream (O and
+ * down projection; only these split K), 2 = gate/up (128 gate columns and their 128 up columns, or 64 and 64; never split).  Tiles of
+ * half the columns are taken where they still fit the SMs in one round.  Host only: for checking the planner without a GPU. */
 edgefm_status edgefm_debug_prefill_plan(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t *out2);
 
 /* Host-only check of the planner: how the step kernel for `tokens` tokens per call (1, 2, 4 or 8) is laid out for a shape on n_sms SMs with

@@ -515,10 +515,9 @@ constexpr int PF_SPLIT_MAX = 8;               // K splits of a contraction that 
 // the tensor pipe, bounds the narrow tiles.  Gate/up runs wide: 128 gate columns and their 128 up partners.
 // Few tokens leave most SMs idle with these tiles, and the pass is a chain of latencies: every CTA pulls its whole K through one SM
 // (77 tokens, 0.5B shape: QKV on 9 CTAs 17 us, O on 7 CTAs 22 us, gate/up on 38 CTAs 23 us).  Where tiles of half the columns still
-// fit the SMs in one round they are taken: PF_SLIM, 64 columns, or PF_NARROW for gate/up, 64 + 64 (use_slim).
+// fit the SMs in one round they are taken: PF_SLIM, 64 columns, or PF_NARROW for gate/up, 64 + 64.
 // The kernel is persistent (one CTA per SM, tiles dealt round-robin, neighbours sharing a weight tile) with TWO accumulators
 // in tensor memory, so that the epilogue of a tile runs under the main loop of the next.
-enum { PF_NARROW = 0, PF_SLIM = 1, PF_WIDE = 2 };
 template <int SHAPE> struct GemmCfg {
     static constexpr int BN = SHAPE == PF_WIDE ? 256 : SHAPE == PF_SLIM ? 64 : 128;
     static constexpr int STAGES = SHAPE == PF_WIDE ? 3 : SHAPE == PF_SLIM ? 5 : 4;
@@ -1327,23 +1326,12 @@ const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const 
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill GEMM launch failed";
 }
 
-// Shape and K split.  Cost model: the rounds the SMs need (units / SMs, rounded up) times the cost of a unit; a wide tile does
-// twice the work of a narrow one for 1.33 x the operand traffic (1.6), a K split divides a unit's cost and adds a little for
-// the partial sums (5 %).  Only the contractions that add to the residual stream split (their partial sums are added by the
-// norm kernel that follows, in a fixed order); a split keeps at least 12 k-blocks per unit and is considered only when the
-// unsplit tiles do not fill the SMs once (with more tiles the partial-sum traffic costs more than the better balance gains:
-// 7B shape, 2048 tokens, 48.0 -> 50.7 ms).
-// Half as many columns per tile where the tiles (and their K splits) still fit the SMs in one round; a QKV tile is whole heads.
-bool use_slim(int epilogue, int M, int N, int d, int splits, int num_sms) {
-    if (epilogue == EPI_LOGITS || (epilogue == EPI_QKV && d != 64)) return false;
-    return ((N + 63) / 64) * ((M + PF_BM - 1) / PF_BM) * splits <= num_sms;
-}
 template <int EPI>
 const char *launch_gemm(const uint16_t *a, size_t a_plane, const void *w, long long w_rows, GemmArgs &g, int num_sms, cudaStream_t s) {
     CUtensorMap ma, ml, mb;
-    int wide = 1;
-    prefill_plan_contraction(EPI, g.M, g.N, g.K, num_sms, &wide, &g.splits);
-    const bool slim = use_slim(EPI, g.M, g.N, g.d, g.splits, num_sms);
+    int shape = PF_WIDE;
+    prefill_plan_contraction(EPI, g.d, g.M, g.N, g.K, num_sms, &shape, &g.splits);
+    const bool slim = shape == (EPI == EPI_SWIGLU ? PF_NARROW : PF_SLIM);
     if (!encode_operand_map(&ma, a, g.M, g.K) || !encode_operand_map(&ml, a + a_plane, g.M, g.K) || !encode_operand_map(&mb, w, w_rows, g.K, slim ? 64 : 128))
         return "cuTensorMapEncodeTiled failed";
     if constexpr (EPI == EPI_SWIGLU) {
@@ -1351,7 +1339,7 @@ const char *launch_gemm(const uint16_t *a, size_t a_plane, const void *w, long l
     } else {
         if constexpr (EPI != EPI_LOGITS)
             if (slim) return launch_gemm_cfg<EPI, PF_SLIM>(ma, ml, mb, g, num_sms, s);
-        return wide ? launch_gemm_cfg<EPI, PF_WIDE>(ma, ml, mb, g, num_sms, s) : launch_gemm_cfg<EPI, PF_NARROW>(ma, ml, mb, g, num_sms, s);
+        return shape == PF_WIDE ? launch_gemm_cfg<EPI, PF_WIDE>(ma, ml, mb, g, num_sms, s) : launch_gemm_cfg<EPI, PF_NARROW>(ma, ml, mb, g, num_sms, s);
     }
 }
 
@@ -1412,24 +1400,34 @@ const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *v
 
 }  // namespace
 
-void prefill_plan_contraction(int epilogue, int M, int N, int K, int num_sms, int *wide, int *splits) {
+// Shape and K split.  Cost model: the rounds the SMs need (units / SMs, rounded up) times the cost of a unit; a wide tile does
+// twice the work of a narrow one for 1.33 x the operand traffic (1.6), a K split divides a unit's cost and adds a little for
+// the partial sums (5 %).  Only the contractions that add to the residual stream split (their partial sums are added by the
+// norm kernel that follows, in a fixed order); a split keeps at least 12 k-blocks per unit and is considered only when the
+// unsplit tiles do not fill the SMs once (with more tiles the partial-sum traffic costs more than the better balance gains:
+// 7B shape, 2048 tokens, 48.0 -> 50.7 ms).
+// Half as many columns per tile (PF_SLIM; gate/up: PF_NARROW) where the tiles and their K splits still fit the SMs in one round; a QKV tile is whole
+// heads.
+void prefill_plan_contraction(int epilogue, int head_dim, int M, int N, int K, int num_sms, int *shape, int *splits) {
     const int m_tiles = (M + PF_BM - 1) / PF_BM, kb = (K + PF_BK - 1) / PF_BK;
-    *wide = 1;
+    *shape = PF_WIDE;
     *splits = 1;
-    if (epilogue == EPI_SWIGLU) return;
-    const int tiles[2] = {((N + 127) / 128) * m_tiles, ((N + 255) / 256) * m_tiles};
-    const double cost[2] = {1.0, 1.6};
-    int best_shape = 0, best_split = 1;
-    double best = 1e30;
-    for (int shape = 0; shape < 2; ++shape)
-        for (int sp = 1; sp <= (epilogue == EPI_RESID ? (m_tiles == 1 ? PF_SPLIT_MAX : 4) : 1); ++sp) {
-            if (sp > 1 && (kb / sp < 12 || tiles[shape] > num_sms)) break;   // split only grids that leave SMs idle in their one round
-            const int units = tiles[shape] * sp;
-            const double t = ((units + num_sms - 1) / num_sms) * cost[shape] / sp * (sp > 1 ? 1.05 : 1.0);
-            if (t < best - 1e-9) { best = t; best_shape = shape; best_split = sp; }
-        }
-    *wide = best_shape;
-    *splits = best_split;
+    if (epilogue != EPI_SWIGLU) {
+        const int tiles[2] = {((N + 127) / 128) * m_tiles, ((N + 255) / 256) * m_tiles};
+        const double cost[2] = {1.0, 1.6};
+        int best_wide = 0;
+        double best = 1e30;
+        for (int wide = 0; wide < 2; ++wide)
+            for (int sp = 1; sp <= (epilogue == EPI_RESID ? (m_tiles == 1 ? PF_SPLIT_MAX : 4) : 1); ++sp) {
+                if (sp > 1 && (kb / sp < 12 || tiles[wide] > num_sms)) break;   // split only grids that leave SMs idle in their one round
+                const int units = tiles[wide] * sp;
+                const double t = ((units + num_sms - 1) / num_sms) * cost[wide] / sp * (sp > 1 ? 1.05 : 1.0);
+                if (t < best - 1e-9) { best = t; best_wide = wide; *splits = sp; }
+            }
+        *shape = best_wide ? PF_WIDE : PF_NARROW;
+    }
+    if (epilogue == EPI_LOGITS || (epilogue == EPI_QKV && head_dim != 64) || ((N + 63) / 64) * m_tiles * *splits > num_sms) return;
+    *shape = epilogue == EPI_SWIGLU ? PF_NARROW : PF_SLIM;
 }
 
 size_t prefill_buffer_bytes(const edgefm_shape &sh, int chunk) {

@@ -53,9 +53,11 @@ struct PrefillModel {
     int num_sms;
 };
 
+// Tile shapes of a contraction: 128, 64 or 256 output columns (gate/up: 64 gate and 64 up, or 128 and 128).
+enum { PF_NARROW = 0, PF_SLIM = 1, PF_WIDE = 2 };
 // Tile shape and K split a contraction of [M x K] x [K x N] gets on num_sms SMs (host logic, no device needed).
-// epilogue: 0 = QKV, 1 = added to the residual stream (O, down), 2 = gate/up.  *wide: 256-column tiles; *splits: K units per tile.
-void prefill_plan_contraction(int epilogue, int M, int N, int K, int num_sms, int *wide, int *splits);
+// epilogue: 0 = QKV (heads of head_dim), 1 = added to the residual stream (O, down), 2 = gate/up, 3 = logits of a verified block.
+void prefill_plan_contraction(int epilogue, int head_dim, int M, int N, int K, int num_sms, int *shape, int *splits);
 
 // Bytes the work buffers of a pass over `chunk` tokens take.
 size_t prefill_buffer_bytes(const edgefm_shape &sh, int chunk);

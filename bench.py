@@ -454,7 +454,7 @@ def main():
     t0 = time.perf_counter()
     tok, pos = tok0, pos0
     for _ in range(steps):
-        edgefm_decode_step(handle, tok, pos, stream, None, ctx.next_token.data_ptr())   # request block: host -> device
+        edgefm_decode_step(handle, tok, pos, stream, None, ctx.next_token.data_ptr())   # token and position: arguments of the launch
         host_tok.copy_(ctx.next_token, non_blocking=True)                                # result: device -> host
         torch.cuda.current_stream().synchronize()
         tok, pos = int(host_tok[0]), pos + 1
@@ -492,7 +492,7 @@ def main():
             "roofline": {"bound": "hbm", "kernel": f"step_kernel: the whole decode step ({launches} kernel launch per token)",
                          "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "peak_source": peak_src,
                          "bytes_per_launch": bytes_per_step, "frac_of_nominal_8TBs": gbs / NOMINAL_HBM_GBS, "traffic": traffic, "traffic_source": traffic_src},
-            "e2e": {"value": e2e_ms / tokens, "unit": UNIT, "h2d_bytes_per_step": 48, "d2h_bytes_per_step": 4},
+            "e2e": {"value": e2e_ms / tokens, "unit": UNIT, "h2d_bytes_per_step": 8, "d2h_bytes_per_step": 4},
             "gpu_launches": launches * steps * n_seq,
             "clocks": clocks,
             "cpu_baseline": cpu,

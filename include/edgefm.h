@@ -321,17 +321,6 @@ edgefm_status edgefm_debug_step_plan(const edgefm_shape *shape, int32_t max_cont
                                      int32_t smem_bytes, int32_t *out40, int32_t op, int32_t cta, uint32_t *chunks_out, int32_t capacity,
                                      int32_t *n_chunks);
 
-/* Host-only check of the planner: the tile schedule of one weight-streaming operator (kind: 0 QKV pairs, 1 residual rows,
- * 2 gate/up pairs, 3 output-layer rows; units rows or pairs; K columns; head_half = head_dim / 2 for kind 0) for n_ctas CTAs
- * of n_warps consumer warps whose ring slots hold slot_rows rows.  tiles_out receives one 64-bit descriptor per tile, CTA by
- * CTA and warp by warp (tiles_per_warp [n_ctas * n_warps] counts them); combines_out four 32-bit words per entry
- * (combines_per_cta [n_ctas]); variant_rows [4] the box heights of the operator's tensor maps; *n_tiles / *n_combines the
- * totals (call once with NULL outputs to size the buffers).  Needs no GPU.  BAD_SHAPE when the operator does not fit. */
-edgefm_status edgefm_debug_plan_operator(int32_t kind, int32_t units, int32_t K, int32_t head_half, int32_t op_index, int32_t n_ctas,
-                                         int32_t n_warps, int32_t slot_rows, uint64_t *tiles_out, int64_t tiles_cap,
-                                         int32_t *tiles_per_warp, uint32_t *combines_out, int64_t combines_cap,
-                                         int32_t *combines_per_cta, int32_t *variant_rows, int64_t *n_tiles, int64_t *n_combines);
-
 /*
  * edgefm_decode_step_static -- one decode step that allocates nothing (the paper has no counterpart; this
  * entry point exists for callers that cannot allocate device memory).

@@ -51,7 +51,7 @@ class _Weights(ctypes.Structure):
 
 EXPORTS = ("edgefm_create", "edgefm_prefill_kv", "edgefm_decode_step", "edgefm_destroy", "edgefm_get_length",
            "edgefm_export_kv", "edgefm_get_launches_per_step", "edgefm_last_error", "edgefm_version",
-           "edgefm_sync_status", "edgefm_debug_profile", "edgefm_debug_set_wait_limit", "edgefm_debug_set_prefill_wait", "edgefm_debug_prefill_plan", "edgefm_debug_plan", "edgefm_debug_step_plan", "edgefm_debug_plan_operator", "edgefm_decode_step_static", "edgefm_set_vocab_subset",
+           "edgefm_sync_status", "edgefm_debug_profile", "edgefm_debug_set_wait_limit", "edgefm_debug_set_prefill_wait", "edgefm_debug_prefill_plan", "edgefm_debug_plan", "edgefm_debug_step_plan", "edgefm_decode_step_static", "edgefm_set_vocab_subset",
            "edgefm_append_kv", "edgefm_create_with_options", "edgefm_export_kv_int8", "edgefm_verify_block", "edgefm_sync_length", "edgefm_prefill_tokens", "edgefm_prefill")
 
 
@@ -107,8 +107,6 @@ def load_library():
     L.edgefm_debug_plan.argtypes = [vp, ctypes.POINTER(i32)]
     L.edgefm_debug_step_plan.restype = ctypes.c_int
     L.edgefm_debug_step_plan.argtypes = [ctypes.POINTER(_Shape)] + [i32] * 5 + [ctypes.POINTER(i32), i32, i32, vp, i32, ctypes.POINTER(i32)]
-    L.edgefm_debug_plan_operator.restype = ctypes.c_int
-    L.edgefm_debug_plan_operator.argtypes = [i32] * 8 + [vp, i64, vp, vp, i64, vp, vp, ctypes.POINTER(i64), ctypes.POINTER(i64)]
     L.edgefm_decode_step_static.restype = ctypes.c_int
     L.edgefm_decode_step_static.argtypes = [ctypes.POINTER(_Shape), ctypes.POINTER(_Weights), vp, vp, i32, i32, i32, i32, vp, vp, vp]
     L.edgefm_append_kv.restype = ctypes.c_int
@@ -243,9 +241,8 @@ def edgefm_debug_plan(ctx) -> dict:
     """Launch geometry of the context's step kernel."""
     out = (ctypes.c_int32 * 8)()
     _check(load_library().edgefm_debug_plan(ctx, out), ctx)
-    keys = ("ctas", "consumer_warps", "ring_slots_per_warp", "slot_bytes", "dynamic_smem_bytes", "max_tiles_per_cta", "schedule_smem_bytes",
-            "long_context_build")
-    return dict(zip(keys, list(out)))
+    keys = ("ctas", "consumer_warps", "ring_chunks", "max_chunk_bytes", "dynamic_smem_bytes", "ring_bytes", "table_bytes")
+    return dict(zip(keys, list(out)))      # (the eighth number is unused)
 
 
 STEP_PLAN = ("ctas", "dynamic_smem_bytes", "ring_bytes", "max_chunk_bytes", "table_bytes", "list_len", "tight", "unit_table_bytes", "kv_block", "act_slots",
@@ -270,44 +267,6 @@ def edgefm_debug_step_plan(shape: dict, max_context, kv_format="bf16", tokens=1,
     chunks = np.zeros((n.value, 6), np.uint32)
     call(chunks.ctypes.data, n.value)
     return plan, chunks
-
-
-def edgefm_debug_plan_operator(kind, units, K, head_half, op_index, n_ctas, n_warps, slot_rows):
-    """Host-only: the tile schedule the planner makes for one operator.  Returns a dict with
-    tiles [cta][warp] -> list of decoded tile dicts, combines [cta] -> list of dicts, variant_rows."""
-    import numpy as np
-    L = load_library()
-    per_warp = np.zeros(n_ctas * n_warps, np.int32)
-    per_cta = np.zeros(n_ctas, np.int32)
-    variants = np.zeros(4, np.int32)
-    nt, nc = ctypes.c_int64(), ctypes.c_int64()
-    args = (kind, units, K, head_half, op_index, n_ctas, n_warps, slot_rows)
-    _check(L.edgefm_debug_plan_operator(*args, None, 0, per_warp.ctypes.data, None, 0, per_cta.ctypes.data, variants.ctypes.data,
-                                        ctypes.byref(nt), ctypes.byref(nc)))
-    tiles = np.zeros(max(nt.value, 1), np.uint64)
-    comb = np.zeros(max(nc.value, 1) * 4, np.uint32)
-    _check(L.edgefm_debug_plan_operator(*args, tiles.ctypes.data, tiles.size, per_warp.ctypes.data, comb.ctypes.data, nc.value, per_cta.ctypes.data,
-                                        variants.ctypes.data, ctypes.byref(nt), ctypes.byref(nc)))
-    out_tiles, pos = [], 0
-    for c in range(n_ctas):
-        row = []
-        for w in range(n_warps):
-            lst = []
-            for _ in range(per_warp[c * n_warps + w]):
-                d = int(tiles[pos]); pos += 1
-                x, y = d & 0xffffffff, d >> 32
-                lst.append(dict(unit_base=x & 0xfffff, kcol=(x >> 20) & 0xff, variant=(x >> 28) & 3, first=bool(x >> 30 & 1), flush=bool(x >> 31 & 1),
-                                m=y & 31, v0=(y >> 5) & 15, direct=bool(y >> 9 & 1), slot=(y >> 10) & 1023, op=(y >> 20) & 7))
-            row.append(lst)
-        out_tiles.append(row)
-    out_comb, pos = [], 0
-    for c in range(n_ctas):
-        lst = []
-        for _ in range(per_cta[c]):
-            e = comb[4 * pos: 4 * pos + 4]; pos += 1
-            lst.append(dict(unit_base=int(e[0]), m=int(e[1]) & 0xff, v0=int(e[1]) >> 8, first_slot=int(e[2]), n_slots=int(e[3])))
-        out_comb.append(lst)
-    return dict(tiles=out_tiles, combines=out_comb, variant_rows=[int(v) for v in variants if v])
 
 
 def edgefm_debug_profile(ctx):
@@ -391,7 +350,7 @@ class DecodeContext:
         with torch.cuda.device(self.device):
             self.handle = edgefm_create(shape, device_weight_ptrs, max_context, kv_format, block_tokens=block_tokens)
         self.block_tokens = max(1, block_tokens)
-        # rows for the longest block a call may carry: block_tokens through the step kernel, up to 8 through the dense path
+        # rows for the longest block a call may carry: up to eight tokens on any context
         self.block_logits = torch.empty((max(self.block_tokens, 8), cfg.vocab), dtype=torch.float32, device=self.device)
         self.logits = self.block_logits[0]
         self.next_token = torch.zeros(1, dtype=torch.int32, device=self.device)
@@ -434,7 +393,7 @@ class DecodeContext:
         edgefm_prefill_tokens(self.handle, tokens, position, self._stream())
 
     def prefill(self, tokens, position=0, want_logits=True):
-        """The prefill phase for a prompt: dense contractions for all but the last token, a decode step for the last."""
+        """The prefill phase for a prompt: dense contractions (of fewer than eight tokens the last one takes a decode step)."""
         edgefm_prefill(self.handle, tokens, position, self._stream(), self.logits.data_ptr() if want_logits else None,
                        self.next_token.data_ptr())
 

@@ -12,7 +12,7 @@
 #include <vector>
 
 #include "common.cuh"
-#include "step_plan.h"
+#include "tensor_map.h"
 #include "prefill.h"
 #include "step_types.h"
 
@@ -251,9 +251,10 @@ cudaError_t run_step(edgefm_ctx::Build *b, const StepRequest &r, cudaStream_t s)
 
 // Zeroed exchange buffers (with unit tables) and tensor maps of a build, complete when the call returns: the first launch may go to any stream,
 // and work on the legacy stream is ordered against neither a non-blocking one nor the return of a pageable copy.
-cudaError_t init_build(const StepLaunch &sl, void *ll, void *maps, const void *host_maps, size_t map_bytes) {
+// own_stream: other work may be under way, which this neither waits for nor disturbs (0.2 ms more than on the legacy stream).
+cudaError_t init_build(const StepLaunch &sl, void *ll, void *maps, const void *host_maps, size_t map_bytes, bool own_stream) {
     cudaStream_t own = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+    cudaError_t e = own_stream ? cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) : cudaSuccess;
     if (e != cudaSuccess) return e;
     std::vector<unsigned> units(sl.unit_tab_bytes / 4);
     e = cudaMemsetAsync(ll, 0, sl.ll_bytes, own);
@@ -263,7 +264,7 @@ cudaError_t init_build(const StepLaunch &sl, void *ll, void *maps, const void *h
         e = cudaMemcpyAsync(const_cast<unsigned *>(sl.p.unit_tab), units.data(), sl.unit_tab_bytes, cudaMemcpyHostToDevice, own);
     }
     const cudaError_t done = cudaStreamSynchronize(own);
-    cudaStreamDestroy(own);
+    if (own) cudaStreamDestroy(own);
     return e != cudaSuccess ? e : done;
 }
 
@@ -282,7 +283,7 @@ cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char *
         const bool sub = c->vocab_subset > 0;
         if (!step_maps(p, c->layers.data(), sub ? static_cast<const void *>(c->sub_lm) : c->lm_head, sub ? c->vocab_subset : c->shape.vocab, maps.data())) return cudaErrorUnknown;
         if (!b->maps && (e = cudaMalloc(reinterpret_cast<void **>(&b->maps), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
-        if ((e = init_build(sl, b->ll, b->maps, maps.data(), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
+        if ((e = init_build(sl, b->ll, b->maps, maps.data(), maps.size() * sizeof(CUtensorMap), b == &c->wide)) != cudaSuccess) return e;
         p.maps = b->maps;
         p.map_fence = 1;   // edgefm_set_vocab_subset rewrites the output layer's map
     }
@@ -1056,37 +1057,5 @@ extern "C" edgefm_status edgefm_debug_step_plan(const edgefm_shape *shape, int32
         std::copy(v, v + 5, out40 + 15 + 5 * o);
     }
     *n_chunks = cta < sl.grid ? step_chunks(sl, op, cta, chunks_out, chunks_out ? capacity : 0) : 0;
-    return EDGEFM_OK;
-}
-
-// Host-only diagnostics: the tile schedule of one operator, in the form the kernel reads, for checking the planner
-// without a GPU.  tiles_out receives the tiles CTA by CTA, warp by warp (tiles_per_warp [n_ctas * n_warps] counts them);
-// combines_out four words per entry (combines_per_cta [n_ctas]); variant_rows [4] the box heights of the tensor maps.
-extern "C" edgefm_status edgefm_debug_plan_operator(int32_t kind, int32_t units, int32_t K, int32_t head_half, int32_t op_index, int32_t n_ctas,
-                                                    int32_t n_warps, int32_t slot_rows, uint64_t *tiles_out, int64_t tiles_cap,
-                                                    int32_t *tiles_per_warp, uint32_t *combines_out, int64_t combines_cap,
-                                                    int32_t *combines_per_cta, int32_t *variant_rows, int64_t *n_tiles, int64_t *n_combines) {
-    if (!tiles_per_warp || !combines_per_cta || !variant_rows || !n_tiles || !n_combines || n_ctas < 1 || n_warps < 1)
-        return fail(nullptr, EDGEFM_ERR_INVALID_ARG, "bad argument");
-    OpShape os{kind, units, K, op_paired(kind) ? 2 * units : units, head_half};
-    OpSchedule S;
-    if (const char *why = plan_op(os, op_index, n_ctas, n_warps, slot_rows, &S)) return fail(nullptr, EDGEFM_ERR_BAD_SHAPE, "%s", why);
-    int64_t nt = 0, nc = 0;
-    for (int c = 0; c < n_ctas; ++c) {
-        for (int w = 0; w < n_warps; ++w) {
-            tiles_per_warp[c * n_warps + w] = static_cast<int32_t>(S.tiles[c][w].size());
-            for (const uint2 &d : S.tiles[c][w]) {
-                if (tiles_out && nt < tiles_cap) tiles_out[nt] = static_cast<uint64_t>(d.x) | static_cast<uint64_t>(d.y) << 32;
-                ++nt;
-            }
-        }
-        combines_per_cta[c] = static_cast<int32_t>(S.combines[c].size());
-        for (const MkCombine &e : S.combines[c]) {
-            if (combines_out && nc < combines_cap) { combines_out[4 * nc] = e.x; combines_out[4 * nc + 1] = e.y; combines_out[4 * nc + 2] = e.z; combines_out[4 * nc + 3] = e.w; }
-            ++nc;
-        }
-    }
-    for (int v = 0; v < MK_MAX_VARIANTS; ++v) variant_rows[v] = v < S.n_variants ? S.variant_rows[v] : 0;
-    *n_tiles = nt; *n_combines = nc;
     return EDGEFM_OK;
 }

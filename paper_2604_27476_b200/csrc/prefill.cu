@@ -19,7 +19,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
-#include "step_plan.h"
+#include "tensor_map.h"
 
 namespace edgefm {
 namespace {

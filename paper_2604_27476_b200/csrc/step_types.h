@@ -6,7 +6,7 @@
 
 #include "../../include/edgefm.h"
 #include "common.cuh"
-#include "step_plan.h"
+#include "tensor_map.h"
 
 namespace edgefm {
 

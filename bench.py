@@ -200,7 +200,7 @@ def run_block(args, cfg):
     k, v = make_kv(cfg)
     ptrs, keep = upload_weights(weights, dev)
     B = args.block_tokens
-    dense = B > 4          # blocks of more than four tokens take the dense path (prefill kernels) on a plain context; every call then
+    dense = B > 4          # blocks of more than four tokens run on a plain context (the build for eight); every call then
                            # reads the accepted length and the next token back to the host (part of the timed loop)
     ctx = DecodeContext(cfg, ptrs, cfg.cache_len + B * steps + B + 2, dev, block_tokens=0 if dense else B)
     kd = torch.from_numpy(k.view(np.int16)).to(dev)

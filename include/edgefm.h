@@ -240,8 +240,8 @@ edgefm_status edgefm_export_kv_int8(edgefm_ctx *ctx, void *k_codes_out, void *v_
 edgefm_status edgefm_get_launches_per_step(const edgefm_ctx *ctx, int32_t *n_launches_host);
 
 /* Synchronise `stream`, then report whether a bounded device-side wait of the persistent step kernel
- * expired or one of its self-checks failed (EDGEFM_ERR_TIMEOUT; the context is then unusable and must be destroyed)
- * or all is well.  ctx == NULL: the status left by the last edgefm_decode_step_static on the current device. */
+ * expired or one of its self-checks failed (EDGEFM_ERR_TIMEOUT; the context is then unusable and must be destroyed:
+ * behind an expired wait later steps do nothing and new cache rows do not reset the status) or all is well.  ctx == NULL: the status left by the last edgefm_decode_step_static on the current device. */
 edgefm_status edgefm_sync_status(edgefm_ctx *ctx, void *stream);
 
 /*
@@ -330,7 +330,7 @@ edgefm_status edgefm_debug_step_plan(const edgefm_shape *shape, int32_t max_cont
  * latency-critical threads that cannot take the implicit device synchronisation of cudaMalloc / cudaFree.
  * edgefm_create allocates a KV cache and work buffers; this call does neither.  It is the same persistent step
  * kernel as edgefm_decode_step, with all its work buffers (residual stream, queries, attention partials, MLP
- * activations, operator table, tile schedule, tensor maps, counters, device state) carved out of a fixed 4 MiB array
+ * activations, layer table, tensor maps, device state) carved out of a fixed 4 MiB array
  * that is part of the loaded library image on every GPU, and with the KV cache owned by the caller:
  *   shape, weights   as for edgefm_create (read during the call; device buffers borrowed until the step has run);
  *                    at most 96 layers, and the work buffers of the shape must fit the 4 MiB, else
@@ -340,8 +340,8 @@ edgefm_status edgefm_debug_step_plan(const edgefm_shape *shape, int32_t max_cont
  *   cur_len          filled slots before the step (the caller keeps the count; 0 <= cur_len < max_context).
  *   token_id, position  both explicit (>= 0); nothing is remembered between calls.
  *   logits_out       DEVICE fp32 [vocab] or NULL;  next_token_out  DEVICE int32 [1] or NULL.
- * The work is enqueued on `stream` (stream-ordered copies of the schedule and one memset of the counters, then the
- * kernel) and the call returns without synchronising.  It calls no cudaMalloc, cudaFree or other allocating
+ * The work is enqueued on `stream` (stream-ordered copies of the layer table and the tensor maps and one memset of the exchange
+ * buffers, then the kernel) and the call returns without synchronising.  It calls no cudaMalloc, cudaFree or other allocating
  * routine.  The first call on a device also looks up the device address of the scratch array (once per device,
  * with that device current).  The copies read host memory of the call itself, so `stream` must NOT be in capture
  * mode: a capturing stream is refused with EDGEFM_ERR_INVALID_ARG before anything is enqueued.

@@ -249,27 +249,20 @@ cudaError_t run_step(edgefm_ctx::Build *b, const StepRequest &r, cudaStream_t s)
     return launch_step(b->launch, s);
 }
 
-// Zeroed exchange buffers (with unit tables) and tensor maps of a build, complete when the call returns: the first launch may go to any stream,
-// and work on the legacy stream is ordered against neither a non-blocking one nor the return of a pageable copy.
-// own_stream: other work may be under way, which this neither waits for nor disturbs (0.2 ms more than on the legacy stream).
-cudaError_t init_build(const StepLaunch &sl, void *ll, void *maps, const void *host_maps, size_t map_bytes, bool own_stream) {
-    cudaStream_t own = nullptr;
-    cudaError_t e = own_stream ? cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) : cudaSuccess;
-    if (e != cudaSuccess) return e;
+// Zeroed exchange buffers (with unit tables) and tensor maps of a build.  Enqueued on the stream of its first launch: the legacy stream is not
+// ordered before a non-blocking one, nor the return of a pageable copy before its transfer.
+cudaError_t init_build(const StepLaunch &sl, void *ll, void *maps, const void *host_maps, size_t map_bytes, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(ll, 0, sl.ll_bytes, s);
+    // (pageable copies: the runtime stages the bytes before returning, so the sources may go)
+    if (e == cudaSuccess) e = cudaMemcpyAsync(maps, host_maps, map_bytes, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess || !sl.unit_tab_bytes) return e;
     std::vector<unsigned> units(sl.unit_tab_bytes / 4);
-    e = cudaMemsetAsync(ll, 0, sl.ll_bytes, own);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(maps, host_maps, map_bytes, cudaMemcpyHostToDevice, own);
-    if (e == cudaSuccess && !units.empty()) {
-        step_unit_table(sl, units.data());
-        e = cudaMemcpyAsync(const_cast<unsigned *>(sl.p.unit_tab), units.data(), sl.unit_tab_bytes, cudaMemcpyHostToDevice, own);
-    }
-    const cudaError_t done = cudaStreamSynchronize(own);
-    if (own) cudaStreamDestroy(own);
-    return e != cudaSuccess ? e : done;
+    step_unit_table(sl, units.data());
+    return cudaMemcpyAsync(const_cast<unsigned *>(sl.p.unit_tab), units.data(), sl.unit_tab_bytes, cudaMemcpyHostToDevice, s);
 }
 
-// Plan and buffers of the build for `mt` tokens per call.  *why: the shape does not fit.
-cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char **why) {
+// Plan and buffers of the build for `mt` tokens per call, ready for launches on `s` (which is not being captured).  *why: the shape does not fit.
+cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, cudaStream_t s, const char **why) {
     int smem_optin = 0, per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
     if (e != cudaSuccess) return e;
@@ -283,7 +276,7 @@ cudaError_t make_build(edgefm_ctx *c, int mt, edgefm_ctx::Build *b, const char *
         const bool sub = c->vocab_subset > 0;
         if (!step_maps(p, c->layers.data(), sub ? static_cast<const void *>(c->sub_lm) : c->lm_head, sub ? c->vocab_subset : c->shape.vocab, maps.data())) return cudaErrorUnknown;
         if (!b->maps && (e = cudaMalloc(reinterpret_cast<void **>(&b->maps), maps.size() * sizeof(CUtensorMap))) != cudaSuccess) return e;
-        if ((e = init_build(sl, b->ll, b->maps, maps.data(), maps.size() * sizeof(CUtensorMap), b == &c->wide)) != cudaSuccess) return e;
+        if ((e = init_build(sl, b->ll, b->maps, maps.data(), maps.size() * sizeof(CUtensorMap), s)) != cudaSuccess) return e;
         p.maps = b->maps;
         p.map_fence = 1;   // edgefm_set_vocab_subset rewrites the output layer's map
     }
@@ -434,7 +427,7 @@ edgefm_status edgefm_create_with_options(const edgefm_shape *shape, const edgefm
     }
     {
         const char *why = nullptr;
-        CREATE_TRY(make_build(c, M, &c->step, &why));
+        CREATE_TRY(make_build(c, M, &c->step, nullptr, &why));
         if (why) return bail(EDGEFM_ERR_BAD_SHAPE, why, cudaErrorInvalidValue);
     }
     CREATE_TRY(cudaDeviceSynchronize());
@@ -524,7 +517,7 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
                                   int32_t *n_accepted_out, int32_t *next_token_out) {
     if (!ctx) return EDGEFM_ERR_INVALID_ARG;
     if (!tokens) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "null tokens");
-    const bool longer = m > ctx->block_tokens;   // than the context's build carries: the build for eight tokens, or the dense path
+    const bool longer = m > ctx->block_tokens;   // than the context's build carries: the build for eight tokens, or the prompt kernels
     if (m < 1 || m > std::max(ctx->block_tokens, PF_VERIFY_MAX))
         return fail(ctx, EDGEFM_ERR_INVALID_ARG, "m = %d: blocks of 1 .. %d tokens", m, std::max(ctx->block_tokens, PF_VERIFY_MAX));
     if (longer && (tokens[0] < 0 || position < 0))
@@ -550,7 +543,7 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
             prompt_kernels = true;
         } else {
             const char *why = nullptr;
-            CUDA_TRY(ctx, make_build(ctx, PF_VERIFY_MAX, &ctx->wide, &why));
+            CUDA_TRY(ctx, make_build(ctx, PF_VERIFY_MAX, &ctx->wide, s, &why));
             prompt_kernels = ctx->wide_refused = why != nullptr;
         }
     }
@@ -615,11 +608,11 @@ edgefm_status edgefm_prefill_tokens(edgefm_ctx *ctx, const int32_t *tokens, int3
     return EDGEFM_OK;
 }
 
-}  // extern "C" (helpers of the dense path follow)
+}  // extern "C" (helpers of the prompt kernels follow)
 
 namespace {
 
-// Work buffers of the dense path (prefill, long verified blocks): allocated at the first use, kept.
+// Work buffers of the prompt kernels (prefill, verified blocks the step kernel does not take): allocated at the first use, kept.
 edgefm_status ensure_prefill_buffers(edgefm_ctx *ctx) {
     if (ctx->pf.chunk == 0) {
         const int chunk = std::min(PF_CHUNK_MAX, ctx->max_context);

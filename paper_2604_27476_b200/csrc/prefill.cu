@@ -1,7 +1,7 @@
 // Prompt processing for sm_100a: KV <- Prefill(x_1:T) (Eq. 3 of the paper).
 //
 // The T given tokens go through the layers together, so every projection is a dense [T x K] x [K x N] contraction:
-//   * prefill_gemm_kernel: one 128 x 128 (gate/up: 128 x 256) output tile per CTA.  A producer thread stages bf16 operand
+//   * prefill_gemm_kernel: persistent, output tiles of 128 x 64, 128 or 256.  A producer thread stages bf16 operand
 //     tiles in shared memory by TMA (128-byte swizzle), one thread issues tcgen05.mma with the fp32 accumulator in tensor
 //     memory, four warps read the accumulator back (tcgen05.ld) and apply the operator's epilogue:
 //       QKV      : + bias, rotate-half RoPE of q and k, q to the work buffer, k and v rows to the cache;

@@ -10,12 +10,12 @@
 namespace edgefm {
 
 constexpr int PF_HEAD_GRID_MAX = 1024;   // CTAs of the output-layer kernels (candidate slots: PF_HEAD_GRID_MAX x PF_VERIFY_MAX)
-constexpr int PF_VERIFY_MAX = 8;         // tokens of a block verified through the dense path
+constexpr int PF_VERIFY_MAX = 8;         // tokens of the longest block that can be verified
 #ifndef PF_CHUNK_MAX_VALUE
 #define PF_CHUNK_MAX_VALUE 4096
 #endif
 constexpr int PF_CHUNK_MAX = PF_CHUNK_MAX_VALUE;   // tokens per pass over the layers (longer prompts take several passes); 4096 instead of
-                                                  // 2048 took a 32768-token prompt of the 1.5B shape from 393 to 351 ms   // tokens per pass over the layers (longer prompts take several passes)
+                                                  // 2048 took a 32768-token prompt of the 1.5B shape from 393 to 351 ms
 
 // Work buffers of one pass, owned by the context, allocated at the first prefill call.
 struct PrefillBuffers {
@@ -79,7 +79,7 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
 const char *prefill_head(const PrefillModel &m, PrefillBuffers *b, int row, const void *final_norm, const void *lm, const int *ids, int rows,
                          float *logits_out, int *next_token_out, int token, int pos, cudaStream_t stream);
 
-// Block verification through the dense path (Sec. 3.11): after prefill_run(..., n tokens, whole_last_layer = true), the logits of
+// Block verification through the prompt kernels (Sec. 3.11): after prefill_run(..., n tokens, whole_last_layer = true), the logits of
 // all n rows ([n][rows], or nullptr), the greedy acceptance on the device and the state update (cache length slot0 + accepted).
 const char *prefill_verify_head(const PrefillModel &m, PrefillBuffers *b, int n, const void *final_norm, const void *lm, const int *ids, int rows,
                                 float *logits_out, int *n_accepted_out, int *next_token_out, int slot0, int pos, cudaStream_t stream);

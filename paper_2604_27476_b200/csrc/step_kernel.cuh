@@ -5,7 +5,7 @@
 // and what an exchange costs.
 //
 //   * Weights (step_feed.cuh).  A CTA owns a contiguous range of the rows of every operator, i.e. a contiguous range of memory.
-//     One thread feeds a ring in shared memory with bulk copies (cp.async.bulk, 24 - 50 KB each) in the order of the whole step --
+//     One thread feeds a ring in shared memory with bulk copies (cp.async.bulk, up to 68 KB each) in the order of the whole step --
 //     QKV rows, this CTA's K/V cache rows, O rows, gate/up rows, down rows, next layer, ..., output layer -- independent of the
 //     computation; another asks L2 for what comes after the ring.  (A bulk copy costs its issuer the same few hundred cycles
 //     whatever its size: measured from L2, 6 / 24 / 48 KB copies from one such loop reached 2.2 / 9 / 18 TB/s over the chip.)
@@ -18,10 +18,11 @@
 //     trip to L2 instead of store, fence, counter, poll, load (a release waits for everything its SM has under way: 0.6 us idle,
 //     2 us while the weights stream).  Vectors that are multiplied next travel as their bf16 pieces, split (and weighted for the norm)
 //     once by the owner instead of by every reader.  Every CTA writes its values into 128-byte lines of its own (packets of several
-//     writers in one line cost 0.3 - 1 us: the pollers' copies of the line are invalidated by every write).
+//     writers in one line cost 0.3 - 1 us: the pollers' copies of the line are invalidated by every write); only the MLP activations
+//     lie in natural order, with two writers in most lines where CTAs meet.
 //     Polling grows with the tokens.  For four and more the owners write such vectors plainly, as the products want them, every CTA
-//     counts up one counter, and a feeding thread that has seen all of them fetches the vector with one bulk copy (a block of four
-//     took 1530 us with packets and 1286 us so, a single token 976 and 1016 us).  MLP activations too long for the shared memory go
+//     counts up one counter, and a feeding thread that has seen all of them fetches the vector with one bulk copy (when
+//     the two were compared a block of four took 1530 us with packets and 1286 us so, a single token 976 and 1016 us).  MLP activations too long for the shared memory go
 //     this way too, by segments.  A buffer is rewritten one layer later; a CTA that writes it then has seen, in
 //     between, an exchange to which every CTA contributes only after reading the old contents.
 //   * Attention (step_attention.cuh).  CTA (token, kv head, chunk) holds the chunk's K/V rows in its ring before the queries exist,

@@ -1,5 +1,5 @@
 """Parity at the sizes of the benchmark configurations (Qwen2.5-shaped decoders), in the launch
-configuration bench.py times: one graph replay per token, tokens chained on the device.
+configuration bench.py times: one launch per token, tokens chained on the device.
 
 Protocol: the oracle free-runs greedily from the seeded first token; the CUDA path is (a) fed the
 oracle's tokens step by step and compared logit by logit, then (b) re-primed and left to run free

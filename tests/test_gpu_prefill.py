@@ -89,7 +89,7 @@ def test_prompt_on_the_1_5b_shape():
 
 
 def test_prompt_behind_a_long_prefix():
-    """8200 prefix rows (the context then runs the long-context build of the step kernel for the prompt's last token): the
+    """8200 prefix rows: the
     queries attend to 65 key blocks, the first 64 of them wholly inside the prefix."""
     run_case(CONFIGS["tiny"].with_(qkv_bias=True), 8200, 150, 9)
 

@@ -199,9 +199,7 @@ def test_statefulness_export_then_prefill():
 
 @pytest.mark.parametrize("variant", ["g2_d64", "g7_d128_bias"])
 def test_long_context_build_crosses_the_attention_mode_switch(variant):
-    """max_context > 8192 selects the long-context build of the kernel (8 warps per CTA, both attention modes).
-    Starting at 8188 cached positions, the steps cross the switch from one-head-per-CTA attention (merged in the
-    O-projection prologue) to grouped attention (merged by the last CTA of a group)."""
+    """Steps that cross 8192 cached positions, each CTA's chunk then holding more than one block of positions."""
     cfg = TINY if variant == "g2_d64" else TINY.with_(n_q_heads=7, n_kv_heads=1, head_dim=128, hidden=320, ffn=512, vocab=3000,
                                                          qkv_bias=True)
     pair = Pair(cfg, seed=77, cache_len=8188, max_context=8200)

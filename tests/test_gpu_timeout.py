@@ -1,5 +1,5 @@
-"""The bounded device-side waits of the step kernel, driven to expiry without any fault: the grid barrier is told to
-expect one arrival more than there are CTAs and the bound is shortened to 2 ms, so the first barrier of the next step
+"""The bounded device-side waits of the step kernel, driven to expiry without any fault: its exchanges are told to expect what no CTA
+sends (another tag; an arrival more than there are CTAs) and the bound is shortened to 2 ms, so the first exchange of the next step
 gives up.  The kernel must return, the status must read EDGEFM_ERR_TIMEOUT, the context must still be destroyable, and a
 fresh context on the same weights must work."""
 import time
@@ -12,7 +12,7 @@ from helpers import Pair, assert_logits_close
 pytestmark = pytest.mark.gpu
 
 
-def test_grid_barrier_wait_expires_and_is_reported():
+def test_exchange_wait_expires_and_is_reported():
     import torch
     from paper_2604_27476_b200 import (DecodeContext, EdgefmError, Status, edgefm_debug_set_wait_limit, edgefm_sync_status)
     cfg = CONFIGS["tiny"]
@@ -24,7 +24,7 @@ def test_grid_barrier_wait_expires_and_is_reported():
         pair.ctx.step(tok, pos)                                   # a normal step first
         edgefm_sync_status(pair.ctx.handle, stream)
         assert_logits_close(pair.ctx.logits.cpu().numpy(), ref, "before")
-        edgefm_debug_set_wait_limit(pair.ctx.handle, 2_000_000, 1)    # 2 ms; the barrier now waits for a CTA that does not exist
+        edgefm_debug_set_wait_limit(pair.ctx.handle, 2_000_000, 1)    # 2 ms; the exchanges now wait for what nobody sends
         t0 = time.perf_counter()
         pair.ctx.step(nxt, pos + 1)
         with pytest.raises(EdgefmError) as ei:

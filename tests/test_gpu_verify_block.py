@@ -1,5 +1,5 @@
-"""Block verification (Sec. 3.11 of the paper): two tokens pass through the step kernel in one call, the weights streamed
-once.  The oracle verifies the block as the paper states it, token by token with plain decode steps; the draft model is not
+"""Block verification (Sec. 3.11 of the paper): two to eight tokens pass through the step kernel in one call, the weights streamed
+once; where a shape does not fit the build for eight, through the prompt kernels.  The oracle verifies the block as the paper states it, token by token with plain decode steps; the draft model is not
 part of either side, proposals are made here (the oracle's own greedy token = a proposal that must be accepted, anything
 else = one that must be rejected)."""
 import numpy as np
@@ -95,13 +95,13 @@ def test_block_calls_are_validated():
     block = Pair(cfg, cache_len=3, max_context=4, block_tokens=2)
     try:
         with pytest.raises(EdgefmError) as ei:
-            plain.ctx.verify_block([-1, 2], -1)                    # a plain context verifies through the dense path: tokens must be given
+            plain.ctx.verify_block([-1, 2], -1)                    # longer than the context's build carries: tokens must be given
         assert ei.value.status == Status.ERR_INVALID_ARG
         with pytest.raises(EdgefmError) as ei:
             block.ctx.verify_block(list(range(1, 10)), 3)          # more than eight tokens
         assert ei.value.status == Status.ERR_INVALID_ARG
         with pytest.raises(EdgefmError) as ei:
-            block.ctx.verify_block([1, 2, 3], 3)                   # the dense path for three tokens, one free slot
+            block.ctx.verify_block([1, 2, 3], 3)                   # the build for eight tokens, one free slot
         assert ei.value.status == Status.ERR_CONTEXT_FULL
         with pytest.raises(EdgefmError) as ei:
             block.ctx.verify_block([1, cfg.vocab], 3)
@@ -211,12 +211,28 @@ def test_blocks_of_four_match_the_oracle_verification(name):
         pair.close()
 
 
-@pytest.mark.parametrize("name,kv_format", [("tiny", None), ("tiny", "int8"), ("qwen2.5-1.5b", None)])
-def test_blocks_of_up_to_eight_tokens_through_the_dense_path(name, kv_format):
-    """Blocks longer than the context's block_tokens (here a plain context) are verified by the prefill kernels: all m tokens
-    through the layers together, one pass over the output matrix for all rows, the acceptance rule on the device."""
+# a shape whose vectors for eight tokens do not fit the shared memory: its blocks take the prompt kernels
+DENSE = CONFIGS["tiny"].with_(hidden=6144, ffn=1024, vocab=1500, n_layers=2, qkv_bias=True)
+
+
+def has_eight_token_build(cfg, max_context, kv_format):
+    from paper_2604_27476_b200 import EdgefmError, edgefm_debug_step_plan
+    shape = dict(n_layers=cfg.n_layers, hidden=cfg.hidden, n_q_heads=cfg.n_q_heads, n_kv_heads=cfg.n_kv_heads, head_dim=cfg.head_dim, ffn=cfg.ffn,
+                 vocab=cfg.vocab, rms_eps=cfg.rms_eps, rope_theta=cfg.rope_theta, qkv_bias=int(cfg.qkv_bias))
+    try:
+        return bool(edgefm_debug_step_plan(shape, max_context, kv_format or "bf16", tokens=8))
+    except EdgefmError:
+        return False
+
+
+@pytest.mark.parametrize("name,kv_format", [("tiny", None), ("tiny", "int8"), ("qwen2.5-1.5b", None), ("dense", None), ("dense", "int8")])
+def test_blocks_of_up_to_eight_tokens(name, kv_format):
+    """Blocks longer than the context's block_tokens (here a plain context): the build of the step kernel for eight tokens or, "dense", the prompt
+    kernels (all m tokens through the layers together, one pass over the output matrix for all rows), the acceptance rule on the
+    device."""
     import torch
-    cfg = CONFIGS[name] if name != "tiny" else CONFIGS[name].with_(qkv_bias=True)
+    cfg = DENSE if name == "dense" else CONFIGS[name] if name != "tiny" else CONFIGS[name].with_(qkv_bias=True)
+    assert has_eight_token_build(cfg, 104, kv_format) == (name != "dense")
     T0 = 40
     pair = Pair(cfg, cache_len=T0, max_context=T0 + 64, kv_format=kv_format)
     try:
@@ -264,12 +280,14 @@ def test_blocks_of_up_to_eight_tokens_through_the_dense_path(name, kv_format):
         pair.close()
 
 
-def test_dense_block_with_a_pruned_output_layer():
-    """The dense path on a context whose output layer is pruned: greedy tokens and acceptance are taken over the subset (here every
+@pytest.mark.parametrize("dense", [False, True])
+def test_long_block_with_a_pruned_output_layer(dense):
+    """Both paths of long blocks on a context whose output layer is pruned: greedy tokens and acceptance are taken over the subset (here every
     second id plus the oracle's own choices, so that the oracle's unrestricted verification stays the reference)."""
     import torch
-    cfg = CONFIGS["tiny"].with_(qkv_bias=True)
+    cfg = DENSE if dense else CONFIGS["tiny"].with_(qkv_bias=True)
     T0 = 24
+    assert has_eight_token_build(cfg, T0 + 16, None) == (not dense)
     pair = Pair(cfg, cache_len=T0, max_context=T0 + 16)
     try:
         tok, pos, m = 17, T0 + 2, 6

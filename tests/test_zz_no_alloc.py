@@ -25,7 +25,7 @@ def test_static_scratch_step_matches_context_step_twice(variant):
     if variant == "far_tables":       # the unit tables lie in the scratch array, too
         cfg = cfg.with_(hidden=24056, ffn=160, vocab=300, n_layers=1)
     T0, Tmax = cfg.cache_len, cfg.cache_len + 4
-    if variant == "long_context_build":   # max_context > 8192 selects the other build of the kernel
+    if variant == "long_context_build":   # a cache for more than 8192 positions
         T0, Tmax = 300, 8300
     pair = Pair(cfg, cache_len=T0, max_context=Tmax)
     try:

@@ -828,6 +828,17 @@ edgefm_status edgefm_debug_prefill_plan(int32_t epilogue, int32_t M, int32_t N, 
     return EDGEFM_OK;
 }
 
+edgefm_status edgefm_debug_prefill_launch(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t *out5) {
+    if (!out5 || epilogue < 0 || epilogue > 3 || M < 1 || N < 1 || K < 1 || num_sms < 1) return EDGEFM_ERR_INVALID_ARG;
+    const PrefillPlan p = prefill_plan(epilogue == 3 ? 0 : epilogue, epilogue == 3 ? 64 : 128, M, N, K, num_sms);
+    out5[0] = p.columns;
+    out5[1] = p.splits;
+    out5[2] = p.cluster;
+    out5[3] = p.pairs;
+    out5[4] = p.swap;
+    return EDGEFM_OK;
+}
+
 edgefm_status edgefm_export_kv(edgefm_ctx *ctx, void *k_out, void *v_out, void *stream) {
     if (!ctx) return EDGEFM_ERR_INVALID_ARG;
     if (!k_out || !v_out) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "null output");

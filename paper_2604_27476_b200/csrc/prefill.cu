@@ -1,15 +1,17 @@
 // Prompt processing for sm_100a: KV <- Prefill(x_1:T) (Eq. 3 of the paper).
 //
 // The T given tokens go through the layers together, so every projection is a dense [T x K] x [K x N] contraction:
-//   * prefill_gemm_kernel: persistent, output tiles of 128 x 64, 128 or 256.  A producer thread stages bf16 operand
+//   * prefill_gemm_kernel: persistent, output tiles of 128 x 128 or 256.  A producer thread stages bf16 operand
 //     tiles in shared memory by TMA (128-byte swizzle), one thread issues tcgen05.mma with the fp32 accumulator in tensor
 //     memory, four warps read the accumulator back (tcgen05.ld) and apply the operator's epilogue:
 //       QKV      : + bias, rotate-half RoPE of q and k, q to the work buffer, k and v rows to the cache;
-//       O / down : added to the fp32 residual stream;
+//       O / down : added to the fp32 residual stream; the rows the next contraction reads (x * w, for the norm) with their sums of squares;
 //       gate/up  : SwiGLU, silu(gate) * up, to the bf16 activation buffer.
+//     RMSNorm's factor 1 / rms multiplies the results of QKV and gate/up instead of their operand rows.
+//   * prefill_tile_kernel: the same contractions where the tiles fit the SMs in one round: clusters of CTAs share the K of a tile.
 //   * prefill_attention_tc_kernel: causal attention of the T queries over the cache rows (prefix + the T new rows), also on
 //     tcgen05: S = Q K^T and O = P V in tensor memory, online softmax by warps that own the rows (see the kernel).
-//   * rmsnorm / embedding kernels: one row per warp.
+//   * prefill_norm_kernel: embedding, and the norm behind a contraction that leaves K-split partial sums; one CTA per row.
 // Every activation enters the tensor cores as TWO bf16 pieces (hi + lo, 16 mantissa bits; twice the multiplies, one load of
 // the weight tile), because single bf16 activations put the logits of a 28-layer model outside the step's tolerance
 // (measured: 3.6e-2 max-abs).  The residual stream stays fp32.
@@ -65,8 +67,10 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
 }
 
 // Programmatic dependent launch: every kernel of the prefill chain lets its successor be launched as soon as all of its own CTAs
-// have started (pdl_trigger, first statement), and touches global memory only after its predecessor has completed and its writes
-// are visible (pdl_wait).  What overlaps is the successor's launch and set-up (barriers, tensor memory, descriptor fetch).
+// have started (pdl_trigger), and touches what other kernels write only after its predecessor has completed and its writes are visible
+// (pdl_wait).  What overlaps is the successor's launch and set-up (barriers, tensor memory, descriptor fetch, first weight tiles).  A kernel
+// that allocates tensor memory triggers behind the allocation: several kernels may be resident on an SM at once, and one that waits for
+// its predecessor must never hold the columns the predecessor still needs.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -94,6 +98,32 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+// The same over a pair of CTAs (a cluster of two): 256 x N x 16, issued by the first.  Either CTA holds 128 rows of A, half of B's rows and
+// its own rows of the accumulator, at the same places.
+__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// one arrival at the barrier of both CTAs when the pair's multiplies issued so far have finished
+__device__ __forceinline__ void umma_commit_pair(uint64_t *bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+                 "h"(static_cast<uint16_t>(3))
+                 : "memory");
+}
+// a tile into this CTA's shared memory, its bytes counted at a barrier of the pair's first CTA (a shared::cluster address)
+__device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(map), "r"(x), "r"(y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // The mbarrier receives one arrival when every tcgen05.mma issued so far by this thread has finished.
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
@@ -486,6 +516,12 @@ struct GemmArgs {
     int *error;
     uint32_t wait_limit;      // polls a wait on an mbarrier may take
     uint32_t extra_arrivals;  // 0; 1 (tests): the stage barriers expect an arrival nobody makes, so the first wait runs out
+    // RMSNorm of the operand rows, where the contraction before left x * w without the factor 1 / rms (a factor of the whole row, so it
+    // may as well multiply the row's results): sums of squares of its pieces, [ss_pieces][ss_stride]; null = rows are normalised
+    const float *ss_in;
+    int ss_pieces;
+    size_t ss_stride;
+    float eps;
     // QKV
     const uint16_t *bias;     // [N] or null
     const float2 *rope;       // [M][d/2]
@@ -498,56 +534,223 @@ struct GemmArgs {
     long long head_stride;
     // O / down
     float *resid;             // [M][N]
+    const uint16_t *norm_w;   // weights of the norm that follows, or null; then the epilogue also leaves
+    uint16_t *xw;             // ... x * w of the new residual stream, [2][..][N]: hi and lo planes
+    size_t x_plane;
+    float *ss_out;            // ... and the sums of squares of its pieces (at most 64 columns of a tile), [piece][ss_stride]
     int splits;               // K split into this many units per output tile (1 = none).  With a split the units write their
     float *part;              // partial sums to part[split][..][N] (planes `part_plane` elements apart) instead of adding to resid;
     size_t part_plane;        // the norm kernel that follows adds the planes to the residual stream in a fixed order.
     // gate/up
     uint16_t *act;            // [2][..][N]: hi and lo planes
     size_t act_plane;
+    int bn;                   // output columns of a tile: 64, 128 or 256; pairs that add to the residual stream: any multiple of 16 from 128 to 256
+    // prefill_tile_kernel
+    int cluster;              // CTAs that share the K of an output tile
+    int a_rows;               // rows of an activation tile that are loaded (a multiple of 8, at most 128)
+    int tmem_cols;            // tensor memory a CTA allocates (a power of two)
+    int stages;
 };
 
 constexpr int PF_BM = 128, PF_BK = 64;
 constexpr int PF_SPLIT_MAX = 8;               // K splits of a contraction that adds to the residual stream: up to 4, up to 8 when the
                                              // tokens fit one row tile (short prompts, verified blocks: the grids are smallest there)
 
+// ---- epilogues: eight lanes take a row, four rows per warp and step -----------------------------------------------------------
+// Accumulators come out of tensor memory a row per thread; stored like that, an instruction touches 32 lines (1.5B shape, 2048 tokens:
+// O took 43 us and the norm behind it 6, now 29 together; QKV 37, now 33).  So a chunk of 64 accumulator columns passes through
+// shared memory, and a lane then holds four consecutive columns of each of the chunk's two 32-column halves (a, b): 64 to 128 bytes of
+// a row per eight lanes.  The halves are the pairs an operator needs together: gate and up, or the two halves of a rotated head.
+template <int EPI, int N_STEP> __device__ __forceinline__ void chunk_halves(int chunk, int d, int &a, int &b) {
+    if (EPI == EPI_SWIGLU) { a = 32 * chunk; b = N_STEP + 32 * chunk; }
+    else if (EPI == EPI_QKV && d == 128) { a = (chunk >> 1) * 128 + (chunk & 1) * 32; b = a + 64; }
+    else { a = 64 * chunk; b = a + 32; }
+}
+// what a lane needs besides the accumulators: of its columns (biases, norm weights), and of a row and its columns (residuals, rotation)
+struct ColVals { uint2 a, b; };
+struct RowVals { float4 a, b; };
+
+template <int EPI> __device__ __forceinline__ ColVals load_cols(const GemmArgs &g, int col_a, int col_b) {
+    ColVals c{make_uint2(0u, 0u), make_uint2(0u, 0u)};
+    const uint16_t *v = EPI == EPI_QKV ? g.bias : EPI == EPI_RESID ? g.norm_w : nullptr;
+    if (v && col_a < g.N) c.a = *reinterpret_cast<const uint2 *>(v + col_a);
+    if (v && col_b < g.N) c.b = *reinterpret_cast<const uint2 *>(v + col_b);
+    return c;
+}
+template <int EPI> __device__ __forceinline__ RowVals load_row(const GemmArgs &g, int row, int col_a, int col_b) {
+    RowVals r;
+    r.a = r.b = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row >= g.M) return r;
+    if (EPI == EPI_RESID && g.splits == 1) {
+        const float *p = g.resid + static_cast<size_t>(row) * g.N;
+        if (col_a < g.N) r.a = *reinterpret_cast<const float4 *>(p + col_a);
+        if (col_b < g.N) r.b = *reinterpret_cast<const float4 *>(p + col_b);
+    } else if (EPI == EPI_QKV && col_a < (g.nq + g.nkv) * g.d) {          // (cos, sin) of four pairs
+        const float4 *p = reinterpret_cast<const float4 *>(g.rope + static_cast<size_t>(row) * (g.d >> 1) + (col_a & (g.d - 1)));
+        r.a = p[0];
+        r.b = p[1];
+    }
+    return r;
+}
+__device__ __forceinline__ void store_split4(uint16_t *p, size_t plane, const float *v) {
+    uint2 hi, lo;
+    split2x2(v[0], v[1], hi.x, lo.x);
+    split2x2(v[2], v[3], hi.y, lo.y);
+    *reinterpret_cast<uint2 *>(p) = hi;
+    *reinterpret_cast<uint2 *>(p + plane) = lo;
+}
+__device__ __forceinline__ uint2 pack4_bf16(const float *v) { return make_uint2(pack2_bf16(v[0], v[1]), pack2_bf16(v[2], v[3])); }
+__device__ __forceinline__ void unpack4(uint2 u, float *v) { v[0] = bf16lo(u.x); v[1] = bf16hi(u.x); v[2] = bf16lo(u.y); v[3] = bf16hi(u.y); }
+
+// A lane's eight results of one row (output columns col_a .. col_a + 3 and col_b .. col_b + 3; gate/up: column col_a of both).  rs: 1 / rms
+// of the operand row.  Returns the lane's share of the row's sum of squares (EPI_RESID with norm_w).
+template <int EPI>
+__device__ __forceinline__ float finish_row(const GemmArgs &g, int row, int col_a, int col_b, float4 va, float4 vb, const ColVals &cv,
+                                            const RowVals &rv, float rs, int split) {
+    float a[4] = {va.x, va.y, va.z, va.w}, b[4] = {vb.x, vb.y, vb.z, vb.w}, ss = 0.f;
+    if (row >= g.M) return ss;
+    if constexpr (EPI == EPI_RESID) {
+        if (g.splits > 1) {              // a partial sum: added to the stream by the norm kernel
+            float *p = g.part + split * g.part_plane + static_cast<size_t>(row) * g.N;
+            if (col_a < g.N) *reinterpret_cast<float4 *>(p + col_a) = va;
+            if (col_b < g.N) *reinterpret_cast<float4 *>(p + col_b) = vb;
+            return ss;
+        }
+        auto half = [&](float *v, float4 r, uint2 w4, int col) {
+            if (col >= g.N) return;
+            v[0] += r.x; v[1] += r.y; v[2] += r.z; v[3] += r.w;
+            *reinterpret_cast<float4 *>(g.resid + static_cast<size_t>(row) * g.N + col) = make_float4(v[0], v[1], v[2], v[3]);
+            if (!g.norm_w) return;
+            float w[4];
+            unpack4(w4, w);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { ss = fmaf(v[i], v[i], ss); w[i] *= v[i]; }
+            store_split4(g.xw + static_cast<size_t>(row) * g.N + col, g.x_plane, w);
+        };
+        half(a, rv.a, cv.a, col_a);
+        half(b, rv.b, cv.b, col_b);
+    } else if constexpr (EPI == EPI_LOGITS) {   // N need not be a multiple of 4 (a pruned vocabulary): scalar stores
+        float *p = g.resid + static_cast<size_t>(row) * g.N;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (col_a + i < g.N) p[col_a + i] = a[i];
+            if (col_b + i < g.N) p[col_b + i] = b[i];
+        }
+    } else if constexpr (EPI == EPI_SWIGLU) {
+        if (col_a < g.N) {
+            float o[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float gate = a[i] * rs, up = b[i] * rs;
+                o[i] = gate / (1.f + __expf(-gate)) * up;
+            }
+            store_split4(g.act + static_cast<size_t>(row) * g.N + col_a, g.act_plane, o);
+        }
+    } else {                             // EPI_QKV: the chunk's halves are the two halves of (32 pairs of) a head; N is whole heads
+        float ba[4], bb[4];
+        unpack4(cv.a, ba);
+        unpack4(cv.b, bb);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { a[i] = fmaf(a[i], rs, ba[i]); b[i] = fmaf(b[i], rs, bb[i]); }
+        const int head = col_a / g.d, j = col_a & (g.d - 1), jb = j + (col_b - col_a);
+        if (head < g.nq + g.nkv) {       // q or k: rotate-half pairs (j, j + d/2)
+            const float c[4] = {rv.a.x, rv.a.z, rv.b.x, rv.b.z}, s[4] = {rv.a.y, rv.a.w, rv.b.y, rv.b.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float x = a[i], y = b[i];
+                a[i] = x * c[i] - y * s[i];
+                b[i] = y * c[i] + x * s[i];
+            }
+            if (head < g.nq) {           // queries keep both pieces
+                uint16_t *dst = g.q_out + static_cast<size_t>(row) * g.nq * g.d + static_cast<size_t>(head) * g.d;
+                store_split4(dst + j, g.q_plane, a);
+                store_split4(dst + jb, g.q_plane, b);
+                return ss;
+            }
+        }
+        const bool is_v = head >= g.nq + g.nkv;
+        const int hk = head - g.nq - (is_v ? g.nkv : 0);
+        if (float *f = is_v ? g.v_stage : g.k_stage) {   // compressed cache: fp32 rows for the quantiser
+            f += hk * g.stage_stride + static_cast<size_t>(row) * g.d;
+            *reinterpret_cast<float4 *>(f + j) = make_float4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<float4 *>(f + jb) = make_float4(b[0], b[1], b[2], b[3]);
+        } else {
+            uint16_t *dst = (is_v ? g.v_rows : g.k_rows) + hk * g.head_stride + static_cast<size_t>(row) * g.d;
+            *reinterpret_cast<uint2 *>(dst + j) = pack4_bf16(a);
+            *reinterpret_cast<uint2 *>(dst + jb) = pack4_bf16(b);
+        }
+    }
+    return ss;
+}
+// 1 / rms of an operand row from the sums of squares of its pieces
+__device__ __forceinline__ float row_scale(const GemmArgs &g, int row) {
+    if (!g.ss_in || row >= g.M) return 1.f;
+    float ss = 0.f;
+#pragma unroll 4
+    for (int t = 0; t < g.ss_pieces; ++t) ss += g.ss_in[t * g.ss_stride + row];
+    return rsqrtf(ss / static_cast<float>(g.K) + g.eps);
+}
+// the sum over the eight lanes of a row, stored by the first of them
+__device__ __forceinline__ void store_row_ss(const GemmArgs &g, float ss, int row, int piece, int lane) {
+    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 4);
+    if ((lane & 7) == 0 && row < g.M) g.ss_out[piece * g.ss_stride + row] = ss;
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+    cluster_arrive();
+    cluster_wait();
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {   // the same place in the shared memory of another CTA of the cluster
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
 // Tile shapes.  PF_NARROW: 128 output columns, 4 stages of 48 KB.  PF_WIDE: 256 output columns, 3 stages of 64 KB: per k-block
 // 64 KB of operands feed twice the multiplies of a narrow tile's 48 KB, which matters because operand delivery from L2, not
 // the tensor pipe, bounds the narrow tiles.  Gate/up runs wide: 128 gate columns and their 128 up partners.
-// Few tokens leave most SMs idle with these tiles, and the pass is a chain of latencies: every CTA pulls its whole K through one SM
-// (77 tokens, 0.5B shape: QKV on 9 CTAs 17 us, O on 7 CTAs 22 us, gate/up on 38 CTAs 23 us).  Where tiles of half the columns still
-// fit the SMs in one round they are taken: PF_SLIM, 64 columns, or PF_NARROW for gate/up, 64 + 64.
+// PAIR: two row tiles, one in either CTA of a cluster of two, multiplied together (cta_group::2): a CTA fetches half of the weight tile only,
+// 48 KB per k-block instead of 64, which leaves room for a fourth stage (gate/up and QKV by single CTAs, the rest by pairs: 4200 tokens, 7B
+// shape, 97.2 ms, all by pairs 94.8; 1000 tokens, 3B, 12.60 and 12.43; these passes run into the power limit).
 // The kernel is persistent (one CTA per SM, tiles dealt round-robin, neighbours sharing a weight tile) with TWO accumulators
 // in tensor memory, so that the epilogue of a tile runs under the main loop of the next.
-template <int SHAPE> struct GemmCfg {
-    static constexpr int BN = SHAPE == PF_WIDE ? 256 : SHAPE == PF_SLIM ? 64 : 128;
-    static constexpr int STAGES = SHAPE == PF_WIDE ? 3 : SHAPE == PF_SLIM ? 5 : 4;
-    static constexpr int A_BYTES = PF_BM * PF_BK * 2, B_BYTES = BN * PF_BK * 2;
+template <int SHAPE, bool PAIR> struct GemmCfg {
+    static constexpr int BN = SHAPE == PF_WIDE ? 256 : 128;
+    static constexpr int STAGES = SHAPE == PF_WIDE && !PAIR ? 3 : 4;
+    static constexpr int A_BYTES = PF_BM * PF_BK * 2, B_BYTES = BN * PF_BK * 2 / (PAIR ? 2 : 1);
     static constexpr int STAGE_BYTES = 2 * A_BYTES + B_BYTES;          // A hi, A lo, B
-    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;   // + room to align the first stage to 1024 bytes
+    static constexpr int CHUNK_BYTES = PF_BM * 64 * 4;                 // the epilogue's chunk of 64 columns
+    static constexpr int SMEM = STAGES * STAGE_BYTES + CHUNK_BYTES + 1024;   // + room to align the first stage to 1024 bytes
 };
 
-template <int EPI, int SHAPE>
+template <int EPI, int SHAPE, bool PAIR>
 __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant__ CUtensorMap map_a_hi,
                                                            const __grid_constant__ CUtensorMap map_a_lo,
                                                            const __grid_constant__ CUtensorMap map_b, const GemmArgs g) {
-    pdl_trigger();
-    using C = GemmCfg<SHAPE>;
-    static_assert(EPI != EPI_SWIGLU || SHAPE != PF_SLIM, "gate and up share one accumulator");
-    constexpr int N_STEP = EPI == EPI_SWIGLU ? C::BN / 2 : C::BN;   // output columns (of g.N) a CTA covers
+    using C = GemmCfg<SHAPE, PAIR>;
+    static_assert(!PAIR || SHAPE == PF_WIDE, "a CTA of a pair fetches 128 of the 256 columns");
+    const int BN = PAIR && EPI == EPI_RESID ? g.bn : C::BN;
+    const int N_STEP = EPI == EPI_SWIGLU ? C::BN / 2 : BN;          // output columns (of g.N) a tile covers
+    constexpr int CTAS = PAIR ? 2 : 1, TILE_M = CTAS * PF_BM;
     extern __shared__ uint8_t pf_dyn[];
     __shared__ uint64_t full_bar[C::STAGES], empty_bar[C::STAGES], acc_full[2], acc_empty[2], drain_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     uint8_t *tiles = pf_dyn + ((1024u - (smem_u32(pf_dyn) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m_tiles = (g.M + PF_BM - 1) / PF_BM, n_tiles = (g.N + N_STEP - 1) / N_STEP;
+    const int rank = PAIR ? blockIdx.x & 1 : 0, worker = blockIdx.x / CTAS, workers = gridDim.x / CTAS;
+    const int m_tiles = (g.M + TILE_M - 1) / TILE_M, n_tiles = (g.N + N_STEP - 1) / N_STEP;
     const int KB = (g.K + PF_BK - 1) / PF_BK;
     const int splits = EPI == EPI_RESID ? g.splits : 1;
-    const int my_tiles = (m_tiles * n_tiles * splits - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
-    // unit u of the grid-wide list: row tile u % m_tiles (neighbouring CTAs share a weight tile), then the K split, then the column tile
+    const int my_tiles = (m_tiles * n_tiles * splits - worker + workers - 1) / workers;
+    // unit u of the grid-wide list: row tile u % m_tiles (neighbours share a weight tile), then the K split, then the column tile
     auto unit_of = [&](int i, int &m0, int &n0, int &kb0, int &kb1) {
-        const int u = blockIdx.x + i * gridDim.x, rest = u / m_tiles, sp = rest % splits;
-        m0 = (u % m_tiles) * PF_BM;
+        const int u = worker + i * workers, rest = u / m_tiles, sp = rest % splits;
+        m0 = (u % m_tiles) * TILE_M + rank * PF_BM;
         n0 = (rest / splits) * N_STEP;
         kb0 = sp * KB / splits;
         kb1 = (sp + 1) * KB / splits;
@@ -557,22 +760,28 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
     if (threadIdx.x == 0) {
         prefetch_map(&map_a_hi); prefetch_map(&map_a_lo); prefetch_map(&map_b);
         for (int s = 0; s < C::STAGES; ++s) { mbar_init(&full_bar[s], 1 + g.extra_arrivals); mbar_init(&empty_bar[s], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4 * CTAS); }
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {   // two accumulators: 2 BN columns of tensor memory, 128 lanes
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(2 * C::BN) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(2 * C::BN) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(2 * C::BN) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) cluster_sync(); else __syncthreads();   // a pair: the peer's barriers and tensor memory are there, too
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    pdl_wait();   // set-up done; from here on the kernel reads what its predecessor wrote
+    pdl_trigger();   // (behind the allocation: see pdl_trigger)
+    pdl_wait();      // set-up done; from here on the kernel reads what its predecessor wrote
 
-    if (warp == 0 && lane == 0) {            // producer: operand tiles by TMA
+    if (warp == 0 && lane == 0) {            // producer: operand tiles by TMA; a pair's bytes are counted by its first CTA
         bool ok = true;
         int issued = 0;
         for (int i = 0, it = 0; i < my_tiles && ok; ++i) {
@@ -582,22 +791,39 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
             const int s = it % C::STAGES;
             if (it >= C::STAGES && !mbar_wait(&empty_bar[s], ((it / C::STAGES) - 1) & 1, &abort_flag, g.wait_limit)) { ok = false; break; }
             uint8_t *a = tiles + s * C::STAGE_BYTES, *b = a + 2 * C::A_BYTES;
-            mbar_expect_tx(&full_bar[s], C::STAGE_BYTES);
-            tma_load_2d(a, &map_a_hi, kb * PF_BK, m0, &full_bar[s]);
-            tma_load_2d(a + C::A_BYTES, &map_a_lo, kb * PF_BK, m0, &full_bar[s]);
-            tma_load_2d(b, &map_b, kb * PF_BK, n0, &full_bar[s]);
-            if (EPI == EPI_SWIGLU) tma_load_2d(b + N_STEP * PF_BK * 2, &map_b, kb * PF_BK, g.N + n0, &full_bar[s]);
-            else if (C::BN == 256) tma_load_2d(b + 128 * PF_BK * 2, &map_b, kb * PF_BK, 128 + n0, &full_bar[s]);
+            if (rank == 0) mbar_expect_tx(&full_bar[s], PAIR ? 2 * (2 * C::A_BYTES + BN * PF_BK) : C::STAGE_BYTES);
+            if constexpr (PAIR) {
+                // B's rows: the first half here, the others in the peer (gate/up: the gate columns, the up columns)
+                const uint32_t bar = cluster_addr(smem_u32(&full_bar[s]), 0);
+                tma_load_2d_pair(a, &map_a_hi, kb * PF_BK, m0, bar);
+                tma_load_2d_pair(a + C::A_BYTES, &map_a_lo, kb * PF_BK, m0, bar);
+                tma_load_2d_pair(b, &map_b, kb * PF_BK, n0 + rank * (EPI == EPI_SWIGLU ? g.N : BN / 2), bar);
+            } else {
+                tma_load_2d(a, &map_a_hi, kb * PF_BK, m0, &full_bar[s]);
+                tma_load_2d(a + C::A_BYTES, &map_a_lo, kb * PF_BK, m0, &full_bar[s]);
+                tma_load_2d(b, &map_b, kb * PF_BK, n0, &full_bar[s]);
+                if (EPI == EPI_SWIGLU) tma_load_2d(b + N_STEP * PF_BK * 2, &map_b, kb * PF_BK, g.N + n0, &full_bar[s]);
+                else if (C::BN == 256) tma_load_2d(b + 128 * PF_BK * 2, &map_b, kb * PF_BK, 128 + n0, &full_bar[s]);
+            }
             issued = it + 1;
           }
         }
         if (abort_flag) {   // giving up: the copies still in flight must land before the CTA's shared memory is released
             int dummy = 0;
-            for (int j = issued > C::STAGES ? issued - C::STAGES : 0; j < issued; ++j)
-                mbar_wait(&full_bar[j % C::STAGES], (j / C::STAGES) & 1, &dummy, g.wait_limit);
+            if (rank == 0)
+                for (int j = issued > C::STAGES ? issued - C::STAGES : 0; j < issued; ++j)
+                    mbar_wait(&full_bar[j % C::STAGES], (j / C::STAGES) & 1, &dummy, g.wait_limit);
+            // a pair's copies are counted by the first CTA, which may have given up before it expected all of them: they land within
+            // microseconds, the pair leaves together 0.2 ms later
+            if (PAIR)
+                for (const long long t0 = clock64(); clock64() - t0 < 400000;) { }
         }
-    } else if (warp == 1 && lane == 0) {     // issuer: per stage 4 tcgen05.mma (K = 16 each) for the hi pieces, 4 for the lo pieces
-        constexpr uint32_t idesc = umma_idesc_bf16(PF_BM, C::BN);
+    } else if (warp == 1 && lane == 0 && rank == 0) {     // issuer: per stage 4 tcgen05.mma (K = 16 each) for the hi pieces, 4 for the lo pieces
+        const uint32_t idesc = umma_idesc_bf16(TILE_M, BN);
+        auto mma = [&](uint32_t acc, uint64_t da, uint64_t db, uint32_t accumulate) {
+            if constexpr (PAIR) umma_bf16_pair(acc, da, db, idesc, accumulate); else umma_bf16(acc, da, db, idesc, accumulate);
+        };
+        auto commit = [&](uint64_t *bar) { if constexpr (PAIR) umma_commit_pair(bar); else umma_commit(bar); };
         bool ok = true;
         for (int i = 0, it = 0; i < my_tiles && ok; ++i) {
           const int buf = i & 1;
@@ -615,192 +841,302 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
             const uint32_t a = smem_u32(tiles + s * C::STAGE_BYTES), b = a + 2 * C::A_BYTES;
             const uint64_t da = umma_desc_sw128(a), dl = umma_desc_sw128(a + C::A_BYTES), db = umma_desc_sw128(b);
 #pragma unroll
-            for (int k = 0; k < PF_BK / 16; ++k) umma_bf16(acc, da + 2 * k, db + 2 * k, idesc, ((kb - kb0) | k) != 0);
+            for (int k = 0; k < PF_BK / 16; ++k) mma(acc, da + 2 * k, db + 2 * k, ((kb - kb0) | k) != 0);
 #pragma unroll
-            for (int k = 0; k < PF_BK / 16; ++k) umma_bf16(acc, dl + 2 * k, db + 2 * k, idesc, 1);
-            umma_commit(&empty_bar[s]);      // the stage is free again when these have read it
+            for (int k = 0; k < PF_BK / 16; ++k) mma(acc, dl + 2 * k, db + 2 * k, 1);
+            commit(&empty_bar[s]);           // the stage is free again when these have read it
           }
-          if (ok) umma_commit(&acc_full[buf]);
+          if (ok) commit(&acc_full[buf]);
         }
         if (!ok) {          // giving up: the multiplies already issued must finish before the tensor memory is freed
             int dummy = 0;
-            umma_commit(&drain_bar);
+            commit(&drain_bar);
             mbar_wait(&drain_bar, 0, &dummy, g.wait_limit);
         }
     } else if (warp >= 2) {                  // epilogue: warp w may read lanes 32 (w % 4) .. + 31 of tensor memory
-      const int quarter = warp & 3;
+      const int quarter = warp & 3, sub = lane >> 3, c8 = lane & 7;
+      float4 *chunk = reinterpret_cast<float4 *>(tiles + C::STAGES * C::STAGE_BYTES) + quarter * 32 * 16;   // this warp's 32 rows x 64 columns
       for (int i = 0; i < my_tiles; ++i) {
         int m0, n0, kb0, kb1;
         const int sp = unit_of(i, m0, n0, kb0, kb1), buf = i & 1;
+        const float rs_own = EPI == EPI_QKV || EPI == EPI_SWIGLU ? row_scale(g, m0 + quarter * 32 + lane) : 1.f;
         const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (i >> 1) & 1, &abort_flag, g.wait_limit));   // warp-uniform: tcgen05.ld is .aligned
         if (!ok) break;
         tc_fence_after();
-        const int row = m0 + quarter * 32 + lane;
-        const bool live = row < g.M;
         const uint32_t trow = tmem + buf * C::BN + (static_cast<uint32_t>(quarter * 32) << 16);
-        {
-            if (EPI == EPI_RESID) {
-                for (int c = 0; c < N_STEP / 32; ++c) {
-                    const int n = n0 + c * 32;
-                    if (n >= g.N) break;
-                    float v[32];
-                    tmem_ld32(trow + c * 32, v);
-                    tmem_ld_wait();
-                    if (live && splits > 1) {   // a partial sum: stored, added to the stream by the norm kernel
-                        float4 *p = reinterpret_cast<float4 *>(g.part + sp * g.part_plane + static_cast<size_t>(row) * g.N + n);
+        for (int ch = 0; ch < (BN + 63) / 64; ++ch) {
+            int ca, cb;
+            chunk_halves<EPI, EPI == EPI_SWIGLU ? C::BN / 2 : C::BN>(ch, g.d, ca, cb);
+            if (n0 + ca >= g.N) break;
+            int col_a = n0 + ca + 4 * c8, col_b = n0 + cb + 4 * c8;
+            if (PAIR && EPI == EPI_RESID) {          // the last chunk may reach past the tile
+                if (ca + 4 * c8 >= BN) col_a = g.N;
+                if (cb + 4 * c8 >= BN) col_b = g.N;
+            }
+            const ColVals cv = load_cols<EPI>(g, col_a, col_b);
+            RowVals rv[8];
+            if constexpr (EPI == EPI_QKV || EPI == EPI_RESID) {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if (n + 4 * i + 3 < g.N) p[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                    } else if (live) {
-                        float4 *p = reinterpret_cast<float4 *>(g.resid + static_cast<size_t>(row) * g.N + n);
+                for (int q = 0; q < 8; ++q) rv[q] = load_row<EPI>(g, m0 + quarter * 32 + 4 * q + sub, col_a, col_b);
+            }
+            __syncwarp();                    // the chunk before has been read
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if (n + 4 * i + 3 < g.N) {
-                                float4 o = p[i];
-                                o.x += v[4 * i]; o.y += v[4 * i + 1]; o.z += v[4 * i + 2]; o.w += v[4 * i + 3];
-                                p[i] = o;
-                            }
-                    }
-                }
-            } else if (EPI == EPI_LOGITS) {
-                for (int c = 0; c < N_STEP / 32; ++c) {
-                    const int n = n0 + c * 32;
-                    if (n >= g.N) break;
-                    float v[32];
-                    tmem_ld32(trow + c * 32, v);
-                    tmem_ld_wait();
-                    if (live) {                      // N need not be a multiple of 4 (a pruned vocabulary): scalar stores
-                        float *p = g.resid + static_cast<size_t>(row) * g.N + n;
+            for (int hf = 0; hf < 2; ++hf) { // 16-byte pieces of a row, their index xor the row: no bank conflicts either way
+                float v[32];
+                tmem_ld32(trow + (hf ? cb : ca), v);
+                tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (n + i < g.N) p[i] = v[i];
-                    }
-                }
-            } else if (EPI == EPI_SWIGLU) {
-                for (int c = 0; c < N_STEP / 32; ++c) {
-                    const int n = n0 + c * 32;
-                    if (n >= g.N) break;
-                    float gt[32], up[32];
-                    tmem_ld32(trow + c * 32, gt);
-                    tmem_ld32(trow + N_STEP + c * 32, up);
-                    tmem_ld_wait();
-                    if (live) {
-                        uint4 *p = reinterpret_cast<uint4 *>(g.act + static_cast<size_t>(row) * g.N + n);
+                for (int q = 0; q < 8; ++q)
+                    chunk[lane * 16 + ((hf * 8 + q) ^ (lane & 7))] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            }
+            __syncwarp();
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (n + 8 * i + 7 < g.N) {
-                                float o[8];
-#pragma unroll
-                                for (int j = 0; j < 8; ++j) o[j] = gt[8 * i + j] / (1.f + __expf(-gt[8 * i + j])) * up[8 * i + j];
-                                uint4 hi, lo;
-                                split2x2(o[0], o[1], hi.x, lo.x); split2x2(o[2], o[3], hi.y, lo.y);
-                                split2x2(o[4], o[5], hi.z, lo.z); split2x2(o[6], o[7], hi.w, lo.w);
-                                p[i] = hi;
-                                *reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p + i) + g.act_plane) = lo;
-                            }
-                    }
-                }
-            } else {   // EPI_QKV
-                const int half = g.d >> 1;
-                for (int off = 0; off < N_STEP; off += g.d) {
-                    const int col0 = n0 + off;
-                    if (col0 >= g.N) break;
-                    const int head = col0 / g.d;
-                    if (head < g.nq + g.nkv) {   // q or k: rotate-half pairs (j, j + d/2)
-                        const bool is_q = head < g.nq;
-                        uint16_t *dst = is_q ? g.q_out + static_cast<size_t>(row) * g.nq * g.d + static_cast<size_t>(head) * g.d
-                                                    : g.k_rows + (head - g.nq) * g.head_stride + static_cast<size_t>(row) * g.d;
-                        for (int j0 = 0; j0 < half; j0 += 32) {
-                            float lo[32], hi[32];
-                            tmem_ld32(trow + off + j0, lo);
-                            tmem_ld32(trow + off + half + j0, hi);
-                            tmem_ld_wait();
-                            if (live) {
-                                const float2 *cs = g.rope + static_cast<size_t>(row) * half + j0;
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    float a[8], b[8], bx[8], by[8];
-                                    if (g.bias) {                        // eight biases per 16-byte load
-                                        const uint4 u = *reinterpret_cast<const uint4 *>(g.bias + col0 + j0 + 8 * i);
-                                        const uint4 w = *reinterpret_cast<const uint4 *>(g.bias + col0 + half + j0 + 8 * i);
-                                        bx[0] = bf16lo(u.x); bx[1] = bf16hi(u.x); bx[2] = bf16lo(u.y); bx[3] = bf16hi(u.y);
-                                        bx[4] = bf16lo(u.z); bx[5] = bf16hi(u.z); bx[6] = bf16lo(u.w); bx[7] = bf16hi(u.w);
-                                        by[0] = bf16lo(w.x); by[1] = bf16hi(w.x); by[2] = bf16lo(w.y); by[3] = bf16hi(w.y);
-                                        by[4] = bf16lo(w.z); by[5] = bf16hi(w.z); by[6] = bf16lo(w.w); by[7] = bf16hi(w.w);
-                                    }
-#pragma unroll
-                                    for (int j = 0; j < 8; j += 2) {
-                                        const int e = 8 * i + j;
-                                        const float4 t = *reinterpret_cast<const float4 *>(cs + e);   // (cos, sin) of two pairs
-                                        float x0 = lo[e], y0 = hi[e], x1 = lo[e + 1], y1 = hi[e + 1];
-                                        if (g.bias) { x0 += bx[j]; y0 += by[j]; x1 += bx[j + 1]; y1 += by[j + 1]; }
-                                        a[j] = x0 * t.x - y0 * t.y;
-                                        b[j] = y0 * t.x + x0 * t.y;
-                                        a[j + 1] = x1 * t.z - y1 * t.w;
-                                        b[j + 1] = y1 * t.z + x1 * t.w;
-                                    }
-                                    uint4 ah, al, bh, bl;
-                                    split2x2(a[0], a[1], ah.x, al.x); split2x2(a[2], a[3], ah.y, al.y);
-                                    split2x2(a[4], a[5], ah.z, al.z); split2x2(a[6], a[7], ah.w, al.w);
-                                    split2x2(b[0], b[1], bh.x, bl.x); split2x2(b[2], b[3], bh.y, bl.y);
-                                    split2x2(b[4], b[5], bh.z, bl.z); split2x2(b[6], b[7], bh.w, bl.w);
-                                    if (!is_q && g.k_stage) {                                  // compressed cache: k in fp32 for the quantiser
-                                        float *f = g.k_stage + (head - g.nq) * g.stage_stride + static_cast<size_t>(row) * g.d + j0 + 8 * i;
-                                        *reinterpret_cast<float4 *>(f) = make_float4(a[0], a[1], a[2], a[3]);
-                                        *reinterpret_cast<float4 *>(f + 4) = make_float4(a[4], a[5], a[6], a[7]);
-                                        *reinterpret_cast<float4 *>(f + half) = make_float4(b[0], b[1], b[2], b[3]);
-                                        *reinterpret_cast<float4 *>(f + half + 4) = make_float4(b[4], b[5], b[6], b[7]);
-                                        continue;
-                                    }
-                                    *reinterpret_cast<uint4 *>(dst + j0 + 8 * i) = ah;          // k rows: the hi piece IS the bf16 row
-                                    *reinterpret_cast<uint4 *>(dst + half + j0 + 8 * i) = bh;
-                                    if (is_q) {                                                // queries keep both pieces
-                                        *reinterpret_cast<uint4 *>(dst + g.q_plane + j0 + 8 * i) = al;
-                                        *reinterpret_cast<uint4 *>(dst + g.q_plane + half + j0 + 8 * i) = bl;
-                                    }
-                                }
-                            }
-                        }
-                    } else {                     // v: bias only
-                        uint16_t *dst = g.v_rows + (head - g.nq - g.nkv) * g.head_stride + static_cast<size_t>(row) * g.d;
-                        for (int j0 = 0; j0 < g.d; j0 += 32) {
-                            float v[32];
-                            tmem_ld32(trow + off + j0, v);
-                            tmem_ld_wait();
-                            if (live) {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    float o[8];
-#pragma unroll
-                                    for (int j = 0; j < 8; ++j)
-                                        o[j] = v[8 * i + j] + (g.bias ? bf16_bits_to_f32(g.bias[col0 + j0 + 8 * i + j]) : 0.f);
-                                    if (g.v_stage) {
-                                        float *f = g.v_stage + (head - g.nq - g.nkv) * g.stage_stride + static_cast<size_t>(row) * g.d + j0 + 8 * i;
-                                        *reinterpret_cast<float4 *>(f) = make_float4(o[0], o[1], o[2], o[3]);
-                                        *reinterpret_cast<float4 *>(f + 4) = make_float4(o[4], o[5], o[6], o[7]);
-                                        continue;
-                                    }
-                                    *reinterpret_cast<uint4 *>(dst + j0 + 8 * i) =
-                                        make_uint4(pack2_bf16(o[0], o[1]), pack2_bf16(o[2], o[3]), pack2_bf16(o[4], o[5]), pack2_bf16(o[6], o[7]));
-                                }
-                            }
-                        }
-                    }
-                }
+            for (int q = 0; q < 8; ++q) {
+                const int r = 4 * q + sub, row = m0 + quarter * 32 + r;
+                const float4 va = chunk[r * 16 + (c8 ^ (r & 7))], vb = chunk[r * 16 + 8 + (c8 ^ (r & 7))];
+                const float rs = __shfl_sync(0xffffffffu, rs_own, r);
+                const float ss = finish_row<EPI>(g, row, col_a, col_b, va, vb, cv, rv[q], rs, sp);
+                if (EPI == EPI_RESID && g.norm_w && g.splits == 1) store_row_ss(g, ss, row, n0 / BN * ((BN + 63) / 64) + ch, lane);
             }
         }
         tc_fence_before();           // the accumulator may be overwritten: this warp has read its quarter
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[buf]);
+        if (lane == 0) {
+            if (rank == 0) mbar_arrive(&acc_empty[buf]); else mbar_arrive_remote(cluster_addr(smem_u32(&acc_empty[buf]), 0));
+        }
       }
     }
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    if constexpr (PAIR) cluster_sync(); else __syncthreads();   // a pair leaves together: the first CTA's multiplies use both
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C::BN) : "memory");
+        if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C::BN) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C::BN) : "memory");
     }
     if (threadIdx.x == 0 && abort_flag) atomicExch(g.error, 1);
+}
+
+// The same contraction where the tiles fit the SMs in one round (short prompts): a cluster of g.cluster CTAs shares the K of one output
+// tile, the partial tiles meet through distributed shared memory, every CTA finishes its share of the rows (77 tokens behind 1024, 0.5B
+// shape: 1882 us a prompt by the persistent kernel and its K splits, 1438 so; 9 behind 2048, 1.5B: 2744 and 1799).  Such a pass is a
+// chain of latencies, so everything here shortens the chain:
+//   * tiles of half the columns where those fit the round, too: PF_SLIM, 64 columns, or PF_NARROW for gate/up, 64 + 64;
+//   * the K of a tile is spread over up to eight SMs, and no partial sums pass through global memory and a kernel of their own;
+//   * the weight tiles of the first stages are requested, the rest of this CTA's weights sent for to L2, BEFORE the predecessor is
+//     waited for (nothing writes weights);
+//   * at most 110 KB of shared memory where a CTA has few k-blocks: two CTAs per SM, so that the successor's set-up and first weights overlap
+//     this kernel's end; twice that where it has many (two stages of 48 KB: 27 us for 35 k-blocks, 1.8 MB, of a down projection);
+//   * an activation tile is loaded without its idle rows (a multiple of 8; the multiplies read whatever lies behind it, for rows nobody
+//     looks at);
+//   * SWAP, where the tokens (padded to 8) are fewer than the tile's columns: the weights are the 128 rows of the multiply and the tokens its
+//     columns, hi and lo pieces side by side, so that four multiplies of 2 x tokens columns take the place of eight of the tile's width
+//     over 128 rows (which for 9 tokens, 1.5B shape, are 6.3 us of multiplies in a gate/up tile, by arithmetic: more than its weights take).
+constexpr int TILE_STAGES_MAX = 8, TILE_THREADS = 256, TILE_SMEM = 110 * 1024, TILE_SMEM_DEEP = 220 * 1024, TILE_AHEAD = 32;
+
+__device__ __forceinline__ float4 cluster_ld4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ int cluster_ld1(uint32_t addr) {
+    int v;
+    asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void prefetch_tile_l2(const CUtensorMap *map, int x, int y) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
+}
+
+template <int EPI, int BN, bool SWAP>
+__global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __grid_constant__ CUtensorMap map_a_hi,
+                                                                       const __grid_constant__ CUtensorMap map_a_lo,
+                                                                       const __grid_constant__ CUtensorMap map_b, const GemmArgs g) {
+    constexpr int N_STEP = EPI == EPI_SWIGLU ? BN / 2 : BN, B_PARTS = EPI == EPI_SWIGLU || BN == 256 ? 2 : 1, CHUNKS = BN / 64;
+    extern __shared__ uint8_t pf_dyn[];
+    __shared__ uint64_t full_bar[TILE_STAGES_MAX], empty_bar[TILE_STAGES_MAX], acc_full, drain_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    __shared__ float rs_sm[PF_BM];
+    uint8_t *tiles = pf_dyn + ((1024u - (smem_u32(pf_dyn) & 1023u)) & 1023u);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int S = g.cluster, tile = blockIdx.x / S, rank = blockIdx.x - tile * S, KB = (g.K + PF_BK - 1) / PF_BK;
+    const int m_tiles = (g.M + PF_BM - 1) / PF_BM, n_tile = tile / m_tiles, m0 = (tile - n_tile * m_tiles) * PF_BM, n0 = n_tile * N_STEP;
+    const int kb0 = rank * KB / S, nkb = (rank + 1) * KB / S - kb0;
+    const int a_bytes = g.a_rows * PF_BK * 2, stage_bytes = 2 * a_bytes + BN * PF_BK * 2;
+    const int live = min(PF_BM, g.M - m0), r0 = rank * live / S, r1 = (rank + 1) * live / S;   // rows of the tile; those this CTA finishes
+
+    if (threadIdx.x == 0) {
+        prefetch_map(&map_b); prefetch_map(&map_a_hi); prefetch_map(&map_a_lo);
+#pragma unroll 1
+        for (int s = 0; s < g.stages; ++s) { mbar_init(&full_bar[s], 1 + g.extra_arrivals); mbar_init(&empty_bar[s], 1); }
+        mbar_init(&acc_full, 1);
+        mbar_init(&drain_bar, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(g.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+    pdl_trigger();
+
+    if (warp == 0 && lane == 0) {            // producer
+        const int first = min(nkb, g.stages);
+        // it: k-block of this CTA; what: 0 = its weight tile into stage s, 1 = asked for from memory only
+        auto load_b = [&](int it, int s, bool into) {
+            const int x = (kb0 + it) * PF_BK;
+            uint8_t *b = tiles + s * stage_bytes + 2 * a_bytes;
+            if (into) mbar_expect_tx(&full_bar[s], stage_bytes);
+#pragma unroll
+            for (int part = 0; part < B_PARTS; ++part) {     // gate and up, or 128 and 128 columns
+                const int y = n0 + part * (EPI == EPI_SWIGLU ? g.N : 128);
+                if (into) tma_load_2d(b + part * (BN * PF_BK * 2 / B_PARTS), &map_b, x, y, &full_bar[s]);
+                else prefetch_tile_l2(&map_b, x, y);
+            }
+        };
+        auto load_a = [&](int it, int s) {
+            uint8_t *a = tiles + s * stage_bytes;
+            tma_load_2d(a, &map_a_hi, (kb0 + it) * PF_BK, m0, &full_bar[s]);
+            tma_load_2d(a + a_bytes, &map_a_lo, (kb0 + it) * PF_BK, m0, &full_bar[s]);
+        };
+        const int ahead = m0 == 0 ? min(nkb, first + TILE_AHEAD) : first;
+#pragma unroll 1
+        for (int it = 0; it < ahead; ++it) load_b(it, it, it < first);
+        pdl_wait();
+        int it = 0;
+#pragma unroll 1
+        for (int s = 0, phase = 1; it < nkb; ++it) {      // from the second round on: the stage is free when its multiplies are done
+            if (it >= first) {
+                if (!mbar_wait(&empty_bar[s], phase, &abort_flag, g.wait_limit)) break;
+                load_b(it, s, true);
+            }
+            load_a(it, s);
+            if (++s == g.stages) { s = 0; phase ^= 1; }
+        }
+        if (abort_flag) {   // giving up: the copies still in flight must land before the shared memory is used again or released
+            int dummy = 0;
+#pragma unroll 1
+            for (int j = it > g.stages ? it - g.stages : 0; j < it; ++j)
+                mbar_wait(&full_bar[j % g.stages], (j / g.stages) & 1, &dummy, g.wait_limit);
+        }
+    } else if (warp == 1 && lane == 0) {     // issuer
+        pdl_wait();
+        const uint32_t idesc = umma_idesc_bf16(PF_BM, SWAP ? 2 * g.a_rows : BN);
+        bool ok = true;
+#pragma unroll 1
+        for (int it = 0, s = 0, phase = 0; it < nkb; ++it) {
+            ok = mbar_wait(&full_bar[s], phase, &abort_flag, g.wait_limit);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t a = smem_u32(tiles + s * stage_bytes);
+            const uint64_t da = umma_desc_sw128(a), db = umma_desc_sw128(a + 2 * a_bytes);
+            if constexpr (SWAP) {            // (the lo rows lie right behind the hi rows)
+#pragma unroll
+                for (int k = 0; k < PF_BK / 16; ++k) umma_bf16(tmem, db + 2 * k, da + 2 * k, idesc, (it | k) != 0);
+            } else {
+                const uint64_t dl = umma_desc_sw128(a + a_bytes);
+#pragma unroll
+                for (int k = 0; k < PF_BK / 16; ++k) umma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (it | k) != 0);
+#pragma unroll
+                for (int k = 0; k < PF_BK / 16; ++k) umma_bf16(tmem, dl + 2 * k, db + 2 * k, idesc, 1);
+            }
+            umma_commit(&empty_bar[s]);
+            if (++s == g.stages) { s = 0; phase ^= 1; }
+        }
+        umma_commit(ok ? &acc_full : &drain_bar);
+        if (!ok) {          // giving up: the multiplies already issued must finish before the tensor memory is freed
+            int dummy = 0;
+            mbar_wait(&drain_bar, 0, &dummy, g.wait_limit);
+        }
+    }
+    __syncwarp();
+    pdl_wait();
+    if ((warp & 6) == 2 && EPI != EPI_RESID)        // the scales of this CTA's rows
+        for (int r = r0 + threadIdx.x - 64; r < r1; r += 64) rs_sm[r] = row_scale(g, m0 + r);
+
+    // Steps of the epilogue, a warp each: row group (4 rows) item / chunks, chunk item % chunks.  The first step's vectors are fetched under
+    // the main loop, then the CTAs meet.
+    const int sub = lane >> 3, c8 = lane & 7, items = ((r1 - r0 + 3) / 4) * CHUNKS;
+    const uint32_t base = smem_u32(tiles);
+#pragma unroll 1
+    for (int item = warp; item == warp || item < items; item += TILE_THREADS / 32) {
+        const int group = item / CHUNKS, chunk = item % CHUNKS, r = r0 + group * 4 + sub;
+        const int row = r < r1 ? m0 + r : g.M;                       // (g.M: a lane without a row)
+        int ca, cb;
+        chunk_halves<EPI, N_STEP>(chunk, g.d, ca, cb);
+        const int col_a = n0 + ca + 4 * c8, col_b = n0 + cb + 4 * c8;
+        const ColVals cv = load_cols<EPI>(g, col_a, col_b);
+        const RowVals rv = load_row<EPI>(g, row, col_a, col_b);
+        if (item == warp) {
+            if (warp >= 4 && (warp & 3) * 32 < (SWAP ? BN : live)) {   // the partial tile into shared memory, over the ring: all its copies have landed and been read
+                const int t = (warp & 3) * 32 + lane;                    // row of the tile; swapped: its column
+                const uint32_t trow = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+                if (__all_sync(0xffffffffu, mbar_wait(&acc_full, 0, &abort_flag, g.wait_limit))) {
+                    tc_fence_after();
+                    if constexpr (SWAP) {
+                        float *dst = reinterpret_cast<float *>(tiles);
+#pragma unroll 1
+                        for (int t0 = 0; t0 < live; t0 += 32) {
+                            float hi[32], lo[32];
+                            tmem_ld32(trow + t0, hi);
+                            tmem_ld32(trow + g.a_rows + t0, lo);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int i = 0; i < 32; ++i)
+                                if (t0 + i < live) dst[(t0 + i) * BN + ((((t >> 2) ^ (i & 7)) << 2) | (t & 3))] = hi[i] + lo[i];
+                        }
+                    } else {
+                        float4 *dst = reinterpret_cast<float4 *>(tiles) + t * (BN / 4);
+#pragma unroll 1
+                        for (int c = 0; c < BN / 32; ++c) {
+                            float v[32];
+                            tmem_ld32(trow + c * 32, v);
+                            tmem_ld_wait();
+                            if (t < live) {
+#pragma unroll
+                                for (int q = 0; q < 8; ++q) dst[(c * 8 + q) ^ (t & 7)] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                }
+            }
+            __syncwarp();
+            if (S > 1) cluster_sync(); else __syncthreads();
+            // of any CTA of the cluster: nothing is written
+            const bool dead = S > 1 ? __any_sync(0xffffffffu, lane < S && cluster_ld1(cluster_addr(smem_u32(&abort_flag), lane)) != 0) : abort_flag != 0;
+            if (dead || item >= items) {
+                if (S > 1) cluster_arrive();
+                break;
+            }
+        }
+        const int rc = min(r, r1 - 1);
+        const uint32_t off = base + rc * BN * 4, pa = off + ((ca / 4 + c8) ^ (rc & 7)) * 16, pb = off + ((cb / 4 + c8) ^ (rc & 7)) * 16;
+        float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
+#pragma unroll 4
+        for (int q = 0; q < S; ++q) {        // in the order of K
+            const float4 x = cluster_ld4(S > 1 ? cluster_addr(pa, q) : pa), y = cluster_ld4(S > 1 ? cluster_addr(pb, q) : pb);
+            va.x += x.x; va.y += x.y; va.z += x.z; va.w += x.w;
+            vb.x += y.x; vb.y += y.y; vb.z += y.z; vb.w += y.w;
+        }
+        // Nobody leaves while its shared memory may still be read.  A warp arrives behind its last read, before it stores: an arrival that
+        // releases stores to global memory waits for them (2.5 us).
+        if (S > 1 && item + TILE_THREADS / 32 >= items) cluster_arrive();
+        if (n0 + ca >= g.N) continue;        // a chunk past the matrix
+        const float ss = finish_row<EPI>(g, row, col_a, col_b, va, vb, cv, rv, EPI == EPI_RESID ? 1.f : rs_sm[rc], 0);
+        if (EPI == EPI_RESID && g.norm_w) store_row_ss(g, ss, row, n_tile * CHUNKS + chunk, lane);
+    }
+    if (warp == 1) {                         // (behind the barrier in the loop: the accumulator has been read)
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.tmem_cols) : "memory");
+    }
+    if (threadIdx.x == 0 && abort_flag) atomicExch(g.error, 1);
+    if (S > 1) cluster_wait();
 }
 
 // ---- causal attention on tcgen05 ---------------------------------------------------------------------------------------------
@@ -860,7 +1196,6 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
     // Q8: the cache holds 8-bit codes and a scale per row (k_scale, v_scale: this layer's [nkv][max_context]); map_k / map_v then
     // describe byte matrices; two more warps expand the codes to bf16 (exactly) into the operand layout, the softmax multiplies
     // the scores by the keys' scales and folds the values' scales into the probabilities.
-    pdl_trigger();
     using C = AttnCfg<D>;
     extern __shared__ uint8_t at_tc_dyn[];
     __shared__ uint64_t kraw_full, kraw_empty, vraw_full;
@@ -904,6 +1239,7 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    pdl_trigger();
     pdl_wait();   // set-up done; from here on the kernel reads what its predecessor wrote
 
     if (warp == 0 && lane == 0) {            // producer: the query tile once, then the K and V rows of every key block
@@ -1287,19 +1623,36 @@ __global__ void __launch_bounds__(D / 4) prefill_attention_merge_kernel(const fl
 // instructions are then no-ops).
 thread_local bool g_pdl = false;
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
+cudaError_t launch_cluster(dim3 cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (g_pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster.x * cluster.z > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster.x;
+        attr[n].val.clusterDim.y = 1;
+        attr[n].val.clusterDim.z = cluster.z;
+        ++n;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = g_pdl ? 1 : 0;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
+    return launch_cluster(dim3(1), kernel, grid, block, smem, stream, static_cast<KArgs>(args)...);
+}
+
+// Clusters of c CTAs, one CTA per SM, that run at once: a cluster stays within a GPC of (about) 18 SMs.
+int clusters_at_once(int c, int num_sms) { return num_sms / 18 * (18 / c) + num_sms % 18 / c; }
 
 // ---- host side ---------------------------------------------------------------------------------------------------------------
 // Map of a row-major bf16 [rows][K] matrix; a box is box_rows rows x 64 columns (one 128-byte swizzled row each); rows and
@@ -1315,32 +1668,70 @@ bool encode_operand_map(CUtensorMap *m, const void *base, long long rows, int K,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int EPI, int SHAPE>
-const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, const GemmArgs &g, int num_sms, cudaStream_t s) {
-    using C = GemmCfg<SHAPE>;
-    if (cudaFuncSetAttribute(prefill_gemm_kernel<EPI, SHAPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
+template <int EPI, int SHAPE, bool PAIR>
+const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, const GemmArgs &g, int units, int workers, cudaStream_t s) {
+    using C = GemmCfg<SHAPE, PAIR>;
+    if (cudaFuncSetAttribute(prefill_gemm_kernel<EPI, SHAPE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
         return "cudaFuncSetAttribute failed";
-    const int n_step = EPI == EPI_SWIGLU ? C::BN / 2 : C::BN;
-    const int units = ((g.N + n_step - 1) / n_step) * ((g.M + PF_BM - 1) / PF_BM) * (EPI == EPI_RESID ? g.splits : 1);
-    launch_pdl(prefill_gemm_kernel<EPI, SHAPE>, dim3(units < num_sms ? units : num_sms), dim3(192), C::SMEM, s, ma, ml, mb, g);
+    const int ctas = PAIR ? 2 : 1;
+    launch_cluster(dim3(ctas), prefill_gemm_kernel<EPI, SHAPE, PAIR>, dim3((units < workers ? units : workers) * ctas), dim3(192), C::SMEM, s, ma, ml, mb, g);
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill GEMM launch failed";
+}
+
+template <int EPI, int BN, bool SWAP>
+const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, GemmArgs &g, cudaStream_t s) {
+    const int n_step = EPI == EPI_SWIGLU ? BN / 2 : BN, tiles = ((g.N + n_step - 1) / n_step) * ((g.M + PF_BM - 1) / PF_BM);
+    const int a_bytes = g.a_rows * PF_BK * 2, stage = 2 * a_bytes + BN * PF_BK * 2;
+    const int kb = ((g.K + PF_BK - 1) / PF_BK + g.cluster - 1) / g.cluster;      // of the CTA with the most
+    // the multiplies read 128 rows of the operand that has 128, from the start of either piece or (swapped) of the weights: room behind the
+    // last stage for those that are not loaded
+    const int reach = (SWAP ? 2 : 1) * a_bytes + PF_BM * PF_BK * 2, slack = reach > stage ? reach - stage : 0;
+    g.stages = (TILE_SMEM - 1024 - slack) / stage;
+    if (kb > 2 * g.stages) g.stages = (TILE_SMEM_DEEP - 1024 - slack) / stage;
+    if (g.stages > TILE_STAGES_MAX) g.stages = TILE_STAGES_MAX;
+    if (g.stages > kb) g.stages = kb;
+    const int ring = g.stages * stage + slack, partial = g.a_rows * BN * 4;
+    const int smem = 1024 + (ring > partial ? ring : partial);
+    // swapped: the pieces' columns are read 32 at a time
+    const int cols = SWAP ? g.a_rows + (g.a_rows + 31) / 32 * 32 : BN;
+    for (g.tmem_cols = 32; g.tmem_cols < cols;) g.tmem_cols *= 2;
+    if (cudaFuncSetAttribute(prefill_tile_kernel<EPI, BN, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM_DEEP) != cudaSuccess)
+        return "cudaFuncSetAttribute failed";
+    launch_cluster(dim3(g.cluster), prefill_tile_kernel<EPI, BN, SWAP>, dim3(tiles * g.cluster), dim3(TILE_THREADS), static_cast<size_t>(smem), s, ma, ml, mb, g);
+    return cudaGetLastError() == cudaSuccess ? nullptr : "prefill contraction launch failed";
 }
 
 template <int EPI>
 const char *launch_gemm(const uint16_t *a, size_t a_plane, const void *w, long long w_rows, GemmArgs &g, int num_sms, cudaStream_t s) {
     CUtensorMap ma, ml, mb;
-    int shape = PF_WIDE;
-    prefill_plan_contraction(EPI, g.d, g.M, g.N, g.K, num_sms, &shape, &g.splits);
-    const bool slim = shape == (EPI == EPI_SWIGLU ? PF_NARROW : PF_SLIM);
-    if (!encode_operand_map(&ma, a, g.M, g.K) || !encode_operand_map(&ml, a + a_plane, g.M, g.K) || !encode_operand_map(&mb, w, w_rows, g.K, slim ? 64 : 128))
+    const PrefillPlan plan = prefill_plan(EPI, g.d, g.M, g.N, g.K, num_sms);
+    g.cluster = plan.cluster;
+    g.splits = plan.splits;
+    g.bn = plan.columns;
+    g.a_rows = g.cluster && g.M < PF_BM ? (g.M + 7) & ~7 : PF_BM;
+    const int b_rows = EPI == EPI_SWIGLU ? (plan.columns == 128 ? 64 : 128) : plan.pairs ? plan.columns / 2 : plan.columns < 128 ? plan.columns : 128;
+    if (!encode_operand_map(&ma, a, g.M, g.K, g.a_rows) || !encode_operand_map(&ml, a + a_plane, g.M, g.K, g.a_rows) ||
+        !encode_operand_map(&mb, w, w_rows, g.K, b_rows))
         return "cuTensorMapEncodeTiled failed";
-    if constexpr (EPI == EPI_SWIGLU) {
-        return slim ? launch_gemm_cfg<EPI, PF_NARROW>(ma, ml, mb, g, num_sms, s) : launch_gemm_cfg<EPI, PF_WIDE>(ma, ml, mb, g, num_sms, s);
-    } else {
-        if constexpr (EPI != EPI_LOGITS)
-            if (slim) return launch_gemm_cfg<EPI, PF_SLIM>(ma, ml, mb, g, num_sms, s);
-        return shape == PF_WIDE ? launch_gemm_cfg<EPI, PF_WIDE>(ma, ml, mb, g, num_sms, s) : launch_gemm_cfg<EPI, PF_NARROW>(ma, ml, mb, g, num_sms, s);
+    if (EPI == EPI_RESID) {       // whole tiles have (columns + 63) / 64 pieces each, the last what is left of the matrix
+        const int whole = (g.N - 1) / g.bn;
+        g.ss_pieces = whole * ((g.bn + 63) / 64) + (g.N - whole * g.bn + 63) / 64;
     }
+    if constexpr (EPI != EPI_LOGITS)
+        if (g.cluster) {
+            if constexpr (EPI != EPI_SWIGLU) {
+                if (plan.columns == 256) return launch_tile<EPI, 256, false>(ma, ml, mb, g, s);
+                if (plan.columns == 64) return plan.swap ? launch_tile<EPI, 64, true>(ma, ml, mb, g, s) : launch_tile<EPI, 64, false>(ma, ml, mb, g, s);
+            }
+            return plan.swap ? launch_tile<EPI, 128, true>(ma, ml, mb, g, s) : launch_tile<EPI, 128, false>(ma, ml, mb, g, s);
+        }
+    const int m_tiles = (g.M + PF_BM - 1) / PF_BM;
+    if constexpr (EPI != EPI_SWIGLU)
+        if (plan.columns == 128) return launch_gemm_cfg<EPI, PF_NARROW, false>(ma, ml, mb, g, m_tiles * ((g.N + 127) / 128) * g.splits, num_sms, s);
+    const int n_step = EPI == EPI_SWIGLU ? 128 : g.bn, units = ((g.N + n_step - 1) / n_step) * g.splits;
+    if constexpr (EPI != EPI_LOGITS)
+        if (plan.pairs) return launch_gemm_cfg<EPI, PF_WIDE, true>(ma, ml, mb, g, (m_tiles + 1) / 2 * units, num_sms / 2, s);
+    return launch_gemm_cfg<EPI, PF_WIDE, false>(ma, ml, mb, g, m_tiles * units, num_sms, s);
 }
 
 // Map of a byte matrix [rows][row_bytes] (the codes of a compressed cache); a box is box_rows whole rows, unswizzled.
@@ -1430,9 +1821,56 @@ void prefill_plan_contraction(int epilogue, int head_dim, int M, int N, int K, i
     *shape = epilogue == EPI_SWIGLU ? PF_NARROW : PF_SLIM;
 }
 
+// What runs: the tile shape and K split of prefill_plan_contraction, refined.
+PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int num_sms) {
+    int shape, splits;
+    prefill_plan_contraction(epilogue, head_dim, M, N, K, num_sms, &shape, &splits);
+    const int m_tiles = (M + PF_BM - 1) / PF_BM, kb = (K + PF_BK - 1) / PF_BK;
+    PrefillPlan p{shape == PF_WIDE ? 256 : shape == PF_SLIM ? 64 : 128, splits, 0, false, false};
+    const int n_step = epilogue == EPI_SWIGLU ? p.columns / 2 : p.columns, tiles = m_tiles * ((N + n_step - 1) / n_step);
+    if (epilogue == EPI_LOGITS) return p;
+    // Clusters where the tiles fit the SMs in one round.  A k-block costs a CTA what its operands take at 64 bytes per cycle, or its multiplies:
+    // 4 cycles per column over 128 rows, or (swapped, the weights are the rows) 4 per token; sharing a tile's K costs the exchange of the
+    // partial tiles, about 2000 cycles.  Tiles of 256 columns halve the traffic of several row tiles' activations.
+    if (shape != PF_WIDE) {
+        if (tiles > num_sms) return p;
+        const int rows = M < PF_BM ? (M + 7) & ~7 : PF_BM, base = p.columns;
+        int best = 1 << 30;
+        for (int bn = base; bn <= (epilogue == EPI_SWIGLU || m_tiles == 1 ? base : 256); bn *= 2) {
+            const int t = m_tiles * ((N + bn - 1) / bn), step = epilogue == EPI_SWIGLU ? tiles : t;
+            for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && (c == 1 ? step <= num_sms : step <= clusters_at_once(c, num_sms)); ++c) {
+                const bool swap = rows < bn && bn <= 128 && rows < PF_BM;
+                const int multiplies = 4 * (swap ? (rows > 32 ? rows : 32) : bn), operands = 4 * rows + 2 * bn;
+                const int cost = (kb + c - 1) / c * (multiplies > operands ? multiplies : operands) + (c > 1 ? 2000 : 0);
+                if (cost < best) { best = cost; p.columns = bn; p.cluster = c; p.swap = swap; }
+            }
+        }
+        p.splits = 1;
+        return p;
+    }
+    // Pairs of CTAs where they need no more rounds over the SMs (an odd number of row tiles leaves one CTA of a pair without work).
+    const int workers = num_sms / 2, m_pairs = (m_tiles + 1) / 2;
+    if (m_tiles < 2 || workers < 1) return p;
+    auto rounds = [](int units, int n) { return (units + n - 1) / n; };
+    p.pairs = rounds(m_pairs * ((N + n_step - 1) / n_step) * splits, workers) <= rounds(tiles * splits, num_sms);
+    // A contraction that adds to the residual stream takes the number of columns that fills its rounds best: a k-block costs a CTA 4 cycles
+    // per column in the tensor cores, or what its operands (32 KB of activations, 64 bytes per column) take at 64 bytes per cycle; a K split costs its
+    // partial sums a pass through memory and the norm kernel (about a tenth).  (4096 tokens, 7B shape: 160 columns, 4.97 rounds, against 3.03
+    // rounds of 256: O 212 -> 202 us, down 930 -> 894, at the power limit.)
+    if (epilogue == EPI_RESID) {
+        double best = p.pairs ? rounds(m_pairs * ((N + 255) / 256) * splits, workers) * 1024. / splits : rounds(tiles * splits, num_sms) * 1075. / splits;
+        if (splits > 1) best *= 1.05 * 1.1;
+        for (int bn = 128; bn <= 256; bn += 16) {
+            const double cost = rounds(m_pairs * ((N + bn - 1) / bn), workers) * static_cast<double>(4 * bn > 512 + bn ? 4 * bn : 512 + bn);
+            if (cost < best - 1e-9) { best = cost; p.columns = bn; p.splits = 1; p.pairs = true; }
+        }
+    }
+    return p;
+}
+
 size_t prefill_buffer_bytes(const edgefm_shape &sh, int chunk) {
     const size_t c = static_cast<size_t>(chunk), qd = static_cast<size_t>(sh.n_q_heads) * sh.head_dim;
-    return c * sh.hidden * 4 * (1 + PF_SPLIT_MAX) + c * sh.hidden * 4 + 2 * c * qd * 4 + c * sh.ffn * 4 + c * (sh.head_dim / 2) * 8 + c * 4 + 256;
+    return c * sh.hidden * 4 * (1 + PF_SPLIT_MAX) + c * sh.hidden * 4 + c * PF_SS_PIECES(sh.hidden) * 4 + 2 * c * qd * 4 + c * sh.ffn * 4 + c * (sh.head_dim / 2) * 8 + c * 4 + 256;
 }
 
 cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, bool kv8) {
@@ -1440,6 +1878,7 @@ cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, 
     cudaError_t e;
     if ((e = cudaMalloc(&b->resid, c * sh.hidden * 4)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->xn, c * sh.hidden * 4)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->ss, c * PF_SS_PIECES(sh.hidden) * 4)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->part, c * sh.hidden * 4 * PF_SPLIT_MAX)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->q, c * qd * 4)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->attn, c * qd * 4)) != cudaSuccess) return e;
@@ -1462,7 +1901,7 @@ cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, 
 }
 
 void prefill_free(PrefillBuffers *b) {
-    cudaFree(b->resid); cudaFree(b->xn); cudaFree(b->part); cudaFree(b->kv_stage); cudaFree(b->q); cudaFree(b->attn); cudaFree(b->act); cudaFree(b->rope);
+    cudaFree(b->resid); cudaFree(b->xn); cudaFree(b->part); cudaFree(b->ss); cudaFree(b->kv_stage); cudaFree(b->q); cudaFree(b->attn); cudaFree(b->act); cudaFree(b->rope);
     cudaFree(b->tokens); cudaFree(b->error); cudaFree(b->logits); cudaFree(b->att_o); cudaFree(b->att_ml); cudaFree(b->head_val); cudaFree(b->head_idx); cudaFree(b->head_ticket);
     *b = PrefillBuffers{};
 }
@@ -1483,6 +1922,8 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
                                                   static_cast<const uint16_t *>(m.embed), b->tokens, n, H, sh.rms_eps, m.state,
                                                   slot0 + n, position + n, nullptr, 0, 0);
     count += 2;
+    int pieces = 0;
+    bool raw = false;    // xn holds x * w of the residual stream, its sums of squares in b->ss (else normalised rows)
     for (int l = 0; l < sh.n_layers; ++l) {
         const edgefm_layer_weights &w = m.layers[l];
         const bool kv8 = m.k_scale != nullptr;   // compressed cache: one byte per element and a scale per row
@@ -1492,6 +1933,11 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
         GemmArgs g{};
         g.M = n; g.error = b->error; g.wait_limit = b->wait_limit; g.extra_arrivals = b->extra_arrivals;
         g.N = n_qkv; g.K = H;
+        // a contraction that reads xn scales its results by 1 / rms where the rows are not normalised; one that adds to the residual stream
+        // prepares xn for the next, or leaves K-split partial sums to the norm kernel
+        g.ss_stride = cap; g.ss_pieces = pieces; g.eps = sh.rms_eps;
+        g.xw = b->xn; g.x_plane = x_plane; g.ss_out = b->ss;
+        g.ss_in = raw ? b->ss : nullptr;
         g.bias = sh.qkv_bias ? static_cast<const uint16_t *>(w.bqkv) : nullptr;
         if (g.bias && (reinterpret_cast<uintptr_t>(g.bias) & 15u)) return "edgefm_prefill reads bqkv in 16-byte pieces: the vector must be 16-byte aligned";
         g.rope = b->rope; g.q_out = b->q; g.q_plane = q_plane;
@@ -1512,17 +1958,29 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
                                 : launch_attention_tc<128>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->error, b->att_o, b->att_ml, m.num_sms, s);
         if (e) return e;
         g.N = H; g.K = qd; g.resid = b->resid; g.part = b->part; g.part_plane = x_plane;
+        g.norm_w = static_cast<const uint16_t *>(w.post_norm);
         if ((e = launch_gemm<EPI_RESID>(b->attn, q_plane, w.wo, H, g, m.num_sms, s))) return e;
-        launch_pdl(prefill_norm_kernel, dim3(norm_grid), dim3(128), 0, s, b->resid, b->xn, x_plane, static_cast<const uint16_t *>(w.post_norm), nullptr, nullptr, n, H,
-                                                      sh.rms_eps, nullptr, 0, 0, b->part, g.splits, x_plane);
+        if (g.splits > 1) {
+            launch_pdl(prefill_norm_kernel, dim3(norm_grid), dim3(128), 0, s, b->resid, b->xn, x_plane, g.norm_w, nullptr, nullptr, n, H,
+                       sh.rms_eps, nullptr, 0, 0, b->part, g.splits, x_plane);
+            ++count;
+        }
+        g.ss_in = g.splits > 1 ? nullptr : b->ss;
         g.N = F; g.K = H; g.act = b->act; g.act_plane = f_plane;
         if ((e = launch_gemm<EPI_SWIGLU>(b->xn, x_plane, w.w_gate_up, 2LL * F, g, m.num_sms, s))) return e;
         g.N = H; g.K = F;
+        // behind the last layer nothing is normalised here (the norm kernel runs for the partial sums alone)
+        const bool last = l + 1 == sh.n_layers;
+        g.norm_w = last ? nullptr : static_cast<const uint16_t *>(m.layers[l + 1].input_norm);
         if ((e = launch_gemm<EPI_RESID>(b->act, f_plane, w.w_down, H, g, m.num_sms, s))) return e;
-        // (behind the last layer the norm weights do not matter: the kernel runs for the K-split partial sums of the down projection)
-        launch_pdl(prefill_norm_kernel, dim3(norm_grid), dim3(128), 0, s, b->resid, b->xn, x_plane, static_cast<const uint16_t *>(m.layers[l + 1 < sh.n_layers ? l + 1 : l].input_norm),
-                                                      nullptr, nullptr, n, H, sh.rms_eps, nullptr, 0, 0, b->part, g.splits, x_plane);
-        count += 6;
+        if (g.splits > 1) {
+            launch_pdl(prefill_norm_kernel, dim3(norm_grid), dim3(128), 0, s, b->resid, b->xn, x_plane,
+                       last ? static_cast<const uint16_t *>(w.input_norm) : g.norm_w, nullptr, nullptr, n, H, sh.rms_eps, nullptr, 0, 0, b->part, g.splits, x_plane);
+            ++count;
+        }
+        raw = g.splits == 1;
+        pieces = g.ss_pieces;
+        count += 4;
     }
     if (cudaGetLastError() != cudaSuccess) return "prefill kernel launch failed";
     if (launches) *launches = count;

@@ -17,13 +17,17 @@ constexpr int PF_VERIFY_MAX = 8;         // tokens of the longest block that can
 constexpr int PF_CHUNK_MAX = PF_CHUNK_MAX_VALUE;   // tokens per pass over the layers (longer prompts take several passes); 4096 instead of
                                                   // 2048 took a 32768-token prompt of the 1.5B shape from 393 to 351 ms
 
+// pieces of a row of the residual stream at most: tiles of 64 or 128 columns have one per 64, those of 144 have three
+constexpr int PF_SS_PIECES(int hidden) { return hidden / 64 * 3 / 2 + 4; }
+
 // Work buffers of one pass, owned by the context, allocated at the first prefill call.
 struct PrefillBuffers {
     int chunk = 0;               // rows the buffers hold
     float *resid = nullptr;      // residual stream fp32 [chunk][H]
+    float *ss = nullptr;         // sums of squares of the residual stream's pieces, fp32 [PF_SS_PIECES(H)][chunk]
     float *part = nullptr;       // K-split partial sums of the O / down contraction, fp32 [8][chunk][H]
     // activations as two bf16 planes each (hi = bf16(x), lo = bf16(x - hi)):
-    uint16_t *xn = nullptr;      // normalised activations [2][chunk][H]
+    uint16_t *xn = nullptr;      // normalised activations, or x * w with the sums of squares in `ss` [2][chunk][H]
     uint16_t *q = nullptr;       // rotated queries [2][chunk][nq d]
     uint16_t *attn = nullptr;    // attention output [2][chunk][nq d]
     uint16_t *act = nullptr;     // SwiGLU output [2][chunk][F]
@@ -58,6 +62,12 @@ enum { PF_NARROW = 0, PF_SLIM = 1, PF_WIDE = 2 };
 // Tile shape and K split a contraction of [M x K] x [K x N] gets on num_sms SMs (host logic, no device needed).
 // epilogue: 0 = QKV (heads of head_dim), 1 = added to the residual stream (O, down), 2 = gate/up, 3 = logits of a verified block.
 void prefill_plan_contraction(int epilogue, int head_dim, int M, int N, int K, int num_sms, int *shape, int *splits);
+// What runs for such a contraction: output columns of a tile (gate/up: gate and up columns together), K units that leave partial sums in global
+// memory, CTAs of a cluster that share the K of a tile (0: the persistent kernel), and whether two row tiles are multiplied by a pair of CTAs.
+// swap: in a cluster the weights are the rows of the multiply and the tokens its columns.
+struct PrefillPlan { int columns, splits, cluster; bool pairs, swap; };
+constexpr int PF_CLUSTER_MAX = 8;
+PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int num_sms);
 
 // Bytes the work buffers of a pass over `chunk` tokens take.
 size_t prefill_buffer_bytes(const edgefm_shape &sh, int chunk);

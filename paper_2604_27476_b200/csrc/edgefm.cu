@@ -616,7 +616,7 @@ namespace {
 edgefm_status ensure_prefill_buffers(edgefm_ctx *ctx) {
     if (ctx->pf.chunk == 0) {
         const int chunk = std::min(PF_CHUNK_MAX, ctx->max_context);
-        if (prefill_alloc(&ctx->pf, ctx->shape, chunk, ctx->kv_format == EDGEFM_KV_INT8) != cudaSuccess) {
+        if (prefill_alloc(&ctx->pf, ctx->shape, chunk, ctx->kv_format == EDGEFM_KV_INT8, ctx->num_sms) != cudaSuccess) {
             cudaGetLastError();
             prefill_free(&ctx->pf);
             return fail(ctx, EDGEFM_ERR_OUT_OF_MEMORY, "work buffers of the dense path (%zu bytes)", prefill_buffer_bytes(ctx->shape, chunk));

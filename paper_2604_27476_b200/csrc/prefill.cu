@@ -142,24 +142,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
-    uint32_t *r = reinterpret_cast<uint32_t *>(v);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-template <int N> __device__ __forceinline__ void tmem_ld(uint32_t taddr, float *v) {
-    static_assert(N == 16 || N % 32 == 0, "16 columns or a multiple of 32");
-    if constexpr (N == 16) {
-        tmem_ld16(taddr, v);
-    } else {
-#pragma unroll
-        for (int c = 0; c < N / 32; ++c) tmem_ld32(taddr + c * 32, v + c * 32);
-    }
-}
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float *v) {
     const uint32_t *r = reinterpret_cast<const uint32_t *>(v);
     asm volatile(
@@ -178,16 +160,16 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float *v) {
         "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
 }
-template <int N> __device__ __forceinline__ void tmem_st(uint32_t taddr, const float *v) {
-    static_assert(N == 16 || N % 32 == 0, "16 columns or a multiple of 32");
-    if constexpr (N == 16) {
-        tmem_st16(taddr, v);
-    } else {
-#pragma unroll
-        for (int c = 0; c < N / 32; ++c) tmem_st32(taddr + c * 32, v + c * 32);
-    }
-}
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// the values of a tmem_ld32 issued earlier are there (nothing that uses them moves above this)
+__device__ __forceinline__ void tmem_ld_ready(float *v) {
+    uint32_t *r = reinterpret_cast<uint32_t *>(v);
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]),
+                   "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]),
+                   "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]),
+                   "+r"(r[31])::"memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor of a K-major bf16 tile written by TMA with the 128-byte swizzle: rows of 64 elements
@@ -239,7 +221,6 @@ __device__ __forceinline__ void split2x2_trunc(float a, float b, uint32_t &hi, u
 // (cos, sin) of angle (position + t) * theta^(-2 j / d), evaluated in double and rounded once.
 __global__ void __launch_bounds__(256) prefill_rope_kernel(float2 *rope, int n, int half, int position, double theta) {
     pdl_trigger();
-    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n * half) return;
     const int t = i / half, j = i % half;
@@ -1140,28 +1121,26 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
 }
 
 // ---- causal attention on tcgen05 ---------------------------------------------------------------------------------------------
-// One CTA = 128 queries of one head (a query = a lane of tensor memory, two softmax threads per query); keys in blocks of 128.
-// Per block j:  S_j = Q K_j^T (tcgen05.mma, M 128, N 128, K = D; queries as two bf16 pieces) into one of two S buffers in
-// tensor memory;  the softmax warps read their part of the row twice (tcgen05.ld; once for the maximum, once for the
-// exponentials), mask on diagonal blocks, update the running maximum and sum, and store the probabilities as two bf16 pieces
-// into tensor memory (tcgen05.st, two keys per column);  O_j = P_j V_j (M 128, N = D, K = 128 keys; P from tensor memory, V straight
-// from its cache rows as an MN-major B operand), accumulated over the blocks in tensor memory;  the exponentials are taken
-// against a reference maximum that moves only when a row's maximum has grown by more than 2^8 (then the row of O and the row
-// sum are rescaled once, tcgen05.ld / tcgen05.st).  The scores and P V are issued by two threads (warps 1 and 2), the K and V
-// tiles have barriers of their own.
-//   tensor memory: S0 [0, 128), S1 [128, 256), O [256, 256 + D), P hi [384, 448), P lo [448, 512)
-//   shared memory: Q 2 x D/64 x 16 KB | 2 stages x (K D/64 x 16 KB, V D/64 x 16 KB)   (compressed cache: one stage + landing areas)
-#ifndef AT_PARTS_VALUE
-#define AT_PARTS_VALUE 2
-#endif
-constexpr int AT_BM = 128, AT_BN = 128, AT_PARTS = AT_PARTS_VALUE;
-constexpr int AT_KVS_MAX = 2;  // stages of the K / V tiles: two on the bf16 cache, one on the compressed cache (whose tiles are
-                               // expanded in place)
-constexpr int AT_PB = 2;       // the probabilities of a block live in tensor memory as two halves of 64 keys with barriers of their own:
-                               // P V of the first half runs while the softmax still works on the second
-constexpr int AT_SPLIT_MAX = 8; // CTAs that share the key blocks of a lone query tile
+// One CTA = 128 queries of one head (a query = a lane of tensor memory); keys in blocks of 128, dealt in turn to two groups of four
+// softmax warps, which run half a block apart: while one group exponentiates, the tensor cores work for the other.  Per block j:
+// S_j = Q K_j^T (tcgen05.mma, M 128, N 128, K = D; queries as two bf16 pieces) into the group's half of tensor memory;  a softmax
+// thread owns a row: it reads its 128 scores twice (tcgen05.ld; once for the maximum, once for the exponentials), masks on diagonal
+// blocks, and stores the probabilities as two bf16 pieces over the scores they came from (two keys per column; 32 scores become 16
+// columns of hi and 16 of lo);  O += P_j V_j (M 128, N = D, K = 128 keys; P from tensor memory, V straight from its cache rows as an
+// MN-major B operand), a sum of its own per group in tensor memory.  The exponentials are taken against a reference maximum that
+// moves only when the row's maximum has grown by more than 2^8 (then the row of O and the row sum are rescaled once).  At the end
+// the groups' sums (and those of the other CTAs of a cluster) meet in shared memory.  The scores and P V are issued by two threads
+// (warps 1 and 2), the K and V tiles have barriers of their own.
+//   tensor memory: scores and probabilities [0, 128) and [128, 256), O [256, 256 + D) and [256 + D, 256 + 2 D)
+//   shared memory: Q 2 x D/64 x 16 KB | 2 stages x (K D/64 x 16 KB, V D/64 x 16 KB)   (compressed cache: + landing areas)
+// With one group of eight warps, two threads to a row, a block took 2.6 us, now 2.0: every block's chain of scores, maximum (exchanged between
+// the two threads), exponentials and P V was walked with nothing beside it.  A prompt of 700 tokens behind 3000, 0.5B shape: 4067 -> 3635 us;
+// 271 behind 1000, 1.5B: 4016 -> 3648; 2048, 1.5B: attention 43 -> 38 us a layer.
+constexpr int AT_BM = 128, AT_BN = 128;
+constexpr int AT_GROUPS = 2;
+constexpr int AT_SPLIT_MAX = 16; // CTAs that share the key blocks of a query tile
 constexpr int AT_CW = 4;       // compressed cache: warps that expand the codes (AT_BN / AT_CW rows of a tile each)
-constexpr int AT_THREADS = 96 + 128 * AT_PARTS;   // producer, two issuers, softmax warps
+constexpr int AT_THREADS = 96 + 128 * AT_GROUPS;   // producer, two issuers, softmax warps
 
 // B operand in MN-major form for P V: the V tile is D/64 blocks of [64 keys][64 d] (128-byte rows, 128-byte swizzle).  N (= d)
 // runs along a row, K (= keys) across rows: groups of 8 keys are 1024 bytes apart (stride byte offset), the 64-column blocks
@@ -1175,46 +1154,44 @@ template <int D> struct AttnCfg {
     static constexpr int KBLK = D / 64;                        // 64-column blocks of a row of q, k, v
     static constexpr int Q_BYTES = 2 * KBLK * AT_BM * 128;     // two pieces
     static constexpr int K_BYTES = KBLK * AT_BN * 128, V_BYTES = K_BYTES;
-    static constexpr int SMEM = Q_BYTES + 2 * (K_BYTES + V_BYTES) + 1024;     // bf16 cache: two stages of K and V
-    // compressed cache: the 8-bit K tile has a landing area of its own, so that it can load while the scores of the block
-    // before still read the operand tile; the V tile lands in the first half of its operand tile's own place when a row of
-    // codes is as long as a 128-byte operand row (D = 128: every row is then expanded in place; there is no room for a second
-    // landing area), D = 64 gets one
+    static_assert(Q_BYTES == AT_BM * D * 4, "the rows of O pass through the place of Q, those of the second group through the first stage");
+    static constexpr int SMEM = Q_BYTES + 2 * (K_BYTES + V_BYTES) + 1024;     // two stages of K and V
+    // compressed cache: the 8-bit K tile has a landing area of its own, so that it can load while the scores of the blocks before still
+    // read the operand tiles; a V tile lands in the first half of its operand tile's own place when a row of codes is as long as a
+    // 128-byte operand row (D = 128: every row is then expanded in place; there is no room for more landing areas), D = 64 gets two
     static constexpr int RAW_BYTES = AT_BN * D;
-    static constexpr int SMEM_Q8 = Q_BYTES + (K_BYTES + V_BYTES) + (D == 128 ? 1 : 2) * RAW_BYTES + 1024;
-    static constexpr int TMEM_COLS = 2 * AT_BN + 2 * D <= 256 ? 256 : 512;   // S0, S1, O0, O1
+    static constexpr int SMEM_Q8 = SMEM + (D == 128 ? 1 : 3) * RAW_BYTES;
+    static constexpr int TMEM_COLS = 512;
 };
 
 template <int D, bool Q8>
-__global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q_hi,
+__global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1) prefill_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q_hi,
                                                                    const __grid_constant__ CUtensorMap map_q_lo,
                                                                    const __grid_constant__ CUtensorMap map_k,
                                                                    const __grid_constant__ CUtensorMap map_v, uint16_t *out, size_t plane,
                                                                    int T, int slot0, int nq, int group, int max_context,
                                                                    float scale_log2, uint32_t wait_limit, int *error, const float *k_scale,
-                                                                   const float *v_scale, float *part_o, float *part_ml) {
+                                                                   const float *v_scale, float *part_o, float2 *part_ml) {
     // Q8: the cache holds 8-bit codes and a scale per row (k_scale, v_scale: this layer's [nkv][max_context]); map_k / map_v then
     // describe byte matrices; two more warps expand the codes to bf16 (exactly) into the operand layout, the softmax multiplies
     // the scores by the keys' scales and folds the values' scales into the probabilities.
     using C = AttnCfg<D>;
     extern __shared__ uint8_t at_tc_dyn[];
-    __shared__ uint64_t kraw_full, kraw_empty, vraw_full;
+    __shared__ uint64_t kraw_full, kraw_empty, vraw_full[2];
     __shared__ __align__(16) float sc_k[Q8 ? 4 : 1][AT_BN], sc_v[Q8 ? 4 : 1][AT_BN];   // scales of the last four key blocks
-    constexpr int AT_KVS = Q8 ? 1 : 2;
-    __shared__ uint64_t q_full, k_full[AT_KVS_MAX], k_empty[AT_KVS_MAX], v_full[AT_KVS_MAX], v_empty[AT_KVS_MAX], s_full[2], s_empty[2], p_full[AT_PB], p_empty[AT_PB], o_full[2], o_empty[2], drain_bar[2], pair_bar[4];
+    __shared__ uint64_t q_full, k_full[2], k_empty[2], v_full[2], v_empty[2], s_full[2], p_full[2][2], pv_done[2], all_done, drain_bar[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ float xchg[2][AT_PARTS][AT_BM];      // row maxima / sums passed between the two threads of a row
+    __shared__ float2 row_ml[AT_GROUPS][AT_BM];     // reference maximum and sum of every row, at the end
     uint8_t *base = at_tc_dyn + ((1024u - (smem_u32(at_tc_dyn) & 1023u)) & 1023u);
-    uint8_t *sq = base, *skv = sq + C::Q_BYTES, *sraw = skv + AT_KVS * (C::K_BYTES + C::V_BYTES);   // sraw: landing area of the codes (Q8)
-    const uint32_t tmem_p_off = 2 * AT_BN + 128;             // P in tensor memory: hi piece 64 columns (128 keys, two per column), then lo
+    uint8_t *sq = base, *skv = sq + C::Q_BYTES, *sraw = skv + 2 * (C::K_BYTES + C::V_BYTES);   // sraw: landing areas of the codes (Q8)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // grid (heads, query tiles): CTAs start in linear order, so every head's longest tile (the last queries) starts first
     const int t0 = (gridDim.y - 1 - blockIdx.y) * AT_BM;
     const int h = blockIdx.x, hk = h / group;
     const int last_key = slot0 + min(t0 + AT_BM - 1, T - 1);
-    // gridDim.z > 1 (few queries behind a long cache): the key blocks are shared out among gridDim.z CTAs; each leaves its
-    // unnormalised row of O, its reference maximum and its row sum in part_o / part_ml, prefill_attention_merge_kernel adds them
+    // gridDim.z > 1 (a grid that would leave SMs idle): the key blocks of a query tile are shared out among gridDim.z CTAs;
+    // each leaves its unnormalised rows of O, their reference maxima and sums in part_o / part_ml, prefill_attention_merge_kernel adds them
     const int nb_total = last_key / AT_BN + 1, splits = gridDim.z;
     const int j0 = static_cast<int>(blockIdx.z) * nb_total / splits;          // first key block of this CTA
     const int nb = (static_cast<int>(blockIdx.z) + 1) * nb_total / splits - j0;   // its key blocks (indices below are local)
@@ -1222,12 +1199,12 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
     if (threadIdx.x == 0) {
         prefetch_map(&map_q_hi); prefetch_map(&map_q_lo); prefetch_map(&map_k); prefetch_map(&map_v);
         mbar_init(&q_full, 1);
-        for (int i = 0; i < AT_KVS; ++i) { mbar_init(&k_full[i], Q8 ? AT_CW : 1); mbar_init(&k_empty[i], 1); mbar_init(&v_full[i], Q8 ? AT_CW : 1); mbar_init(&v_empty[i], 1); }
-        mbar_init(&kraw_full, 1); mbar_init(&kraw_empty, AT_CW); mbar_init(&vraw_full, 1);
-        for (int i = 0; i < AT_PB; ++i) { mbar_init(&p_full[i], 4 * AT_PARTS); mbar_init(&p_empty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&s_empty[i], 4 * AT_PARTS); mbar_init(&o_full[i], 1); mbar_init(&o_empty[i], 4 * AT_PARTS); }
-        mbar_init(&drain_bar[0], 1); mbar_init(&drain_bar[1], 1);
-        for (int i = 0; i < 4; ++i) mbar_init(&pair_bar[i], AT_PARTS);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&k_full[i], Q8 ? AT_CW : 1); mbar_init(&k_empty[i], 1); mbar_init(&v_full[i], Q8 ? AT_CW : 1); mbar_init(&v_empty[i], 1);
+            mbar_init(&vraw_full[i], 1); mbar_init(&s_full[i], 1); mbar_init(&pv_done[i], 1); mbar_init(&drain_bar[i], 1);
+            mbar_init(&p_full[i][0], 4); mbar_init(&p_full[i][1], 4);
+        }
+        mbar_init(&kraw_full, 1); mbar_init(&kraw_empty, AT_CW); mbar_init(&all_done, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1240,69 +1217,85 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
     pdl_trigger();
+    if (threadIdx.x == 0)                    // the cache rows are sent for to L2 (a hint: rows that are still being written are read later)
+#pragma unroll 1
+        for (int j = j0; j < j0 + min(nb, 4); ++j)
+            for (int kb = 0; kb < (Q8 ? 1 : C::KBLK); ++kb) {
+                prefetch_tile_l2(&map_k, kb * 64, hk * max_context + j * AT_BN);
+                prefetch_tile_l2(&map_v, kb * 64, hk * max_context + j * AT_BN);
+            }
     pdl_wait();   // set-up done; from here on the kernel reads what its predecessor wrote
 
     if (warp == 0 && lane == 0) {            // producer: the query tile once, then the K and V rows of every key block
-        mbar_expect_tx(&q_full, C::Q_BYTES);
-        for (int kb = 0; kb < C::KBLK; ++kb) {
-            tma_load_2d(sq + kb * AT_BM * 128, &map_q_hi, h * D + kb * 64, t0, &q_full);
-            tma_load_2d(sq + (C::KBLK + kb) * AT_BM * 128, &map_q_lo, h * D + kb * 64, t0, &q_full);
+        if (nb > 0) {
+            mbar_expect_tx(&q_full, C::Q_BYTES);
+            for (int kb = 0; kb < C::KBLK; ++kb) {
+                tma_load_2d(sq + kb * AT_BM * 128, &map_q_hi, h * D + kb * 64, t0, &q_full);
+                tma_load_2d(sq + (C::KBLK + kb) * AT_BM * 128, &map_q_lo, h * D + kb * 64, t0, &q_full);
+            }
         }
-        // K and V of a block have barriers of their own: the K tile is free again as soon as S_j is done, a block earlier than
-        // the V tile, and the next scores need only K.  Order of issue: K_0, then K_{j+1} before V_j, so that the wait for V's
-        // tile (P V of the block before) never holds the next K tile back.
+        // K and V of a block have barriers of their own: the K tile is free again as soon as S_j is done, before the V tile, and the
+        // next scores need only K.  Order of issue: K_0, then K_{j+1} before V_j, so that the wait for V's tile never holds the next
+        // K tile back.  Block j uses stage j & 1.
         int nk = 0, nv = 0;
         auto load_k = [&](int j) {
-            const int st = j % AT_KVS;
+            const int st = j & 1, y = hk * max_context + (j0 + j) * AT_BN;
             uint8_t *k = skv + st * (C::K_BYTES + C::V_BYTES);
-            if (j >= AT_KVS && !mbar_wait(Q8 ? &kraw_empty : &k_empty[st], ((j / AT_KVS) - 1) & 1, &abort_flag, wait_limit)) return false;
             if constexpr (Q8) {
+                if (j >= 1 && !mbar_wait(&kraw_empty, (j - 1) & 1, &abort_flag, wait_limit)) return false;
                 mbar_expect_tx(&kraw_full, C::RAW_BYTES);
-                tma_load_2d(sraw, &map_k, 0, hk * max_context + (j0 + j) * AT_BN, &kraw_full);
+                tma_load_2d(sraw, &map_k, 0, y, &kraw_full);
             } else {
+                if (j >= 2 && !mbar_wait(&k_empty[st], ((j >> 1) - 1) & 1, &abort_flag, wait_limit)) return false;
                 mbar_expect_tx(&k_full[st], C::K_BYTES);
-                for (int kb = 0; kb < C::KBLK; ++kb) tma_load_2d(k + kb * AT_BN * 128, &map_k, kb * 64, hk * max_context + (j0 + j) * AT_BN, &k_full[st]);
+                for (int kb = 0; kb < C::KBLK; ++kb) tma_load_2d(k + kb * AT_BN * 128, &map_k, kb * 64, y, &k_full[st]);
             }
             nk = j + 1;
             return true;
         };
         auto load_v = [&](int j) {
-            const int st = j % AT_KVS;
+            const int st = j & 1, y = hk * max_context + (j0 + j) * AT_BN;
             uint8_t *v = skv + st * (C::K_BYTES + C::V_BYTES) + C::K_BYTES;
-            if (j >= AT_KVS && !mbar_wait(&v_empty[st], ((j / AT_KVS) - 1) & 1, &abort_flag, wait_limit)) return false;
+            if (j >= 2 && !mbar_wait(&v_empty[st], ((j >> 1) - 1) & 1, &abort_flag, wait_limit)) return false;
             if constexpr (Q8) {
-                mbar_expect_tx(&vraw_full, C::RAW_BYTES);
-                tma_load_2d(D == 128 ? v : sraw + C::RAW_BYTES, &map_v, 0, hk * max_context + (j0 + j) * AT_BN, &vraw_full);
+                mbar_expect_tx(&vraw_full[st], C::RAW_BYTES);
+                tma_load_2d(D == 128 ? v : sraw + (1 + st) * C::RAW_BYTES, &map_v, 0, y, &vraw_full[st]);
             } else {
                 mbar_expect_tx(&v_full[st], C::V_BYTES);
-                for (int kb = 0; kb < C::KBLK; ++kb) tma_load_2d(v + kb * AT_BN * 128, &map_v, kb * 64, hk * max_context + (j0 + j) * AT_BN, &v_full[st]);
+                for (int kb = 0; kb < C::KBLK; ++kb) tma_load_2d(v + kb * AT_BN * 128, &map_v, kb * 64, y, &v_full[st]);
             }
             nv = j + 1;
             return true;
         };
-        bool ok = load_k(0);
+        bool ok = nb > 0 && load_k(0);
+#pragma unroll 1
         for (int j = 0; j < nb && ok; ++j) {
             if (j + 1 < nb) ok = load_k(j + 1);
             if (ok) ok = load_v(j);
         }
         if (abort_flag) {   // giving up: the copies in flight must land before the shared memory is released
             int dummy = 0;
-            mbar_wait(&q_full, 0, &dummy, wait_limit);
-            for (int j = nk > AT_KVS ? nk - AT_KVS : 0; j < nk; ++j) mbar_wait(Q8 ? &kraw_full : &k_full[j % AT_KVS], (j / AT_KVS) & 1, &dummy, wait_limit);
-            for (int j = nv > AT_KVS ? nv - AT_KVS : 0; j < nv; ++j) mbar_wait(Q8 ? &vraw_full : &v_full[j % AT_KVS], (j / AT_KVS) & 1, &dummy, wait_limit);
+            if (nb > 0) mbar_wait(&q_full, 0, &dummy, wait_limit);
+            if (Q8) { if (nk > 0) mbar_wait(&kraw_full, (nk - 1) & 1, &dummy, wait_limit); }
+            else
+#pragma unroll 1
+            for (int j = nk > 2 ? nk - 2 : 0; j < nk; ++j) mbar_wait(&k_full[j & 1], (j >> 1) & 1, &dummy, wait_limit);
+#pragma unroll 1
+            for (int j = nv > 2 ? nv - 2 : 0; j < nv; ++j) mbar_wait(Q8 ? &vraw_full[j & 1] : &v_full[j & 1], (j >> 1) & 1, &dummy, wait_limit);
         }
     } else if (warp == 1 && lane == 0) {     // issuer of the scores: S_j = Q K_j^T, hi pieces then lo pieces
         // (two issuing threads, scores here and P V in warp 2: a tcgen05.mma takes about 40 ns to issue, and one thread issuing
         // both, with its six waits per block, was what bounded the kernel: 2.3 us per block)
         constexpr uint32_t idesc_s = umma_idesc_bf16(AT_BM, AT_BN);
-        bool ok = mbar_wait(&q_full, 0, &abort_flag, wait_limit);
+        bool ok = nb == 0 || mbar_wait(&q_full, 0, &abort_flag, wait_limit);
+#pragma unroll 1
         for (int j = 0; j < nb && ok; ++j) {
-            const int st = j % AT_KVS, sb = j & 1;
-            ok = mbar_wait(&k_full[st], (j / AT_KVS) & 1, &abort_flag, wait_limit);
-            if (ok && j >= 2) ok = mbar_wait(&s_empty[sb], ((j >> 1) - 1) & 1, &abort_flag, wait_limit);   // the softmax has read S_{j-2}
+            const int g = j & 1, i = j >> 1;     // the group's i-th block
+            ok = mbar_wait(&k_full[g], i & 1, &abort_flag, wait_limit);
+            if (ok && i >= 1) ok = mbar_wait(&pv_done[g], (i - 1) & 1, &abort_flag, wait_limit);   // P_{j-2}, which lies over S_{j-2}, has been multiplied
             if (!ok) break;
             tc_fence_after();
-            const uint32_t k = smem_u32(skv + st * (C::K_BYTES + C::V_BYTES)), acc = tmem + sb * AT_BN;
+            const uint32_t k = smem_u32(skv + g * (C::K_BYTES + C::V_BYTES)), acc = tmem + g * AT_BN;
 #pragma unroll
             for (int piece = 0; piece < 2; ++piece)
 #pragma unroll
@@ -1312,46 +1305,47 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) umma_bf16(acc, da + 2 * kk, db + 2 * kk, idesc_s, (piece | kb | kk) != 0);
                 }
-            umma_commit(&s_full[sb]);
-            umma_commit(&k_empty[st]);       // the K rows are free when these have read them
+            umma_commit(&s_full[g]);
+            umma_commit(&k_empty[g]);        // the K rows are free when these have read them
         }
         if (!ok) {
             int dummy = 0;
             umma_commit(&drain_bar[0]);
             mbar_wait(&drain_bar[0], 0, &dummy, wait_limit);
         }
-    } else if (warp == 2 && lane == 0) {     // issuer of O_j = P_j V_j
+    } else if (warp == 2 && lane == 0) {     // issuer of O += P_j V_j, the block's two halves of 64 keys as they come
         constexpr uint32_t idesc_o = umma_idesc_bf16(AT_BM, D) | (1u << 16);   // B (= V) is MN-major
         bool ok = true;
+#pragma unroll 1
         for (int j = 0; j < nb && ok; ++j) {
-            const int st = j % AT_KVS;
-            ok = mbar_wait(&v_full[st], (j / AT_KVS) & 1, &abort_flag, wait_limit);
-            const uint32_t v = smem_u32(skv + st * (C::K_BYTES + C::V_BYTES) + C::K_BYTES);
+            const int g = j & 1, i = j >> 1;
+            ok = mbar_wait(&v_full[g], i & 1, &abort_flag, wait_limit);
+            const uint32_t v = smem_u32(skv + g * (C::K_BYTES + C::V_BYTES) + C::K_BYTES);
 #pragma unroll
-            for (int h = 0; h < 2 && ok; ++h) {          // the two 64-key halves of the block
-                ok = mbar_wait(&p_full[h], j & 1, &abort_flag, wait_limit);
+            for (int half = 0; half < 2 && ok; ++half) {
+                ok = mbar_wait(&p_full[g][half], i & 1, &abort_flag, wait_limit);
                 if (!ok) break;
                 tc_fence_after();
 #pragma unroll
-                for (int piece = 0; piece < 2; ++piece)
+                for (int kg = 4 * half; kg < 4 * half + 4; ++kg)     // 16 keys: 8 columns of either piece of P, 2048 bytes of the V tile
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)       // 16 keys: 8 columns of P in tensor memory, 2048 bytes of the V tile
-                        umma_bf16_ts(tmem + 2 * AT_BN, tmem + tmem_p_off + h * 64 + piece * 32 + kk * 8,
-                                     umma_desc_sw128_mn(v + (h * 4 + kk) * 2048, AT_BN * 128), idesc_o, (j | h | piece | kk) != 0);   // O accumulates
-                umma_commit(&p_empty[h]);
+                    for (int piece = 0; piece < 2; ++piece)
+                        umma_bf16_ts(tmem + 2 * AT_BN + g * D, tmem + g * AT_BN + (kg >> 1) * 32 + piece * 16 + (kg & 1) * 8,
+                                     umma_desc_sw128_mn(v + kg * 2048, AT_BN * 128), idesc_o, (i | kg | piece) != 0);
             }
             if (!ok) break;
-            umma_commit(&o_full[0]);
-            umma_commit(&v_empty[st]);
+            umma_commit(&pv_done[g]);
+            umma_commit(&v_empty[g]);
         }
-        if (!ok) {
+        if (ok) {
+            umma_commit(&all_done);
+        } else {
             int dummy = 0;
             umma_commit(&drain_bar[1]);
             mbar_wait(&drain_bar[1], 0, &dummy, wait_limit);
         }
     }
     else if (Q8 && warp >= AT_THREADS / 32) {   // compressed cache: expand the 8-bit tiles to bf16 operand tiles (AT_CW warps, AT_BN / AT_CW rows each)
-        static_assert(!Q8 || AT_KVS == 1, "one raw tile of K and of V in flight");
         const int cw = warp - AT_THREADS / 32;
         constexpr int LPR = D / 16, RPS = 32 / LPR;       // lanes per row of codes (16 codes each), rows per step
         constexpr int ROWS = AT_BN / AT_CW;               // rows of a tile this warp expands
@@ -1394,10 +1388,10 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
                 *reinterpret_cast<uint4 *>(dst + (((2 * (c & 3) + 1) ^ (row & 7)) << 4)) = b;
             }
         };
-        uint8_t *k = skv, *v = k + C::K_BYTES;
         auto expand_k = [&](int j) {
-            if (!(warp_wait(&kraw_full, j & 1) && (j == 0 || warp_wait(&k_empty[0], (j - 1) & 1)))) return false;   // the codes are here, the operand tile is free
-            expand_tile(k, sraw);
+            const int st = j & 1;
+            if (!(warp_wait(&kraw_full, j & 1) && (j < 2 || warp_wait(&k_empty[st], ((j >> 1) - 1) & 1)))) return false;   // the codes are here, the operand tile is free
+            expand_tile(skv + st * (C::K_BYTES + C::V_BYTES), sraw);
             __syncwarp();
             if (lane == 0) mbar_arrive(&kraw_empty);       // the next K tile may land
             for (int i = lane; i < ROWS; i += 32) {        // the scales of this block's keys (both kinds: they are in memory already)
@@ -1407,31 +1401,33 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&k_full[0]);
+            if (lane == 0) mbar_arrive(&k_full[st]);
             return true;
         };
-        bool ok = expand_k(0);
+        bool ok = nb > 0 && expand_k(0);
+#pragma unroll 1
         for (int j = 0; j < nb && ok; ++j) {              // like the producer: the next K tile before this block's V tile
             if (j + 1 < nb) ok = expand_k(j + 1);
             if (!ok) break;
-            ok = warp_wait(&vraw_full, j & 1);
+            const int st = j & 1;
+            ok = warp_wait(&vraw_full[st], (j >> 1) & 1);
             if (!ok) break;
-            expand_tile(v, D == 128 ? v : sraw + C::RAW_BYTES);
+            uint8_t *v = skv + st * (C::K_BYTES + C::V_BYTES) + C::K_BYTES;
+            expand_tile(v, D == 128 ? v : sraw + (1 + st) * C::RAW_BYTES);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&v_full[0]);
+            if (lane == 0) mbar_arrive(&v_full[st]);
         }
     }
-    else if (warp >= 3) {                    // softmax: AT_PARTS threads per query row (= lane of tensor memory), AT_BN / AT_PARTS keys of a block each
-        const int quarter = warp & 3, part = (warp - 3) >> 2, row = quarter * 32 + lane;
-        const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+    else if (warp >= 3) {                    // softmax: a thread per query row (= lane of tensor memory), the groups take blocks in turn
+        const int quarter = warp & 3, g = (warp - 3) >> 2, row = quarter * 32 + lane;
+        const uint32_t tlane = tmem + (static_cast<uint32_t>(quarter * 32) << 16), srow = tlane + g * AT_BN, orow = tlane + 2 * AT_BN + g * D;
         const int qi = slot0 + t0 + row;     // cache slot of this query: it sees the keys 0 .. qi
-        constexpr int DP = D / AT_PARTS;     // this thread's columns of the output row
         // The output row accumulates in tensor memory over the blocks (P V with accumulation).  The exponentials are taken
         // against a reference maximum m_ref that moves only when the row's maximum has grown by more than 2^8 in the
         // exponent (or at the first block); then the row of O and the row sum are rescaled once.  In between the
         // probabilities may reach 2^8, which fp32 sums and the two bf16 pieces carry without loss.
-        float m_ref = -INFINITY, l_run = 0.f;
+        float m_ref = -1e30f, l_run = 0.f;   // (a row that sees none of its keys keeps a finite reference)
         bool ok = true;
         // one lane waits / arrives for its warp (an mbarrier operation per thread would cost more than the arithmetic)
         auto warp_wait = [&](uint64_t *bar, int parity) {
@@ -1439,149 +1435,173 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
             if (lane == 0) r = mbar_wait(bar, parity, &abort_flag, wait_limit) ? 1 : 0;
             return __shfl_sync(0xffffffffu, r, 0) != 0;
         };
-        auto warp_arrive = [&](uint64_t *bar) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar);
-        };
-        auto row_sync = [&](int round) {     // the AT_PARTS warps of a quarter meet (bounded like every other wait)
-            warp_arrive(&pair_bar[quarter]);
-            return warp_wait(&pair_bar[quarter], round & 1);
-        };
-        for (int j = 0; j < nb; ++j) {
-            ok = warp_wait(&s_full[j & 1], (j >> 1) & 1);
+#pragma unroll 1
+        for (int j = g; j < nb; j += AT_GROUPS) {
+            const int i = j >> 1;
+            ok = warp_wait(&s_full[g], i & 1);
             if (!ok) break;
             tc_fence_after();
-            const bool diagonal = (j0 + j) * AT_BN + AT_BN - 1 > slot0 + t0;   // some query of the tile does not see the whole block
-            // this thread's keys: 32 of the block's first half (chunk 0), 32 of its second half (chunk 1)
-            static_assert(AT_PARTS == 2 && AT_BN == 128, "two threads per row, 2 x 32 keys each");
-            const uint32_t srow = trow + (j & 1) * AT_BN + part * 32;
-            auto load_chunk = [&](int c, float *v) {    // scores of chunk c, scaled (Q8) and masked
-                tmem_ld32(srow + c * 64, v);
-                tmem_ld_wait();
+            const int key0 = (j0 + j) * AT_BN;
+            const bool diagonal = key0 + AT_BN - 1 > slot0 + t0;   // some query of the tile does not see the whole block
+            auto receive = [&](int c, float *v) {       // 32 scores, scaled (Q8) and masked
+                tmem_ld_ready(v);
                 if constexpr (Q8) {                   // scores of codes -> scores: the keys' scales (16-byte shared-memory reads)
-                    const float4 *sk = reinterpret_cast<const float4 *>(&sc_k[j & 3][c * 64 + part * 32]);
+                    const float4 *sk = reinterpret_cast<const float4 *>(&sc_k[j & 3][c * 32]);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float4 f = sk[i];
-                        v[4 * i] *= f.x; v[4 * i + 1] *= f.y; v[4 * i + 2] *= f.z; v[4 * i + 3] *= f.w;
+                    for (int e = 0; e < 8; ++e) {
+                        const float4 f = sk[e];
+                        v[4 * e] *= f.x; v[4 * e + 1] *= f.y; v[4 * e + 2] *= f.z; v[4 * e + 3] *= f.w;
                     }
                 }
                 if (diagonal) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        if ((j0 + j) * AT_BN + c * 64 + part * 32 + i > qi) v[i] = -INFINITY;
+                    for (int e = 0; e < 32; ++e)
+                        if (key0 + c * 32 + e > qi) v[e] = -INFINITY;
                 }
             };
-            float mx = -INFINITY;
+            // Both passes go over the chunks two by two, the next chunk's scores under way: eight chunks written out are more
+            // instructions than the caches next to the schedulers hold, one at a time waits for every read.
+            // (Compressed cache: one at a time all the same, its warps have registers for one.)
+            constexpr bool PING = !Q8;
+            float va[32], vb[PING ? 32 : 1];
+            float mx = m_ref;
+            auto fold = [&](const float *v) {
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {         // pass 1: the maximum over this thread's keys the query sees
-                float v[32];
-                load_chunk(c, v);
-#pragma unroll
-                for (int i = 0; i < 32; i += 4) mx = fmaxf(mx, fmaxf(fmaxf(v[i], v[i + 1]), fmaxf(v[i + 2], v[i + 3])));
+                for (int e = 0; e < 32; e += 4) mx = fmaxf(mx, fmaxf(fmaxf(v[e], v[e + 1]), fmaxf(v[e + 2], v[e + 3])));
+            };
+            tmem_ld32(srow, va);
+#pragma unroll 1
+            for (int c = 0; c < 4; c += PING ? 2 : 1) {      // pass 1: the maximum over the keys the query sees
+                receive(c, va);
+                if constexpr (PING) {
+                    tmem_ld32(srow + (c + 1) * 32, vb);
+                    fold(va);
+                    receive(c + 1, vb);
+                    tmem_ld32(srow + ((c + 2) & 3) * 32, va);     // (at the end: the first again)
+                    fold(vb);
+                } else {
+                    fold(va);
+                    tmem_ld32(srow + ((c + 1) & 3) * 32, va);
+                }
             }
-            xchg[j & 1][part][row] = mx;     // the row maximum needs the other threads' keys
-            ok = row_sync(j);
-            if (!ok) break;
-            mx = m_ref;
-#pragma unroll
-            for (int q = 0; q < AT_PARTS; ++q) mx = fmaxf(mx, xchg[j & 1][q][row]);
-            if (j == 0) {
-                m_ref = fmaxf(mx, -1e30f);   // nothing accumulated yet (a row that sees none of this CTA's keys keeps a finite reference)
+            if (i == 0) {
+                m_ref = mx;
             } else if (__any_sync(0xffffffffu, (mx - m_ref) * scale_log2 > 8.f)) {
-                // some row of this warp has outgrown its reference (both warps of a quarter see the same rows and maxima, so they
-                // decide alike): every row moves its reference to its maximum and rescales its sum and its part of O, once the
-                // multiplies of the blocks before are done (the next one waits for this block's probabilities)
-                ok = warp_wait(&o_full[0], (j - 1) & 1);
+                // some row of this warp has outgrown its reference: every row moves its reference to its maximum and rescales its sum
+                // and its row of O (the multiply of the group's block before is done: these scores lie where its probabilities lay)
+                ok = warp_wait(&pv_done[g], (i - 1) & 1);
                 if (!ok) break;
                 tc_fence_after();
                 const float f = fast_exp2((m_ref - mx) * scale_log2);
                 l_run *= f;
-                {
-                    float v[DP];
-                    tmem_ld<DP>(trow + 2 * AT_BN + part * DP, v);
+#pragma unroll 1
+                for (int c = 0; c < D / 32; ++c) {
+                    float v[32];
+                    tmem_ld32(orow + c * 32, v);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < DP; ++i) v[i] *= f;
-                    tmem_st<DP>(trow + 2 * AT_BN + part * DP, v);
+                    for (int e = 0; e < 32; ++e) v[e] *= f;
+                    tmem_st32(orow + c * 32, v);
                 }
                 tmem_st_wait();
-                tc_fence_before();
                 m_ref = mx;
             }
             const float neg = -m_ref * scale_log2;
             float sum0 = 0.f, sum1 = 0.f;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {         // pass 2: probabilities as two bf16 pieces, half by half
-                float v[32];
-                load_chunk(c, v);
-                if (c == 1) {
-                    tc_fence_before();
-                    warp_arrive(&s_empty[j & 1]);     // S_j has been read for the last time
-                }
+            auto spend = [&](int c, const float *v) {     // probabilities as two bf16 pieces over the scores
                 uint32_t phi[16], plo[16];        // two keys per word
 #pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    const float p0 = fast_exp2(fmaf(v[i], scale_log2, neg)), p1 = fast_exp2(fmaf(v[i + 1], scale_log2, neg));
+                for (int e = 0; e < 32; e += 2) {
+                    const float p0 = fast_exp2(fmaf(v[e], scale_log2, neg)), p1 = fast_exp2(fmaf(v[e + 1], scale_log2, neg));
                     sum0 += p0;
                     sum1 += p1;
                     if constexpr (Q8) {               // the values' scales ride on the probabilities
-                        const float2 f = *reinterpret_cast<const float2 *>(&sc_v[j & 3][c * 64 + part * 32 + i]);
-                        split2x2_trunc(p0 * f.x, p1 * f.y, phi[i / 2], plo[i / 2]);
+                        const float2 f = *reinterpret_cast<const float2 *>(&sc_v[j & 3][c * 32 + e]);
+                        split2x2_trunc(p0 * f.x, p1 * f.y, phi[e / 2], plo[e / 2]);
                     } else {
-                        split2x2_trunc(p0, p1, phi[i / 2], plo[i / 2]);
+                        split2x2_trunc(p0, p1, phi[e / 2], plo[e / 2]);
                     }
                 }
-                if (j >= 1) {                     // this half's multiply of the block before is done
-                    ok = warp_wait(&p_empty[c], (j - 1) & 1);
-                    if (!ok) break;
-                }
                 // P as the A operand in tensor memory: lane = query row, a column holds two consecutive keys (bf16)
-                tmem_st16(trow + tmem_p_off + c * 64 + part * 16, reinterpret_cast<const float *>(phi));
-                tmem_st16(trow + tmem_p_off + c * 64 + 32 + part * 16, reinterpret_cast<const float *>(plo));
-                tmem_st_wait();
+                tmem_st16(srow + c * 32, reinterpret_cast<const float *>(phi));
+                tmem_st16(srow + c * 32 + 16, reinterpret_cast<const float *>(plo));
+            };
+#pragma unroll 1
+            for (int c = 0; c < 4; c += PING ? 2 : 1) {      // pass 2
+                receive(c, va);
+                if constexpr (PING) {
+                    tmem_ld32(srow + (c + 1) * 32, vb);
+                    spend(c, va);
+                    receive(c + 1, vb);
+                    if (c == 0) tmem_ld32(srow + 64, va);
+                    spend(c + 1, vb);
+                } else {
+                    spend(c, va);
+                    if (c < 3) tmem_ld32(srow + (c + 1) * 32, va);
+                    if ((c & 1) == 0) continue;
+                }
+                tmem_st_wait();                   // a half is complete
                 tc_fence_before();
-                warp_arrive(&p_full[c]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&p_full[g][c >> 1]);
             }
-            if (!ok) break;
             l_run += sum0 + sum1;
         }
-        float o[DP];
-        if (ok) ok = warp_wait(&o_full[0], (nb - 1) & 1);   // the last block's multiply
+        if (ok && nb > 0) ok = warp_wait(&all_done, 0);   // the last multiply: Q, K and V have been read for the last time
         if (ok) {
+            // the unnormalised row over the query tile / the first stage: 16-byte pieces, their index xor the row
             tc_fence_after();
-            tmem_ld<DP>(trow + 2 * AT_BN + part * DP, o);
-            tmem_ld_wait();
-        }
-        if (ok) {
-            xchg[nb & 1][part][row] = l_run; // the parts of the row sum
-            ok = row_sync(nb);
-            l_run = 0.f;
+            float4 *dst = reinterpret_cast<float4 *>(sq + g * C::Q_BYTES) + row * (D / 4);
+#pragma unroll 1
+            for (int c = 0; c < D / 32; ++c) {
+                float v[32];
+                if (g < nb) {
+                    tmem_ld32(orow + c * 32, v);
+                    tmem_ld_wait();
+                } else {
 #pragma unroll
-            for (int q = 0; q < AT_PARTS; ++q) l_run += xchg[nb & 1][q][row];
-        }
-        const int t = t0 + row;
-        if (ok && t < T && splits > 1) {     // partial result of this CTA's key blocks
-            const size_t slot = (static_cast<size_t>(blockIdx.z) * AT_BM + row) * nq + h;
-            float *dst = part_o + slot * D + part * DP;
+                    for (int e = 0; e < 32; ++e) v[e] = 0.f;
+                }
 #pragma unroll
-            for (int i = 0; i < DP; i += 4) *reinterpret_cast<float4 *>(dst + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
-            if (part == 0) { part_ml[slot * 2] = m_ref; part_ml[slot * 2 + 1] = l_run; }
-        } else if (ok && t < T) {
-            const float inv = 1.f / l_run;
-            uint16_t *dst = out + static_cast<size_t>(t) * nq * D + static_cast<size_t>(h) * D + part * DP;
-#pragma unroll
-            for (int i = 0; i < DP; i += 8) {
-                uint4 hi, lo;
-                split2x2(o[i] * inv, o[i + 1] * inv, hi.x, lo.x); split2x2(o[i + 2] * inv, o[i + 3] * inv, hi.y, lo.y);
-                split2x2(o[i + 4] * inv, o[i + 5] * inv, hi.z, lo.z); split2x2(o[i + 6] * inv, o[i + 7] * inv, hi.w, lo.w);
-                *reinterpret_cast<uint4 *>(dst + i) = hi;
-                *reinterpret_cast<uint4 *>(dst + plane + i) = lo;
+                for (int e = 0; e < 8; ++e) dst[(c * 8 + e) ^ (row & 7)] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
             }
+            row_ml[g][row] = make_float2(m_ref, l_run);
         }
     }
     tc_fence_before();
     __syncthreads();
+    if (!abort_flag) {
+        // O = sum O_g 2^((m_g - M) c), L = sum l_g 2^((m_g - M) c) over the two groups, M = max m_g; a warp per row, D / 32 columns per lane: O / L, or (one of
+        // several CTAs) O, M and L
+        constexpr int V = D / 32;
+        const int live = min(AT_BM, T - t0);
+#pragma unroll 1
+        for (int r = warp; r < live; r += AT_THREADS / 32 + (Q8 ? AT_CW : 0)) {
+            const float2 a = row_ml[0][r], b = row_ml[1][r];
+            const float top = fmaxf(a.x, b.x), wa = fast_exp2((a.x - top) * scale_log2), wb = fast_exp2((b.x - top) * scale_log2), l = fmaf(a.y, wa, b.y * wb);
+            const float *x = reinterpret_cast<const float *>(sq) + r * D + (((lane * V / 4) ^ (r & 7)) << 2) + lane * V % 4, *y = x + C::Q_BYTES / 4;
+            float o[V];
+#pragma unroll
+            for (int i = 0; i < V; ++i) o[i] = fmaf(x[i], wa, y[i] * wb);
+            const size_t i = static_cast<size_t>(t0 + r) * nq + h;
+            if (splits > 1) {
+                const size_t slot = static_cast<size_t>(blockIdx.z) * gridDim.y * AT_BM * nq + i;
+                if (lane == 0) part_ml[slot] = make_float2(top, l);
+#pragma unroll
+                for (int e = 0; e < V; e += 2) *reinterpret_cast<float2 *>(part_o + slot * D + lane * V + e) = make_float2(o[e], o[e + 1]);
+                continue;
+            }
+            const float inv = 1.f / l;
+            uint16_t *dst = out + i * D + lane * V;
+#pragma unroll
+            for (int e = 0; e < V; e += 2) {
+                uint32_t hi, lo;
+                split2x2(o[e] * inv, o[e + 1] * inv, hi, lo);
+                *reinterpret_cast<uint32_t *>(dst + e) = hi;
+                *reinterpret_cast<uint32_t *>(dst + plane + e) = lo;
+            }
+        }
+    }
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(AttnCfg<D>::TMEM_COLS) : "memory");
@@ -1589,32 +1609,43 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0)) prefill_at
     if (threadIdx.x == 0 && abort_flag) atomicExch(error, 1);
 }
 
-// Adds the partial results of a query tile whose key blocks were shared out among `splits` CTAs: for row t and head h,
-// M = max m_s, O = sum O_s 2^((m_s - M) c), L = sum l_s 2^((m_s - M) c), out = O / L as two bf16 planes.  grid (T, nq), D / 4 threads.
+// Adds the partial rows of query tiles whose key blocks were shared out: for row t and head h, M = max m_p,
+// O = sum O_p 2^((m_p - M) c), L = sum l_p 2^((m_p - M) c), out = O / L as two bf16 planes.  A warp per row, D / 32 columns per lane, all parts'
+// loads under way together.  (A cluster's CTAs merging through distributed shared memory took 11 us where these 2.6 us and the stores
+// do: code that runs once per CTA comes from memory line by line, and the clusters of a full CTA per SM wait for a free GPC.)
+static_assert(AT_SPLIT_MAX <= 32, "a lane per part");
 template <int D>
-__global__ void __launch_bounds__(D / 4) prefill_attention_merge_kernel(const float *part_o, const float *part_ml, int splits, uint16_t *out,
-                                                                        size_t plane, int nq, float scale_log2) {
+__global__ void __launch_bounds__(128) prefill_attention_merge_kernel(const float *part_o, const float2 *part_ml, int parts, int rows, uint16_t *out, size_t plane, int T,
+                                                                      int nq, float scale_log2) {
     pdl_trigger();
     pdl_wait();
-    const int t = blockIdx.x, h = blockIdx.y, i = threadIdx.x * 4;
-    float mmax = -INFINITY;
-    for (int s = 0; s < splits; ++s) mmax = fmaxf(mmax, part_ml[((static_cast<size_t>(s) * AT_BM + t) * nq + h) * 2]);
-    float l = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = 0; s < splits; ++s) {
-        const size_t slot = (static_cast<size_t>(s) * AT_BM + t) * nq + h;
-        const float w = fast_exp2((part_ml[slot * 2] - mmax) * scale_log2);
-        const float4 o = *reinterpret_cast<const float4 *>(part_o + slot * D + i);
-        l = fmaf(part_ml[slot * 2 + 1], w, l);
-        acc.x = fmaf(o.x, w, acc.x); acc.y = fmaf(o.y, w, acc.y); acc.z = fmaf(o.z, w, acc.z); acc.w = fmaf(o.w, w, acc.w);
+    constexpr int V = D / 32;
+    const int lane = threadIdx.x & 31, i = blockIdx.x * 4 + (threadIdx.x >> 5);    // row and head: t * nq + h
+    if (i >= T * nq) return;
+    const size_t part = static_cast<size_t>(rows) * nq;      // partial rows of a part
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (lane < parts) ml = part_ml[lane * part + i];
+    const float top = warp_max(ml.x), w = lane < parts ? fast_exp2((ml.x - top) * scale_log2) : 0.f, inv = 1.f / warp_sum(ml.y * w);
+    float acc[V] = {};
+#pragma unroll 8
+    for (int p = 0; p < parts; ++p) {
+        const float *src = part_o + (p * part + i) * D + lane * V;
+        const float f = __shfl_sync(0xffffffffu, w, p);
+#pragma unroll
+        for (int e = 0; e < V; e += 2) {
+            const float2 x = *reinterpret_cast<const float2 *>(src + e);
+            acc[e] = fmaf(x.x, f, acc[e]);
+            acc[e + 1] = fmaf(x.y, f, acc[e + 1]);
+        }
     }
-    const float inv = 1.f / l;
-    uint2 hi, lo;
-    split2x2(acc.x * inv, acc.y * inv, hi.x, lo.x);
-    split2x2(acc.z * inv, acc.w * inv, hi.y, lo.y);
-    uint16_t *dst = out + static_cast<size_t>(t) * nq * D + static_cast<size_t>(h) * D + i;
-    *reinterpret_cast<uint2 *>(dst) = hi;
-    *reinterpret_cast<uint2 *>(dst + plane) = lo;
+    uint16_t *dst = out + static_cast<size_t>(i) * D + lane * V;
+#pragma unroll
+    for (int e = 0; e < V; e += 2) {
+        uint32_t hi, lo;
+        split2x2(acc[e] * inv, acc[e + 1] * inv, hi, lo);
+        *reinterpret_cast<uint32_t *>(dst + e) = hi;
+        *reinterpret_cast<uint32_t *>(dst + plane + e) = lo;
+    }
 }
 
 // Launch with the programmatic-stream-serialization attribute (see pdl_trigger / pdl_wait) for passes of up to 1024 tokens:
@@ -1747,30 +1778,28 @@ bool encode_bytes_map(CUtensorMap *m, const void *base, long long rows, int row_
 }
 
 // kc / vc: this layer's cache, bf16 rows or (k_scale != nullptr) rows of 8-bit codes with their scales.
-// A single query tile behind a long cache (a short suffix behind a prefix, a verified block) would run on n_q CTAs only: its key
-// blocks are then shared out among up to AT_SPLIT_MAX CTAs per head and the partial results merged (part_o / part_ml: room for
-// AT_SPLIT_MAX x 128 rows).
+// Few query tiles behind a long cache (a short suffix behind a prefix, a verified block) would run on few CTAs, each walking the whole cache: the key
+// blocks are then shared out among as many CTAs as fit the SMs once, and their partial rows merged (part_o / part_ml: room for
+// num_sms tiles of 128 rows).  Two blocks cost a CTA about 3.5 us (one for either group), the merge about as much.
 template <int D>
 const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *vc, const float *k_scale, const float *v_scale, uint16_t *out,
                                 size_t plane, int T, int slot0, int nq, int nkv, int max_context, uint32_t wait_limit, int *error,
-                                float *part_o, float *part_ml, int num_sms, cudaStream_t s) {
-    CUtensorMap mqh, mql, mk, mv;
+                                float *part_o, float2 *part_ml, int num_sms, cudaStream_t s) {
     const long long kv_rows = static_cast<long long>(nkv) * max_context;
     const bool q8 = k_scale != nullptr;
+    CUtensorMap mqh, mql, mk, mv;
     if (!encode_operand_map(&mqh, q, T, nq * D) || !encode_operand_map(&mql, q + plane, T, nq * D)) return "cuTensorMapEncodeTiled failed";
     if (q8 ? (!encode_bytes_map(&mk, kc, kv_rows, D, AT_BN) || !encode_bytes_map(&mv, vc, kv_rows, D, AT_BN))
            : (!encode_operand_map(&mk, kc, kv_rows, D, AT_BN) || !encode_operand_map(&mv, vc, kv_rows, D, AT_BN)))
         return "cuTensorMapEncodeTiled failed";
     const float scale_log2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(D)));
+    const int blocks = (slot0 + T - 1) / AT_BN + 1, tiles = (T + AT_BM - 1) / AT_BM;
     int splits = 1;
-    if (T <= AT_BM) {
-        const int blocks = (slot0 + T - 1) / AT_BN + 1;
-        splits = num_sms / nq;                       // CTAs per head that still fit the SMs once
-        if (splits > AT_SPLIT_MAX) splits = AT_SPLIT_MAX;
-        if (splits > blocks / 2) splits = blocks / 2;   // at least two key blocks per CTA
-        if (splits < 1) splits = 1;
+    for (int c = 2, best = (blocks + 1) / 2; c <= AT_SPLIT_MAX && c * nq * tiles <= num_sms; ++c) {
+        const int cost = ((blocks + c - 1) / c + 1) / 2 + 1;
+        if (cost < best) { splits = c; best = cost; }
     }
-    const dim3 grid(nq, (T + AT_BM - 1) / AT_BM, splits);
+    const dim3 grid(nq, tiles, splits);
     if (q8) {
         if (cudaFuncSetAttribute(prefill_attention_tc_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::SMEM_Q8) != cudaSuccess)
             return "cudaFuncSetAttribute failed";
@@ -1780,12 +1809,12 @@ const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *v
         if (cudaFuncSetAttribute(prefill_attention_tc_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::SMEM) != cudaSuccess)
             return "cudaFuncSetAttribute failed";
         launch_pdl(prefill_attention_tc_kernel<D, false>, grid, dim3(AT_THREADS), AttnCfg<D>::SMEM, s, mqh, mql, mk, mv, out, plane, T, slot0, nq,
-                   nq / nkv, max_context, scale_log2, wait_limit, error, static_cast<const float *>(nullptr), static_cast<const float *>(nullptr), part_o,
-                   part_ml);
+                   nq / nkv, max_context, scale_log2, wait_limit, error, static_cast<const float *>(nullptr), static_cast<const float *>(nullptr),
+                   part_o, part_ml);
     }
     if (splits > 1)
-        launch_pdl(prefill_attention_merge_kernel<D>, dim3(T, nq), dim3(D / 4), 0, s, static_cast<const float *>(part_o),
-                   static_cast<const float *>(part_ml), splits, out, plane, nq, scale_log2);
+        launch_pdl(prefill_attention_merge_kernel<D>, dim3((T * nq + 3) / 4), dim3(128), 0, s, static_cast<const float *>(part_o), static_cast<const float2 *>(part_ml),
+                   splits, tiles * AT_BM, out, plane, T, nq, scale_log2);
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill attention launch failed";
 }
 
@@ -1873,7 +1902,7 @@ size_t prefill_buffer_bytes(const edgefm_shape &sh, int chunk) {
     return c * sh.hidden * 4 * (1 + PF_SPLIT_MAX) + c * sh.hidden * 4 + c * PF_SS_PIECES(sh.hidden) * 4 + 2 * c * qd * 4 + c * sh.ffn * 4 + c * (sh.head_dim / 2) * 8 + c * 4 + 256;
 }
 
-cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, bool kv8) {
+cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, bool kv8, int num_sms) {
     const size_t c = static_cast<size_t>(chunk), qd = static_cast<size_t>(sh.n_q_heads) * sh.head_dim;
     cudaError_t e;
     if ((e = cudaMalloc(&b->resid, c * sh.hidden * 4)) != cudaSuccess) return e;
@@ -1889,8 +1918,9 @@ cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, 
     if ((e = cudaMalloc(&b->error, 4)) != cudaSuccess) return e;
     b->logits_rows = sh.vocab;
     if ((e = cudaMalloc(&b->logits, static_cast<size_t>(PF_VERIFY_MAX) * sh.vocab * 4)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&b->att_o, static_cast<size_t>(AT_SPLIT_MAX) * AT_BM * qd * 4)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&b->att_ml, static_cast<size_t>(AT_SPLIT_MAX) * AT_BM * sh.n_q_heads * 2 * 4)) != cudaSuccess) return e;
+    const size_t part_rows = static_cast<size_t>(num_sms) * AT_BM;
+    if ((e = cudaMalloc(&b->att_o, part_rows * sh.head_dim * 4)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->att_ml, part_rows * sizeof(float2))) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->head_val, PF_HEAD_GRID_MAX * PF_VERIFY_MAX * 4)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->head_idx, PF_HEAD_GRID_MAX * PF_VERIFY_MAX * 4)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->head_ticket, 4)) != cudaSuccess) return e;
@@ -1916,7 +1946,10 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
     int count = 0;
     g_pdl = n <= 1024;
     if (cudaMemcpyAsync(b->tokens, tokens, static_cast<size_t>(n) * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) return "token upload failed";
-    launch_pdl(prefill_rope_kernel, dim3((n * (d / 2) + 255) / 256), dim3(256), 0, s, b->rope, n, d / 2, position, static_cast<double>(sh.rope_theta));
+    // The first kernel of a pass is launched the plain way: it starts when everything enqueued before is complete, and so does, whatever overlaps
+    // below, every kernel of the pass.  The contractions read weights before they wait for their predecessors; what an earlier kernel wrote
+    // (weights a caller has changed, the rows of a vocabulary subset) is there by then.
+    prefill_rope_kernel<<<dim3((n * (d / 2) + 255) / 256), dim3(256), 0, s>>>(b->rope, n, d / 2, position, static_cast<double>(sh.rope_theta));
     const int norm_grid = n;
     launch_pdl(prefill_norm_kernel, dim3(norm_grid), dim3(128), 0, s, b->resid, b->xn, x_plane, static_cast<const uint16_t *>(m.layers[0].input_norm),
                                                   static_cast<const uint16_t *>(m.embed), b->tokens, n, H, sh.rms_eps, m.state,

@@ -35,8 +35,8 @@ struct PrefillBuffers {
     float2 *rope = nullptr;      // (cos, sin) of the chunk's positions, [chunk][d/2]
     int *tokens = nullptr;       // device copy of the chunk's token ids
     int *error = nullptr;        // device word: non-zero when a bounded wait of a GEMM ran out
-    float *att_o = nullptr;      // attention of a lone query tile shared out among CTAs: partial rows fp32 [8][128][nq d]
-    float *att_ml = nullptr;     // ... and their (reference maximum, row sum) [8][128][nq][2]
+    float *att_o = nullptr;      // attention whose key blocks are shared out among CTAs: partial rows fp32 [SMs x 128][d]
+    float2 *att_ml = nullptr;    // ... and their (reference maximum, row sum)
     float *logits = nullptr;     // verified blocks: logits of the block's rows when the caller wants none, fp32 [8][vocab]
     int logits_rows = 0;
     float *head_val = nullptr;   // output layer: the CTAs' greedy candidates
@@ -72,7 +72,7 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
 // Bytes the work buffers of a pass over `chunk` tokens take.
 size_t prefill_buffer_bytes(const edgefm_shape &sh, int chunk);
 // Allocate / free.  Returns a CUDA error.
-cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, bool kv8);
+cudaError_t prefill_alloc(PrefillBuffers *b, const edgefm_shape &sh, int chunk, bool kv8, int num_sms);
 void prefill_free(PrefillBuffers *b);
 
 // Enqueue the layers for `n` tokens (host ids) whose cache rows go to slots [slot0, slot0 + n) at rotary positions

@@ -326,15 +326,21 @@ __global__ void __launch_bounds__(256) prefill_quantize_rows_kernel(const float 
 // Output layer for ONE row (the prompt's last token): final RMSNorm, logits = W x over `rows` rows of the output matrix (bf16
 // weights, fp32 x and sums), greedy token (larger value wins, equal values -> lower row), and the device state a decode step
 // would leave.  A matrix-vector product: bound by the one pass over W.  grid: any; 256 threads; dynamic shared memory H floats.
-__global__ void __launch_bounds__(256) prefill_head_kernel(const float *x, const uint16_t *wnorm, const uint16_t *lm, const int *ids, int rows,
+constexpr int HEAD_CTAS_PER_SM = 3;   // 2: 16 warps an SM leave its loads idle between two groups of rows (2.6 TB/s where a row is 1792 bytes long)
+__global__ void __launch_bounds__(256, HEAD_CTAS_PER_SM) prefill_head_kernel(const float *x, const uint16_t *wnorm, const uint16_t *lm, const int *ids, int rows,
                                                            int H, float eps, float *logits_out, int *next_token_out, float *part_val,
                                                            int *part_idx, unsigned *ticket, StepState *st, int token, int pos) {
     extern __shared__ __align__(16) float pf_xs[];
     __shared__ float red[8], bvs[8];
     __shared__ int bis[8], is_last;
+    // four rows per round, two rounds of columns unrolled: 96 KB of loads in flight per SM (two rows, 16 KB: 2.6 TB/s)
+    constexpr int R = 4;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, stride = gridDim.x * 8;
     pdl_trigger();
+    for (int i = 0; i < R; ++i)          // the first round's rows are sent for to L2 while the predecessor still runs (nothing writes weights)
+        if (const int r = blockIdx.x * 8 + warp + i * stride; r < rows)
+            for (int j = lane * 64; j < H; j += 2048) asm volatile("prefetch.global.L2 [%0];" ::"l"(lm + static_cast<size_t>(r) * H + j));
     pdl_wait();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     float ss = 0.f;
     for (int j = tid; j < H; j += 256) ss = fmaf(x[j], x[j], ss);
     ss = warp_sum(ss);
@@ -346,9 +352,6 @@ __global__ void __launch_bounds__(256) prefill_head_kernel(const float *x, const
     __syncthreads();
     float bv = -INFINITY;
     int bi = 0x7fffffff;
-    const int stride = gridDim.x * 8;
-    // four rows per round, two rounds of columns unrolled: 64 KB of loads in flight per SM (two rows, 16 KB: 2.6 TB/s)
-    constexpr int R = 4;
     for (int row = blockIdx.x * 8 + warp; row < rows; row += R * stride) {
         const uint16_t *w[R];
         float a[R];
@@ -2023,7 +2026,7 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
 const char *prefill_head(const PrefillModel &m, PrefillBuffers *b, int row, const void *final_norm, const void *lm, const int *ids, int rows,
                          float *logits_out, int *next_token_out, int token, int pos, cudaStream_t s) {
     const int H = m.shape.hidden;
-    int grid = 2 * m.num_sms;
+    int grid = HEAD_CTAS_PER_SM * m.num_sms;
     if (grid > PF_HEAD_GRID_MAX) grid = PF_HEAD_GRID_MAX;
     if (grid * 8 > rows) grid = (rows + 7) / 8;
     if (H * 4 > 40 * 1024 &&

@@ -1651,11 +1651,9 @@ __global__ void __launch_bounds__(128) prefill_attention_merge_kernel(const floa
     }
 }
 
-// Launch with the programmatic-stream-serialization attribute (see pdl_trigger / pdl_wait) for passes of up to 1024 tokens:
-// there the kernels are short and the launch gaps are 3 - 5 % of a prompt (512 tokens: 4.37 -> 4.17 ms); longer passes lose 1 - 3 %
-// with it (7B shape, 2048 tokens: 44.8 -> 46.5 ms), so they are launched the plain way (the kernels' griddepcontrol
-// instructions are then no-ops).
-thread_local bool g_pdl = false;
+// Launch with the programmatic-stream-serialization attribute (see pdl_trigger / pdl_wait), in clusters of cluster.x CTAs.  Long passes
+// gain, too, where their kernels are short: 1423 tokens, 0.5B shape 4455 -> 4023 us, 2541 tokens 6075 -> 5838; 2048, 1.5B 11205 -> 11065; 4200,
+// 7B, no difference.  (Launched before the tensor memory was allocated the successors cost long passes 1 - 3 %.)
 template <typename... KArgs, typename... Args>
 cudaError_t launch_cluster(dim3 cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
     cudaLaunchConfig_t cfg{};
@@ -1665,10 +1663,8 @@ cudaError_t launch_cluster(dim3 cluster, void (*kernel)(KArgs...), dim3 grid, di
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     int n = 0;
-    if (g_pdl) {
-        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[n++].val.programmaticStreamSerializationAllowed = 1;
-    }
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
     if (cluster.x * cluster.z > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
         attr[n].val.clusterDim.x = cluster.x;
@@ -1947,7 +1943,6 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
     const long long head_stride = static_cast<long long>(m.max_context) * d;
     const size_t cap = static_cast<size_t>(b->chunk), x_plane = cap * H, q_plane = cap * qd, f_plane = cap * F;   // hi / lo planes
     int count = 0;
-    g_pdl = n <= 1024;
     if (cudaMemcpyAsync(b->tokens, tokens, static_cast<size_t>(n) * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) return "token upload failed";
     // The first kernel of a pass is launched the plain way: it starts when everything enqueued before is complete, and so does, whatever overlaps
     // below, every kernel of the pass.  The contractions read weights before they wait for their predecessors; what an earlier kernel wrote

@@ -1142,7 +1142,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
 constexpr int AT_BM = 128, AT_BN = 128;
 constexpr int AT_GROUPS = 2;
 constexpr int AT_SPLIT_MAX = 16; // CTAs that share the key blocks of a query tile
-constexpr int AT_CW = 4;       // compressed cache: warps that expand the codes (AT_BN / AT_CW rows of a tile each)
+constexpr int AT_CW = 8;       // compressed cache: warps that expand the codes (AT_BN / AT_CW rows of a tile each); with four of them, which
+                               // fetched the scales behind the codes, 1000 tokens of the 3B shape took 12322 us instead of 12123
 constexpr int AT_THREADS = 96 + 128 * AT_GROUPS;   // producer, two issuers, softmax warps
 
 // B operand in MN-major form for P V: the V tile is D/64 blocks of [64 keys][64 d] (128-byte rows, 128-byte swizzle).  N (= d)
@@ -1393,14 +1394,22 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
         };
         auto expand_k = [&](int j) {
             const int st = j & 1;
+            // the scales of this block's keys (both kinds: they are in memory already), asked for before the codes are awaited: behind them
+            // they put a trip to memory into every block
+            static_assert(ROWS <= 32, "a lane per row");
+            float ks = 0.f, vs = 0.f;
+            if (lane < ROWS) {
+                const size_t key = static_cast<size_t>(hk) * max_context + min((j0 + j) * AT_BN + cw * ROWS + lane, last_key);
+                ks = k_scale[key];
+                vs = v_scale[key];
+            }
             if (!(warp_wait(&kraw_full, j & 1) && (j < 2 || warp_wait(&k_empty[st], ((j >> 1) - 1) & 1)))) return false;   // the codes are here, the operand tile is free
             expand_tile(skv + st * (C::K_BYTES + C::V_BYTES), sraw);
             __syncwarp();
             if (lane == 0) mbar_arrive(&kraw_empty);       // the next K tile may land
-            for (int i = lane; i < ROWS; i += 32) {        // the scales of this block's keys (both kinds: they are in memory already)
-                const int key = min((j0 + j) * AT_BN + cw * ROWS + i, last_key);
-                sc_k[j & 3][cw * ROWS + i] = k_scale[static_cast<size_t>(hk) * max_context + key];
-                sc_v[j & 3][cw * ROWS + i] = v_scale[static_cast<size_t>(hk) * max_context + key];
+            if (lane < ROWS) {
+                sc_k[j & 3][cw * ROWS + lane] = ks;
+                sc_v[j & 3][cw * ROWS + lane] = vs;
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();

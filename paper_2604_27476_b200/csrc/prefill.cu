@@ -1718,7 +1718,7 @@ const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const 
 }
 
 template <int EPI, int BN, bool SWAP>
-const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, GemmArgs &g, cudaStream_t s) {
+const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, GemmArgs &g, int num_sms, cudaStream_t s) {
     const int n_step = EPI == EPI_SWIGLU ? BN / 2 : BN, tiles = ((g.N + n_step - 1) / n_step) * ((g.M + PF_BM - 1) / PF_BM);
     const int a_bytes = g.a_rows * PF_BK * 2, stage = 2 * a_bytes + BN * PF_BK * 2;
     const int kb = ((g.K + PF_BK - 1) / PF_BK + g.cluster - 1) / g.cluster;      // of the CTA with the most
@@ -1726,7 +1726,7 @@ const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUte
     // last stage for those that are not loaded
     const int reach = (SWAP ? 2 : 1) * a_bytes + PF_BM * PF_BK * 2, slack = reach > stage ? reach - stage : 0;
     g.stages = (TILE_SMEM - 1024 - slack) / stage;
-    if (kb > 2 * g.stages) g.stages = (TILE_SMEM_DEEP - 1024 - slack) / stage;
+    if (kb > 2 * g.stages && tiles * g.cluster <= num_sms) g.stages = (TILE_SMEM_DEEP - 1024 - slack) / stage;
     if (g.stages > TILE_STAGES_MAX) g.stages = TILE_STAGES_MAX;
     if (g.stages > kb) g.stages = kb;
     const int ring = g.stages * stage + slack, partial = g.a_rows * BN * 4;
@@ -1759,10 +1759,10 @@ const char *launch_gemm(const uint16_t *a, size_t a_plane, const void *w, long l
     if constexpr (EPI != EPI_LOGITS)
         if (g.cluster) {
             if constexpr (EPI != EPI_SWIGLU) {
-                if (plan.columns == 256) return launch_tile<EPI, 256, false>(ma, ml, mb, g, s);
-                if (plan.columns == 64) return plan.swap ? launch_tile<EPI, 64, true>(ma, ml, mb, g, s) : launch_tile<EPI, 64, false>(ma, ml, mb, g, s);
+                if (plan.columns == 256) return launch_tile<EPI, 256, false>(ma, ml, mb, g, num_sms, s);
+                if (plan.columns == 64) return plan.swap ? launch_tile<EPI, 64, true>(ma, ml, mb, g, num_sms, s) : launch_tile<EPI, 64, false>(ma, ml, mb, g, num_sms, s);
             }
-            return plan.swap ? launch_tile<EPI, 128, true>(ma, ml, mb, g, s) : launch_tile<EPI, 128, false>(ma, ml, mb, g, s);
+            return plan.swap ? launch_tile<EPI, 128, true>(ma, ml, mb, g, num_sms, s) : launch_tile<EPI, 128, false>(ma, ml, mb, g, num_sms, s);
         }
     const int m_tiles = (g.M + PF_BM - 1) / PF_BM;
     if constexpr (EPI != EPI_SWIGLU)
@@ -1884,6 +1884,13 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
         }
         p.splits = 1;
         return p;
+    }
+    // Gate/up of one row tile with more tiles than SMs: 64 + 64 columns, two CTAs per SM.  A pass over so many weights is bound by what an SM
+    // asks for from memory at a time, and the persistent kernel's stages of 64 KB are half activations (64 tokens, 7B shape: 63 us for 271 MB;
+    // the prompt 4355 -> 4185 us so).
+    if (epilogue == EPI_SWIGLU && m_tiles == 1 && (N + 63) / 64 <= 2 * num_sms) {
+        const int rows = M < PF_BM ? (M + 7) & ~7 : PF_BM;
+        return PrefillPlan{128, 1, 1, false, rows < PF_BM};
     }
     // Pairs of CTAs where they need no more rounds over the SMs (an odd number of row tiles leaves one CTA of a pair without work).
     const int workers = num_sms / 2, m_pairs = (m_tiles + 1) / 2;

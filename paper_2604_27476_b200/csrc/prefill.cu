@@ -1102,9 +1102,13 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
         const int rc = min(r, r1 - 1);
         const uint32_t off = base + rc * BN * 4, pa = off + ((ca / 4 + c8) ^ (rc & 7)) * 16, pb = off + ((cb / 4 + c8) ^ (rc & 7)) * 16;
         float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
+        if (S == 1) {
+            va = *reinterpret_cast<const float4 *>(tiles + (pa - base));
+            vb = *reinterpret_cast<const float4 *>(tiles + (pb - base));
+        }
 #pragma unroll 4
-        for (int q = 0; q < S; ++q) {        // in the order of K
-            const float4 x = cluster_ld4(S > 1 ? cluster_addr(pa, q) : pa), y = cluster_ld4(S > 1 ? cluster_addr(pb, q) : pb);
+        for (int q = 0; q < S && S > 1; ++q) {        // in the order of K
+            const float4 x = cluster_ld4(cluster_addr(pa, q)), y = cluster_ld4(cluster_addr(pb, q));
             va.x += x.x; va.y += x.y; va.z += x.z; va.w += x.w;
             vb.x += y.x; vb.y += y.y; vb.z += y.z; vb.w += y.w;
         }

@@ -931,8 +931,9 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
 //     this kernel's end; twice that where it has many (two stages of 48 KB: 27 us for 35 k-blocks, 1.8 MB, of a down projection);
 //   * an activation tile is loaded without its idle rows (a multiple of 8; the multiplies read whatever lies behind it, for rows nobody
 //     looks at);
-//   * SWAP, where the tokens (padded to 8) are fewer than the tile's columns: the weights are the 128 rows of the multiply and the tokens its
-//     columns, hi and lo pieces side by side, so that four multiplies of 2 x tokens columns take the place of eight of the tile's width
+//   * SWAP, up to 256 tokens: the weights are the 128 rows of the multiply and the tokens its columns.  Two row tiles then share one weight
+//     tile, and idle rows cost nothing.  Where the tokens (padded to 8) are fewer than the tile's columns the hi and lo pieces lie side by
+//     side, so that four multiplies of 2 x tokens columns take the place of eight of the tile's width
 //     over 128 rows (which for 9 tokens, 1.5B shape, are 6.3 us of multiplies in a gate/up tile, by arithmetic: more than its weights take).
 constexpr int TILE_STAGES_MAX = 8, TILE_THREADS = 256, TILE_SMEM = 110 * 1024, TILE_SMEM_DEEP = 220 * 1024, TILE_AHEAD = 32;
 
@@ -954,19 +955,20 @@ template <int EPI, int BN, bool SWAP>
 __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __grid_constant__ CUtensorMap map_a_hi,
                                                                        const __grid_constant__ CUtensorMap map_a_lo,
                                                                        const __grid_constant__ CUtensorMap map_b, const GemmArgs g) {
+    constexpr int ROWS = SWAP ? 2 * PF_BM : PF_BM;       // of a tile at most
     constexpr int N_STEP = EPI == EPI_SWIGLU ? BN / 2 : BN, B_PARTS = EPI == EPI_SWIGLU || BN == 256 ? 2 : 1, CHUNKS = BN / 64;
     extern __shared__ uint8_t pf_dyn[];
     __shared__ uint64_t full_bar[TILE_STAGES_MAX], empty_bar[TILE_STAGES_MAX], acc_full, drain_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ float rs_sm[PF_BM];
+    __shared__ float rs_sm[ROWS];
     uint8_t *tiles = pf_dyn + ((1024u - (smem_u32(pf_dyn) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = g.cluster, tile = blockIdx.x / S, rank = blockIdx.x - tile * S, KB = (g.K + PF_BK - 1) / PF_BK;
-    const int m_tiles = (g.M + PF_BM - 1) / PF_BM, n_tile = tile / m_tiles, m0 = (tile - n_tile * m_tiles) * PF_BM, n0 = n_tile * N_STEP;
+    const int m_tiles = (g.M + ROWS - 1) / ROWS, n_tile = tile / m_tiles, m0 = (tile - n_tile * m_tiles) * ROWS, n0 = n_tile * N_STEP;
     const int kb0 = rank * KB / S, nkb = (rank + 1) * KB / S - kb0;
     const int a_bytes = g.a_rows * PF_BK * 2, stage_bytes = 2 * a_bytes + BN * PF_BK * 2;
-    const int live = min(PF_BM, g.M - m0), r0 = rank * live / S, r1 = (rank + 1) * live / S;   // rows of the tile; those this CTA finishes
+    const int live = min(ROWS, g.M - m0), r0 = rank * live / S, r1 = (rank + 1) * live / S;   // rows of the tile; those this CTA finishes
 
     if (threadIdx.x == 0) {
         prefetch_map(&map_b); prefetch_map(&map_a_hi); prefetch_map(&map_a_lo);
@@ -1028,7 +1030,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
         }
     } else if (warp == 1 && lane == 0) {     // issuer
         pdl_wait();
-        const uint32_t idesc = umma_idesc_bf16(PF_BM, SWAP ? 2 * g.a_rows : BN);
+        const bool side = 2 * g.a_rows <= 256;            // SWAP: hi and lo columns side by side (more do not fit one multiply)
+        const uint32_t idesc = umma_idesc_bf16(PF_BM, !SWAP ? BN : side ? 2 * g.a_rows : g.a_rows);
         bool ok = true;
 #pragma unroll 1
         for (int it = 0, s = 0, phase = 0; it < nkb; ++it) {
@@ -1040,6 +1043,11 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
             if constexpr (SWAP) {            // (the lo rows lie right behind the hi rows)
 #pragma unroll
                 for (int k = 0; k < PF_BK / 16; ++k) umma_bf16(tmem, db + 2 * k, da + 2 * k, idesc, (it | k) != 0);
+                if (!side) {
+                    const uint64_t dl = umma_desc_sw128(a + a_bytes);
+#pragma unroll
+                    for (int k = 0; k < PF_BK / 16; ++k) umma_bf16(tmem, db + 2 * k, dl + 2 * k, idesc, 1);
+                }
             } else {
                 const uint64_t dl = umma_desc_sw128(a + a_bytes);
 #pragma unroll
@@ -1086,7 +1094,12 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
                         for (int t0 = 0; t0 < live; t0 += 32) {
                             float hi[32], lo[32];
                             tmem_ld32(trow + t0, hi);
-                            tmem_ld32(trow + g.a_rows + t0, lo);
+                            if (2 * g.a_rows <= 256) {
+                                tmem_ld32(trow + g.a_rows + t0, lo);
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < 32; ++i) lo[i] = 0.f;
+                            }
                             tmem_ld_wait();
 #pragma unroll
                             for (int i = 0; i < 32; ++i)
@@ -1712,8 +1725,20 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     return launch_cluster(dim3(1), kernel, grid, block, smem, stream, static_cast<KArgs>(args)...);
 }
 
-// Clusters of c CTAs, one CTA per SM, that run at once: a cluster stays within a GPC of (about) 18 SMs.
-int clusters_at_once(int c, int num_sms) { return num_sms / 18 * (18 / c) + num_sms % 18 / c; }
+// Clusters of c CTAs, one CTA per SM, that run at once: a cluster stays within a GPC.  Of 148 SMs, as cudaOccupancyMaxActiveClusters has it on a B200;
+// one tile more than that is a second round (1.5B shape, 152 tokens: O and down as 24 clusters of six took 14 us a layer more than 12 of eight).
+int clusters_at_once(int c, int num_sms) {
+    constexpr int AT_148[PF_CLUSTER_MAX + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    return AT_148[c] * num_sms / 148;
+}
+// The same for a contraction's clusters of c: with few k-blocks each its CTAs take half an SM's shared memory, and any that are no more than the SMs fit.
+int tiles_at_once(int c, int kb, int rows, int bn, int num_sms) {
+    const int stages = (TILE_SMEM - 1024) / (rows * PF_BK * 4 + bn * PF_BK * 2), one = clusters_at_once(c, num_sms);
+    return (kb + c - 1) / c > 2 * stages ? one : num_sms / c < 2 * one ? num_sms / c : 2 * one;
+}
+
+// Rows of an activation tile that are loaded, up to 256 tokens: whole groups of 8, of 16 where the pieces are multiplied one after the other.
+int swapped_rows(int M) { return M <= PF_BM ? (M + 7) & ~7 : (M + 15) & ~15; }
 
 // ---- host side ---------------------------------------------------------------------------------------------------------------
 // Map of a row-major bf16 [rows][K] matrix; a box is box_rows rows x 64 columns (one 128-byte swizzled row each); rows and
@@ -1741,7 +1766,7 @@ const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const 
 
 template <int EPI, int BN, bool SWAP>
 const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, GemmArgs &g, int num_sms, cudaStream_t s) {
-    const int n_step = EPI == EPI_SWIGLU ? BN / 2 : BN, tiles = ((g.N + n_step - 1) / n_step) * ((g.M + PF_BM - 1) / PF_BM);
+    const int n_step = EPI == EPI_SWIGLU ? BN / 2 : BN, tiles = ((g.N + n_step - 1) / n_step) * (SWAP ? 1 : (g.M + PF_BM - 1) / PF_BM);
     const int a_bytes = g.a_rows * PF_BK * 2, stage = 2 * a_bytes + BN * PF_BK * 2;
     const int kb = ((g.K + PF_BK - 1) / PF_BK + g.cluster - 1) / g.cluster;      // of the CTA with the most
     // the multiplies read 128 rows of the operand that has 128, from the start of either piece or (swapped) of the weights: room behind the
@@ -1753,8 +1778,8 @@ const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUte
     if (g.stages > kb) g.stages = kb;
     const int ring = g.stages * stage + slack, partial = g.a_rows * BN * 4;
     const int smem = 1024 + (ring > partial ? ring : partial);
-    // swapped: the pieces' columns are read 32 at a time
-    const int cols = SWAP ? g.a_rows + (g.a_rows + 31) / 32 * 32 : BN;
+    // swapped: the pieces' columns (side by side where they fit one multiply) are read 32 at a time
+    const int cols = SWAP ? (2 * g.a_rows <= 256 ? g.a_rows : 0) + (g.a_rows + 31) / 32 * 32 : BN;
     for (g.tmem_cols = 32; g.tmem_cols < cols;) g.tmem_cols *= 2;
     if (cudaFuncSetAttribute(prefill_tile_kernel<EPI, BN, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM_DEEP) != cudaSuccess)
         return "cudaFuncSetAttribute failed";
@@ -1769,7 +1794,7 @@ const char *launch_gemm(const uint16_t *a, size_t a_plane, const void *w, long l
     g.cluster = plan.cluster;
     g.splits = plan.splits;
     g.bn = plan.columns;
-    g.a_rows = g.cluster && g.M < PF_BM ? (g.M + 7) & ~7 : PF_BM;
+    g.a_rows = g.cluster && (g.M < PF_BM || plan.swap) ? swapped_rows(g.M) : PF_BM;
     const int b_rows = EPI == EPI_SWIGLU ? (plan.columns == 128 ? 64 : 128) : plan.pairs ? plan.columns / 2 : plan.columns < 128 ? plan.columns : 128;
     if (!encode_operand_map(&ma, a, g.M, g.K, g.a_rows) || !encode_operand_map(&ml, a + a_plane, g.M, g.K, g.a_rows) ||
         !encode_operand_map(&mb, w, w_rows, g.K, b_rows))
@@ -1888,6 +1913,17 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
     PrefillPlan p{shape == PF_WIDE ? 256 : shape == PF_SLIM ? 64 : 128, splits, 0, false, false};
     const int n_step = epilogue == EPI_SWIGLU ? p.columns / 2 : p.columns, tiles = m_tiles * ((N + n_step - 1) / n_step);
     if (epilogue == EPI_LOGITS) return p;
+    // 129 to 256 tokens: the tokens as the columns of one row of tiles (gate/up: 64 + 64 columns), if these fit the SMs once and no other tiles that do
+    // are cheaper.
+    PrefillPlan wide_swap{128, 1, 0, false, true};
+    int wide_swap_cost = 1 << 30;
+    if (m_tiles == 2) {
+        const int steps = (N + (epilogue == EPI_SWIGLU ? 63 : 127)) / (epilogue == EPI_SWIGLU ? 64 : 128), block = 4 * swapped_rows(M) + 2 * 128;
+        for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && steps <= tiles_at_once(c, kb, swapped_rows(M), 128, num_sms); ++c) {
+            const int cost = (kb + c - 1) / c * block + (c > 1 ? 2000 : 0);
+            if (cost < wide_swap_cost) { wide_swap.cluster = c; wide_swap_cost = cost; }
+        }
+    }
     // Clusters where the tiles fit the SMs in one round.  A k-block costs a CTA what its operands take at 64 bytes per cycle, or its multiplies:
     // 4 cycles per column over 128 rows, or (swapped, the weights are the rows) 4 per token; sharing a tile's K costs the exchange of the
     // partial tiles, about 2000 cycles.  Tiles of 256 columns halve the traffic of several row tiles' activations.
@@ -1897,7 +1933,7 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
         int best = 1 << 30;
         for (int bn = base; bn <= (epilogue == EPI_SWIGLU || m_tiles == 1 ? base : 256); bn *= 2) {
             const int t = m_tiles * ((N + bn - 1) / bn), step = epilogue == EPI_SWIGLU ? tiles : t;
-            for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && (c == 1 ? step <= num_sms : step <= clusters_at_once(c, num_sms)); ++c) {
+            for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && step <= tiles_at_once(c, kb, rows, bn, num_sms); ++c) {
                 const bool swap = rows < bn && bn <= 128 && rows < PF_BM;
                 const int multiplies = 4 * (swap ? (rows > 32 ? rows : 32) : bn), operands = 4 * rows + 2 * bn;
                 const int cost = (kb + c - 1) / c * (multiplies > operands ? multiplies : operands) + (c > 1 ? 2000 : 0);
@@ -1905,8 +1941,9 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
             }
         }
         p.splits = 1;
-        return p;
+        return wide_swap_cost < best ? wide_swap : p;
     }
+    if (wide_swap.cluster) return wide_swap;
     // Gate/up of one row tile with more tiles than SMs: 64 + 64 columns, two CTAs per SM.  A pass over so many weights is bound by what an SM
     // asks for from memory at a time, and the persistent kernel's stages of 64 KB are half activations (64 tokens, 7B shape: 63 us for 271 MB;
     // the prompt 4355 -> 4185 us so).

@@ -19,6 +19,11 @@ CASES = {
     "three_row_tiles_one_row": (dict(hidden=264, ffn=520), 0, 257),
     "odd_head_in_a_tile_of_two": (dict(n_q_heads=5, n_kv_heads=1, ffn=200), 0, 140),
     "heads_of_128_by_clusters": (dict(hidden=1152, n_q_heads=6, n_kv_heads=2, head_dim=128, ffn=1032, n_layers=1, vocab=300), 40, 61),
+    # two row tiles as the columns of one row of tiles: one token into the second, a ragged group of 16, all of it, one token too many
+    "two_row_tiles_first": (dict(hidden=1024, ffn=4096, n_layers=1, vocab=300), 0, 129),
+    "two_row_tiles_ragged": (dict(hidden=1152, n_q_heads=6, n_kv_heads=2, head_dim=128, ffn=1032, n_layers=1, vocab=300), 5, 201),
+    "two_row_tiles_full": (dict(hidden=264, ffn=520), 0, 256),
+    "two_row_tiles_one_k_tile": (dict(hidden=64, n_q_heads=1, n_kv_heads=1, ffn=72, vocab=40), 0, 250),
     # the persistent kernel, row tiles in pairs: an even number, an odd one, a last tile of one row
     "pairs_even": (dict(ffn=9480, n_layers=1, vocab=500), 0, 256),
     "pairs_odd": (dict(ffn=9480, n_layers=1, vocab=500), 3, 300),

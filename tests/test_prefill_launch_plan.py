@@ -14,7 +14,7 @@ def tiles(M, N, columns):
 
 def test_launches():
     ops = [op for name in CONFIGS for op in shapes(CONFIGS[name]).values()] + list(ODD.values())
-    for (epi, N, K), M, sms in itertools.product(ops, (1, 8, 15, 64, 77, 121, 128, 129, 257, 384, 1000, 2048, 4096), (148, 132, 20)):
+    for (epi, N, K), M, sms in itertools.product(ops, (1, 8, 15, 64, 77, 121, 128, 129, 256, 257, 384, 1000, 2048, 4096), (148, 132, 20)):
         columns, splits, cluster, pairs, swapped = edgefm_debug_prefill_launch(epi, M, N, K, sms)
         step, kb = (columns // 2 if epi == SWIGLU else columns), -(-K // 64)
         what = (epi, M, N, K, sms)
@@ -22,14 +22,14 @@ def test_launches():
         if cluster:
             assert splits == 1 and not pairs and columns in (64, 128, 256), what
             assert 1 <= cluster <= min(8, kb), what                           # no CTA without a k-block
-            assert tiles(M, N, step) * cluster <= sms or (epi == SWIGLU and M <= 128 and cluster == 1 and tiles(M, N, step) <= 2 * sms), what   # one or two CTAs per SM
+            assert tiles(min(M, 128) if swapped else M, N, step) * cluster <= sms or (epi == SWIGLU and M <= 128 and cluster == 1 and tiles(M, N, step) <= 2 * sms), what   # one or two CTAs per SM
         else:
             assert columns in (128, 256) or (pairs and epi == RESID), what
             assert 1 <= splits <= 8 and (splits == 1 or epi == RESID), what
         if pairs:
             assert M > 128 and columns >= 128, what
-        if swapped:                                                           # fewer padded tokens than columns, both pieces side by side
-            assert cluster and M < 128 and -(-M // 8) * 8 < columns <= 128, what
+        if swapped:                    # fewer padded tokens than columns, both pieces side by side; or two row tiles that share weight tiles
+            assert cluster and columns <= 128 and (-(-M // 8) * 8 < columns if M < 128 else 128 < M <= 256), what
         if epi == QKV:
             assert columns % 128 == 0, what                                   # whole heads of 128
         if epi == SWIGLU:

@@ -295,11 +295,11 @@ edgefm_status edgefm_debug_plan(const edgefm_ctx *ctx, int32_t *out8);
  * next step runs into the bound.  Synchronises the device. */
 edgefm_status edgefm_debug_set_wait_limit(edgefm_ctx *ctx, uint32_t limit_ns, int32_t extra_barrier_arrivals);
 
-/* The same for the contractions of edgefm_prefill: every wait on a shared-memory barrier gives up after `polls` polls
+/* The same for the contractions and the attention of edgefm_prefill: every wait on a shared-memory barrier gives up after `polls` polls
  * (2^24 by default; >= 1024), raises an error word that edgefm_sync_status reports as EDGEFM_ERR_TIMEOUT, waits (bounded) for
  * its own copies and multiplies in flight, frees its tensor memory and returns.  extra_arrivals = 1 (0 in production) makes
- * the stage barriers expect an arrival nobody makes, so that the first wait of every contraction enqueued afterwards runs
- * into the bound without any fault.  Host only. */
+ * the stage barriers (attention: the queries' barrier) expect an arrival nobody makes, so that the first wait of every such kernel
+ * enqueued afterwards runs into the bound without any fault.  Host only. */
 edgefm_status edgefm_debug_set_prefill_wait(edgefm_ctx *ctx, uint32_t polls, int32_t extra_arrivals);
 
 /* The first stage of the plan of a contraction of [M tokens x K] x [K x N] of edgefm_prefill on num_sms SMs: out2 = {output tile: 0 = 128

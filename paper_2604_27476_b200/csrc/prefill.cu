@@ -58,6 +58,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     *abort_flag = 1;
     return false;
 }
+// A CTA that gives up waits for what it has under way (copies into its shared memory, multiplies), in the end with a bound of its own.
+constexpr uint32_t PF_LAND_POLLS = 1u << 24;
+__device__ __forceinline__ void mbar_land(uint64_t *bar, uint32_t parity) {
+    int given_up = 0;
+    mbar_wait(bar, parity, &given_up, PF_LAND_POLLS);
+}
+// The copies of a ring: `issued` stages were asked for, the last `stages` of them may be on their way.  To be called behind a barrier that every
+// wait of the CTA precedes: a producer that has sent for everything is done long before another thread's wait runs out.  extra_arrivals: the
+// arrivals that nobody else makes (GemmArgs).
+__device__ __forceinline__ void ring_land(uint64_t *full_bar, int issued, int stages, uint32_t extra_arrivals) {
+#pragma unroll 1
+    for (int j = issued > stages ? issued - stages : 0; j < issued; ++j) {
+        uint64_t *bar = full_bar + j % stages;
+        for (uint32_t e = 0; e < extra_arrivals; ++e) mbar_arrive(bar);
+        mbar_land(bar, (j / stages) & 1);
+    }
+}
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
@@ -723,7 +740,7 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
     extern __shared__ uint8_t pf_dyn[];
     __shared__ uint64_t full_bar[C::STAGES], empty_bar[C::STAGES], acc_full[2], acc_empty[2], drain_bar;
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, issued_sm;        // issued_sm: stages this CTA's producer has sent for
     uint8_t *tiles = pf_dyn + ((1024u - (smem_u32(pf_dyn) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = PAIR ? blockIdx.x & 1 : 0, worker = blockIdx.x / CTAS, workers = gridDim.x / CTAS;
@@ -808,16 +825,11 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
             issued = it + 1;
           }
         }
-        if (abort_flag) {   // giving up: the copies still in flight must land before the CTA's shared memory is released
-            int dummy = 0;
-            if (rank == 0)
-                for (int j = issued > C::STAGES ? issued - C::STAGES : 0; j < issued; ++j)
-                    mbar_wait(&full_bar[j % C::STAGES], (j / C::STAGES) & 1, &dummy, g.wait_limit);
-            // a pair's copies are counted by the first CTA, which may have given up before it expected all of them: they land within
-            // microseconds, the pair leaves together 0.2 ms later
-            if (PAIR)
-                for (const long long t0 = clock64(); clock64() - t0 < 400000;) { }
-        }
+        issued_sm = issued;
+        // a pair's copies are counted by the first CTA, which may have given up before it expected all of them: they land within
+        // microseconds, the pair leaves together 0.2 ms later
+        if (PAIR && abort_flag)
+            for (const long long t0 = clock64(); clock64() - t0 < 400000;) { }
     } else if (warp == 1 && lane == 0) {     // issuer (of a pair, the first CTA's): per stage 4 tcgen05.mma (K = 16 each) for the hi pieces, 4 for the lo pieces
         const uint32_t idesc = umma_idesc_bf16(TILE_M, BN);
         auto mma = [&](uint32_t acc, uint64_t da, uint64_t db, uint32_t accumulate) {
@@ -850,9 +862,8 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
           if (ok) commit(&acc_full[buf]);
         }
         if (!ok) {          // giving up: the multiplies already issued must finish before the tensor memory is freed
-            int dummy = 0;
             commit(&drain_bar);
-            mbar_wait(&drain_bar, 0, &dummy, g.wait_limit);
+            mbar_land(&drain_bar, 0);
         }
     } else if (warp >= 2) {                  // epilogue: warp w may read lanes 32 (w % 4) .. + 31 of tensor memory
       const int quarter = warp & 3, sub = lane >> 3, c8 = lane & 7;
@@ -916,7 +927,10 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
         if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C::BN) : "memory");
         else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C::BN) : "memory");
     }
-    if (threadIdx.x == 0 && abort_flag) atomicExch(g.error, 1);
+    if (threadIdx.x == 0 && abort_flag) {        // the CTA's shared memory is released when this thread leaves
+        if (rank == 0) ring_land(full_bar, issued_sm, C::STAGES, g.extra_arrivals);
+        atomicExch(g.error, 1);
+    }
 }
 
 // The same contraction where the tiles fit the SMs in one round (short prompts): a cluster of g.cluster CTAs shares the K of one output
@@ -960,7 +974,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
     extern __shared__ uint8_t pf_dyn[];
     __shared__ uint64_t full_bar[TILE_STAGES_MAX], empty_bar[TILE_STAGES_MAX], acc_full, drain_bar;
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, issued_sm;
     __shared__ float rs_sm[ROWS];
     uint8_t *tiles = pf_dyn + ((1024u - (smem_u32(pf_dyn) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1022,12 +1036,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
             load_a(it, s);
             if (++s == g.stages) { s = 0; phase ^= 1; }
         }
-        if (abort_flag) {   // giving up: the copies still in flight must land before the shared memory is used again or released
-            int dummy = 0;
-#pragma unroll 1
-            for (int j = it > g.stages ? it - g.stages : 0; j < it; ++j)
-                mbar_wait(&full_bar[j % g.stages], (j / g.stages) & 1, &dummy, g.wait_limit);
-        }
+        issued_sm = it;
     } else if (warp == 1 && lane == 0) {     // issuer
         pdl_wait();
         const bool side = 2 * g.a_rows <= 256;            // SWAP: hi and lo columns side by side (more do not fit one multiply)
@@ -1059,10 +1068,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
             if (++s == g.stages) { s = 0; phase ^= 1; }
         }
         umma_commit(ok ? &acc_full : &drain_bar);
-        if (!ok) {          // giving up: the multiplies already issued must finish before the tensor memory is freed
-            int dummy = 0;
-            mbar_wait(&drain_bar, 0, &dummy, g.wait_limit);
-        }
+        if (!ok) mbar_land(&drain_bar, 0);   // giving up: the multiplies already issued must finish before the tensor memory is freed
     }
     __syncwarp();
     pdl_wait();
@@ -1154,7 +1160,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.tmem_cols) : "memory");
     }
-    if (threadIdx.x == 0 && abort_flag) atomicExch(g.error, 1);
+    if (threadIdx.x == 0 && abort_flag) {    // (a CTA that has given up writes no partial tile over its ring)
+        ring_land(full_bar, issued_sm, g.stages, g.extra_arrivals);
+        atomicExch(g.error, 1);
+    }
     if (S > 1) cluster_wait();
 }
 
@@ -1209,8 +1218,8 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
                                                                    const __grid_constant__ CUtensorMap map_k,
                                                                    const __grid_constant__ CUtensorMap map_v, uint16_t *out, size_t plane,
                                                                    int T, int slot0, int nq, int group, int max_context,
-                                                                   float scale_log2, uint32_t wait_limit, int *error, const float *k_scale,
-                                                                   const float *v_scale, float *part_o, float2 *part_ml) {
+                                                                   float scale_log2, uint32_t wait_limit, uint32_t extra_arrivals, int *error,
+                                                                   const float *k_scale, const float *v_scale, float *part_o, float2 *part_ml) {
     // Q8: the cache holds 8-bit codes and a scale per row (k_scale, v_scale: this layer's [nkv][max_context]); map_k / map_v then
     // describe byte matrices; two more warps expand the codes to bf16 (exactly) into the operand layout, the softmax multiplies
     // the scores by the keys' scales and folds the values' scales into the probabilities.
@@ -1220,7 +1229,7 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
     __shared__ __align__(16) float sc_k[Q8 ? 4 : 1][AT_BN], sc_v[Q8 ? 4 : 1][AT_BN];   // scales of the last four key blocks
     __shared__ uint64_t q_full, k_full[2], k_empty[2], v_full[2], v_empty[2], s_full[2], p_full[2][2], pv_done[2], all_done, drain_bar[2];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, issued_k, issued_v;  // key blocks whose K, V the producer has sent for
     __shared__ float2 row_ml[AT_GROUPS][AT_BM];     // reference maximum and sum of every row, at the end
     uint8_t *base = at_tc_dyn + ((1024u - (smem_u32(at_tc_dyn) & 1023u)) & 1023u);
     uint8_t *sq = base, *skv = sq + C::Q_BYTES, *sraw = skv + 2 * (C::K_BYTES + C::V_BYTES);   // sraw: landing areas of the codes (Q8)
@@ -1237,7 +1246,7 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
 
     if (threadIdx.x == 0) {
         prefetch_map(&map_q_hi); prefetch_map(&map_q_lo); prefetch_map(&map_k); prefetch_map(&map_v);
-        mbar_init(&q_full, 1);
+        mbar_init(&q_full, 1 + extra_arrivals);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&k_full[i], Q8 ? AT_CW : 1); mbar_init(&k_empty[i], 1); mbar_init(&v_full[i], Q8 ? AT_CW : 1); mbar_init(&v_empty[i], 1);
             mbar_init(&vraw_full[i], 1); mbar_init(&s_full[i], 1); mbar_init(&pv_done[i], 1); mbar_init(&drain_bar[i], 1);
@@ -1312,16 +1321,8 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
             if (j + 1 < nb) ok = load_k(j + 1);
             if (ok) ok = load_v(j);
         }
-        if (abort_flag) {   // giving up: the copies in flight must land before the shared memory is released
-            int dummy = 0;
-            if (nb > 0) mbar_wait(&q_full, 0, &dummy, wait_limit);
-            if (Q8) { if (nk > 0) mbar_wait(&kraw_full, (nk - 1) & 1, &dummy, wait_limit); }
-            else
-#pragma unroll 1
-            for (int j = nk > 2 ? nk - 2 : 0; j < nk; ++j) mbar_wait(&k_full[j & 1], (j >> 1) & 1, &dummy, wait_limit);
-#pragma unroll 1
-            for (int j = nv > 2 ? nv - 2 : 0; j < nv; ++j) mbar_wait(Q8 ? &vraw_full[j & 1] : &v_full[j & 1], (j >> 1) & 1, &dummy, wait_limit);
-        }
+        issued_k = nk;
+        issued_v = nv;
     } else if (warp == 1 && lane == 0) {     // issuer of the scores: S_j = Q K_j^T, hi pieces then lo pieces
         // (two issuing threads, scores here and P V in warp 2: a tcgen05.mma takes about 40 ns to issue, and one thread issuing
         // both, with its six waits per block, was what bounded the kernel: 2.3 us per block)
@@ -1348,9 +1349,8 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
             umma_commit(&k_empty[g]);        // the K rows are free when these have read them
         }
         if (!ok) {
-            int dummy = 0;
             umma_commit(&drain_bar[0]);
-            mbar_wait(&drain_bar[0], 0, &dummy, wait_limit);
+            mbar_land(&drain_bar[0], 0);
         }
     } else if (warp == 2 && lane == 0) {     // issuer of O += P_j V_j, the block's two halves of 64 keys as they come
         constexpr uint32_t idesc_o = umma_idesc_bf16(AT_BM, D) | (1u << 16);   // B (= V) is MN-major
@@ -1379,9 +1379,8 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
         if (ok) {
             umma_commit(&all_done);
         } else {
-            int dummy = 0;
             umma_commit(&drain_bar[1]);
-            mbar_wait(&drain_bar[1], 0, &dummy, wait_limit);
+            mbar_land(&drain_bar[1], 0);
         }
     }
     else if (Q8 && warp >= AT_THREADS / 32) {   // compressed cache: expand the 8-bit tiles to bf16 operand tiles (AT_CW warps, AT_BN / AT_CW rows each)
@@ -1653,7 +1652,20 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(AttnCfg<D>::TMEM_COLS) : "memory");
     }
-    if (threadIdx.x == 0 && abort_flag) atomicExch(error, 1);
+    if (threadIdx.x == 0 && abort_flag) {    // the copies in flight land before this thread leaves and the shared memory is released (see ring_land)
+        if (nb > 0) {
+            for (uint32_t e = 0; e < extra_arrivals; ++e) mbar_arrive(&q_full);
+            mbar_land(&q_full, 0);
+        }
+        if constexpr (Q8) {
+            if (issued_k > 0) mbar_land(&kraw_full, (issued_k - 1) & 1);
+            ring_land(vraw_full, issued_v, 2, 0);
+        } else {
+            ring_land(k_full, issued_k, 2, 0);
+            ring_land(v_full, issued_v, 2, 0);
+        }
+        atomicExch(error, 1);
+    }
 }
 
 // Adds the partial rows of query tiles whose key blocks were shared out: for row t and head h, M = max m_p,
@@ -1838,7 +1850,7 @@ bool encode_bytes_map(CUtensorMap *m, const void *base, long long rows, int row_
 // num_sms tiles of 128 rows).  Two blocks cost a CTA about 3.5 us (one for either group), the merge about as much.
 template <int D>
 const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *vc, const float *k_scale, const float *v_scale, uint16_t *out,
-                                size_t plane, int T, int slot0, int nq, int nkv, int max_context, uint32_t wait_limit, int *error,
+                                size_t plane, int T, int slot0, int nq, int nkv, int max_context, uint32_t wait_limit, uint32_t extra_arrivals, int *error,
                                 float *part_o, float2 *part_ml, int num_sms, cudaStream_t s) {
     const long long kv_rows = static_cast<long long>(nkv) * max_context;
     const bool q8 = k_scale != nullptr;
@@ -1859,12 +1871,12 @@ const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *v
         if (cudaFuncSetAttribute(prefill_attention_tc_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::SMEM_Q8) != cudaSuccess)
             return "cudaFuncSetAttribute failed";
         launch_pdl(prefill_attention_tc_kernel<D, true>, grid, dim3(AT_THREADS + 32 * AT_CW), AttnCfg<D>::SMEM_Q8, s, mqh, mql, mk, mv, out, plane, T,
-                   slot0, nq, nq / nkv, max_context, scale_log2, wait_limit, error, k_scale, v_scale, part_o, part_ml);
+                   slot0, nq, nq / nkv, max_context, scale_log2, wait_limit, extra_arrivals, error, k_scale, v_scale, part_o, part_ml);
     } else {
         if (cudaFuncSetAttribute(prefill_attention_tc_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::SMEM) != cudaSuccess)
             return "cudaFuncSetAttribute failed";
         launch_pdl(prefill_attention_tc_kernel<D, false>, grid, dim3(AT_THREADS), AttnCfg<D>::SMEM, s, mqh, mql, mk, mv, out, plane, T, slot0, nq,
-                   nq / nkv, max_context, scale_log2, wait_limit, error, static_cast<const float *>(nullptr), static_cast<const float *>(nullptr),
+                   nq / nkv, max_context, scale_log2, wait_limit, extra_arrivals, error, static_cast<const float *>(nullptr), static_cast<const float *>(nullptr),
                    part_o, part_ml);
     }
     if (splits > 1)
@@ -2060,8 +2072,8 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
         if (l == sh.n_layers - 1 && !whole_last_layer) break;   // the rest of the last layer feeds nothing that is kept
         const void *ka = kv8 ? static_cast<const void *>(kc8) : kc, *va = kv8 ? static_cast<const void *>(vc8) : vc;
         const float *ksc = kv8 ? m.k_scale + layer_rows : nullptr, *vsc = kv8 ? m.v_scale + layer_rows : nullptr;
-        const char *e = d == 64 ? launch_attention_tc<64>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->error, b->att_o, b->att_ml, m.num_sms, s)
-                                : launch_attention_tc<128>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->error, b->att_o, b->att_ml, m.num_sms, s);
+        const char *e = d == 64 ? launch_attention_tc<64>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->extra_arrivals, b->error, b->att_o, b->att_ml, m.num_sms, s)
+                                : launch_attention_tc<128>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->extra_arrivals, b->error, b->att_o, b->att_ml, m.num_sms, s);
         if (e) return e;
         g.N = H; g.K = qd; g.resid = b->resid; g.part = b->part; g.part_plane = x_plane;
         g.norm_w = static_cast<const uint16_t *>(w.post_norm);

@@ -43,7 +43,7 @@ struct PrefillBuffers {
     int *head_idx = nullptr;
     unsigned *head_ticket = nullptr;
     uint32_t wait_limit = 1u << 24;   // polls per wait (far beyond any legitimate wait of a tile)
-    uint32_t extra_arrivals = 0;      // tests only: 1 makes the first wait of every contraction run out
+    uint32_t extra_arrivals = 0;      // tests only: 1 makes the first wait of every contraction and of the attention run out
 };
 
 struct PrefillModel {

@@ -154,3 +154,59 @@ def test_prefill_contraction_wait_expires_and_is_reported():
         other.close()
     finally:
         pair.close()
+
+
+#: what gives up: (changes to the tiny shape, prompt, cache format)
+GIVE_UP = {
+    "tiles": (dict(), 40, None),
+    "tiles_int8": (dict(), 40, "int8"),
+    "persistent": (dict(ffn=9480, n_layers=1, vocab=500), 300, None),
+}
+
+
+def gives_up_as(cfg, n):
+    """The (cluster, pairs) of the shape's contractions with n tokens."""
+    from paper_2604_27476_b200 import edgefm_debug_prefill_launch
+    from test_prefill_plan import shapes
+    return {edgefm_debug_prefill_launch(epi, n, N, K)[2:4] for epi, N, K in shapes(cfg).values()}
+
+
+@pytest.mark.parametrize("polls", [1024, 1 << 16])
+@pytest.mark.parametrize("name", list(GIVE_UP))
+def test_a_prompt_cta_that_gives_up_waits_for_its_copies(name, polls):
+    """Contractions and attention whose first wait runs out, the producing thread long done with its part (few k-blocks) or stopped by its
+    ring: the copies under way must land before the CTA's shared memory is someone else's.  Other contexts, whose kernels follow at once
+    on the same stream, compute what they always do, to the bit."""
+    import numpy as np
+    import torch
+    from edgefm_synth import make_weights
+    from paper_2604_27476_b200 import DecodeContext, EdgefmError, Status, edgefm_debug_set_prefill_wait, upload_weights
+    more, n, kv_format = GIVE_UP[name]
+    cfg = CONFIGS["tiny"].with_(qkv_bias=True, **more)
+    plans = gives_up_as(cfg, n)
+    assert any(c > 0 for c, _ in plans) if name.startswith("tiles") else (0, int(name == "pairs")) in plans
+    ptrs, keep = upload_weights(make_weights(cfg))
+    toks = np.random.default_rng(5).integers(0, cfg.vocab, n).tolist()
+    ctx, *others = [DecodeContext(cfg, ptrs, n, kv_format=kv_format) for _ in range(4)]
+    try:
+        others[0].prefill(toks, 0)
+        torch.cuda.synchronize()
+        others[0].sync_status()
+        want = others[0].logits.cpu()
+        others[0].append_kv(0)
+        edgefm_debug_set_prefill_wait(ctx.handle, polls, 1)
+        t0 = time.perf_counter()
+        ctx.prefill(toks, 0)
+        for o in others:
+            o.prefill(toks, 0)
+        torch.cuda.synchronize()
+        assert time.perf_counter() - t0 < 5.0
+        with pytest.raises(EdgefmError) as ei:
+            ctx.sync_status()
+        assert ei.value.status == Status.ERR_TIMEOUT
+        for o in others:
+            o.sync_status()
+            assert torch.equal(o.logits.cpu(), want)
+    finally:
+        for c in (ctx, *others):
+            c.close()

@@ -61,19 +61,35 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
 // A CTA that gives up waits for what it has under way (copies into its shared memory, multiplies), in the end with a bound of its own.
 constexpr uint32_t PF_LAND_POLLS = 1u << 24;
 __device__ __forceinline__ void mbar_land(uint64_t *bar, uint32_t parity) {
-    int given_up = 0;
-    mbar_wait(bar, parity, &given_up, PF_LAND_POLLS);
+#pragma unroll 1
+    for (uint32_t i = 0; i < PF_LAND_POLLS && !mbar_try_wait(bar, parity); ++i) { }
 }
 // The copies of a ring: `issued` stages were asked for, the last `stages` of them may be on their way.  To be called behind a barrier that every
 // wait of the CTA precedes: a producer that has sent for everything is done long before another thread's wait runs out.  extra_arrivals: the
-// arrivals that nobody else makes (GemmArgs).
-__device__ __forceinline__ void ring_land(uint64_t *full_bar, int issued, int stages, uint32_t extra_arrivals) {
+// arrivals that nobody else makes (GemmArgs).  Not inlined: it hardly ever runs, and cost the clustered kernel up to 7 registers.
+__device__ __noinline__ void ring_land(uint64_t *full_bar, int issued, int stages, uint32_t extra_arrivals) {
 #pragma unroll 1
     for (int j = issued > stages ? issued - stages : 0; j < issued; ++j) {
         uint64_t *bar = full_bar + j % stages;
         for (uint32_t e = 0; e < extra_arrivals; ++e) mbar_arrive(bar);
         mbar_land(bar, (j / stages) & 1);
     }
+}
+// The same for a pair of CTAs, whose copies the first one counts: it has sent for `mine` stages and expected both CTAs' bytes for each, the second
+// for `peers`.  Neither is more than a ring ahead (a stage is sent for again when the multiplies of both have read it), so every stage
+// named here waits in its last phase.  What only one of them has sent for is put right: the first CTA expects the other's half, or counts the
+// half that will not come as landed.
+__device__ __forceinline__ void mbar_complete_tx(uint64_t *bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void pair_land(uint64_t *full_bar, int mine, int peers, int stages, uint32_t half_bytes, uint32_t extra_arrivals) {
+    const int issued = mine > peers ? mine : peers;
+#pragma unroll 1
+    for (int j = issued > stages ? issued - stages : 0; j < issued; ++j) {
+        if (j >= mine) mbar_expect_tx(full_bar + j % stages, half_bytes);
+        else if (j >= peers) mbar_complete_tx(full_bar + j % stages, half_bytes);
+    }
+    ring_land(full_bar, issued, stages, extra_arrivals);
 }
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
@@ -710,6 +726,12 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {   //
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+__device__ __forceinline__ int cluster_ld1(uint32_t addr) {
+    int v;
+    asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_st1(uint32_t addr, int v) { asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 
 // Tile shapes.  PF_NARROW: 128 output columns, 4 stages of 48 KB.  PF_WIDE: 256 output columns, 3 stages of 64 KB: per k-block
 // 64 KB of operands feed twice the multiplies of a narrow tile's 48 KB, which matters because operand delivery from L2, not
@@ -740,7 +762,7 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
     extern __shared__ uint8_t pf_dyn[];
     __shared__ uint64_t full_bar[C::STAGES], empty_bar[C::STAGES], acc_full[2], acc_empty[2], drain_bar;
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag, issued_sm;        // issued_sm: stages this CTA's producer has sent for
+    __shared__ int abort_flag, issued_sm, drained_sm;   // stages this CTA's producer has sent for; 1: its issuer has given up (drain_bar has an arrival)
     uint8_t *tiles = pf_dyn + ((1024u - (smem_u32(pf_dyn) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = PAIR ? blockIdx.x & 1 : 0, worker = blockIdx.x / CTAS, workers = gridDim.x / CTAS;
@@ -763,7 +785,7 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
         for (int s = 0; s < C::STAGES; ++s) { mbar_init(&full_bar[s], 1 + g.extra_arrivals); mbar_init(&empty_bar[s], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4 * CTAS); }
         mbar_init(&drain_bar, 1);
-        abort_flag = 0;
+        abort_flag = drained_sm = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {   // two accumulators: 2 BN columns of tensor memory, 128 lanes
@@ -826,10 +848,6 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
           }
         }
         issued_sm = issued;
-        // a pair's copies are counted by the first CTA, which may have given up before it expected all of them: they land within
-        // microseconds, the pair leaves together 0.2 ms later
-        if (PAIR && abort_flag)
-            for (const long long t0 = clock64(); clock64() - t0 < 400000;) { }
     } else if (warp == 1 && lane == 0) {     // issuer (of a pair, the first CTA's): per stage 4 tcgen05.mma (K = 16 each) for the hi pieces, 4 for the lo pieces
         const uint32_t idesc = umma_idesc_bf16(TILE_M, BN);
         auto mma = [&](uint32_t acc, uint64_t da, uint64_t db, uint32_t accumulate) {
@@ -864,6 +882,7 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
         if (!ok) {          // giving up: the multiplies already issued must finish before the tensor memory is freed
             commit(&drain_bar);
             mbar_land(&drain_bar, 0);
+            drained_sm = 1;
         }
     } else if (warp >= 2) {                  // epilogue: warp w may read lanes 32 (w % 4) .. + 31 of tensor memory
       const int quarter = warp & 3, sub = lane >> 3, c8 = lane & 7;
@@ -921,14 +940,28 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
     }
     tc_fence_before();
     __syncwarp();
-    if constexpr (PAIR) cluster_sync(); else __syncthreads();   // a pair leaves together: the first CTA's multiplies use both
+    if constexpr (PAIR) {                    // a pair leaves together: the first CTA's multiplies use both; it gives up together, too
+        const uint32_t peer_abort = cluster_addr(smem_u32(&abort_flag), rank ^ 1);
+        if (abort_flag) cluster_st1(peer_abort, 1);
+        cluster_sync();
+        if (abort_flag) {
+            if (threadIdx.x == 0) {
+                const int peers = cluster_ld1(cluster_addr(smem_u32(&issued_sm), rank ^ 1));
+                if (rank == 0) pair_land(full_bar, issued_sm, peers, C::STAGES, 2 * C::A_BYTES + BN * PF_BK, g.extra_arrivals);
+                else if (cluster_ld1(cluster_addr(smem_u32(&drained_sm), 0))) mbar_land(&drain_bar, 0);   // the first CTA's commit arrives here, too
+            }
+            cluster_sync();
+        }
+    } else {
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after();
         if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C::BN) : "memory");
         else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C::BN) : "memory");
     }
     if (threadIdx.x == 0 && abort_flag) {        // the CTA's shared memory is released when this thread leaves
-        if (rank == 0) ring_land(full_bar, issued_sm, C::STAGES, g.extra_arrivals);
+        if (!PAIR) ring_land(full_bar, issued_sm, C::STAGES, g.extra_arrivals);
         atomicExch(g.error, 1);
     }
 }
@@ -954,11 +987,6 @@ constexpr int TILE_STAGES_MAX = 8, TILE_THREADS = 256, TILE_SMEM = 110 * 1024, T
 __device__ __forceinline__ float4 cluster_ld4(uint32_t addr) {
     float4 v;
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ int cluster_ld1(uint32_t addr) {
-    int v;
-    asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ void prefetch_tile_l2(const CUtensorMap *map, int x, int y) {

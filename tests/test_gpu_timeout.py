@@ -161,6 +161,8 @@ GIVE_UP = {
     "tiles": (dict(), 40, None),
     "tiles_int8": (dict(), 40, "int8"),
     "persistent": (dict(ffn=9480, n_layers=1, vocab=500), 300, None),
+    "pairs": (dict(hidden=3072, n_q_heads=1, n_kv_heads=1, ffn=1872, n_layers=1, vocab=500), 858, None),     # seven row tiles: the last pair has one
+    "pairs_few_k_blocks": (dict(hidden=64, ffn=2560, n_layers=1, vocab=500), 421, None),                     # all of K in the ring at once
 }
 
 
@@ -184,7 +186,7 @@ def test_a_prompt_cta_that_gives_up_waits_for_its_copies(name, polls):
     more, n, kv_format = GIVE_UP[name]
     cfg = CONFIGS["tiny"].with_(qkv_bias=True, **more)
     plans = gives_up_as(cfg, n)
-    assert any(c > 0 for c, _ in plans) if name.startswith("tiles") else (0, int(name == "pairs")) in plans
+    assert any(c > 0 for c, _ in plans) if name.startswith("tiles") else (0, int(name.startswith("pairs"))) in plans
     ptrs, keep = upload_weights(make_weights(cfg))
     toks = np.random.default_rng(5).integers(0, cfg.vocab, n).tolist()
     ctx, *others = [DecodeContext(cfg, ptrs, n, kv_format=kv_format) for _ in range(4)]

@@ -974,7 +974,7 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
 //   * the K of a tile is spread over up to eight SMs, and no partial sums pass through global memory and a kernel of their own;
 //   * the weight tiles of the first stages are requested, the rest of this CTA's weights sent for to L2, BEFORE the predecessor is
 //     waited for (nothing writes weights);
-//   * at most 110 KB of shared memory where a CTA has few k-blocks: two CTAs per SM, so that the successor's set-up and first weights overlap
+//   * at most 110 KB of shared memory where a CTA has few k-blocks and a partial tile that is no larger: two CTAs per SM, so that the successor's set-up and first weights overlap
 //     this kernel's end; twice that where it has many (two stages of 48 KB: 27 us for 35 k-blocks, 1.8 MB, of a down projection);
 //   * an activation tile is loaded without its idle rows (a multiple of 8; the multiplies read whatever lies behind it, for rows nobody
 //     looks at);
@@ -1771,10 +1771,26 @@ int clusters_at_once(int c, int num_sms) {
     constexpr int AT_148[PF_CLUSTER_MAX + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
     return AT_148[c] * num_sms / 148;
 }
-// The same for a contraction's clusters of c: with few k-blocks each its CTAs take half an SM's shared memory, and any that are no more than the SMs fit.
-int tiles_at_once(int c, int kb, int rows, int bn, int num_sms) {
-    const int stages = (TILE_SMEM - 1024) / (rows * PF_BK * 4 + bn * PF_BK * 2), one = clusters_at_once(c, num_sms);
-    return (kb + c - 1) / c > 2 * stages ? one : num_sms / c < 2 * one ? num_sms / c : 2 * one;
+// Ring and shared memory of a CTA of prefill_tile_kernel with kb k-blocks: `rows` of activations (as loaded), tiles of bn columns.  deep: one CTA per SM
+// where the k-blocks are many.  The partial tile lies over the ring and may be the larger of the two (256 columns; 217 and more rows swapped).
+struct TileRoom { int stages, smem; };
+TileRoom tile_room(int rows, int bn, bool swap, int kb, bool deep) {
+    const int a_bytes = rows * PF_BK * 2, stage = 2 * a_bytes + bn * PF_BK * 2;
+    // the multiplies read 128 rows of the operand that has 128, from the start of either piece or (swapped) of the weights: room behind the
+    // last stage for those that are not loaded
+    const int reach = (swap ? 2 : 1) * a_bytes + PF_BM * PF_BK * 2, slack = reach > stage ? reach - stage : 0;
+    int stages = (TILE_SMEM - 1024 - slack) / stage;
+    if (kb > 2 * stages && deep) stages = (TILE_SMEM_DEEP - 1024 - slack) / stage;
+    if (stages > TILE_STAGES_MAX) stages = TILE_STAGES_MAX;
+    if (stages > kb) stages = kb;
+    const int ring = stages * stage + slack, partial = rows * bn * 4;
+    return {stages, 1024 + (ring > partial ? ring : partial)};
+}
+// Clusters of c that run at once in a contraction of kb k-blocks: where two of its CTAs fit an SM, any that are no more than the SMs.  (Taken for granted
+// for tiles of 256 columns, 0.5B shape, 450 tokens, QKV and O ran as 20 clusters of seven in two rounds: 2719 us a prompt, 2334 as it is.)
+int tiles_at_once(int c, int kb, int rows, int bn, bool swap, int num_sms) {
+    const int one = clusters_at_once(c, num_sms), two = num_sms / c < 2 * one ? num_sms / c : 2 * one;
+    return tile_room(rows, bn, swap, (kb + c - 1) / c, true).smem <= TILE_SMEM ? two : one;
 }
 
 // Rows of an activation tile that are loaded, up to 256 tokens: whole groups of 8, of 16 where the pieces are multiplied one after the other.
@@ -1807,23 +1823,15 @@ const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const 
 template <int EPI, int BN, bool SWAP>
 const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, GemmArgs &g, int num_sms, cudaStream_t s) {
     const int n_step = EPI == EPI_SWIGLU ? BN / 2 : BN, tiles = ((g.N + n_step - 1) / n_step) * (SWAP ? 1 : (g.M + PF_BM - 1) / PF_BM);
-    const int a_bytes = g.a_rows * PF_BK * 2, stage = 2 * a_bytes + BN * PF_BK * 2;
     const int kb = ((g.K + PF_BK - 1) / PF_BK + g.cluster - 1) / g.cluster;      // of the CTA with the most
-    // the multiplies read 128 rows of the operand that has 128, from the start of either piece or (swapped) of the weights: room behind the
-    // last stage for those that are not loaded
-    const int reach = (SWAP ? 2 : 1) * a_bytes + PF_BM * PF_BK * 2, slack = reach > stage ? reach - stage : 0;
-    g.stages = (TILE_SMEM - 1024 - slack) / stage;
-    if (kb > 2 * g.stages && tiles * g.cluster <= num_sms) g.stages = (TILE_SMEM_DEEP - 1024 - slack) / stage;
-    if (g.stages > TILE_STAGES_MAX) g.stages = TILE_STAGES_MAX;
-    if (g.stages > kb) g.stages = kb;
-    const int ring = g.stages * stage + slack, partial = g.a_rows * BN * 4;
-    const int smem = 1024 + (ring > partial ? ring : partial);
+    const TileRoom room = tile_room(g.a_rows, BN, SWAP, kb, tiles * g.cluster <= num_sms);
+    g.stages = room.stages;
     // swapped: the pieces' columns (side by side where they fit one multiply) are read 32 at a time
     const int cols = SWAP ? (2 * g.a_rows <= 256 ? g.a_rows : 0) + (g.a_rows + 31) / 32 * 32 : BN;
     for (g.tmem_cols = 32; g.tmem_cols < cols;) g.tmem_cols *= 2;
     if (cudaFuncSetAttribute(prefill_tile_kernel<EPI, BN, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM_DEEP) != cudaSuccess)
         return "cudaFuncSetAttribute failed";
-    launch_cluster(dim3(g.cluster), prefill_tile_kernel<EPI, BN, SWAP>, dim3(tiles * g.cluster), dim3(TILE_THREADS), static_cast<size_t>(smem), s, ma, ml, mb, g);
+    launch_cluster(dim3(g.cluster), prefill_tile_kernel<EPI, BN, SWAP>, dim3(tiles * g.cluster), dim3(TILE_THREADS), static_cast<size_t>(room.smem), s, ma, ml, mb, g);
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill contraction launch failed";
 }
 
@@ -1959,7 +1967,7 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
     int wide_swap_cost = 1 << 30;
     if (m_tiles == 2) {
         const int steps = (N + (epilogue == EPI_SWIGLU ? 63 : 127)) / (epilogue == EPI_SWIGLU ? 64 : 128), block = 4 * swapped_rows(M) + 2 * 128;
-        for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && steps <= tiles_at_once(c, kb, swapped_rows(M), 128, num_sms); ++c) {
+        for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && steps <= tiles_at_once(c, kb, swapped_rows(M), 128, true, num_sms); ++c) {
             const int cost = (kb + c - 1) / c * block + (c > 1 ? 2000 : 0);
             if (cost < wide_swap_cost) { wide_swap.cluster = c; wide_swap_cost = cost; }
         }
@@ -1973,8 +1981,8 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
         int best = 1 << 30;
         for (int bn = base; bn <= (epilogue == EPI_SWIGLU || m_tiles == 1 ? base : 256); bn *= 2) {
             const int t = m_tiles * ((N + bn - 1) / bn), step = epilogue == EPI_SWIGLU ? tiles : t;
-            for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && step <= tiles_at_once(c, kb, rows, bn, num_sms); ++c) {
-                const bool swap = rows < bn && bn <= 128 && rows < PF_BM;
+            const bool swap = rows < bn && bn <= 128 && rows < PF_BM;
+            for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && step <= tiles_at_once(c, kb, rows, bn, swap, num_sms); ++c) {
                 const int multiplies = 4 * (swap ? (rows > 32 ? rows : 32) : bn), operands = 4 * rows + 2 * bn;
                 const int cost = (kb + c - 1) / c * (multiplies > operands ? multiplies : operands) + (c > 1 ? 2000 : 0);
                 if (cost < best) { best = cost; p.columns = bn; p.cluster = c; p.swap = swap; }

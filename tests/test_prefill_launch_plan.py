@@ -36,6 +36,18 @@ def test_launches():
             assert columns in (128, 256), what
 
 
+def test_clusters_run_at_once():
+    """A partial tile of more than half an SM's shared memory (256 columns; 217 and more swapped rows) leaves one CTA per SM, and of such clusters
+    only so many fit the GPCs: one tile more is a second round (0.5B shape, 450 tokens: 20 clusters of seven where 15 run at once)."""
+    one_per_sm = (0, 148, 74, 45, 33, 26, 22, 15, 15)
+    for name, M in itertools.product(CONFIGS, itertools.chain(range(8, 700, 8), range(700, 4097, 100))):
+        for op, (epi, N, K) in shapes(CONFIGS[name]).items():
+            columns, _, cluster, _, swapped = edgefm_debug_prefill_launch(epi, M, N, K)
+            rows = M if swapped and M > 128 else min(M, 128)
+            if cluster and rows * columns * 4 > 109 * 1024:
+                assert tiles(min(M, 128) if swapped else M, N, columns // 2 if epi == SWIGLU else columns) <= one_per_sm[cluster], (name, op, M)
+
+
 def test_short_prompts_share_the_k_of_a_tile():
     """77 tokens of the 0.5B shape: QKV, O and down run on 90 to 112 CTAs instead of 14 to 18."""
     s = shapes(CONFIGS["qwen2.5-0.5b"])

@@ -561,7 +561,7 @@ struct GemmArgs {
     // gate/up
     uint16_t *act;            // [2][..][N]: hi and lo planes
     size_t act_plane;
-    int bn;                   // output columns of a tile: 64, 128 or 256; pairs that add to the residual stream: any multiple of 16 from 128 to 256
+    int bn;                   // output columns of a tile: 64, 128 or 256; pairs that add to the residual stream: any multiple of 16 from 144 to 256
     // prefill_tile_kernel
     int cluster;              // CTAs that share the K of an output tile
     int a_rows;               // rows of an activation tile that are loaded (a multiple of 8, at most 128)
@@ -2011,7 +2011,7 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
     if (epilogue == EPI_RESID) {
         double best = p.pairs ? rounds(m_pairs * ((N + 255) / 256) * splits, workers) * 1024. / splits : rounds(tiles * splits, num_sms) * 1075. / splits;
         if (splits > 1) best *= 1.05 * 1.1;
-        for (int bn = 128; bn <= 256; bn += 16) {
+        for (int bn = 144; bn <= 256; bn += 16) {        // (128 columns are single CTAs' tiles, see launch_gemm)
             const double cost = rounds(m_pairs * ((N + bn - 1) / bn), workers) * static_cast<double>(4 * bn > 512 + bn ? 4 * bn : 512 + bn);
             if (cost < best - 1e-9) { best = cost; p.columns = bn; p.splits = 1; p.pairs = true; }
         }

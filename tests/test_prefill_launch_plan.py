@@ -27,7 +27,7 @@ def test_launches():
             assert columns in (128, 256) or (pairs and epi == RESID), what
             assert 1 <= splits <= 8 and (splits == 1 or epi == RESID), what
         if pairs:
-            assert M > 128 and columns >= 128, what
+            assert M > 128 and columns > 128, what                            # tiles of 128 columns are launched as single CTAs'
         if swapped:                    # fewer padded tokens than columns, both pieces side by side; or two row tiles that share weight tiles
             assert cluster and columns <= 128 and (-(-M // 8) * 8 < columns if M < 128 else 128 < M <= 256), what
         if epi == QKV:

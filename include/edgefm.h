@@ -302,13 +302,13 @@ edgefm_status edgefm_debug_set_wait_limit(edgefm_ctx *ctx, uint32_t limit_ns, in
  * enqueued afterwards runs into the bound without any fault.  Host only. */
 edgefm_status edgefm_debug_set_prefill_wait(edgefm_ctx *ctx, uint32_t polls, int32_t extra_arrivals);
 
-/* The first stage of the plan of a contraction of [M tokens x K] x [K x N] of edgefm_prefill on num_sms SMs: out2 = {output tile: 0 = 128
- * columns, 1 = 256, 2 = 64, K units per output tile} (edgefm_debug_prefill_launch: what is made of it).  epilogue: 0 = QKV with heads of 128, 3 = with heads of 64, 1 = added to the residual stream (O and
- * down projection; only these split K), 2 = gate/up (128 gate columns and their 128 up columns, or 64 and 64; never split).  Tiles of
- * half the columns are taken where they still fit the SMs in one round.  Host only: for checking the planner without a GPU. */
+/* How edgefm_prefill tiles a contraction of [M tokens x K] x [K x N] on num_sms SMs: out2 = {output tile: 0 = 128 columns, 1 = more (256, or
+ * what fills the rounds of pairs of CTAs best), 2 = 64, K units per output tile, whether their sums meet in a cluster or in the norm
+ * kernel}.  epilogue: 0 = QKV with heads of 128, 3 = with heads of 64, 1 = added to the residual stream (O and down projection), 2 = gate/up
+ * (gate and up columns together).  Host only: for checking the planner without a GPU; edgefm_debug_prefill_launch gives the same plan in full. */
 edgefm_status edgefm_debug_prefill_plan(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t *out2);
 
-/* What runs for such a contraction: out5 = {output columns of a tile (gate and up columns together), K units that leave partial sums in
+/* The whole plan of such a contraction: out5 = {output columns of a tile (gate and up columns together), K units that leave partial sums in
  * global memory, CTAs of a cluster that share the K of a tile (0: the persistent kernel), 1 = row tiles are multiplied two by two by
  * pairs of CTAs, 1 = the weights are the rows of the multiply and the tokens its columns}.  Host only. */
 edgefm_status edgefm_debug_prefill_launch(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t *out5);

@@ -220,7 +220,7 @@ def edgefm_sync_status(ctx, stream=None):
 
 
 def edgefm_debug_prefill_plan(epilogue, M, N, K, num_sms=148):
-    """(tile, splits) the prefill planner gives a contraction (host only): tile 0 = 128 output columns, 1 = 256, 2 = 64."""
+    """(tile, K units) the prefill planner gives a contraction (host only): tile 0 = 128 output columns, 1 = more, 2 = 64."""
     L = load_library()
     L.edgefm_debug_prefill_plan.restype = ctypes.c_int
     L.edgefm_debug_prefill_plan.argtypes = [ctypes.c_int32] * 5 + [ctypes.POINTER(ctypes.c_int32)]

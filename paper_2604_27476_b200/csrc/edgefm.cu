@@ -821,10 +821,9 @@ edgefm_status edgefm_debug_set_prefill_wait(edgefm_ctx *ctx, uint32_t polls, int
 
 edgefm_status edgefm_debug_prefill_plan(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t *out2) {
     if (!out2 || epilogue < 0 || epilogue > 3 || M < 1 || N < 1 || K < 1 || num_sms < 1) return EDGEFM_ERR_INVALID_ARG;
-    int shape = 0, splits = 0;
-    prefill_plan_contraction(epilogue == 3 ? 0 : epilogue, epilogue == 3 ? 64 : 128, M, N, K, num_sms, &shape, &splits);
-    out2[0] = shape == PF_WIDE ? 1 : shape == PF_SLIM ? 2 : 0;
-    out2[1] = splits;
+    const PrefillPlan p = prefill_plan(epilogue == 3 ? 0 : epilogue, epilogue == 3 ? 64 : 128, M, N, K, num_sms);
+    out2[0] = p.columns == 64 ? 2 : p.columns == 128 ? 0 : 1;
+    out2[1] = p.cluster ? p.cluster : p.splits;
     return EDGEFM_OK;
 }
 

@@ -733,7 +733,7 @@ __device__ __forceinline__ int cluster_ld1(uint32_t addr) {
 }
 __device__ __forceinline__ void cluster_st1(uint32_t addr, int v) { asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 
-// Tile shapes.  PF_NARROW: 128 output columns, 4 stages of 48 KB.  PF_WIDE: 256 output columns, 3 stages of 64 KB: per k-block
+// COLUMNS of a tile.  128: 4 stages of 48 KB.  256: 3 stages of 64 KB, per k-block
 // 64 KB of operands feed twice the multiplies of a narrow tile's 48 KB, which matters because operand delivery from L2, not
 // the tensor pipe, bounds the narrow tiles.  Gate/up runs wide: 128 gate columns and their 128 up partners.
 // PAIR: two row tiles, one in either CTA of a cluster of two, multiplied together (cta_group::2): a CTA fetches half of the weight tile only,
@@ -741,21 +741,21 @@ __device__ __forceinline__ void cluster_st1(uint32_t addr, int v) { asm volatile
 // shape, 97.2 ms, all by pairs 94.8; 1000 tokens, 3B, 12.60 and 12.43; these passes run into the power limit).
 // The kernel is persistent (one CTA per SM, tiles dealt round-robin, neighbours sharing a weight tile) with TWO accumulators
 // in tensor memory, so that the epilogue of a tile runs under the main loop of the next.
-template <int SHAPE, bool PAIR> struct GemmCfg {
-    static constexpr int BN = SHAPE == PF_WIDE ? 256 : 128;
-    static constexpr int STAGES = SHAPE == PF_WIDE && !PAIR ? 3 : 4;
+template <int COLUMNS, bool PAIR> struct GemmCfg {
+    static constexpr int BN = COLUMNS;
+    static constexpr int STAGES = COLUMNS == 256 && !PAIR ? 3 : 4;
     static constexpr int A_BYTES = PF_BM * PF_BK * 2, B_BYTES = BN * PF_BK * 2 / (PAIR ? 2 : 1);
     static constexpr int STAGE_BYTES = 2 * A_BYTES + B_BYTES;          // A hi, A lo, B
     static constexpr int CHUNK_BYTES = PF_BM * 64 * 4;                 // the epilogue's chunk of 64 columns
     static constexpr int SMEM = STAGES * STAGE_BYTES + CHUNK_BYTES + 1024;   // + room to align the first stage to 1024 bytes
 };
 
-template <int EPI, int SHAPE, bool PAIR>
+template <int EPI, int COLUMNS, bool PAIR>
 __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant__ CUtensorMap map_a_hi,
                                                            const __grid_constant__ CUtensorMap map_a_lo,
                                                            const __grid_constant__ CUtensorMap map_b, const GemmArgs g) {
-    using C = GemmCfg<SHAPE, PAIR>;
-    static_assert(!PAIR || SHAPE == PF_WIDE, "a CTA of a pair fetches 128 of the 256 columns");
+    using C = GemmCfg<COLUMNS, PAIR>;
+    static_assert(!PAIR || COLUMNS == 256, "a CTA of a pair fetches 128 of the 256 columns");
     const int BN = PAIR && EPI == EPI_RESID ? g.bn : C::BN;
     const int N_STEP = EPI == EPI_SWIGLU ? C::BN / 2 : BN;          // output columns (of g.N) a tile covers
     constexpr int CTAS = PAIR ? 2 : 1, TILE_M = CTAS * PF_BM;
@@ -970,7 +970,7 @@ __global__ void __launch_bounds__(192) prefill_gemm_kernel(const __grid_constant
 // tile, the partial tiles meet through distributed shared memory, every CTA finishes its share of the rows (77 tokens behind 1024, 0.5B
 // shape: 1882 us a prompt by the persistent kernel and its K splits, 1438 so; 9 behind 2048, 1.5B: 2744 and 1799).  Such a pass is a
 // chain of latencies, so everything here shortens the chain:
-//   * tiles of half the columns where those fit the round, too: PF_SLIM, 64 columns, or PF_NARROW for gate/up, 64 + 64;
+//   * tiles of half the columns where those fit the round, too: 64, or 64 + 64 for gate/up;
 //   * the K of a tile is spread over up to eight SMs, and no partial sums pass through global memory and a kernel of their own;
 //   * the weight tiles of the first stages are requested, the rest of this CTA's weights sent for to L2, BEFORE the predecessor is
 //     waited for (nothing writes weights);
@@ -1810,13 +1810,13 @@ bool encode_operand_map(CUtensorMap *m, const void *base, long long rows, int K,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int EPI, int SHAPE, bool PAIR>
+template <int EPI, int COLUMNS, bool PAIR>
 const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const CUtensorMap &mb, const GemmArgs &g, int units, int workers, cudaStream_t s) {
-    using C = GemmCfg<SHAPE, PAIR>;
-    if (cudaFuncSetAttribute(prefill_gemm_kernel<EPI, SHAPE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
+    using C = GemmCfg<COLUMNS, PAIR>;
+    if (cudaFuncSetAttribute(prefill_gemm_kernel<EPI, COLUMNS, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
         return "cudaFuncSetAttribute failed";
     const int ctas = PAIR ? 2 : 1;
-    launch_cluster(dim3(ctas), prefill_gemm_kernel<EPI, SHAPE, PAIR>, dim3((units < workers ? units : workers) * ctas), dim3(192), C::SMEM, s, ma, ml, mb, g);
+    launch_cluster(dim3(ctas), prefill_gemm_kernel<EPI, COLUMNS, PAIR>, dim3((units < workers ? units : workers) * ctas), dim3(192), C::SMEM, s, ma, ml, mb, g);
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill GEMM launch failed";
 }
 
@@ -1861,11 +1861,11 @@ const char *launch_gemm(const uint16_t *a, size_t a_plane, const void *w, long l
         }
     const int m_tiles = (g.M + PF_BM - 1) / PF_BM;
     if constexpr (EPI != EPI_SWIGLU)
-        if (plan.columns == 128) return launch_gemm_cfg<EPI, PF_NARROW, false>(ma, ml, mb, g, m_tiles * ((g.N + 127) / 128) * g.splits, num_sms, s);
+        if (plan.columns == 128) return launch_gemm_cfg<EPI, 128, false>(ma, ml, mb, g, m_tiles * ((g.N + 127) / 128) * g.splits, num_sms, s);
     const int n_step = EPI == EPI_SWIGLU ? 128 : g.bn, units = ((g.N + n_step - 1) / n_step) * g.splits;
     if constexpr (EPI != EPI_LOGITS)
-        if (plan.pairs) return launch_gemm_cfg<EPI, PF_WIDE, true>(ma, ml, mb, g, (m_tiles + 1) / 2 * units, num_sms / 2, s);
-    return launch_gemm_cfg<EPI, PF_WIDE, false>(ma, ml, mb, g, m_tiles * units, num_sms, s);
+        if (plan.pairs) return launch_gemm_cfg<EPI, 256, true>(ma, ml, mb, g, (m_tiles + 1) / 2 * units, num_sms / 2, s);
+    return launch_gemm_cfg<EPI, 256, false>(ma, ml, mb, g, m_tiles * units, num_sms, s);
 }
 
 // Map of a byte matrix [rows][row_bytes] (the codes of a compressed cache); a box is box_rows whole rows, unswizzled.
@@ -1923,44 +1923,36 @@ const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *v
 
 }  // namespace
 
-// Shape and K split.  Cost model: the rounds the SMs need (units / SMs, rounded up) times the cost of a unit; a wide tile does
-// twice the work of a narrow one for 1.33 x the operand traffic (1.6), a K split divides a unit's cost and adds a little for
-// the partial sums (5 %).  Only the contractions that add to the residual stream split (their partial sums are added by the
-// norm kernel that follows, in a fixed order); a split keeps at least 12 k-blocks per unit and is considered only when the
-// unsplit tiles do not fill the SMs once (with more tiles the partial-sum traffic costs more than the better balance gains:
-// 7B shape, 2048 tokens, 48.0 -> 50.7 ms).
-// Half as many columns per tile (PF_SLIM; gate/up: PF_NARROW) where the tiles and their K splits still fit the SMs in one round; a QKV tile is whole
-// heads.
-void prefill_plan_contraction(int epilogue, int head_dim, int M, int N, int K, int num_sms, int *shape, int *splits) {
-    const int m_tiles = (M + PF_BM - 1) / PF_BM, kb = (K + PF_BK - 1) / PF_BK;
-    *shape = PF_WIDE;
-    *splits = 1;
-    if (epilogue != EPI_SWIGLU) {
-        const int tiles[2] = {((N + 127) / 128) * m_tiles, ((N + 255) / 256) * m_tiles};
-        const double cost[2] = {1.0, 1.6};
-        int best_wide = 0;
-        double best = 1e30;
-        for (int wide = 0; wide < 2; ++wide)
-            for (int sp = 1; sp <= (epilogue == EPI_RESID ? (m_tiles == 1 ? PF_SPLIT_MAX : 4) : 1); ++sp) {
-                if (sp > 1 && (kb / sp < 12 || tiles[wide] > num_sms)) break;   // split only grids that leave SMs idle in their one round
-                const int units = tiles[wide] * sp;
-                const double t = ((units + num_sms - 1) / num_sms) * cost[wide] / sp * (sp > 1 ? 1.05 : 1.0);
-                if (t < best - 1e-9) { best = t; best_wide = wide; *splits = sp; }
-            }
-        *shape = best_wide ? PF_WIDE : PF_NARROW;
-    }
-    if (epilogue == EPI_LOGITS || (epilogue == EPI_QKV && head_dim != 64) || ((N + 63) / 64) * m_tiles * *splits > num_sms) return;
-    *shape = epilogue == EPI_SWIGLU ? PF_NARROW : PF_SLIM;
-}
-
-// What runs: the tile shape and K split of prefill_plan_contraction, refined.
+// What a contraction is launched as (host logic, depends on the sizes and the SM count alone).
 PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int num_sms) {
-    int shape, splits;
-    prefill_plan_contraction(epilogue, head_dim, M, N, K, num_sms, &shape, &splits);
     const int m_tiles = (M + PF_BM - 1) / PF_BM, kb = (K + PF_BK - 1) / PF_BK;
-    PrefillPlan p{shape == PF_WIDE ? 256 : shape == PF_SLIM ? 64 : 128, splits, 0, false, false};
-    const int n_step = epilogue == EPI_SWIGLU ? p.columns / 2 : p.columns, tiles = m_tiles * ((N + n_step - 1) / n_step);
+    auto rounds = [](int units, int n) { return (units + n - 1) / n; };
+    auto tiles_of = [&](int step) { return m_tiles * ((N + step - 1) / step); };      // step: output columns a tile covers
+    // What the persistent kernel would take with single CTAs: the rounds over the SMs times the cost of a unit; a tile of 256 columns does twice the
+    // work of one of 128 for 1.33 x the operand traffic (1.6), a K split divides a unit's cost and adds a little for the partial sums (5 %).
+    // Only the contractions that add to the residual stream split; a split keeps at least 12 k-blocks per unit and is considered only when the
+    // unsplit tiles do not fill the SMs once (with more tiles the partial-sum traffic costs more than the better balance gains: 7B shape,
+    // 2048 tokens, 48.0 -> 50.7 ms).  Gate/up: 128 gate columns and their 128 up columns.
+    PrefillPlan p{256, 1, 0, false, false};
+    if (epilogue != EPI_SWIGLU) {
+        double best = 1e30;
+        for (int columns = 128; columns <= 256; columns *= 2)
+            for (int sp = 1; sp <= (epilogue == EPI_RESID ? (m_tiles == 1 ? PF_SPLIT_MAX : 4) : 1); ++sp) {
+                if (sp > 1 && (kb / sp < 12 || tiles_of(columns) > num_sms)) break;
+                const double t = rounds(tiles_of(columns) * sp, num_sms) * (columns == 256 ? 1.6 : 1.0) / sp * (sp > 1 ? 1.05 : 1.0);
+                if (t < best - 1e-9) { best = t; p.columns = columns; p.splits = sp; }
+            }
+    }
     if (epilogue == EPI_LOGITS) return p;
+    // Columns of the smallest tiles that clusters are made of: 64 (a QKV tile is whole heads; gate/up: 64 + 64) where those fit the SMs in one round
+    // with the K split above, 128 where it has no use for more; else (0) the tiles are too many.
+    int base = 0;
+    if ((epilogue != EPI_QKV || head_dim == 64) && tiles_of(64) * p.splits <= num_sms) {
+        base = epilogue == EPI_SWIGLU ? 128 : 64;
+    } else if (p.columns == 128) {
+        if (tiles_of(128) > num_sms) return p;
+        base = 128;
+    }
     // 129 to 256 tokens: the tokens as the columns of one row of tiles (gate/up: 64 + 64 columns), if these fit the SMs once and no other tiles that do
     // are cheaper.
     PrefillPlan wide_swap{128, 1, 0, false, true};
@@ -1975,14 +1967,13 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
     // Clusters where the tiles fit the SMs in one round.  A k-block costs a CTA what its operands take at 64 bytes per cycle, or its multiplies:
     // 4 cycles per column over 128 rows, or (swapped, the weights are the rows) 4 per token; sharing a tile's K costs the exchange of the
     // partial tiles, about 2000 cycles.  Tiles of 256 columns halve the traffic of several row tiles' activations.
-    if (shape != PF_WIDE) {
-        if (tiles > num_sms) return p;
-        const int rows = M < PF_BM ? (M + 7) & ~7 : PF_BM, base = p.columns;
+    if (base) {
+        const int rows = M < PF_BM ? (M + 7) & ~7 : PF_BM;
         int best = 1 << 30;
         for (int bn = base; bn <= (epilogue == EPI_SWIGLU || m_tiles == 1 ? base : 256); bn *= 2) {
-            const int t = m_tiles * ((N + bn - 1) / bn), step = epilogue == EPI_SWIGLU ? tiles : t;
+            const int tiles = tiles_of(epilogue == EPI_SWIGLU ? bn / 2 : bn);
             const bool swap = rows < bn && bn <= 128 && rows < PF_BM;
-            for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && step <= tiles_at_once(c, kb, rows, bn, swap, num_sms); ++c) {
+            for (int c = 1; c <= PF_CLUSTER_MAX && c <= kb && tiles <= tiles_at_once(c, kb, rows, bn, swap, num_sms); ++c) {
                 const int multiplies = 4 * (swap ? (rows > 32 ? rows : 32) : bn), operands = 4 * rows + 2 * bn;
                 const int cost = (kb + c - 1) / c * (multiplies > operands ? multiplies : operands) + (c > 1 ? 2000 : 0);
                 if (cost < best) { best = cost; p.columns = bn; p.cluster = c; p.swap = swap; }
@@ -2000,17 +1991,16 @@ PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int nu
         return PrefillPlan{128, 1, 1, false, rows < PF_BM};
     }
     // Pairs of CTAs where they need no more rounds over the SMs (an odd number of row tiles leaves one CTA of a pair without work).
-    const int workers = num_sms / 2, m_pairs = (m_tiles + 1) / 2;
+    const int workers = num_sms / 2, m_pairs = (m_tiles + 1) / 2, n_step = epilogue == EPI_SWIGLU ? 128 : 256;
     if (m_tiles < 2 || workers < 1) return p;
-    auto rounds = [](int units, int n) { return (units + n - 1) / n; };
-    p.pairs = rounds(m_pairs * ((N + n_step - 1) / n_step) * splits, workers) <= rounds(tiles * splits, num_sms);
+    p.pairs = rounds(m_pairs * ((N + n_step - 1) / n_step) * p.splits, workers) <= rounds(tiles_of(n_step) * p.splits, num_sms);
     // A contraction that adds to the residual stream takes the number of columns that fills its rounds best: a k-block costs a CTA 4 cycles
     // per column in the tensor cores, or what its operands (32 KB of activations, 64 bytes per column) take at 64 bytes per cycle; a K split costs its
     // partial sums a pass through memory and the norm kernel (about a tenth).  (4096 tokens, 7B shape: 160 columns, 4.97 rounds, against 3.03
     // rounds of 256: O 212 -> 202 us, down 930 -> 894, at the power limit.)
     if (epilogue == EPI_RESID) {
-        double best = p.pairs ? rounds(m_pairs * ((N + 255) / 256) * splits, workers) * 1024. / splits : rounds(tiles * splits, num_sms) * 1075. / splits;
-        if (splits > 1) best *= 1.05 * 1.1;
+        double best = p.pairs ? rounds(m_pairs * ((N + 255) / 256) * p.splits, workers) * 1024. / p.splits : rounds(tiles_of(256) * p.splits, num_sms) * 1075. / p.splits;
+        if (p.splits > 1) best *= 1.05 * 1.1;
         for (int bn = 144; bn <= 256; bn += 16) {        // (128 columns are single CTAs' tiles, see launch_gemm)
             const double cost = rounds(m_pairs * ((N + bn - 1) / bn), workers) * static_cast<double>(4 * bn > 512 + bn ? 4 * bn : 512 + bn);
             if (cost < best - 1e-9) { best = cost; p.columns = bn; p.splits = 1; p.pairs = true; }

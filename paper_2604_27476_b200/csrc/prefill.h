@@ -57,12 +57,9 @@ struct PrefillModel {
     int num_sms;
 };
 
-// Tile shapes of a contraction: 128, 64 or 256 output columns (gate/up: 64 gate and 64 up, or 128 and 128).
-enum { PF_NARROW = 0, PF_SLIM = 1, PF_WIDE = 2 };
-// Tile shape and K split a contraction of [M x K] x [K x N] gets on num_sms SMs (host logic, no device needed).
+// How a contraction of [M x K] x [K x N] is launched on num_sms SMs (host logic, no device needed).
 // epilogue: 0 = QKV (heads of head_dim), 1 = added to the residual stream (O, down), 2 = gate/up, 3 = logits of a verified block.
-void prefill_plan_contraction(int epilogue, int head_dim, int M, int N, int K, int num_sms, int *shape, int *splits);
-// What runs for such a contraction: output columns of a tile (gate/up: gate and up columns together), K units that leave partial sums in global
+// Output columns of a tile (gate/up: gate and up columns together), K units that leave partial sums in global
 // memory, CTAs of a cluster that share the K of a tile (0: the persistent kernel), and whether two row tiles are multiplied by a pair of CTAs.
 // swap: in a cluster the weights are the rows of the multiply and the tokens its columns.
 struct PrefillPlan { int columns, splits, cluster; bool pairs, swap; };

@@ -319,23 +319,9 @@ def run_prefill(args, cfg):
             "ms_min": times[0], "prompt_tokens_per_s": T / (ms * 1e-3),
             "roofline": {"bound": "tensor", "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak, "traffic": None,
                          "note": "achieved counts the method's flops; the tensor cores execute twice that (two bf16 pieces per activation); peak = measured sustained cuBLAS bf16 rate" + ("" if peaks.get("bf16_tflops_sustained") else " (fallback)")},
-            "gpu_launches": len(times) * ctx_prefill_launches(cfg, args.kv_format == "int8", T), "clocks": clocks}
+            "gpu_launches": len(times) * ctx.prefill_launches, "clocks": clocks}
     print(json.dumps(line), flush=True)
     ctx.close()
-
-
-def ctx_prefill_launches(cfg, kv_int8, tokens):
-    """Kernels one edgefm_prefill call (8 tokens or more) enqueues at least: per pass of up to 4096 tokens the rope table and the embedding /
-    norm, 5 per layer (QKV, attention, O, gate/up, down; one more compresses the new rows of an 8-bit cache, one more norms behind a
-    contraction that leaves K-split partial sums), then the output layer.  (Shared-out attention adds a merge, not counted.)"""
-    from paper_2604_27476_b200 import edgefm_debug_prefill_launch
-    count, qd = 1, cfg.n_q_heads * cfg.head_dim
-    while tokens > 0:
-        m = min(tokens, 4096)
-        norms = sum(edgefm_debug_prefill_launch(1, m, cfg.hidden, k)[1] > 1 for k in (qd, cfg.ffn))
-        count += 2 + (5 + norms + bool(kv_int8)) * cfg.n_layers
-        tokens -= m
-    return count
 
 
 def main():

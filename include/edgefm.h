@@ -239,6 +239,9 @@ edgefm_status edgefm_export_kv_int8(edgefm_ctx *ctx, void *k_codes_out, void *v_
 /* Number of kernel launches one decode step performs (always 1). */
 edgefm_status edgefm_get_launches_per_step(const edgefm_ctx *ctx, int32_t *n_launches_host);
 
+/* Number of kernels the last edgefm_prefill of this context enqueued (or the last edgefm_verify_block that took the prompt kernels). */
+edgefm_status edgefm_get_prefill_launches(const edgefm_ctx *ctx, int32_t *n_launches_host);
+
 /* Synchronise `stream`, then report whether a bounded device-side wait of the persistent step kernel
  * expired or one of its self-checks failed (EDGEFM_ERR_TIMEOUT; the context is then unusable and must be destroyed:
  * behind an expired wait later steps do nothing and new cache rows do not reset the status) or all is well.  ctx == NULL: the status left by the last edgefm_decode_step_static on the current device. */

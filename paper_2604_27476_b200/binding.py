@@ -50,7 +50,7 @@ class _Weights(ctypes.Structure):
 
 
 EXPORTS = ("edgefm_create", "edgefm_prefill_kv", "edgefm_decode_step", "edgefm_destroy", "edgefm_get_length",
-           "edgefm_export_kv", "edgefm_get_launches_per_step", "edgefm_last_error", "edgefm_version",
+           "edgefm_export_kv", "edgefm_get_launches_per_step", "edgefm_get_prefill_launches", "edgefm_last_error", "edgefm_version",
            "edgefm_sync_status", "edgefm_debug_profile", "edgefm_debug_set_wait_limit", "edgefm_debug_set_prefill_wait", "edgefm_debug_prefill_plan", "edgefm_debug_prefill_launch", "edgefm_debug_plan", "edgefm_debug_step_plan", "edgefm_decode_step_static", "edgefm_set_vocab_subset",
            "edgefm_append_kv", "edgefm_create_with_options", "edgefm_export_kv_int8", "edgefm_verify_block", "edgefm_sync_length", "edgefm_prefill_tokens", "edgefm_prefill")
 
@@ -95,6 +95,8 @@ def load_library():
     L.edgefm_export_kv.argtypes = [vp, vp, vp, vp]
     L.edgefm_get_launches_per_step.restype = ctypes.c_int
     L.edgefm_get_launches_per_step.argtypes = [vp, ctypes.POINTER(i32)]
+    L.edgefm_get_prefill_launches.restype = ctypes.c_int
+    L.edgefm_get_prefill_launches.argtypes = [vp, ctypes.POINTER(i32)]
     L.edgefm_sync_status.restype = ctypes.c_int
     L.edgefm_sync_status.argtypes = [vp, vp]
     L.edgefm_debug_profile.restype = ctypes.c_int
@@ -181,6 +183,12 @@ def edgefm_get_length(ctx) -> int:
 def edgefm_get_launches_per_step(ctx) -> int:
     n = ctypes.c_int32()
     _check(load_library().edgefm_get_launches_per_step(ctx, ctypes.byref(n)), ctx)
+    return n.value
+
+
+def edgefm_get_prefill_launches(ctx) -> int:
+    n = ctypes.c_int32()
+    _check(load_library().edgefm_get_prefill_launches(ctx, ctypes.byref(n)), ctx)
     return n.value
 
 
@@ -447,6 +455,10 @@ class DecodeContext:
     @property
     def launches_per_step(self) -> int:
         return edgefm_get_launches_per_step(self.handle)
+
+    @property
+    def prefill_launches(self) -> int:
+        return edgefm_get_prefill_launches(self.handle)
 
     def close(self):
         if getattr(self, "handle", None):

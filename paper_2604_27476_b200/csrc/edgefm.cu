@@ -161,7 +161,7 @@ struct edgefm_ctx {
     StepState *host_state = nullptr;      // pinned: edgefm_sync_length reads the device's state with one wait
     int launches_per_step = 0;
     PrefillBuffers pf;           // work buffers of edgefm_prefill, allocated at its first call
-    int prefill_launches = 0;    // kernels the last edgefm_prefill enqueued
+    int prefill_launches = 0;    // kernels the last edgefm_prefill (or block through the prompt kernels) enqueued
     uint32_t pf_wait_limit = 1u << 24, pf_extra_arrivals = 0;   // edgefm_debug_set_prefill_wait
 
     uint32_t spin_limit = 1000000000u;   // edgefm_debug_set_wait_limit: 1 s
@@ -560,11 +560,11 @@ edgefm_status edgefm_verify_block(edgefm_ctx *ctx, const int32_t *tokens, int32_
         const bool sub = ctx->vocab_subset > 0;
         if (const char *e = prefill_verify_head(pm, &ctx->pf, m, ctx->final_norm, sub ? static_cast<const void *>(ctx->sub_lm) : ctx->lm_head,
                                                 sub ? ctx->vocab_ids : nullptr, sub ? ctx->vocab_subset : ctx->shape.vocab, logits_out, n_accepted_out,
-                                                next_token_out, slot0, position, s)) {
+                                                next_token_out, slot0, position, s, &launches)) {
             cudaGetLastError();
             return fail(ctx, EDGEFM_ERR_CUDA, "%s", e);
         }
-        ctx->prefill_launches = launches + 1;
+        ctx->prefill_launches = launches;
         ctx->cur_len += m;     // an upper bound until edgefm_sync_length
         ctx->len_exact = false;
         ctx->have_token = true;
@@ -767,6 +767,12 @@ edgefm_status edgefm_set_vocab_subset(edgefm_ctx *ctx, const int32_t *token_ids,
 edgefm_status edgefm_get_launches_per_step(const edgefm_ctx *ctx, int32_t *n) {
     if (!ctx || !n) return EDGEFM_ERR_INVALID_ARG;
     *n = ctx->launches_per_step;
+    return EDGEFM_OK;
+}
+
+edgefm_status edgefm_get_prefill_launches(const edgefm_ctx *ctx, int32_t *n) {
+    if (!ctx || !n) return EDGEFM_ERR_INVALID_ARG;
+    *n = ctx->prefill_launches;
     return EDGEFM_OK;
 }
 

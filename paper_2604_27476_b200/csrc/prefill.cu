@@ -1887,7 +1887,7 @@ bool encode_bytes_map(CUtensorMap *m, const void *base, long long rows, int row_
 template <int D>
 const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *vc, const float *k_scale, const float *v_scale, uint16_t *out,
                                 size_t plane, int T, int slot0, int nq, int nkv, int max_context, uint32_t wait_limit, uint32_t extra_arrivals, int *error,
-                                float *part_o, float2 *part_ml, int num_sms, cudaStream_t s) {
+                                float *part_o, float2 *part_ml, int num_sms, cudaStream_t s, int *launches) {
     const long long kv_rows = static_cast<long long>(nkv) * max_context;
     const bool q8 = k_scale != nullptr;
     CUtensorMap mqh, mql, mk, mv;
@@ -1918,6 +1918,7 @@ const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *v
     if (splits > 1)
         launch_pdl(prefill_attention_merge_kernel<D>, dim3((T * nq + 3) / 4), dim3(128), 0, s, static_cast<const float *>(part_o), static_cast<const float2 *>(part_ml),
                    splits, tiles * AT_BM, out, plane, T, nq, scale_log2);
+    *launches += splits > 1 ? 2 : 1;
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill attention launch failed";
 }
 
@@ -2098,9 +2099,9 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
         if (l == sh.n_layers - 1 && !whole_last_layer) break;   // the rest of the last layer feeds nothing that is kept
         const void *ka = kv8 ? static_cast<const void *>(kc8) : kc, *va = kv8 ? static_cast<const void *>(vc8) : vc;
         const float *ksc = kv8 ? m.k_scale + layer_rows : nullptr, *vsc = kv8 ? m.v_scale + layer_rows : nullptr;
-        const char *e = d == 64 ? launch_attention_tc<64>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->extra_arrivals, b->error, b->att_o, b->att_ml, m.num_sms, s)
-                                : launch_attention_tc<128>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->extra_arrivals, b->error, b->att_o, b->att_ml, m.num_sms, s);
-        if (e) return e;
+        const char *e = d == 64 ? launch_attention_tc<64>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->extra_arrivals, b->error, b->att_o, b->att_ml, m.num_sms, s, &count)
+                                : launch_attention_tc<128>(b->q, ka, va, ksc, vsc, b->attn, q_plane, n, slot0, nq, nkv, m.max_context, b->wait_limit, b->extra_arrivals, b->error, b->att_o, b->att_ml, m.num_sms, s, &count);
+        if (e) return e;      // (attention and its merge are counted where they are launched)
         g.N = H; g.K = qd; g.resid = b->resid; g.part = b->part; g.part_plane = x_plane;
         g.norm_w = static_cast<const uint16_t *>(w.post_norm);
         if ((e = launch_gemm<EPI_RESID>(b->attn, q_plane, w.wo, H, g, m.num_sms, s))) return e;
@@ -2124,7 +2125,7 @@ const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t 
         }
         raw = g.splits == 1;
         pieces = g.ss_pieces;
-        count += 4;
+        count += 3;
     }
     if (cudaGetLastError() != cudaSuccess) return "prefill kernel launch failed";
     if (launches) *launches = count;
@@ -2147,7 +2148,7 @@ const char *prefill_head(const PrefillModel &m, PrefillBuffers *b, int row, cons
 }
 
 const char *prefill_verify_head(const PrefillModel &m, PrefillBuffers *b, int n, const void *final_norm, const void *lm, const int *ids, int rows,
-                                float *logits_out, int *n_accepted_out, int *next_token_out, int slot0, int pos, cudaStream_t s) {
+                                float *logits_out, int *n_accepted_out, int *next_token_out, int slot0, int pos, cudaStream_t s, int *launches) {
     // final norm of the block's rows (two bf16 planes), the logits of all rows as ONE contraction over the output matrix on the
     // tensor cores (into the caller's buffer or the work buffer), then the greedy tokens and the acceptance rule
     const int H = m.shape.hidden;
@@ -2166,6 +2167,7 @@ const char *prefill_verify_head(const PrefillModel &m, PrefillBuffers *b, int n,
     if (grid * 256 > rows) grid = (rows + 255) / 256;
     launch_pdl(prefill_verify_pick_kernel, dim3(grid), dim3(256), 0, s, static_cast<const float *>(logits), ids, rows, n, static_cast<const int *>(b->tokens),
                b->head_val, b->head_idx, b->head_ticket, m.state, slot0, pos, n_accepted_out, next_token_out);
+    *launches += 3;
     return cudaGetLastError() == cudaSuccess ? nullptr : "block verification output layer launch failed";
 }
 

@@ -76,7 +76,7 @@ void prefill_free(PrefillBuffers *b);
 // position .. position + n - 1.  Every layer's K and V rows are written.  whole_last_layer = false: the last layer's attention
 // and MLP are skipped (their result would only feed an output layer nobody reads); true: they run, and the residual stream
 // behind the last layer is left in PrefillBuffers::resid for prefill_head.  Sets the device state to cache length slot0 + n.
-// Returns nullptr or a message.
+// *launches: the kernels enqueued.  Returns nullptr or a message.
 const char *prefill_run(const PrefillModel &m, PrefillBuffers *b, const int32_t *tokens, int n, int slot0, int position, bool whole_last_layer,
                         cudaStream_t stream, int *launches);
 
@@ -87,8 +87,9 @@ const char *prefill_head(const PrefillModel &m, PrefillBuffers *b, int row, cons
                          float *logits_out, int *next_token_out, int token, int pos, cudaStream_t stream);
 
 // Block verification through the prompt kernels (Sec. 3.11): after prefill_run(..., n tokens, whole_last_layer = true), the logits of
-// all n rows ([n][rows], or nullptr), the greedy acceptance on the device and the state update (cache length slot0 + accepted).
+// all n rows ([n][rows], or nullptr), the greedy acceptance on the device and the state update (cache length slot0 + accepted).  Adds its
+// kernels to *launches.
 const char *prefill_verify_head(const PrefillModel &m, PrefillBuffers *b, int n, const void *final_norm, const void *lm, const int *ids, int rows,
-                                float *logits_out, int *n_accepted_out, int *next_token_out, int slot0, int pos, cudaStream_t stream);
+                                float *logits_out, int *n_accepted_out, int *next_token_out, int slot0, int pos, cudaStream_t stream, int *launches);
 
 }  // namespace edgefm

@@ -213,3 +213,35 @@ def test_prompt_into_the_compressed_cache(name, T0, n):
             assert int(pair.ctx.next_token.item()) == ref_next
     finally:
         pair.close()
+
+
+@pytest.mark.parametrize("T0,n,kv_format", [(0, 5, None), (0, 9, None), (0, 9, "int8"), (2100, 130, None), (20, 300, "int8"), (0, 4200, None)])
+def test_launch_count_of_a_prompt(T0, n, kv_format):
+    """The library's count of the kernels a prompt enqueues, against the kernel nodes of the same call recorded by a stream capture (never run):
+    short prompts that end in a decode step, shared-out attention with its merge, the 8-bit cache, a prompt of two passes."""
+    import torch
+    from cuda.bindings import runtime as rt
+    pair = Pair(CONFIGS["tiny"], cache_len=T0, max_context=T0 + n, kv_format=kv_format)
+
+    def ok(result):
+        assert int(result[0]) == 0, result[0]
+        return result[1] if len(result) == 2 else result[1:]
+
+    try:
+        ctx, toks = pair.ctx, [1] * n
+        ctx.prefill(toks, T0)                                  # buffers are made outside a capture
+        eager = ctx.prefill_launches
+        torch.cuda.synchronize()
+        ctx.append_kv(T0)
+        torch.cuda.synchronize()
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            ok(rt.cudaStreamBeginCapture(s.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal))
+            ctx.prefill(toks, T0)
+            graph = ok(rt.cudaStreamEndCapture(s.cuda_stream))
+        nodes, count = ok(rt.cudaGraphGetNodes(graph, 8192))
+        kinds = [ok(rt.cudaGraphNodeGetType(node)) for node in nodes[:count]]
+        ok(rt.cudaGraphDestroy(graph))
+        assert kinds.count(rt.cudaGraphNodeType.cudaGraphNodeTypeKernel) == ctx.prefill_launches == eager
+    finally:
+        pair.close()

@@ -316,6 +316,10 @@ edgefm_status edgefm_debug_prefill_plan(int32_t epilogue, int32_t M, int32_t N, 
  * pairs of CTAs, 1 = the weights are the rows of the multiply and the tokens its columns}.  Host only. */
 edgefm_status edgefm_debug_prefill_launch(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t *out5);
 
+/* How many CTAs share the key blocks (128 keys) of a tile of 128 queries in edgefm_prefill's attention: T tokens of n_q_heads heads behind
+ * slot0 cached positions.  More than 1: a kernel that merges their partial rows follows.  Host only. */
+edgefm_status edgefm_debug_prefill_attention(int32_t T, int32_t slot0, int32_t n_q_heads, int32_t num_sms, int32_t *parts);
+
 /* Host-only check of the planner: how the step kernel for `tokens` tokens per call (1, 2, 4 or 8) is laid out for a shape on n_sms SMs with
  * smem_bytes of shared memory per CTA.  out40 = {CTAs, dynamic shared memory, bytes of the ring, bytes of its largest chunk, bytes of the
  * tables, chunks the list has room for, 1 = a tight build (no list, unit tables in global memory), bytes of these tables, cached

@@ -51,7 +51,7 @@ class _Weights(ctypes.Structure):
 
 EXPORTS = ("edgefm_create", "edgefm_prefill_kv", "edgefm_decode_step", "edgefm_destroy", "edgefm_get_length",
            "edgefm_export_kv", "edgefm_get_launches_per_step", "edgefm_get_prefill_launches", "edgefm_last_error", "edgefm_version",
-           "edgefm_sync_status", "edgefm_debug_profile", "edgefm_debug_set_wait_limit", "edgefm_debug_set_prefill_wait", "edgefm_debug_prefill_plan", "edgefm_debug_prefill_launch", "edgefm_debug_plan", "edgefm_debug_step_plan", "edgefm_decode_step_static", "edgefm_set_vocab_subset",
+           "edgefm_sync_status", "edgefm_debug_profile", "edgefm_debug_set_wait_limit", "edgefm_debug_set_prefill_wait", "edgefm_debug_prefill_plan", "edgefm_debug_prefill_launch", "edgefm_debug_prefill_attention", "edgefm_debug_plan", "edgefm_debug_step_plan", "edgefm_decode_step_static", "edgefm_set_vocab_subset",
            "edgefm_append_kv", "edgefm_create_with_options", "edgefm_export_kv_int8", "edgefm_verify_block", "edgefm_sync_length", "edgefm_prefill_tokens", "edgefm_prefill")
 
 
@@ -245,6 +245,16 @@ def edgefm_debug_prefill_launch(epilogue, M, N, K, num_sms=148):
     out = (ctypes.c_int32 * 5)()
     _check(L.edgefm_debug_prefill_launch(epilogue, M, N, K, num_sms, out), None)
     return tuple(int(v) for v in out)
+
+
+def edgefm_debug_prefill_attention(T, slot0, n_q_heads, num_sms=148) -> int:
+    """CTAs that share the key blocks of a tile of 128 queries of a prompt (host only)."""
+    L = load_library()
+    L.edgefm_debug_prefill_attention.restype = ctypes.c_int
+    L.edgefm_debug_prefill_attention.argtypes = [ctypes.c_int32] * 4 + [ctypes.POINTER(ctypes.c_int32)]
+    out = ctypes.c_int32()
+    _check(L.edgefm_debug_prefill_attention(T, slot0, n_q_heads, num_sms, ctypes.byref(out)), None)
+    return out.value
 
 
 def edgefm_debug_set_prefill_wait(ctx, polls, extra_arrivals=0):

@@ -844,6 +844,12 @@ edgefm_status edgefm_debug_prefill_launch(int32_t epilogue, int32_t M, int32_t N
     return EDGEFM_OK;
 }
 
+edgefm_status edgefm_debug_prefill_attention(int32_t T, int32_t slot0, int32_t n_q_heads, int32_t num_sms, int32_t *parts) {
+    if (!parts || T < 1 || slot0 < 0 || n_q_heads < 1 || num_sms < 1) return EDGEFM_ERR_INVALID_ARG;
+    *parts = prefill_attention_parts(T, slot0, n_q_heads, num_sms);
+    return EDGEFM_OK;
+}
+
 edgefm_status edgefm_export_kv(edgefm_ctx *ctx, void *k_out, void *v_out, void *stream) {
     if (!ctx) return EDGEFM_ERR_INVALID_ARG;
     if (!k_out || !v_out) return fail(ctx, EDGEFM_ERR_INVALID_ARG, "null output");

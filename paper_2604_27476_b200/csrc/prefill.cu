@@ -1881,9 +1881,8 @@ bool encode_bytes_map(CUtensorMap *m, const void *base, long long rows, int row_
 }
 
 // kc / vc: this layer's cache, bf16 rows or (k_scale != nullptr) rows of 8-bit codes with their scales.
-// Few query tiles behind a long cache (a short suffix behind a prefix, a verified block) would run on few CTAs, each walking the whole cache: the key
-// blocks are then shared out among as many CTAs as fit the SMs once, and their partial rows merged (part_o / part_ml: room for
-// num_sms tiles of 128 rows).  Two blocks cost a CTA about 3.5 us (one for either group), the merge about as much.
+// The key blocks of a query tile may be shared out (prefill_attention_parts); the partial rows are then merged (part_o / part_ml: room for num_sms tiles
+// of 128 rows).
 template <int D>
 const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *vc, const float *k_scale, const float *v_scale, uint16_t *out,
                                 size_t plane, int T, int slot0, int nq, int nkv, int max_context, uint32_t wait_limit, uint32_t extra_arrivals, int *error,
@@ -1896,12 +1895,7 @@ const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *v
            : (!encode_operand_map(&mk, kc, kv_rows, D, AT_BN) || !encode_operand_map(&mv, vc, kv_rows, D, AT_BN)))
         return "cuTensorMapEncodeTiled failed";
     const float scale_log2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(D)));
-    const int blocks = (slot0 + T - 1) / AT_BN + 1, tiles = (T + AT_BM - 1) / AT_BM;
-    int splits = 1;
-    for (int c = 2, best = (blocks + 1) / 2; c <= AT_SPLIT_MAX && c * nq * tiles <= num_sms; ++c) {
-        const int cost = ((blocks + c - 1) / c + 1) / 2 + 1;
-        if (cost < best) { splits = c; best = cost; }
-    }
+    const int tiles = (T + AT_BM - 1) / AT_BM, splits = prefill_attention_parts(T, slot0, nq, num_sms);
     const dim3 grid(nq, tiles, splits);
     if (q8) {
         if (cudaFuncSetAttribute(prefill_attention_tc_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::SMEM_Q8) != cudaSuccess)
@@ -1923,6 +1917,19 @@ const char *launch_attention_tc(const uint16_t *q, const void *kc, const void *v
 }
 
 }  // namespace
+
+// Few query tiles behind a long cache (a short suffix behind a prefix, a verified block) would run on few CTAs, each walking the whole cache: the key
+// blocks are then shared out among as many CTAs as fit the SMs once.  Two blocks cost a CTA about 3.5 us (one for either group), the merge about
+// as much.
+int prefill_attention_parts(int T, int slot0, int nq, int num_sms) {
+    const int blocks = (slot0 + T - 1) / AT_BN + 1, tiles = (T + AT_BM - 1) / AT_BM;
+    int parts = 1;
+    for (int c = 2, best = (blocks + 1) / 2; c <= AT_SPLIT_MAX && c * nq * tiles <= num_sms; ++c) {
+        const int cost = ((blocks + c - 1) / c + 1) / 2 + 1;
+        if (cost < best) { parts = c; best = cost; }
+    }
+    return parts;
+}
 
 // What a contraction is launched as (host logic, depends on the sizes and the SM count alone).
 PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int num_sms) {

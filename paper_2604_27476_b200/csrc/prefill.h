@@ -65,6 +65,8 @@ struct PrefillModel {
 struct PrefillPlan { int columns, splits, cluster; bool pairs, swap; };
 constexpr int PF_CLUSTER_MAX = 8;
 PrefillPlan prefill_plan(int epilogue, int head_dim, int M, int N, int K, int num_sms);
+// CTAs that share the key blocks of a query tile: T queries of nq heads behind slot0 cached rows (host logic).
+int prefill_attention_parts(int T, int slot0, int nq, int num_sms);
 
 // Bytes the work buffers of a pass over `chunk` tokens take.
 size_t prefill_buffer_bytes(const edgefm_shape &sh, int chunk);

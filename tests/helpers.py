@@ -52,6 +52,19 @@ def assert_appended_rows_close(gpu_bits: np.ndarray, ref_bits: np.ndarray):
     assert np.mean(gpu_bits == ref_bits) > 0.97
 
 
+def random_norms(weights: dict, seed: int = 1) -> dict:
+    """The same weights with norm vectors that are not one, N(1, 0.2^2) as bf16 and different in every layer (a norm with another's weights, or
+    with none, passes where all of them are one)."""
+    rng = np.random.default_rng(seed)
+
+    def norm(like):
+        f = (1 + 0.2 * rng.standard_normal(like.shape)).astype(np.float32)
+        return ((f.view(np.uint32) + 0x8000) >> 16).astype(np.uint16)
+
+    layers = [dict(lw, input_norm=norm(lw["input_norm"]), post_norm=norm(lw["post_norm"])) for lw in weights["layers"]]
+    return dict(weights, layers=layers, final_norm=norm(weights["final_norm"]))
+
+
 class Pair:
     """The oracle model and the CUDA context fed from the same host weights and KV prefix."""
 

@@ -43,9 +43,9 @@ def assert_rows_close(gpu_bits, ref_bits, what):
     return worst
 
 
-def run_case(cfg, T0, n, seed, follow=True):
+def run_case(cfg, T0, n, seed, follow=True, weights=None):
     import torch
-    pair = Pair(cfg, cache_len=T0, max_context=T0 + n + 3)
+    pair = Pair(cfg, cache_len=T0, max_context=T0 + n + 3, weights=weights)
     try:
         rng = np.random.default_rng(seed)
         toks = rng.integers(0, cfg.vocab, n).tolist()
@@ -175,7 +175,7 @@ def test_prefill_then_block_verification_and_pruned_vocabulary():
         pair.close()
 
 
-@pytest.mark.parametrize("name,T0,n", [("tiny", 0, 9), ("tiny", 20, 300), ("tiny", 5, 4200), ("tiny", 3000, 50), ("qwen2.5-1.5b", 32, 200)])
+@pytest.mark.parametrize("name,T0,n", [("tiny", 0, 9), ("tiny", 20, 300), ("tiny", 5, 4200), ("tiny", 3000, 50), ("tiny", 0, 1000), ("qwen2.5-1.5b", 32, 200)])
 def test_prompt_into_the_compressed_cache(name, T0, n):
     """The same prefill on a context with the 8-bit cache (Sec. 3.9): the new rows are compressed from their fp32 values (k
     after RoPE, v) exactly as the decode step compresses its own row, and attention reads codes x scales for every row, the

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from edgefm_synth import CONFIGS, first_token, make_kv, make_weights
-from helpers import (LOGIT_MAX_ABS, Pair, TOKEN_MARGIN, assert_appended_rows_close, assert_logits_close, top2_margin)
+from helpers import (LOGIT_MAX_ABS, Pair, TOKEN_MARGIN, assert_appended_rows_close, assert_logits_close, random_norms, top2_margin)
 
 pytestmark = pytest.mark.gpu
 
@@ -207,4 +207,29 @@ def test_long_context_build_crosses_the_attention_mode_switch(variant):
         run_teacher_forced(pair, 9, 5, 8188)          # attends 8189 .. 8197 positions
         check_cache_against_oracle(pair, 8188, 9)
     finally:
+        pair.close()
+
+
+@pytest.mark.parametrize("head_dim,block_tokens", [(64, 0), (128, 0), (64, 4)], ids=["heads_of_64", "heads_of_128", "blocks"])
+def test_norm_weights_that_are_not_one(head_dim, block_tokens):
+    """Every layer's two norms and the last one have weights of their own: plain steps, then blocks of four (on a context built for them) and eight."""
+    import torch
+    cfg = TINY.with_(head_dim=head_dim, qkv_bias=True)
+    pair = Pair(cfg, cache_len=40, max_context=64, weights=random_norms(make_weights(cfg)), block_tokens=block_tokens)
+    try:
+        tok, pos = first_token(cfg), 40
+        run_teacher_forced(pair, 3, tok, pos)
+        check_cache_against_oracle(pair, 40, 3)
+        pair.ctx.sync_length()
+        for m in (4, 8):
+            length = pair.oracle.cur_len
+            block = [tok] + list(range(5, 4 + m))
+            ref_rows, ref_acc, _ = pair.oracle.verify_block(block, length)
+            pair.ctx.verify_block(block, length)
+            assert pair.ctx.sync_length() == pair.oracle.cur_len == length + ref_acc
+            got = pair.ctx.block_logits.cpu().numpy()
+            for t in range(ref_acc):
+                assert_logits_close(got[t], ref_rows[t], f"block of {m}, row {t}")
+    finally:
+        torch.cuda.synchronize()
         pair.close()

@@ -27,29 +27,17 @@ import numpy as np
 
 from edgefm_synth import CONFIGS, GLOBAL_SEED, first_token, make_kv, make_weights
 
-# DRAM traffic of one launch of the step kernel: dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of
-# that kernel, per configuration, with the profile summary (and the source revision it names) the figure comes from.
-# Only captured configurations have a value; a figure is only as current as its summary says.
-NCU_TRAFFIC = {"qwen2.5-1.5b": {"bytes": None, "source": "profiles/step_kernel_qwen2.5-1.5b_ctx2048.md"}}
+# DRAM traffic of one launch of the step kernel, dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture, per configuration, and the
+# source revision it was taken at.  Only captured configurations have a value; a figure is only as current as its revision.
+NCU_TRAFFIC = {"qwen2.5-1.5b": (3.1516e9 + 5.447e6, "6449c7a")}
 
 
 def ncu_traffic(name):
-    """(bytes or None, where the figure comes from): parsed from the profile summary, which states read and write bytes."""
-    import re
-    ent = NCU_TRAFFIC.get(name)
-    if not ent:
+    """(bytes or None, where the figure comes from)."""
+    if name not in NCU_TRAFFIC:
         return None, None
-    path = ROOT / ent["source"]
-    try:
-        text = path.read_text()
-        rd = re.search(r"dram__bytes_read\.sum\s*\|\s*([0-9.]+)\s*GB", text)
-        wr = re.search(r"dram__bytes_write\.sum\s*\|\s*([0-9.]+)\s*MB", text)
-        rev = re.search(r"source revision:\s*`?([0-9a-f]{7,40})", text)
-        if rd and wr:
-            return float(rd.group(1)) * 1e9 + float(wr.group(1)) * 1e6, f"{ent['source']}" + (f" (revision {rev.group(1)})" if rev else "")
-    except OSError:
-        pass
-    return None, None
+    traffic, revision = NCU_TRAFFIC[name]
+    return traffic, f"ncu, one launch of the step kernel (revision {revision})"
 
 METRIC = "batch1_decode_ms_per_token"
 UNIT = "ms/token"

@@ -1204,7 +1204,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) prefill_tile_kernel(const __g
 // columns of hi and 16 of lo);  O += P_j V_j (M 128, N = D, K = 128 keys; P from tensor memory, V straight from its cache rows as an
 // MN-major B operand), a sum of its own per group in tensor memory.  The exponentials are taken against a reference maximum that
 // moves only when the row's maximum has grown by more than 2^8 (then the row of O and the row sum are rescaled once).  At the end
-// the groups' sums (and those of the other CTAs of a cluster) meet in shared memory.  The scores and P V are issued by two threads
+// the groups' sums meet in shared memory (those of the CTAs that share a query tile's key blocks in prefill_attention_merge_kernel).  The scores and P V are issued by two threads
 // (warps 1 and 2), the K and V tiles have barriers of their own.
 //   tensor memory: scores and probabilities [0, 128) and [128, 256), O [256, 256 + D) and [256 + D, 256 + 2 D)
 //   shared memory: Q 2 x D/64 x 16 KB | 2 stages x (K D/64 x 16 KB, V D/64 x 16 KB)   (compressed cache: + landing areas)
@@ -1249,7 +1249,7 @@ __global__ void __launch_bounds__(AT_THREADS + (Q8 ? 32 * AT_CW : 0), Q8 ? 0 : 1
                                                                    float scale_log2, uint32_t wait_limit, uint32_t extra_arrivals, int *error,
                                                                    const float *k_scale, const float *v_scale, float *part_o, float2 *part_ml) {
     // Q8: the cache holds 8-bit codes and a scale per row (k_scale, v_scale: this layer's [nkv][max_context]); map_k / map_v then
-    // describe byte matrices; two more warps expand the codes to bf16 (exactly) into the operand layout, the softmax multiplies
+    // describe byte matrices; AT_CW more warps expand the codes to bf16 (exactly) into the operand layout, the softmax multiplies
     // the scores by the keys' scales and folds the values' scales into the probabilities.
     using C = AttnCfg<D>;
     extern __shared__ uint8_t at_tc_dyn[];
@@ -1735,11 +1735,11 @@ __global__ void __launch_bounds__(128) prefill_attention_merge_kernel(const floa
     }
 }
 
-// Launch with the programmatic-stream-serialization attribute (see pdl_trigger / pdl_wait), in clusters of cluster.x CTAs.  Long passes
+// Launch with the programmatic-stream-serialization attribute (see pdl_trigger / pdl_wait), in clusters of that many CTAs.  Long passes
 // gain, too, where their kernels are short: 1423 tokens, 0.5B shape 4455 -> 4023 us, 2541 tokens 6075 -> 5838; 2048, 1.5B 11205 -> 11065; 4200,
 // 7B, no difference.  (Launched before the tensor memory was allocated the successors cost long passes 1 - 3 %.)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster(dim3 cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
+cudaError_t launch_cluster(int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -1749,11 +1749,11 @@ cudaError_t launch_cluster(dim3 cluster, void (*kernel)(KArgs...), dim3 grid, di
     int n = 0;
     attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[n++].val.programmaticStreamSerializationAllowed = 1;
-    if (cluster.x * cluster.z > 1) {
+    if (cluster > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
-        attr[n].val.clusterDim.x = cluster.x;
+        attr[n].val.clusterDim.x = cluster;
         attr[n].val.clusterDim.y = 1;
-        attr[n].val.clusterDim.z = cluster.z;
+        attr[n].val.clusterDim.z = 1;
         ++n;
     }
     cfg.attrs = attr;
@@ -1762,10 +1762,12 @@ cudaError_t launch_cluster(dim3 cluster, void (*kernel)(KArgs...), dim3 grid, di
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
-    return launch_cluster(dim3(1), kernel, grid, block, smem, stream, static_cast<KArgs>(args)...);
+    return launch_cluster(1, kernel, grid, block, smem, stream, static_cast<KArgs>(args)...);
 }
 
-// Clusters of c CTAs, one CTA per SM, that run at once: a cluster stays within a GPC.  Of 148 SMs, as cudaOccupancyMaxActiveClusters has it on a B200;
+// Clusters of c CTAs, one CTA per SM, that run at once: a cluster stays within a GPC.  Of 148 SMs, what cudaOccupancyMaxActiveClusters answered on each of
+// five B200s; a table, so that the plan and with it the order of the sums depend on the sizes and the SM count alone (on a GPU with other GPCs a plan
+// may take a second round);
 // one tile more than that is a second round (1.5B shape, 152 tokens: O and down as 24 clusters of six took 14 us a layer more than 12 of eight).
 int clusters_at_once(int c, int num_sms) {
     constexpr int AT_148[PF_CLUSTER_MAX + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
@@ -1816,7 +1818,7 @@ const char *launch_gemm_cfg(const CUtensorMap &ma, const CUtensorMap &ml, const 
     if (cudaFuncSetAttribute(prefill_gemm_kernel<EPI, COLUMNS, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
         return "cudaFuncSetAttribute failed";
     const int ctas = PAIR ? 2 : 1;
-    launch_cluster(dim3(ctas), prefill_gemm_kernel<EPI, COLUMNS, PAIR>, dim3((units < workers ? units : workers) * ctas), dim3(192), C::SMEM, s, ma, ml, mb, g);
+    launch_cluster(ctas, prefill_gemm_kernel<EPI, COLUMNS, PAIR>, dim3((units < workers ? units : workers) * ctas), dim3(192), C::SMEM, s, ma, ml, mb, g);
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill GEMM launch failed";
 }
 
@@ -1831,7 +1833,7 @@ const char *launch_tile(const CUtensorMap &ma, const CUtensorMap &ml, const CUte
     for (g.tmem_cols = 32; g.tmem_cols < cols;) g.tmem_cols *= 2;
     if (cudaFuncSetAttribute(prefill_tile_kernel<EPI, BN, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM_DEEP) != cudaSuccess)
         return "cudaFuncSetAttribute failed";
-    launch_cluster(dim3(g.cluster), prefill_tile_kernel<EPI, BN, SWAP>, dim3(tiles * g.cluster), dim3(TILE_THREADS), static_cast<size_t>(room.smem), s, ma, ml, mb, g);
+    launch_cluster(g.cluster, prefill_tile_kernel<EPI, BN, SWAP>, dim3(tiles * g.cluster), dim3(TILE_THREADS), static_cast<size_t>(room.smem), s, ma, ml, mb, g);
     return cudaGetLastError() == cudaSuccess ? nullptr : "prefill contraction launch failed";
 }
 

@@ -49,7 +49,7 @@ def test_clusters_run_at_once():
 
 
 def test_short_prompts_share_the_k_of_a_tile():
-    """77 tokens of the 0.5B shape: QKV, O and down run on 90 to 112 CTAs instead of 14 to 18."""
+    """77 tokens of the 0.5B shape: QKV, O and down run on 98 to 126 CTAs instead of 14 to 18."""
     s = shapes(CONFIGS["qwen2.5-0.5b"])
     for op, least in (("qkv", 5), ("o", 7), ("down", 8)):
         epi, N, K = s[op]
